@@ -112,9 +112,11 @@ void smat_plan_destroy(smat_plan* plan);
 
 smat_status smat_get_geometry(const smat_plan* plan, smat_geometry* out);
 
-/* 1 when this plan runs its causal branch on the tcgen05 tensor-core kernels (bf16, d_k = d_v = 128, block
- * boundary and recent length multiples of 128, SMAT_FLAG_SIMT_ONLY not set), 0 when it runs on the fp32 ALUs.
- * A property of the shape, not of the device. */
+/* 1 when this plan's forward runs its causal branch on the tcgen05 tensor-core kernels (bf16, d_k = d_v = 128,
+ * SMAT_FLAG_SIMT_ONLY and SMAT_FLAG_GATED not set), 0 when it runs on the fp32 ALUs.  Plans whose block boundary or
+ * recent length is not a multiple of 128 keep fp32 tables and split every fp32 operand of a tensor-core product into
+ * two bf16 parts, and their backward runs on the fp32 ALUs (with SMAT_FLAG_PER_TILE_STATES the forward too, and this
+ * returns 0).  A property of the shape, not of the device. */
 int smat_uses_tensor_cores(const smat_plan* plan);
 
 /* 1 when smat_forward_gated / smat_backward_gated of this plan (SMAT_FLAG_GATED) run on the tensor-core kernels: the
@@ -248,7 +250,8 @@ smat_status smat_debug_mask(const smat_plan* plan, uint8_t* mask, void* cuda_str
  * For d = 1 there is no separate F/U: the single state U_0 = F_0 is carried by the scan, and
  * F and U receive that state (the incoming state of the first recent chunk or tile).
  * Tensor-core plans have per-tile states only after a forward of a plan created with SMAT_FLAG_PER_TILE_STATES, or
- * after smat_backward; the two-level form keeps one state per segment of tiles, which is no per-chunk table: there
+ * after smat_backward (plans whose blocks are not whole 128-token tiles: after smat_backward, fp32 per chunk); the
+ * two-level form keeps one state per segment of tiles, which is no per-chunk table: there
  * Sin (and, for d = 1, F and U) must be NULL, otherwise SMAT_ERR_UNSUPPORTED is returned.
  * Asynchronous on `cuda_stream`.
  */

@@ -32,6 +32,8 @@ struct smat_plan {
   smat_plan* inner;
   size_t off_inner;
   bool tc;             // tensor-core kernels for the causal branch
+  bool ragged_tc;      // ... of the forward only, for blocks that are not whole 128-token tiles: fp32 tables, and the
+                       // state and the scores split into two bf16 parts (backward: fp32-ALU kernels)
   bool u_bf16;         // forward keeps the type table U in bf16 and reads it with the tensor-core typed read
   bool pool_tc;        // forward pools the profile table on the tensor cores (enough tokens per profile)
   bool f_bf16;         // the profile table is kept in bf16 (d = 2: it is the type table; tab_tc: it is an MMA operand)
@@ -42,7 +44,8 @@ struct smat_plan {
   bool ubar_bf16;      // ... and keeps them in bf16
   bool fbar_bf16;      // the per-profile adjoint states (transposed tabulation) are kept in bf16
   mutable int launches;
-  mutable bool tile_states;       // the last call left one bf16 incoming state per 128-token tile at off_sin
+  mutable bool tile_states;       // the last call left its incoming states at off_sin (bf16 per 128-token tile; on plans
+                                  // with ragged_tc fp32 per chunk)
   mutable bool kept_tile_states;  // the last forward left them at off_sin_tiles for the backward (KEEP_FORWARD_TABLES)
   mutable bool kept_gated_forward;  // the last call was the tensor-core gated forward: λ, the rescaled K copies, U and the
                                     // per-tile states are still in the workspace (used under KEEP_FORWARD_TABLES)
@@ -395,6 +398,8 @@ smat_status smat_plan_create(smat_plan** out, int batch, int heads, int64_t T, i
   // them is checked by the calls that launch.
   pl->tc = dtype == SMAT_BF16 && d_k == 128 && d_v == 128 && !(flags & (SMAT_FLAG_SIMT_ONLY | SMAT_FLAG_GATED)) && g.n % 128 == 0 &&
            g.m % 128 == 0 && g.n >= 128;
+  pl->ragged_tc = dtype == SMAT_BF16 && d_k == 128 && d_v == 128 && !pl->tc &&
+                  !(flags & (SMAT_FLAG_SIMT_ONLY | SMAT_FLAG_GATED | SMAT_FLAG_PER_TILE_STATES));
   if (!g.dense_G && (smat_tabulate_alg2_slab(g.B, pl->rp) < 1)) { delete pl; return SMAT_ERR_UNSUPPORTED; }
   // d >= 3 on the tensor-core path: U is only ever a bf16 MMA operand, so it is stored as bf16 (half the bytes)
   pl->tab_tc = pl->tc && !g.dense_G && !(flags & (SMAT_FLAG_ALG2_TABULATION | SMAT_FLAG_ALU_TABULATION)) &&
@@ -520,7 +525,7 @@ smat_status smat_get_geometry(const smat_plan* pl, smat_geometry* out) {
   return SMAT_OK;
 }
 
-int smat_uses_tensor_cores(const smat_plan* pl) { return pl && pl->tc ? 1 : 0; }
+int smat_uses_tensor_cores(const smat_plan* pl) { return pl && (pl->tc || pl->ragged_tc) ? 1 : 0; }
 
 int smat_gated_forward_uses_tensor_cores(const smat_plan* pl) { return pl && pl->inner ? 1 : 0; }
 
@@ -606,11 +611,12 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
       int nseg0 = 0, nseg1 = 0;
       smat_segment_counts(tiles0, tiles1, pl->bh, L, &nseg0, &nseg1);
       const int64_t nseg = nseg0 + nseg1;
-      SMAT_TRY(cx, "segment_state_tc", smat_launch_segment_state_tc(K, V, seg, tiles0, tiles1, nseg0, nseg1, pl->bh, status, cx.st));
+      const int64_t rows0 = tiles0 * 128, rows1 = tiles1 * 128;
+      SMAT_TRY(cx, "segment_state_tc", smat_launch_segment_state_tc(K, V, seg, rows0, rows1, nseg0, nseg1, pl->bh, status, cx.st));
       SMAT_TRY(cx, "segment_scan", smat_launch_scan(seg, pl->rp, nseg, pl->bh, 0, nseg0, nseg0, nseg, 0, cx.st));
       const bool keep = (pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES) != 0;   // a backward will want the per-tile states
-      SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, seg, ylr, lr ? pl->geo.n : pl->T, O,
-                                                                       tiles0, tiles1, nseg0, nseg1, pl->bh, status, cx.st,
+      SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, seg, ylr, 0, lr ? pl->geo.n : pl->T, O,
+                                                                       rows0, rows1, nseg0, nseg1, pl->bh, status, cx.st,
                                                                        keep ? cx.ws + pl->off_sin_tiles : nullptr));
       pl->kept_tile_states = keep;
     } else {
@@ -620,6 +626,30 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
                                                                    lr ? pl->geo.n : pl->T, O, pl->T, pl->bh, status,
                                                                    cx.st));                   // step 7
     }
+    pl->launches = cx.launches;
+    return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;
+  }
+  if (pl->ragged_tc) {
+    pl->tile_states = false;
+    // Blocks that are not whole tiles: tables as on the fp32-ALU path (steps 2-4), the causal branch in its two-level
+    // form over tiles of which the last of a block is partial.
+    int* status = reinterpret_cast<int*>(cx.ws + pl->off_status);
+    float* ylr = cx.f(pl->off_acc);
+    float* seg = cx.f(pl->off_sin);
+    const bool lr = !pl->geo.dense_G;
+    const int64_t rows0 = lr ? pl->geo.n : pl->T, rows1 = lr ? pl->geo.m : 0;
+    if (lr) {
+      build_type_table(cx, K, V);
+      zero_unrouted(cx, SMAT_GM_TYPE, ylr, 512);
+      state_read(cx, "read_type", SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, nullptr, ylr, nullptr);
+    }
+    int nseg0 = 0, nseg1 = 0;
+    smat_segment_counts((rows0 + 127) / 128, (rows1 + 127) / 128, pl->bh, 2, &nseg0, &nseg1);
+    const int64_t nseg = nseg0 + nseg1;
+    SMAT_TRY(cx, "segment_state_tc", smat_launch_segment_state_tc(K, V, seg, rows0, rows1, nseg0, nseg1, pl->bh, status, cx.st));
+    SMAT_TRY(cx, "segment_scan", smat_launch_scan(seg, pl->rp, nseg, pl->bh, 0, nseg0, nseg0, nseg, 0, cx.st));
+    SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, seg, ylr, 1, lr ? pl->geo.n : pl->T, O, rows0,
+                                                                     rows1, nseg0, nseg1, pl->bh, status, cx.st));
     pl->launches = cx.launches;
     return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;
   }
@@ -753,6 +783,7 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
     return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;
   }
   build_forward_tables(cx, K, V);
+  pl->tile_states = true;
   float* sin = cx.f(pl->off_sin);
   float* dbar = cx.f(pl->off_dbar);
   float* acc = cx.f(pl->off_acc);
@@ -1139,6 +1170,8 @@ smat_status smat_debug_tables(const smat_plan* pl, const void* workspace, float*
   const char* ws = static_cast<const char*>(workspace);
   const size_t state = (size_t)pl->rp * sizeof(float);
   cudaError_t err = cudaSuccess;
+  // blocks that are not whole tiles: per-chunk states exist only after the (fp32-ALU) backward
+  if (pl->ragged_tc && (Sin || (pl->geo.dense_G && (F || U))) && !pl->tile_states) return SMAT_ERR_UNSUPPORTED;
   if (pl->tc) {
     // Tensor-core plans: incoming states exist per 128-token tile (bf16) after a per-tile forward or a backward; the
     // two-level form keeps only one state per segment of tiles, which is no per-chunk table.

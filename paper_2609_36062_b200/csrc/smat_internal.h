@@ -197,11 +197,15 @@ cudaError_t smat_launch_routing_lists(const int32_t* prof, const int32_t* type, 
 cudaError_t smat_launch_zero_unrouted(const int32_t* key, int64_t count, int64_t G, int64_t first, void* rows, int64_t T,
                                       int row_bytes, int bh, cudaStream_t st);
 // Two-level causal branch: segment totals, then (after an exclusive scan of the totals) per-segment fused output.
+// Block 0 holds rows0 tokens of every head and block 1 the rows1 after them (0: one block, d = 1); the last tile of a
+// block may be partial.
 int smat_segment_tiles(int64_t tiles_block0, int64_t tiles_block1, int bh);
 void smat_segment_counts(int64_t tiles0, int64_t tiles1, int bh, int L, int* nseg0, int* nseg1);
-cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* totals, int64_t tiles0, int64_t tiles1,
+cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* totals, int64_t rows0, int64_t rows1,
                                          int nseg0, int nseg1, int bh, int* status, cudaStream_t st);
+// ylr_f32 = 0: long-range rows in bf16, blocks of whole tiles.  ylr_f32 = 1: fp32 rows, any blocks, and the state and
+// the scores enter their products as a bf16 part plus a bf16 remainder.
 cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const void* V, const float* seg_in,
-                                          const void* ylr_bf16, int64_t n_lr, void* O, int64_t tiles0, int64_t tiles1,
+                                          const void* ylr, int ylr_f32, int64_t n_lr, void* O, int64_t rows0, int64_t rows1,
                                           int nseg0, int nseg1, int bh, int* status, cudaStream_t st,
                                           void* sin_tiles = nullptr);

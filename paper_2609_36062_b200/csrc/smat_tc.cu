@@ -660,7 +660,13 @@ constexpr int SEG_STATE_SMEM = SEG_STATE_STAGES * 4 * BOX_BYTES + 1024 + 256;
 struct SegCut {
   int nseg0, nseg;
   int64_t tiles0, tiles1;
+  int64_t rows0, rows;   // tokens of block 0, and of the head: block 1 starts at token rows0, each block's last tile may
+                         // be partial (rows0 = 128 tiles0 and so on when the blocks are whole tiles)
 };
+// First token of tile `tile` (tiles are numbered through both blocks).
+__device__ __forceinline__ int64_t seg_tile_row(const SegCut& c, int64_t tile) {
+  return tile < c.tiles0 ? tile * TILE : c.rows0 + (tile - c.tiles0) * TILE;
+}
 __device__ __forceinline__ void seg_range(const SegCut& c, int seg, int64_t* tile0, int* count) {
   if (seg < c.nseg0) {
     const int64_t a = (int64_t)seg * c.tiles0 / c.nseg0, b = (int64_t)(seg + 1) * c.tiles0 / c.nseg0;
@@ -715,7 +721,8 @@ __global__ void __launch_bounds__(192) segment_state_tc_kernel(const __grid_cons
       const int s = it % SEG_STATE_STAGES;
       if (it >= SEG_STATE_STAGES && !mbar_wait(empty + s, ((it / SEG_STATE_STAGES) - 1) & 1, wc)) break;
       uint8_t* st = smem + s * 4 * BOX_BYTES;
-      const int row = (int)((int64_t)bh * prm.T + (tile0 + it) * TILE);
+      // (every tile of a segment that is not its block's last one is whole)
+      const int row = (int)((int64_t)bh * prm.T + seg_tile_row(prm.cut, tile0) + (int64_t)it * TILE);
       mbar_expect_tx(full + s, 4 * BOX_BYTES);
       tma_load_2d(st, &tmK, 0, row, full + s);
       tma_load_2d(st + BOX_BYTES, &tmK, HALF, row, full + s);
@@ -764,10 +771,19 @@ __global__ void __launch_bounds__(192) segment_state_tc_kernel(const __grid_cons
   }
 }
 
-// Shared memory of segment_output_tc_kernel: two stages of (Q, K, V: two boxes each) and one 32 KB tile that holds the
-// bf16 copy of the running state while O = Q S is formed and the rounded score tile P afterwards.
-constexpr int SEG_OUT_STAGE = 6 * BOX_BYTES;
-constexpr int SEG_OUT_SMEM = 2 * SEG_OUT_STAGE + 2 * BOX_BYTES + 1024 + 256;
+// Shared memory of segment_output_tc_kernel.
+//   plain : two stages of (Q, K, V: two boxes each) and one 32 KB tile for the bf16 copy of the running state
+//   SPLIT : two stages of (Q, K), one of V, and the state as two bf16 tiles (leading part and remainder)
+// The rounded score tile P takes the place of the tile's own Q (its remainder that of K) once the MMAs have read them.
+template <bool SPLIT>
+struct SegOutLayout {
+  static constexpr int STAGE = (SPLIT ? 4 : 6) * BOX_BYTES;
+  static constexpr int V = SPLIT ? 2 * STAGE : 4 * BOX_BYTES;      // V of stage s: V + s * V_STRIDE
+  static constexpr int V_STRIDE = SPLIT ? 0 : STAGE;
+  static constexpr int STATE = SPLIT ? 2 * STAGE + 2 * BOX_BYTES : 2 * STAGE;
+  static constexpr int BARS = STATE + (SPLIT ? 4 : 2) * BOX_BYTES;
+  static constexpr int SMEM = BARS + 1024 + 256;
+};
 
 struct SegOutParams {
   int64_t T;
@@ -775,48 +791,69 @@ struct SegOutParams {
   int nseg;
   const float* seg_in;   // [bh][nseg][128][128] state entering each segment
   int64_t n_lr;
-  const __nv_bfloat16* ylr;   // [bh][T][128] long-range rows, bf16 (rows t >= n_lr are added)
+  const __nv_bfloat16* ylr;   // plain: [bh][T][128] long-range rows, bf16 (rows t >= n_lr are added)
+  const float* ylr32;         // SPLIT: the same rows in fp32
   __nv_bfloat16* O;
-  __nv_bfloat16* sin_tiles;   // optional [bh][T/128][128][128]: the bf16 state entering every tile, for a later backward
+  __nv_bfloat16* sin_tiles;   // plain, optional [bh][T/128][128][128]: the bf16 state entering every tile, for a later backward
   int* status;
 };
 
 // One CTA per (segment, head), all 128 output columns.
 //   warps 0-15 : each owns 32 rows x 32 columns of every TMEM tile (state, scores, output)
-//   warp 16    : TMA producer (two stages);   warp 17 : MMA issuer
+//   warp 16    : TMA producer;   warp 17 : MMA issuer
 // TMEM columns: running state S [0,128), scores [128,256), two output accumulators [256,384) and [384,512).
-// Per tile:  Sc = Q Kᵀ ;  O = Q S_bf16 ;  O += tril(Sc)_bf16 V ;  S += Kᵀ V.
+// Per tile b, in issue order:  O = Q S_b ; S += Kᵀ V ; (next tile's) Sc = Q Kᵀ ; O += tril(Sc_b) V.
+// The state's own chain — publish S_b, Q S and Kᵀ V, read S_{b+1} back — does not wait for the score tile: while the
+// tensor core forms the next scores the epilogue warps store P, while it forms P V they publish the next state, and
+// the output rows leave during the next tile's first two products.  (With P and the state sharing one tile, so that
+// every product waited for the previous one's operand, a tile took about 6000 cycles: 0.240 ms at d = 1, 16 heads of
+// 64 K tokens, where this order takes 0.205; its 1.07 GB need 0.161 at the HBM rate.)
+// SPLIT: for blocks that are not whole tiles, whose plans keep fp32 tables: the state and the score tile enter their
+// products as a leading bf16 part plus a bf16 remainder (16 bits of the fp32 value), the long-range rows arrive in
+// fp32, and the rows past a block's end load as zeros and are not stored.  (32 heads of 5056 tokens, d = 3: 0.071 ms,
+// where chunk states, scan, scores, state read and output on the fp32 ALUs took 1.23 ms; 0.12 of it is now the two
+// kernels before this one and itself.)
 constexpr int SEG_EPI_WARPS = 16;
 constexpr int SEG_OUT_THREADS = 32 * (SEG_EPI_WARPS + 2);
 
-__global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
-                                                                const __grid_constant__ CUtensorMap tmK,
-                                                                const __grid_constant__ CUtensorMap tmV,
-                                                                const SegOutParams prm) {
+// tensor maps of Q, K, V as [head][row of the block][128]: a box that runs past the block's rows is filled with zeros
+struct SegOutMaps {
+  CUtensorMap q[2], k[2], v[2];
+};
+
+template <bool SPLIT>
+__global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(const __grid_constant__ SegOutMaps maps,
+                                                                            const SegOutParams prm) {
+  using Lay = SegOutLayout<SPLIT>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint8_t* sSP = smem + 2 * SEG_OUT_STAGE;           // 128 x 128 bf16, two 64-column blocks: S_bf16, then P
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sSP + 2 * BOX_BYTES);
-  uint64_t* full = bars;          // [2] tile operands landed
-  uint64_t* empty = bars + 2;     // [2] tile operands consumed
-  uint64_t* bar_s = bars + 4;     // bf16 state written (one arrival per warp)
-  uint64_t* bar_sc = bars + 5;    // scores in TMEM
-  uint64_t* bar_qs = bars + 6;    // O = Q S finished: the shared tile may take P
-  uint64_t* bar_p = bars + 7;     // P written (one arrival per warp)
-  uint64_t* bar_o = bars + 8;     // output in TMEM and state updated
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 9);
+  uint8_t* sS = smem + Lay::STATE;                   // 128 x 128 bf16 state, two 64-column blocks (SPLIT: then its remainder)
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Lay::BARS);
+  uint64_t* full = bars;           // [2] Q, K (plain: and V) landed
+  uint64_t* empty = bars + 2;      // [2] ... and consumed
+  uint64_t* vfull = bars + 4;      // SPLIT: V landed
+  uint64_t* vempty = bars + 5;     // SPLIT: ... and consumed
+  uint64_t* bar_s = bars + 6;      // bf16 state written (one arrival per warp)
+  uint64_t* bar_sc = bars + 7;     // scores in TMEM
+  uint64_t* bar_scr = bars + 8;    // scores read out (one arrival per warp)
+  uint64_t* bar_qk = bars + 9;     // Q S finished and the state updated: Q, K and the shared state may be overwritten
+  uint64_t* bar_p = bars + 10;     // P written (one arrival per warp)
+  uint64_t* bar_o = bars + 11;     // output complete
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 12);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int seg = blockIdx.x, bh = blockIdx.y;
   int64_t tile0;
   int Lc;
   seg_range(prm.cut, seg, &tile0, &Lc);
+  const int blk = seg < prm.cut.nseg0 ? 0 : 1;
   const WaitCtx wc{cta_abort, prm.status};
   if (threadIdx.x == 0) {
     *cta_abort = 0;
     mbar_init(full, 1); mbar_init(full + 1, 1); mbar_init(empty, 1); mbar_init(empty + 1, 1);
-    mbar_init(bar_s, SEG_EPI_WARPS); mbar_init(bar_sc, 1); mbar_init(bar_qs, 1); mbar_init(bar_p, SEG_EPI_WARPS);
-    mbar_init(bar_o, 1);
+    mbar_init(vfull, 1); mbar_init(vempty, 1);
+    mbar_init(bar_s, SEG_EPI_WARPS); mbar_init(bar_sc, 1); mbar_init(bar_scr, SEG_EPI_WARPS); mbar_init(bar_qk, 1);
+    mbar_init(bar_p, SEG_EPI_WARPS); mbar_init(bar_o, 1);
     fence_barrier_init();
   }
   if (warp == SEG_EPI_WARPS) tmem_alloc(tmem_slot, 512);
@@ -827,18 +864,26 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
   const uint32_t tmem_s = tmem_base, tmem_sc = tmem_base + TILE, tmem_o0 = tmem_base + 2 * TILE;
 
   if (warp == SEG_EPI_WARPS && lane == 0) {
+    const CUtensorMap *mq = &maps.q[blk], *mk = &maps.k[blk], *mv = &maps.v[blk];
+    const int row_first = (int)((tile0 - (blk ? prm.cut.tiles0 : 0)) * TILE);   // row inside the block
     for (int it = 0; it < Lc; ++it) {
       const int s = it & 1;
       if (it >= 2 && !mbar_wait(empty + s, ((it >> 1) - 1) & 1, wc)) break;
-      uint8_t* st = smem + s * SEG_OUT_STAGE;
-      const int row = (int)((int64_t)bh * prm.T + (tile0 + it) * TILE);
-      mbar_expect_tx(full + s, SEG_OUT_STAGE);
-      tma_load_2d(st, &tmQ, 0, row, full + s);
-      tma_load_2d(st + BOX_BYTES, &tmQ, HALF, row, full + s);
-      tma_load_2d(st + 2 * BOX_BYTES, &tmK, 0, row, full + s);
-      tma_load_2d(st + 3 * BOX_BYTES, &tmK, HALF, row, full + s);
-      tma_load_2d(st + 4 * BOX_BYTES, &tmV, 0, row, full + s);
-      tma_load_2d(st + 5 * BOX_BYTES, &tmV, HALF, row, full + s);
+      uint8_t* st = smem + s * Lay::STAGE;
+      uint8_t* sv = smem + Lay::V + s * Lay::V_STRIDE;
+      const int row = row_first + it * TILE;
+      uint64_t* bv = SPLIT ? vfull : full + s;
+      mbar_expect_tx(full + s, Lay::STAGE);
+      tma_load_3d(st, mq, 0, row, bh, full + s);
+      tma_load_3d(st + BOX_BYTES, mq, HALF, row, bh, full + s);
+      tma_load_3d(st + 2 * BOX_BYTES, mk, 0, row, bh, full + s);
+      tma_load_3d(st + 3 * BOX_BYTES, mk, HALF, row, bh, full + s);
+      if (SPLIT) {
+        if (it >= 1 && !mbar_wait(vempty, (it - 1) & 1, wc)) break;
+        mbar_expect_tx(vfull, 2 * BOX_BYTES);
+      }
+      tma_load_3d(sv, mv, 0, row, bh, bv);
+      tma_load_3d(sv + BOX_BYTES, mv, HALF, row, bh, bv);
     }
   } else if (warp == SEG_EPI_WARPS + 1 && lane == 0) {
     constexpr uint32_t idesc_sc = make_idesc(TILE, TILE, 0, 0);   // Q Kᵀ: both K-major
@@ -847,46 +892,75 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
     // Descriptors are built once; inside the loops only constants are added (16-byte units): this lone thread pays
     // the full latency of every instruction it issues.
     constexpr uint32_t BOX16 = BOX_BYTES >> 4;
-    const uint64_t dSP_k = make_desc(smem_u32(sSP), 16, 1024);           // shared tile read K-major (P)
-    const uint64_t dSP_mn = make_desc(smem_u32(sSP), BOX_BYTES, 1024);   // and MN-major (S)
+    const uint64_t dS_mn = make_desc(smem_u32(sS), BOX_BYTES, 1024);
     uint64_t dQ_k[2], dK_k[2], dK_mn[2], dV_mn[2];
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
-      const uint32_t sQ = smem_u32(smem + s * SEG_OUT_STAGE);
+      const uint32_t sQ = smem_u32(smem + s * Lay::STAGE);
       dQ_k[s] = make_desc(sQ, 16, 1024);
       dK_k[s] = make_desc(sQ + 2 * BOX_BYTES, 16, 1024);
       dK_mn[s] = make_desc(sQ + 2 * BOX_BYTES, BOX_BYTES, 1024);
-      dV_mn[s] = make_desc(sQ + 4 * BOX_BYTES, BOX_BYTES, 1024);
+      dV_mn[s] = make_desc(smem_u32(smem + Lay::V + s * Lay::V_STRIDE), BOX_BYTES, 1024);
     }
-    for (int it = 0; it < Lc; ++it) {
-      const int s = it & 1;
-      const uint64_t qk = s ? dQ_k[1] : dQ_k[0], kk_ = s ? dK_k[1] : dK_k[0];
-      const uint64_t kmn = s ? dK_mn[1] : dK_mn[0], vmn = s ? dV_mn[1] : dV_mn[0];
-      const uint32_t tmem_o = tmem_o0 + (it & 1) * TILE;
-      if (!mbar_wait(full + s, (it >> 1) & 1, wc)) break;
+    auto scores = [&](int it) {   // Sc = Q Kᵀ of tile `it`
+      const uint64_t qk = (it & 1) ? dQ_k[1] : dQ_k[0], kk_ = (it & 1) ? dK_k[1] : dK_k[0];
+      if (!mbar_wait(full + (it & 1), (it >> 1) & 1, wc)) return false;
       fence_after_sync();
 #pragma unroll
-      for (int kk = 0; kk < TILE / 16; ++kk) {   // Sc = Q Kᵀ (the score tile was read out before bar_p of the last tile)
+      for (int kk = 0; kk < TILE / 16; ++kk) {
         const uint64_t off = (uint64_t)((kk >> 2) * BOX16 + (kk & 3) * 2);
         mma_bf16(tmem_sc, qk + off, kk_ + off, idesc_sc, kk != 0);
       }
       mma_commit(bar_sc);
-      if (!mbar_wait(bar_s, it & 1, wc)) break;  // bf16 state in the shared tile; output buffer of tile it-2 read out
+      return true;
+    };
+    bool ok = scores(0);
+    for (int it = 0; it < Lc && ok; ++it) {
+      const int s = it & 1;
+      const uint64_t qk = s ? dQ_k[1] : dQ_k[0], kk_ = s ? dK_k[1] : dK_k[0];
+      const uint64_t kmn = s ? dK_mn[1] : dK_mn[0], vmn = s ? dV_mn[1] : dV_mn[0];
+      const uint32_t tmem_o = tmem_o0 + s * TILE;
+      ok = mbar_wait(bar_s, it & 1, wc);   // bf16 state in the shared tile; output buffer of tile it-2 read out
+      if (!ok) break;
       fence_after_sync();
 #pragma unroll
       for (int kk = 0; kk < TILE / 16; ++kk)     // O = Q S
-        mma_bf16(tmem_o, qk + (uint64_t)((kk >> 2) * BOX16 + (kk & 3) * 2), dSP_mn + (uint64_t)(kk * 128), idesc_o, kk != 0);
-      mma_commit(bar_qs);
-      if (!mbar_wait(bar_p, it & 1, wc)) break;
+        mma_bf16(tmem_o, qk + (uint64_t)((kk >> 2) * BOX16 + (kk & 3) * 2), dS_mn + (uint64_t)(kk * 128), idesc_o, kk != 0);
+      if (SPLIT) {
+#pragma unroll
+        for (int kk = 0; kk < TILE / 16; ++kk)   // ... plus Q times the state's remainder
+          mma_bf16(tmem_o, qk + (uint64_t)((kk >> 2) * BOX16 + (kk & 3) * 2), dS_mn + (uint64_t)(2 * BOX16 + kk * 128), idesc_o, 1);
+        ok = mbar_wait(vfull, it & 1, wc);
+        if (!ok) break;
+        fence_after_sync();
+      }
+      if (it + 1 < Lc) {
+#pragma unroll
+        for (int kk = 0; kk < TILE / 16; ++kk)   // S += Kᵀ V
+          mma_bf16(tmem_s, kmn + (uint64_t)(kk * 128), vmn + (uint64_t)(kk * 128), idesc_s, 1);
+      }
+      mma_commit(bar_qk);
+      ok = mbar_wait(bar_scr, it & 1, wc);       // this tile's scores are in registers
+      if (!ok) break;
+      // the next tile's scores first if its rows have landed (they hide the store of P); a late load must not hold up
+      // this tile's last product, which frees the stage for the load after it
+      const bool early = it + 1 < Lc && mbar_test(full + (s ^ 1), ((it + 1) >> 1) & 1);
+      if (early) ok = scores(it + 1);
+      if (ok) ok = mbar_wait(bar_p, it & 1, wc);
+      if (!ok) break;
       fence_after_sync();
 #pragma unroll
-      for (int kk = 0; kk < TILE / 16; ++kk)     // O += P V
-        mma_bf16(tmem_o, dSP_k + (uint64_t)((kk >> 2) * BOX16 + (kk & 3) * 2), vmn + (uint64_t)(kk * 128), idesc_o, 1);
+      for (int kk = 0; kk < TILE / 16; ++kk)     // O += P V (P lies where Q was)
+        mma_bf16(tmem_o, qk + (uint64_t)((kk >> 2) * BOX16 + (kk & 3) * 2), vmn + (uint64_t)(kk * 128), idesc_o, 1);
+      if (SPLIT) {
 #pragma unroll
-      for (int kk = 0; kk < TILE / 16; ++kk)     // S += Kᵀ V
-        mma_bf16(tmem_s, kmn + (uint64_t)(kk * 128), vmn + (uint64_t)(kk * 128), idesc_s, 1);
-      mma_commit(bar_o);
+        for (int kk = 0; kk < TILE / 16; ++kk)   // ... plus the remainder of P (where K was)
+          mma_bf16(tmem_o, kk_ + (uint64_t)((kk >> 2) * BOX16 + (kk & 3) * 2), vmn + (uint64_t)(kk * 128), idesc_o, 1);
+        mma_commit(vempty);
+      }
       mma_commit(empty + s);
+      mma_commit(bar_o);
+      if (it + 1 < Lc && !early) ok = scores(it + 1);
     }
   } else if (warp < SEG_EPI_WARPS) {
     // Sixteen warps: warp w owns the lane quarter w % 4 (32 rows) and the column quarter w / 4 (32 columns) of every
@@ -897,32 +971,54 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t col0 = cq * 32;
     // this thread's 64 bytes (four 16-byte chunks) of its row in the 64-column block that holds its columns
-    uint8_t* my_tile = sSP + (cq >> 1) * BOX_BYTES + m * 128;
+    const uint32_t my_off = (cq >> 1) * BOX_BYTES + m * 128;
     const int ch0 = (cq & 1) * 4;
-    auto store_row = [&](const uint4 (&pk)[4]) {
+    auto store_row = [&](uint8_t* tile, const uint4 (&pk)[4]) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(my_tile + (((ch0 + c) ^ (m & 7)) << 4)) = pk[c];
+      for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(tile + my_off + (((ch0 + c) ^ (m & 7)) << 4)) = pk[c];
+    };
+    auto pack_row = [&](const float (&f)[32], uint4 (&pk)[4]) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        pk[c] = make_uint4(pack_bf16(f[8 * c], f[8 * c + 1]), pack_bf16(f[8 * c + 2], f[8 * c + 3]),
+                           pack_bf16(f[8 * c + 4], f[8 * c + 5]), pack_bf16(f[8 * c + 6], f[8 * c + 7]));
+    };
+    // f minus its bf16 rounding (exact in fp32)
+    auto remainder = [&](float (&f)[32], const uint4 (&pk)[4]) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const uint32_t w[4] = {pk[c].x, pk[c].y, pk[c].z, pk[c].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          f[8 * c + 2 * e] -= __uint_as_float(w[e] << 16);
+          f[8 * c + 2 * e + 1] -= __uint_as_float(w[e] & 0xffff0000u);
+        }
+      }
     };
     // bf16 copy of this thread's 32 state columns into the shared tile (and, when a backward will want the state
     // entering tile `tile`, into the per-tile table as well: 64 bytes of row m)
     auto publish_state = [&](const uint32_t (&v)[32], int64_t tile) {
+      float f[32];
       uint4 pk[4];
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
-        pk[c] = make_uint4(pack_bf16(__uint_as_float(v[8 * c]), __uint_as_float(v[8 * c + 1])),
-                           pack_bf16(__uint_as_float(v[8 * c + 2]), __uint_as_float(v[8 * c + 3])),
-                           pack_bf16(__uint_as_float(v[8 * c + 4]), __uint_as_float(v[8 * c + 5])),
-                           pack_bf16(__uint_as_float(v[8 * c + 6]), __uint_as_float(v[8 * c + 7])));
-      store_row(pk);
-      if (prm.sin_tiles) {
-        __nv_bfloat16* dst = prm.sin_tiles + (((int64_t)bh * (prm.T / TILE) + tile) * TILE + m) * TILE + col0;
-        st_global_v8(dst, pk[0].x, pk[0].y, pk[0].z, pk[0].w, pk[1].x, pk[1].y, pk[1].z, pk[1].w);
-        st_global_v8(dst + 16, pk[2].x, pk[2].y, pk[2].z, pk[2].w, pk[3].x, pk[3].y, pk[3].z, pk[3].w);
+      for (int e = 0; e < 32; ++e) f[e] = __uint_as_float(v[e]);
+      pack_row(f, pk);
+      store_row(sS, pk);
+      if (SPLIT) {
+        uint4 lo[4];
+        remainder(f, pk);
+        pack_row(f, lo);
+        store_row(sS + 2 * BOX_BYTES, lo);
       }
       fence_proxy_async();
       fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_s);   // one arrival per warp: 512 arrivals on one barrier serialise
+      if (!SPLIT && prm.sin_tiles) {
+        __nv_bfloat16* dst = prm.sin_tiles + (((int64_t)bh * (prm.T / TILE) + tile) * TILE + m) * TILE + col0;
+        st_global_v8(dst, pk[0].x, pk[0].y, pk[0].z, pk[0].w, pk[1].x, pk[1].y, pk[1].z, pk[1].w);
+        st_global_v8(dst + 16, pk[2].x, pk[2].y, pk[2].z, pk[2].w, pk[3].x, pk[3].y, pk[3].z, pk[3].w);
+      }
     };
     {  // state entering the segment: global fp32 -> TMEM (accumulator) and the shared tile
       uint32_t v[32];
@@ -936,51 +1032,53 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
       tmem_st_wait();
       publish_state(v, tile0);
     }
+    const int64_t row_first = seg_tile_row(prm.cut, tile0), row_end = blk ? prm.cut.rows : prm.cut.rows0;
     for (int it = 0; it < Lc; ++it) {
-      // --- scores of this tile -> masked bf16 P (registers), stored once O = Q S has consumed the shared tile ---
+      uint8_t* stage = smem + (it & 1) * Lay::STAGE;
+      // --- scores of this tile -> masked bf16 P (registers), stored once Q and K have been consumed ---
       if (!mbar_wait(bar_sc, it & 1, wc)) break;
       fence_after_sync();
-      uint4 pk[4];
+      uint4 pk[4], plo[4];
       {
         uint32_t v[32];
+        float f[32];
         tmem_ld32(tmem_sc + lane_base + col0, v);
         tmem_ld_wait();
+        fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_scr);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          uint32_t w[4];
-#pragma unroll
-          for (int h2 = 0; h2 < 4; ++h2) {
-            const int k0 = (int)col0 + i * 8 + h2 * 2;
-            const float lo = (k0 <= m) ? __uint_as_float(v[i * 8 + h2 * 2]) : 0.f;
-            const float hi = (k0 + 1 <= m) ? __uint_as_float(v[i * 8 + h2 * 2 + 1]) : 0.f;
-            w[h2] = pack_bf16(lo, hi);
-          }
-          pk[i] = make_uint4(w[0], w[1], w[2], w[3]);
-        }
+        for (int e = 0; e < 32; ++e) f[e] = ((int)col0 + e <= m) ? __uint_as_float(v[e]) : 0.f;
+        pack_row(f, pk);
+        if (SPLIT) { remainder(f, pk); pack_row(f, plo); }
       }
-      if (!mbar_wait(bar_qs, it & 1, wc)) break;
-      store_row(pk);
+      if (!mbar_wait(bar_qk, it & 1, wc)) break;
+      fence_after_sync();
+      store_row(stage, pk);
+      if (SPLIT) store_row(stage + 2 * BOX_BYTES, plo);
       fence_proxy_async();
       fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_p);
-      // --- long-range rows of this tile, fetched while the MMAs run ---
-      const int64_t t = (tile0 + it) * TILE + m;
-      const bool add_lr = t >= prm.n_lr;
-      uint4 y[4];                                    // 32 bf16 values
-      if (add_lr) {
-        const uint4* y4 = reinterpret_cast<const uint4*>(prm.ylr + ((int64_t)bh * prm.T + t) * TILE + col0);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) y[i] = __ldg(y4 + i);
-      }
-      if (!mbar_wait(bar_o, it & 1, wc)) break;
-      fence_after_sync();
-      if (it + 1 < Lc) {  // the state now includes this tile: publish it for the next one first (critical path)
+      if (it + 1 < Lc) {  // the state now includes this tile: publish it for the next one
         uint32_t v[32];
         tmem_ld32(tmem_s + lane_base + col0, v);
         tmem_ld_wait();
         publish_state(v, tile0 + it + 1);
       }
+      // --- long-range rows of this tile, fetched while the MMAs run ---
+      const int64_t t = row_first + (int64_t)it * TILE + m;
+      const bool live = !SPLIT || t < row_end;
+      const bool add_lr = live && t >= prm.n_lr;
+      uint4 y[SPLIT ? 8 : 4];                        // 32 bf16 or fp32 values
+      if (add_lr) {
+        const uint4* y4 = SPLIT ? reinterpret_cast<const uint4*>(prm.ylr32 + ((int64_t)bh * prm.T + t) * TILE + col0)
+                                : reinterpret_cast<const uint4*>(prm.ylr + ((int64_t)bh * prm.T + t) * TILE + col0);
+#pragma unroll
+        for (int i = 0; i < (SPLIT ? 8 : 4); ++i) y[i] = __ldg(y4 + i);
+      }
+      if (!mbar_wait(bar_o, it & 1, wc)) break;
+      fence_after_sync();
       __nv_bfloat16* dst = prm.O + ((int64_t)bh * prm.T + t) * TILE + col0;
       const uint32_t tmem_o = tmem_o0 + (it & 1) * TILE;
       uint32_t v[32];
@@ -993,20 +1091,28 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
 #pragma unroll
         for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[i * 8 + e]);
         if (add_lr) {
-          const uint32_t yy[4] = {y[i].x, y[i].y, y[i].z, y[i].w};
+          if (SPLIT) {
+            const uint4 a = y[2 * i], c = y[SPLIT ? 2 * i + 1 : 0];
+            f[0] += __uint_as_float(a.x); f[1] += __uint_as_float(a.y); f[2] += __uint_as_float(a.z); f[3] += __uint_as_float(a.w);
+            f[4] += __uint_as_float(c.x); f[5] += __uint_as_float(c.y); f[6] += __uint_as_float(c.z); f[7] += __uint_as_float(c.w);
+          } else {
+            const uint32_t yy[4] = {y[i].x, y[i].y, y[i].z, y[i].w};
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            f[2 * e] += __uint_as_float(yy[e] << 16);
-            f[2 * e + 1] += __uint_as_float(yy[e] & 0xffff0000u);
+            for (int e = 0; e < 4; ++e) {
+              f[2 * e] += __uint_as_float(yy[e] << 16);
+              f[2 * e + 1] += __uint_as_float(yy[e] & 0xffff0000u);
+            }
           }
         }
         w[4 * i] = pack_bf16(f[0], f[1]); w[4 * i + 1] = pack_bf16(f[2], f[3]);
         w[4 * i + 2] = pack_bf16(f[4], f[5]); w[4 * i + 3] = pack_bf16(f[6], f[7]);
       }
+      if (live) {
 #pragma unroll
-      for (int h8 = 0; h8 < 2; ++h8)   // whole 32-byte sectors
-        st_global_v8(dst + 16 * h8, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
-                     w[8 * h8 + 5], w[8 * h8 + 6], w[8 * h8 + 7]);
+        for (int h8 = 0; h8 < 2; ++h8)   // whole 32-byte sectors
+          st_global_v8(dst + 16 * h8, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
+                       w[8 * h8 + 5], w[8 * h8 + 6], w[8 * h8 + 7]);
+      }
     }
   }
   fence_before_sync();
@@ -1452,6 +1558,20 @@ bool make_map(CUtensorMap* map, const void* base, uint64_t rows, int box_rows = 
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Rows of one block of every head: [heads][rows][128] bf16 with `head_rows` rows from head to head, box = 64 columns x
+// 128 rows; rows past the block's end read as zeros.
+bool make_block_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t head_rows, uint64_t heads) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  const cuuint64_t dims[3] = {(cuuint64_t)TILE, (cuuint64_t)rows, (cuuint64_t)heads};
+  const cuuint64_t strides[2] = {(cuuint64_t)TILE * 2, (cuuint64_t)head_rows * TILE * 2};
+  const cuuint32_t box[3] = {(cuuint32_t)HALF, (cuuint32_t)TILE, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace
 
 // bf16 matrix [rows, inner] row-major; box = box_inner x box_rows; optional 128-byte swizzle (box_inner = 64 then).
@@ -1685,9 +1805,9 @@ void smat_segment_counts(int64_t tiles0, int64_t tiles1, int bh, int L, int* nse
     const int64_t rounds = ((n0 + n1) * bh + sms - 1) / sms;
     return (double)rounds * ((double)lmax + overhead);
   };
-  int64_t best0 = tiles0 / L, best1 = tiles1 / L;
+  const int64_t max0 = tiles0 / 2 > 0 ? tiles0 / 2 : 1, max1 = tiles1 > 1 ? tiles1 / 2 : tiles1;
+  int64_t best0 = tiles0 >= L ? tiles0 / L : 1, best1 = tiles1 >= L ? tiles1 / L : tiles1 > 0;
   double best = cost(best0, best1) * 0.96;
-  const int64_t max0 = tiles0 / 2 > 0 ? tiles0 / 2 : 1, max1 = tiles1 / 2;
   for (int64_t n0 = 1; n0 <= max0 && n0 <= 512; ++n0) {
     if ((tiles0 + n0 - 1) / n0 > 16) continue;
     // block 1 gets the count that gives it the same longest segment, or one more segment
@@ -1702,14 +1822,22 @@ void smat_segment_counts(int64_t tiles0, int64_t tiles1, int bh, int L, int* nse
   *nseg0 = (int)best0; *nseg1 = (int)best1;
 }
 
-cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* totals, int64_t tiles0, int64_t tiles1,
+static SegCut segment_cut(int64_t rows0, int64_t rows1, int nseg0, int nseg1) {
+  SegCut c;
+  c.nseg0 = nseg0; c.nseg = nseg0 + nseg1;
+  c.tiles0 = (rows0 + TILE - 1) / TILE; c.tiles1 = (rows1 + TILE - 1) / TILE;
+  c.rows0 = rows0; c.rows = rows0 + rows1;
+  return c;
+}
+
+cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* totals, int64_t rows0, int64_t rows1,
                                          int nseg0, int nseg1, int bh, int* status, cudaStream_t st) {
-  const int64_t T = (tiles0 + tiles1) * TILE;
+  const int64_t T = rows0 + rows1;
   CUtensorMap tmK, tmV;
   if (!make_map(&tmK, K, (uint64_t)bh * T) || !make_map(&tmV, V, (uint64_t)bh * T)) return cudaErrorInvalidValue;
   SegStateParams prm;
   prm.T = T; prm.nseg = nseg0 + nseg1; prm.totals = totals; prm.status = status;
-  prm.cut.nseg0 = nseg0; prm.cut.nseg = nseg0 + nseg1; prm.cut.tiles0 = tiles0; prm.cut.tiles1 = tiles1;
+  prm.cut = segment_cut(rows0, rows1, nseg0, nseg1);
   cudaError_t err =
       cudaFuncSetAttribute(segment_state_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SEG_STATE_SMEM);
   if (err != cudaSuccess) return err;
@@ -1719,23 +1847,31 @@ cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* to
 }
 
 cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const void* V, const float* seg_in,
-                                          const void* ylr_bf16, int64_t n_lr, void* O, int64_t tiles0, int64_t tiles1,
+                                          const void* ylr, int ylr_f32, int64_t n_lr, void* O, int64_t rows0, int64_t rows1,
                                           int nseg0, int nseg1, int bh, int* status, cudaStream_t st, void* sin_tiles) {
-  const int64_t T = (tiles0 + tiles1) * TILE;
-  CUtensorMap tmQ, tmK, tmV;
-  if (!make_map(&tmQ, Q, (uint64_t)bh * T) || !make_map(&tmK, K, (uint64_t)bh * T) ||
-      !make_map(&tmV, V, (uint64_t)bh * T))
-    return cudaErrorInvalidValue;
+  const int64_t T = rows0 + rows1;
+  SegOutMaps maps;
+  const void* src[3] = {Q, K, V};
+  CUtensorMap* dst[3] = {maps.q, maps.k, maps.v};
+  for (int i = 0; i < 3; ++i) {
+    const __nv_bfloat16* base = static_cast<const __nv_bfloat16*>(src[i]);
+    if (!make_block_map(&dst[i][0], base, (uint64_t)rows0, (uint64_t)T, (uint64_t)bh)) return cudaErrorInvalidValue;
+    dst[i][1] = dst[i][0];
+    if (rows1 && !make_block_map(&dst[i][1], base + rows0 * TILE, (uint64_t)rows1, (uint64_t)T, (uint64_t)bh)) return cudaErrorInvalidValue;
+  }
   SegOutParams prm;
-  prm.T = T; prm.nseg = nseg0 + nseg1; prm.seg_in = seg_in; prm.n_lr = n_lr; prm.ylr = static_cast<const __nv_bfloat16*>(ylr_bf16);
-  prm.cut.nseg0 = nseg0; prm.cut.nseg = nseg0 + nseg1; prm.cut.tiles0 = tiles0; prm.cut.tiles1 = tiles1;
+  prm.T = T; prm.nseg = nseg0 + nseg1; prm.seg_in = seg_in; prm.n_lr = n_lr;
+  prm.ylr = static_cast<const __nv_bfloat16*>(ylr);
+  prm.ylr32 = static_cast<const float*>(ylr);
+  prm.cut = segment_cut(rows0, rows1, nseg0, nseg1);
   prm.O = static_cast<__nv_bfloat16*>(O);
   prm.sin_tiles = static_cast<__nv_bfloat16*>(sin_tiles);
   prm.status = status;
-  cudaError_t err =
-      cudaFuncSetAttribute(segment_output_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SEG_OUT_SMEM);
+  auto kernel = ylr_f32 ? segment_output_tc_kernel<true> : segment_output_tc_kernel<false>;
+  const int smem = ylr_f32 ? SegOutLayout<true>::SMEM : SegOutLayout<false>::SMEM;
+  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
   dim3 grid((unsigned)prm.nseg, (unsigned)bh);
-  segment_output_tc_kernel<<<grid, SEG_OUT_THREADS, SEG_OUT_SMEM, st>>>(tmQ, tmK, tmV, prm);
+  kernel<<<grid, SEG_OUT_THREADS, smem, st>>>(maps, prm);
   return cudaGetLastError();
 }

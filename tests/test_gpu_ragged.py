@@ -1,0 +1,71 @@
+"""Forward passes whose blocks are not whole 128-token tiles (bf16, 128-wide heads): tensor-core causal branch with
+partial last tiles and fp32 tables, against the fp64 dense-mask oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import smat_oracle as so
+from paper_2609_36062_b200 import binding, synth
+from tests.helpers import device_inputs, rel_err, to_numpy64
+
+pytestmark = pytest.mark.gpu
+
+# (d, T, chunk): last tiles of 16, 32, 64, 112 and 127-odd rows, one-tile blocks, blocks longer and shorter than a tile,
+# a whole first block with a partial second one, several segments per block, d = 1 with a partial last tile
+CASES = [(2, 32, 16), (1, 16, 16), (2, 128, 64), (3, 224, 16), (3, 320, 32), (1, 336, 16), (2, 320, 64), (4, 1120, 16),
+         (3, 1472, 64), (2, 2368, 64), (1, 2624, 64), (3, 4288, 64)]
+
+
+def _case(d, T, c):
+    w = synth.Workload("ragged", d, 1, 3, T, 128, 128, c, "bf16", "normalised", 17 + T)
+    host, dev = device_inputs(w)
+    return w, host, dev
+
+
+@pytest.mark.parametrize("d,T,c", CASES)
+def test_partial_tiles_match_the_dense_oracle(d, T, c):
+    w, host, dev = _case(d, T, c)
+    plan = binding.SmatPlan(1, 3, T, 128, 128, d, c, "bf16")
+    assert plan.uses_tensor_cores() and plan.type_table_element_bytes() == 4
+    O = plan.forward(dev["q"], dev["k"], dev["v"])
+    plan.check_status()
+    alu = binding.SmatPlan(1, 3, T, 128, 128, d, c, "bf16", flags=binding.FLAG_SIMT_ONLY)
+    A = alu.forward(dev["q"], dev["k"], dev["v"])
+    M = so.dense_mask(T, c, d)
+    for h in range(w.bh):
+        Q64, K64, V64 = (synth.as_float64(w, host[x][h]) for x in ("q", "k", "v"))
+        ref = so.forward_dense(Q64, K64, V64, M)
+        # the fp32 tables and the split operands leave the rounding of the stored output, half a bf16 ulp: 2^-8 of the
+        # largest value and no more
+        assert rel_err(to_numpy64(O[0, h]), ref) <= 2.0 ** -8
+        assert np.linalg.norm(to_numpy64(O[0, h]) - ref) <= 1.02 * np.linalg.norm(to_numpy64(A[0, h]) - ref)
+
+
+def test_rows_past_a_block_do_not_reach_it():
+    """Non-finite keys and values behind a block's end (of the recent block, of the next head) stay out of its rows."""
+    w, _, dev = _case(3, 1472, 64)
+    plan = binding.SmatPlan(1, 3, w.T, 128, 128, 3, 64, "bf16")
+    n = plan.geometry().n
+    clean = plan.forward(dev["q"], dev["k"], dev["v"])
+    k, v = dev["k"].clone(), dev["v"].clone()
+    k[0, 0, n:], v[0, 0, n:] = float("inf"), float("nan")
+    k[0, 2], v[0, 2] = float("nan"), float("inf")
+    dirty = plan.forward(dev["q"], k, v)
+    plan.check_status()
+    assert torch.equal(dirty[0, 0, :n], clean[0, 0, :n]) and torch.equal(dirty[0, 1], clean[0, 1])
+
+
+def test_routed_tokens_of_no_group_add_nothing():
+    w, host, dev = _case(3, 1120, 16)
+    plan = binding.SmatPlan(1, 3, w.T, 128, 128, 3, 16, "bf16")
+    geo = so.geometry(w.T, 16, 3)
+    rng = np.random.default_rng(2)
+    prof = rng.integers(-2, geo.P, (3, geo.n)).astype(np.int32)
+    typ = rng.integers(0, geo.B + 3, (3, geo.m)).astype(np.int32)
+    O = plan.forward(dev["q"], dev["k"], dev["v"], prof=torch.from_numpy(prof).cuda(), type=torch.from_numpy(typ).cuda())
+    plan.check_status()
+    rows = np.arange(w.T)
+    for h in range(3):
+        Q64, K64, V64 = (synth.as_float64(w, host[x][h]) for x in ("q", "k", "v"))
+        ref = so.routed_forward_rows(Q64, K64, V64, geo, prof[h], typ[h], rows)
+        assert rel_err(to_numpy64(O[0, h]), ref) <= 2.0 ** -8
