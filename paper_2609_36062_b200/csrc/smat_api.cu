@@ -4,6 +4,7 @@
 
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 
 #include "../../include/smat.h"
@@ -20,8 +21,8 @@ struct smat_plan {
   SmatGeo geo;
   int64_t rp;          // state entries
   // workspace layout (byte offsets, 256-byte aligned)
-  size_t off_status, off_sin, off_F, off_U, off_acc, off_tileA, off_W, off_fwd_end;
-  size_t off_dbar, off_ubar, off_fbar, off_tileG, off_bwd_end;
+  size_t off_status, off_sin, off_F, off_U, off_acc, off_W, off_fwd_end;
+  size_t off_dbar, off_ubar, off_fbar, off_acc2, off_bwd_end;
   size_t off_plist, off_poffs, off_tlist, off_toffs;   // token lists of user-supplied routing (int32)
   size_t off_lr3;         // tensor-core backward: third buffer of bf16 long-range rows (the first two share off_acc)
   size_t off_sin_tiles;   // KEEP_FORWARD_TABLES on tensor-core plans: the bf16 state entering every tile, left by the forward
@@ -118,13 +119,6 @@ smat_status build_geometry(SmatGeo* g, int64_t T, int64_t c, int d, int q_overri
   return SMAT_OK;
 }
 
-SmatOperand operand(const void* ptr, int bf16, int64_t s_bh, int64_t s_g, int64_t s0, int64_t s1, int tok0 = 0,
-                    int tok1 = 0) {
-  SmatOperand o; o.ptr = ptr; o.bf16 = bf16; o.s_bh = s_bh; o.s_g = s_g; o.s0 = s0; o.s1 = s1;
-  o.tok0 = tok0; o.tok1 = tok1;
-  return o;
-}
-
 SmatGroupSpec group(const smat_plan* pl, int mode) {
   SmatGroupSpec s; s.mode = mode; s.n = pl->geo.n; s.T = pl->T; s.c = pl->c;
   s.period = mode == SMAT_GM_PROFILE ? pl->geo.P : pl->geo.B;
@@ -212,73 +206,88 @@ int64_t group_count(const smat_plan* pl, int mode) {
 }
 
 // state[bh][g] (r x p, fp32) = Σ_{tokens of g} a_tᵀ b_t   with a: [T, r], b: [T, p]
+SmatPoolJob pool_job(const Ctx& cx, int mode, const void* a, const void* b, float* state) {
+  SmatPoolJob j;
+  j.a = a; j.b = b; j.state = state; j.grp = group(cx, mode); j.groups = group_count(cx.pl, mode);
+  return j;
+}
+void pool(Ctx& cx, const char* name, std::initializer_list<SmatPoolJob> jobs) {
+  const smat_plan* pl = cx.pl;
+  SmatPoolArgs a{};
+  for (const SmatPoolJob& j : jobs) a.job[a.jobs++] = j;
+  SMAT_TRY(cx, name, smat_launch_pool(a, pl->dtype == SMAT_BF16, pl->T, pl->bh, pl->r, pl->p, cx.st));
+}
 void outer_sum(Ctx& cx, const char* name, int mode, const void* a, const void* b, float* state) {
-  const smat_plan* pl = cx.pl;
-  const int bf = pl->dtype == SMAT_BF16;
-  const int64_t G = group_count(pl, mode);
-  SMAT_TRY(cx, name, smat_launch_pool(a, b, bf, state, group(cx, mode), pl->T, G, pl->bh, pl->r, pl->p, cx.st));
+  pool(cx, name, {pool_job(cx, mode, a, b, state)});
 }
 
-// out[bh][t] (+)= x_t · state_g(t)  (transposed = 0: x: [T, r] contracts the first state index, out: [T, p];
-//                                     transposed = 1: x: [T, p] contracts the second state index, out: [T, r])
-// `out_final` (plan dtype) receives acc_in + product when non-null; otherwise the fp32 accumulator is updated.
-void state_read(Ctx& cx, const char* name, int mode, const void* x, const float* state, int transposed, const float* acc_in,
-                float* acc_out, void* out_final) {
+// out[bh][t] = x_t · state_g(t), fp32 rows (transposed = 0: x: [T, r] contracts the first state index, out: [T, p];
+//                                           transposed = 1: x: [T, p] contracts the second state index, out: [T, r])
+SmatReadJob read_job(const Ctx& cx, int mode, const void* x, const float* state, int transposed, float* out) {
+  SmatReadJob j;
+  j.x = x; j.state = state; j.out = out; j.grp = group(cx, mode); j.groups = group_count(cx.pl, mode); j.trans = transposed;
+  return j;
+}
+void state_read(Ctx& cx, const char* name, std::initializer_list<SmatReadJob> jobs) {
   const smat_plan* pl = cx.pl;
-  const int bf = pl->dtype == SMAT_BF16;
-  const int64_t G = group_count(pl, mode);
-  const int kdim = transposed ? pl->p : pl->r, odim = transposed ? pl->r : pl->p;
-  if (mode != SMAT_GM_CHUNK && !out_final) {  // a handful of tokens per state: stream the state once
-    SMAT_TRY(cx, name, smat_launch_state_read(x, bf, state, transposed, acc_in, acc_out, group(cx, mode), pl->T, G,
-                                              pl->bh, pl->r, pl->p, reinterpret_cast<int*>(cx.ws + pl->off_status),
-                                              cx.st));
-    return;
+  SmatReadArgs a{};
+  for (const SmatReadJob& j : jobs) a.job[a.jobs++] = j;
+  SMAT_TRY(cx, name, smat_launch_state_read(a, pl->dtype == SMAT_BF16, pl->T, pl->bh, pl->r, pl->p,
+                                            reinterpret_cast<int*>(cx.ws + pl->off_status), cx.st));
+}
+
+// The within-chunk tiles of one output (see tile_rows_kernel); acc rows acc_lo <= t < acc_hi are added.
+SmatTileJob tile_job(const void* p1, const void* p2, const void* p3, const void* p4, const float* st, int st_trans, int upper,
+                     const float* acc, int64_t acc_lo, int64_t acc_hi, void* out) {
+  SmatTileJob j;
+  j.p1 = p1; j.p2 = p2; j.p3 = p3; j.p4 = p4; j.st = st; j.st_trans = st_trans; j.upper = upper;
+  j.acc = acc; j.acc_lo = acc_lo; j.acc_hi = acc_hi; j.out = out;
+  return j;
+}
+void tile_rows(Ctx& cx, const char* name, int score_dim, int out_dim, std::initializer_list<SmatTileJob> jobs, const float* lam) {
+  const smat_plan* pl = cx.pl;
+  SmatTileArgs a{};
+  for (const SmatTileJob& j : jobs) a.job[a.jobs++] = j;
+  a.T = pl->T; a.c = (int)pl->c; a.NC = (int)pl->NC; a.lam = lam;
+  SMAT_TRY(cx, name, smat_launch_tile_rows(a, pl->dtype == SMAT_BF16, score_dim, out_dim, pl->bh, cx.st));
+}
+// dQ, dK (score products over d_v, d_k columns out) and dV (the other way round): one launch when d_k = d_v.
+void adjoint_tiles(Ctx& cx, const char* name, const SmatTileJob& dq, const SmatTileJob& dk, const SmatTileJob& dv,
+                   const float* lam) {
+  const smat_plan* pl = cx.pl;
+  if (pl->r == pl->p) {
+    tile_rows(cx, name, pl->p, pl->r, {dq, dk, dv}, lam);
+  } else {
+    tile_rows(cx, name, pl->p, pl->r, {dq, dk}, lam);
+    tile_rows(cx, name, pl->r, pl->p, {dv}, lam);
   }
-  SmatGemmArgs g{};
-  g.A = operand(x, bf, pl->T * kdim, 0, kdim, 1, 1, 0);
-  g.B = transposed ? operand(state, 0, G * pl->rp, pl->rp, 1, pl->p) : operand(state, 0, G * pl->rp, pl->rp, pl->p, 1);
-  g.Cin = operand(acc_in, 0, pl->T * odim, 0, odim, 1, 1, 0);
-  g.C = out_final ? operand(out_final, bf, pl->T * odim, 0, odim, 1, 1, 0)
-                  : operand(acc_out, 0, pl->T * odim, 0, odim, 1, 1, 0);
-  g.K = kdim; g.N = odim; g.tokM = 1; g.grp = group(cx, mode);
-  SMAT_TRY(cx, name, smat_launch_gemm(g, (int)max_group_tokens(pl, mode), odim, G, pl->bh, cx.st));
 }
 
-// tile[bh][chunk] (c x c, fp32) = tril(X_b Y_bᵀ), X, Y: [T, dim]
-void tril_scores(Ctx& cx, const char* name, const void* x, const void* y, int dim, float* tile, const float* lam = nullptr) {
-  const smat_plan* pl = cx.pl;
-  const int bf = pl->dtype == SMAT_BF16;
-  SmatGemmArgs g{};
-  g.A = operand(x, bf, pl->T * dim, 0, dim, 1, 1, 0);
-  g.B = operand(y, bf, pl->T * dim, 0, 1, dim, 0, 1);
-  g.C = operand(tile, 0, pl->NC * pl->c * pl->c, pl->c * pl->c, pl->c, 1);
-  g.K = dim; g.tokM = 1; g.tokN = 1; g.tril = 1; g.grp = group(pl, SMAT_GM_CHUNK); g.lam = lam;
-  SMAT_TRY(cx, name, smat_launch_gemm(g, (int)pl->c, (int)pl->c, pl->NC, pl->bh, cx.st));
-}
-
-// out[bh][t in chunk] = acc_in + tile_b(ᵀ) · Y_b     (tile c x c; Y: [T, dim])
-void tile_apply(Ctx& cx, const char* name, const float* tile, int tile_transposed, const void* y, int dim, const float* acc_in,
-                float* acc_out, void* out_final) {
-  const smat_plan* pl = cx.pl;
-  const int bf = pl->dtype == SMAT_BF16;
-  const int64_t cc = pl->c * pl->c;
-  SmatGemmArgs g{};
-  g.A = tile_transposed ? operand(tile, 0, pl->NC * cc, cc, 1, pl->c) : operand(tile, 0, pl->NC * cc, cc, pl->c, 1);
-  g.B = operand(y, bf, pl->T * dim, 0, dim, 1, 1, 0);
-  g.Cin = operand(acc_in, 0, pl->T * dim, 0, dim, 1, 1, 0);
-  g.C = out_final ? operand(out_final, bf, pl->T * dim, 0, dim, 1, 1, 0)
-                  : operand(acc_out, 0, pl->T * dim, 0, dim, 1, 1, 0);
-  g.N = dim; g.tokM = 1; g.tokK = 1; g.grp = group(pl, SMAT_GM_CHUNK);
-  SMAT_TRY(cx, name, smat_launch_gemm(g, (int)pl->c, dim, pl->NC, pl->bh, cx.st));
-}
-
-void scan_states(Ctx& cx, const char* name, float* S, int reverse) {
+SmatScanJob scan_job(const Ctx& cx, float* S, int reverse) {
   const smat_plan* pl = cx.pl;
   const int64_t ncd = pl->geo.n / pl->c;
-  if (pl->geo.dense_G)  // d = 1: U_0 = F_0 is exactly the carry across the boundary, so the scan runs through
-    SMAT_TRY(cx, name, smat_launch_scan(S, pl->rp, pl->NC, pl->bh, 0, pl->NC, 0, 0, reverse, cx.st));
-  else
-    SMAT_TRY(cx, name, smat_launch_scan(S, pl->rp, pl->NC, pl->bh, 0, ncd, ncd, pl->NC, reverse, cx.st));
+  SmatScanJob j;
+  j.S = S; j.reverse = reverse; j.lo0 = 0;
+  if (pl->geo.dense_G) {  // d = 1: U_0 = F_0 is exactly the carry across the boundary, so the scan runs through
+    j.hi0 = pl->NC; j.lo1 = j.hi1 = 0;
+  } else {
+    j.hi0 = ncd; j.lo1 = ncd; j.hi1 = pl->NC;
+  }
+  return j;
+}
+void scan_states(Ctx& cx, const char* name, std::initializer_list<SmatScanJob> jobs) {
+  const smat_plan* pl = cx.pl;
+  SmatScanArgs a{};
+  for (const SmatScanJob& j : jobs) a.job[a.jobs++] = j;
+  SMAT_TRY(cx, name, smat_launch_scan(a, pl->rp, pl->NC, pl->bh, cx.st));
+}
+// Exclusive prefix sums of the segment totals of both blocks.
+void scan_segments(Ctx& cx, float* seg, int64_t nseg0, int64_t nseg) {
+  const smat_plan* pl = cx.pl;
+  SmatScanArgs a{};
+  a.jobs = 1;
+  a.job[0] = SmatScanJob{seg, 0, nseg0, nseg0, nseg, 0};
+  SMAT_TRY(cx, "segment_scan", smat_launch_scan(a, pl->rp, nseg, pl->bh, cx.st));
 }
 
 smat_status check_common(const smat_plan* pl, const void* ws, size_t ws_bytes, int for_backward) {
@@ -314,17 +323,6 @@ void tabulate_tc(Ctx& cx, const char* name, const void* in, void* out, int trans
   SMAT_TRY(cx, name, smat_launch_tabulate_tc(in, out, cx.ws + pl->off_W, pl->geo, pl->rp, pl->bh, transpose,
                                              reinterpret_cast<int*>(cx.ws + pl->off_status), cx.st, &launches));
   cx.launches += launches - 1;
-}
-
-// Steps 2-3 and 5-6 of Algorithm 1: the tables S_in, F, U.
-void build_forward_tables(Ctx& cx, const void* K, const void* V) {
-  const smat_plan* pl = cx.pl;
-  if (!pl->geo.dense_G) {
-    outer_sum(cx, "pool", SMAT_GM_PROFILE, K, V, cx.f(pl->off_F));                                         // step 2
-    tabulate(cx, "tabulate", cx.f(pl->off_F), cx.f(pl->off_U), 0);                                 // step 3
-  }
-  outer_sum(cx, "chunk_state", SMAT_GM_CHUNK, K, V, cx.f(pl->off_sin));                                           // step 5
-  scan_states(cx, "scan", cx.f(pl->off_sin), 0);                                                           // step 6
 }
 
 // Steps 2-3 of Algorithm 1 alone, as the plan's forward runs them: the type table U ends in the workspace at the
@@ -420,12 +418,11 @@ smat_status smat_plan_create(smat_plan** out, int batch, int heads, int64_t T, i
   pl->ubar_bf16 = pl->ubar_tc && ((g.D == 1 && fbar_by_read) || pl->tab_tc);   // d = 2: F̄ is Ū itself
   pl->fbar_bf16 = pl->tc && !g.dense_G && (pl->tab_tc || (g.D == 1 ? pl->ubar_bf16 : fbar_by_read));
   // Workspace regions, each sized for the element type the plan stores there.  Tensor-core plans keep the causal
-  // states per 128-token tile in bf16 (or, in the two-level form, fewer fp32 segment states in the same region) and
-  // have no score-tile buffers; the fp32-ALU plans keep one fp32 state per chunk and two fp32 score-tile buffers.
+  // states per 128-token tile in bf16 (or, in the two-level form, fewer fp32 segment states in the same region); the
+  // fp32-ALU plans keep one fp32 state per chunk.
   const size_t entries = (size_t)pl->rp;
   const int wide = d_k > d_v ? d_k : d_v;
   const size_t causal = pl->tc ? (size_t)pl->bh * (T / 128) * entries * 2 : (size_t)pl->bh * pl->NC * entries * 4;
-  const size_t tiles = pl->tc ? 0 : (size_t)pl->bh * T * chunk * sizeof(float);
   size_t off = 0;
   pl->off_status = off; off = align_up(off + 256);
   pl->off_sin = off;    off = align_up(off + causal);
@@ -434,7 +431,6 @@ smat_status smat_plan_create(smat_plan** out, int batch, int heads, int64_t T, i
   pl->off_F = off;      off = align_up(off + (g.dense_G || alias ? 0 : (size_t)pl->bh * g.P * entries * (pl->f_bf16 ? 2 : 4)));
   pl->off_U = off;      off = align_up(off + (g.dense_G ? 0 : (size_t)pl->bh * g.B * entries * (pl->u_bf16 ? 2 : 4)));
   pl->off_acc = off;    off = align_up(off + (size_t)pl->bh * T * wide * sizeof(float));
-  pl->off_tileA = off;  off = align_up(off + tiles);
   pl->off_W = off;      off = align_up(off + (pl->tab_tc ? (size_t)smat_tabulate_tc_scratch_elems(g, pl->rp, pl->bh) * 2 : 0));
   pl->off_sin_tiles = off;
   off = align_up(off + (pl->tc && (flags & SMAT_FLAG_KEEP_FORWARD_TABLES) ? (size_t)pl->bh * (T / 128) * entries * 2 : 0));
@@ -476,7 +472,7 @@ smat_status smat_plan_create(smat_plan** out, int batch, int heads, int64_t T, i
   pl->off_dbar = off;   off = align_up(off + causal);
   pl->off_ubar = off;   off = align_up(off + (g.dense_G || alias ? 0 : (size_t)pl->bh * g.B * entries * (pl->ubar_bf16 ? 2 : 4)));
   pl->off_fbar = off;   off = align_up(off + (g.dense_G ? 0 : (size_t)pl->bh * g.P * entries * (pl->fbar_bf16 ? 2 : 4)));
-  pl->off_tileG = off;  off = align_up(off + tiles);
+  pl->off_acc2 = off;   off = align_up(off + (pl->tc ? 0 : (size_t)pl->bh * T * d_v * sizeof(float)));   // dV's long-range rows
   pl->off_bwd_end = off;
   *out = pl;
   return SMAT_OK;
@@ -602,7 +598,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
                                                                group(cx, SMAT_GM_TYPE), pl->geo.B, pl->T, pl->bh, status,
                                                                cx.st));
       else
-        state_read(cx, "read_type", SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, nullptr, ylr, nullptr);
+        state_read(cx, "read_type", {read_job(cx, SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, ylr)});
     }
     pl->tile_states = L < 2;
     pl->kept_tile_states = false;
@@ -613,7 +609,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
       const int64_t nseg = nseg0 + nseg1;
       const int64_t rows0 = tiles0 * 128, rows1 = tiles1 * 128;
       SMAT_TRY(cx, "segment_state_tc", smat_launch_segment_state_tc(K, V, seg, rows0, rows1, nseg0, nseg1, pl->bh, status, cx.st));
-      SMAT_TRY(cx, "segment_scan", smat_launch_scan(seg, pl->rp, nseg, pl->bh, 0, nseg0, nseg0, nseg, 0, cx.st));
+      scan_segments(cx, seg, nseg0, nseg);
       const bool keep = (pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES) != 0;   // a backward will want the per-tile states
       SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, seg, ylr, 0, lr ? pl->geo.n : pl->T, O,
                                                                        rows0, rows1, nseg0, nseg1, pl->bh, status, cx.st,
@@ -641,26 +637,31 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     if (lr) {
       build_type_table(cx, K, V);
       zero_unrouted(cx, SMAT_GM_TYPE, ylr, 512);
-      state_read(cx, "read_type", SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, nullptr, ylr, nullptr);
+      state_read(cx, "read_type", {read_job(cx, SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, ylr)});
     }
     int nseg0 = 0, nseg1 = 0;
     smat_segment_counts((rows0 + 127) / 128, (rows1 + 127) / 128, pl->bh, 2, &nseg0, &nseg1);
     const int64_t nseg = nseg0 + nseg1;
     SMAT_TRY(cx, "segment_state_tc", smat_launch_segment_state_tc(K, V, seg, rows0, rows1, nseg0, nseg1, pl->bh, status, cx.st));
-    SMAT_TRY(cx, "segment_scan", smat_launch_scan(seg, pl->rp, nseg, pl->bh, 0, nseg0, nseg0, nseg, 0, cx.st));
+    scan_segments(cx, seg, nseg0, nseg);
     SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, seg, ylr, 1, lr ? pl->geo.n : pl->T, O, rows0,
                                                                      rows1, nseg0, nseg1, pl->bh, status, cx.st));
     pl->launches = cx.launches;
     return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;
   }
-  build_forward_tables(cx, K, V);
-  float* acc = cx.f(pl->off_acc);
-  float* tileA = cx.f(pl->off_tileA);
-  tril_scores(cx, "scores", Q, K, pl->r, tileA);                           // within-chunk scores, Eq. "local"
-  state_read(cx, "read_chunk", SMAT_GM_CHUNK, Q, cx.f(pl->off_sin), 0, nullptr, acc, nullptr);  // earlier chunks
-  if (!pl->geo.dense_G)                                                    // step 4: typed read, rows in place
-    state_read(cx, "read_type", SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, acc, acc, nullptr);
-  tile_apply(cx, "output", tileA, 0, V, pl->p, acc, nullptr, O);                     // step 7
+  // fp32-ALU path.  Long-range and causal states are pooled together; the typed rows are added by the tile kernel.
+  const bool lr = !pl->geo.dense_G;
+  float *sin = cx.f(pl->off_sin), *acc = cx.f(pl->off_acc);
+  const SmatPoolJob chunks = pool_job(cx, SMAT_GM_CHUNK, K, V, sin);
+  if (lr) pool(cx, "pool", {pool_job(cx, SMAT_GM_PROFILE, K, V, cx.f(pl->off_F)), chunks});           // steps 2, 5
+  else pool(cx, "pool", {chunks});
+  scan_states(cx, "scan", {scan_job(cx, sin, 0)});                                                   // step 6
+  if (lr) {
+    tabulate(cx, "tabulate", cx.f(pl->off_F), cx.f(pl->off_U), 0);                                   // step 3
+    zero_unrouted(cx, SMAT_GM_TYPE, acc, pl->p * 4);
+    state_read(cx, "read_type", {read_job(cx, SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, acc)});           // step 4
+  }
+  tile_rows(cx, "tiles", pl->r, pl->p, {tile_job(Q, K, V, Q, sin, 0, 0, acc, lr ? pl->geo.n : pl->T, pl->T, O)}, nullptr);   // step 7
   pl->launches = cx.launches;
   return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;
 }
@@ -739,7 +740,7 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
         SMAT_TRY(cx, "bwd_dq_type_tc", smat_launch_state_read_tc(dO, cx.ws + pl->off_U, lrbuf, lrbuf, 1, types, pl->geo.B,
                                                                  pl->T, pl->bh, status, cx.st));
       else
-        state_read(cx, "bwd_dq_type", SMAT_GM_TYPE, dO, cx.f(pl->off_U), 1, nullptr, lrbuf, nullptr);
+        state_read(cx, "bwd_dq_type", {read_job(cx, SMAT_GM_TYPE, dO, cx.f(pl->off_U), 1, lrbuf)});
       SMAT_TRY(cx, "bwd_dq_tile_tc", smat_launch_chunk_adjoint_tc(0, Q, K, V, dO, sin_tiles, cx.ws + pl->off_dbar,
                                                                   lrbuf, n, pl->T, dQ, pl->T, pl->bh, status, cx.st,
                                                                   pl->u_bf16 ? 1 : 0));
@@ -749,7 +750,7 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
         SMAT_TRY(cx, "bwd_dk_profile_tc", smat_launch_state_read_tc(V, cx.ws + pl->off_fbar, lrbuf, lrbuf, 1, profs, pl->geo.P,
                                                                     pl->T, pl->bh, status, cx.st));
       else
-        state_read(cx, "bwd_dk_profile", SMAT_GM_PROFILE, V, cx.f(pl->off_fbar), 1, nullptr, lrbuf, nullptr);
+        state_read(cx, "bwd_dk_profile", {read_job(cx, SMAT_GM_PROFILE, V, cx.f(pl->off_fbar), 1, lrbuf)});
       SMAT_TRY(cx, "bwd_dk_tile_tc", smat_launch_chunk_adjoint_tc(1, Q, K, V, dO, sin_tiles, cx.ws + pl->off_dbar,
                                                                   lrbuf, 0, n, dK, pl->T, pl->bh, status, cx.st,
                                                                   fbar_is_bf16 ? 1 : 0));
@@ -759,7 +760,7 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
         SMAT_TRY(cx, "bwd_dv_profile_tc", smat_launch_state_read_tc(K, cx.ws + pl->off_fbar, lrbuf, lrbuf, 0, profs, pl->geo.P,
                                                                     pl->T, pl->bh, status, cx.st));
       else
-        state_read(cx, "bwd_dv_profile", SMAT_GM_PROFILE, K, cx.f(pl->off_fbar), 0, nullptr, lrbuf, nullptr);
+        state_read(cx, "bwd_dv_profile", {read_job(cx, SMAT_GM_PROFILE, K, cx.f(pl->off_fbar), 0, lrbuf)});
       SMAT_TRY(cx, "bwd_dv_tile_tc", smat_launch_chunk_adjoint_tc(2, Q, K, V, dO, sin_tiles, cx.ws + pl->off_dbar,
                                                                   lrbuf, 0, n, dV, pl->T, pl->bh, status, cx.st,
                                                                   fbar_is_bf16 ? 1 : 0));
@@ -782,35 +783,30 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
     pl->launches = cx.launches;
     return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;
   }
-  build_forward_tables(cx, K, V);
+  // fp32-ALU path: every state of both directions from one pooling launch; S̄_in_b = Q_bᵀ dO_b and D̄ = its exclusive
+  // suffix scan (scan adjoint); Ū_h = Σ q dOᵀ over the type, F̄ = Cᵀ Ū (Eq. "lr-adjoint").
   pl->tile_states = true;
-  float* sin = cx.f(pl->off_sin);
-  float* dbar = cx.f(pl->off_dbar);
-  float* acc = cx.f(pl->off_acc);
-  float* tileA = cx.f(pl->off_tileA);
-  float* tileG = cx.f(pl->off_tileG);
-  // S̄_in_b = Q_bᵀ dO_b, then D̄ = exclusive suffix scan (scan adjoint)
-  outer_sum(cx, "bwd_chunk_state", SMAT_GM_CHUNK, Q, dO, dbar);
-  scan_states(cx, "bwd_scan", dbar, 1);
-  // long-range adjoints: Ū_h = Σ q dOᵀ over the type, F̄ = Cᵀ Ū   (Eq. "lr-adjoint")
+  float *sin = cx.f(pl->off_sin), *dbar = cx.f(pl->off_dbar);
+  float *acc = cx.f(pl->off_acc), *acc_v = cx.f(pl->off_acc2);
+  const SmatPoolJob cf = pool_job(cx, SMAT_GM_CHUNK, K, V, sin), cb = pool_job(cx, SMAT_GM_CHUNK, Q, dO, dbar);
+  if (lr) pool(cx, "bwd_pool", {pool_job(cx, SMAT_GM_PROFILE, K, V, cx.f(pl->off_F)), cf, cb,
+                                pool_job(cx, SMAT_GM_TYPE, Q, dO, cx.f(pl->off_ubar))});
+  else pool(cx, "bwd_pool", {cf, cb});
+  scan_states(cx, "bwd_scan", {scan_job(cx, sin, 0), scan_job(cx, dbar, 1)});
   if (lr) {
-    outer_sum(cx, "bwd_pool_type", SMAT_GM_TYPE, Q, dO, cx.f(pl->off_ubar));
+    tabulate(cx, "tabulate", cx.f(pl->off_F), cx.f(pl->off_U), 0);
     tabulate(cx, "bwd_tabulate_t", cx.f(pl->off_ubar), cx.f(pl->off_fbar), 1);
+    // dQ's long-range rows are recent and dK's distant: they share a buffer
+    zero_unrouted(cx, SMAT_GM_TYPE, acc, pl->r * 4);
+    zero_unrouted(cx, SMAT_GM_PROFILE, acc, pl->r * 4);
+    zero_unrouted(cx, SMAT_GM_PROFILE, acc_v, pl->p * 4);
+    state_read(cx, "bwd_reads", {read_job(cx, SMAT_GM_TYPE, dO, cx.f(pl->off_U), 1, acc),
+                                 read_job(cx, SMAT_GM_PROFILE, V, cx.f(pl->off_fbar), 1, acc),
+                                 read_job(cx, SMAT_GM_PROFILE, K, cx.f(pl->off_fbar), 0, acc_v)});
   }
-  tril_scores(cx, "bwd_scores_qk", Q, K, pl->r, tileA);    // A = tril(Q Kᵀ)
-  tril_scores(cx, "bwd_scores_gv", dO, V, pl->p, tileG);   // tril(dO Vᵀ)
-  // dQ = dO S_inᵀ + U_type dO (recent) + tril(dO Vᵀ) K                      (Eq. "local-adjoint", Eq. "lr-adjoint")
-  state_read(cx, "bwd_dq_chunk", SMAT_GM_CHUNK, dO, sin, 1, nullptr, acc, nullptr);
-  if (lr) state_read(cx, "bwd_dq_type", SMAT_GM_TYPE, dO, cx.f(pl->off_U), 1, acc, acc, nullptr);
-  tile_apply(cx, "bwd_dq_tile", tileG, 0, K, pl->r, acc, nullptr, dQ);
-  // dK = tril(dO Vᵀ)ᵀ Q + F̄_prof v (distant) + D̄ v
-  tile_apply(cx, "bwd_dk_tile", tileG, 1, Q, pl->r, nullptr, acc, nullptr);
-  if (lr) state_read(cx, "bwd_dk_profile", SMAT_GM_PROFILE, V, cx.f(pl->off_fbar), 1, acc, acc, nullptr);
-  state_read(cx, "bwd_dk_chunk", SMAT_GM_CHUNK, V, dbar, 1, acc, nullptr, dK);
-  // dV = Aᵀ dO + F̄_profᵀ k (distant) + D̄ᵀ k
-  tile_apply(cx, "bwd_dv_tile", tileA, 1, dO, pl->p, nullptr, acc, nullptr);
-  if (lr) state_read(cx, "bwd_dv_profile", SMAT_GM_PROFILE, K, cx.f(pl->off_fbar), 0, acc, acc, nullptr);
-  state_read(cx, "bwd_dv_chunk", SMAT_GM_CHUNK, K, dbar, 0, acc, nullptr, dV);
+  const int64_t n = lr ? pl->geo.n : 0, from = lr ? n : pl->T;
+  adjoint_tiles(cx, "bwd_tiles", tile_job(dO, V, K, dO, sin, 1, 0, acc, from, pl->T, dQ),
+                tile_job(V, dO, Q, V, dbar, 1, 1, acc, 0, n, dK), tile_job(K, Q, dO, K, dbar, 0, 1, acc_v, 0, n, dV), nullptr);
   pl->launches = cx.launches;
   return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;
 }
@@ -842,19 +838,13 @@ void gated_scan(Ctx& cx, const char* name, float* S, const float* lam, int rever
     SMAT_TRY(cx, name, smat_launch_gated_scan(S, lam, pl->rp, pl->NC, pl->c, pl->bh, 0, ncd, ncd, pl->NC, reverse, cx.st));
 }
 
-// λ, the rescaled inputs and the forward tables (S_in, F, U) of the gated pass.
-void gated_forward_tables(Ctx& cx, const Gated& gt, const void* Q, const void* K, const void* V, const float* log_a) {
+// λ and the rescaled inputs of the gated pass.
+void gated_inputs(Ctx& cx, const Gated& gt, const void* Q, const void* K, const float* log_a) {
   const smat_plan* pl = cx.pl;
   SMAT_TRY(cx, "gate_prefix", smat_launch_head_scan(log_a, gt.lam, pl->T, pl->bh, 0, cx.st));
   gate_scale(cx, "gate_scale_q", Q, nullptr, gt.qc, gt.lam, 0, pl->r);       // exp(λ_i - λ_{e(b-1)}) q_i
   gate_scale(cx, "gate_scale_k", K, nullptr, gt.kc, gt.lam, 1, pl->r);       // exp(λ_{e(b)} - λ_j) k_j
-  if (!pl->geo.dense_G) {
-    gate_scale(cx, "gate_scale_lr", K, Q, gt.lr, gt.lam, 2, pl->r);          // keys and queries split at the boundary
-    outer_sum(cx, "pool", SMAT_GM_PROFILE, gt.lr, V, cx.f(pl->off_F));
-    tabulate(cx, "tabulate", cx.f(pl->off_F), cx.f(pl->off_U), 0);
-  }
-  outer_sum(cx, "chunk_state", SMAT_GM_CHUNK, gt.kc, V, cx.f(pl->off_sin));
-  gated_scan(cx, "gated_scan", cx.f(pl->off_sin), gt.lam, 0);
+  if (!pl->geo.dense_G) gate_scale(cx, "gate_scale_lr", K, Q, gt.lr, gt.lam, 2, pl->r);   // keys and queries split at the boundary
 }
 
 // Gated forward on the tensor cores (bf16, d_k = d_v = 128, blocks of whole 128-token tiles).  The long-range part is
@@ -883,7 +873,7 @@ smat_status forward_gated_tc(Ctx& cx, const Gated& gt, const void* Q, const void
                                                              group(ci, SMAT_GM_TYPE), in->geo.B, in->T, in->bh, status,
                                                              ci.st));                        // step 4 on the rescaled queries
     else
-      state_read(ci, "read_type", SMAT_GM_TYPE, gt.lr, ci.f(in->off_U), 0, nullptr, ylr, nullptr);
+      state_read(ci, "read_type", {read_job(ci, SMAT_GM_TYPE, gt.lr, ci.f(in->off_U), 0, ylr)});
   }
   SMAT_TRY(ci, "gated_chunk_scan_tc", smat_launch_chunk_scan_tc(gt.kc, V, ci.ws + in->off_sin, in->T, in->bh, in->geo.n,
                                                                  lr ? 0 : 1, 0, status, ci.st, gt.lam));
@@ -1039,13 +1029,19 @@ smat_status smat_forward_gated(const smat_plan* pl, const void* Q, const void* K
   cx.err = clear_status(cx);
   const Gated gt = gated_buffers(cx);
   if (pl->inner) return forward_gated_tc(cx, gt, Q, K, V, log_a, O);
-  gated_forward_tables(cx, gt, Q, K, V, log_a);
-  float* acc = cx.f(pl->off_acc);
-  float* tileA = cx.f(pl->off_tileA);
-  tril_scores(cx, "scores", Q, K, pl->r, tileA, gt.lam);                         // tril(QKᵀ) ⊙ exp(λ_i - λ_j)
-  state_read(cx, "read_chunk", SMAT_GM_CHUNK, gt.qc, cx.f(pl->off_sin), 0, nullptr, acc, nullptr);
-  if (!pl->geo.dense_G) state_read(cx, "read_type", SMAT_GM_TYPE, gt.lr, cx.f(pl->off_U), 0, acc, acc, nullptr);
-  tile_apply(cx, "output", tileA, 0, V, pl->p, acc, nullptr, O);
+  const bool lr = !pl->geo.dense_G;
+  float *sin = cx.f(pl->off_sin), *acc = cx.f(pl->off_acc);
+  gated_inputs(cx, gt, Q, K, log_a);
+  const SmatPoolJob chunks = pool_job(cx, SMAT_GM_CHUNK, gt.kc, V, sin);
+  if (lr) pool(cx, "pool", {pool_job(cx, SMAT_GM_PROFILE, gt.lr, V, cx.f(pl->off_F)), chunks});
+  else pool(cx, "pool", {chunks});
+  gated_scan(cx, "gated_scan", sin, gt.lam, 0);
+  if (lr) {
+    tabulate(cx, "tabulate", cx.f(pl->off_F), cx.f(pl->off_U), 0);
+    state_read(cx, "read_type", {read_job(cx, SMAT_GM_TYPE, gt.lr, cx.f(pl->off_U), 0, acc)});
+  }
+  // tril(QKᵀ) ⊙ exp(λ_i - λ_j), and the rescaled queries on the incoming state
+  tile_rows(cx, "tiles", pl->r, pl->p, {tile_job(Q, K, V, gt.qc, sin, 0, 0, acc, lr ? pl->geo.n : pl->T, pl->T, O)}, gt.lam);
   pl->launches = cx.launches;
   return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;
 }
@@ -1068,36 +1064,31 @@ smat_status smat_backward_gated(const smat_plan* pl, const void* Q, const void* 
   const bool lr = !pl->geo.dense_G;
   const Gated gt = gated_buffers(cx);
   if (gated_backward_on_tc(pl)) return backward_gated_tc(cx, gt, Q, K, V, log_a, dO, dQ, dK, dV, dlog_a, after_gated_forward);
-  gated_forward_tables(cx, gt, Q, K, V, log_a);
+  gated_inputs(cx, gt, Q, K, log_a);
   gate_scale(cx, "bwd_gate_scale_do", dO, nullptr, gt.doc, gt.lam, 0, pl->p);    // exp(λ_i - λ_{e(b-1)}) dO_i
   gate_scale(cx, "bwd_gate_scale_v", V, nullptr, gt.vc, gt.lam, 1, pl->p);       // exp(λ_{e(b)} - λ_j) v_j
   if (lr) gate_scale(cx, "bwd_gate_scale_lr", V, dO, gt.vlr, gt.lam, 2, pl->p);  // values / upstream rows at the boundary
-  float* sin = cx.f(pl->off_sin);
-  float* dbar = cx.f(pl->off_dbar);
-  float* acc = cx.f(pl->off_acc);
-  float* tileA = cx.f(pl->off_tileA);
-  float* tileG = cx.f(pl->off_tileG);
+  float *sin = cx.f(pl->off_sin), *dbar = cx.f(pl->off_dbar);
+  float *acc = cx.f(pl->off_acc), *acc_v = cx.f(pl->off_acc2);
   // adjoint of the carried state: S̄_in_b = Σ_i (scaled q_i) dO_iᵀ, then the decayed suffix recursion
-  outer_sum(cx, "bwd_chunk_state", SMAT_GM_CHUNK, gt.qc, dO, dbar);
+  const SmatPoolJob cf = pool_job(cx, SMAT_GM_CHUNK, gt.kc, V, sin), cb = pool_job(cx, SMAT_GM_CHUNK, gt.qc, dO, dbar);
+  if (lr) pool(cx, "bwd_pool", {pool_job(cx, SMAT_GM_PROFILE, gt.lr, V, cx.f(pl->off_F)), cf, cb,
+                                pool_job(cx, SMAT_GM_TYPE, gt.lr, dO, cx.f(pl->off_ubar))});
+  else pool(cx, "bwd_pool", {cf, cb});
+  gated_scan(cx, "gated_scan", sin, gt.lam, 0);
   gated_scan(cx, "bwd_gated_scan", dbar, gt.lam, 1);
   if (lr) {
-    outer_sum(cx, "bwd_pool_type", SMAT_GM_TYPE, gt.lr, dO, cx.f(pl->off_ubar));
+    tabulate(cx, "tabulate", cx.f(pl->off_F), cx.f(pl->off_U), 0);
     tabulate(cx, "bwd_tabulate_t", cx.f(pl->off_ubar), cx.f(pl->off_fbar), 1);
+    state_read(cx, "bwd_reads", {read_job(cx, SMAT_GM_TYPE, gt.vlr, cx.f(pl->off_U), 1, acc),
+                                 read_job(cx, SMAT_GM_PROFILE, gt.vlr, cx.f(pl->off_fbar), 1, acc),
+                                 read_job(cx, SMAT_GM_PROFILE, gt.lr, cx.f(pl->off_fbar), 0, acc_v)});
   }
-  tril_scores(cx, "bwd_scores_qk", Q, K, pl->r, tileA, gt.lam);
-  tril_scores(cx, "bwd_scores_gv", dO, V, pl->p, tileG, gt.lam);
-  // dQ_i = S_in (scaled dO_i) + U_type (boundary-scaled dO_i) + Σ_j G_ij k_j
-  state_read(cx, "bwd_dq_chunk", SMAT_GM_CHUNK, gt.doc, sin, 1, nullptr, acc, nullptr);
-  if (lr) state_read(cx, "bwd_dq_type", SMAT_GM_TYPE, gt.vlr, cx.f(pl->off_U), 1, acc, acc, nullptr);
-  tile_apply(cx, "bwd_dq_tile", tileG, 0, K, pl->r, acc, nullptr, dQ);
-  // dK_j = Σ_i G_ij q_i + F̄_prof (boundary-scaled v_j) + D̄ (chunk-scaled v_j)
-  tile_apply(cx, "bwd_dk_tile", tileG, 1, Q, pl->r, nullptr, acc, nullptr);
-  if (lr) state_read(cx, "bwd_dk_profile", SMAT_GM_PROFILE, gt.vlr, cx.f(pl->off_fbar), 1, acc, acc, nullptr);
-  state_read(cx, "bwd_dk_chunk", SMAT_GM_CHUNK, gt.vc, dbar, 1, acc, nullptr, dK);
-  // dV_j = Σ_i A_ij dO_i + F̄_profᵀ (boundary-scaled k_j) + D̄ᵀ (chunk-scaled k_j)
-  tile_apply(cx, "bwd_dv_tile", tileA, 1, dO, pl->p, nullptr, acc, nullptr);
-  if (lr) state_read(cx, "bwd_dv_profile", SMAT_GM_PROFILE, gt.lr, cx.f(pl->off_fbar), 0, acc, acc, nullptr);
-  state_read(cx, "bwd_dv_chunk", SMAT_GM_CHUNK, gt.kc, dbar, 0, acc, nullptr, dV);
+  // dQ_i = Σ_j G_ij k_j + S_in (scaled dO_i);  dK_j = Σ_i G_ij q_i + D̄ (scaled v_j);  dV_j = Σ_i A_ij dO_i + D̄ᵀ (scaled k_j)
+  const int64_t n = lr ? pl->geo.n : 0, from = lr ? n : pl->T;
+  adjoint_tiles(cx, "bwd_tiles", tile_job(dO, V, K, gt.doc, sin, 1, 0, acc, from, pl->T, dQ),
+                tile_job(V, dO, Q, gt.vc, dbar, 1, 1, acc, 0, n, dK), tile_job(K, Q, dO, gt.kc, dbar, 0, 1, acc_v, 0, n, dV),
+                gt.lam);
   // gates: dλ_t = q_t·dQ_t - k_t·dK_t, and log a_k enters every λ_t with t >= k
   float* dlam = cx.f(pl->off_dlam);
   SMAT_TRY(cx, "bwd_gate_dlam", smat_launch_gate_dlam(Q, dQ, K, dK, dlam, pl->dtype == SMAT_BF16, pl->r, pl->T, pl->bh, cx.st));

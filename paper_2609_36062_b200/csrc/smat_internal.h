@@ -59,33 +59,39 @@ SMAT_HD SmatTokens smat_group_tokens(const SmatGroupSpec& s, int64_t bh, int64_t
   return r;
 }
 
-// ---- generic batched small GEMM on the fp32 ALUs ---------------------------------------------------
-// C(m,n) = [Cin(m,n) +] Σ_k A(m,k) B(k,n), optionally zeroed above the diagonal (n > m).
-// An operand element lives at  ptr + bh*s_bh + g*s_g + X0*s0 + X1*s1  where Xi is the logical
-// index itself or, when the operand's tok flag for that index is set, the token it maps to.
-struct SmatOperand {
-  const void* ptr;
-  int bf16;  // 0: float, 1: __nv_bfloat16
-  int64_t s_bh, s_g, s0, s1;
-  int tok0, tok1;  // 1: that logical index of this operand is a token position of the group
+// ---- within-chunk tiles on the fp32 ALUs ------------------------------------------------------------
+// Out[i] = Σ_j X_ij P3_j + P4_i · St (+ acc[i] for rows acc_lo <= t < acc_hi), X_ij = P1_i · P2_j for j <= i (upper:
+// j >= i) of the same chunk.  P1, P2, P4 have score_dim columns, P3, acc and Out out_dim; the states are
+// [bh][NC][score_dim][out_dim], or [..][out_dim][score_dim] with st_trans.
+struct SmatTileJob {
+  const void *p1, *p2, *p3, *p4;   // [bh][T][.] rows in the plan's dtype
+  const float* st;
+  const float* acc;                // [bh][T][out_dim] fp32
+  int64_t acc_lo, acc_hi;
+  void* out;
+  int upper, st_trans;
 };
-
-struct SmatGemmArgs {
-  SmatOperand A, B, C, Cin;  // Cin.ptr == nullptr: no addend.  Cin is always float.
-  int M, N, K;               // extents of the dimensions that are not token dimensions
-  int tokM, tokN, tokK;      // 1: that dimension runs over the group's tokens (extent = token count)
-  int tril;
-  int tilesN;                // number of 64-wide column tiles launched
-  SmatGroupSpec grp;
-  const float* lam;          // gated variant: prefix sums of the log-gates [bh][T]; a tril tile over the tokens of a chunk
-                             // is multiplied entrywise by exp(λ_m - λ_n) (null: no decay)
+struct SmatTileArgs {
+  SmatTileJob job[3];
+  int jobs;
+  int64_t T;
+  int c, NC;
+  const float* lam;                // gated variant: prefix sums of the log-gates [bh][T]; X_ij is multiplied by the decay
 };
+cudaError_t smat_launch_tile_rows(const SmatTileArgs& a, int bf16, int score_dim, int out_dim, int bh, cudaStream_t st);
 
-cudaError_t smat_launch_gemm(const SmatGemmArgs& a, int max_M, int max_N, int64_t groups, int bh, cudaStream_t st);
-
-// Exclusive scan of per-chunk states in place, over up to two independent chunk ranges; reverse = suffix scan.
-cudaError_t smat_launch_scan(float* S, int64_t state_elems, int64_t NC, int bh, int64_t lo0, int64_t hi0, int64_t lo1,
-                             int64_t hi1, int reverse, cudaStream_t st);
+// Exclusive scans of per-chunk states [bh][NC][state] in place, over up to two independent chunk ranges each;
+// reverse = suffix scan.
+struct SmatScanJob {
+  float* S;
+  int64_t lo0, hi0, lo1, hi1;
+  int reverse;
+};
+struct SmatScanArgs {
+  SmatScanJob job[2];
+  int jobs;
+};
+cudaError_t smat_launch_scan(const SmatScanArgs& a, int64_t state_elems, int64_t NC, int bh, cudaStream_t st);
 
 // Algorithm 2 (direct form) and its transpose, one slab of state entries per CTA held in shared memory.
 // transpose = 0: out[h] = Σ_{x ∈ H_h} in[x]  (in: P states, out: B states)
@@ -97,14 +103,36 @@ int smat_tabulate_alg2_slab(int64_t rows_in, int64_t state_elems);
 
 cudaError_t smat_launch_mask(uint8_t* mask, const SmatGeo& geo, cudaStream_t st);
 
-// Pooling of outer products into one fp32 state per group: state[bh][g] = Σ_{tokens of g} a_tᵀ b_t.
-cudaError_t smat_launch_pool(const void* A, const void* Bm, int bf16, float* state, const SmatGroupSpec& grp,
-                             int64_t Tlen, int64_t groups, int bh, int r, int p, cudaStream_t st);
+// Pooling of outer products into one fp32 state per group: state[bh][g] = Σ_{tokens of g} a_tᵀ b_t (a: r columns,
+// b: p columns), for up to four sets of groups in one launch.
+struct SmatPoolJob {
+  const void *a, *b;               // [bh][T][.] rows in the plan's dtype
+  float* state;
+  SmatGroupSpec grp;
+  int64_t groups;                  // states per head
+};
+struct SmatPoolArgs {
+  SmatPoolJob job[4];
+  int jobs;
+};
+cudaError_t smat_launch_pool(const SmatPoolArgs& a, int bf16, int64_t Tlen, int bh, int r, int p, cudaStream_t st);
 
-// Routed read of per-group states: acc_out[t] = acc_in[t] + x_t · state[g(t)] for the tokens of every group.
-cudaError_t smat_launch_state_read(const void* X, int bf16, const float* state, int transposed, const float* acc_in,
-                                   float* acc_out, const SmatGroupSpec& grp, int64_t Tlen, int64_t groups, int bh,
-                                   int r, int p, int* status, cudaStream_t st);
+// Routed reads of per-group fp32 states [r][p]: out[t] = x_t · state[g(t)] for the tokens of every group (trans: the
+// second state index is contracted), fp32 rows, for up to three sets in one launch.
+struct SmatReadJob {
+  const void* x;                   // [bh][T][r] rows (trans: [bh][T][p])
+  const float* state;
+  float* out;                      // [bh][T][p] (trans: [bh][T][r])
+  SmatGroupSpec grp;
+  int64_t groups;
+  int trans;
+};
+struct SmatReadArgs {
+  SmatReadJob job[3];
+  int jobs;
+};
+cudaError_t smat_launch_state_read(const SmatReadArgs& a, int bf16, int64_t Tlen, int bh, int r, int p, int* status,
+                                   cudaStream_t st);
 
 // Staged exact tabulation (same sums as Algorithm 2, one coordinate at a time). Slab = 0: not available.
 int smat_tabulate_staged_slab(const SmatGeo& geo, int64_t state_elems, int transpose);

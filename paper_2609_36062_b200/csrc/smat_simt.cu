@@ -1,132 +1,243 @@
-// fp32-ALU kernels of libsmat: the generic grouped GEMM (every contraction of Algorithm 1 and of the
-// backward pass when no tensor-core kernel applies: fp32 inputs, odd shapes), the chunk-state scans,
-// the direct form of Algorithm 2 and its transpose, and the debug mask.
+// fp32-ALU kernels of libsmat: the within-chunk tiles of the forward and of the backward pass when no tensor-core
+// kernel applies (fp32 inputs, other head widths), the chunk-state scans, the direct form of Algorithm 2 and its
+// transpose, and the debug mask.
 #include <cuda_bf16.h>
 
 #include "smat_internal.h"
+#include "smat_launch.cuh"
+#include "smat_tc.cuh"
 
 namespace {
 
-constexpr int TILE = 64;   // output tile edge
-constexpr int KSTEP = 16;  // reduction step
-constexpr int LDS = TILE + 4;
+using tc::cp_async16;
+using tc::cp_async_commit;
+using tc::cp_async_wait;
 
-__device__ __forceinline__ float load_elem(const SmatOperand& o, int64_t off) {
-  if (o.bf16) return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(o.ptr)[off]);
-  return reinterpret_cast<const float*>(o.ptr)[off];
+// ---- within-chunk tiles ------------------------------------------------------------------------------------------
+// Out[i] = Σ_j X_ij P3_j + P4_i · St (+ addend row),   X_ij = P1_i · P2_j where j <= i (upper: j >= i) in i's chunk:
+//     O  : P1 = Q,  P2 = K,  P3 = V,  P4 = Q,  St = S_in              dQ : P1 = dO, P2 = V,  P3 = K,  P4 = dO, St = S_inᵀ
+//     dK : P1 = V,  P2 = dO, P3 = Q,  P4 = V,  St = D̄ᵀ (upper)        dV : P1 = K,  P2 = Q,  P3 = dO, P4 = K,  St = D̄ (upper)
+// (Eq. "local", Eq. "local-adjoint" with the broadcast of the scanned states.)  A CTA takes 32 rows of one chunk: the
+// scores of 64 columns at a time go through shared memory, two operand buffers alternate between the next columns'
+// P2 / P3 and the 64-row pieces of the state, fetched while the other one is used.  Everything is fp32.
+// One launch serves the forward tile, or the three adjoints (jobs).  What it replaces — scores, state product and
+// tile product as separate launches of a general 64 x 64 product, with the score tiles in memory — took 21 launches
+// and 259 us for forward + backward of one 512-token head (64 wide, chunk 64).
+constexpr int ROWS = 32;      // rows per CTA
+constexpr int COLS = 64;      // score columns per step, and rows of a state piece
+constexpr int TILE_THREADS = 256;
+
+template <typename T, int SD, int OD>
+struct TileLayout {
+  static constexpr int SROW = SD * (int)sizeof(T) + 16;   // bytes per staged row (padded by one 16-byte chunk)
+  static constexpr int OROW = OD * (int)sizeof(T) + 16;
+  static constexpr int STROW = OD * 4 + 16;               // one row of a state piece [k][n]
+  static constexpr int BUF = COLS * STROW > COLS * (SROW > OROW ? SROW : OROW) ? COLS * STROW : COLS * (SROW > OROW ? SROW : OROW);
+  static constexpr int XROW = COLS + 4;                   // floats
+  static constexpr int OFF_P4 = ROWS * SROW;
+  static constexpr int OFF_A = 2 * ROWS * SROW;
+  static constexpr int OFF_B = OFF_A + BUF;
+  static constexpr int OFF_X = OFF_B + BUF;
+  static constexpr int SMEM = OFF_X + ROWS * XROW * 4;
+};
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 ld4(const __nv_bfloat16* p) {
+  const uint2 w = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
+                     __uint_as_float(w.y & 0xffff0000u));
+}
+__device__ __forceinline__ void st4(float* p, const float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void st4(__nv_bfloat16* p, const float4 v) {
+  *reinterpret_cast<uint2*>(p) = make_uint2(tc::pack_bf16(v.x, v.y), tc::pack_bf16(v.z, v.w));
+}
+__device__ __forceinline__ float dot4(const float4 a, const float4 b, float acc) {
+  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
+}
+__device__ __forceinline__ float4 fma4(float s, const float4 b, float4 a) {
+  a.x = fmaf(s, b.x, a.x); a.y = fmaf(s, b.y, a.y); a.z = fmaf(s, b.z, a.z); a.w = fmaf(s, b.w, a.w);
+  return a;
 }
 
-__global__ void __launch_bounds__(256) gemm_grouped_kernel(const SmatGemmArgs a) {
-  const int64_t g = blockIdx.y;
-  const int64_t bh = blockIdx.z;
-  const SmatTokens tk = smat_group_tokens(a.grp, bh, g);
-  const int64_t cnt = tk.cnt;
-  const int M = a.tokM ? (int)cnt : a.M;
-  const int N = a.tokN ? (int)cnt : a.N;
-  const int K = a.tokK ? (int)cnt : a.K;
-  const int m0 = (blockIdx.x / a.tilesN) * TILE;
-  const int n0 = (blockIdx.x % a.tilesN) * TILE;
-  if (m0 >= M || n0 >= N) return;
-
-  __shared__ __align__(16) float As[KSTEP][LDS];
-  __shared__ __align__(16) float Bs[KSTEP][LDS];
-
+template <typename T, int SD, int OD>
+__global__ void __launch_bounds__(TILE_THREADS, 2) tile_rows_kernel(const __grid_constant__ SmatTileArgs a) {
+  using L = TileLayout<T, SD, OD>;
+  extern __shared__ __align__(16) uint8_t smem[];
+  pdl_trigger();
+  uint8_t *s1 = smem, *s4 = smem + L::OFF_P4, *sA = smem + L::OFF_A, *sB = smem + L::OFF_B;
+  float* sX = reinterpret_cast<float*>(smem + L::OFF_X);
+  const int blocks = (a.c + ROWS - 1) / ROWS;                 // row blocks of a chunk
+  const int per_job = a.NC * blocks;
+  const int which = blockIdx.x / per_job, rest = blockIdx.x - which * per_job;
+  const SmatTileJob& job = a.job[which];
+  const int chunk = rest / blocks, m0 = (rest - chunk * blocks) * ROWS;
+  const int64_t bh = blockIdx.y;
+  const int rows = a.c - m0 < ROWS ? a.c - m0 : ROWS;
+  const int64_t t0 = (int64_t)chunk * a.c;                    // first token of the chunk
+  const int64_t row0 = bh * a.T + t0;
   const int tid = threadIdx.x;
-  const int ty = tid >> 4, tx = tid & 15;
-  float acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  constexpr int OC = OD / 4, RG = TILE_THREADS / OC, RPT = ROWS / RG;   // output columns / 4, row groups, rows per thread
+  const int oc = tid % OC, rg = tid / OC;
 
-  const int64_t baseA = bh * a.A.s_bh + g * a.A.s_g;
-  const int64_t baseB = bh * a.B.s_bh + g * a.B.s_g;
-  const bool a_k_contig = (a.A.s1 == 1 && !a.A.tok1);
-  const bool b_n_contig = (a.B.s1 == 1 && !a.B.tok1);
-  const bool skip = a.tril && (n0 > m0 + TILE - 1);  // tile entirely above the diagonal
-
-  for (int k0 = 0; k0 < K && !skip; k0 += KSTEP) {
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const int e = tid + 256 * p;
-      int mm, kk;
-      if (a_k_contig) { kk = e & (KSTEP - 1); mm = e >> 4; } else { mm = e & (TILE - 1); kk = e >> 6; }
-      float v = 0.f;
-      if (m0 + mm < M && k0 + kk < K) {
-        const int64_t x0 = a.A.tok0 ? tk.at(m0 + mm) : (int64_t)(m0 + mm);
-        const int64_t x1 = a.A.tok1 ? tk.at(k0 + kk) : (int64_t)(k0 + kk);
-        v = load_elem(a.A, baseA + x0 * a.A.s0 + x1 * a.A.s1);
-      }
-      As[kk][mm] = v;
+  auto stage_rows = [&](uint8_t* dst, const void* src, int first, int count, int dim, int pitch) {
+    const int chunks = dim * (int)sizeof(T) / 16;
+    const uint8_t* base = static_cast<const uint8_t*>(src) + (row0 + first) * dim * (int64_t)sizeof(T);
+    for (int i = tid; i < count * chunks; i += TILE_THREADS) {
+      const int r = i / chunks, ch = i - r * chunks;
+      cp_async16(dst + r * pitch + ch * 16, base + (int64_t)i * 16);
     }
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const int e = tid + 256 * p;
-      int nn, kk;
-      if (b_n_contig) { nn = e & (TILE - 1); kk = e >> 6; } else { kk = e & (KSTEP - 1); nn = e >> 4; }
-      float v = 0.f;
-      if (n0 + nn < N && k0 + kk < K) {
-        const int64_t x0 = a.B.tok0 ? tk.at(k0 + kk) : (int64_t)(k0 + kk);
-        const int64_t x1 = a.B.tok1 ? tk.at(n0 + nn) : (int64_t)(n0 + nn);
-        v = load_elem(a.B, baseB + x0 * a.B.s0 + x1 * a.B.s1);
+  };
+  const float* st = job.st + (bh * a.NC + chunk) * (int64_t)(SD * OD);
+  // 64 rows of the state as the product reads it ([k][n], n contiguous)
+  auto stage_state = [&](uint8_t* dst, int piece) {
+    if (!job.st_trans) {
+      for (int i = tid; i < COLS * OC; i += TILE_THREADS) {
+        const int k = i / OC, ch = i - k * OC;
+        cp_async16(dst + k * L::STROW + ch * 16, st + (int64_t)(piece * COLS + k) * OD + ch * 4);
       }
-      Bs[kk][nn] = v;
+    } else {   // stored [n][k]: neighbouring lanes take neighbouring n, so that the scattered words hit different banks
+      float* d = reinterpret_cast<float*>(dst);
+      constexpr int PER = COLS / 4 * OD / TILE_THREADS;
+      float4 v[PER];
+#pragma unroll
+      for (int u = 0; u < PER; ++u) {
+        const int i = tid + u * TILE_THREADS, n = i % OD, k4 = i / OD;
+        v[u] = ld4(st + (int64_t)n * SD + piece * COLS + k4 * 4);
+      }
+#pragma unroll
+      for (int u = 0; u < PER; ++u) {
+        const int i = tid + u * TILE_THREADS, n = i % OD, k4 = i / OD;
+        float* p = d + (k4 * 4) * (L::STROW / 4) + n;
+        p[0] = v[u].x; p[L::STROW / 4] = v[u].y; p[2 * (L::STROW / 4)] = v[u].z; p[3 * (L::STROW / 4)] = v[u].w;
+      }
+    }
+  };
+  const int kb0 = job.upper ? m0 / COLS : 0;
+  const int kb1 = job.upper ? (a.c - 1) / COLS : (m0 + rows - 1) / COLS;
+  auto cols_of = [&](int kb) { return a.c - kb * COLS < COLS ? a.c - kb * COLS : COLS; };
+  const bool own4 = job.p4 != job.p1;
+  float4 acc[RPT];
+#pragma unroll
+  for (int r = 0; r < RPT; ++r) acc[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+
+  pdl_wait();
+  stage_rows(s1, job.p1, m0, rows, SD, L::SROW);
+  if (own4) stage_rows(s4, job.p4, m0, rows, SD, L::SROW);
+  stage_rows(sA, job.p2, kb0 * COLS, cols_of(kb0), SD, L::SROW);
+  cp_async_commit();
+  stage_rows(sB, job.p3, kb0 * COLS, cols_of(kb0), OD, L::OROW);
+  cp_async_commit();
+  for (int kb = kb0; kb <= kb1; ++kb) {
+    const int cols = cols_of(kb);
+    cp_async_wait<1>();
+    __syncthreads();
+    {   // scores: two rows x four columns per thread
+      const int ty = tid >> 4, tx = tid & 15;
+      float x[2][4];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[i][j] = 0.f;
+#pragma unroll 4
+      for (int k = 0; k < SD; k += 4) {
+        float4 av[2], bv[4];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) av[i] = ld4(reinterpret_cast<const T*>(s1 + (ty * 2 + i) * L::SROW) + k);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) bv[j] = ld4(reinterpret_cast<const T*>(sA + (tx + 16 * j) * L::SROW) + k);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) x[i][j] = dot4(av[i], bv[j], x[i][j]);
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int m = m0 + ty * 2 + i, n = kb * COLS + tx + 16 * j;   // positions inside the chunk
+          const bool in = m < a.c && n < a.c && (job.upper ? n >= m : n <= m);
+          float v = in ? x[i][j] : 0.f;
+          if (a.lam && in) {   // gated: decay between the key's and the query's position
+            const float* l = a.lam + row0;
+            v *= job.upper ? __expf(l[n] - l[m]) : __expf(l[m] - l[n]);
+          }
+          sX[(ty * 2 + i) * L::XROW + tx + 16 * j] = v;
+        }
     }
     __syncthreads();
+    if (kb < kb1) stage_rows(sA, job.p2, (kb + 1) * COLS, cols_of(kb + 1), SD, L::SROW);
+    else stage_state(sA, 0);
+    cp_async_commit();
+    cp_async_wait<1>();
+    __syncthreads();
+#pragma unroll 4
+    for (int k = 0; k < cols; k += 4) {
+      float4 xv[RPT], bv[4];
 #pragma unroll
-    for (int kk = 0; kk < KSTEP; ++kk) {
-      const float4 av = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
-      const float4 bv = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
-      const float ar[4] = {av.x, av.y, av.z, av.w};
-      const float br[4] = {bv.x, bv.y, bv.z, bv.w};
+      for (int r = 0; r < RPT; ++r) xv[r] = ld4(sX + (rg * RPT + r) * L::XROW + k);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int j = 0; j < 4; ++j) bv[j] = ld4(reinterpret_cast<const T*>(sB + (k + j) * L::OROW) + oc * 4);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(ar[i], br[j], acc[i][j]);
+      for (int r = 0; r < RPT; ++r) {
+        acc[r] = fma4(xv[r].x, bv[0], acc[r]); acc[r] = fma4(xv[r].y, bv[1], acc[r]);
+        acc[r] = fma4(xv[r].z, bv[2], acc[r]); acc[r] = fma4(xv[r].w, bv[3], acc[r]);
+      }
     }
     __syncthreads();
+    if (kb < kb1) stage_rows(sB, job.p3, (kb + 1) * COLS, cols_of(kb + 1), OD, L::OROW);
+    else if (SD > COLS) stage_state(sB, 1);
+    cp_async_commit();
   }
-
-  const int64_t baseC = bh * a.C.s_bh + g * a.C.s_g;
-  const int64_t baseI = bh * a.Cin.s_bh + g * a.Cin.s_g;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
-    if (m >= M) continue;
-    const int64_t x0 = a.C.tok0 ? tk.at(m) : (int64_t)m;
+  for (int piece = 0; piece < SD / COLS; ++piece) {
+    if (piece == 0) cp_async_wait<1>(); else cp_async_wait<0>();
+    __syncthreads();
+    const uint8_t* sp = own4 ? s4 : s1;
+    const uint8_t* buf = piece ? sB : sA;
+#pragma unroll 4
+    for (int k = 0; k < COLS; k += 4) {
+      float4 av[RPT], bv[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= N) continue;
-      const int64_t x1 = a.C.tok1 ? tk.at(n) : (int64_t)n;
-      float v = (a.tril && n > m) ? 0.f : acc[i][j];
-      if (a.lam && a.tril && n <= m) {   // gated: decay between the key's and the query's position
-        const float* l = a.lam + bh * a.grp.T;
-        v *= __expf(l[tk.at(m)] - l[tk.at(n)]);
+      for (int r = 0; r < RPT; ++r) av[r] = ld4(reinterpret_cast<const T*>(sp + (rg * RPT + r) * L::SROW) + piece * COLS + k);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) bv[j] = ld4(reinterpret_cast<const float*>(buf + (k + j) * L::STROW) + oc * 4);
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) {
+        acc[r] = fma4(av[r].x, bv[0], acc[r]); acc[r] = fma4(av[r].y, bv[1], acc[r]);
+        acc[r] = fma4(av[r].z, bv[2], acc[r]); acc[r] = fma4(av[r].w, bv[3], acc[r]);
       }
-      if (a.Cin.ptr) v += reinterpret_cast<const float*>(a.Cin.ptr)[baseI + x0 * a.Cin.s0 + x1 * a.Cin.s1];
-      const int64_t off = baseC + x0 * a.C.s0 + x1 * a.C.s1;
-      if (a.C.bf16)
-        reinterpret_cast<__nv_bfloat16*>(const_cast<void*>(a.C.ptr))[off] = __float2bfloat16_rn(v);
-      else
-        reinterpret_cast<float*>(const_cast<void*>(a.C.ptr))[off] = v;
     }
+  }
+#pragma unroll
+  for (int r = 0; r < RPT; ++r) {
+    const int m = rg * RPT + r;
+    if (m >= rows) continue;
+    const int64_t t = t0 + m0 + m, off = (bh * a.T + t) * OD + oc * 4;
+    float4 v = acc[r];
+    if (t >= job.acc_lo && t < job.acc_hi) {
+      const float4 y = ld4(job.acc + off);
+      v.x += y.x; v.y += y.y; v.z += y.z; v.w += y.w;
+    }
+    st4(static_cast<T*>(job.out) + off, v);
   }
 }
 
 // ---- scan --------------------------------------------------------------------------------------
 // Each thread owns four consecutive state entries and walks the chunks of its range in order.
 // Loads are issued sixteen chunks ahead of the dependent additions.
-__global__ void __launch_bounds__(256) scan_kernel(float* S, int64_t state_elems, int64_t NC, int64_t lo0, int64_t hi0,
-                                                   int64_t lo1, int64_t hi1, int reverse) {
+__global__ void __launch_bounds__(256) scan_kernel(const __grid_constant__ SmatScanArgs a, int64_t state_elems, int64_t NC) {
+  pdl_trigger();
   const int64_t e4 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e4 * 4 >= state_elems) return;
   const int64_t bh = blockIdx.y;
-  const int64_t lo = blockIdx.z ? lo1 : lo0, hi = blockIdx.z ? hi1 : hi0;
-  float4* base = reinterpret_cast<float4*>(S + bh * NC * state_elems) + e4;
+  const SmatScanJob& job = a.job[blockIdx.z >> 1];
+  const int range = blockIdx.z & 1, reverse = job.reverse;
+  const int64_t lo = range ? job.lo1 : job.lo0, hi = range ? job.hi1 : job.hi0;
+  float4* base = reinterpret_cast<float4*>(job.S + bh * NC * state_elems) + e4;
   const int64_t stride4 = state_elems / 4;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   constexpr int AHEAD = 16;
+  pdl_wait();
   for (int64_t s = 0; s < hi - lo; s += AHEAD) {
     float4 v[AHEAD];
 #pragma unroll
@@ -231,22 +342,27 @@ __global__ void mask_kernel(uint8_t* mask, const SmatGeo geo) {
 
 }  // namespace
 
-cudaError_t smat_launch_gemm(const SmatGemmArgs& a_in, int max_M, int max_N, int64_t groups, int bh, cudaStream_t st) {
-  if (groups <= 0 || max_M <= 0 || max_N <= 0) return cudaSuccess;
-  SmatGemmArgs a = a_in;
-  a.tilesN = (max_N + TILE - 1) / TILE;
-  const int tilesM = (max_M + TILE - 1) / TILE;
-  dim3 grid((unsigned)(tilesM * a.tilesN), (unsigned)groups, (unsigned)bh);
-  gemm_grouped_kernel<<<grid, 256, 0, st>>>(a);
-  return cudaGetLastError();
+template <typename T, int SD, int OD>
+static cudaError_t launch_tile_rows(const SmatTileArgs& a, int bh, cudaStream_t st) {
+  constexpr int smem = TileLayout<T, SD, OD>::SMEM;
+  cudaError_t err = cudaFuncSetAttribute(tile_rows_kernel<T, SD, OD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (err != cudaSuccess) return err;
+  const dim3 grid((unsigned)(a.jobs * a.NC * ((a.c + ROWS - 1) / ROWS)), (unsigned)bh);
+  return smat_launch_pdl(tile_rows_kernel<T, SD, OD>, grid, TILE_THREADS, smem, st, a);
 }
 
-cudaError_t smat_launch_scan(float* S, int64_t state_elems, int64_t NC, int bh, int64_t lo0, int64_t hi0, int64_t lo1,
-                             int64_t hi1, int reverse, cudaStream_t st) {
-  const int ranges = (hi1 > lo1) ? 2 : 1;
-  dim3 grid((unsigned)((state_elems / 4 + 255) / 256), (unsigned)bh, (unsigned)ranges);
-  scan_kernel<<<grid, 256, 0, st>>>(S, state_elems, NC, lo0, hi0, lo1, hi1, reverse);
-  return cudaGetLastError();
+cudaError_t smat_launch_tile_rows(const SmatTileArgs& a, int bf16, int score_dim, int out_dim, int bh, cudaStream_t st) {
+#define SMAT_TILE(SV, OV)                                                                                     \
+  if (score_dim == SV && out_dim == OV)                                                                       \
+    return bf16 ? launch_tile_rows<__nv_bfloat16, SV, OV>(a, bh, st) : launch_tile_rows<float, SV, OV>(a, bh, st);
+  SMAT_TILE(64, 64) SMAT_TILE(64, 128) SMAT_TILE(128, 64) SMAT_TILE(128, 128)
+#undef SMAT_TILE
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t smat_launch_scan(const SmatScanArgs& a, int64_t state_elems, int64_t NC, int bh, cudaStream_t st) {
+  const dim3 grid((unsigned)((state_elems / 4 + 255) / 256), (unsigned)bh, (unsigned)(2 * a.jobs));
+  return smat_launch_pdl(scan_kernel, grid, 256, 0, st, a, state_elems, NC);
 }
 
 int smat_tabulate_alg2_slab(int64_t rows_in, int64_t state_elems) {

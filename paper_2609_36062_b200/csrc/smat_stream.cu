@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 
 #include "smat_internal.h"
+#include "smat_launch.cuh"
 #include "smat_tc.cuh"
 
 namespace {
@@ -29,12 +30,10 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
   return make_float4(__low2float(lo), __high2float(lo), __low2float(hi), __high2float(hi));
 }
 
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+using tc::bulk_load;
+using tc::cp_async16;
+using tc::cp_async_commit;
+using tc::cp_async_wait;
 
 __device__ __forceinline__ void bulk_store(void* gmem, const void* smem, uint32_t bytes) {
   asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gmem), "r"(smem_u32(smem)), "r"(bytes)
@@ -46,20 +45,44 @@ __device__ __forceinline__ void bulk_store_wait_read() {
   asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
 }
 __device__ __forceinline__ void bulk_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_load(void* smem, const void* gmem, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(smem)),
-               "l"(gmem), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
-
-
 // ---- pooling ----------------------------------------------------------------------------------------------------
+// The items of all jobs in one list: job j's (head, group) pairs follow those of job j - 1.
+struct PoolList {
+  SmatPoolArgs a;
+  int64_t first[5];        // first item of job j; first[jobs] = all items
+};
+
+// One pass of the kernel: up to TK tokens of one item.
+template <int TK>
+struct PoolCursor {
+  const PoolList* l;
+  int64_t item, stride;
+  int job;
+  int64_t bh, k0, cnt;
+  SmatTokens tk;
+  __device__ PoolCursor(const PoolList& list, int64_t first, int64_t step) : l(&list), item(first), stride(step) { load(); }
+  __device__ bool valid() const { return item < l->first[l->a.jobs]; }
+  __device__ void load() {
+    k0 = 0; cnt = 0; job = 0;
+    if (!valid()) return;
+    while (item >= l->first[job + 1]) ++job;
+    const int64_t at = item - l->first[job];
+    bh = at / l->a.job[job].groups;
+    tk = smat_group_tokens(l->a.job[job].grp, bh, at - bh * l->a.job[job].groups);
+    cnt = tk.cnt;
+  }
+  __device__ bool last() const { return k0 + TK >= cnt; }
+  __device__ int tokens() const { const int64_t left = cnt - k0; return (int)(left < TK ? (left > 0 ? left : 0) : TK); }
+  __device__ void next() {
+    if (last()) { item += stride; load(); } else k0 += TK;
+  }
+};
+
+// Two token buffers alternate over the passes, also inside a group of many tokens: the next pass's rows (of the same
+// group or of the next item) travel while this pass is summed.
 template <int R, int PD, typename T>
-__global__ void __launch_bounds__(256) pool_stream_kernel(const T* __restrict__ A, const T* __restrict__ Bm,
-                                                          float* __restrict__ state, SmatGroupSpec grp, int64_t Tlen,
-                                                          int64_t groups, int64_t items) {
-  constexpr int TK = sizeof(T) == 2 ? 32 : 16;  // tokens staged per tile
+__global__ void __launch_bounds__(256) pool_stream_kernel(const __grid_constant__ PoolList list, int64_t Tlen) {
+  constexpr int TK = sizeof(T) == 2 ? 32 : 16;  // tokens staged per pass
   constexpr int NJ4 = PD / 4;
   constexpr int NG = 256 / NJ4;
   constexpr int NS = R / NG;
@@ -68,126 +91,132 @@ __global__ void __launch_bounds__(256) pool_stream_kernel(const T* __restrict__ 
   float* outb = reinterpret_cast<float*>(smem_raw);                  // [R*PD]
   T* a_raw = reinterpret_cast<T*>(smem_raw + R * PD * 4);            // [2][TK][R]
   T* b_raw = a_raw + 2 * TK * R;                                     // [2][TK][PD]
+  pdl_trigger();
   const int tid = threadIdx.x;
   const int j4 = tid % NJ4, ig = tid / NJ4;
 
-  auto prefetch = [&](int64_t item, int buf) {  // first tile of tokens of an item, raw, through cp.async
-    if (item < items) {
-      const int64_t bh = item / groups, g = item - bh * groups;
-      const SmatTokens tk = smat_group_tokens(grp, bh, g);
-      const int64_t cnt = tk.cnt;
-      const int kn = (int)(cnt < TK ? cnt : TK);
-      const T* Ab = A + bh * Tlen * R;
-      const T* Bb = Bm + bh * Tlen * PD;
+  auto fetch = [&](const PoolCursor<TK>& c, int buf) {
+    if (c.valid()) {
+      const int kn = c.tokens();
+      const T* Ab = static_cast<const T*>(list.a.job[c.job].a) + c.bh * Tlen * R;
+      const T* Bb = static_cast<const T*>(list.a.job[c.job].b) + c.bh * Tlen * PD;
       for (int idx = tid; idx < kn * RC; idx += 256) {
-        const int k = idx / RC, c = idx - k * RC;
-        cp_async16(reinterpret_cast<uint8_t*>(a_raw + (buf * TK + k) * R) + c * 16,
-                   reinterpret_cast<const uint8_t*>(Ab + tk.at(k) * R) + c * 16);
+        const int k = idx / RC, ch = idx - k * RC;
+        cp_async16(reinterpret_cast<uint8_t*>(a_raw + (buf * TK + k) * R) + ch * 16,
+                   reinterpret_cast<const uint8_t*>(Ab + c.tk.at(c.k0 + k) * R) + ch * 16);
       }
       for (int idx = tid; idx < kn * PC; idx += 256) {
-        const int k = idx / PC, c = idx - k * PC;
-        cp_async16(reinterpret_cast<uint8_t*>(b_raw + (buf * TK + k) * PD) + c * 16,
-                   reinterpret_cast<const uint8_t*>(Bb + tk.at(k) * PD) + c * 16);
+        const int k = idx / PC, ch = idx - k * PC;
+        cp_async16(reinterpret_cast<uint8_t*>(b_raw + (buf * TK + k) * PD) + ch * 16,
+                   reinterpret_cast<const uint8_t*>(Bb + c.tk.at(c.k0 + k) * PD) + ch * 16);
       }
     }
     cp_async_commit();
   };
 
-  prefetch(blockIdx.x, 0);
-  int n = 0;
-  for (int64_t item = blockIdx.x; item < items; item += gridDim.x, ++n) {
+  pdl_wait();   // (the token lists of a routed call come from the kernel before)
+  PoolCursor<TK> cur(list, blockIdx.x, gridDim.x);
+  fetch(cur, 0);
+  float4 acc[NS];
+  for (int n = 0; cur.valid(); ++n) {
     const int buf = n & 1;
-    prefetch(item + gridDim.x, buf ^ 1);
+    PoolCursor<TK> nxt = cur;
+    nxt.next();
+    fetch(nxt, buf ^ 1);
     cp_async_wait<1>();
     __syncthreads();
-    const int64_t bh = item / groups, g = item - bh * groups;
-    const SmatTokens tk = smat_group_tokens(grp, bh, g);
-    const int64_t cnt = tk.cnt;
-    float4 acc[NS];
+    if (cur.k0 == 0) {
 #pragma unroll
-    for (int s = 0; s < NS; ++s) acc[s] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int64_t k0 = 0; k0 < cnt; k0 += TK) {
-      const int kn = (int)((cnt - k0) < TK ? (cnt - k0) : TK);
-      if (k0 > 0) {  // groups with more than one tile of tokens: fetch the further tiles in place
-        __syncthreads();
-        const T* Ab = A + bh * Tlen * R;
-        const T* Bb = Bm + bh * Tlen * PD;
-        for (int idx = tid; idx < kn * RC; idx += 256) {
-          const int k = idx / RC, c = idx - k * RC;
-          cp_async16(reinterpret_cast<uint8_t*>(a_raw + (buf * TK + k) * R) + c * 16,
-                     reinterpret_cast<const uint8_t*>(Ab + tk.at(k0 + k) * R) + c * 16);
-        }
-        for (int idx = tid; idx < kn * PC; idx += 256) {
-          const int k = idx / PC, c = idx - k * PC;
-          cp_async16(reinterpret_cast<uint8_t*>(b_raw + (buf * TK + k) * PD) + c * 16,
-                     reinterpret_cast<const uint8_t*>(Bb + tk.at(k0 + k) * PD) + c * 16);
-        }
-        cp_async_commit();
-        cp_async_wait<0>();
-        __syncthreads();
-      }
-      const T* as = a_raw + buf * TK * R;
-      const T* bs = b_raw + buf * TK * PD;
-      for (int k = 0; k < kn; ++k) {
-        const float4 b4 = load4(bs + k * PD + j4 * 4);
-#pragma unroll
-        for (int s = 0; s < NS; ++s) acc[s] = fma4(to_float(as[k * R + ig + s * NG]), b4, acc[s]);
-      }
+      for (int s = 0; s < NS; ++s) acc[s] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    // the previous item's bulk store reads the same buffer: it must have finished reading (the other CTA
-    // resident on this SM keeps the memory pipe busy meanwhile)
-    if (tid == 0) bulk_store_wait_read<0>();
-    __syncthreads();
-    float* ob = outb;
+    const int kn = cur.tokens();
+    const T* as = a_raw + buf * TK * R;
+    const T* bs = b_raw + buf * TK * PD;
+    for (int k = 0; k < kn; ++k) {
+      const float4 b4 = load4(bs + k * PD + j4 * 4);
 #pragma unroll
-    for (int s = 0; s < NS; ++s) *reinterpret_cast<float4*>(ob + (ig + s * NG) * PD + j4 * 4) = acc[s];
-    tc::fence_proxy_async();
-    __syncthreads();
-    if (tid == 0) bulk_store(state + item * (int64_t)(R * PD), ob, R * PD * 4);
+      for (int s = 0; s < NS; ++s) acc[s] = fma4(to_float(as[k * R + ig + s * NG]), b4, acc[s]);
+    }
+    if (cur.last()) {
+      // the previous item's bulk store reads the same buffer: it must have finished reading (the other CTA
+      // resident on this SM keeps the memory pipe busy meanwhile)
+      if (tid == 0) bulk_store_wait_read<0>();
+      __syncthreads();
+#pragma unroll
+      for (int s = 0; s < NS; ++s) *reinterpret_cast<float4*>(outb + (ig + s * NG) * PD + j4 * 4) = acc[s];
+      tc::fence_proxy_async();
+      __syncthreads();
+      if (tid == 0) bulk_store(list.a.job[cur.job].state + (cur.item - list.first[cur.job]) * (int64_t)(R * PD), outb, R * PD * 4);
+    } else {
+      __syncthreads();   // the buffer just read is the next fetch's target
+    }
+    cur = nxt;
   }
   if (tid == 0) bulk_store_wait_all();
   cp_async_wait<0>();
 }
 
 // ---- routed read ----------------------------------------------------------------------------------------------------
+struct ReadList {
+  SmatReadArgs a;
+  int64_t first[4];
+};
+
 // Two CTAs share an SM; each owns one 64 KB state buffer, so one CTA's contraction overlaps the other's bulk load.
-template <int R, int PD, int TRANS, typename T>
-__global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const T* __restrict__ X,
-                                                                   const float* __restrict__ state,
-                                                                   const float* acc_in, float* acc_out,
-                                                                   SmatGroupSpec grp, int64_t Tlen, int64_t groups,
-                                                                   int64_t items, int* status) {
-  constexpr int KT = 8;
-  constexpr int NJ4 = PD / 4;
-  constexpr int NG = 256 / NJ4;
+template <int R, int PD, typename T>
+struct ReadLayout {
+  static constexpr int KT = 8;                              // tokens per pass over a state
+  static constexpr int NJ4 = PD / 4, NG = 256 / NJ4;
+  static constexpr int XM = R > PD ? R : PD;
+  static constexpr int RED = KT * R > NG * KT * PD ? KT * R : NG * KT * PD;
+  static constexpr int SMEM = R * PD * 4 + RED * 4 + 2 * KT * XM * (int)sizeof(T) + KT * XM * 4 + 64;
+};
+
+template <int R, int PD, typename T>
+__global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_constant__ ReadList list, int64_t Tlen,
+                                                                   int* status) {
+  using L = ReadLayout<R, PD, T>;
+  constexpr int KT = L::KT, NJ4 = L::NJ4, NG = L::NG;
   constexpr int RPG = R / NG;
-  constexpr int XD = TRANS ? PD : R;
-  constexpr int OD = TRANS ? R : PD;
-  constexpr int RED = TRANS ? KT * R : NG * KT * PD;
-  constexpr int XC = XD * (int)sizeof(T) / 16;  // 16-byte chunks per x row
   extern __shared__ __align__(128) uint8_t smem_raw[];
   float* Sb = reinterpret_cast<float*>(smem_raw);        // [R*PD]
   float* red = Sb + R * PD;                              // [RED]
-  T* Xraw = reinterpret_cast<T*>(red + RED);             // [2][KT][XD] raw rows of the first KT tokens of an item
-  float* Xs = reinterpret_cast<float*>(Xraw + 2 * KT * XD);  // [KT][XD]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(Xs + KT * XD);
+  T* Xraw = reinterpret_cast<T*>(red + L::RED);          // [2][KT][XM] raw rows of the first KT tokens of an item
+  float* Xs = reinterpret_cast<float*>(Xraw + 2 * KT * L::XM);  // [KT][XM]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(Xs + KT * L::XM);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(bar + 1);
+  pdl_trigger();
   const tc::WaitCtx wc{cta_abort, status};
   const int tid = threadIdx.x;
   const int j4 = tid % NJ4, ig = tid / NJ4;
   constexpr uint32_t SBYTES = R * PD * 4;
-
+  const int64_t items = list.first[list.a.jobs];
+  auto job_of = [&](int64_t item) {
+    int j = 0;
+    while (item >= list.first[j + 1]) ++j;
+    return j;
+  };
+  auto tokens_of = [&](int64_t item, int j, int64_t* bh) {
+    const int64_t at = item - list.first[j];
+    *bh = at / list.a.job[j].groups;
+    return smat_group_tokens(list.a.job[j].grp, *bh, at - *bh * list.a.job[j].groups);
+  };
+  auto state_of = [&](int64_t item) {
+    const int j = job_of(item);
+    return list.a.job[j].state + (item - list.first[j]) * (int64_t)(R * PD);
+  };
   auto prefetch_x = [&](int64_t item, int buf) {
     if (item < items) {
-      const int64_t bh = item / groups, g = item - bh * groups;
-      const SmatTokens tk = smat_group_tokens(grp, bh, g);
-      const int64_t cnt = tk.cnt;
-      const int kn = (int)(cnt < KT ? cnt : KT);
-      const T* Xb = X + bh * Tlen * XD;
-      for (int idx = tid; idx < kn * XC; idx += 256) {
-        const int k = idx / XC, c = idx - k * XC;
-        cp_async16(reinterpret_cast<uint8_t*>(Xraw + (buf * KT + k) * XD) + c * 16,
-                   reinterpret_cast<const uint8_t*>(Xb + tk.at(k) * XD) + c * 16);
+      const int j = job_of(item);
+      int64_t bh;
+      const SmatTokens tk = tokens_of(item, j, &bh);
+      const int xd = list.a.job[j].trans ? PD : R, xc = xd * (int)sizeof(T) / 16;   // 16-byte chunks per x row
+      const int kn = (int)(tk.cnt < KT ? tk.cnt : KT);
+      const T* Xb = static_cast<const T*>(list.a.job[j].x) + bh * Tlen * xd;
+      for (int idx = tid; idx < kn * xc; idx += 256) {
+        const int k = idx / xc, c = idx - k * xc;
+        cp_async16(reinterpret_cast<uint8_t*>(Xraw + (buf * KT + k) * L::XM) + c * 16,
+                   reinterpret_cast<const uint8_t*>(Xb + tk.at(k) * xd) + c * 16);
       }
     }
     cp_async_commit();
@@ -197,20 +226,24 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const T* __re
     *cta_abort = 0;
     tc::mbar_init(bar, 1);
     tc::fence_barrier_init();
-    if ((int64_t)blockIdx.x < items) {
-      tc::mbar_expect_tx(bar, SBYTES);
-      bulk_load(Sb, state + (int64_t)blockIdx.x * (R * PD), SBYTES, bar);
-    }
+  }
+  pdl_wait();
+  if (tid == 0 && (int64_t)blockIdx.x < items) {
+    tc::mbar_expect_tx(bar, SBYTES);
+    bulk_load(Sb, state_of(blockIdx.x), SBYTES, bar);
   }
   prefetch_x(blockIdx.x, 0);
   __syncthreads();
   int n = 0;
   for (int64_t item = blockIdx.x; item < items; item += gridDim.x, ++n) {
     const int buf = n & 1;
-    const int64_t bh = item / groups, g = item - bh * groups;
-    const SmatTokens tk = smat_group_tokens(grp, bh, g);
+    const int j = job_of(item);
+    int64_t bh;
+    const SmatTokens tk = tokens_of(item, j, &bh);
     const int64_t cnt = tk.cnt;
-    const T* Xb = X + bh * Tlen * XD;
+    const int trans = list.a.job[j].trans, xd = trans ? PD : R, od = trans ? R : PD;
+    const T* Xb = static_cast<const T*>(list.a.job[j].x) + bh * Tlen * xd;
+    float* out = list.a.job[j].out + bh * Tlen * od;
     const float4* S4 = reinterpret_cast<const float4*>(Sb);
     prefetch_x(item + gridDim.x, buf ^ 1);
     cp_async_wait<1>();
@@ -218,14 +251,14 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const T* __re
     __syncthreads();
     for (int64_t k0 = 0; k0 < cnt && ok; k0 += KT) {
       const int kn = (int)((cnt - k0) < KT ? (cnt - k0) : KT);
-      for (int idx = tid; idx < KT * XD; idx += 256) {
-        const int k = idx / XD, i = idx % XD;
+      for (int idx = tid; idx < KT * xd; idx += 256) {
+        const int k = idx / xd, i = idx - k * xd;
         float v = 0.f;
-        if (k < kn) v = k0 == 0 ? to_float(Xraw[(buf * KT + k) * XD + i]) : to_float(Xb[tk.at(k0 + k) * XD + i]);
-        Xs[idx] = v;
+        if (k < kn) v = k0 == 0 ? to_float(Xraw[(buf * KT + k) * L::XM + i]) : to_float(Xb[tk.at(k0 + k) * xd + i]);
+        Xs[k * L::XM + i] = v;
       }
       __syncthreads();
-      if (!TRANS) {
+      if (!trans) {
         float4 acc[KT];
 #pragma unroll
         for (int k = 0; k < KT; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -234,18 +267,17 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const T* __re
           const int i = ig * RPG + s;
           const float4 u = S4[i * NJ4 + j4];
 #pragma unroll
-          for (int k = 0; k < KT; ++k) acc[k] = fma4(Xs[k * XD + i], u, acc[k]);
+          for (int k = 0; k < KT; ++k) acc[k] = fma4(Xs[k * L::XM + i], u, acc[k]);
         }
 #pragma unroll
         for (int k = 0; k < KT; ++k) *reinterpret_cast<float4*>(red + (ig * KT + k) * PD + j4 * 4) = acc[k];
         __syncthreads();
         for (int idx = tid; idx < kn * PD; idx += 256) {
-          const int k = idx / PD, j = idx % PD;
+          const int k = idx / PD, jj = idx % PD;
           float v = 0.f;
 #pragma unroll
-          for (int w = 0; w < NG; ++w) v += red[(w * KT + k) * PD + j];
-          const int64_t off = (bh * Tlen + tk.at(k0 + k)) * OD + j;
-          acc_out[off] = v + (acc_in ? acc_in[off] : 0.f);
+          for (int w = 0; w < NG; ++w) v += red[(w * KT + k) * PD + jj];
+          out[tk.at(k0 + k) * PD + jj] = v;
         }
       } else {
 #pragma unroll 2
@@ -255,7 +287,7 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const T* __re
           float part[KT];
 #pragma unroll
           for (int k = 0; k < KT; ++k) {
-            const float4 x4 = *reinterpret_cast<const float4*>(Xs + k * XD + j4 * 4);
+            const float4 x4 = *reinterpret_cast<const float4*>(Xs + k * L::XM + j4 * 4);
             part[k] = u.x * x4.x + u.y * x4.y + u.z * x4.z + u.w * x4.w;
           }
 #pragma unroll
@@ -269,8 +301,7 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const T* __re
         __syncthreads();
         for (int idx = tid; idx < kn * R; idx += 256) {
           const int k = idx / R, i = idx % R;
-          const int64_t off = (bh * Tlen + tk.at(k0 + k)) * OD + i;
-          acc_out[off] = red[k * R + i] + (acc_in ? acc_in[off] : 0.f);
+          out[tk.at(k0 + k) * R + i] = red[k * R + i];
         }
       }
       __syncthreads();
@@ -280,7 +311,7 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const T* __re
       const int64_t nxt = item + gridDim.x;
       if (nxt < items && !*cta_abort) {
         tc::mbar_expect_tx(bar, SBYTES);
-        bulk_load(Sb, state + nxt * (int64_t)(R * PD), SBYTES, bar);
+        bulk_load(Sb, state_of(nxt), SBYTES, bar);
       }
     }
   }
@@ -304,59 +335,54 @@ int sm_count() {
 }
 
 template <int R, int PD, typename T>
-cudaError_t launch_pool(const void* A, const void* Bm, float* state, const SmatGroupSpec& grp, int64_t Tlen,
-                        int64_t groups, int bh, cudaStream_t st) {
+cudaError_t launch_pool(const PoolList& list, int64_t Tlen, cudaStream_t st) {
   constexpr int TK = sizeof(T) == 2 ? 32 : 16;
   const size_t smem = R * PD * 4 + 2 * TK * (R + PD) * sizeof(T);
   cudaError_t err = set_smem(pool_stream_kernel<R, PD, T>, smem);
   if (err != cudaSuccess) return err;
-  const int64_t items = groups * bh;
+  const int64_t items = list.first[list.a.jobs];
   const int per_sm = smem <= 110 * 1024 ? 2 : 1;
   const int64_t grid = items < (int64_t)sm_count() * per_sm ? items : (int64_t)sm_count() * per_sm;
-  pool_stream_kernel<R, PD, T><<<(unsigned)grid, 256, smem, st>>>(static_cast<const T*>(A), static_cast<const T*>(Bm),
-                                                                   state, grp, Tlen, groups, items);
-  return cudaGetLastError();
+  return smat_launch_pdl(pool_stream_kernel<R, PD, T>, dim3((unsigned)grid), 256, smem, st, list, Tlen);
 }
 
-template <int R, int PD, int TRANS, typename T>
-cudaError_t launch_read(const void* X, const float* state, const float* acc_in, float* acc_out,
-                        const SmatGroupSpec& grp, int64_t Tlen, int64_t groups, int bh, int* status, cudaStream_t st) {
-  constexpr int KT = 8;
-  constexpr int NG = 256 / (PD / 4);
-  constexpr int XD = TRANS ? PD : R;
-  const size_t smem = R * PD * 4 + (TRANS ? KT * R : NG * KT * PD) * 4 + 2 * KT * XD * sizeof(T) + KT * XD * 4 + 64;
-  cudaError_t err = set_smem(state_read_stream_kernel<R, PD, TRANS, T>, smem);
+template <int R, int PD, typename T>
+cudaError_t launch_read(const ReadList& list, int64_t Tlen, int* status, cudaStream_t st) {
+  const size_t smem = ReadLayout<R, PD, T>::SMEM;
+  cudaError_t err = set_smem(state_read_stream_kernel<R, PD, T>, smem);
   if (err != cudaSuccess) return err;
-  const int64_t items = groups * bh;
-  const int per_sm = smem <= 110 * 1024 ? 2 : 1;
+  const int64_t items = list.first[list.a.jobs];
+  const int per_sm = smem <= 112 * 1024 ? 2 : 1;
   const int64_t grid = items < (int64_t)sm_count() * per_sm ? items : (int64_t)sm_count() * per_sm;
-  state_read_stream_kernel<R, PD, TRANS, T><<<(unsigned)grid, 256, smem, st>>>(
-      static_cast<const T*>(X), state, acc_in, acc_out, grp, Tlen, groups, items, status);
-  return cudaGetLastError();
+  return smat_launch_pdl(state_read_stream_kernel<R, PD, T>, dim3((unsigned)grid), 256, smem, st, list, Tlen, status);
 }
 
 }  // namespace
 
-cudaError_t smat_launch_pool(const void* A, const void* Bm, int bf16, float* state, const SmatGroupSpec& grp,
-                             int64_t Tlen, int64_t groups, int bh, int r, int p, cudaStream_t st) {
-#define SMAT_POOL(RV, PV)                                                                                       \
-  if (r == RV && p == PV)                                                                                       \
-    return bf16 ? launch_pool<RV, PV, __nv_bfloat16>(A, Bm, state, grp, Tlen, groups, bh, st)                   \
-                : launch_pool<RV, PV, float>(A, Bm, state, grp, Tlen, groups, bh, st);
+cudaError_t smat_launch_pool(const SmatPoolArgs& a, int bf16, int64_t Tlen, int bh, int r, int p, cudaStream_t st) {
+  PoolList list;
+  list.a = a;
+  list.first[0] = 0;
+  for (int j = 0; j < a.jobs; ++j) list.first[j + 1] = list.first[j] + a.job[j].groups * bh;
+#define SMAT_POOL(RV, PV)                                                                                          \
+  if (r == RV && p == PV)                                                                                          \
+    return bf16 ? launch_pool<RV, PV, __nv_bfloat16>(list, Tlen, st) : launch_pool<RV, PV, float>(list, Tlen, st);
   SMAT_POOL(128, 128) SMAT_POOL(64, 64) SMAT_POOL(64, 128) SMAT_POOL(128, 64)
 #undef SMAT_POOL
   return cudaErrorInvalidValue;
 }
 
-cudaError_t smat_launch_state_read(const void* X, int bf16, const float* state, int transposed, const float* acc_in,
-                                   float* acc_out, const SmatGroupSpec& grp, int64_t Tlen, int64_t groups, int bh,
-                                   int r, int p, int* status, cudaStream_t st) {
-#define SMAT_READ(RV, PV, TV)                                                                                        \
-  if (r == RV && p == PV && transposed == TV)                                                                        \
-    return bf16 ? launch_read<RV, PV, TV, __nv_bfloat16>(X, state, acc_in, acc_out, grp, Tlen, groups, bh, status, st) \
-                : launch_read<RV, PV, TV, float>(X, state, acc_in, acc_out, grp, Tlen, groups, bh, status, st);
-  SMAT_READ(128, 128, 0) SMAT_READ(64, 64, 0) SMAT_READ(64, 128, 0) SMAT_READ(128, 64, 0)
-  SMAT_READ(128, 128, 1) SMAT_READ(64, 64, 1) SMAT_READ(64, 128, 1) SMAT_READ(128, 64, 1)
+cudaError_t smat_launch_state_read(const SmatReadArgs& a, int bf16, int64_t Tlen, int bh, int r, int p, int* status,
+                                   cudaStream_t st) {
+  ReadList list;
+  list.a = a;
+  list.first[0] = 0;
+  for (int j = 0; j < a.jobs; ++j) list.first[j + 1] = list.first[j] + a.job[j].groups * bh;
+#define SMAT_READ(RV, PV)                                                                        \
+  if (r == RV && p == PV)                                                                        \
+    return bf16 ? launch_read<RV, PV, __nv_bfloat16>(list, Tlen, status, st)                     \
+                : launch_read<RV, PV, float>(list, Tlen, status, st);
+  SMAT_READ(128, 128) SMAT_READ(64, 64) SMAT_READ(64, 128) SMAT_READ(128, 64)
 #undef SMAT_READ
   return cudaErrorInvalidValue;
 }
