@@ -4,11 +4,12 @@
 // and with scalar gates (Sec. 3.2; the table then holds the keys rescaled to the block boundary)
 //     S_t = a_t S_{t-1} + k_t v_tᵀ ,   g_t = a_t g_{t-1} ,   o_t = q_tᵀ (g_t U_type(t) + S_t) ,
 // O(r p) work per token and head.  One step reads S and one type state and writes S back: it is a stream over
-// 3 states per head, so it runs on the plain ALUs with vectorised loads, one CTA per head.
+// 3 states per head, so it runs on the plain ALUs with vectorised loads.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include "smat_internal.h"
+#include "smat_launch.cuh"
 
 namespace {
 
@@ -38,42 +39,82 @@ __device__ __forceinline__ float4 load_u4<__nv_bfloat16>(const __nv_bfloat16* p)
                      __uint_as_float(w.y & 0xffff0000u));
 }
 
-// One CTA per head, blockDim = 256.  Thread (i0 = tid / (p / 4), j4 = tid % (p / 4)) walks the rows i0, i0 + R, ...
-// of the r x p state with its four columns, so that a warp touches whole 128-byte lines.
-template <typename T, typename TU>
-__global__ void __launch_bounds__(256) decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k,
+// One CTA per head and 32 columns of the state (128 bytes of a row), so that even a handful of sequences spreads over
+// the SMs.  Thread (row tid / 8, columns 4 (tid % 8)) walks the rows 32 at a time with every load of its share in
+// flight before the first use: a CTA's 24 KB are one round trip to memory.  The partial outputs meet by shuffles and
+// one row of shared memory per warp (no atomics: the sum's order is fixed).  Bound by the 84 MB a step of 512 heads
+// moves: 15.7 us (12.7 at the HBM rate), where one CTA per head with one row pass in flight at a time took 22.1.
+constexpr int DEC_COLS = 32, DEC_ROWS = 32, DEC_THREADS = 256;
+
+template <typename T, typename TU, int PASSES>
+__global__ void __launch_bounds__(DEC_THREADS) decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k,
                                                           const T* __restrict__ v, T* __restrict__ o,
                                                           float* __restrict__ S, const TU* __restrict__ U, int64_t type,
-                                                          int64_t types, int r, int p, const float* __restrict__ log_a,
+                                                          int64_t types, int p, const float* __restrict__ log_a,
                                                           float* __restrict__ log_g) {
-  __shared__ float s_q[128], s_k[128], s_o[128];
-  const int bh = blockIdx.x, tid = threadIdx.x;
-  // gated: a = this token's gate, g = the product of the gates since the block boundary (kept as its logarithm)
-  float a = 1.f, g = 1.f, lg = 0.f;
-  if (log_a) { lg = log_g[bh] + log_a[bh]; a = __expf(log_a[bh]); g = __expf(lg); }
-  const int cols4 = p / 4, rows_per_pass = 256 / cols4;
-  const int j = (tid % cols4) * 4, i0 = tid / cols4;
-  if (tid < r) { s_q[tid] = to_f32(q[(int64_t)bh * r + tid]); s_k[tid] = to_f32(k[(int64_t)bh * r + tid]); }
-  if (tid < p) s_o[tid] = 0.f;
-  __syncthreads();
+  constexpr int r = PASSES * DEC_ROWS;
+  __shared__ float part[DEC_THREADS / 32][DEC_COLS];
+  pdl_trigger();
+  const int bh = blockIdx.y, tid = threadIdx.x, j0 = blockIdx.x * DEC_COLS;
+  const int j = j0 + (tid & 7) * 4, i0 = tid >> 3;
+  pdl_wait();
+  float* Sh = S + (int64_t)bh * r * p + j;
+  const TU* Uh = U + ((int64_t)bh * types + type) * r * p + j;
+  float4 s[PASSES], u[PASSES];
+  float qi[PASSES], ki[PASSES];
+#pragma unroll
+  for (int n = 0; n < PASSES; ++n) {
+    const int64_t off = (int64_t)(n * DEC_ROWS + i0) * p;
+    s[n] = *reinterpret_cast<const float4*>(Sh + off);
+    u[n] = load_u4<TU>(Uh + off);
+  }
+#pragma unroll
+  for (int n = 0; n < PASSES; ++n) {
+    qi[n] = to_f32(q[(int64_t)bh * r + n * DEC_ROWS + i0]);
+    ki[n] = to_f32(k[(int64_t)bh * r + n * DEC_ROWS + i0]);
+  }
   const T* vrow = v + (int64_t)bh * p + j;
   const float v0 = to_f32(vrow[0]), v1 = to_f32(vrow[1]), v2 = to_f32(vrow[2]), v3 = to_f32(vrow[3]);
-  float* Sh = S + (int64_t)bh * r * p;
-  const TU* Uh = U + ((int64_t)bh * types + type) * r * p;
-  float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-  for (int i = i0; i < r; i += rows_per_pass) {
-    float4 s = *reinterpret_cast<const float4*>(Sh + (int64_t)i * p + j);
-    const float ki = s_k[i], qi = s_q[i];
-    s.x = fmaf(ki, v0, a * s.x); s.y = fmaf(ki, v1, a * s.y); s.z = fmaf(ki, v2, a * s.z); s.w = fmaf(ki, v3, a * s.w);
-    *reinterpret_cast<float4*>(Sh + (int64_t)i * p + j) = s;     // S_t = a_t S_{t-1} + k vᵀ
-    const float4 u = load_u4<TU>(Uh + (int64_t)i * p + j);
-    a0 = fmaf(qi, fmaf(g, u.x, s.x), a0); a1 = fmaf(qi, fmaf(g, u.y, s.y), a1);
-    a2 = fmaf(qi, fmaf(g, u.z, s.z), a2); a3 = fmaf(qi, fmaf(g, u.w, s.w), a3);
+  // gated: a = this token's gate, g = the product of the gates since the block boundary (kept as its logarithm)
+  float a = 1.f, g = 1.f;
+  float lg = 0.f;
+  if (log_a) { lg = log_g[bh] + log_a[bh]; a = __expf(log_a[bh]); g = __expf(lg); }
+  float o4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int n = 0; n < PASSES; ++n) {
+    s[n].x = fmaf(ki[n], v0, a * s[n].x); s[n].y = fmaf(ki[n], v1, a * s[n].y);
+    s[n].z = fmaf(ki[n], v2, a * s[n].z); s[n].w = fmaf(ki[n], v3, a * s[n].w);
+    *reinterpret_cast<float4*>(Sh + (int64_t)(n * DEC_ROWS + i0) * p) = s[n];     // S_t = a_t S_{t-1} + k vᵀ
+    o4[0] = fmaf(qi[n], fmaf(g, u[n].x, s[n].x), o4[0]); o4[1] = fmaf(qi[n], fmaf(g, u[n].y, s[n].y), o4[1]);
+    o4[2] = fmaf(qi[n], fmaf(g, u[n].z, s[n].z), o4[2]); o4[3] = fmaf(qi[n], fmaf(g, u[n].w, s[n].w), o4[3]);
   }
-  atomicAdd(&s_o[j], a0); atomicAdd(&s_o[j + 1], a1); atomicAdd(&s_o[j + 2], a2); atomicAdd(&s_o[j + 3], a3);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {   // the four rows a warp holds in each of its passes
+    o4[c] += __shfl_xor_sync(0xffffffffu, o4[c], 8);
+    o4[c] += __shfl_xor_sync(0xffffffffu, o4[c], 16);
+  }
+  if ((tid & 31) < 8) *reinterpret_cast<float4*>(&part[tid >> 5][(tid & 7) * 4]) = make_float4(o4[0], o4[1], o4[2], o4[3]);
   __syncthreads();
-  if (tid < p) store_out(o + (int64_t)bh * p + tid, s_o[tid]);
-  if (log_a && tid == 0) log_g[bh] = lg;   // every thread read the old value before the first barrier
+  if (tid < DEC_COLS) {
+    float sum = 0.f;
+#pragma unroll
+    for (int w = 0; w < DEC_THREADS / 32; ++w) sum += part[w][tid];
+    store_out(o + (int64_t)bh * p + j0 + tid, sum);
+  }
+  if (log_a) {   // gated launches cluster the CTAs of a head: the running gate moves on once all of them have read it
+    asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+    if (blockIdx.x == 0 && tid == 0) log_g[bh] = lg;
+  }
+}
+
+template <typename T, typename TU>
+cudaError_t launch_step(const void* q, const void* k, const void* v, void* o, float* S, const void* U, int64_t type,
+                        int64_t types, int r, int p, int bh, cudaStream_t st, const float* log_a, float* log_g) {
+  auto kernel = r == 64 ? decode_step_kernel<T, TU, 2> : decode_step_kernel<T, TU, 4>;
+  const unsigned slices = (unsigned)(p / DEC_COLS);
+  return smat_launch_pdl_cluster(kernel, dim3(slices, (unsigned)bh), DEC_THREADS, 0, log_a ? slices : 1u, st,
+                                 static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v),
+                                 static_cast<T*>(o), S, static_cast<const TU*>(U), type, types, p, log_a, log_g);
 }
 
 }  // namespace
@@ -83,22 +124,9 @@ __global__ void __launch_bounds__(256) decode_step_kernel(const T* __restrict__ 
 cudaError_t smat_launch_decode_step(const void* q, const void* k, const void* v, void* o, float* S, const void* U,
                                     int u_bf16, int in_bf16, int64_t type, int64_t types, int r, int p, int bh,
                                     cudaStream_t st, const float* log_a, float* log_g) {
-  if (r > 128 || p > 128 || p % 4 || 256 % (p / 4)) return cudaErrorInvalidValue;
-  if (in_bf16) {
-    const __nv_bfloat16 *qq = static_cast<const __nv_bfloat16*>(q), *kk = static_cast<const __nv_bfloat16*>(k),
-                        *vv = static_cast<const __nv_bfloat16*>(v);
-    __nv_bfloat16* oo = static_cast<__nv_bfloat16*>(o);
-    if (u_bf16)
-      decode_step_kernel<__nv_bfloat16, __nv_bfloat16><<<bh, 256, 0, st>>>(qq, kk, vv, oo, S, static_cast<const __nv_bfloat16*>(U),
-                                                                         type, types, r, p, log_a, log_g);
-    else
-      decode_step_kernel<__nv_bfloat16, float><<<bh, 256, 0, st>>>(qq, kk, vv, oo, S, static_cast<const float*>(U), type,
-                                                                 types, r, p, log_a, log_g);
-  } else {
-    if (u_bf16) return cudaErrorInvalidValue;
-    decode_step_kernel<float, float><<<bh, 256, 0, st>>>(static_cast<const float*>(q), static_cast<const float*>(k),
-                                                         static_cast<const float*>(v), static_cast<float*>(o), S,
-                                                         static_cast<const float*>(U), type, types, r, p, log_a, log_g);
-  }
-  return cudaGetLastError();
+  if ((r != 64 && r != 128) || (p != 64 && p != 128)) return cudaErrorInvalidValue;
+  if (!in_bf16)
+    return u_bf16 ? cudaErrorInvalidValue : launch_step<float, float>(q, k, v, o, S, U, type, types, r, p, bh, st, log_a, log_g);
+  return u_bf16 ? launch_step<__nv_bfloat16, __nv_bfloat16>(q, k, v, o, S, U, type, types, r, p, bh, st, log_a, log_g)
+                : launch_step<__nv_bfloat16, float>(q, k, v, o, S, U, type, types, r, p, bh, st, log_a, log_g);
 }
