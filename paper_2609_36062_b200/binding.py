@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libsmat.so: argument marshalling only, same names as the C boundary.
+"""Thin binding of libsmat.so: argument marshalling only, same names as the C boundary.  The passes and the decoding
+steps go through the native extension _smat_torch (checks, output allocation, launch), everything else through ctypes.
 
 Every step of the path runs inside the library's CUDA kernels.  PyTorch is used for device
 memory and streams.  There is no CPU fallback: if the shared library is missing or the device
@@ -168,6 +169,20 @@ def _stream(stream) -> int:
     return s.cuda_stream
 
 
+_ext = None
+
+
+def _extension():
+    """The native call layer (built in-tree with the library); raises if it is missing."""
+    global _ext
+    if _ext is None:
+        load_library()
+        from . import _smat_torch
+        _smat_torch.set_error(SmatError)
+        _ext = _smat_torch
+    return _ext
+
+
 _TORCH_DTYPE = {SMAT_F32: torch.float32, SMAT_BF16: torch.bfloat16}
 
 STATIC_MAX_TILES = 1024
@@ -226,6 +241,8 @@ class SmatPlan:
         _check(self.lib.smat_plan_create(ctypes.byref(handle), batch, heads, T, d_k, d_v, d, chunk, q_override,
                                          self.dtype_code, flags), "smat_plan_create")
         self.handle = handle
+        self._native = _extension().Plan(handle.value, batch, heads, T, d_k, d_v, int(self.dtype_code == SMAT_BF16))
+        self._ws_bytes = tuple(int(self.lib.smat_workspace_bytes(handle, i)) for i in (0, 1))
         self._ws = None
 
     def __del__(self):
@@ -255,7 +272,12 @@ class SmatPlan:
         return int(self.lib.smat_profile_table_element_bytes(self.handle))
 
     def workspace_bytes(self, for_backward: bool = False) -> int:
-        return int(self.lib.smat_workspace_bytes(self.handle, int(for_backward)))
+        return self._ws_bytes[bool(for_backward)]
+
+    def _own_workspace(self, for_backward: bool, like: torch.Tensor) -> torch.Tensor:
+        if not like.is_cuda:
+            raise ValueError("expected CUDA tensors")
+        return self.workspace(for_backward, like.device)
 
     def workspace(self, for_backward: bool = False, device="cuda") -> torch.Tensor:
         need = self.workspace_bytes(for_backward)
@@ -285,69 +307,24 @@ class SmatPlan:
             raise ValueError(f"{name}: expected contiguous {self.torch_dtype} of shape {(b, h, T, last)}, "
                              f"got {t.dtype} {tuple(t.shape)}")
 
-    def _check_routing(self, prof, typ):
-        b, h, _, _, _ = self.shape
-        g = self.geometry()
-        for name, t, count in (("prof", prof, g.n), ("type", typ, g.m)):
-            if not (t.is_cuda and t.dtype == torch.int32 and t.is_contiguous() and tuple(t.shape) == (b * h, count)):
-                raise ValueError(f"{name}: expected a contiguous CUDA int32 tensor of shape {(b * h, count)}")
-
     def forward(self, Q, K, V, O=None, workspace=None, stream=None, prof=None, type=None):
         """smat_forward, or smat_forward_routed when prof [batch*heads, n] and type [batch*heads, m] are given."""
-        _, _, _, dk, dv = self.shape
-        self._check_tensor(Q, dk, "Q"); self._check_tensor(K, dk, "K"); self._check_tensor(V, dv, "V")
-        if O is None:
-            O = torch.empty_like(V)
-        self._check_tensor(O, dv, "O")
-        ws = self.workspace(False, Q.device) if workspace is None else workspace
-        if prof is not None or type is not None:
-            self._check_routing(prof, type)
-            _check(self.lib.smat_forward_routed(self.handle, _ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(prof), _ptr(type),
-                                                _ptr(ws), ws.numel(), _stream(stream)), "smat_forward_routed")
-            return O
-        _check(self.lib.smat_forward(self.handle, _ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(ws), ws.numel(),
-                                     _stream(stream)), "smat_forward")
-        return O
+        ws = self._own_workspace(False, Q) if workspace is None else workspace
+        return self._native.forward(0, Q, K, V, None, O, ws, stream, prof, type)
 
     def backward(self, Q, K, V, dO, dQ=None, dK=None, dV=None, workspace=None, stream=None, prof=None, type=None):
-        _, _, _, dk, dv = self.shape
-        self._check_tensor(Q, dk, "Q"); self._check_tensor(K, dk, "K"); self._check_tensor(V, dv, "V")
-        self._check_tensor(dO, dv, "dO")
-        dQ = torch.empty_like(Q) if dQ is None else dQ
-        dK = torch.empty_like(K) if dK is None else dK
-        dV = torch.empty_like(V) if dV is None else dV
-        ws = self.workspace(True, Q.device) if workspace is None else workspace
-        if prof is not None or type is not None:
-            self._check_routing(prof, type)
-            _check(self.lib.smat_backward_routed(self.handle, _ptr(Q), _ptr(K), _ptr(V), _ptr(dO), _ptr(dQ), _ptr(dK),
-                                                 _ptr(dV), _ptr(prof), _ptr(type), _ptr(ws), ws.numel(), _stream(stream)),
-                   "smat_backward_routed")
-            return dQ, dK, dV
-        _check(self.lib.smat_backward(self.handle, _ptr(Q), _ptr(K), _ptr(V), _ptr(dO), _ptr(dQ), _ptr(dK), _ptr(dV),
-                                      _ptr(ws), ws.numel(), _stream(stream)), "smat_backward")
-        return dQ, dK, dV
+        ws = self._own_workspace(True, Q) if workspace is None else workspace
+        return self._native.backward(0, Q, K, V, None, None, dO, dQ, dK, dV, None, ws, stream, prof, type)
 
     # -- normalised output ------------------------------------------------------------------------
     def forward_normalized(self, Q, K, V, O=None, workspace=None, stream=None):
         """V: p - 1 value columns and the normaliser column last; O: normalised values and the normaliser last."""
-        _, _, _, dk, dv = self.shape
-        self._check_tensor(Q, dk, "Q"); self._check_tensor(K, dk, "K"); self._check_tensor(V, dv, "V")
-        O = torch.empty_like(V) if O is None else O
-        ws = self.workspace(False, Q.device) if workspace is None else workspace
-        _check(self.lib.smat_forward_normalized(self.handle, _ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(ws), ws.numel(),
-                                                _stream(stream)), "smat_forward_normalized")
-        return O
+        ws = self._own_workspace(False, Q) if workspace is None else workspace
+        return self._native.forward(2, Q, K, V, None, O, ws, stream, None, None)
 
     def backward_normalized(self, Q, K, V, O, dO, workspace=None, stream=None):
-        _, _, _, dk, dv = self.shape
-        self._check_tensor(Q, dk, "Q"); self._check_tensor(K, dk, "K"); self._check_tensor(V, dv, "V")
-        self._check_tensor(O, dv, "O"); self._check_tensor(dO, dv, "dO")
-        dQ, dK, dV = torch.empty_like(Q), torch.empty_like(K), torch.empty_like(V)
-        ws = self.workspace(True, Q.device) if workspace is None else workspace
-        _check(self.lib.smat_backward_normalized(self.handle, _ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(dO), _ptr(dQ),
-                                                 _ptr(dK), _ptr(dV), _ptr(ws), ws.numel(), _stream(stream)),
-               "smat_backward_normalized")
-        return dQ, dK, dV
+        ws = self._own_workspace(True, Q) if workspace is None else workspace
+        return self._native.backward(2, Q, K, V, None, O, dO, None, None, None, None, ws, stream, None, None)
 
     # -- scalar-gated variant ---------------------------------------------------------------------
     def _check_gates(self, log_a):
@@ -356,29 +333,12 @@ class SmatPlan:
             raise ValueError(f"log_a: expected a contiguous CUDA float32 tensor of shape {(b * h, T)}")
 
     def forward_gated(self, Q, K, V, log_a, O=None, workspace=None, stream=None):
-        _, _, _, dk, dv = self.shape
-        self._check_tensor(Q, dk, "Q"); self._check_tensor(K, dk, "K"); self._check_tensor(V, dv, "V")
-        self._check_gates(log_a)
-        O = torch.empty_like(V) if O is None else O
-        ws = self.workspace(False, Q.device) if workspace is None else workspace
-        _check(self.lib.smat_forward_gated(self.handle, _ptr(Q), _ptr(K), _ptr(V), _ptr(log_a), _ptr(O), _ptr(ws),
-                                           ws.numel(), _stream(stream)), "smat_forward_gated")
-        return O
+        ws = self._own_workspace(False, Q) if workspace is None else workspace
+        return self._native.forward(1, Q, K, V, log_a, O, ws, stream, None, None)
 
     def backward_gated(self, Q, K, V, log_a, dO, dQ=None, dK=None, dV=None, dlog_a=None, workspace=None, stream=None):
-        _, _, _, dk, dv = self.shape
-        self._check_tensor(Q, dk, "Q"); self._check_tensor(K, dk, "K"); self._check_tensor(V, dv, "V")
-        self._check_tensor(dO, dv, "dO")
-        self._check_gates(log_a)
-        dQ = torch.empty_like(Q) if dQ is None else dQ
-        dK = torch.empty_like(K) if dK is None else dK
-        dV = torch.empty_like(V) if dV is None else dV
-        dla = torch.empty_like(log_a) if dlog_a is None else dlog_a
-        ws = self.workspace(True, Q.device) if workspace is None else workspace
-        _check(self.lib.smat_backward_gated(self.handle, _ptr(Q), _ptr(K), _ptr(V), _ptr(log_a), _ptr(dO), _ptr(dQ),
-                                            _ptr(dK), _ptr(dV), _ptr(dla), _ptr(ws), ws.numel(), _stream(stream)),
-               "smat_backward_gated")
-        return dQ, dK, dV, dla
+        ws = self._own_workspace(True, Q) if workspace is None else workspace
+        return self._native.backward(1, Q, K, V, log_a, None, dO, dQ, dK, dV, dlog_a, ws, stream, None, None)
 
     # -- cached decoding -----------------------------------------------------------------------
     def decode_cache(self, device="cuda") -> torch.Tensor:
@@ -393,14 +353,7 @@ class SmatPlan:
                                           _stream(stream)), "smat_decode_begin")
 
     def decode_step(self, q, k, v, t: int, cache, o=None, stream=None):
-        b, h, _, dk, dv = self.shape
-        for name, x, dim in (("q", q, dk), ("k", k, dk), ("v", v, dv)):
-            if not (x.is_cuda and x.is_contiguous() and x.dtype == self.torch_dtype and tuple(x.shape) == (b, h, dim)):
-                raise ValueError(f"{name}: expected a contiguous CUDA tensor [{b}, {h}, {dim}] of the plan's dtype")
-        o = torch.empty_like(v) if o is None else o
-        _check(self.lib.smat_decode_step(self.handle, _ptr(q), _ptr(k), _ptr(v), int(t), _ptr(o), _ptr(cache), cache.numel(),
-                                         _stream(stream)), "smat_decode_step")
-        return o
+        return self._native.decode_step(q, k, v, None, t, cache, o, stream)
 
     def decode_begin_gated(self, K, V, log_a, cache, workspace=None, stream=None) -> None:
         _, _, _, dk, dv = self.shape
@@ -412,16 +365,9 @@ class SmatPlan:
                                                 _ptr(ws), ws.numel(), _stream(stream)), "smat_decode_begin_gated")
 
     def decode_step_gated(self, q, k, v, log_a_t, t: int, cache, o=None, stream=None):
-        b, h, _, dk, dv = self.shape
-        for name, x, dim in (("q", q, dk), ("k", k, dk), ("v", v, dv)):
-            if not (x.is_cuda and x.is_contiguous() and x.dtype == self.torch_dtype and tuple(x.shape) == (b, h, dim)):
-                raise ValueError(f"{name}: expected a contiguous CUDA tensor [{b}, {h}, {dim}] of the plan's dtype")
-        if not (log_a_t.is_cuda and log_a_t.is_contiguous() and log_a_t.dtype == torch.float32 and log_a_t.numel() == b * h):
-            raise ValueError(f"log_a_t: expected a contiguous CUDA fp32 tensor of {b * h} log-gates")
-        o = torch.empty_like(v) if o is None else o
-        _check(self.lib.smat_decode_step_gated(self.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(log_a_t), int(t), _ptr(o),
-                                               _ptr(cache), cache.numel(), _stream(stream)), "smat_decode_step_gated")
-        return o
+        if log_a_t is None:
+            raise ValueError("log_a_t: expected the log-gates of token t")
+        return self._native.decode_step(q, k, v, log_a_t, t, cache, o, stream)
 
     # -- verification exports ------------------------------------------------------------------
     def routing_indices(self):
