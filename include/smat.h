@@ -71,9 +71,8 @@ typedef enum { SMAT_F32 = 0, SMAT_BF16 = 1 } smat_dtype;
                                         with staged sums on the fp32 ALUs instead of the Radon stages on the tensor cores
                                         (which keep F, U and the stage intermediate in bf16) */
 
-#define SMAT_FLAG_D3_SHARED_SUMS 32u /* d = 3 with a prime beyond the tensor-core tabulation: form every q-term sum
-                                        straight from the shared-memory slab (one output row per thread) instead of
-                                        the register-resident form (K slopes x q offsets per thread) */
+#define SMAT_FLAG_D3_SHARED_SUMS 32u /* d = 3 with a prime from 19 on: form every q-term sum on the fp32 ALUs from the
+                                        shared-memory slab (one output row per thread) instead of on the tensor cores */
 
 #define SMAT_FLAG_SEPARATE_TILE_ADJOINTS 256u /* tensor-core backward: dQ, dK, dV of a tile by three launches of the general
                                                  tile-product kernel instead of the one fused kernel (for comparison) */

@@ -37,8 +37,8 @@
 // q = 11 also sends its output tiles off by TMA: the epilogue writes the rounded tile into the item's own ring slot
 // (as large as a tile, and dead once the MMAs have read it) in the box layout, and lane 0 of warp 18 issues the tile
 // stores and frees the slot; the bulk of the stores bypasses the LSU.
-// The kernel exists twice: radon_tc_kernel<false> for one stage per launch with every index through the MMAs (q = 13,
-// 17, 19 and the small primes), without cache hints, phase tables or ALU warps; radon_tc_kernel<true> with them.
+// The kernel exists twice: radon_tc_kernel<false> for one stage per launch with every index through the MMAs (q = 17
+// and the small primes), without cache hints, phase tables or ALU warps; radon_tc_kernel<true> with them.
 // (The tile-store path is written for several slots per item and several parts and is compiled into both, but the
 // launcher switches it on for q = 11 only: it was measured slower than the direct stores for q = 13 and 17.)
 #include <cuda.h>
@@ -46,11 +46,14 @@
 #include <cuda_runtime.h>
 
 #include "smat_internal.h"
+#include "smat_radon.cuh"
 #include "smat_tc.cuh"
 
 namespace {
 
 using namespace tc;
+using tc::tma_load_4d;
+using tc::tma_load_5d;
 
 constexpr int TILE_ROWS = 128;                    // output indices per tile (MMA M)
 constexpr int EPI_WARPS = 16;
@@ -63,18 +66,6 @@ constexpr int ALU_MAX_ROWS = 8;
 constexpr int RADON_THREADS = 32 * (ALU_WARP + ALU_WARPS);
 constexpr int MAX_ACC = 4;                        // accumulators in flight: what the R columns leave of 512, at most 4
 constexpr int RADON_EXCHANGE_CTAS = 148;          // CTAs of a one-launch two-stage tabulation (one exchange slab each)
-constexpr int ROW_INVALID = -1;
-constexpr int ROW_VERT = 1 << 30;                 // flag: row of the extra ("vertical") class
-
-// One index space of the transform: idx = lo + q*hi, hi in [0, q]; hi == q is the extra class (a = ∞ on the
-// type side).  Rows are counted inside one head.
-struct RadonSide {
-  int32_t count;                   // q*q, or q*q + q with the extra class
-  int32_t s_lo, s_hi, s_img;       // regular rows: img*s_img + lo*s_lo + hi*s_hi
-  int32_t v0, sv_lo, sv_img;       // extra class : v0 + img*sv_img + lo*sv_lo
-  int32_t vert_from;               // images >= vert_from carry the extra class
-  int64_t rows_per_head;
-};
 
 // One stage: input and output index spaces, and where the rows live.  A "private" table is the exchange buffer of the
 // two-stage kernel: [CTA][rows_per_head][128 entries], one slab per CTA, rewritten for every slab so that it stays in L2.
@@ -146,12 +137,6 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, c
   return __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
 }
 
-__device__ __forceinline__ int side_row(const RadonSide& s, int idx, int q) {
-  if (idx >= s.count) return ROW_INVALID;
-  const int lo = idx % q, hi = idx / q;
-  return hi < q ? lo * s.s_lo + hi * s.s_hi : (ROW_VERT | lo * s.sv_lo);
-}
-
 // Row of the streamed operand that holds input index (lo, line): slot line / sps, then the line's q rows.
 __device__ __forceinline__ int operand_row(const RadonParams& p, int line, int lo) {
   if (line >= p.q) return p.nreg * p.sr + lo;                 // extra class: a slot of its own
@@ -198,21 +183,6 @@ __device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* m
   asm volatile(
       "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4, %5}], [%6], %7;"
       ::"r"(smem_u32(smem_dst)), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(bar)), "l"(pol)
-      : "memory");
-}
-
-__device__ __forceinline__ void tma_load_5d(void* smem_dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
-                                            int c4, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
-      ::"r"(smem_u32(smem_dst)), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(smem_u32(bar))
-      : "memory");
-}
-__device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
-                                            uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
-      ::"r"(smem_u32(smem_dst)), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(bar))
       : "memory");
 }
 
@@ -815,65 +785,6 @@ bool radon_layout_ok(int q, const RadonShape& sh, int ring, int mini_bytes, int 
   return ok;
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn radon_encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult qr;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qr) == cudaSuccess &&
-        qr == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
-  return fn;
-}
-
-// bf16 rows of rp entries.  Dimensions (fastest first): entry, then `rank - 1` row indices with the given sizes and
-// strides in rows; box = 64 entries x box[] rows; 128-byte swizzle; out-of-bounds reads give zeros.
-bool radon_map(CUtensorMap* map, const void* base, int64_t rp, int rank, const int64_t* sizes, const int64_t* row_strides,
-               const int* box) {
-  EncodeTiledFn fn = radon_encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[5], strides[4];
-  cuuint32_t bx[5], estr[5];
-  dims[0] = (cuuint64_t)rp; bx[0] = 64; estr[0] = 1;
-  for (int i = 1; i < rank; ++i) {
-    dims[i] = (cuuint64_t)sizes[i - 1];
-    strides[i - 1] = (cuuint64_t)row_strides[i - 1] * (cuuint64_t)rp * 2;
-    bx[i] = (cuuint32_t)box[i - 1];
-    estr[i] = 1;
-  }
-  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, bx, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-RadonSide side(int count, int s_lo, int s_hi, int s_img, int64_t rows_per_head, int v0 = 0, int sv_lo = 0,
-               int sv_img = 0, int vert_from = 1 << 29) {
-  RadonSide s;
-  s.count = count; s.s_lo = s_lo; s.s_hi = s_hi; s.s_img = s_img; s.v0 = v0; s.sv_lo = sv_lo; s.sv_img = sv_img;
-  s.vert_from = vert_from; s.rows_per_head = rows_per_head;
-  return s;
-}
-
-// One stage as the host states it; src / dst are whole tables [bh][rows_per_head][rp], or the private exchange buffer.
-struct StageSpec {
-  RadonSide in, out;
-  int images;
-  const void* src;
-  void* dst;
-  bool src_private, dst_private;
-};
-
-StageSpec stage(const RadonSide& in, const RadonSide& out, int images, const void* src, void* dst, bool src_private = false,
-                bool dst_private = false) {
-  StageSpec s;
-  s.in = in; s.out = out; s.images = images; s.src = src; s.dst = dst; s.src_private = src_private; s.dst_private = dst_private;
-  return s;
-}
-
 // nph = 1: one stage over the whole tables.  nph = 2: both stages in one launch, which must share R (the same
 // direction, the same index counts) and exchange their rows through the private buffer.
 cudaError_t launch_radon(int q, int transpose, int nph, const StageSpec* sp, int64_t rp, int bh, int* status,
@@ -1038,6 +949,13 @@ int64_t smat_tabulate_tc_scratch_elems(const SmatGeo& geo, int64_t state_elems, 
   return (int64_t)bh * rows * state_elems;
 }
 
+// Which of the two kernels runs a stage.  The one that generates R loads an image once where the resident one has two or
+// three CTAs load it, but shares its issue slots and tensor memory with the generators.  Measured (ms, resident against
+// generated): q = 13, d = 3, 32 heads 0.083 / 0.073, transposed 0.092 / 0.072; q = 13, d = 4, 8 heads 0.462 / 0.425,
+// transposed (4 heads) 0.289 / 0.274; q = 17, d = 3, 64 heads 0.263 / 0.299, transposed 0.331 / 0.293; q = 17, d = 4,
+// 8 heads 1.14 / 1.26.  At q <= 11 one CTA covers an image either way.
+static bool generates_matrix(int q, int D, int transpose) { return q == 13 || (q == 17 && D == 2 && transpose); }
+
 // transpose = 0: in = F [bh][P][rp] bf16, out = U [bh][B][rp] bf16.  transpose = 1: in = Ū [bh][B][rp], out = F̄ [bh][P][rp].
 // scratch: smat_tabulate_tc_scratch_elems bf16 (d = 4 only).  One launch for d = 3; one or two for d = 4.
 cudaError_t smat_launch_tabulate_tc(const void* in, void* out, void* scratch, const SmatGeo& geo, int64_t state_elems,
@@ -1049,6 +967,7 @@ cudaError_t smat_launch_tabulate_tc(const void* in, void* out, void* scratch, co
     const RadonSide typ = side(qq + q, 1, q, 0, geo.B, qq, 1, 0, 0);
     const StageSpec sp = transpose ? stage(typ, pts, 1, in, out) : stage(pts, typ, 1, in, out);
     *launches = 1;
+    if (generates_matrix(q, 2, transpose)) return launch_radon_wide(q, transpose, sp, state_elems, bh, status, st);
     return launch_radon(q, transpose, 1, &sp, state_elems, bh, status, st);
   }
   if (geo.D != 3) return cudaErrorInvalidValue;
@@ -1071,7 +990,22 @@ cudaError_t smat_launch_tabulate_tc(const void* in, void* out, void* scratch, co
     return launch_radon(q, transpose, 2, sp, state_elems, bh, status, st);
   }
   *launches = 2;
-  cudaError_t err = launch_radon(q, transpose, 1, &sp[0], state_elems, bh, status, st);
-  if (err != cudaSuccess) return err;
-  return launch_radon(q, transpose, 1, &sp[1], state_elems, bh, status, st);
+  for (int i = 0; i < 2; ++i) {
+    const cudaError_t err = generates_matrix(q, 3, transpose)
+                                ? launch_radon_wide(q, transpose, sp[i], state_elems, bh, status, st)
+                                : launch_radon(q, transpose, 1, &sp[i], state_elems, bh, status, st);
+    if (err != cudaSuccess) return err;
+  }
+  return cudaSuccess;
+}
+
+int smat_tabulate_d3_wide_supported(const SmatGeo& geo, int64_t state_elems) {
+  return geo.D == 2 && geo.q >= 19 && state_elems % 128 == 0 && radon_wide_fits(geo.q) ? 1 : 0;
+}
+
+cudaError_t smat_launch_tabulate_d3_wide(const void* in, void* out, const SmatGeo& geo, int64_t state_elems, int bh,
+                                         int* status, cudaStream_t st) {
+  const int q = geo.q, qq = q * q;
+  const StageSpec sp = stage(side(qq, 1, q, 0, geo.P), side(qq + q, 1, q, 0, geo.B, qq, 1, 0, 0), 1, in, out);
+  return launch_radon_wide(q, 0, sp, state_elems, bh, status, st);
 }

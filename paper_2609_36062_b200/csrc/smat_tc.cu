@@ -810,9 +810,9 @@ struct SegOutParams {
 // 64 K tokens, where this order takes 0.205; its 1.07 GB need 0.161 at the HBM rate.)
 // SPLIT: for blocks that are not whole tiles, whose plans keep fp32 tables: the state and the score tile enter their
 // products as a leading bf16 part plus a bf16 remainder (16 bits of the fp32 value), the long-range rows arrive in
-// fp32, and the rows past a block's end load as zeros and are not stored.  (32 heads of 5056 tokens, d = 3: 0.071 ms,
-// where chunk states, scan, scores, state read and output on the fp32 ALUs took 1.23 ms; 0.12 of it is now the two
-// kernels before this one and itself.)
+// fp32, and the rows past a block's end load as zeros and are not stored.  (32 heads of 5056 tokens, d = 3: 0.071 ms, and
+// 0.028 for the segment totals and their scan, where chunk states, scan, scores, state read and output on the fp32 ALUs
+// took 1.23 ms.)
 constexpr int SEG_EPI_WARPS = 16;
 constexpr int SEG_OUT_THREADS = 32 * (SEG_EPI_WARPS + 2);
 
@@ -1348,8 +1348,6 @@ struct PoolParams {
   const __nv_bfloat16* K;  // rows giving the first state index
   const __nv_bfloat16* V;  // rows giving the second state index
   void* F;                 // [bh][groups][128][128] fp32 or bf16
-  int slab_major;          // bf16 only: store as [bh][512 slabs of 32 entries][groups][32] instead (a slab of entries of
-                           // every state contiguous, the order the register-resident d = 3 tabulation reads)
   int* status;
 };
 
@@ -1460,10 +1458,6 @@ __global__ void __launch_bounds__(160) pool_tc_kernel(const PoolParams prm) {
           }
           if (OUT_BF16) {
             __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(prm.F) + (item * TILE + i) * TILE + cb * 32;
-            if (prm.slab_major) {   // entries 32 (4 i + cb) .. + 31 of this state are slab 4 i + cb of its head
-              const int64_t head = item / prm.groups, g = item - head * prm.groups;
-              dst = static_cast<__nv_bfloat16*>(prm.F) + ((head * (TILE * TILE / 32) + (4 * i + cb)) * prm.groups + g) * 32;
-            }
 #pragma unroll
             for (int h8 = 0; h8 < 2; ++h8) {  // whole 32-byte sectors
               uint32_t w[8];
@@ -1764,11 +1758,8 @@ static cudaError_t launch_pool_tc(const PoolParams& prm, cudaStream_t st) {
 }
 
 cudaError_t smat_launch_pool_tc(const void* K, const void* V, void* F, int out_bf16, const SmatGroupSpec& grp,
-                                int64_t groups, int64_t max_tokens, int64_t T, int bh, int* status, cudaStream_t st,
-                                int slab_major) {
+                                int64_t groups, int64_t max_tokens, int64_t T, int bh, int* status, cudaStream_t st) {
   PoolParams prm;
-  if (slab_major && !out_bf16) return cudaErrorInvalidValue;
-  prm.slab_major = slab_major;
   prm.T = T; prm.grp = grp; prm.groups = groups; prm.items = (int64_t)bh * groups;
   prm.K = static_cast<const __nv_bfloat16*>(K);
   prm.V = static_cast<const __nv_bfloat16*>(V);

@@ -153,6 +153,7 @@ PyObject* plan_forward(PyObject* self, PyObject* const* a, Py_ssize_t n) {
     at::Tensor O;
     void *ws, *st;
     size_t bytes;
+    if (kind == 0 && a[5] != Py_None && !tensor(a[5], "O", p.dtype, sv)) return nullptr;
     if (!output(a[5], "O", *V, &O) || !workspace(a[6], "workspace", &ws, &bytes) || !stream(a[7], &st)) return nullptr;
     int rc;
     const char* what;

@@ -112,7 +112,7 @@ def stage_work(name: str, T, c, r, p, e, geo, u_bytes=4, f_bytes=4) -> Work:
         "pool_tc":     Work(2 * n * rp, 0, n * (r + p) * e + P * sf),
         "tabulate":    Work(0, geo.nnzC * rp, P * st + B * su),
         "tabulate_tc": Work(0, geo.nnzC * rp, P * sf + B * su),
-        "tabulate_regs": Work(0, geo.nnzC * rp, P * sf + B * su),      # the same sums on the fp32 ALUs (bf16 tables)
+        "tabulate_wide": Work(0, geo.nnzC * rp, P * sf + B * su),      # the same on the tensor cores, larger primes
         "tabulate_bf16": Work(0, geo.nnzC * rp, P * sf + B * su),
         "bwd_tabulate_t_tc": Work(0, geo.nnzC * rp, B * su + P * sf),
         "bwd_pool_type_tc": Work(2 * m * rp, 0, m * (r + p) * e + B * su),
@@ -145,4 +145,4 @@ def stage_work(name: str, T, c, r, p, e, geo, u_bytes=4, f_bytes=4) -> Work:
 
 
 # Stages whose additions run on the fp32 ALUs (the other tabulations form the same sums on the tensor cores).
-ALU_STAGES = ("tabulate", "tabulate_regs", "tabulate_bf16", "bwd_tabulate_t")
+ALU_STAGES = ("tabulate", "tabulate_bf16", "bwd_tabulate_t")
