@@ -27,14 +27,19 @@ __device__ __forceinline__ void store_out<float>(float* p, float v) { *p = v; }
 template <>
 __device__ __forceinline__ void store_out<__nv_bfloat16>(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
 
-// four consecutive entries of a type state
+// Four consecutive entries of a state, past the L1 cache: nothing of it is read twice in a step.
 template <typename TU>
-__device__ __forceinline__ float4 load_u4(const TU* p);
+__device__ __forceinline__ float4 load_state4(const TU* p);
 template <>
-__device__ __forceinline__ float4 load_u4<float>(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 load_state4<float>(const float* p) {
+  float4 v;
+  asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
 template <>
-__device__ __forceinline__ float4 load_u4<__nv_bfloat16>(const __nv_bfloat16* p) {
-  const uint2 w = *reinterpret_cast<const uint2*>(p);
+__device__ __forceinline__ float4 load_state4<__nv_bfloat16>(const __nv_bfloat16* p) {
+  uint2 w;
+  asm volatile("ld.global.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(w.x), "=r"(w.y) : "l"(p));
   return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
                      __uint_as_float(w.y & 0xffff0000u));
 }
@@ -43,30 +48,34 @@ __device__ __forceinline__ float4 load_u4<__nv_bfloat16>(const __nv_bfloat16* p)
 // the SMs.  Thread (row tid / 8, columns 4 (tid % 8)) walks the rows 32 at a time with every load of its share in
 // flight before the first use: a CTA's 24 KB are one round trip to memory.  The partial outputs meet by shuffles and
 // one row of shared memory per warp (no atomics: the sum's order is fixed).  Bound by the 84 MB a step of 512 heads
-// moves: 15.7 us (12.7 at the HBM rate), where one CTA per head with one row pass in flight at a time took 22.1.
+// moves: 14.6 us (12.8 at the HBM rate; 15.7 without the prefetch), where one CTA per head with one row pass in flight at
+// a time took 22.1.
 constexpr int DEC_COLS = 32, DEC_ROWS = 32, DEC_THREADS = 256;
 
 template <typename T, typename TU, int PASSES>
-__global__ void __launch_bounds__(DEC_THREADS) decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k,
-                                                          const T* __restrict__ v, T* __restrict__ o,
-                                                          float* __restrict__ S, const TU* __restrict__ U, int64_t type,
-                                                          int64_t types, int p, const float* __restrict__ log_a,
-                                                          float* __restrict__ log_g) {
+__global__ void __launch_bounds__(DEC_THREADS) decode_step_kernel(const T* q, const T* k,
+                                                          const T* v, T* o,
+                                                          float* S, const TU* U, int64_t type,
+                                                          int64_t types, int p, const float* log_a,
+                                                          float* log_g) {
   constexpr int r = PASSES * DEC_ROWS;
   __shared__ float part[DEC_THREADS / 32][DEC_COLS];
   pdl_trigger();
   const int bh = blockIdx.y, tid = threadIdx.x, j0 = blockIdx.x * DEC_COLS;
   const int j = j0 + (tid & 7) * 4, i0 = tid >> 3;
+  const TU* Ub = U + ((int64_t)bh * types + type) * r * p;
+  // the type state is on its way to L2 while the step before finishes (a hint: it reads nothing)
+  if (tid < r) asm volatile("prefetch.global.L2 [%0];" ::"l"(Ub + (int64_t)tid * p + j0));
   pdl_wait();
   float* Sh = S + (int64_t)bh * r * p + j;
-  const TU* Uh = U + ((int64_t)bh * types + type) * r * p + j;
+  const TU* Uh = Ub + j;
   float4 s[PASSES], u[PASSES];
   float qi[PASSES], ki[PASSES];
 #pragma unroll
   for (int n = 0; n < PASSES; ++n) {
     const int64_t off = (int64_t)(n * DEC_ROWS + i0) * p;
-    s[n] = *reinterpret_cast<const float4*>(Sh + off);
-    u[n] = load_u4<TU>(Uh + off);
+    s[n] = load_state4<float>(Sh + off);
+    u[n] = load_state4<TU>(Uh + off);
   }
 #pragma unroll
   for (int n = 0; n < PASSES; ++n) {
