@@ -6,14 +6,17 @@
 #include <cuda_runtime.h>
 
 #include "smat_internal.h"
+#include "smat_launch.cuh"
 
 namespace {
 
 // Inclusive prefix (reverse = 0) or suffix (reverse = 1) sum of one row of `len` floats per head; one CTA per head.
-__global__ void __launch_bounds__(1024) head_scan_kernel(const float* __restrict__ in, float* __restrict__ out, int64_t len,
+__global__ void __launch_bounds__(1024) head_scan_kernel(const float* in, float* out, int64_t len,
                                                          int reverse) {
   __shared__ float warp_sum[32];
   __shared__ float carry;
+  pdl_trigger();
+  pdl_wait();
   const int tid = threadIdx.x;
   const float* src = in + (int64_t)blockIdx.x * len;
   float* dst = out + (int64_t)blockIdx.x * len;
@@ -46,9 +49,11 @@ __global__ void __launch_bounds__(1024) head_scan_kernel(const float* __restrict
 //   mode 2 (the block boundary)      : t <  n: src = A, f = exp(λ_{n-1} - λ_t)   (key side, folded into Z_j)
 //                                      t >= n: src = B, f = exp(λ_t - λ_{n-1})   (query side, on the read)
 template <typename T>
-__global__ void gate_scale_kernel(const T* __restrict__ A, const T* __restrict__ B, T* __restrict__ out,
-                                  const float* __restrict__ lam, int mode, int64_t n, int64_t c, int64_t Tlen, int dim,
+__global__ void gate_scale_kernel(const T* A, const T* B, T* out,
+                                  const float* lam, int mode, int64_t n, int64_t c, int64_t Tlen, int dim,
                                   int64_t rows) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   if (row >= rows) return;
   const int lane = threadIdx.x & 31;
@@ -87,9 +92,11 @@ __global__ void gate_scale_kernel(const T* __restrict__ A, const T* __restrict__
 //   out[b] = running;  running = γ_b running + in[b],   γ_b = exp(λ_{e(b)} - λ_{s(b)-1}) = the product of chunk b's gates.
 // Forward this is S_in (Lemma "Gated SMat": the carried state is decayed by every chunk it passes); in reverse it is the
 // adjoint recursion of the same scan.
-__global__ void __launch_bounds__(256) gated_scan_kernel(float* S, const float* __restrict__ lam, int64_t state_elems,
+__global__ void __launch_bounds__(256) gated_scan_kernel(float* S, const float* lam, int64_t state_elems,
                                                          int64_t NC, int64_t c, int64_t lo0, int64_t hi0, int64_t lo1,
                                                          int64_t hi1, int reverse) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t e4 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e4 * 4 >= state_elems) return;
   const int64_t bh = blockIdx.y;
@@ -109,8 +116,10 @@ __global__ void __launch_bounds__(256) gated_scan_kernel(float* S, const float* 
 
 // dλ_t = q_t·dQ_t - k_t·dK_t (every edge's contribution enters once as a query and once as a key); one warp per token.
 template <typename T>
-__global__ void gate_dlam_kernel(const T* __restrict__ Q, const T* __restrict__ dQ, const T* __restrict__ K,
-                                 const T* __restrict__ dK, float* __restrict__ dlam, int dim, int64_t rows) {
+__global__ void gate_dlam_kernel(const T* Q, const T* dQ, const T* K,
+                                 const T* dK, float* dlam, int dim, int64_t rows) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   if (row >= rows) return;
   const int lane = threadIdx.x & 31;
@@ -125,8 +134,7 @@ __global__ void gate_dlam_kernel(const T* __restrict__ Q, const T* __restrict__ 
 }  // namespace
 
 cudaError_t smat_launch_head_scan(const float* in, float* out, int64_t len, int bh, int reverse, cudaStream_t st) {
-  head_scan_kernel<<<(unsigned)bh, 1024, 0, st>>>(in, out, len, reverse);
-  return cudaGetLastError();
+  return smat_launch_pdl(head_scan_kernel, dim3((unsigned)bh), 1024, 0, st, in, out, len, reverse);
 }
 
 cudaError_t smat_launch_gate_scale(const void* A, const void* B, void* out, const float* lam, int mode, int bf16,
@@ -134,21 +142,17 @@ cudaError_t smat_launch_gate_scale(const void* A, const void* B, void* out, cons
   const int64_t rows = (int64_t)bh * T;
   const unsigned blocks = (unsigned)((rows * 32 + 255) / 256);
   if (bf16)
-    gate_scale_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(A),
-                                                             static_cast<const __nv_bfloat16*>(B),
-                                                             static_cast<__nv_bfloat16*>(out), lam, mode, n, c, T, dim, rows);
-  else
-    gate_scale_kernel<float><<<blocks, 256, 0, st>>>(static_cast<const float*>(A), static_cast<const float*>(B),
-                                                     static_cast<float*>(out), lam, mode, n, c, T, dim, rows);
-  return cudaGetLastError();
+    return smat_launch_pdl(gate_scale_kernel<__nv_bfloat16>, dim3(blocks), 256, 0, st, static_cast<const __nv_bfloat16*>(A),
+                           static_cast<const __nv_bfloat16*>(B), static_cast<__nv_bfloat16*>(out), lam, mode, n, c, T, dim, rows);
+  return smat_launch_pdl(gate_scale_kernel<float>, dim3(blocks), 256, 0, st, static_cast<const float*>(A),
+                         static_cast<const float*>(B), static_cast<float*>(out), lam, mode, n, c, T, dim, rows);
 }
 
 cudaError_t smat_launch_gated_scan(float* S, const float* lam, int64_t state_elems, int64_t NC, int64_t c, int bh,
                                    int64_t lo0, int64_t hi0, int64_t lo1, int64_t hi1, int reverse, cudaStream_t st) {
   const int ranges = (hi1 > lo1) ? 2 : 1;
   dim3 grid((unsigned)((state_elems / 4 + 255) / 256), (unsigned)bh, (unsigned)ranges);
-  gated_scan_kernel<<<grid, 256, 0, st>>>(S, lam, state_elems, NC, c, lo0, hi0, lo1, hi1, reverse);
-  return cudaGetLastError();
+  return smat_launch_pdl(gated_scan_kernel, grid, 256, 0, st, S, lam, state_elems, NC, c, lo0, hi0, lo1, hi1, reverse);
 }
 
 cudaError_t smat_launch_gate_dlam(const void* Q, const void* dQ, const void* K, const void* dK, float* dlam, int bf16,
@@ -156,15 +160,12 @@ cudaError_t smat_launch_gate_dlam(const void* Q, const void* dQ, const void* K, 
   const int64_t rows = (int64_t)bh * T;
   const unsigned blocks = (unsigned)((rows * 32 + 255) / 256);
   if (bf16)
-    gate_dlam_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(Q),
-                                                            static_cast<const __nv_bfloat16*>(dQ),
-                                                            static_cast<const __nv_bfloat16*>(K),
-                                                            static_cast<const __nv_bfloat16*>(dK), dlam, dim, rows);
-  else
-    gate_dlam_kernel<float><<<blocks, 256, 0, st>>>(static_cast<const float*>(Q), static_cast<const float*>(dQ),
-                                                    static_cast<const float*>(K), static_cast<const float*>(dK), dlam, dim,
-                                                    rows);
-  return cudaGetLastError();
+    return smat_launch_pdl(gate_dlam_kernel<__nv_bfloat16>, dim3(blocks), 256, 0, st, static_cast<const __nv_bfloat16*>(Q),
+                           static_cast<const __nv_bfloat16*>(dQ), static_cast<const __nv_bfloat16*>(K),
+                           static_cast<const __nv_bfloat16*>(dK), dlam, dim, rows);
+  return smat_launch_pdl(gate_dlam_kernel<float>, dim3(blocks), 256, 0, st, static_cast<const float*>(Q),
+                         static_cast<const float*>(dQ), static_cast<const float*>(K), static_cast<const float*>(dK), dlam, dim,
+                         rows);
 }
 
 // ---- normalised output (Sec. 2: augmented value v̄ = [v; 1], one final division) ------------------------------------
@@ -189,7 +190,9 @@ struct Quad {
 
 // V̄ = V with its last column set to one.
 template <typename T>
-__global__ void augment_value_kernel(const T* __restrict__ V, T* __restrict__ Vbar, int p, int64_t rows) {
+__global__ void augment_value_kernel(const T* V, T* Vbar, int p, int64_t rows) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   if (row >= rows) return;
   const int lane = threadIdx.x & 31;
@@ -207,7 +210,9 @@ __global__ void augment_value_kernel(const T* __restrict__ V, T* __restrict__ Vb
 
 // O = ȳ_{1:p-1} / ȳ_p, and the normaliser ȳ_p itself in the last column.  One warp per row.
 template <typename T>
-__global__ void normalize_rows_kernel(const T* __restrict__ Y, T* __restrict__ O, int p, int64_t rows) {
+__global__ void normalize_rows_kernel(const T* Y, T* O, int p, int64_t rows) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   if (row >= rows) return;
   const int lane = threadIdx.x & 31;
@@ -229,8 +234,10 @@ __global__ void normalize_rows_kernel(const T* __restrict__ Y, T* __restrict__ O
 // Upstream of the linear pass from the upstream of the normalised output (the backward of the final division):
 //   dȳ_c = dO_c / z (c < p-1),   dȳ_p = dO_p - Σ_{c<p-1} dO_c O_c / z,   z = the normaliser kept in O's last column.
 template <typename T>
-__global__ void normalize_adjoint_kernel(const T* __restrict__ O, const T* __restrict__ dO, T* __restrict__ dY, int p,
+__global__ void normalize_adjoint_kernel(const T* O, const T* dO, T* dY, int p,
                                          int64_t rows) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   if (row >= rows) return;
   const int lane = threadIdx.x & 31;
@@ -271,7 +278,9 @@ __global__ void normalize_adjoint_kernel(const T* __restrict__ O, const T* __res
 
 // The ones column of V̄ is a constant: its gradient is dropped.
 template <typename T>
-__global__ void clear_last_column_kernel(T* __restrict__ dV, int p, int64_t rows) {
+__global__ void clear_last_column_kernel(T* dV, int p, int64_t rows) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (row < rows) dV[row * p + p - 1] = (T)0.0f;
 }
@@ -280,15 +289,16 @@ template <typename T>
 cudaError_t normalize_step(int step, const void* a, const void* b, void* out, int p, int64_t rows, cudaStream_t st) {
   const unsigned warp_blocks = (unsigned)((rows * 32 + 255) / 256);
   if (step == 0)
-    augment_value_kernel<T><<<warp_blocks, 256, 0, st>>>(static_cast<const T*>(a), static_cast<T*>(out), p, rows);
-  else if (step == 1)
-    normalize_rows_kernel<T><<<warp_blocks, 256, 0, st>>>(static_cast<const T*>(a), static_cast<T*>(out), p, rows);
-  else if (step == 2)
-    normalize_adjoint_kernel<T><<<warp_blocks, 256, 0, st>>>(static_cast<const T*>(a), static_cast<const T*>(b),
-                                                             static_cast<T*>(out), p, rows);
-  else
-    clear_last_column_kernel<T><<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(static_cast<T*>(out), p, rows);
-  return cudaGetLastError();
+    return smat_launch_pdl(augment_value_kernel<T>, dim3(warp_blocks), 256, 0, st, static_cast<const T*>(a),
+                           static_cast<T*>(out), p, rows);
+  if (step == 1)
+    return smat_launch_pdl(normalize_rows_kernel<T>, dim3(warp_blocks), 256, 0, st, static_cast<const T*>(a),
+                           static_cast<T*>(out), p, rows);
+  if (step == 2)
+    return smat_launch_pdl(normalize_adjoint_kernel<T>, dim3(warp_blocks), 256, 0, st, static_cast<const T*>(a),
+                           static_cast<const T*>(b), static_cast<T*>(out), p, rows);
+  return smat_launch_pdl(clear_last_column_kernel<T>, dim3((unsigned)((rows + 255) / 256)), 256, 0, st, static_cast<T*>(out),
+                         p, rows);
 }
 
 }  // namespace

@@ -37,8 +37,8 @@
 // q = 11 also sends its output tiles off by TMA: the epilogue writes the rounded tile into the item's own ring slot
 // (as large as a tile, and dead once the MMAs have read it) in the box layout, and lane 0 of warp 18 issues the tile
 // stores and frees the slot; the bulk of the stores bypasses the LSU.
-// The kernel exists twice: radon_tc_kernel<false> for one stage per launch with every index through the MMAs (q = 17
-// and the small primes), without cache hints, phase tables or ALU warps; radon_tc_kernel<true> with them.
+// The kernel exists twice: radon_tc_kernel<false, .> for one stage per launch with every index through the MMAs (q = 17
+// and the small primes), without cache hints, phase tables or ALU warps; radon_tc_kernel<true, .> with them.
 // (The tile-store path is written for several slots per item and several parts and is compiled into both, but the
 // launcher switches it on for q = 11 only: it was measured slower than the direct stores for q = 13 and 17.)
 #include <cuda.h>
@@ -46,6 +46,7 @@
 #include <cuda_runtime.h>
 
 #include "smat_internal.h"
+#include "smat_launch.cuh"
 #include "smat_radon.cuh"
 #include "smat_tc.cuh"
 
@@ -266,7 +267,10 @@ __device__ __forceinline__ void issue_slot_steps(int steps, uint32_t tmem_d, uin
 
 // FEAT = false is the plain instantiation (one stage per launch, every index through the MMAs, direct stores, no cache
 // hints): the single-thread roles pay for every instruction, and the prime-specific paths would cost the others time.
-template <bool FEAT>
+// EARLY: launched to overlap with the kernel before it (see smat_launch.cuh).  q = 17 does without: its launches take
+// hundreds of microseconds, and with the waits compiled in they ran 1 % slower (16 heads of 64 K tokens, d = 4: the pass
+// 4166 us against 4126).
+template <bool FEAT, bool EARLY>
 __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid_constant__ CUtensorMap tm_reg0,
                                                                     const __grid_constant__ CUtensorMap tm_vert0,
                                                                     const __grid_constant__ CUtensorMap tm_reg1,
@@ -353,6 +357,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
+  if (EARLY) pdl_trigger();
   const uint32_t tmem_acc = tmem_base + r_cols;
 
   // per phase: streaming tables, or the exchange rows (two-stage kernel only)
@@ -368,6 +373,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
   // goes back to the producer when the stores have read it.  Lane 0 of the second MMA warp when every item is one
   // slot (that warp has no items then), else lane 0 of warp 19.
   auto store_role = [&]() {
+    if (EARLY) pdl_wait();
     const uint32_t ring = (uint32_t)prm.ring;
     uint32_t slot = 0, prev_slot = 0;
     uint32_t sidx = 0, spar = 0;                                // the item's "staged" barrier (items mod ring) and its parity
@@ -424,6 +430,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
 
   if (warp == PROD_WARP && lane == 0) {
     // ---- TMA producer -----------------------------------------------------------------------------------------
+    if (EARLY) pdl_wait();
     // The two single-thread roles keep running slot / parity counters: a lone thread pays the full latency of every
     // instruction, so divisions by the ring size inside the loop would show in the kernel time.
     uint32_t slot = 0, par = 0;                               // ring position; parity of the empty barrier's phase to wait for
@@ -546,6 +553,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
     // instead of a second, nearly empty tile paying for every MMA again.  A task is one leftover index and 8 state
     // entries (one 16-byte chunk of the swizzled slot); 16 neighbouring tasks store 256 contiguous bytes.
     if (alu_here) {
+      if (EARLY) pdl_wait();
       const int tid_a = (warp - ALU_WARP) * 32 + lane, tasks = prm.alu_rows * 16;
       const uint32_t ring = (uint32_t)prm.ring;
       uint32_t slot = 0, par = 0;
@@ -604,6 +612,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
     }
   } else if (warp < EPI_WARPS) {
     // ---- epilogue ---------------------------------------------------------------------------------------------
+    if (EARLY) pdl_wait();
     // Warp w reads lane quarter w % 4 (32 output indices) and the 32-entry column chunk w / 4 of every item.
     const int qd = warp & 3, cb = warp >> 2;
     const int orow = qd * 32 + lane;                            // output index of this CTA = TMEM lane
@@ -879,12 +888,17 @@ cudaError_t launch_radon(int q, int transpose, int nph, const StageSpec* sp, int
     prm.ph[1] = prm.ph[0]; tm_reg[1] = tm_reg[0]; tm_vert[1] = tm_vert[0]; tm_oreg[1] = tm_oreg[0]; tm_overt[1] = tm_overt[0];
   }
   const bool feat = nph > 1 || prm.alu_rows > 0;
-  auto kernel = feat ? radon_tc_kernel<true> : radon_tc_kernel<false>;
+  // the plain instantiation has no use for the two ALU warps
+  const unsigned threads = feat ? RADON_THREADS : 32 * (ALU_WARP + (prm.tma_out ? 1 : 0));
+  const bool early = feat || q < 17;
+  auto kernel = feat ? radon_tc_kernel<true, true> : (early ? radon_tc_kernel<false, true> : radon_tc_kernel<false, false>);
   cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
-  // the plain instantiation has no use for the two ALU warps
-  kernel<<<(unsigned)ctas, feat ? RADON_THREADS : 32 * (ALU_WARP + (prm.tma_out ? 1 : 0)), smem, st>>>(tm_reg[0], tm_vert[0], tm_reg[1], tm_vert[1],
-                                                                            tm_oreg[0], tm_overt[0], tm_oreg[1], tm_overt[1], prm);
+  if (early)
+    return smat_launch_pdl(kernel, dim3((unsigned)ctas), threads, smem, st, tm_reg[0], tm_vert[0], tm_reg[1], tm_vert[1],
+                           tm_oreg[0], tm_overt[0], tm_oreg[1], tm_overt[1], prm);
+  kernel<<<(unsigned)ctas, threads, smem, st>>>(tm_reg[0], tm_vert[0], tm_reg[1], tm_vert[1], tm_oreg[0], tm_overt[0],
+                                                tm_oreg[1], tm_overt[1], prm);
   return cudaGetLastError();
 }
 

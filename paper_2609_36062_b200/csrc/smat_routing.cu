@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "smat_internal.h"
+#include "smat_launch.cuh"
 
 namespace {
 
@@ -29,7 +30,9 @@ struct RouteParams {
   int warps;               // W: rows of per-warp counters in shared memory
 };
 
-__global__ void __launch_bounds__(ROUTE_THREADS) routing_lists_kernel(const RouteParams prm) {
+__global__ void __launch_bounds__(ROUTE_THREADS) routing_lists_kernel(const __grid_constant__ RouteParams prm) {
+  pdl_trigger();
+  pdl_wait();
   extern __shared__ int32_t rows[];     // [1 + W][G + 1]: row 0 totals / offsets, row 1 + w the counters of warp w
   const int kind = blockIdx.y;
   const int64_t bh = blockIdx.x, n = prm.count[kind], G = prm.G[kind], pitch = G + 1;
@@ -114,8 +117,10 @@ __global__ void __launch_bounds__(ROUTE_THREADS) routing_lists_kernel(const Rout
 
 // Rows of tokens that belong to no group are never written by a routed read; whoever adds those rows afterwards must
 // find zeros there.  One thread per token reads its key; the (rare) token whose key is out of range zeroes its row.
-__global__ void zero_unrouted_rows_kernel(const int32_t* __restrict__ key, int64_t count, int64_t G, int64_t first,
-                                          uint8_t* __restrict__ rows, int64_t T, int row_bytes, int64_t total) {
+__global__ void zero_unrouted_rows_kernel(const int32_t* key, int64_t count, int64_t G, int64_t first,
+                                          uint8_t* rows, int64_t T, int row_bytes, int64_t total) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= total) return;
   const int32_t k = key[w];
@@ -130,9 +135,8 @@ __global__ void zero_unrouted_rows_kernel(const int32_t* __restrict__ key, int64
 cudaError_t smat_launch_zero_unrouted(const int32_t* key, int64_t count, int64_t G, int64_t first, void* rows, int64_t T,
                                       int row_bytes, int bh, cudaStream_t st) {
   const int64_t total = (int64_t)bh * count;
-  zero_unrouted_rows_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(key, count, G, first,
-                                                                               static_cast<uint8_t*>(rows), T, row_bytes, total);
-  return cudaGetLastError();
+  return smat_launch_pdl(zero_unrouted_rows_kernel, dim3((unsigned)((total + 255) / 256)), 256, 0, st, key, count, G, first,
+                         static_cast<uint8_t*>(rows), T, row_bytes, total);
 }
 
 // Largest group count the list builder handles (its cursors live in shared memory).
@@ -154,6 +158,5 @@ cudaError_t smat_launch_routing_lists(const int32_t* prof, const int32_t* type, 
   cudaError_t err = cudaFuncSetAttribute(routing_lists_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   dim3 grid((unsigned)bh, 2);
-  routing_lists_kernel<<<grid, ROUTE_THREADS, smem, st>>>(prm);
-  return cudaGetLastError();
+  return smat_launch_pdl(routing_lists_kernel, grid, ROUTE_THREADS, smem, st, prm);
 }

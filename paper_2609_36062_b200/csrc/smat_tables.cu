@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 
 #include "smat_internal.h"
+#include "smat_launch.cuh"
 
 namespace {
 
@@ -46,10 +47,12 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // of E consecutive entries, keeps F[:, slab] in shared memory and writes U[:, slab].
 // Layout in shared memory: point index major, E floats per point; a thread owns one float4 of an item.
 template <int D, int BF16>
-__global__ void __launch_bounds__(1024, 1) tabulate_staged_kernel(const float* __restrict__ in, void* __restrict__ out,
+__global__ void __launch_bounds__(1024, 1) tabulate_staged_kernel(const float* in, void* out,
                                                               int q, int64_t P, int64_t Bn, int64_t state_elems,
                                                               int E) {
   extern __shared__ __align__(16) float4 smem4[];
+  pdl_trigger();
+  pdl_wait();
   const int L4 = E / 4;                 // float4 lanes per item
   const int NT = blockDim.x;
   const int IPP = NT / L4;              // items per pass
@@ -206,8 +209,10 @@ __device__ __noinline__ void radon_inplace(float* base) {
 // Larger fields do not fit a q x q image in the registers of one thread and use tabulate_staged_kernel.
 template <int Q, int E, int BF16>
 __global__ void __maxnreg__(Q <= 11 ? 168 : 224)
-    tabulate_radon3_kernel(const float* __restrict__ in, void* __restrict__ out, int P, int Bn, int64_t state_elems) {
+    tabulate_radon3_kernel(const float* in, void* out, int P, int Bn, int64_t state_elems) {
   extern __shared__ __align__(16) float4 smem4[];
+  pdl_trigger();
+  pdl_wait();
   constexpr int q = Q, qq = Q * Q;
   constexpr int L4 = E / 4;
   constexpr int log2L4 = E == 32 ? 3 : 2;
@@ -269,10 +274,12 @@ __global__ void __maxnreg__(Q <= 11 ? 168 : 224)
 
 // Transpose for D = 2:  F̄[x1, x2] = Σ_{a2} Ū[(1,a2), x1 + a2 x2] + Ū[(0,1), x2]
 template <int BF16>
-__global__ void __launch_bounds__(1024, 1) tabulate_staged_t2_kernel(const float* __restrict__ in, void* __restrict__ out,
+__global__ void __launch_bounds__(1024, 1) tabulate_staged_t2_kernel(const float* in, void* out,
                                                                  int q, int64_t P, int64_t Bn, int64_t state_elems,
                                                                  int E) {
   extern __shared__ __align__(16) float4 smem4[];
+  pdl_trigger();
+  pdl_wait();
   const int L4 = E / 4, NT = blockDim.x, IPP = NT / L4;
   const int tid = threadIdx.x;
   const int l = tid % L4, it0 = tid / L4;
@@ -310,7 +317,7 @@ cudaError_t set_smem(K kernel, size_t bytes) {
 
 }  // namespace
 
-__global__ void widen_bf16_kernel(const __nv_bfloat16* __restrict__ src, float* __restrict__ dst, int64_t count) {
+__global__ void widen_bf16_kernel(const __nv_bfloat16* src, float* dst, int64_t count) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < count) dst[i] = __bfloat162float(src[i]);
 }
@@ -361,10 +368,10 @@ cudaError_t smat_launch_tabulate_staged(const float* in, void* out, const SmatGe
     const int nr = (QV * EV + 31) / 32 * 32; /* one thread per (image, entry) */                                 \
     if (out_bf16) {                                                                                              \
       if ((err = set_smem(tabulate_radon3_kernel<QV, EV, 1>, smem)) != cudaSuccess) return err;                  \
-      tabulate_radon3_kernel<QV, EV, 1><<<grid, nr, smem, st>>>(in, out, (int)geo.P, (int)geo.B, state_elems);   \
+      return smat_launch_pdl(tabulate_radon3_kernel<QV, EV, 1>, grid, nr, smem, st, in, out, (int)geo.P, (int)geo.B, state_elems); \
     } else {                                                                                                     \
       if ((err = set_smem(tabulate_radon3_kernel<QV, EV, 0>, smem)) != cudaSuccess) return err;                  \
-      tabulate_radon3_kernel<QV, EV, 0><<<grid, nr, smem, st>>>(in, out, (int)geo.P, (int)geo.B, state_elems);   \
+      return smat_launch_pdl(tabulate_radon3_kernel<QV, EV, 0>, grid, nr, smem, st, in, out, (int)geo.P, (int)geo.B, state_elems); \
     }                                                                                                            \
     return cudaGetLastError();                                                                                   \
   }
@@ -375,16 +382,16 @@ cudaError_t smat_launch_tabulate_staged(const float* in, void* out, const SmatGe
   if (geo.D == 2 && transpose) {
     if (out_bf16) {
       if ((err = set_smem(tabulate_staged_t2_kernel<1>, smem)) != cudaSuccess) return err;
-      tabulate_staged_t2_kernel<1><<<grid, nt, smem, st>>>(in, out, geo.q, geo.P, geo.B, state_elems, E);
+      return smat_launch_pdl(tabulate_staged_t2_kernel<1>, grid, nt, smem, st, in, out, geo.q, geo.P, geo.B, state_elems, E);
     } else {
       if ((err = set_smem(tabulate_staged_t2_kernel<0>, smem)) != cudaSuccess) return err;
-      tabulate_staged_t2_kernel<0><<<grid, nt, smem, st>>>(in, out, geo.q, geo.P, geo.B, state_elems, E);
+      return smat_launch_pdl(tabulate_staged_t2_kernel<0>, grid, nt, smem, st, in, out, geo.q, geo.P, geo.B, state_elems, E);
     }
   } else {
 #define SMAT_STAGED(DV, BV)                                                                         \
   if (geo.D == DV && out_bf16 == BV) {                                                              \
     if ((err = set_smem(tabulate_staged_kernel<DV, BV>, smem)) != cudaSuccess) return err;          \
-    tabulate_staged_kernel<DV, BV><<<grid, nt, smem, st>>>(in, out, geo.q, geo.P, geo.B, state_elems, E); \
+    return smat_launch_pdl(tabulate_staged_kernel<DV, BV>, grid, nt, smem, st, in, out, geo.q, geo.P, geo.B, state_elems, E); \
   }
     SMAT_STAGED(2, 0) SMAT_STAGED(2, 1) SMAT_STAGED(3, 0) SMAT_STAGED(3, 1)
 #undef SMAT_STAGED
@@ -396,10 +403,12 @@ cudaError_t smat_launch_tabulate_staged(const float* in, void* out, const SmatGe
 // U = R F (the two-dimensional Radon sums of Algorithm 2 for d = 3) from a bf16 profile table: the slab F[:, e0 .. e0+E)
 // sits in shared memory as bf16, a thread owns 8 entries of one output row and adds in fp32.  Against the fp32 form
 // this halves the shared-memory bytes per addition, which is what bounds these sums.
-__global__ void __launch_bounds__(256) tabulate_d3_bf16_kernel(const __nv_bfloat16* __restrict__ in,
-                                                               __nv_bfloat16* __restrict__ out, int q, int64_t P,
+__global__ void __launch_bounds__(256) tabulate_d3_bf16_kernel(const __nv_bfloat16* in,
+                                                               __nv_bfloat16* out, int q, int64_t P,
                                                                int64_t Bn, int64_t state_elems, int E) {
   extern __shared__ __align__(16) uint4 smem8[];            // [P][E / 8]: 8 bf16 per element
+  pdl_trigger();
+  pdl_wait();
   const int L8 = E / 8, NT = blockDim.x, tid = threadIdx.x;
   const int l = tid % L8, it0 = tid / L8, IPP = NT / L8;
   const int64_t bh = blockIdx.y, e0 = (int64_t)blockIdx.x * E;
@@ -468,9 +477,8 @@ cudaError_t smat_launch_tabulate_d3_bf16(const void* in, void* out, const SmatGe
   cudaError_t err = set_smem(tabulate_d3_bf16_kernel, smem);
   if (err != cudaSuccess) return err;
   dim3 grid((unsigned)(state_elems / E), (unsigned)bh);
-  tabulate_d3_bf16_kernel<<<grid, 256, smem, st>>>(static_cast<const __nv_bfloat16*>(in), static_cast<__nv_bfloat16*>(out),
-                                                   geo.q, geo.P, geo.B, state_elems, E);
-  return cudaGetLastError();
+  return smat_launch_pdl(tabulate_d3_bf16_kernel, grid, 256, smem, st, static_cast<const __nv_bfloat16*>(in),
+                         static_cast<__nv_bfloat16*>(out), geo.q, geo.P, geo.B, state_elems, E);
 }
 
 cudaError_t smat_launch_widen_bf16(const void* src_bf16, float* dst, int64_t count, cudaStream_t st) {

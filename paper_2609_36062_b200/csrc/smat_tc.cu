@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include "smat_internal.h"
+#include "smat_launch.cuh"
 #include "smat_tc.cuh"
 
 namespace {
@@ -77,6 +78,8 @@ __global__ void __launch_bounds__(192) chunk_scan_tc_kernel(const __grid_constan
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
+  pdl_trigger();   // (after the allocation: a kernel that starts early must not take the tensor memory first)
+  pdl_wait();
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 4 && lane == 0) {
@@ -221,7 +224,6 @@ __global__ void __launch_bounds__(160) tile_product_tc_kernel(const __grid_const
   const int bh = blockIdx.y;
   const int64_t row0 = (int64_t)bh * prm.T + (int64_t)b * TILE;
   const WaitCtx wc{cta_abort, prm.status};
-  if (GATED && threadIdx.x < TILE) sLam[threadIdx.x] = prm.lam[row0 + threadIdx.x];
 
   if (threadIdx.x == 0) {
     *cta_abort = 0;
@@ -232,7 +234,13 @@ __global__ void __launch_bounds__(160) tile_product_tc_kernel(const __grid_const
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
+  pdl_trigger();
+  pdl_wait();
   const uint32_t tmem_base = *tmem_slot;
+  if (GATED) {
+    if (threadIdx.x < TILE) sLam[threadIdx.x] = prm.lam[row0 + threadIdx.x];
+    __syncthreads();
+  }
   const uint32_t tmem_sc = tmem_base, tmem_o = tmem_base + TILE;
   const uint32_t tmem_st = GATED ? tmem_base + TILE + HALF : tmem_o;   // accumulator of the state product
 
@@ -353,7 +361,7 @@ __global__ void __launch_bounds__(160) tile_product_tc_kernel(const __grid_const
 #pragma unroll
             for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[i * 8 + e]);
             if (add_lr && prm.addend16) {
-              const uint4 a = __ldg(y16 + cb * 4 + i);   // 8 bf16 values
+              const uint4 a = *(y16 + cb * 4 + i);   // 8 bf16 values
               const uint32_t yy[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
@@ -361,7 +369,7 @@ __global__ void __launch_bounds__(160) tile_product_tc_kernel(const __grid_const
                 f[2 * e + 1] += __uint_as_float(yy[e] & 0xffff0000u);
               }
             } else if (add_lr) {
-              const float4 a = __ldg(y4 + cb * 8 + i * 2), c = __ldg(y4 + cb * 8 + i * 2 + 1);
+              const float4 a = *(y4 + cb * 8 + i * 2), c = *(y4 + cb * 8 + i * 2 + 1);
               f[0] += a.x; f[1] += a.y; f[2] += a.z; f[3] += a.w;
               f[4] += c.x; f[5] += c.y; f[6] += c.z; f[7] += c.w;
             }
@@ -445,7 +453,6 @@ __global__ void __launch_bounds__(160) bwd_tile_fused_tc_kernel(const __grid_con
   const int b = blockIdx.x, bh = blockIdx.y;
   const int64_t row0 = (int64_t)bh * prm.T + (int64_t)b * TILE;
   const WaitCtx wc{cta_abort, prm.status};
-  if (GATED && threadIdx.x < TILE) sLam[threadIdx.x] = prm.lam[row0 + threadIdx.x];
   if (threadIdx.x == 0) {
     *cta_abort = 0;
     mbar_init(bar_in0, 1); mbar_init(bar_in1, 1); mbar_init(bar_sc, 1); mbar_init(bar_p, 4); mbar_init(bar_x, 1);
@@ -456,7 +463,13 @@ __global__ void __launch_bounds__(160) bwd_tile_fused_tc_kernel(const __grid_con
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
+  pdl_trigger();
+  pdl_wait();
   const uint32_t tmem_base = *tmem_slot;
+  if (GATED) {
+    if (threadIdx.x < TILE) sLam[threadIdx.x] = prm.lam[row0 + threadIdx.x];
+    __syncthreads();
+  }
   const uint32_t tm_sc = tmem_base, tm_dq = tmem_base + TILE, tm_dk = tmem_base + 2 * TILE, tm_dv = tmem_base + 3 * TILE;
 
   if (warp == 4 && lane == 0) {
@@ -571,7 +584,7 @@ __global__ void __launch_bounds__(160) bwd_tile_fused_tc_kernel(const __grid_con
 #pragma unroll
           for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[i * 8 + e]);
           if (add) {
-            const uint4 a = __ldg(y16 + cb * 4 + i);
+            const uint4 a = *(y16 + cb * 4 + i);
             const uint32_t yy[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -715,6 +728,8 @@ __global__ void __launch_bounds__(192) segment_state_tc_kernel(const __grid_cons
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
+  pdl_trigger();
+  pdl_wait();
   const uint32_t tmem_d = *tmem_slot;
   if (warp == 4 && lane == 0) {
     for (int it = 0; it < Lc; ++it) {
@@ -860,6 +875,8 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
+  pdl_trigger();
+  pdl_wait();
   const uint32_t tmem_base = *tmem_slot;
   const uint32_t tmem_s = tmem_base, tmem_sc = tmem_base + TILE, tmem_o0 = tmem_base + 2 * TILE;
 
@@ -1025,7 +1042,7 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
       const uint4* src = reinterpret_cast<const uint4*>(prm.seg_in + (((int64_t)bh * prm.nseg + seg) * TILE + m) * TILE + col0);
 #pragma unroll
       for (int q4 = 0; q4 < 8; ++q4) {
-        const uint4 a = __ldg(src + q4);
+        const uint4 a = *(src + q4);
         v[4 * q4] = a.x; v[4 * q4 + 1] = a.y; v[4 * q4 + 2] = a.z; v[4 * q4 + 3] = a.w;
       }
       tmem_st32(tmem_s + lane_base + col0, v);
@@ -1075,7 +1092,7 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
         const uint4* y4 = SPLIT ? reinterpret_cast<const uint4*>(prm.ylr32 + ((int64_t)bh * prm.T + t) * TILE + col0)
                                 : reinterpret_cast<const uint4*>(prm.ylr + ((int64_t)bh * prm.T + t) * TILE + col0);
 #pragma unroll
-        for (int i = 0; i < (SPLIT ? 8 : 4); ++i) y[i] = __ldg(y4 + i);
+        for (int i = 0; i < (SPLIT ? 8 : 4); ++i) y[i] = *(y4 + i);
       }
       if (!mbar_wait(bar_o, it & 1, wc)) break;
       fence_after_sync();
@@ -1210,6 +1227,8 @@ __global__ void __launch_bounds__(160) state_read_tc_kernel(const __grid_constan
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
+  pdl_trigger();
+  pdl_wait();
   const uint32_t tmem_d = *tmem_slot;
   constexpr uint32_t idesc = make_idesc(TILE, TILE, 0, TRANS ? 0 : 1);
   constexpr uint32_t idesc2 = make_idesc(TILE, TILE, 0, 1);
@@ -1378,7 +1397,7 @@ struct PoolPass {
 };
 
 template <int TOK, int OUT_BF16>
-__global__ void __launch_bounds__(160) pool_tc_kernel(const PoolParams prm) {
+__global__ void __launch_bounds__(160) pool_tc_kernel(const __grid_constant__ PoolParams prm) {
   constexpr int OP_BYTES = 2 * TOK * 128;  // one operand: two 64-feature blocks of TOK rows x 128 bytes
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -1405,6 +1424,8 @@ __global__ void __launch_bounds__(160) pool_tc_kernel(const PoolParams prm) {
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
+  pdl_trigger();
+  pdl_wait();
   const uint32_t tmem_d = *tmem_slot;
   constexpr uint32_t idesc = make_idesc(TILE, TILE, 1, 1);
   PoolPass<TOK> cur(prm, blockIdx.x, gridDim.x);
@@ -1610,8 +1631,7 @@ cudaError_t smat_launch_chunk_scan_tc(const void* K, const void* V, void* Sin_bf
   cudaError_t err = cudaFuncSetAttribute(chunk_scan_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SCAN_SMEM);
   if (err != cudaSuccess) return err;
   dim3 grid((unsigned)(blocks * 2), (unsigned)bh);
-  chunk_scan_tc_kernel<<<grid, 192, SCAN_SMEM, st>>>(tmK, tmV, prm);
-  return cudaGetLastError();
+  return smat_launch_pdl(chunk_scan_tc_kernel, grid, 192, SCAN_SMEM, st, tmK, tmV, prm);
 }
 
 template <bool P4_IS_P1, bool XT, bool ST_KMAJOR, bool GATED = false>
@@ -1634,8 +1654,7 @@ static cudaError_t launch_tile_product(const void* P1, const void* P2, const voi
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, OUT_SMEM);
   if (err != cudaSuccess) return err;
   dim3 grid((unsigned)(NC * 2), (unsigned)bh);
-  tile_product_tc_kernel<P4_IS_P1, XT, ST_KMAJOR, GATED><<<grid, 160, OUT_SMEM, st>>>(tm1, tm2, tm3, tmS, prm);
-  return cudaGetLastError();
+  return smat_launch_pdl(tile_product_tc_kernel<P4_IS_P1, XT, ST_KMAJOR, GATED>, grid, 160, OUT_SMEM, st, tm1, tm2, tm3, tmS, prm);
 }
 
 cudaError_t smat_launch_chunk_output_tc(const void* Q, const void* K, const void* V, const void* Sin_bf16,
@@ -1683,8 +1702,7 @@ cudaError_t smat_launch_bwd_tiles_fused_tc(const void* Q, const void* K, const v
   cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSED_SMEM);
   if (err != cudaSuccess) return err;
   dim3 grid((unsigned)NC, (unsigned)bh);
-  kernel<<<grid, 160, FUSED_SMEM, st>>>(tmQ, tmK, tmV, tmG, tmS, tmD, prm);
-  return cudaGetLastError();
+  return smat_launch_pdl(kernel, grid, 160, FUSED_SMEM, st, tmQ, tmK, tmV, tmG, tmS, tmD, prm);
 }
 
 // Both adjoint reads of the profile states in one launch: out_t[t] = St x_t (rows Xt, the second state index
@@ -1709,8 +1727,7 @@ cudaError_t smat_launch_state_read_dual_tc(const void* Xt, const void* Xn, const
   const int64_t grid = prm.items < 2LL * sms ? prm.items : 2LL * sms;   // 256 columns of tensor memory and 97 KB each
   cudaError_t err = cudaFuncSetAttribute(state_read_tc_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
-  state_read_tc_kernel<1, 1><<<(unsigned)grid, 160, smem, st>>>(tmU, prm);
-  return cudaGetLastError();
+  return smat_launch_pdl(state_read_tc_kernel<1, 1>, dim3((unsigned)grid), 160, smem, st, tmU, prm);
 }
 
 cudaError_t smat_launch_state_read_tc(const void* X, const void* state_bf16, float* out, void* out_bf16, int transposed,
@@ -1729,17 +1746,10 @@ cudaError_t smat_launch_state_read_tc(const void* X, const void* state_bf16, flo
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t grid = prm.items < 3LL * sms ? prm.items : 3LL * sms;
-  cudaError_t err;
-  if (transposed) {
-    err = cudaFuncSetAttribute(state_read_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, READ_SMEM);
-    if (err != cudaSuccess) return err;
-    state_read_tc_kernel<1><<<(unsigned)grid, 160, READ_SMEM, st>>>(tmU, prm);
-  } else {
-    err = cudaFuncSetAttribute(state_read_tc_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, READ_SMEM);
-    if (err != cudaSuccess) return err;
-    state_read_tc_kernel<0><<<(unsigned)grid, 160, READ_SMEM, st>>>(tmU, prm);
-  }
-  return cudaGetLastError();
+  auto kernel = transposed ? state_read_tc_kernel<1> : state_read_tc_kernel<0>;
+  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, READ_SMEM);
+  if (err != cudaSuccess) return err;
+  return smat_launch_pdl(kernel, dim3((unsigned)grid), 160, READ_SMEM, st, tmU, prm);
 }
 
 template <int TOK, int OUT_BF16>
@@ -1753,8 +1763,7 @@ static cudaError_t launch_pool_tc(const PoolParams& prm, cudaStream_t st) {
   // each CTA holds 128 columns of tensor memory, so at most four fit an SM
   const int per_sm = smem <= 54 * 1024 ? 4 : (smem <= 72 * 1024 ? 3 : (smem <= 110 * 1024 ? 2 : 1));
   const int64_t grid = prm.items < (int64_t)per_sm * sms ? prm.items : (int64_t)per_sm * sms;
-  pool_tc_kernel<TOK, OUT_BF16><<<(unsigned)grid, 160, smem, st>>>(prm);
-  return cudaGetLastError();
+  return smat_launch_pdl(pool_tc_kernel<TOK, OUT_BF16>, dim3((unsigned)grid), 160, smem, st, prm);
 }
 
 cudaError_t smat_launch_pool_tc(const void* K, const void* V, void* F, int out_bf16, const SmatGroupSpec& grp,
@@ -1833,8 +1842,7 @@ cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* to
       cudaFuncSetAttribute(segment_state_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SEG_STATE_SMEM);
   if (err != cudaSuccess) return err;
   dim3 grid((unsigned)prm.nseg, (unsigned)bh);
-  segment_state_tc_kernel<<<grid, 192, SEG_STATE_SMEM, st>>>(tmK, tmV, prm);
-  return cudaGetLastError();
+  return smat_launch_pdl(segment_state_tc_kernel, grid, 192, SEG_STATE_SMEM, st, tmK, tmV, prm);
 }
 
 cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const void* V, const float* seg_in,
@@ -1863,6 +1871,5 @@ cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const vo
   cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
   dim3 grid((unsigned)prm.nseg, (unsigned)bh);
-  kernel<<<grid, SEG_OUT_THREADS, smem, st>>>(maps, prm);
-  return cudaGetLastError();
+  return smat_launch_pdl(kernel, grid, SEG_OUT_THREADS, smem, st, maps, prm);
 }
