@@ -861,9 +861,9 @@ smat_status forward_gated_tc(Ctx& cx, const Gated& gt, const void* Q, const void
   ci.rec = pl;
   int* status = reinterpret_cast<int*>(ci.ws + in->off_status);
   SMAT_TRY(cx, "gate_prefix", smat_launch_head_scan(log_a, gt.lam, pl->T, pl->bh, 0, cx.st));
-  SMAT_TRY(cx, "gate_scale_k", smat_launch_gate_scale(K, nullptr, gt.kc, gt.lam, 1, 1, pl->geo.n, 128, pl->T, pl->r, pl->bh,
-                                                      cx.st));                                // exp(λ_{tile end} - λ_j) k_j
-  if (lr) gate_scale(cx, "gate_scale_lr", K, Q, gt.lr, gt.lam, 2, pl->r);                    // split at the boundary
+  // exp(λ_{tile end} - λ_j) k_j, and keys and queries split at the boundary
+  SMAT_TRY(cx, "gate_scale", smat_launch_gate_scale_pair(K, K, Q, gt.kc, lr ? gt.lr : nullptr, gt.lam, 1, pl->geo.n, pl->T,
+                                                         pl->bh, cx.st));
   ci.err = cx.err;
   float* ylr = ci.f(in->off_acc);
   if (lr) {
@@ -894,7 +894,7 @@ bool gated_backward_on_tc(const smat_plan* pl) {
 // Gated backward on the tensor cores: the ungated adjoint pipeline on rescaled copies (Ū from the boundary-scaled
 // queries, the reads of U and F̄ on the boundary-scaled dO, V and K), the decayed scans for S_in (keys rescaled to the
 // end of their tile) and D̄ (queries rescaled to the start of theirs, reverse order), and the fused tile kernel with
-// the decays on both score tiles and the row factors on the three state products.  dλ_t = q_t·dQ_t - k_t·dK_t.
+// the decays on both score tiles and the row factors on the three state products; it also forms dλ_t = q_t·dQ_t - k_t·dK_t.
 smat_status backward_gated_tc(Ctx& cx, const Gated& gt, const void* Q, const void* K, const void* V, const float* log_a,
                               const void* dO, void* dQ, void* dK, void* dV, float* dlog_a, bool after_gated_forward) {
   const smat_plan* pl = cx.pl;
@@ -909,14 +909,15 @@ smat_status backward_gated_tc(Ctx& cx, const Gated& gt, const void* Q, const voi
   const bool kept = (pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES) && after_gated_forward;
   if (!kept) {
     SMAT_TRY(cx, "gate_prefix", smat_launch_head_scan(log_a, gt.lam, pl->T, pl->bh, 0, cx.st));
-    SMAT_TRY(cx, "gate_scale_k", smat_launch_gate_scale(K, nullptr, gt.kc, gt.lam, 1, 1, n, 128, pl->T, pl->r, pl->bh, cx.st));
-    if (lr) gate_scale(cx, "gate_scale_lr", K, Q, gt.lr, gt.lam, 2, pl->r);
+    SMAT_TRY(cx, "gate_scale", smat_launch_gate_scale_pair(K, K, Q, gt.kc, lr ? gt.lr : nullptr, gt.lam, 1, n, pl->T, pl->bh,
+                                                           cx.st));
   }
-  SMAT_TRY(cx, "bwd_gate_scale_q", smat_launch_gate_scale(Q, nullptr, gt.qc, gt.lam, 0, 1, n, 128, pl->T, pl->r, pl->bh, cx.st));
-  if (lr) gate_scale(cx, "bwd_gate_scale_lr", V, dO, gt.vlr, gt.lam, 2, pl->p);
+  SMAT_TRY(cx, "bwd_gate_scale", smat_launch_gate_scale_pair(Q, V, dO, gt.qc, lr ? gt.vlr : nullptr, gt.lam, 0, n, pl->T,
+                                                             pl->bh, cx.st));
   ci.err = cx.err;
   char* sin = ci.ws + in->off_sin;
   char* dbar = ci.ws + in->off_dbar;
+  float* dlam = cx.f(pl->off_dlam);
   char *lr_q = nullptr, *lr_k = nullptr, *lr_v = nullptr;
   if (lr) {
     const SmatGroupSpec types = group(ci, SMAT_GM_TYPE), profs = group(ci, SMAT_GM_PROFILE);
@@ -945,11 +946,9 @@ smat_status backward_gated_tc(Ctx& cx, const Gated& gt, const void* Q, const voi
                                                                       ci.st, gt.lam));
   SMAT_TRY(ci, "bwd_gated_tiles_fused_tc", smat_launch_bwd_tiles_fused_tc(Q, K, V, dO, sin, dbar, lr_q, lr_k, lr_v,
                                                                            lr ? n : in->T, dQ, dK, dV, in->T, in->bh, status,
-                                                                           ci.st, gt.lam));
+                                                                           ci.st, gt.lam, dlam));
   cx.err = ci.err;
   cx.launches += ci.launches;
-  float* dlam = cx.f(pl->off_dlam);
-  SMAT_TRY(cx, "bwd_gate_dlam", smat_launch_gate_dlam(Q, dQ, K, dK, dlam, 1, pl->r, pl->T, pl->bh, cx.st));
   SMAT_TRY(cx, "bwd_gate_suffix", smat_launch_head_scan(dlam, dlog_a, pl->T, pl->bh, 1, cx.st));
   pl->launches = cx.launches;
   return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;

@@ -10,36 +10,53 @@
 
 namespace {
 
-// Inclusive prefix (reverse = 0) or suffix (reverse = 1) sum of one row of `len` floats per head; one CTA per head.
-__global__ void __launch_bounds__(1024) head_scan_kernel(const float* in, float* out, int64_t len,
-                                                         int reverse) {
-  __shared__ float warp_sum[32];
-  __shared__ float carry;
+// Inclusive prefix (reverse = 0) or suffix (reverse = 1) sum of one row of `len` floats per head; one CTA per head, 4096
+// values per turn: a warp scans 128 neighbouring values, the warp totals are scanned by shuffles.  Bound by its few
+// dependent steps (32 heads of 4096: 7 us alone, 11 with one value per thread and turn and the totals summed one by one).
+__global__ void __launch_bounds__(1024) head_scan_kernel(const float* in, float* out, int64_t len, int reverse) {
   pdl_trigger();
-  pdl_wait();
-  const int tid = threadIdx.x;
+  __shared__ float warp_sum[2][32];
+  constexpr int PER = 4;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float* src = in + (int64_t)blockIdx.x * len;
   float* dst = out + (int64_t)blockIdx.x * len;
-  if (tid == 0) carry = 0.f;
-  __syncthreads();
-  for (int64_t base = 0; base < len; base += 1024) {
-    const int64_t k = base + tid;
-    const int64_t idx = reverse ? len - 1 - k : k;
-    const float v = k < len ? src[idx] : 0.f;
-    float x = v;
+  float carry = 0.f;
+  pdl_wait();
+  for (int64_t base = 0, turn = 0; base < len; base += 1024 * PER, turn ^= 1) {
+    const int64_t k0 = base + warp * 32 * PER + lane;
+    float x[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int64_t k = k0 + 32 * i;
+      x[i] = k < len ? src[reverse ? len - 1 - k : k] : 0.f;
+    }
+    float run = 0.f;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const float y = __shfl_up_sync(0xffffffffu, x[i], d);
+        if (lane >= d) x[i] += y;
+      }
+      x[i] += run;
+      run = __shfl_sync(0xffffffffu, x[i], 31);
+    }
+    if (lane == 31) warp_sum[turn][warp] = run;
+    __syncthreads();
+    const float own = warp_sum[turn][lane];
+    float tot = own;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-      const float y = __shfl_up_sync(0xffffffffu, x, d);
-      if ((tid & 31) >= d) x += y;
+      const float y = __shfl_up_sync(0xffffffffu, tot, d);
+      if (lane >= d) tot += y;
     }
-    if ((tid & 31) == 31) warp_sum[tid >> 5] = x;
-    __syncthreads();
-    float before = carry;
-    for (int w = 0; w < (tid >> 5); ++w) before += warp_sum[w];
-    if (k < len) dst[idx] = before + x;
-    __syncthreads();
-    if (tid == 1023) carry = before + x;
-    __syncthreads();
+    const float before = carry + __shfl_sync(0xffffffffu, tot - own, warp);
+    carry += __shfl_sync(0xffffffffu, tot, 31);
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int64_t k = k0 + 32 * i;
+      if (k < len) dst[reverse ? len - 1 - k : k] = before + x[i];
+    }
   }
 }
 
@@ -86,6 +103,54 @@ __global__ void gate_scale_kernel(const T* A, const T* B, T* out,
     return;
   }
   for (int i = lane; i < dim; i += 32) out[row * dim + i] = (T)((float)src[row * dim + i] * f);
+}
+
+// Both rescaled copies a tensor-core pass needs, from one read of their rows (bf16, 128 columns):
+//   out1[t] = A[t] * f(t), the query side (mode 0) or key side (mode 1) of t's 128-token tile;
+//   out2[t] = (t < n ? B : C)[t] * f(t) at the block boundary (null: d = 1, no long-range branch).
+// Sixteen lanes per row, eight rows in flight per warp.  32 heads of 4096 tokens (117 MB): 0.021 ms, where two launches
+// with 8 bytes per lane and one row per warp took 0.056.
+constexpr int SCALE_ROWS = 4;   // rows per half warp
+__device__ __forceinline__ uint4 scale8(const uint4 v, float f) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  uint32_t o[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const __nv_bfloat162 p = __floats2bfloat162_rn(__uint_as_float(w[i] << 16) * f, __uint_as_float(w[i] & 0xffff0000u) * f);
+    o[i] = *reinterpret_cast<const uint32_t*>(&p);
+  }
+  return make_uint4(o[0], o[1], o[2], o[3]);
+}
+__global__ void __launch_bounds__(256) gate_scale_pair_kernel(const uint4* A, const uint4* B, const uint4* C, uint4* out1,
+                                                              uint4* out2, const float* lam, int mode, int64_t n,
+                                                              int64_t Tlen, int64_t rows) {
+  pdl_trigger();
+  pdl_wait();
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
+  const int lane = threadIdx.x & 31, col = lane & 15;
+  uint4 a[SCALE_ROWS], b[SCALE_ROWS];
+  float f1[SCALE_ROWS], f2[SCALE_ROWS];
+#pragma unroll
+  for (int u = 0; u < SCALE_ROWS; ++u) {
+    const int64_t row = (warp * SCALE_ROWS + u) * 2 + (lane >> 4);
+    if (row >= rows) continue;
+    const int64_t bh = row / Tlen, t = row - bh * Tlen;
+    const float* l = lam + bh * Tlen;
+    const uint4* src2 = t < n ? B : C;
+    a[u] = A[row * 16 + col];
+    b[u] = a[u];
+    if (out2 && src2 != A) b[u] = src2[row * 16 + col];
+    const int64_t t0 = t & ~(int64_t)127;
+    f1[u] = mode == 0 ? __expf(l[t] - (t0 > 0 ? l[t0 - 1] : 0.f)) : __expf(l[t0 + 127] - l[t]);
+    if (out2) f2[u] = t < n ? __expf(l[n - 1] - l[t]) : __expf(l[t] - l[n - 1]);
+  }
+#pragma unroll
+  for (int u = 0; u < SCALE_ROWS; ++u) {
+    const int64_t row = (warp * SCALE_ROWS + u) * 2 + (lane >> 4);
+    if (row >= rows) continue;
+    out1[row * 16 + col] = scale8(a[u], f1[u]);
+    if (out2) out2[row * 16 + col] = scale8(b[u], f2[u]);
+  }
 }
 
 // Decayed exclusive scan of per-chunk states in place: walking the chunks of a range in order (or in reverse),
@@ -146,6 +211,14 @@ cudaError_t smat_launch_gate_scale(const void* A, const void* B, void* out, cons
                            static_cast<const __nv_bfloat16*>(B), static_cast<__nv_bfloat16*>(out), lam, mode, n, c, T, dim, rows);
   return smat_launch_pdl(gate_scale_kernel<float>, dim3(blocks), 256, 0, st, static_cast<const float*>(A),
                          static_cast<const float*>(B), static_cast<float*>(out), lam, mode, n, c, T, dim, rows);
+}
+
+cudaError_t smat_launch_gate_scale_pair(const void* A, const void* B, const void* C, void* out1, void* out2, const float* lam,
+                                        int mode, int64_t n, int64_t T, int bh, cudaStream_t st) {
+  const int64_t rows = (int64_t)bh * T, warps = (rows + 2 * SCALE_ROWS - 1) / (2 * SCALE_ROWS);
+  return smat_launch_pdl(gate_scale_pair_kernel, dim3((unsigned)((warps + 7) / 8)), 256, 0, st, static_cast<const uint4*>(A),
+                         static_cast<const uint4*>(B), static_cast<const uint4*>(C), static_cast<uint4*>(out1),
+                         static_cast<uint4*>(out2), lam, mode, n, T, rows);
 }
 
 cudaError_t smat_launch_gated_scan(float* S, const float* lam, int64_t state_elems, int64_t NC, int64_t c, int bh,

@@ -158,7 +158,7 @@ cudaError_t smat_launch_chunk_adjoint_tc(int which, const void* Q, const void* K
 cudaError_t smat_launch_bwd_tiles_fused_tc(const void* Q, const void* K, const void* V, const void* dO,
                                            const void* Sin_bf16, const void* Dbar_bf16, const void* lr_q, const void* lr_k,
                                            const void* lr_v, int64_t n, void* dQ, void* dK, void* dV, int64_t T, int bh,
-                                           int* status, cudaStream_t st, const float* lam = nullptr);
+                                           int* status, cudaStream_t st, const float* lam = nullptr, float* dlam = nullptr);
 // O_b = Q_b S_in[b] + tril(Q_b K_bᵀ) V_b (+ ylr rows for tokens >= n_lr).
 cudaError_t smat_launch_chunk_output_tc(const void* Q, const void* K, const void* V, const void* Sin_bf16,
                                         const float* ylr, int64_t n_lr, void* O, int64_t T, int bh, int* status,
@@ -202,6 +202,10 @@ cudaError_t smat_launch_pool_tc(const void* K, const void* V, void* F, int out_b
 cudaError_t smat_launch_head_scan(const float* in, float* out, int64_t len, int bh, int reverse, cudaStream_t st);
 cudaError_t smat_launch_gate_scale(const void* A, const void* B, void* out, const float* lam, int mode, int bf16,
                                    int64_t n, int64_t c, int64_t T, int dim, int bh, cudaStream_t st);
+// out1 = A rescaled to its 128-token tile (mode 0: from its start, 1: to its end), out2 = B (t < n) or C rescaled to the
+// block boundary (null: skipped); bf16 rows of 128.
+cudaError_t smat_launch_gate_scale_pair(const void* A, const void* B, const void* C, void* out1, void* out2, const float* lam,
+                                        int mode, int64_t n, int64_t T, int bh, cudaStream_t st);
 cudaError_t smat_launch_gated_scan(float* S, const float* lam, int64_t state_elems, int64_t NC, int64_t c, int bh,
                                    int64_t lo0, int64_t hi0, int64_t lo1, int64_t hi1, int reverse, cudaStream_t st);
 cudaError_t smat_launch_gate_dlam(const void* Q, const void* dQ, const void* K, const void* dK, float* dlam, int bf16,

@@ -393,190 +393,268 @@ __global__ void __launch_bounds__(160) tile_product_tc_kernel(const __grid_const
 }
 
 // ---------------------------------------------------------------------------------------------------------------
-// bwd_tile_fused_tc_kernel: the three within-chunk adjoints of one 128-token tile in ONE CTA (Eq. "local-adjoint"
-// with the broadcast of the scanned state adjoint), all 128 output columns:
+// bwd_tile_fused_tc_kernel: the three within-chunk adjoints of a 128-token tile (Eq. "local-adjoint" with the broadcast
+// of the scanned state adjoint), all 128 output columns; persistent, one CTA per SM:
 //        G = tril(dO Vᵀ),  A = tril(Q Kᵀ)
 //        dQ = dO S_inᵀ + G K,      dK = V D̄ᵀ + Gᵀ Q,      dV = K D̄ + Aᵀ dO      (+ the long-range rows of each)
 // Q, K, V, dO, S_in and D̄ of the tile are loaded once (the three separate tile kernels load 2.7 times as much) and
-// the two score tiles are formed once.  Shared memory: seven 32 KB tiles (Q, K, V, dO, S_in, D̄, X); tensor memory:
-// scores [0,128), dQ [128,256), dK [256,384), dV [384,512).
-//   warp 4 lane 0 : TMA loads (dO, V first: the G scores need nothing else), then every MMA in order
-//   warps 0-3     : one tile row per thread: mask and round G, later A, into the swizzled X tile; read the three
-//                   accumulators, add the long-range rows and store
+// the two score tiles are formed once.  Shared memory: seven 32 KB tiles (Q, K, V, dO, S_in, D̄, and the rounded G; the
+// rounded A takes S_in's place once dO S_inᵀ is formed); tensor memory: G scores, then dV [0,128), dQ [128,256),
+// dK [256,384), A scores [384,512).  Nothing is held twice, but every operand goes back to the producer as soon as its
+// last product is done (V, D̄, then Q and K, then dO and S_in), so that most of the next tile's 192 KB travel while this
+// tile's rows are written out.
+//   warps 0-15 : each owns 32 rows x 32 columns of every 128 x 128 tile: mask and round the scores, read the three
+//                accumulators, add the long-range rows and store
+//   warp 16    : TMA producer;   warp 17 : MMA issuer (whole warps walk the loops, one lane issues)
+// A tile moves 342 KB: 128 heads of 8192 tokens (2.8 GB) take 0.467 ms, 0.43 at the HBM rate; with four epilogue warps and
+// one CTA per tile, whose load, products and stores followed one another, 0.69 (gated, 32 heads of 4096: 0.150 and another
+// 0.040 for dλ, now 0.099 with dλ).
 // ---------------------------------------------------------------------------------------------------------------
-constexpr int FUSED_SMEM = 14 * BOX_BYTES + 1024 + 256 + TILE * 4;   // tiles, alignment, barriers, the tile's λ (gated)
+constexpr int FUSED_EPI_WARPS = 16;
+constexpr int FUSED_THREADS = 32 * (FUSED_EPI_WARPS + 2);
+constexpr int FUSED_SMEM = 14 * BOX_BYTES + 1024 + 256;   // tiles, alignment, barriers
 
 struct FusedParams {
   int64_t T;
   int NC;
+  uint32_t tiles;                    // heads * NC
   int64_t n;                         // rows t >= n add lr_q to dQ; rows t < n add lr_k, lr_v to dK, dV (when non-null)
   const __nv_bfloat16 *lr_q, *lr_k, *lr_v;   // [bh][T][128] bf16
   const float* lam;                  // GATED: inclusive prefix sums of the log-gates [bh][T]
+  float* dlam;                       // GATED: [bh][T] q_t·dQ_t - k_t·dK_t, from the sums before they are rounded
   __nv_bfloat16 *dQ, *dK, *dV;       // [bh][T][128]
   int* status;
 };
+
+__device__ __forceinline__ bool elect_one() {
+  uint32_t pred;
+  asm volatile(
+      "{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(pred));
+  return pred != 0;
+}
 
 // GATED (Lemma "Gated SMat", adjoint side): both score tiles are multiplied by exp(λ_i - λ_j) as they are rounded, and
 // the three state products are scaled row by row in tensor memory before the score products are added to them — row i
 // of dO S_inᵀ by exp(λ_i - λ_{last token before the tile}), row j of V D̄ᵀ and of K D̄ by exp(λ_{last token of the
 // tile} - λ_j).  S_in and D̄ are the decayed per-tile states.
 template <bool GATED>
-__global__ void __launch_bounds__(160) bwd_tile_fused_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
+__global__ void __launch_bounds__(FUSED_THREADS, 1) bwd_tile_fused_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
                                                                 const __grid_constant__ CUtensorMap tmK,
                                                                 const __grid_constant__ CUtensorMap tmV,
                                                                 const __grid_constant__ CUtensorMap tmG,
                                                                 const __grid_constant__ CUtensorMap tmSin,
                                                                 const __grid_constant__ CUtensorMap tmDb,
-                                                                const FusedParams prm) {
+                                                                const __grid_constant__ FusedParams prm) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* sQ = smem;
   uint8_t* sK = smem + 2 * BOX_BYTES;
   uint8_t* sV = smem + 4 * BOX_BYTES;
   uint8_t* sG = smem + 6 * BOX_BYTES;      // dO
-  uint8_t* sS = smem + 8 * BOX_BYTES;      // S_in of the tile
+  uint8_t* sS = smem + 8 * BOX_BYTES;      // S_in of the tile, then the masked, rounded A
   uint8_t* sD = smem + 10 * BOX_BYTES;     // D̄ of the tile
-  uint8_t* sX = smem + 12 * BOX_BYTES;     // masked, rounded score tile (G, then A)
+  uint8_t* sX = smem + 12 * BOX_BYTES;     // masked, rounded G
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 14 * BOX_BYTES);
-  uint64_t* bar_in0 = bars + 0;   // dO, V landed
-  uint64_t* bar_in1 = bars + 1;   // Q, K, S_in, D̄ landed
-  uint64_t* bar_sc = bars + 2;    // a score tile is in tensor memory (two phases: G, then A)
-  uint64_t* bar_p = bars + 3;     // X written (one arrival per warp; two phases)
-  uint64_t* bar_x = bars + 4;     // the MMAs that read X = G have finished: dQ, dK complete, X may be overwritten
-  uint64_t* bar_o = bars + 5;     // dV complete
-  uint64_t* bar_st = bars + 6;    // GATED: the three state products are in tensor memory
-  uint64_t* bar_sl = bars + 7;    // GATED: ... and scaled (one arrival per warp)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 8);
+  // every barrier completes once per tile
+  uint64_t *f_qk = bars + 0, *f_v = bars + 1, *f_g = bars + 2, *f_d = bars + 3, *f_s = bars + 4;   // operands landed
+  uint64_t *e_v = bars + 5, *e_d = bars + 6, *e_qk = bars + 7, *e_gs = bars + 8;                   // ... and consumed
+  uint64_t* b_sca = bars + 9;     // A scores in tensor memory
+  uint64_t* b_scg = bars + 10;    // G scores in tensor memory
+  uint64_t* b_st = bars + 11;     // dO S_inᵀ, V D̄ᵀ formed
+  uint64_t* b_st2 = bars + 12;    // GATED: K D̄ formed
+  uint64_t* b_qk = bars + 13;     // dQ, dK complete
+  uint64_t* b_dv = bars + 14;     // dV complete
+  // one arrival per epilogue warp:
+  uint64_t* p_g = bars + 15;      // rounded G written, its scores read out
+  uint64_t* p_a = bars + 16;      // rounded A written, its scores read out
+  uint64_t* o_qk = bars + 17;     // dQ, dK read out (GATED: and this tile's Q, K)
+  uint64_t* o_v = bars + 18;      // dV read out
+  uint64_t* sl_qk = bars + 19;    // GATED: dO S_inᵀ, V D̄ᵀ scaled
+  uint64_t* sl_v = bars + 20;     // GATED: K D̄ scaled
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 21);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float* sLam = reinterpret_cast<float*>(smem + 14 * BOX_BYTES + 256);   // [128] λ of the tile's tokens (GATED)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = blockIdx.x, bh = blockIdx.y;
-  const int64_t row0 = (int64_t)bh * prm.T + (int64_t)b * TILE;
   const WaitCtx wc{cta_abort, prm.status};
   if (threadIdx.x == 0) {
     *cta_abort = 0;
-    mbar_init(bar_in0, 1); mbar_init(bar_in1, 1); mbar_init(bar_sc, 1); mbar_init(bar_p, 4); mbar_init(bar_x, 1);
-    mbar_init(bar_o, 1); mbar_init(bar_st, 1); mbar_init(bar_sl, 4);
+    for (int i = 0; i < 15; ++i) mbar_init(bars + i, 1);
+    for (int i = 15; i < 21; ++i) mbar_init(bars + i, FUSED_EPI_WARPS);
     fence_barrier_init();
   }
-  if (warp == 4) tmem_alloc(tmem_slot, 512);
+  if (warp == FUSED_EPI_WARPS) tmem_alloc(tmem_slot, 512);
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
   pdl_trigger();
   pdl_wait();
   const uint32_t tmem_base = *tmem_slot;
-  if (GATED) {
-    if (threadIdx.x < TILE) sLam[threadIdx.x] = prm.lam[row0 + threadIdx.x];
-    __syncthreads();
-  }
-  const uint32_t tm_sc = tmem_base, tm_dq = tmem_base + TILE, tm_dk = tmem_base + 2 * TILE, tm_dv = tmem_base + 3 * TILE;
+  const uint32_t tm_g = tmem_base, tm_dq = tmem_base + TILE, tm_dk = tmem_base + 2 * TILE, tm_a = tmem_base + 3 * TILE;
+  const uint32_t tm_dv = tm_g;
 
-  if (warp == 4 && lane == 0) {
-    auto load_tile = [&](uint8_t* dst, const CUtensorMap* map, int row, uint64_t* bar) {
+  if (warp == FUSED_EPI_WARPS) {
+    const bool leader = elect_one();
+    uint32_t prev = 1;                         // parity of the tile before: a fresh barrier lets the first tile through
+    bool ok = true;
+    auto wait = [&](uint64_t* bar) { ok = ok && __all_sync(0xffffffffu, mbar_wait(bar, prev, wc)); return ok; };
+    auto load = [&](uint8_t* dst, const CUtensorMap* map, int row, uint64_t* bar) {
       tma_load_2d(dst, map, 0, row, bar);
       tma_load_2d(dst + BOX_BYTES, map, HALF, row, bar);
     };
-    mbar_expect_tx(bar_in0, 4 * BOX_BYTES);
-    load_tile(sG, &tmG, (int)row0, bar_in0);
-    load_tile(sV, &tmV, (int)row0, bar_in0);
-    mbar_expect_tx(bar_in1, 8 * BOX_BYTES);
-    load_tile(sQ, &tmQ, (int)row0, bar_in1);
-    load_tile(sK, &tmK, (int)row0, bar_in1);
-    const int srow = (int)(((int64_t)bh * prm.NC + b) * TILE);
-    load_tile(sS, &tmSin, srow, bar_in1);
-    load_tile(sD, &tmDb, srow, bar_in1);
-
+    for (uint32_t tile = blockIdx.x; tile < prm.tiles && ok; tile += gridDim.x, prev ^= 1) {
+      const int row = (int)(tile * TILE);      // tokens and states alike: both are [heads][tiles][128 rows]
+      if (!wait(e_v)) break;
+      if (leader) { mbar_expect_tx(f_v, 2 * BOX_BYTES); load(sV, &tmV, row, f_v); }
+      if (!wait(e_d)) break;
+      if (leader) { mbar_expect_tx(f_d, 2 * BOX_BYTES); load(sD, &tmDb, row, f_d); }
+      if (!wait(e_qk) || (GATED && !wait(o_qk))) break;
+      if (leader) { mbar_expect_tx(f_qk, 4 * BOX_BYTES); load(sQ, &tmQ, row, f_qk); load(sK, &tmK, row, f_qk); }
+      if (!wait(e_gs)) break;
+      if (leader) {
+        mbar_expect_tx(f_g, 2 * BOX_BYTES); load(sG, &tmG, row, f_g);
+        mbar_expect_tx(f_s, 2 * BOX_BYTES); load(sS, &tmSin, row, f_s);
+      }
+    }
+  } else if (warp == FUSED_EPI_WARPS + 1) {
+    const bool leader = elect_one();
     constexpr uint32_t id_kk = make_idesc(TILE, TILE, 0, 0);   // A K-major, B K-major
     constexpr uint32_t id_km = make_idesc(TILE, TILE, 0, 1);   // A K-major, B MN-major
     constexpr uint32_t id_mm = make_idesc(TILE, TILE, 1, 1);   // A MN-major, B MN-major
     // K-major view of a [128 rows][128 k] tile (two 64-wide k blocks 16 KB apart), K-step kk; MN-major view of a
     // [128 k rows][128 n] tile (16 rows = 2048 bytes per K-step, the two 64-wide n blocks 16 KB apart)
-    auto kmaj = [](const uint8_t* t, int kk) { return make_desc(smem_u32(t) + (kk >> 2) * BOX_BYTES + (kk & 3) * 32, 16, 1024); };
-    auto mnmaj = [](const uint8_t* t, int kk) { return make_desc(smem_u32(t) + kk * 2048, BOX_BYTES, 1024); };
-    bool ok = mbar_wait(bar_in0, 0, wc);
-    if (ok) {
+    constexpr uint32_t BOX16 = BOX_BYTES >> 4;
+    auto kmaj = [](const uint8_t* t) { return make_desc(smem_u32(t), 16, 1024); };
+    auto mnmaj = [](const uint8_t* t) { return make_desc(smem_u32(t), BOX_BYTES, 1024); };
+    const uint64_t q_k = kmaj(sQ), k_k = kmaj(sK), v_k = kmaj(sV), g_k = kmaj(sG), s_k = kmaj(sS), d_k = kmaj(sD), x_k = kmaj(sX);
+    const uint64_t q_m = mnmaj(sQ), k_m = mnmaj(sK), g_m = mnmaj(sG), s_m = mnmaj(sS), d_m = mnmaj(sD), x_m = mnmaj(sX);
+    auto koff = [](int kk) { return (uint64_t)((kk >> 2) * BOX16 + (kk & 3) * 2); };
+    auto moff = [](int kk) { return (uint64_t)(kk * 128); };
+    uint32_t par = 0;
+    bool ok = true;
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      ok = ok && __all_sync(0xffffffffu, mbar_wait(bar, parity, wc));
       fence_after_sync();
+      return ok;
+    };
+    for (uint32_t tile = blockIdx.x; tile < prm.tiles && ok; tile += gridDim.x, par ^= 1) {
+      if (!wait(f_qk, par)) break;             // (the A scores of the tile before were read out before its last product)
+      if (leader) {
 #pragma unroll
-      for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_sc, kmaj(sG, kk), kmaj(sV, kk), id_kk, kk != 0);   // dO Vᵀ
-      mma_commit(bar_sc);
-      ok = mbar_wait(bar_in1, 0, wc);
+        for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_a, q_k + koff(kk), k_k + koff(kk), id_kk, kk != 0);      // Q Kᵀ
+        mma_commit(b_sca);
+      }
+      if (!wait(f_v, par) || !wait(f_g, par) || !wait(o_v, par ^ 1)) break;
+      if (leader) {
+#pragma unroll
+        for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_g, g_k + koff(kk), v_k + koff(kk), id_kk, kk != 0);      // dO Vᵀ
+        mma_commit(b_scg);
+      }
+      if (!wait(f_s, par) || !wait(f_d, par) || !wait(o_qk, par ^ 1)) break;
+      if (leader) {
+#pragma unroll
+        for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_dq, g_k + koff(kk), s_k + koff(kk), id_kk, kk != 0);     // dO S_inᵀ
+#pragma unroll
+        for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_dk, v_k + koff(kk), d_k + koff(kk), id_kk, kk != 0);     // V D̄ᵀ
+        mma_commit(b_st);
+        mma_commit(e_v);
+      }
+      if (!wait(p_g, par)) break;              // rounded G in shared memory; its scores have left tensor memory
+      if (leader) {
+#pragma unroll
+        for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_dv, k_k + koff(kk), d_m + moff(kk), id_km, kk != 0);     // K D̄
+        mma_commit(e_d);
+        if (GATED) mma_commit(b_st2);
+      }
+      if (GATED && !wait(sl_qk, par)) break;   // the state products carry their row factors
+      if (leader) {
+#pragma unroll
+        for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_dq, x_k + koff(kk), k_m + moff(kk), id_km, 1);           // G K
+#pragma unroll
+        for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_dk, x_m + moff(kk), q_m + moff(kk), id_mm, 1);           // Gᵀ Q
+        mma_commit(b_qk);
+        mma_commit(e_qk);
+      }
+      if (!wait(p_a, par) || (GATED && !wait(sl_v, par))) break;
+      if (leader) {
+#pragma unroll
+        for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_dv, s_m + moff(kk), g_m + moff(kk), id_mm, 1);           // Aᵀ dO
+        mma_commit(b_dv);
+        mma_commit(e_gs);
+      }
     }
-    if (ok) {
-      fence_after_sync();
-#pragma unroll
-      for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_dq, kmaj(sG, kk), kmaj(sS, kk), id_kk, kk != 0);   // dO S_inᵀ
-#pragma unroll
-      for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_dk, kmaj(sV, kk), kmaj(sD, kk), id_kk, kk != 0);   // V D̄ᵀ
-#pragma unroll
-      for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_dv, kmaj(sK, kk), mnmaj(sD, kk), id_km, kk != 0);  // K D̄
-      if (GATED) mma_commit(bar_st);
-      ok = mbar_wait(bar_p, 0, wc);          // X = G in shared memory; the G scores have left tensor memory
-      if (GATED && ok) ok = mbar_wait(bar_sl, 0, wc);   // the state products carry their row factors
-    }
-    if (ok) {
-      fence_after_sync();
-#pragma unroll
-      for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_dq, kmaj(sX, kk), mnmaj(sK, kk), id_km, 1);        // G K
-#pragma unroll
-      for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_dk, mnmaj(sX, kk), mnmaj(sQ, kk), id_mm, 1);       // Gᵀ Q
-      mma_commit(bar_x);
-#pragma unroll
-      for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_sc, kmaj(sQ, kk), kmaj(sK, kk), id_kk, kk != 0);   // Q Kᵀ
-      mma_commit(bar_sc);
-      ok = mbar_wait(bar_p, 1, wc);          // X = A
-    }
-    if (ok) {
-      fence_after_sync();
-#pragma unroll
-      for (int kk = 0; kk < TILE / 16; ++kk) mma_bf16(tm_dv, mnmaj(sX, kk), mnmaj(sG, kk), id_mm, 1);       // Aᵀ dO
-      mma_commit(bar_o);
-    }
-  } else if (warp < 4) {
-    const int m = warp * 32 + lane;  // row inside the tile = TMEM lane
-    const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-    const float lam_m = GATED ? sLam[m] : 0.f;
-    // masked (column <= row), rounded copy of the score tile into X, swizzled as a K-major operand
-    auto stage_scores = [&]() {
-#pragma unroll
-      for (int cb = 0; cb < 4; ++cb) {
+  } else {
+    const int cq = warp >> 2;                        // column quarter
+    const int m = (warp & 3) * 32 + lane;            // row inside the tile = TMEM lane
+    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+    const uint32_t col0 = cq * 32;
+    // this thread's 64 bytes (four 16-byte chunks) of its row in the 64-column block that holds its columns
+    const uint32_t my_off = (cq >> 1) * BOX_BYTES + m * 128;
+    const int ch0 = (cq & 1) * 4;
+    uint32_t par = 0;
+    auto arrive = [&](uint64_t* bar) {
+      fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar);
+    };
+    for (uint32_t tile = blockIdx.x; tile < prm.tiles; tile += gridDim.x, par ^= 1) {
+      const int64_t row = (int64_t)tile * TILE + m;                                   // [bh][T] row
+      const int64_t bh = tile / (uint32_t)prm.NC, t = row - bh * prm.T;
+      float lam_m = 0.f, lam_c = 0.f, row_in = 1.f, row_out = 1.f;                    // lam_c: of column col0 + lane
+      if (GATED) {
+        const float* l = prm.lam + (int64_t)tile * TILE;
+        lam_m = l[m];
+        lam_c = l[col0 + lane];
+        row_in = __expf(lam_m - (t >= TILE ? l[-1] : 0.f));                           // queries' side: from the tile's start
+        row_out = __expf(l[TILE - 1] - lam_m);                                        // keys' side: to the tile's end
+      }
+      // masked (column <= row), rounded copy of this thread's part of a score tile, swizzled as a K-major operand
+      auto round_scores = [&](uint32_t tm_sc, uint4 (&pk)[4]) {
         uint32_t v[32];
-        tmem_ld32(tm_sc + lane_base + cb * 32, v);
+        tmem_ld32(tm_sc + lane_base + col0, v);
         tmem_ld_wait();
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          uint32_t pk[4];
+          uint32_t w[4];
 #pragma unroll
           for (int h2 = 0; h2 < 4; ++h2) {
-            const int k0 = cb * 32 + i * 8 + h2 * 2;
-            float lo = (k0 <= m) ? __uint_as_float(v[i * 8 + h2 * 2]) : 0.f;
-            float hi = (k0 + 1 <= m) ? __uint_as_float(v[i * 8 + h2 * 2 + 1]) : 0.f;
+            const int e = i * 8 + h2 * 2, k0 = (int)col0 + e;
+            float lo = (k0 <= m) ? __uint_as_float(v[e]) : 0.f;
+            float hi = (k0 + 1 <= m) ? __uint_as_float(v[e + 1]) : 0.f;
             if (GATED) {   // exponents of non-positive differences only
-              if (k0 <= m) lo *= __expf(lam_m - sLam[k0]);
-              if (k0 + 1 <= m) hi *= __expf(lam_m - sLam[k0 + 1]);
+              const float l0 = __shfl_sync(0xffffffffu, lam_c, e), l1 = __shfl_sync(0xffffffffu, lam_c, e + 1);
+              if (k0 <= m) lo *= __expf(lam_m - l0);
+              if (k0 + 1 <= m) hi *= __expf(lam_m - l1);
             }
-            pk[h2] = pack_bf16(lo, hi);
+            w[h2] = pack_bf16(lo, hi);
           }
-          const int j8 = cb * 4 + i;
-          uint8_t* dst = sX + (j8 >> 3) * BOX_BYTES + m * 128 + (((j8 & 7) ^ (m & 7)) << 4);
-          *reinterpret_cast<uint4*>(dst) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+          pk[i] = make_uint4(w[0], w[1], w[2], w[3]);
         }
-      }
-      fence_proxy_async();
-      fence_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar_p);
-    };
-    // one accumulator row (128 columns) plus its long-range row, rounded and stored
-    const int64_t t = (int64_t)b * TILE + m;
-    auto store_row = [&](uint32_t tm_acc, const __nv_bfloat16* lr, bool add, __nv_bfloat16* out) {
-      const uint4* y16 = reinterpret_cast<const uint4*>(lr + ((int64_t)bh * prm.T + t) * TILE);
-      __nv_bfloat16* dst = out + ((int64_t)bh * prm.T + t) * TILE;
+      };
+      auto store_scores = [&](uint8_t* dst, const uint4 (&pk)[4], uint64_t* bar) {
 #pragma unroll
-      for (int cb = 0; cb < 4; ++cb) {
+        for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(dst + my_off + (((ch0 + c) ^ (m & 7)) << 4)) = pk[c];
+        fence_proxy_async();
+        arrive(bar);
+      };
+      // GATED: this thread's part of an accumulator times its row's factor, in place
+      auto scale = [&](uint32_t tm_acc, float f) {
         uint32_t v[32];
-        tmem_ld32(tm_acc + lane_base + cb * 32, v);
+        tmem_ld32(tm_acc + lane_base + col0, v);
         tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * f);
+        tmem_st32(tm_acc + lane_base + col0, v);
+      };
+      // long-range rows of this thread's columns, fetched while the MMAs run
+      auto fetch = [&](const __nv_bfloat16* lr, uint4 (&y)[4]) {
+        const uint4* y4 = reinterpret_cast<const uint4*>(lr + row * TILE + col0);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) y[i] = y4[i];
+      };
+      // accumulator part (in v) plus long-range part, rounded and stored; GATED: its product with the same part of this
+      // row of the operand tile `with` (null: none)
+      auto finish = [&](const uint32_t (&v)[32], const uint4 (&y)[4], bool add, __nv_bfloat16* out, const uint8_t* with) {
+        float dot = 0.f;
         uint32_t w[16];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -584,72 +662,91 @@ __global__ void __launch_bounds__(160) bwd_tile_fused_tc_kernel(const __grid_con
 #pragma unroll
           for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[i * 8 + e]);
           if (add) {
-            const uint4 a = *(y16 + cb * 4 + i);
-            const uint32_t yy[4] = {a.x, a.y, a.z, a.w};
+            const uint32_t yy[4] = {y[i].x, y[i].y, y[i].z, y[i].w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               f[2 * e] += __uint_as_float(yy[e] << 16);
               f[2 * e + 1] += __uint_as_float(yy[e] & 0xffff0000u);
             }
           }
+          if (GATED && with) {
+            const uint4 a = *reinterpret_cast<const uint4*>(with + my_off + (((ch0 + i) ^ (m & 7)) << 4));
+            const uint32_t xx[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              dot = fmaf(f[2 * e], __uint_as_float(xx[e] << 16), dot);
+              dot = fmaf(f[2 * e + 1], __uint_as_float(xx[e] & 0xffff0000u), dot);
+            }
+          }
           w[4 * i] = pack_bf16(f[0], f[1]); w[4 * i + 1] = pack_bf16(f[2], f[3]);
           w[4 * i + 2] = pack_bf16(f[4], f[5]); w[4 * i + 3] = pack_bf16(f[6], f[7]);
         }
+        __nv_bfloat16* dst = out + row * TILE + col0;
 #pragma unroll
-        for (int h8 = 0; h8 < 2; ++h8)
-          st_global_v8(dst + cb * 32 + 16 * h8, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
+        for (int h8 = 0; h8 < 2; ++h8)   // whole 32-byte sectors
+          st_global_v8(dst + 16 * h8, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
                        w[8 * h8 + 5], w[8 * h8 + 6], w[8 * h8 + 7]);
-      }
-    };
-    // GATED: one accumulator's rows times this row's factor, in place
-    auto scale_rows = [&](uint32_t tm_acc, float f) {
-#pragma unroll
-      for (int cb = 0; cb < 4; ++cb) {
-        uint32_t v[32];
-        tmem_ld32(tm_acc + lane_base + cb * 32, v);
-        tmem_ld_wait();
-#pragma unroll
-        for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * f);
-        tmem_st32(tm_acc + lane_base + cb * 32, v);
-      }
-    };
-    bool ok = mbar_wait(bar_sc, 0, wc);
-    if (ok) {
+        return dot;
+      };
+      // a tile lies on one side of the block boundary
+      const bool add_q = prm.lr_q != nullptr && t >= prm.n, add_kv = prm.lr_k != nullptr && t < prm.n;
+      uint4 y[4], pk[4];
+      if (!mbar_wait(b_scg, par, wc)) break;
       fence_after_sync();
-      stage_scores();                              // X = G
+      round_scores(tm_g, pk);
+      store_scores(sX, pk, p_g);
+      if (!mbar_wait(b_sca, par, wc)) break;
+      fence_after_sync();
+      round_scores(tm_a, pk);
+      if (add_q) fetch(prm.lr_q, y);
+      if (add_kv) fetch(prm.lr_k, y);
+      if (!mbar_wait(b_st, par, wc)) break;          // S_in has been read: the rounded A takes its place
+      fence_after_sync();
       if (GATED) {
-        ok = mbar_wait(bar_st, 0, wc);
-        if (ok) {
-          fence_after_sync();
-          const float row_in = __expf(lam_m - (b > 0 ? prm.lam[row0 - 1] : 0.f));   // queries' side: from the tile's start
-          const float row_out = __expf(sLam[TILE - 1] - lam_m);                       // keys' side: to the tile's end
-          scale_rows(tm_dq, row_in);
-          scale_rows(tm_dk, row_out);
-          scale_rows(tm_dv, row_out);
-          tmem_st_wait();
-          fence_before_sync();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar_sl);
+        scale(tm_dq, row_in);
+        scale(tm_dk, row_out);
+        tmem_st_wait();
+        arrive(sl_qk);
+      }
+      store_scores(sS, pk, p_a);
+      if (GATED) {
+        if (!mbar_wait(b_st2, par, wc)) break;
+        fence_after_sync();
+        scale(tm_dv, row_out);
+        tmem_st_wait();
+        arrive(sl_v);
+      }
+      if (!mbar_wait(b_qk, par, wc)) break;
+      fence_after_sync();
+      uint32_t v[32];
+      tmem_ld32(tm_dq + lane_base + col0, v);
+      tmem_ld_wait();
+      const float dq = finish(v, y, add_q, prm.dQ, sQ);
+      tmem_ld32(tm_dk + lane_base + col0, v);
+      tmem_ld_wait();
+      if (!GATED) arrive(o_qk);
+      const float dk = finish(v, y, add_kv, prm.dK, sK);
+      if (GATED) {   // the column quarters of dλ meet in the tile that held G (its products are done)
+        float* part = reinterpret_cast<float*>(sX);
+        part[cq * TILE + m] = dq - dk;
+        arrive(o_qk);
+        if (cq == 0) {                               // (the next G is written after these warps' arrival on o_v)
+          if (!mbar_wait(o_qk, par, wc)) break;
+          prm.dlam[row] = (part[m] + part[TILE + m]) + (part[2 * TILE + m] + part[3 * TILE + m]);
         }
       }
-      if (ok) ok = mbar_wait(bar_sc, 1, wc);       // the A scores are in (the MMAs on G were issued before them)
-    }
-    if (ok) ok = mbar_wait(bar_x, 0, wc);          // ... and those MMAs have finished with X: dQ, dK are complete
-    if (ok) {
+      if (add_kv) fetch(prm.lr_v, y);
+      if (!mbar_wait(b_dv, par, wc)) break;
       fence_after_sync();
-      stage_scores();                              // X = A
-      store_row(tm_dq, prm.lr_q, prm.lr_q != nullptr && t >= prm.n, prm.dQ);
-      store_row(tm_dk, prm.lr_k, prm.lr_k != nullptr && t < prm.n, prm.dK);
-      ok = mbar_wait(bar_o, 0, wc);
-    }
-    if (ok) {
-      fence_after_sync();
-      store_row(tm_dv, prm.lr_v, prm.lr_v != nullptr && t < prm.n, prm.dV);
+      tmem_ld32(tm_dv + lane_base + col0, v);
+      tmem_ld_wait();
+      arrive(o_v);
+      finish(v, y, add_kv, prm.dV, nullptr);
     }
   }
   fence_before_sync();
   __syncthreads();
-  if (warp == 4) {
+  if (warp == FUSED_EPI_WARPS) {
     fence_after_sync();
     tmem_dealloc(tmem_base, 512);
   }
@@ -1683,7 +1780,7 @@ cudaError_t smat_launch_chunk_adjoint_tc(int which, const void* Q, const void* K
 cudaError_t smat_launch_bwd_tiles_fused_tc(const void* Q, const void* K, const void* V, const void* dO,
                                            const void* Sin_bf16, const void* Dbar_bf16, const void* lr_q, const void* lr_k,
                                            const void* lr_v, int64_t n, void* dQ, void* dK, void* dV, int64_t T, int bh,
-                                           int* status, cudaStream_t st, const float* lam) {
+                                           int* status, cudaStream_t st, const float* lam, float* dlam) {
   CUtensorMap tmQ, tmK, tmV, tmG, tmS, tmD;
   const int NC = (int)(T / TILE);
   if (!make_map(&tmQ, Q, (uint64_t)bh * T) || !make_map(&tmK, K, (uint64_t)bh * T) || !make_map(&tmV, V, (uint64_t)bh * T) ||
@@ -1691,18 +1788,21 @@ cudaError_t smat_launch_bwd_tiles_fused_tc(const void* Q, const void* K, const v
       !make_map(&tmD, Dbar_bf16, (uint64_t)bh * NC * TILE))
     return cudaErrorInvalidValue;
   FusedParams prm;
-  prm.T = T; prm.NC = NC; prm.n = n;
+  prm.T = T; prm.NC = NC; prm.n = n; prm.tiles = (uint32_t)bh * (uint32_t)NC;
   prm.lr_q = static_cast<const __nv_bfloat16*>(lr_q);
   prm.lr_k = static_cast<const __nv_bfloat16*>(lr_k);
   prm.lr_v = static_cast<const __nv_bfloat16*>(lr_v);
   prm.dQ = static_cast<__nv_bfloat16*>(dQ); prm.dK = static_cast<__nv_bfloat16*>(dK); prm.dV = static_cast<__nv_bfloat16*>(dV);
   prm.status = status;
-  prm.lam = lam;
+  prm.lam = lam; prm.dlam = dlam;
   auto kernel = lam ? bwd_tile_fused_tc_kernel<true> : bwd_tile_fused_tc_kernel<false>;
   cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSED_SMEM);
   if (err != cudaSuccess) return err;
-  dim3 grid((unsigned)NC, (unsigned)bh);
-  return smat_launch_pdl(kernel, grid, 160, FUSED_SMEM, st, tmQ, tmK, tmV, tmG, tmS, tmD, prm);
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const unsigned grid = prm.tiles < (uint32_t)sms ? prm.tiles : (unsigned)sms;
+  return smat_launch_pdl(kernel, dim3(grid), FUSED_THREADS, FUSED_SMEM, st, tmQ, tmK, tmV, tmG, tmS, tmD, prm);
 }
 
 // Both adjoint reads of the profile states in one launch: out_t[t] = St x_t (rows Xt, the second state index
