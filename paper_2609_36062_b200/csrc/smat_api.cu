@@ -310,6 +310,11 @@ bool device_ok() {
 void tabulate(Ctx& cx, const char* name, const float* in, float* out, int transpose, int out_bf16 = 0) {
   const smat_plan* pl = cx.pl;
   if (in == out) return;  // d = 2: hyperplanes are single points, the type table is the profile table
+  if (!(pl->flags & SMAT_FLAG_ALG2_TABULATION) && !transpose && !out_bf16 && smat_tabulate_d3_f32_supported(pl->geo, pl->rp)) {
+    SMAT_TRY(cx, name, smat_launch_tabulate_d3_f32(in, out, pl->geo, pl->rp, pl->bh,
+                                                   reinterpret_cast<int*>(cx.ws + pl->off_status), cx.st));
+    return;
+  }
   if (!(pl->flags & SMAT_FLAG_ALG2_TABULATION) && smat_tabulate_staged_slab(pl->geo, pl->rp, transpose) >= 4)
     SMAT_TRY(cx, name, smat_launch_tabulate_staged(in, out, pl->geo, pl->rp, pl->bh, transpose, out_bf16, cx.st));
   else

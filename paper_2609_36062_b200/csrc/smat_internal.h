@@ -134,6 +134,11 @@ struct SmatReadArgs {
 cudaError_t smat_launch_state_read(const SmatReadArgs& a, int bf16, int64_t Tlen, int bh, int r, int p, int* status,
                                    cudaStream_t st);
 
+// The d = 3 tabulation of fp32 tables with the sums in registers (the primes it is instantiated for).
+int smat_tabulate_d3_f32_supported(const SmatGeo& geo, int64_t state_elems);
+cudaError_t smat_launch_tabulate_d3_f32(const float* in, float* out, const SmatGeo& geo, int64_t state_elems, int bh,
+                                        int* status, cudaStream_t st);
+
 // Staged exact tabulation (same sums as Algorithm 2, one coordinate at a time). Slab = 0: not available.
 int smat_tabulate_staged_slab(const SmatGeo& geo, int64_t state_elems, int transpose);
 // out_bf16 = 1 writes the result table as bf16 (same layout, half the bytes) instead of fp32.

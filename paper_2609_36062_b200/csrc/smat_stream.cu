@@ -132,10 +132,16 @@ __global__ void __launch_bounds__(256) pool_stream_kernel(const __grid_constant_
     const int kn = cur.tokens();
     const T* as = a_raw + buf * TK * R;
     const T* bs = b_raw + buf * TK * PD;
+    // a thread owns NS neighbouring rows, so that their factors come four to a load (one by one they took as many
+    // shared-memory cycles as everything else: 32 heads, 289 states of 9 tokens, 0.138 ms against 0.122)
     for (int k = 0; k < kn; ++k) {
       const float4 b4 = load4(bs + k * PD + j4 * 4);
 #pragma unroll
-      for (int s = 0; s < NS; ++s) acc[s] = fma4(to_float(as[k * R + ig + s * NG]), b4, acc[s]);
+      for (int s = 0; s < NS; s += 4) {
+        const float4 a4 = load4(as + k * R + ig * NS + s);
+        acc[s] = fma4(a4.x, b4, acc[s]); acc[s + 1] = fma4(a4.y, b4, acc[s + 1]);
+        acc[s + 2] = fma4(a4.z, b4, acc[s + 2]); acc[s + 3] = fma4(a4.w, b4, acc[s + 3]);
+      }
     }
     if (cur.last()) {
       // the previous item's bulk store reads the same buffer: it must have finished reading (the other CTA
@@ -143,7 +149,7 @@ __global__ void __launch_bounds__(256) pool_stream_kernel(const __grid_constant_
       if (tid == 0) bulk_store_wait_read<0>();
       __syncthreads();
 #pragma unroll
-      for (int s = 0; s < NS; ++s) *reinterpret_cast<float4*>(outb + (ig + s * NG) * PD + j4 * 4) = acc[s];
+      for (int s = 0; s < NS; ++s) *reinterpret_cast<float4*>(outb + (ig * NS + s) * PD + j4 * 4) = acc[s];
       tc::fence_proxy_async();
       __syncthreads();
       if (tid == 0) bulk_store(list.a.job[cur.job].state + (cur.item - list.first[cur.job]) * (int64_t)(R * PD), outb, R * PD * 4);
@@ -262,22 +268,30 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
         float4 acc[KT];
 #pragma unroll
         for (int k = 0; k < KT; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-        for (int s = 0; s < RPG; ++s) {
+        // four rows at a time, so that a token's factors are one load (32 heads, 307 states, bf16: 0.185 -> 0.177 ms)
+#pragma unroll 2
+        for (int s = 0; s < RPG; s += 4) {
           const int i = ig * RPG + s;
-          const float4 u = S4[i * NJ4 + j4];
+          const float4 u0 = S4[i * NJ4 + j4], u1 = S4[(i + 1) * NJ4 + j4], u2 = S4[(i + 2) * NJ4 + j4], u3 = S4[(i + 3) * NJ4 + j4];
 #pragma unroll
-          for (int k = 0; k < KT; ++k) acc[k] = fma4(Xs[k * L::XM + i], u, acc[k]);
+          for (int k = 0; k < KT; ++k) {
+            const float4 x = *reinterpret_cast<const float4*>(Xs + k * L::XM + i);
+            acc[k] = fma4(x.x, u0, acc[k]); acc[k] = fma4(x.y, u1, acc[k]);
+            acc[k] = fma4(x.z, u2, acc[k]); acc[k] = fma4(x.w, u3, acc[k]);
+          }
         }
 #pragma unroll
         for (int k = 0; k < KT; ++k) *reinterpret_cast<float4*>(red + (ig * KT + k) * PD + j4 * 4) = acc[k];
         __syncthreads();
-        for (int idx = tid; idx < kn * PD; idx += 256) {
-          const int k = idx / PD, jj = idx % PD;
-          float v = 0.f;
+        for (int idx = tid; idx < kn * NJ4; idx += 256) {   // the row groups' partial rows meet in shared memory
+          const int k = idx / NJ4, c = idx - k * NJ4;
+          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-          for (int w = 0; w < NG; ++w) v += red[(w * KT + k) * PD + jj];
-          out[tk.at(k0 + k) * PD + jj] = v;
+          for (int w = 0; w < NG; ++w) {
+            const float4 p = *reinterpret_cast<const float4*>(red + (w * KT + k) * PD + c * 4);
+            v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
+          }
+          *reinterpret_cast<float4*>(out + tk.at(k0 + k) * PD + c * 4) = v;
         }
       } else {
 #pragma unroll 2
