@@ -134,6 +134,11 @@ struct SmatReadArgs {
 cudaError_t smat_launch_state_read(const SmatReadArgs& a, int bf16, int64_t Tlen, int bh, int r, int p, int* status,
                                    cudaStream_t st);
 
+// Both stages of the d = 4 tabulation with the table between them in shared memory (the primes for which it fits).
+int smat_tabulate_slab_supported(int q, int64_t state_elems);
+cudaError_t smat_launch_tabulate_slab(const void* in, void* out, const SmatGeo& geo, int64_t state_elems, int bh, int* status,
+                                      cudaStream_t st);
+
 // The d = 3 tabulation of fp32 tables with the sums in registers (the primes it is instantiated for).
 int smat_tabulate_d3_f32_supported(const SmatGeo& geo, int64_t state_elems);
 cudaError_t smat_launch_tabulate_d3_f32(const float* in, float* out, const SmatGeo& geo, int64_t state_elems, int bh,

@@ -29,7 +29,7 @@
 //   warps 19, 20   : q = 11 only.  q^2 + q = 132 output indices are one tile of 128 and 4 left over, all of the extra
 //                    class (the sum of one line's q rows): these warps add them up from the ring slot itself, so
 //                    that one CTA covers an image instead of two CTAs loading it twice
-// d = 4 with q <= 11: both stages in ONE launch, slab by slab.  Stage 2 of a slab needs stage 1 of every image of the
+// d = 4 with q <= 11 (forward with q = 11: smat_radon_slab.cu instead): both stages in ONE launch, slab by slab.  Stage 2 of a slab needs stage 1 of every image of the
 // same slab and nothing else, so a CTA keeps the slab's W rows in a private exchange buffer (q^3 + q^2 rows of 128
 // entries, rewritten for every slab, stored and loaded with the L2 evict-last priority while F and U stream with
 // evict-first) and the full-size W table is never built.  The storing warps make the slab's rows visible (memory
@@ -985,6 +985,10 @@ cudaError_t smat_launch_tabulate_tc(const void* in, void* out, void* scratch, co
     return launch_radon(q, transpose, 1, &sp, state_elems, bh, status, st);
   }
   if (geo.D != 3) return cudaErrorInvalidValue;
+  if (!transpose && smat_tabulate_slab_supported(q, state_elems)) {
+    *launches = 1;
+    return smat_launch_tabulate_slab(in, out, geo, state_elems, bh, status, st);
+  }
   const int64_t wrows = smat_tabulate_tc_scratch_rows(geo);
   const RadonSide f_side = side(qq, 1, qq, q, geo.P);                       // image x2, points (x1, x3)
   const RadonSide w1_side = side(qq + q, 1, qq, q, wrows, qqq, q, 1, 0);    // (u, a3) -> W[a3][x2][u]; extra class -> G[x3][x2]
