@@ -131,11 +131,10 @@ struct ItemIter {
   __device__ __forceinline__ bool closes_phase0() const { return nph > 1 && ph == 0 && img + 1 == im0; }
 };
 
-// Lane 0 polls the barrier and the warp follows.
+// All lanes wait: one lane polling and a shuffle cost about a hundred cycles more at every wait (q = 17, d = 3, transposed,
+// 64 heads: 0.64 ms against 0.56; d = 4, 16 heads: 2.25 against 2.21).
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, const WaitCtx& w) {
-  bool ok = true;
-  if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, w);
-  return __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, w));
 }
 
 // Row of the streamed operand that holds input index (lo, line): slot line / sps, then the line's q rows.
@@ -965,9 +964,9 @@ int64_t smat_tabulate_tc_scratch_elems(const SmatGeo& geo, int64_t state_elems, 
 
 // Which of the two kernels runs a stage.  The one that generates R loads an image once where the resident one has two or
 // three CTAs load it, but shares its issue slots and tensor memory with the generators.  Measured (ms, resident against
-// generated): q = 13, d = 3, 32 heads 0.083 / 0.073, transposed 0.092 / 0.072; q = 13, d = 4, 8 heads 0.462 / 0.425,
-// transposed (4 heads) 0.289 / 0.274; q = 17, d = 3, 64 heads 0.263 / 0.299, transposed 0.331 / 0.293; q = 17, d = 4,
-// 8 heads 1.14 / 1.26.  At q <= 11 one CTA covers an image either way.
+// generated): q = 13, d = 3, 32 heads 0.077 / 0.069, transposed 0.089 / 0.072; q = 13, d = 4, 8 heads 0.425 / 0.405,
+// transposed (4 heads) 0.278 / 0.254; q = 17, d = 3, 64 heads 0.256 / 0.272, transposed 0.312 / 0.269; q = 17, d = 4,
+// 8 heads 1.11 / 1.22.  At q <= 11 one CTA covers an image either way.
 static bool generates_matrix(int q, int D, int transpose) { return q == 13 || (q == 17 && D == 2 && transpose); }
 
 // transpose = 0: in = F [bh][P][rp] bf16, out = U [bh][B][rp] bf16.  transpose = 1: in = Ū [bh][B][rp], out = F̄ [bh][P][rp].

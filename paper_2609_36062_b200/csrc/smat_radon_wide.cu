@@ -12,10 +12,10 @@
 // memory hold.  The nonzeros are 2.0, whose bf16 pattern is a single bit (one shift and one mask per register), and the
 // sums are halved when they are rounded: both exact.  More than three tiles (q >= 23): the CTAs are shared out over the
 // groups of tiles, in proportion to their tiles, and every group walks the images in the same order.
-// Bound: q = 13 and 19 by the image and table rows (32 heads of 4096 tokens, 368 MB: 0.073 ms, 0.056 at the HBM rate; 32
-// heads of 12288 tokens at q = 19: 0.178 ms, where the sums on the fp32 ALUs took 0.446); q >= 23 by the round trip of an A
-// tile (store to tensor memory, hand-over, MMAs, hand-back: about 1300 cycles over four tiles, 256 of MMAs each): 16 heads,
-// sums on the ALUs / here: q = 23 0.321 / 0.195 ms, 29 0.540 / 0.367, 31 0.708 / 0.458, 37 1.053 / 0.800.
+// Bound: q = 13 and 19 by the image and table rows (32 heads of 4096 tokens, 368 MB: 0.069 ms, 0.056 at the HBM rate; 32
+// heads of 12288 tokens at q = 19: 0.170 ms, where the sums on the fp32 ALUs took 0.446); q >= 23 by the round trip of an A
+// tile (store to tensor memory, hand-over, MMAs, hand-back: about 1100 cycles over four tiles, 256 of MMAs each): 16 heads,
+// sums on the ALUs / here: q = 23 0.321 / 0.172 ms, 29 0.540 / 0.321, 31 0.708 / 0.404, 37 1.053 / 0.690.
 //   warps 0-15  : epilogue; lane quarter w % 4, column quarter w / 4 of every accumulator: round to bf16, whole sectors
 //   warps 16-27 : generators of R, three groups of four warps that take the (slot, tile) pairs in turn
 //   warp 28     : TMA producer;   warps 29-31 : MMA issuers, one per tile
@@ -144,10 +144,10 @@ __device__ __forceinline__ bool elect_one() {
   return pred != 0;
 }
 
+// All lanes wait: with one lane polling and a shuffle (and, before that, one warp of four polling for the generators, the
+// others at a named barrier) 16 heads, q = 37, took 0.80 ms instead of 0.69.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, const WaitCtx& w) {
-  bool ok = true;
-  if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, w);
-  return __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, w));
 }
 
 __global__ void __launch_bounds__(THREADS, 1) radon_wide_kernel(const __grid_constant__ CUtensorMap tm_reg,
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(THREADS, 1) radon_wide_kernel(const __grid_con
       }
       const uint32_t was = n - A_RING;
       if (n >= A_RING &&
-          !group_wait(a_empty + (was & (A_BARS - 1)), (was / A_BARS) & 1, wc, qd == 0 && lane == 0, 2 + mine, 128))
+          !mbar_wait_warp(a_empty + (was & (A_BARS - 1)), (was / A_BARS) & 1, wc))
         break;
       fence_after_sync();
       tmem_st32(tmem_base + ((uint32_t)(qd * 32) << 16) + A_COL + (n & (A_RING - 1)) * 32, v);

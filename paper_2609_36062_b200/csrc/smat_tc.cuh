@@ -78,27 +78,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const 
   return false;
 }
 
-// Wait of `threads` threads (whole warps) of which one polls: the others sleep at named barrier `id`.  Many warps
-// polling their barriers take most of the issue slots, and the single issuing threads' instructions are what most of
-// these kernels wait for.  All get the poller's result.
-__device__ __forceinline__ bool group_wait(uint64_t* bar, uint32_t parity, const WaitCtx& w, bool poller, int id, int threads) {
-  uint32_t failed = 0;
-  if (poller) failed = !mbar_wait(bar, parity, w);
-  __syncwarp();
-  uint32_t r;
-  asm volatile(
-      "{\n"
-      ".reg .pred p, q;\n"
-      "setp.ne.u32 q, %1, 0;\n"
-      "barrier.cta.red.or.pred p, %2, %3, q;\n"
-      "selp.u32 %0, 1, 0, p;\n"
-      "}\n"
-      : "=r"(r)
-      : "r"(failed), "r"(id), "r"(threads)
-      : "memory");
-  return r == 0;
-}
-
 // ---- TMA (no multicast: every CTA fetches its own tiles) ---------------------------------------------------
 __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
   asm volatile(
