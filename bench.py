@@ -37,10 +37,9 @@ SWEEP = ["t4k_d3", "t64k_d1", "t64k_d2", "t64k_d3", "t64k_d4", "t8k_d3_fwdbwd", 
          "t4k_d3_gated", "t4k_d3_gated_fwdbwd"]
 METRIC = "SMat prefill tokens/s"
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of the dominant stage per step — the tabulation, one
-# launch of radon_tc_kernel — from an ncu capture of the 8-head copy of the workload (351.3 MB read + 530.1 MB
-# written), scaled by heads (every head owns its tables; the per-CTA exchange buffer, the only shared footprint,
-# is the same 55 MB at 8 and at 32 heads).
-NCU_TRAFFIC_BYTES = {("t16k_d4", "tabulate_tc"): 881.4e6 * 4}
+# launch of radon_slab_kernel — from an ncu capture of the 8-head copy of the workload: F (349.0 MB) read once, U (383.5 MB)
+# written once but for the 56.0 MB still in the L2 cache at the end; the tables scaled by heads.
+NCU_TRAFFIC_BYTES = {("t16k_d4", "tabulate_tc"): (349.0e6 + 383.5e6) * 4 - 56.0e6}
 
 
 def parse_args():
