@@ -13,9 +13,10 @@
 // sums are halved when they are rounded: both exact.  More than three tiles (q >= 23): the CTAs are shared out over the
 // groups of tiles, in proportion to their tiles, and every group walks the images in the same order.
 // Bound: q = 13 and 19 by the image and table rows (32 heads of 4096 tokens, 368 MB: 0.069 ms, 0.056 at the HBM rate; 32
-// heads of 12288 tokens at q = 19: 0.170 ms, where the sums on the fp32 ALUs took 0.446); q >= 23 by the round trip of an A
-// tile (store to tensor memory, hand-over, MMAs, hand-back: about 1100 cycles over four tiles, 256 of MMAs each): 16 heads,
-// sums on the ALUs / here: q = 23 0.321 / 0.172 ms, 29 0.540 / 0.321, 31 0.708 / 0.404, 37 1.053 / 0.690.
+// heads of 12288 tokens at q = 19: 0.170 ms, where the sums on the fp32 ALUs took 0.446); q >= 23 by the tensor pipe (75 % active
+// at q = 37, whose images the groups read from memory once, 731 MB for a table of 718; two tiles per item and eight A tiles in
+// flight instead of three and four: 0.98 ms instead of 0.69): 16 heads, sums on the ALUs / here: q = 23 0.321 / 0.172 ms,
+// 29 0.540 / 0.321, 31 0.708 / 0.404, 37 1.053 / 0.690.
 //   warps 0-15  : epilogue; lane quarter w % 4, column quarter w / 4 of every accumulator: round to bf16, whole sectors
 //   warps 16-27 : generators of R, three groups of four warps that take the (slot, tile) pairs in turn
 //   warp 28     : TMA producer;   warps 29-31 : MMA issuers, one per tile
