@@ -1,7 +1,9 @@
 // Launches with programmatic dependent launch: a kernel of a pass may be set up (its CTAs placed, barriers
 // initialised, tensor memory taken) while the kernel before it drains, and waits for that kernel's results at
 // pdl_wait().  Every kernel launched this way calls pdl_wait() in every thread that touches global memory, before it
-// does, so completion stays transitive along the stream; pdl_trigger() lets the next kernel start its own set-up.
+// does, and in at least one thread of every CTA, also of one that has nothing to do: a launch whose CTAs all leave without
+// it completes beside the kernel before, and completion would no longer be transitive along the stream.  pdl_trigger()
+// lets the next kernel start its own set-up.
 // Two rules follow.  A kernel that takes tensor memory triggers only after it has it: the next kernel's CTAs start once
 // all of this one's have triggered, and a CTA that took the columns first and then waited for this kernel would never
 // give them back.  And data of earlier kernels is read with plain loads, not through __ldg or const __restrict__ pointers:

@@ -829,7 +829,13 @@ __global__ void __launch_bounds__(192) segment_state_tc_kernel(const __grid_cons
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int seg = blockIdx.x, bh = blockIdx.y;
   // The scan is exclusive: nobody reads the total of a block's last segment (the scan loads it after its last store).
-  if (seg == prm.cut.nseg0 - 1 || seg == prm.cut.nseg - 1) return;
+  // Such a CTA still waits for the kernel before: where every block is one segment no other CTA of the launch does, and
+  // the kernels after this one would run beside that kernel.
+  if (seg == prm.cut.nseg0 - 1 || seg == prm.cut.nseg - 1) {
+    pdl_trigger();
+    pdl_wait();
+    return;
+  }
   int64_t tile0;
   int Lc;
   seg_range(prm.cut, seg, &tile0, &Lc);

@@ -99,3 +99,25 @@ def test_routed_call_is_reproducible_and_validates_its_arguments():
     assert lib.smat_forward_routed(plan.handle, *args, prof.data_ptr() + 2, typ.data_ptr(), ws.data_ptr(), ws.numel(), None) == 6
     with pytest.raises(ValueError):
         plan.forward(dev["q"], dev["k"], dev["v"], prof=prof[:, :-1].contiguous(), type=typ)
+
+
+def test_one_type_takes_every_query_of_a_short_batch():
+    """One segment per block: the launch of the segment totals has nothing to do, and one CTA of the typed read works
+    through all queries of a head.  The output kernel must not start on rows the read has yet to write (NaN before)."""
+    w = synth.Workload("one_type", 3, 4, 32, 2048, 128, 128, 128, "bf16", "normalised", 71)
+    host, dev = device_inputs(w, ("q", "k", "v"))
+    geo = so.geometry(w.T, w.chunk, w.d)
+    cells, _ = so.positional_assignment(geo)
+    types = np.full(geo.m, 5, dtype=np.int32)
+    prof = torch.from_numpy(np.tile(cells, (w.bh, 1))).int().cuda()
+    typ = torch.from_numpy(np.tile(types, (w.bh, 1))).int().cuda()
+    plan = binding.SmatPlan(w.batch, w.heads, w.T, w.d_k, w.d_v, w.d, w.chunk, w.dtype)
+    ws = plan.workspace()
+    ws.fill_(0xFF)
+    O = plan.forward(dev["q"], dev["k"], dev["v"], workspace=ws, prof=prof, type=typ)
+    plan.check_status(ws)
+    assert torch.isfinite(O).all()
+    M = so.routed_dense_mask(geo, cells, types)
+    for h in (0, 77, w.bh - 1):
+        Q64, K64, V64 = (synth.as_float64(w, host[x][h]) for x in ("q", "k", "v"))
+        assert rel_err(to_numpy64(O.reshape(w.bh, w.T, -1)[h]), so.forward_dense(Q64, K64, V64, M)) <= TOL["bf16"]
