@@ -84,14 +84,16 @@ bool stream(PyObject* o, void** st) {
   return !PyErr_Occurred();
 }
 
-// A call into the library with the interpreter lock released (a full launch queue may block it).
+// The interpreter lock is released for a call into the library (a full launch queue may block it).  The library throws
+// nothing; what can throw, the data pointers of tensors without storage among it, is asked for before.
+struct Unlocked {
+  PyThreadState* state = PyEval_SaveThread();
+  ~Unlocked() { PyEval_RestoreThread(state); }
+};
 template <typename F>
 int unlocked(F call) {
-  int rc;
-  Py_BEGIN_ALLOW_THREADS
-  rc = call();
-  Py_END_ALLOW_THREADS
-  return rc;
+  Unlocked lock;
+  return call();
 }
 
 bool arity(Py_ssize_t got, Py_ssize_t want, const char* name) {
@@ -155,25 +157,27 @@ PyObject* plan_forward(PyObject* self, PyObject* const* a, Py_ssize_t n) {
     size_t bytes;
     if (kind == 0 && a[5] != Py_None && !tensor(a[5], "O", p.dtype, sv)) return nullptr;
     if (!output(a[5], "O", *V, &O) || !workspace(a[6], "workspace", &ws, &bytes) || !stream(a[7], &st)) return nullptr;
+    const void *q = Q->data_ptr(), *k = K->data_ptr(), *v = V->data_ptr();
+    void* o = O.data_ptr();
     int rc;
     const char* what;
     if (kind == 1) {
       what = "smat_forward_gated";
-      rc = unlocked([&] { return smat_forward_gated(p.handle, Q->data_ptr(), K->data_ptr(), V->data_ptr(), la->data_ptr<float>(), O.data_ptr(),
-                              ws, bytes, st); });
+      const float* log_a = la->data_ptr<float>();
+      rc = unlocked([&] { return smat_forward_gated(p.handle, q, k, v, log_a, o, ws, bytes, st); });
     } else if (kind == 2) {
       what = "smat_forward_normalized";
-      rc = unlocked([&] { return smat_forward_normalized(p.handle, Q->data_ptr(), K->data_ptr(), V->data_ptr(), O.data_ptr(), ws, bytes, st); });
+      rc = unlocked([&] { return smat_forward_normalized(p.handle, q, k, v, o, ws, bytes, st); });
     } else if (a[8] != Py_None || a[9] != Py_None) {
       const int64_t sp[2] = {p.b * p.h, p.n}, stp[2] = {p.b * p.h, p.m};
       const at::Tensor *prof = tensor(a[8], "prof", at::kInt, sp), *type = prof ? tensor(a[9], "type", at::kInt, stp) : nullptr;
       if (!type) return nullptr;
       what = "smat_forward_routed";
-      rc = unlocked([&] { return smat_forward_routed(p.handle, Q->data_ptr(), K->data_ptr(), V->data_ptr(), O.data_ptr(), prof->data_ptr<int>(),
-                               type->data_ptr<int>(), ws, bytes, st); });
+      const int32_t *cells = prof->data_ptr<int>(), *types = type->data_ptr<int>();
+      rc = unlocked([&] { return smat_forward_routed(p.handle, q, k, v, o, cells, types, ws, bytes, st); });
     } else {
       what = "smat_forward";
-      rc = unlocked([&] { return smat_forward(p.handle, Q->data_ptr(), K->data_ptr(), V->data_ptr(), O.data_ptr(), ws, bytes, st); });
+      rc = unlocked([&] { return smat_forward(p.handle, q, k, v, o, ws, bytes, st); });
     }
     return fail_status(rc, what) ? wrap(O) : nullptr;
   })
@@ -200,27 +204,29 @@ PyObject* plan_backward(PyObject* self, PyObject* const* a, Py_ssize_t n) {
     if (!output(a[7], "dQ", *Q, &dQ) || !output(a[8], "dK", *K, &dK) || !output(a[9], "dV", *V, &dV) ||
         (la && !output(a[10], "dlog_a", *la, &dla)) || !workspace(a[11], "workspace", &ws, &bytes) || !stream(a[12], &st))
       return nullptr;
+    const void *q = Q->data_ptr(), *k = K->data_ptr(), *v = V->data_ptr(), *go = dO->data_ptr();
+    void *gq = dQ.data_ptr(), *gk = dK.data_ptr(), *gv = dV.data_ptr();
     int rc;
     const char* what;
     if (kind == 1) {
       what = "smat_backward_gated";
-      rc = unlocked([&] { return smat_backward_gated(p.handle, Q->data_ptr(), K->data_ptr(), V->data_ptr(), la->data_ptr<float>(), dO->data_ptr(),
-                               dQ.data_ptr(), dK.data_ptr(), dV.data_ptr(), dla.data_ptr<float>(), ws, bytes, st); });
+      const float* log_a = la->data_ptr<float>();
+      float* glog_a = dla.data_ptr<float>();
+      rc = unlocked([&] { return smat_backward_gated(p.handle, q, k, v, log_a, go, gq, gk, gv, glog_a, ws, bytes, st); });
     } else if (kind == 2) {
       what = "smat_backward_normalized";
-      rc = unlocked([&] { return smat_backward_normalized(p.handle, Q->data_ptr(), K->data_ptr(), V->data_ptr(), O->data_ptr(), dO->data_ptr(),
-                                    dQ.data_ptr(), dK.data_ptr(), dV.data_ptr(), ws, bytes, st); });
+      const void* o = O->data_ptr();
+      rc = unlocked([&] { return smat_backward_normalized(p.handle, q, k, v, o, go, gq, gk, gv, ws, bytes, st); });
     } else if (a[13] != Py_None || a[14] != Py_None) {
       const int64_t sp[2] = {p.b * p.h, p.n}, stp[2] = {p.b * p.h, p.m};
       const at::Tensor *prof = tensor(a[13], "prof", at::kInt, sp), *type = prof ? tensor(a[14], "type", at::kInt, stp) : nullptr;
       if (!type) return nullptr;
       what = "smat_backward_routed";
-      rc = unlocked([&] { return smat_backward_routed(p.handle, Q->data_ptr(), K->data_ptr(), V->data_ptr(), dO->data_ptr(), dQ.data_ptr(),
-                                dK.data_ptr(), dV.data_ptr(), prof->data_ptr<int>(), type->data_ptr<int>(), ws, bytes, st); });
+      const int32_t *cells = prof->data_ptr<int>(), *types = type->data_ptr<int>();
+      rc = unlocked([&] { return smat_backward_routed(p.handle, q, k, v, go, gq, gk, gv, cells, types, ws, bytes, st); });
     } else {
       what = "smat_backward";
-      rc = unlocked([&] { return smat_backward(p.handle, Q->data_ptr(), K->data_ptr(), V->data_ptr(), dO->data_ptr(), dQ.data_ptr(), dK.data_ptr(),
-                         dV.data_ptr(), ws, bytes, st); });
+      rc = unlocked([&] { return smat_backward(p.handle, q, k, v, go, gq, gk, gv, ws, bytes, st); });
     }
     if (!fail_status(rc, what)) return nullptr;
     return la ? wrap_all({dQ, dK, dV, dla}) : wrap_all({dQ, dK, dV});
@@ -254,10 +260,12 @@ PyObject* plan_decode_step(PyObject* self, PyObject* const* a, Py_ssize_t n) {
     void *cache, *st;
     size_t bytes;
     if (!workspace(a[5], "cache", &cache, &bytes) || !output(a[6], "o", *v, &o) || !stream(a[7], &st)) return nullptr;
+    const void *qp = q->data_ptr(), *kp = k->data_ptr(), *vp = v->data_ptr();
+    void* op = o.data_ptr();
+    const float* log_a = la ? la->data_ptr<float>() : nullptr;
     const int rc = unlocked([&] {
-      return la ? smat_decode_step_gated(p.handle, q->data_ptr(), k->data_ptr(), v->data_ptr(), la->data_ptr<float>(), t,
-                                         o.data_ptr(), cache, bytes, st)
-                : smat_decode_step(p.handle, q->data_ptr(), k->data_ptr(), v->data_ptr(), t, o.data_ptr(), cache, bytes, st);
+      return la ? smat_decode_step_gated(p.handle, qp, kp, vp, log_a, t, op, cache, bytes, st)
+                : smat_decode_step(p.handle, qp, kp, vp, t, op, cache, bytes, st);
     });
     return fail_status(rc, la ? "smat_decode_step_gated" : "smat_decode_step") ? wrap(o) : nullptr;
   })

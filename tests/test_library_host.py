@@ -172,3 +172,27 @@ def test_gated_plans_size_their_inner_plan_and_decode_cache():
     # a block boundary that is not a whole tile: no inner plan
     ragged = binding.SmatPlan(1, 2, 640, 128, 128, 3, 32, "bf16", flags=binding.FLAG_GATED)
     assert not ragged.gated_forward_uses_tensor_cores()
+
+
+def test_tensors_without_storage_raise_an_error():
+    """Under vmap the operands carry no storage: asking for their data pointer raises (and used to do so with the
+    interpreter lock released, which ended the process)."""
+    import types
+
+    import torch
+    from torch._subclasses import FakeTensorMode
+
+    plan = binding.SmatPlan(1, 1, 256, 64, 64, 2, 32, "f32")
+    cache_plan = binding.SmatPlan(1, 1, 256, 64, 64, 2, 32, "f32", flags=binding.FLAG_GATED)
+    stream = types.SimpleNamespace(cuda_stream=0)
+    with FakeTensorMode():
+        x, row = torch.empty(3, 1, 1, 256, 64, device="cuda"), torch.empty(3, 1, 1, 64, device="cuda")
+        ws, o = torch.empty(1024, dtype=torch.uint8, device="cuda"), torch.empty(1, 1, 256, 64, device="cuda")
+        orow, gate = torch.empty(1, 1, 64, device="cuda"), torch.empty(1, device="cuda")
+        calls = (lambda t, r: plan.forward(t, t, t, O=o, workspace=ws, stream=stream),
+                 lambda t, r: plan.backward(t, t, t, t, dQ=o, dK=o, dV=o, workspace=ws, stream=stream)[0],
+                 lambda t, r: plan.decode_step(r, r, r, 200, ws, o=orow, stream=stream),
+                 lambda t, r: cache_plan.decode_step_gated(r, r, r, gate, 200, ws, o=orow, stream=stream))
+        for call in calls:
+            with pytest.raises(RuntimeError, match="storage"):
+                torch.func.vmap(call)(x, row)
