@@ -48,3 +48,18 @@ def test_measured_add_rate_is_plausible():
     nominal = sms * 128 * 1.965e9                                # lanes x maximum SM clock
     for rate in (scalar, packed):
         assert 0.3 * nominal <= rate <= 2.2 * nominal, (rate, nominal)
+
+
+def test_an_exhausted_device_raises_out_of_memory_error():
+    """The output that forward allocates does not fit: the error is torch's own, which callers catch by its type."""
+    plan = binding.SmatPlan(1, 32, 4096, 128, 128, 1, 64, "f32")
+    x = torch.randn(1, 32, 4096, 128, device="cuda")
+    ws = plan.workspace()
+    torch.cuda.empty_cache()
+    torch.cuda.set_per_process_memory_fraction(1e-6)      # of torch's allocator alone: no further block is granted
+    try:
+        with pytest.raises(torch.OutOfMemoryError):
+            plan.forward(x, x, x, workspace=ws)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    assert plan.forward(x, x, x, workspace=ws).shape == x.shape
