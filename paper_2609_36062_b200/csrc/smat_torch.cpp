@@ -97,6 +97,15 @@ int unlocked(F call) {
   return call();
 }
 
+// Anything int() takes (a position kept as a float or as an array scalar among it).
+bool token_index(PyObject* o, long long* t) {
+  PyObject* n = PyNumber_Long(o);
+  if (!n) return false;
+  *t = PyLong_AsLongLong(n);
+  Py_DECREF(n);
+  return !(*t == -1 && PyErr_Occurred());
+}
+
 bool arity(Py_ssize_t got, Py_ssize_t want, const char* name) {
   if (got == want) return true;
   PyErr_Format(PyExc_TypeError, "%s takes %zd arguments, got %zd", name, want, got);
@@ -247,8 +256,8 @@ PyObject* plan_decode_step(PyObject* self, PyObject* const* a, Py_ssize_t n) {
       return nullptr;
     }
   }
-  const long long t = PyLong_AsLongLong(a[4]);
-  if (t == -1 && PyErr_Occurred()) return nullptr;
+  long long t;
+  if (!token_index(a[4], &t)) return nullptr;
   at::Tensor o;
   void *cache, *st;
   size_t bytes;

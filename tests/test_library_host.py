@@ -192,6 +192,8 @@ def test_tensors_without_storage_raise_an_error():
         calls = (lambda t, r: plan.forward(t, t, t, O=o, workspace=ws, stream=stream),
                  lambda t, r: plan.backward(t, t, t, t, dQ=o, dK=o, dV=o, workspace=ws, stream=stream)[0],
                  lambda t, r: plan.decode_step(r, r, r, 200, ws, o=orow, stream=stream),
+                 lambda t, r: plan.decode_step(r, r, r, 200.0, ws, o=orow, stream=stream),      # any t that int() takes
+                 lambda t, r: plan.decode_step(r, r, r, np.int32(200), ws, o=orow, stream=stream),
                  lambda t, r: cache_plan.decode_step_gated(r, r, r, gate, 200, ws, o=orow, stream=stream))
         for call in calls:
             with pytest.raises(RuntimeError, match="storage"):
