@@ -112,8 +112,8 @@ bool arity(Py_ssize_t got, Py_ssize_t want, const char* name) {
   return false;
 }
 
-// An output: the caller's tensor, or a new one like `like`.  A tensor handed in has the same element type and count
-// and is contiguous; its shape may be another view of the same rows.
+// An output: the caller's tensor, or a new one like `like`.  A tensor handed in has the same element type, is contiguous
+// and holds at least as many elements: another view of the same rows, or a larger buffer whose first part is written.
 bool output(PyObject* o, const char* name, const at::Tensor& like, at::Tensor* out) {
   if (o == Py_None) {
     *out = at::empty_like(like);
@@ -121,12 +121,12 @@ bool output(PyObject* o, const char* name, const at::Tensor& like, at::Tensor* o
   }
   if (THPVariable_Check(o)) {
     const at::Tensor& t = THPVariable_Unpack(o);
-    if (t.is_cuda() && t.scalar_type() == like.scalar_type() && t.numel() == like.numel() && t.is_contiguous()) {
+    if (t.is_cuda() && t.scalar_type() == like.scalar_type() && t.numel() >= like.numel() && t.is_contiguous()) {
       *out = t;
       return true;
     }
   }
-  PyErr_Format(PyExc_ValueError, "%s: expected a contiguous CUDA tensor of %s and shape %s", name,
+  PyErr_Format(PyExc_ValueError, "%s: expected a contiguous CUDA tensor of %s that holds shape %s", name,
                c10::toString(like.scalar_type()), shape_text(like.sizes()).c_str());
   return false;
 }

@@ -198,3 +198,37 @@ def test_tensors_without_storage_raise_an_error():
         for call in calls:
             with pytest.raises(RuntimeError, match="storage"):
                 torch.func.vmap(call)(x, row)
+
+
+def test_output_buffers_may_be_larger_but_not_smaller_or_strided():
+    """Outputs other than forward's O: the first elements of a larger buffer are written; anything a call would write
+    out of, or in another order than the tensor shows, is refused."""
+    import types
+
+    import torch
+    from torch._subclasses import FakeTensorMode
+
+    plan = binding.SmatPlan(1, 1, 256, 64, 64, 2, 32, "f32")
+    stream = types.SimpleNamespace(cuda_stream=0)
+    with FakeTensorMode():
+        x, row = torch.empty(3, 1, 1, 256, 64, device="cuda"), torch.empty(3, 1, 1, 64, device="cuda")
+        ws = torch.empty(1024, dtype=torch.uint8, device="cuda")
+        big, small = torch.empty(2, 256, 64, device="cuda"), torch.empty(1, 1, 255, 64, device="cuda")
+        flat, strided = torch.empty(256 * 64, device="cuda"), torch.empty(1, 1, 64, 256, device="cuda").transpose(2, 3)
+
+        def backward(out):
+            return torch.func.vmap(lambda t: plan.backward(t, t, t, t, dQ=out, dK=out, dV=out, workspace=ws, stream=stream)[0])(x)
+
+        def decode(out):
+            return torch.func.vmap(lambda r: plan.decode_step(r, r, r, 200, ws, o=out, stream=stream))(row)
+
+        for ok in (big, flat):
+            with pytest.raises(RuntimeError, match="storage"):      # past the checks
+                backward(ok)
+        with pytest.raises(RuntimeError, match="storage"):
+            decode(big)
+        for bad in (small, strided, big.to(torch.bfloat16)):
+            with pytest.raises(ValueError):
+                backward(bad)
+        with pytest.raises(ValueError):
+            decode(small[..., :63])
