@@ -361,6 +361,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) tile_product_tc_kernel(const 
         const float4* y4 = reinterpret_cast<const float4*>(prm.addend + ((int64_t)bh * prm.T + t) * TILE + half * HALF);
         const uint4* y16 = reinterpret_cast<const uint4*>(prm.addend16 + ((int64_t)bh * prm.T + t) * TILE + half * HALF);
         uint4* dst = reinterpret_cast<uint4*>(prm.Out + ((int64_t)bh * prm.T + t) * TILE + half * HALF);
+        const bool wide = rows_are_wide(prm.Out);
         {
           const int cb = part;   // 32 of the 64 output columns
           uint32_t v[32];
@@ -397,7 +398,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) tile_product_tc_kernel(const 
           }
 #pragma unroll
           for (int h8 = 0; h8 < 2; ++h8)   // whole 32-byte sectors
-            st_global_v8(dst + cb * 4 + 2 * h8, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
+            st_global_32(dst + cb * 4 + 2 * h8, wide, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
                          w[8 * h8 + 5], w[8 * h8 + 6], w[8 * h8 + 7]);
         }
       }
@@ -609,6 +610,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) bwd_tile_fused_tc_kernel(con
     // this thread's 64 bytes (four 16-byte chunks) of its row in the 64-column block that holds its columns
     const uint32_t my_off = (cq >> 1) * BOX_BYTES + m * 128;
     const int ch0 = (cq & 1) * 4;
+    const bool wide = rows_are_wide(prm.dQ) && rows_are_wide(prm.dK) && rows_are_wide(prm.dV);
     uint32_t par = 0;
     auto arrive = [&](uint64_t* bar) {
       fence_before_sync();
@@ -703,7 +705,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) bwd_tile_fused_tc_kernel(con
         __nv_bfloat16* dst = out + row * TILE + col0;
 #pragma unroll
         for (int h8 = 0; h8 < 2; ++h8)   // whole 32-byte sectors
-          st_global_v8(dst + 16 * h8, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
+          st_global_32(dst + 16 * h8, wide, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
                        w[8 * h8 + 5], w[8 * h8 + 6], w[8 * h8 + 7]);
         return dot;
       };
@@ -1172,6 +1174,7 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
       publish_state(v, tile0);
     }
     const int64_t row_first = seg_tile_row(prm.cut, tile0), row_end = blk ? prm.cut.rows : prm.cut.rows0;
+    const bool wide = rows_are_wide(prm.O);
     for (int it = 0; it < Lc; ++it) {
       uint8_t* stage = smem + (it & 1) * Lay::STAGE;
       // --- scores of this tile -> masked bf16 P (registers), stored once Q and K have been consumed ---
@@ -1249,7 +1252,7 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
       if (live) {
 #pragma unroll
         for (int h8 = 0; h8 < 2; ++h8)   // whole 32-byte sectors
-          st_global_v8(dst + 16 * h8, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
+          st_global_32(dst + 16 * h8, wide, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
                        w[8 * h8 + 5], w[8 * h8 + 6], w[8 * h8 + 7]);
       }
     }

@@ -210,6 +210,19 @@ __device__ __forceinline__ void st_global_v8(void* dst, uint32_t w0, uint32_t w1
                : "memory");
 }
 
+// The same 32 bytes of a caller's array, which is promised to lie on a 16-byte boundary only: `wide` (uniform, from
+// rows_are_wide) says that the array's 256-byte rows start on 32-byte boundaries.
+__device__ __forceinline__ bool rows_are_wide(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31) == 0; }
+__device__ __forceinline__ void st_global_32(void* dst, bool wide, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3,
+                                             uint32_t w4, uint32_t w5, uint32_t w6, uint32_t w7) {
+  if (wide) {
+    st_global_v8(dst, w0, w1, w2, w3, w4, w5, w6, w7);
+  } else {
+    reinterpret_cast<uint4*>(dst)[0] = make_uint4(w0, w1, w2, w3);
+    reinterpret_cast<uint4*>(dst)[1] = make_uint4(w4, w5, w6, w7);
+  }
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&v);
