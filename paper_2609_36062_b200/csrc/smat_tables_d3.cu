@@ -220,6 +220,7 @@ __global__ void __launch_bounds__(D3Layout<Q>::THREADS, 1) tabulate_d3_f32_kerne
     // cannot tell the phase before the one in flight from its own), and the early count would start a second load, a
     // second arrival in one phase.  So a warp first waits until its own slab's load has been started, which is after
     // the phase before it has ended.
+    // Then every lane waits for the slab itself: all of them read what the copy engine wrote.
     bool ok = true;
     if (lane == 0) {
       const long long since = clock64();
@@ -228,9 +229,11 @@ __global__ void __launch_bounds__(D3Layout<Q>::THREADS, 1) tabulate_d3_f32_kerne
         if (clock64() - since > wc.limit) { *cta_abort = 1; atomicExch(prm.status, 1); ok = false; }
         __nanosleep(100);
       }
-      ok = ok && mbar_wait(slab_full + buf, (ks / NBUF) & 1, wc);
     }
-    if (!__shfl_sync(0xffffffffu, (int)ok, 0)) {
+    ok = __all_sync(0xffffffffu, ok);
+    __syncwarp();
+    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(slab_full + buf, (ks / NBUF) & 1, wc));
+    if (!ok) {
       if (lane == 0) {   // shared memory must outlive the copies into it
         for (uint32_t b = 0; b < NBUF; ++b) {
           const uint32_t last = started[b];
