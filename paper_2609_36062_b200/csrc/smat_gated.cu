@@ -43,14 +43,16 @@ __global__ void __launch_bounds__(1024) head_scan_kernel(const float* in, float*
     }
     if (lane == 31) warp_sum[turn][warp] = run;
     __syncthreads();
-    const float own = warp_sum[turn][lane];
-    float tot = own;
+    float tot = warp_sum[turn][lane];
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
       const float y = __shfl_up_sync(0xffffffffu, tot, d);
       if (lane >= d) tot += y;
     }
-    const float before = carry + __shfl_sync(0xffffffffu, tot - own, warp);
+    // the warps before this one, taken from the scan itself: their sum as (sum through this warp) - (this warp's values)
+    // loses the low bits of theirs wherever one strong gate outweighs them, for the tokens before that gate too
+    const float prev = __shfl_sync(0xffffffffu, tot, warp ? warp - 1 : 0);
+    const float before = carry + (warp ? prev : 0.f);
     carry += __shfl_sync(0xffffffffu, tot, 31);
 #pragma unroll
     for (int i = 0; i < PER; ++i) {

@@ -218,3 +218,25 @@ def test_gated_passes_with_the_other_tabulations_of_the_inner_plan(flag):
         for name, got, ref in (("dQ", dQ, rq), ("dK", dK, rk), ("dV", dV, rv)):
             assert rel_err(to_numpy64(got[0, h]), ref) <= TOL["bf16"], (name, h)
         assert rel_err(dla[h].double().cpu().numpy(), rl) <= 5e-2
+
+
+@pytest.mark.parametrize("at", [200, 300, 4500])
+@pytest.mark.parametrize("dtype,dk,c", [("f32", 64, 64), ("bf16", 128, 128)])
+def test_rows_before_a_strong_gate_do_not_notice_it(at, dtype, dk, c):
+    """One gate of e^-10000 among moderate ones: the rows before it are bit for bit what they are without it (their λ must
+    not lose low bits to a sum that it dominates), and on fp32 plans the whole output stays with the oracle."""
+    T = 512 if at < 512 else 8192
+    w = synth.Workload("g3", 3, 1, 1, T, dk, dk, c, dtype, "scaled", 9)
+    host, dev = device_inputs(w)
+    la = _gates(w, 0.9, 4)
+    hit = la.copy()
+    hit[0, at] = -1e4
+    plan = binding.SmatPlan(1, 1, T, dk, dk, 3, c, dtype, flags=binding.FLAG_GATED)
+    a = plan.forward_gated(dev["q"], dev["k"], dev["v"], torch.from_numpy(la).cuda())
+    b = plan.forward_gated(dev["q"], dev["k"], dev["v"], torch.from_numpy(hit).cuda())
+    plan.check_status()
+    assert torch.equal(a[0, 0, :at], b[0, 0, :at])
+    if dtype == "f32" and T == 512:
+        Q64, K64, V64 = (synth.as_float64(w, host[x][0]) for x in ("q", "k", "v"))
+        ref = so.gated_forward_dense(Q64, K64, V64, so.dense_mask(T, c, 3), hit[0].astype(np.float64))
+        assert rel_err(to_numpy64(b[0, 0]), ref) <= TOL["f32"]
