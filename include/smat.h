@@ -341,8 +341,9 @@ smat_status smat_measure_fadd_rate(void* scratch, int packed, double* adds_per_s
  *        pools and tabulates them (steps 2-3 of Algorithm 1, through `workspace` as smat_forward would), stores the
  *        type table in the cache and zeroes S.  workspace: as for smat_forward (for_backward = 0).
  * smat_decode_step  : q, k [B,H,d_k], v [B,H,d_v] device rows of token t for every (batch, head) in the plan's dtype,
- *        o [B,H,d_v] device output in the same dtype.  Steps must be issued for t = n, n+1, ... in order, on one
- *        stream (S is updated in place).  n <= t < T, else SMAT_ERR_SHAPE.
+ *        o [B,H,d_v] device output in the same dtype; it may be the array of q or k (where d_k = d_v) or of v.  Steps
+ *        must be issued for t = n, n+1, ... in order, on one stream (S is updated in place).  n <= t < T, else
+ *        SMAT_ERR_SHAPE.
  * Both launch on the given stream and return without synchronising; errors as for smat_forward. */
 size_t smat_decode_cache_bytes(const smat_plan* plan);
 smat_status smat_decode_begin(const smat_plan* plan, const void* K, const void* V, void* cache, size_t cache_bytes,

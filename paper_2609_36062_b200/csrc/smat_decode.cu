@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(DEC_THREADS) decode_step_kernel(const T* q, co
                                                           const T* v, T* o,
                                                           float* S, const TU* U, int64_t type,
                                                           int64_t types, int p, const float* log_a,
-                                                          float* log_g) {
+                                                          float* log_g, int together) {
   constexpr int r = PASSES * DEC_ROWS;
   __shared__ float part[DEC_THREADS / 32][DEC_COLS];
   pdl_trigger();
@@ -97,6 +97,8 @@ __global__ void __launch_bounds__(DEC_THREADS) decode_step_kernel(const T* q, co
     o4[0] = fmaf(qi[n], fmaf(g, u[n].x, s[n].x), o4[0]); o4[1] = fmaf(qi[n], fmaf(g, u[n].y, s[n].y), o4[1]);
     o4[2] = fmaf(qi[n], fmaf(g, u[n].z, s[n].z), o4[2]); o4[3] = fmaf(qi[n], fmaf(g, u[n].w, s[n].w), o4[3]);
   }
+  // together: the CTAs of a head are a cluster and none writes o or the running gate before all have read q, k and it
+  if (together) asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
 #pragma unroll
   for (int c = 0; c < 4; ++c) {   // the four rows a warp holds in each of its passes
     o4[c] += __shfl_xor_sync(0xffffffffu, o4[c], 8);
@@ -104,16 +106,19 @@ __global__ void __launch_bounds__(DEC_THREADS) decode_step_kernel(const T* q, co
   }
   if ((tid & 31) < 8) *reinterpret_cast<float4*>(&part[tid >> 5][(tid & 7) * 4]) = make_float4(o4[0], o4[1], o4[2], o4[3]);
   __syncthreads();
+  if (together) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   if (tid < DEC_COLS) {
     float sum = 0.f;
 #pragma unroll
     for (int w = 0; w < DEC_THREADS / 32; ++w) sum += part[w][tid];
     store_out(o + (int64_t)bh * p + j0 + tid, sum);
   }
-  if (log_a) {   // gated launches cluster the CTAs of a head: the running gate moves on once all of them have read it
-    asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
-    if (blockIdx.x == 0 && tid == 0) log_g[bh] = lg;
-  }
+  if (log_a && blockIdx.x == 0 && tid == 0) log_g[bh] = lg;
+}
+
+bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return x < y + b_bytes && y < x + a_bytes;
 }
 
 template <typename T, typename TU>
@@ -121,9 +126,12 @@ cudaError_t launch_step(const void* q, const void* k, const void* v, void* o, fl
                         int64_t types, int r, int p, int bh, cudaStream_t st, const float* log_a, float* log_g) {
   auto kernel = r == 64 ? decode_step_kernel<T, TU, 2> : decode_step_kernel<T, TU, 4>;
   const unsigned slices = (unsigned)(p / DEC_COLS);
-  return smat_launch_pdl_cluster(kernel, dim3(slices, (unsigned)bh), DEC_THREADS, 0, log_a ? slices : 1u, st,
+  // o in the place of q or k (o in the place of v needs nothing: a CTA reads just the columns that it writes)
+  const size_t in = (size_t)bh * r * sizeof(T), out = (size_t)bh * p * sizeof(T);
+  const int together = log_a || overlap(o, out, q, in) || overlap(o, out, k, in);
+  return smat_launch_pdl_cluster(kernel, dim3(slices, (unsigned)bh), DEC_THREADS, 0, together ? slices : 1u, st,
                                  static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v),
-                                 static_cast<T*>(o), S, static_cast<const TU*>(U), type, types, p, log_a, log_g);
+                                 static_cast<T*>(o), S, static_cast<const TU*>(U), type, types, p, log_a, log_g, together);
 }
 
 }  // namespace

@@ -133,3 +133,34 @@ def test_gated_and_plain_decode_calls_do_not_mix():
         a = gated.decode_step_gated(row[0], row[1], row[2], la[:, t].contiguous(), t, cg)
         b = plain.decode_step(row[0], row[1], row[2], t, cp)
         assert rel_err(to_numpy64(a), to_numpy64(b)) <= 1e-6
+
+
+@pytest.mark.parametrize("gated", [False, True])
+@pytest.mark.parametrize("dtype,dk,c", [("f32", 64, 64), ("bf16", 128, 128)])
+@pytest.mark.parametrize("place", ["q", "k", "v"])
+def test_the_output_may_take_the_place_of_an_input_row(place, dtype, dk, c, gated):
+    B, H, T = 16, 16, 512                               # 256 heads of two or four CTAs: more than run at once
+    w = synth.Workload("inplace", 2, 1, 1, T, dk, dk, c, dtype, "scaled", 7)
+    _, dev = device_inputs(w)
+    expand = lambda x: x.expand(B, H, T, dk).contiguous()
+    k, v = expand(dev["k"]), expand(dev["v"])
+    la = torch.log(torch.rand(B * H, T, generator=torch.Generator(device="cuda").manual_seed(2), device="cuda") * 0.1 + 0.9)
+    plan = binding.SmatPlan(B, H, T, dk, dk, 2, c, dtype, flags=binding.FLAG_GATED if gated else 0)
+    caches = [plan.decode_cache(), plan.decode_cache()]
+    for cache in caches:
+        if gated:
+            plan.decode_begin_gated(k, v, la, cache)
+        else:
+            plan.decode_begin(k, v, cache)
+    for t in range(256, 288):
+        rows = {n: torch.randn(B, H, dk, generator=torch.Generator(device="cuda").manual_seed(3 * t + i), device="cuda").to(k.dtype)
+                for i, n in enumerate("qkv")}
+        mine = {n: x.clone() for n, x in rows.items()}
+        if gated:
+            a = plan.decode_step_gated(rows["q"], rows["k"], rows["v"], la[:, t].contiguous(), t, caches[0])
+            b = plan.decode_step_gated(mine["q"], mine["k"], mine["v"], la[:, t].contiguous(), t, caches[1], o=mine[place])
+        else:
+            a = plan.decode_step(rows["q"], rows["k"], rows["v"], t, caches[0])
+            b = plan.decode_step(mine["q"], mine["k"], mine["v"], t, caches[1], o=mine[place])
+        assert b.data_ptr() == mine[place].data_ptr() and torch.equal(a, b), t
+    assert torch.equal(caches[0], caches[1])
