@@ -251,11 +251,23 @@ void tile_rows(Ctx& cx, const char* name, int score_dim, int out_dim, std::initi
   a.T = pl->T; a.c = (int)pl->c; a.NC = (int)pl->NC; a.lam = lam;
   SMAT_TRY(cx, name, smat_launch_tile_rows(a, pl->dtype == SMAT_BF16, score_dim, out_dim, pl->bh, cx.st));
 }
-// dQ, dK (score products over d_v, d_k columns out) and dV (the other way round): one launch when d_k = d_v.
+// dQ, dK (score products over d_v, d_k columns out) and dV (the other way round): one launch when d_k = d_v and no
+// gradient takes the place of an operand; else one after the other, so that dK may be V's array and dV any of the four.
 void adjoint_tiles(Ctx& cx, const char* name, const SmatTileJob& dq, const SmatTileJob& dk, const SmatTileJob& dv,
                    const float* lam) {
   const smat_plan* pl = cx.pl;
-  if (pl->r == pl->p) {
+  const size_t rows = (size_t)pl->bh * pl->T * (pl->dtype == SMAT_BF16 ? 2 : 4);
+  bool in_place = false;
+  for (const SmatTileJob* j : {&dq, &dk, &dv}) {
+    const size_t out = rows * (j == &dv ? pl->p : pl->r);
+    in_place = in_place || smat_overlap(j->out, out, dv.p1, rows * pl->r) || smat_overlap(j->out, out, dv.p2, rows * pl->r) ||
+               smat_overlap(j->out, out, dq.p1, rows * pl->p) || smat_overlap(j->out, out, dq.p2, rows * pl->p);   // K, Q, dO, V
+  }
+  if (in_place) {
+    tile_rows(cx, name, pl->p, pl->r, {dq}, lam);
+    tile_rows(cx, name, pl->p, pl->r, {dk}, lam);
+    tile_rows(cx, name, pl->r, pl->p, {dv}, lam);
+  } else if (pl->r == pl->p) {
     tile_rows(cx, name, pl->p, pl->r, {dq, dk, dv}, lam);
   } else {
     tile_rows(cx, name, pl->p, pl->r, {dq, dk}, lam);

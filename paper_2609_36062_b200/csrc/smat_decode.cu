@@ -116,11 +116,6 @@ __global__ void __launch_bounds__(DEC_THREADS) decode_step_kernel(const T* q, co
   if (log_a && blockIdx.x == 0 && tid == 0) log_g[bh] = lg;
 }
 
-bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
-  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
-  return x < y + b_bytes && y < x + a_bytes;
-}
-
 template <typename T, typename TU>
 cudaError_t launch_step(const void* q, const void* k, const void* v, void* o, float* S, const void* U, int64_t type,
                         int64_t types, int r, int p, int bh, cudaStream_t st, const float* log_a, float* log_g) {
@@ -128,7 +123,7 @@ cudaError_t launch_step(const void* q, const void* k, const void* v, void* o, fl
   const unsigned slices = (unsigned)(p / DEC_COLS);
   // o in the place of q or k (o in the place of v needs nothing: a CTA reads just the columns that it writes)
   const size_t in = (size_t)bh * r * sizeof(T), out = (size_t)bh * p * sizeof(T);
-  const int together = log_a || overlap(o, out, q, in) || overlap(o, out, k, in);
+  const int together = log_a || smat_overlap(o, out, q, in) || smat_overlap(o, out, k, in);
   return smat_launch_pdl_cluster(kernel, dim3(slices, (unsigned)bh), DEC_THREADS, 0, together ? slices : 1u, st,
                                  static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v),
                                  static_cast<T*>(o), S, static_cast<const TU*>(U), type, types, p, log_a, log_g, together);

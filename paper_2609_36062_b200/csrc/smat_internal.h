@@ -59,6 +59,12 @@ SMAT_HD SmatTokens smat_group_tokens(const SmatGroupSpec& s, int64_t bh, int64_t
   return r;
 }
 
+// Whether two arrays share memory.
+inline bool smat_overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return x < y + b_bytes && y < x + a_bytes;
+}
+
 // ---- within-chunk tiles on the fp32 ALUs ------------------------------------------------------------
 // Out[i] = Σ_j X_ij P3_j + P4_i · St (+ acc[i] for rows acc_lo <= t < acc_hi), X_ij = P1_i · P2_j for j <= i (upper:
 // j >= i) of the same chunk.  P1, P2, P4 have score_dim columns, P3, acc and Out out_dim; the states are
@@ -77,7 +83,9 @@ struct SmatTileArgs {
   int64_t T;
   int c, NC;
   const float* lam;                // gated variant: prefix sums of the log-gates [bh][T]; X_ij is multiplied by the decay
+  int together;                    // set by the launcher: an output shares memory with its job's P2 or P3
 };
+// The output of a job may be the array of one of that job's operands (row for row).
 cudaError_t smat_launch_tile_rows(const SmatTileArgs& a, int bf16, int score_dim, int out_dim, int bh, cudaStream_t st);
 
 // Exclusive scans of per-chunk states [bh][NC][state] in place, over up to two independent chunk ranges each;

@@ -208,6 +208,9 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) tile_rows_kernel(const __grid
       }
     }
   }
+  // out in the place of P2 or P3, whose rows every row block of the chunk reads: the blocks are a cluster then, and none
+  // stores before all have read
+  if (a.together) asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
 #pragma unroll
   for (int r = 0; r < RPT; ++r) {
     const int m = rg * RPT + r;
@@ -343,12 +346,18 @@ __global__ void mask_kernel(uint8_t* mask, const SmatGeo geo) {
 }  // namespace
 
 template <typename T, int SD, int OD>
-static cudaError_t launch_tile_rows(const SmatTileArgs& a, int bh, cudaStream_t st) {
+static cudaError_t launch_tile_rows(SmatTileArgs a, int bh, cudaStream_t st) {
   constexpr int smem = TileLayout<T, SD, OD>::SMEM;
   cudaError_t err = cudaFuncSetAttribute(tile_rows_kernel<T, SD, OD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
-  const dim3 grid((unsigned)(a.jobs * a.NC * ((a.c + ROWS - 1) / ROWS)), (unsigned)bh);
-  return smat_launch_pdl(tile_rows_kernel<T, SD, OD>, grid, TILE_THREADS, smem, st, a);
+  const unsigned blocks = (unsigned)((a.c + ROWS - 1) / ROWS);
+  const size_t rows = (size_t)bh * a.T * sizeof(T);
+  a.together = 0;
+  for (int j = 0; j < a.jobs; ++j)
+    if (smat_overlap(a.job[j].out, rows * OD, a.job[j].p2, rows * SD) || smat_overlap(a.job[j].out, rows * OD, a.job[j].p3, rows * OD))
+      a.together = 1;
+  const dim3 grid((unsigned)(a.jobs * a.NC) * blocks, (unsigned)bh);
+  return smat_launch_pdl_cluster(tile_rows_kernel<T, SD, OD>, grid, TILE_THREADS, smem, a.together ? blocks : 1u, st, a);
 }
 
 cudaError_t smat_launch_tile_rows(const SmatTileArgs& a, int bf16, int score_dim, int out_dim, int bh, cudaStream_t st) {

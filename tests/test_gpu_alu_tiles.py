@@ -47,3 +47,24 @@ def test_forward_and_gradients(d, T, dk, dv, c, dtype, gated):
         for name, got, ref in zip(("O", "dQ", "dK", "dV"), (O,) + tuple(grads), refs):
             e = rel_err(to_numpy64(got[0, h]), ref)
             assert e <= tol, (name, h, e)
+
+
+@pytest.mark.parametrize("d,T,dim,c,dtype", [(2, 2048, 64, 64, "f32"), (1, 2048, 128, 128, "f32"), (3, 1536, 64, 128, "bf16")])
+def test_outputs_in_the_place_of_operands(d, T, dim, c, dtype):
+    """O may be written over Q, K or V, dK over V and dV over any operand: the row blocks of a chunk share K's and V's
+    rows, so none may store before all have read."""
+    g = torch.Generator(device="cuda").manual_seed(8)
+    dt = torch.float32 if dtype == "f32" else torch.bfloat16
+    x = {n: (torch.randn(1, 8, T, dim, generator=g, device="cuda") / dim ** 0.25).to(dt) for n in ("q", "k", "v", "do")}
+    plan = binding.SmatPlan(1, 8, T, dim, dim, d, c, dtype)
+    O = plan.forward(x["q"], x["k"], x["v"])
+    grads = plan.backward(x["q"], x["k"], x["v"], x["do"])
+    for place in ("q", "k", "v"):
+        y = {n: t.clone() for n, t in x.items()}
+        assert torch.equal(plan.forward(y["q"], y["k"], y["v"], O=y[place]), O), place
+    for dk_place, dv_place in ((None, "do"), (None, "v"), (None, "k"), (None, "q"), ("v", "do")):
+        y = {n: t.clone() for n, t in x.items()}
+        got = plan.backward(y["q"], y["k"], y["v"], y["do"], dK=y.get(dk_place), dV=y[dv_place])
+        plan.check_status()
+        for name, a, b in zip(("dQ", "dK", "dV"), got, grads):
+            assert torch.equal(a, b), (name, dk_place, dv_place)
