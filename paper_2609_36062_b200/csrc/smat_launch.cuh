@@ -3,11 +3,13 @@
 // pdl_wait().  Every kernel launched this way calls pdl_wait() in every thread that touches global memory, before it
 // does, and in at least one thread of every CTA, also of one that has nothing to do: a launch whose CTAs all leave without
 // it completes beside the kernel before, and completion would no longer be transitive along the stream.  pdl_trigger()
-// lets the next kernel start its own set-up.
-// Two rules follow.  A kernel that takes tensor memory triggers only after it has it: the next kernel's CTAs start once
-// all of this one's have triggered, and a CTA that took the columns first and then waited for this kernel would never
-// give them back.  And data of earlier kernels is read with plain loads, not through __ldg or const __restrict__ pointers:
-// the compiler may move such loads of "constant" memory above the wait.
+// lets the next kernel start its own set-up.  Three rules follow.
+// A bounded wait (mbar_wait) for anything that another thread brings about after its pdl_wait() comes after a pdl_wait()
+// of its own: the limit counts this kernel's time, not what is left of the kernel before.
+// A kernel that takes tensor memory triggers only after it has it: the next kernel's CTAs start once all of this one's have
+// triggered, and a CTA that took the columns first and then waited for this kernel would never give them back.
+// Data of earlier kernels is read with plain loads, not through __ldg or const __restrict__ pointers: the compiler may
+// move such loads of "constant" memory above the wait.
 #pragma once
 #include <cuda_runtime.h>
 

@@ -254,6 +254,7 @@ __global__ void __launch_bounds__(THREADS, 1) radon_slab_kernel(const __grid_con
       }
     }
   } else if (warp == MMA1_WARP) {
+    pdl_wait();
     const bool leader = elect_one();
     const uint64_t dF = make_desc(smem_u32(sF), SLOT, 1024), dW = make_desc(smem_u32(sW), SLOT, 1024);
     Ring<NF> f;
@@ -282,6 +283,7 @@ __global__ void __launch_bounds__(THREADS, 1) radon_slab_kernel(const __grid_con
       }
     }
   } else if (warp == MMA2_WARP) {
+    pdl_wait();
     const bool leader = elect_one();
     const uint64_t d0 = make_desc(smem_u32(sW), SLOT, 1024);
     Ring<ACC2> a;
@@ -327,6 +329,7 @@ __global__ void __launch_bounds__(THREADS, 1) radon_slab_kernel(const __grid_con
     }
   } else if (warp >= ALU_WARP) {
     // Output indices 128 ..: the last lines of the extra class.  A warp has one line, a lane two entries.
+    pdl_wait();
     const int u = Q - ALU_ROWS + (warp - ALU_WARP);
     int at[Q];                                            // the line's rows (of an F image, and of G)
 #pragma unroll
@@ -379,6 +382,7 @@ __global__ void __launch_bounds__(THREADS, 1) radon_slab_kernel(const __grid_con
       }
     }
   } else {
+    pdl_wait();
     const int grp = warp >> 2, qd = warp & 3;
     const int n = qd * 32 + lane, x = n % Q, y = n / Q;     // output index (x, slope y); y = q: line x of the extra class
     const uint32_t from = (uint32_t)(qd * 32) << 16;

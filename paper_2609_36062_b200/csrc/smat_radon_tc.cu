@@ -485,6 +485,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
     // ---- MMA issuers: the two threads take the items alternately, so that the issue latency of one item (waits,
     // MMAs, commits: more than the tensor pipe needs for it) overlaps with the other thread's item.  Both phases
     // share R and the slot layout, so the issuers only count items. ---------------------------------------------
+    if (EARLY) pdl_wait();
     const uint32_t me = (uint32_t)(warp - MMA_WARP);
     if (tma_out && me == 1 && prm.nslots == 1) store_role();
     constexpr uint32_t idesc = make_idesc(TILE_ROWS, 128, 0, 1);   // A from tensor memory (R), B MN-major (image rows)

@@ -224,9 +224,10 @@ __global__ void __launch_bounds__(THREADS, 1) radon_wide_kernel(const __grid_con
         v[16 + c] = (c <= 14 ? w.y << (14 - c) : w.y >> 1) & 0x40004000u;
       }
       const uint32_t was = n - A_RING;
-      if (n >= A_RING &&
-          !mbar_wait_warp(a_empty + (was & (A_BARS - 1)), (was / A_BARS) & 1, wc))
-        break;
+      if (n >= A_RING) {   // (the first tiles of R are made while the kernel before runs on)
+        if (n < A_RING + GEN_GROUPS) pdl_wait();
+        if (!mbar_wait_warp(a_empty + (was & (A_BARS - 1)), (was / A_BARS) & 1, wc)) break;
+      }
       fence_after_sync();
       tmem_st32(tmem_base + ((uint32_t)(qd * 32) << 16) + A_COL + (n & (A_RING - 1)) * 32, v);
       tmem_st_wait();
@@ -274,6 +275,7 @@ __global__ void __launch_bounds__(THREADS, 1) radon_wide_kernel(const __grid_con
     // ---- MMA issuers: one warp per tile of the group (its waits, MMAs and commits take longer than the tensor pipe
     // needs for a tile's share of a slot, so one thread for all three tiles would hold the pipe up).  The whole warp
     // walks the loop, so that addresses and descriptors stay in uniform registers; one elected lane issues. ------------
+    pdl_wait();
     const int t = warp - MMA_WARP;
     if (t < nt) {
       constexpr uint32_t idesc = make_idesc(ROWS, NE, 0, 1);    // R from tensor memory, image rows MN-major
