@@ -242,16 +242,9 @@ __global__ void __launch_bounds__(THREADS, 1) radon_slab_kernel(const __grid_con
       if (!ok) break;
       pre = 0;
     }
-    if (!ok && leader) {   // given up: shared memory must outlive the copies into it
-      const long long since = clock64();
-      for (int s = 0; s < NF; ++s) {   // the slots' last loads (a barrier without any lets the parity pass)
-        while (!mbar_try_wait(f_full + f.at, f.par ^ 1) && clock64() - since < wc.limit) {}
-        f.next();
-      }
-      for (int s = 0; s < PRE; ++s) {
-        const uint32_t loads = k + (s < pre ? 1 : 0);
-        while (loads && !mbar_try_wait(p_full + s, (loads - 1) & 1) && clock64() - since < wc.limit) {}
-      }
+    if (leader) {
+      ring_landed(f_full, NF, f.at, f.par ^ 1, wc);
+      for (int s = 0; s < PRE; ++s) landed(p_full + s, (k + (s < pre ? 0 : 1)) & 1, wc);   // k, or k + 1 loads
     }
   } else if (warp == MMA1_WARP) {
     pdl_wait();

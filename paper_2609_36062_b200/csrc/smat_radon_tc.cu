@@ -481,6 +481,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
         }
       }
     }
+    ring_landed(full, (uint32_t)prm.ring, slot, first_lap ? 1u : par, wc);
   } else if (warp >= MMA_WARP && warp < ALU_WARP && lane == 0) {
     // ---- MMA issuers: the two threads take the items alternately, so that the issue latency of one item (waits,
     // MMAs, commits: more than the tensor pipe needs for it) overlaps with the other thread's item.  Both phases

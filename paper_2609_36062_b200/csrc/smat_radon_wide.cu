@@ -271,6 +271,7 @@ __global__ void __launch_bounds__(THREADS, 1) radon_wide_kernel(const __grid_con
         if (++slot == (uint32_t)bbuf) { slot = 0; par ^= 1; }
       }
     }
+    if (leader) ring_landed(b_full, (uint32_t)bbuf, slot, par, wc);
   } else if (warp >= MMA_WARP) {
     // ---- MMA issuers: one warp per tile of the group (its waits, MMAs and commits take longer than the tensor pipe
     // needs for a tile's share of a slot, so one thread for all three tiles would hold the pipe up).  The whole warp

@@ -234,9 +234,11 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
     tc::fence_barrier_init();
   }
   pdl_wait();
+  uint32_t loads = 0;   // started states (thread 0)
   if (tid == 0 && (int64_t)blockIdx.x < items) {
     tc::mbar_expect_tx(bar, SBYTES);
     bulk_load(Sb, state_of(blockIdx.x), SBYTES, bar);
+    ++loads;
   }
   prefetch_x(blockIdx.x, 0);
   __syncthreads();
@@ -326,9 +328,11 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
       if (nxt < items && !*cta_abort) {
         tc::mbar_expect_tx(bar, SBYTES);
         bulk_load(Sb, state_of(nxt), SBYTES, bar);
+        ++loads;
       }
     }
   }
+  if (tid == 0) tc::landed(bar, (loads + 1) & 1, wc);
   cp_async_wait<0>();
 }
 

@@ -233,16 +233,7 @@ __global__ void __launch_bounds__(D3Layout<Q>::THREADS, 1) tabulate_d3_f32_kerne
     ok = __all_sync(0xffffffffu, ok);
     __syncwarp();
     if (ok) ok = __all_sync(0xffffffffu, mbar_wait(slab_full + buf, (ks / NBUF) & 1, wc));
-    if (!ok) {
-      if (lane == 0) {   // shared memory must outlive the copies into it
-        for (uint32_t b = 0; b < NBUF; ++b) {
-          const uint32_t last = started[b];
-          const long long since = clock64();
-          while (last != 0xffffffffu && !mbar_try_wait(slab_full + b, (last / NBUF) & 1) && clock64() - since < wc.limit) {}
-        }
-      }
-      break;
-    }
+    if (!ok) break;
     const uint8_t* mine = smem + buf * L::SLAB_BYTES + lane * (L::EPT * 4);
     // After its last read a task counts itself done; the one that completes the slab's count owns the buffer and starts
     // the load of the slab NBUF further on (every read of the buffer has returned its value by then).
@@ -259,6 +250,9 @@ __global__ void __launch_bounds__(D3Layout<Q>::THREADS, 1) tabulate_d3_f32_kerne
     if (task + 1 < L::TASKS) d3_heavy_task<Q, V>(mine, u, prm.rp, task, release);
     else d3_light_task<Q, V>(mine, u, prm.rp, release);
   }
+  if (lane == 0 && *cta_abort)   // waits were given up: the last load into every buffer has landed all the same
+    for (uint32_t b = 0; b < NBUF; ++b)
+      if (started[b] != 0xffffffffu) landed(slab_full + b, (started[b] / NBUF) & 1, wc);
 }
 
 template <int Q>

@@ -85,7 +85,8 @@ __global__ void __launch_bounds__(192) chunk_scan_tc_kernel(const __grid_constan
   if (warp == 4 && lane == 0) {
     prefetch_tmap(&tmK);
     prefetch_tmap(&tmV);
-    for (int it = 0; it + 1 < hi - lo; ++it) {  // the last visited tile's own sum is never read
+    int it = 0;
+    for (; it + 1 < hi - lo; ++it) {  // the last visited tile's own sum is never read
       const int b = prm.reverse ? hi - 1 - it : lo + it, s = it % SCAN_STAGES;
       if (it >= SCAN_STAGES && !mbar_wait(empty + s, ((it / SCAN_STAGES) - 1) & 1, wc)) break;
       uint8_t* st = smem + s * SCAN_STAGE_BYTES;
@@ -95,6 +96,7 @@ __global__ void __launch_bounds__(192) chunk_scan_tc_kernel(const __grid_constan
       tma_load_2d(st + BOX_BYTES, &tmK, HALF, row, full + s);
       tma_load_2d(st + 2 * BOX_BYTES, &tmV, half * HALF, row, full + s);
     }
+    ring_landed(full, SCAN_STAGES, it % SCAN_STAGES, (it / SCAN_STAGES + 1) & 1, wc);
   } else if (warp == 5 && lane == 0) {
     constexpr uint32_t idesc = make_idesc(TILE, HALF, 1, 1);
     for (int it = 0; it + 1 < hi - lo; ++it) {
@@ -303,6 +305,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) tile_product_tc_kernel(const 
       }
       mma_commit(bar_o);
     }
+    landed(bar_qk, 0, wc);
+    landed(bar_vs, 0, wc);
   } else if (warp < TILE_EPI_WARPS) {
     const int qd = warp & 3, part = warp >> 2;
     const int m = qd * 32 + lane;    // row inside the tile = TMEM lane
@@ -521,19 +525,32 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) bwd_tile_fused_tc_kernel(con
       tma_load_2d(dst, map, 0, row, bar);
       tma_load_2d(dst + BOX_BYTES, map, HALF, row, bar);
     };
+    int begun = 0;                             // operands of the tile whose load has been started
     for (uint32_t tile = blockIdx.x; tile < prm.tiles && ok; tile += gridDim.x, prev ^= 1) {
       const int row = (int)(tile * TILE);      // tokens and states alike: both are [heads][tiles][128 rows]
+      begun = 0;
       if (!wait(e_v)) break;
       if (leader) { mbar_expect_tx(f_v, 2 * BOX_BYTES); load(sV, &tmV, row, f_v); }
+      begun = 1;
       if (!wait(e_d)) break;
       if (leader) { mbar_expect_tx(f_d, 2 * BOX_BYTES); load(sD, &tmDb, row, f_d); }
+      begun = 2;
       if (!wait(e_qk) || (GATED && !wait(o_qk))) break;
       if (leader) { mbar_expect_tx(f_qk, 4 * BOX_BYTES); load(sQ, &tmQ, row, f_qk); load(sK, &tmK, row, f_qk); }
+      begun = 3;
       if (!wait(e_gs)) break;
       if (leader) {
         mbar_expect_tx(f_g, 2 * BOX_BYTES); load(sG, &tmG, row, f_g);
         mbar_expect_tx(f_s, 2 * BOX_BYTES); load(sS, &tmSin, row, f_s);
       }
+    }
+    if (leader) {   // prev: the last tile's parity, or that of the tile before the one that was given up
+      if (ok) begun = 0;
+      landed(f_v, begun > 0 ? prev ^ 1 : prev, wc);
+      landed(f_d, begun > 1 ? prev ^ 1 : prev, wc);
+      landed(f_qk, begun > 2 ? prev ^ 1 : prev, wc);
+      landed(f_g, prev, wc);
+      landed(f_s, prev, wc);
     }
   } else if (warp == FUSED_EPI_WARPS + 1) {
     const bool leader = elect_one();
@@ -856,7 +873,8 @@ __global__ void __launch_bounds__(192) segment_state_tc_kernel(const __grid_cons
   pdl_wait();
   const uint32_t tmem_d = *tmem_slot;
   if (warp == 4 && lane == 0) {
-    for (int it = 0; it < Lc; ++it) {
+    int it = 0;
+    for (; it < Lc; ++it) {
       const int s = it % SEG_STATE_STAGES;
       if (it >= SEG_STATE_STAGES && !mbar_wait(empty + s, ((it / SEG_STATE_STAGES) - 1) & 1, wc)) break;
       uint8_t* st = smem + s * 4 * BOX_BYTES;
@@ -868,6 +886,7 @@ __global__ void __launch_bounds__(192) segment_state_tc_kernel(const __grid_cons
       tma_load_2d(st + 2 * BOX_BYTES, &tmV, 0, row, full + s);
       tma_load_2d(st + 3 * BOX_BYTES, &tmV, HALF, row, full + s);
     }
+    ring_landed(full, SEG_STATE_STAGES, it % SEG_STATE_STAGES, (it / SEG_STATE_STAGES + 1) & 1, wc);
   } else if (warp == 5 && lane == 0) {
     constexpr uint32_t idesc = make_idesc(TILE, TILE, 1, 1);
     bool ok = true;
@@ -1007,7 +1026,8 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
   if (warp == SEG_EPI_WARPS && lane == 0) {
     const CUtensorMap *mq = &maps.q[blk], *mk = &maps.k[blk], *mv = &maps.v[blk];
     const int row_first = (int)((tile0 - (blk ? prm.cut.tiles0 : 0)) * TILE);   // row inside the block
-    for (int it = 0; it < Lc; ++it) {
+    int it = 0, qk = 0;   // tiles whose loads have been started, and whose Q and K have
+    for (; it < Lc; ++it) {
       const int s = it & 1;
       if (it >= 2 && !mbar_wait(empty + s, ((it >> 1) - 1) & 1, wc)) break;
       uint8_t* st = smem + s * Lay::STAGE;
@@ -1019,6 +1039,7 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
       tma_load_3d(st + BOX_BYTES, mq, HALF, row, bh, full + s);
       tma_load_3d(st + 2 * BOX_BYTES, mk, 0, row, bh, full + s);
       tma_load_3d(st + 3 * BOX_BYTES, mk, HALF, row, bh, full + s);
+      ++qk;
       if (SPLIT) {
         if (it >= 1 && !mbar_wait(vempty, (it - 1) & 1, wc)) break;
         mbar_expect_tx(vfull, 2 * BOX_BYTES);
@@ -1026,6 +1047,8 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
       tma_load_3d(sv, mv, 0, row, bh, bv);
       tma_load_3d(sv + BOX_BYTES, mv, HALF, row, bh, bv);
     }
+    ring_landed(full, 2, qk & 1, ((qk >> 1) + 1) & 1, wc);
+    if (SPLIT) landed(vfull, (it + 1) & 1, wc);
   } else if (warp == SEG_EPI_WARPS + 1 && lane == 0) {
     constexpr uint32_t idesc_sc = make_idesc(TILE, TILE, 0, 0);   // Q Kᵀ: both K-major
     constexpr uint32_t idesc_o = make_idesc(TILE, TILE, 0, 1);    // A K-major (Q or P), B MN-major (S or V)
@@ -1431,8 +1454,9 @@ __global__ void __launch_bounds__(160) state_read_tc_kernel(const __grid_constan
       tma_load_2d(sB + BOX_BYTES, &tmU, HALF, row, bar_u);
     };
     uint32_t n_item = 0, n_pass = 0;  // completed uses of bar_u and of bar_a / bar_d / bar_e
+    uint32_t loads = 0;               // started states
     bool ok = true;
-    if (cur.valid()) load_state(cur.item);
+    if (cur.valid()) { load_state(cur.item); ++loads; }
     while (cur.valid() && ok) {
       if (cur.first()) ok = mbar_wait(bar_u, n_item & 1, wc);
       if (ok) ok = mbar_wait(bar_a, n_pass & 1, wc);
@@ -1462,9 +1486,10 @@ __global__ void __launch_bounds__(160) state_read_tc_kernel(const __grid_constan
       ++n_pass;
       if (was_last) {
         ++n_item;
-        if (ok && cur.valid()) load_state(cur.item);          // travels while the product is written out
+        if (ok && cur.valid()) { load_state(cur.item); ++loads; }   // travels while the product is written out
       }
     }
+    landed(bar_u, (loads + 1) & 1, wc);
   }
   fence_before_sync();
   __syncthreads();

@@ -78,6 +78,19 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const 
   return false;
 }
 
+// A producer leaves only when its copies have landed: shared memory must outlive them, also when waits were given up (and
+// the next kernel's CTAs may take it over at once).  Bounded like every wait.
+__device__ __forceinline__ void landed(uint64_t* bar, uint32_t parity, const WaitCtx& w) {
+  const long long start = clock64();
+  while (!mbar_try_wait(bar, parity) && clock64() - start < w.limit) {}
+}
+// The same for a ring of `slots` "full" barriers whose next load would go to slot `next`.  par: what a fresh "empty"
+// barrier passes (1) on the first lap, the other parity on the second, and so on; the slots from `next` on were last
+// loaded a lap earlier, on the first lap never (their barriers let that parity pass).
+__device__ __forceinline__ void ring_landed(uint64_t* full, uint32_t slots, uint32_t next, uint32_t par, const WaitCtx& w) {
+  for (uint32_t s = 0; s < slots; ++s) landed(full + s, s < next ? par ^ 1 : par, w);
+}
+
 // ---- TMA (no multicast: every CTA fetches its own tiles) ---------------------------------------------------
 __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
   asm volatile(
