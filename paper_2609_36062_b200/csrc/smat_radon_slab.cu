@@ -87,9 +87,6 @@ __device__ __forceinline__ bool elect_one() {
       : "=r"(pred));
   return pred != 0;
 }
-__device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity, const WaitCtx& w) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, w));
-}
 __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, const void* smem_src, int c0, int c1, int c2) {
   asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];"
                ::"l"(map), "r"(smem_u32(smem_src)), "r"(c0), "r"(c1), "r"(c2)
@@ -218,7 +215,7 @@ __global__ void __launch_bounds__(THREADS, 1) radon_slab_kernel(const __grid_con
       int e0;
       const int head = slab_head(k, e0);
       auto ring_image = [&](int x2) {
-        ok = wait_warp(f_empty + f.at, f.par ^ 1, wc);
+        ok = mbar_wait_warp(f_empty + f.at, f.par ^ 1, wc);
         if (!ok) return;
         if (leader) {
           mbar_expect_tx(f_full + f.at, TILE_BYTES);
@@ -230,7 +227,7 @@ __global__ void __launch_bounds__(THREADS, 1) radon_slab_kernel(const __grid_con
       for (int x2 = PRE; x2 < PRE + NF && ok; ++x2) ring_image(x2);   // (the ring's slots are free first)
 #pragma unroll 1
       for (pre = 0; pre < PRE && ok; ++pre) {
-        if (k) ok = wait_warp(u_read + pre, (k - 1) & 1, wc);
+        if (k) ok = mbar_wait_warp(u_read + pre, (k - 1) & 1, wc);
         if (!ok) break;
         if (leader) {
           mbar_expect_tx(p_full + pre, TILE_BYTES);
@@ -282,7 +279,7 @@ __global__ void __launch_bounds__(THREADS, 1) radon_slab_kernel(const __grid_con
     Ring<ACC2> a;
     bool ok = true;
     for (uint32_t k = 0; k < my_slabs && ok; ++k) {
-      ok = wait_warp(w_ready, k & 1, wc);
+      ok = mbar_wait_warp(w_ready, k & 1, wc);
 #pragma unroll 1
       for (int img = 0; img < NW && ok; ++img) {
         ok = __all_sync(0xffffffffu, mbar_wait(empty2 + a.at, a.par ^ 1, wc));
@@ -334,7 +331,7 @@ __global__ void __launch_bounds__(THREADS, 1) radon_slab_kernel(const __grid_con
 #pragma unroll 1
       for (int t = 0; t < EARLY && ok; ++t) {
         const bool ring = in_ring(t);
-        ok = ring ? wait_warp(f_full + f.at, f.par, wc) : wait_warp(p_full + t - NF, k & 1, wc);
+        ok = ring ? mbar_wait_warp(f_full + f.at, f.par, wc) : mbar_wait_warp(p_full + t - NF, k & 1, wc);
         if (!ok) break;
         const uint32_t here = rows_sum(ring ? sF + f.at * SLOT : sW + (t - NF) * SLOT, at);
 #pragma unroll
@@ -345,14 +342,14 @@ __global__ void __launch_bounds__(THREADS, 1) radon_slab_kernel(const __grid_con
         if (lane == 0 && t + 1 == EARLY) mbar_arrive(w_free);
         if (ring) f.next();
       }
-      if (ok) ok = wait_warp(w_free, k & 1, wc);
+      if (ok) ok = mbar_wait_warp(w_free, k & 1, wc);
       if (!ok) break;
       uint8_t* g = sW + Q * SLOT;
 #pragma unroll
       for (int t = 0; t < EARLY; ++t) *reinterpret_cast<uint32_t*>(g + at[image_at(t)]) = sum[t];
 #pragma unroll
       for (int x2 = EARLY; x2 < Q; ++x2) {
-        if (ok) ok = wait_warp(f_full + f.at, f.par, wc);
+        if (ok) ok = mbar_wait_warp(f_full + f.at, f.par, wc);
         if (ok) {
           *reinterpret_cast<uint32_t*>(g + at[x2]) = rows_sum(sF + f.at * SLOT, at);
           __syncwarp();
@@ -364,7 +361,7 @@ __global__ void __launch_bounds__(THREADS, 1) radon_slab_kernel(const __grid_con
       fence_proxy_async();
       __syncwarp();
       if (lane == 0) mbar_arrive(w_ready);
-      ok = wait_warp(w_ready, k & 1, wc);
+      ok = mbar_wait_warp(w_ready, k & 1, wc);
       if (!ok) break;
       *reinterpret_cast<uint32_t*>(sMini + pair_at(u, lane)) = rows_sum(g, at);
       fence_proxy_async();
@@ -407,12 +404,12 @@ __global__ void __launch_bounds__(THREADS, 1) radon_slab_kernel(const __grid_con
       for (int t = grp; t < Q; t += GROUPS) {
         const uint32_t item = k * Q + t, at = item % ACC1;
         const int x2 = image_at(t);
-        ok = wait_warp(full1 + at, (item / ACC1) & 1, wc);
+        ok = mbar_wait_warp(full1 + at, (item / ACC1) & 1, wc);
         if (!ok) break;
         uint4 w[8];
         read_acc(acc1 + at * 64, empty1 + at, w);
         if (t == grp) {
-          ok = wait_warp(w_free, k & 1, wc);
+          ok = mbar_wait_warp(w_free, k & 1, wc);
           if (!ok) break;
         }
         // W[a3 = y], row (u = x, x2); the extra class: G, row (x2, x3 = x)
@@ -425,12 +422,12 @@ __global__ void __launch_bounds__(THREADS, 1) radon_slab_kernel(const __grid_con
 #pragma unroll 1
       for (int img = grp; img < NW; img += GROUPS) {
         const uint32_t item = k * NW + img, at = item % ACC2;
-        ok = wait_warp(full2 + grp, (item / GROUPS) & 1, wc);
+        ok = mbar_wait_warp(full2 + grp, (item / GROUPS) & 1, wc);
         if (!ok) break;
         uint4 w[8];
         read_acc(acc2 + at * 64, empty2 + at, w);
         if (img == Q) {
-          ok = wait_warp(alu_done, k & 1, wc);                // the ALU warps have read the image that the tile replaces
+          ok = mbar_wait_warp(alu_done, k & 1, wc);                // the ALU warps have read the image that the tile replaces
           if (!ok) break;
         }
         if (y < Q) put_row(sW + img * SLOT, n, w);

@@ -131,12 +131,6 @@ struct ItemIter {
   __device__ __forceinline__ bool closes_phase0() const { return nph > 1 && ph == 0 && img + 1 == im0; }
 };
 
-// All lanes wait: one lane polling and a shuffle cost about a hundred cycles more at every wait (q = 17, d = 3, transposed,
-// 64 heads: 0.64 ms against 0.56; d = 4, 16 heads: 2.25 against 2.21).
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, const WaitCtx& w) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, w));
-}
-
 // Row of the streamed operand that holds input index (lo, line): slot line / sps, then the line's q rows.
 __device__ __forceinline__ int operand_row(const RadonParams& p, int line, int lo) {
   if (line >= p.q) return p.nreg * p.sr + lo;                 // extra class: a slot of its own

@@ -145,12 +145,6 @@ __device__ __forceinline__ bool elect_one() {
   return pred != 0;
 }
 
-// All lanes wait: with one lane polling and a shuffle (and, before that, one warp of four polling for the generators, the
-// others at a named barrier) 16 heads, q = 37, took 0.80 ms instead of 0.69.
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, const WaitCtx& w) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, w));
-}
-
 __global__ void __launch_bounds__(THREADS, 1) radon_wide_kernel(const __grid_constant__ CUtensorMap tm_reg,
                                                                 const __grid_constant__ CUtensorMap tm_vert,
                                                                 const __grid_constant__ WideParams prm) {

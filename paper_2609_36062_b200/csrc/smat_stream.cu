@@ -255,8 +255,7 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
     const float4* S4 = reinterpret_cast<const float4*>(Sb);
     prefetch_x(item + gridDim.x, buf ^ 1);
     cp_async_wait<1>();
-    bool ok = tc::mbar_wait(bar, n & 1, wc);
-    __syncthreads();
+    const bool ok = __syncthreads_and(tc::mbar_wait(bar, n & 1, wc)) != 0;   // (block-wide barriers follow: all go on, or none)
     for (int64_t k0 = 0; k0 < cnt && ok; k0 += KT) {
       const int kn = (int)((cnt - k0) < KT ? (cnt - k0) : KT);
       for (int idx = tid; idx < KT * xd; idx += 256) {

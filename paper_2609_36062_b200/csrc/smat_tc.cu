@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(192) chunk_scan_tc_kernel(const __grid_constan
         st_global_v8(dst + 2 * j16, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
       }
       if (it + 1 == hi - lo) break;  // every issued MMA has been consumed: nothing is in flight at teardown
-      if (!mbar_wait(dfull + db, (it / SCAN_DBUF) & 1, wc)) break;
+      if (!mbar_wait_warp(dfull + db, (it / SCAN_DBUF) & 1, wc)) break;
       fence_after_sync();
       uint32_t v0[32], v1[32];
       const uint32_t taddr = tmem_base + ((uint32_t)(warp * 32) << 16) + db * HALF;
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) tile_product_tc_kernel(const 
     const int qd = warp & 3, part = warp >> 2;
     const int m = qd * 32 + lane;    // row inside the tile = TMEM lane
     const uint32_t lane_base = (uint32_t)(qd * 32) << 16;
-    if (mbar_wait(bar_sc, 0, wc)) {
+    if (mbar_wait_warp(bar_sc, 0, wc)) {
       fence_after_sync();
       const float lam_m = GATED ? sLam[m] : 0.f;
 #pragma unroll 1
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) tile_product_tc_kernel(const 
       fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_p);   // one arrival per warp
-      if (mbar_wait(bar_o, 0, wc)) {
+      if (mbar_wait_warp(bar_o, 0, wc)) {
         fence_after_sync();
         const int64_t t = (int64_t)b * TILE + m;
         const bool add_lr = t >= prm.add_lo && t < prm.add_hi;
@@ -729,16 +729,16 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) bwd_tile_fused_tc_kernel(con
       // a tile lies on one side of the block boundary
       const bool add_q = prm.lr_q != nullptr && t >= prm.n, add_kv = prm.lr_k != nullptr && t < prm.n;
       uint4 y[4], pk[4];
-      if (!mbar_wait(b_scg, par, wc)) break;
+      if (!mbar_wait_warp(b_scg, par, wc)) break;
       fence_after_sync();
       round_scores(tm_g, pk);
       store_scores(sX, pk, p_g);
-      if (!mbar_wait(b_sca, par, wc)) break;
+      if (!mbar_wait_warp(b_sca, par, wc)) break;
       fence_after_sync();
       round_scores(tm_a, pk);
       if (add_q) fetch(prm.lr_q, y);
       if (add_kv) fetch(prm.lr_k, y);
-      if (!mbar_wait(b_st, par, wc)) break;          // S_in has been read: the rounded A takes its place
+      if (!mbar_wait_warp(b_st, par, wc)) break;          // S_in has been read: the rounded A takes its place
       fence_after_sync();
       if (GATED) {
         scale(tm_dq, row_in);
@@ -748,13 +748,13 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) bwd_tile_fused_tc_kernel(con
       }
       store_scores(sS, pk, p_a);
       if (GATED) {
-        if (!mbar_wait(b_st2, par, wc)) break;
+        if (!mbar_wait_warp(b_st2, par, wc)) break;
         fence_after_sync();
         scale(tm_dv, row_out);
         tmem_st_wait();
         arrive(sl_v);
       }
-      if (!mbar_wait(b_qk, par, wc)) break;
+      if (!mbar_wait_warp(b_qk, par, wc)) break;
       fence_after_sync();
       uint32_t v[32];
       tmem_ld32(tm_dq + lane_base + col0, v);
@@ -769,12 +769,12 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) bwd_tile_fused_tc_kernel(con
         part[cq * TILE + m] = dq - dk;
         arrive(o_qk);
         if (cq == 0) {                               // (the next G is written after these warps' arrival on o_v)
-          if (!mbar_wait(o_qk, par, wc)) break;
+          if (!mbar_wait_warp(o_qk, par, wc)) break;
           prm.dlam[row] = (part[m] + part[TILE + m]) + (part[2 * TILE + m] + part[3 * TILE + m]);
         }
       }
       if (add_kv) fetch(prm.lr_v, y);
-      if (!mbar_wait(b_dv, par, wc)) break;
+      if (!mbar_wait_warp(b_dv, par, wc)) break;
       fence_after_sync();
       tmem_ld32(tm_dv + lane_base + col0, v);
       tmem_ld_wait();
@@ -905,7 +905,7 @@ __global__ void __launch_bounds__(192) segment_state_tc_kernel(const __grid_cons
     }
     if (ok) mma_commit(done);
   } else if (warp < 4) {
-    if (mbar_wait(done, 0, wc)) {
+    if (mbar_wait_warp(done, 0, wc)) {
       fence_after_sync();
       const int i = warp * 32 + lane;
       uint4* dst = reinterpret_cast<uint4*>(prm.totals + (((int64_t)bh * prm.nseg + seg) * TILE + i) * TILE);
@@ -1201,7 +1201,7 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
     for (int it = 0; it < Lc; ++it) {
       uint8_t* stage = smem + (it & 1) * Lay::STAGE;
       // --- scores of this tile -> masked bf16 P (registers), stored once Q and K have been consumed ---
-      if (!mbar_wait(bar_sc, it & 1, wc)) break;
+      if (!mbar_wait_warp(bar_sc, it & 1, wc)) break;
       fence_after_sync();
       uint4 pk[4], plo[4];
       {
@@ -1217,7 +1217,7 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
         pack_row(f, pk);
         if (SPLIT) { remainder(f, pk); pack_row(f, plo); }
       }
-      if (!mbar_wait(bar_qk, it & 1, wc)) break;
+      if (!mbar_wait_warp(bar_qk, it & 1, wc)) break;
       fence_after_sync();
       store_row(stage, pk);
       if (SPLIT) store_row(stage + 2 * BOX_BYTES, plo);
@@ -1242,7 +1242,7 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
 #pragma unroll
         for (int i = 0; i < (SPLIT ? 8 : 4); ++i) y[i] = *(y4 + i);
       }
-      if (!mbar_wait(bar_o, it & 1, wc)) break;
+      if (!mbar_wait_warp(bar_o, it & 1, wc)) break;
       fence_after_sync();
       __nv_bfloat16* dst = prm.O + ((int64_t)bh * prm.T + t) * TILE + col0;
       const uint32_t tmem_o = tmem_o0 + (it & 1) * TILE;
