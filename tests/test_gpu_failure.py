@@ -57,7 +57,11 @@ def test_an_exhausted_device_raises_out_of_memory_error():
     ws = plan.workspace()
     torch.cuda.empty_cache()
     torch.cuda.set_per_process_memory_fraction(1e-6)      # of torch's allocator alone: no further block is granted
+    held = []
     try:
+        with pytest.raises(torch.OutOfMemoryError):       # blocks of this size that the allocator still keeps
+            for _ in range(64):
+                held.append(torch.empty_like(x))
         with pytest.raises(torch.OutOfMemoryError):
             plan.forward(x, x, x, workspace=ws)
     finally:
