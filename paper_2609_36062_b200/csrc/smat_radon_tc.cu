@@ -29,8 +29,8 @@
 //   warps 19, 20   : q = 11 only.  q^2 + q = 132 output indices are one tile of 128 and 4 left over, all of the extra
 //                    class (the sum of one line's q rows): these warps add them up from the ring slot itself, so
 //                    that one CTA covers an image instead of two CTAs loading it twice
-// d = 4 with q <= 11 (forward with q = 11: smat_radon_slab.cu instead): both stages in ONE launch, slab by slab.  Stage 2 of a slab needs stage 1 of every image of the
-// same slab and nothing else, so a CTA keeps the slab's W rows in a private exchange buffer (q^3 + q^2 rows of 128
+// d = 4 with q <= 11 (forward with q = 11: smat_radon_slab.cu instead): both stages in ONE launch, slab by slab.  Stage 2
+// of a slab needs stage 1 of every image of the same slab and nothing else, so a CTA keeps the slab's W rows in a private exchange buffer (q^3 + q^2 rows of 128
 // entries, rewritten for every slab, stored and loaded with the L2 evict-last priority while F and U stream with
 // evict-first) and the full-size W table is never built.  The storing warps make the slab's rows visible (memory
 // fence, proxy fence) and arrive on a barrier the producer waits on before the first stage-2 load.
@@ -40,7 +40,8 @@
 // The kernel exists twice: radon_tc_kernel<false, .> for one stage per launch with every index through the MMAs (q = 17
 // and the small primes), without cache hints, phase tables or ALU warps; radon_tc_kernel<true, .> with them.
 // (The tile-store path is written for several slots per item and several parts and is compiled into both, but the
-// launcher switches it on for q = 11 only: it was measured slower than the direct stores for q = 13 and 17.)
+// launcher switches it on for q = 11 only: it was measured slower than the direct stores for q = 17.  q = 13 and the
+// transposed q = 17 of d = 3 do not come here: see generates_matrix.)
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -812,8 +813,8 @@ cudaError_t launch_radon(int q, int transpose, int nph, const StageSpec* sp, int
   int smem = sh.smem;
   prm.tma_out = 0; prm.mini_bytes = 0;
   prm.lines_pp = sh.rows_pp / q < q ? sh.rows_pp / q : q;
-  // (Tiles of whole lines could leave the same way for q = 13, 17 — the kernel handles several slots per item and
-  // several parts — but there the tile stores were measured 1.6 to 2 times slower than the direct stores.)
+  // (Tiles of whole lines could leave the same way for q = 17 — the kernel handles several slots per item and several
+  // parts — but there the tile stores were measured 1.6 to 2 times slower than the direct stores.)
   if (!transpose && sh.nslots == 1 && sh.sr == TILE_ROWS && sh.parts == 1) {
     const int mini = 2 * ((q + 7) & ~7) * 128, slot = sh.sr * 256;
     int ring = (227 * 1024 - 1024 - 512 - TILE_ROWS * 8) / (slot + mini);
@@ -908,13 +909,55 @@ bool radon_two_stage_fits(int q, int transpose) {
 
 }  // namespace
 
-// 1 when the tensor-core tabulation covers this geometry (d = 3 or 4, q small enough for a resident R).
+// Which of the two kernels runs a stage.  The one that generates R loads an image once where the resident one has two or
+// three CTAs load it, but shares its issue slots and tensor memory with the generators.  Measured (ms, resident against
+// generated): q = 13, d = 3, 32 heads 0.077 / 0.069, transposed 0.089 / 0.072; q = 13, d = 4, 8 heads 0.425 / 0.405,
+// transposed (4 heads) 0.278 / 0.254; q = 17, d = 3, 64 heads 0.256 / 0.272, transposed 0.312 / 0.269; q = 17, d = 4,
+// 8 heads 1.11 / 1.22.  At q <= 11 one CTA covers an image either way.
+static bool generates_matrix(int q, int D, int transpose) { return q == 13 || (q == 17 && D == 2 && transpose); }
+
+// The stages of a tabulation of prime q, D = 2 or 3, without their tables.  fused: those of D = 3 run as one launch with
+// the table between them in the private exchange buffer.
+static int radon_stages(int q, int D, int transpose, bool fused, StageSpec (&sp)[2]) {
+  const int qq = q * q, qqq = qq * q;
+  if (D == 2) {
+    const RadonSide pts = side(qq, 1, q, 0, qq);
+    const RadonSide typ = side(qq + q, 1, q, 0, qq + q, qq, 1, 0, 0);
+    sp[0] = transpose ? stage(typ, pts, 1, nullptr, nullptr) : stage(pts, typ, 1, nullptr, nullptr);
+    return 1;
+  }
+  const int64_t wrows = qqq + qq;
+  const RadonSide f_side = side(qq, 1, qq, q, qqq);                         // image x2, points (x1, x3)
+  const RadonSide w1_side = side(qq + q, 1, qq, q, wrows, qqq, q, 1, 0);    // (u, a3) -> W[a3][x2][u]; extra class -> G[x3][x2]
+  const RadonSide w2_side = side(qq, 1, q, qq, wrows);                      // image a3 (image q: G), points (u, x2)
+  const RadonSide u_side = side(qq + q, 1, q, qq, wrows + q, qqq + qq, 1, 0, q);
+  if (!transpose) {
+    sp[0] = stage(f_side, w1_side, q, nullptr, nullptr, false, fused);
+    sp[1] = stage(w2_side, u_side, q + 1, nullptr, nullptr, fused, false);
+  } else {
+    sp[0] = stage(u_side, w2_side, q + 1, nullptr, nullptr, false, fused);
+    sp[1] = stage(w1_side, f_side, q, nullptr, nullptr, fused, false);
+  }
+  return 2;
+}
+
+// 1 when the tensor-core tabulation covers this geometry (d = 3 or 4): every stage of both directions fits the kernel that
+// would run it.
 int smat_tabulate_tc_supported(const SmatGeo& geo, int64_t state_elems) {
-  if (geo.D != 2 && geo.D != 3) return 0;
-  if (state_elems % 128) return 0;
-  const int qq = geo.q * geo.q;
-  RadonShape a, b;
-  return radon_shape(geo.q, 0, 0, qq + geo.q, &a) && radon_shape(geo.q, 1, 1, qq, &b) ? 1 : 0;
+  if ((geo.D != 2 && geo.D != 3) || state_elems % 128) return 0;
+  const int q = geo.q;
+  if (q > 64) return 0;
+  for (int transpose = 0; transpose < 2; ++transpose) {
+    StageSpec sp[2];
+    const int stages = radon_stages(q, geo.D, transpose, false, sp);
+    for (int i = 0; i < stages; ++i) {
+      RadonShape sh;
+      if (!(generates_matrix(q, geo.D, transpose) ? radon_wide_fits(q, sp[i])
+                                                  : radon_shape(q, transpose, sp[i].in.count > q * q, sp[i].out.count, &sh)))
+        return 0;
+    }
+  }
+  return 1;
 }
 
 // Host-only: 1 when the shared-memory map of every launch shape this prime can take (both directions, with and without
@@ -958,53 +1001,30 @@ int64_t smat_tabulate_tc_scratch_elems(const SmatGeo& geo, int64_t state_elems, 
   return (int64_t)bh * rows * state_elems;
 }
 
-// Which of the two kernels runs a stage.  The one that generates R loads an image once where the resident one has two or
-// three CTAs load it, but shares its issue slots and tensor memory with the generators.  Measured (ms, resident against
-// generated): q = 13, d = 3, 32 heads 0.077 / 0.069, transposed 0.089 / 0.072; q = 13, d = 4, 8 heads 0.425 / 0.405,
-// transposed (4 heads) 0.278 / 0.254; q = 17, d = 3, 64 heads 0.256 / 0.272, transposed 0.312 / 0.269; q = 17, d = 4,
-// 8 heads 1.11 / 1.22.  At q <= 11 one CTA covers an image either way.
-static bool generates_matrix(int q, int D, int transpose) { return q == 13 || (q == 17 && D == 2 && transpose); }
-
 // transpose = 0: in = F [bh][P][rp] bf16, out = U [bh][B][rp] bf16.  transpose = 1: in = Ū [bh][B][rp], out = F̄ [bh][P][rp].
 // scratch: smat_tabulate_tc_scratch_elems bf16 (d = 4 only).  One launch for d = 3; one or two for d = 4.
 cudaError_t smat_launch_tabulate_tc(const void* in, void* out, void* scratch, const SmatGeo& geo, int64_t state_elems,
                                     int bh, int transpose, int* status, cudaStream_t st, int* launches) {
-  const int q = geo.q, qq = q * q, qqq = qq * q;
+  const int q = geo.q;
   *launches = 0;
-  if (geo.D == 2) {
-    const RadonSide pts = side(qq, 1, q, 0, geo.P);
-    const RadonSide typ = side(qq + q, 1, q, 0, geo.B, qq, 1, 0, 0);
-    const StageSpec sp = transpose ? stage(typ, pts, 1, in, out) : stage(pts, typ, 1, in, out);
-    *launches = 1;
-    if (generates_matrix(q, 2, transpose)) return launch_radon_wide(q, transpose, sp, state_elems, bh, status, st);
-    return launch_radon(q, transpose, 1, &sp, state_elems, bh, status, st);
-  }
-  if (geo.D != 3) return cudaErrorInvalidValue;
-  if (!transpose && smat_tabulate_slab_supported(q, state_elems)) {
+  if (geo.D != 2 && geo.D != 3) return cudaErrorInvalidValue;
+  if (geo.D == 3 && !transpose && smat_tabulate_slab_supported(q, state_elems)) {
     *launches = 1;
     return smat_launch_tabulate_slab(in, out, geo, state_elems, bh, status, st);
   }
-  const int64_t wrows = smat_tabulate_tc_scratch_rows(geo);
-  const RadonSide f_side = side(qq, 1, qq, q, geo.P);                       // image x2, points (x1, x3)
-  const RadonSide w1_side = side(qq + q, 1, qq, q, wrows, qqq, q, 1, 0);    // (u, a3) -> W[a3][x2][u]; extra class -> G[x3][x2]
-  const RadonSide w2_side = side(qq, 1, q, qq, wrows);                      // image a3 (image q: G), points (u, x2)
-  const RadonSide u_side = side(qq + q, 1, q, qq, geo.B, qqq + qq, 1, 0, q);
-  const bool fused = radon_two_stage_fits(q, transpose);
+  const bool fused = geo.D == 3 && radon_two_stage_fits(q, transpose);
   StageSpec sp[2];
-  if (!transpose) {
-    sp[0] = stage(f_side, w1_side, q, in, scratch, false, fused);
-    sp[1] = stage(w2_side, u_side, q + 1, scratch, out, fused, false);
-  } else {
-    sp[0] = stage(u_side, w2_side, q + 1, in, scratch, false, fused);
-    sp[1] = stage(w1_side, f_side, q, scratch, out, fused, false);
-  }
+  const int stages = radon_stages(q, geo.D, transpose, fused, sp);
+  sp[0].src = in;
+  sp[stages - 1].dst = out;
+  if (stages == 2) { sp[0].dst = scratch; sp[1].src = scratch; }
   if (fused) {
     *launches = 1;
     return launch_radon(q, transpose, 2, sp, state_elems, bh, status, st);
   }
-  *launches = 2;
-  for (int i = 0; i < 2; ++i) {
-    const cudaError_t err = generates_matrix(q, 3, transpose)
+  *launches = stages;
+  for (int i = 0; i < stages; ++i) {
+    const cudaError_t err = generates_matrix(q, geo.D, transpose)
                                 ? launch_radon_wide(q, transpose, sp[i], state_elems, bh, status, st)
                                 : launch_radon(q, transpose, 1, &sp[i], state_elems, bh, status, st);
     if (err != cudaSuccess) return err;
@@ -1013,12 +1033,16 @@ cudaError_t smat_launch_tabulate_tc(const void* in, void* out, void* scratch, co
 }
 
 int smat_tabulate_d3_wide_supported(const SmatGeo& geo, int64_t state_elems) {
-  return geo.D == 2 && geo.q >= 19 && state_elems % 128 == 0 && radon_wide_fits(geo.q) ? 1 : 0;
+  if (geo.D != 2 || geo.q < 19 || state_elems % 128) return 0;
+  StageSpec sp[2];
+  radon_stages(geo.q, 2, 0, false, sp);
+  return radon_wide_fits(geo.q, sp[0]) ? 1 : 0;
 }
 
 cudaError_t smat_launch_tabulate_d3_wide(const void* in, void* out, const SmatGeo& geo, int64_t state_elems, int bh,
                                          int* status, cudaStream_t st) {
-  const int q = geo.q, qq = q * q;
-  const StageSpec sp = stage(side(qq, 1, q, 0, geo.P), side(qq + q, 1, q, 0, geo.B, qq, 1, 0, 0), 1, in, out);
-  return launch_radon_wide(q, 0, sp, state_elems, bh, status, st);
+  StageSpec sp[2];
+  radon_stages(geo.q, 2, 0, false, sp);
+  sp[0].src = in; sp[0].dst = out;
+  return launch_radon_wide(geo.q, 0, sp[0], state_elems, bh, status, st);
 }

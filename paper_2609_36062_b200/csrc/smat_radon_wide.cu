@@ -379,34 +379,52 @@ static int wide_ring(int nslots, int tiles) {
   return ring > MAX_BBUF ? MAX_BBUF : ring;
 }
 
-bool radon_wide_fits(int q) {
-  const int tiles = (q * q + q + ROWS - 1) / ROWS, nslots = (q * q + SLOT - 1) / SLOT;
-  return q >= 13 && wide_ring(nslots, tiles) >= 4 && 2 * tiles + (tiles + MT - 1) / MT <= 128;
+namespace {
+
+// How a stage's image is cut into ring slots and its outputs into tiles.
+struct WideShape {
+  bool flat;                      // slots of 64 consecutive rows; else whole lines
+  int lines, span, n_reg;         // lines and indices per regular slot, input indices in regular slots
+  int nreg, nslots, tiles, groups, ring, smem;
+};
+
+bool wide_shape(int q, const StageSpec& sp, WideShape* w) {
+  const RadonSide& in = sp.in;
+  const int qq = q * q;
+  if (q < 13) return false;
+  const bool extra = in.count > qq;
+  const bool merged = extra && in.v0 == qq && in.sv_lo == 1 && in.vert_from == 0 && sp.images == 1;   // rows follow on
+  w->flat = in.s_lo == 1 && in.s_hi == q && (!extra || merged);
+  if (!w->flat && q > SLOT) return false;
+  w->lines = w->flat ? 1 : SLOT / q;
+  w->n_reg = w->flat ? in.count : qq;
+  w->span = w->flat ? SLOT : w->lines * q;
+  w->nreg = (w->n_reg + w->span - 1) / w->span;
+  w->nslots = w->nreg + (in.count > w->n_reg ? 1 : 0);
+  w->tiles = (sp.out.count + ROWS - 1) / ROWS;
+  w->groups = (w->tiles + MT - 1) / MT;
+  w->ring = wide_ring(w->nslots, w->tiles);
+  w->smem = wide_fixed_smem(w->nslots, w->tiles) + w->ring * B_SLOT;
+  return w->ring >= 4;
+}
+
+}  // namespace
+
+bool radon_wide_fits(int q, const StageSpec& sp) {
+  WideShape w;
+  return wide_shape(q, sp, &w);
 }
 
 cudaError_t launch_radon_wide(int q, int transpose, const StageSpec& sp, int64_t rp, int bh, int* status, cudaStream_t st) {
   const RadonSide& in = sp.in;
-  const int qq = q * q;
-  if (q < 13 || rp % NE) return cudaErrorInvalidValue;
+  WideShape w;
+  if (!wide_shape(q, sp, &w) || rp % NE) return cudaErrorInvalidValue;
   WideParams prm;
   prm.q = q; prm.transpose = transpose;
   prm.inv_q = (uint32_t)((1ULL << 32) / (uint32_t)q) + 1;
   prm.n_in = in.count;
-  const bool extra = in.count > qq;
-  const bool merged = extra && in.v0 == qq && in.sv_lo == 1 && in.vert_from == 0 && sp.images == 1;   // rows follow on
-  prm.flat = in.s_lo == 1 && in.s_hi == q && (!extra || merged);
-  int sps = 1;
-  if (prm.flat) {
-    prm.n_reg = in.count; prm.span = SLOT;
-  } else {
-    if (q > SLOT) return cudaErrorInvalidValue;
-    sps = SLOT / q;
-    prm.n_reg = qq; prm.span = sps * q;
-  }
-  prm.nreg = (prm.n_reg + prm.span - 1) / prm.span;
-  prm.nslots = prm.nreg + (prm.n_in > prm.n_reg ? 1 : 0);
-  prm.tiles = (sp.out.count + ROWS - 1) / ROWS;
-  prm.groups = (prm.tiles + MT - 1) / MT;
+  prm.flat = w.flat; prm.n_reg = w.n_reg; prm.span = w.span; prm.nreg = w.nreg; prm.nslots = w.nslots;
+  prm.tiles = w.tiles; prm.groups = w.groups; prm.bbuf = w.ring;
   prm.images = sp.images;
   prm.src_heads = bh;
   prm.in_vert_from = in.vert_from;
@@ -419,9 +437,6 @@ cudaError_t launch_radon_wide(int q, int transpose, const StageSpec& sp, int64_t
   const int64_t items = (int64_t)prm.slabs * prm.images;
   if (items * prm.nslots * MT >= (1LL << 31)) return cudaErrorInvalidValue;   // pairs are counted in 32 bits
   prm.items = (uint32_t)items;
-  prm.bbuf = wide_ring(prm.nslots, prm.tiles);
-  if (prm.bbuf < 4) return cudaErrorInvalidConfiguration;
-  const int smem = wide_fixed_smem(prm.nslots, prm.tiles) + prm.bbuf * B_SLOT;
   CUtensorMap tm_reg, tm_vert;
   const int64_t s_img = sp.images > 1 ? in.s_img : in.rows_per_head;   // a size-one dimension keeps its stride valid
   if (prm.flat) {   // (entry of a 64-entry block, row, block, image, head)
@@ -432,7 +447,7 @@ cudaError_t launch_radon_wide(int q, int transpose, const StageSpec& sp, int64_t
   } else {          // (entry, lo, hi, image, head)
     const int64_t sizes[4] = {q, q, sp.images, bh};
     const int64_t strides[4] = {in.s_lo, in.s_hi, s_img, in.rows_per_head};
-    const int box[4] = {q, sps, 1, 1};
+    const int box[4] = {q, w.lines, 1, 1};
     if (!radon_map(&tm_reg, sp.src, rp, 5, sizes, strides, box)) return cudaErrorInvalidValue;
   }
   tm_vert = tm_reg;
@@ -444,12 +459,14 @@ cudaError_t launch_radon_wide(int q, int transpose, const StageSpec& sp, int64_t
     if (!radon_map(&tm_vert, static_cast<const __nv_bfloat16*>(sp.src) + (int64_t)in.v0 * rp, rp, 4, sizes, strides, box))
       return cudaErrorInvalidValue;
   }
-  cudaError_t err = cudaFuncSetAttribute(radon_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t err = cudaFuncSetAttribute(radon_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, w.smem);
   if (err != cudaSuccess) return err;
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t grid = items * prm.groups < sms ? items * prm.groups : sms;   // at least one CTA per group
-  if (grid < 2 * prm.tiles + prm.groups) return cudaErrorInvalidConfiguration;
-  return smat_launch_pdl(radon_wide_kernel, dim3((unsigned)grid), THREADS, smem, st, tm_reg, tm_vert, prm);
+  int64_t grid = items * prm.groups < sms ? items * prm.groups : sms;
+  // Every group of tiles needs a CTA (see first_cta); none waits for another, so that a device with fewer SMs, a slice of
+  // one among them, runs them one after the other.
+  if (grid < 2 * prm.tiles + prm.groups) grid = 2 * prm.tiles + prm.groups;
+  return smat_launch_pdl(radon_wide_kernel, dim3((unsigned)grid), THREADS, w.smem, st, tm_reg, tm_vert, prm);
 }
