@@ -224,7 +224,7 @@ def test_gated_passes_with_the_other_tabulations_of_the_inner_plan(flag):
 @pytest.mark.parametrize("dtype,dk,c", [("f32", 64, 64), ("bf16", 128, 128)])
 def test_rows_before_a_strong_gate_do_not_notice_it(at, dtype, dk, c):
     """One gate of e^-10000 among moderate ones: the rows before it are bit for bit what they are without it (their λ must
-    not lose low bits to a sum that it dominates), and on fp32 plans the whole output stays with the oracle."""
+    not lose low bits to a sum that it dominates), and on fp32 plans the output stays with the oracle."""
     T = 512 if at < 512 else 8192
     w = synth.Workload("g3", 3, 1, 1, T, dk, dk, c, dtype, "scaled", 9)
     host, dev = device_inputs(w)
@@ -239,4 +239,8 @@ def test_rows_before_a_strong_gate_do_not_notice_it(at, dtype, dk, c):
     if dtype == "f32" and T == 512:
         Q64, K64, V64 = (synth.as_float64(w, host[x][0]) for x in ("q", "k", "v"))
         ref = so.gated_forward_dense(Q64, K64, V64, so.dense_mask(T, c, 3), hit[0].astype(np.float64))
-        assert rel_err(to_numpy64(b[0, 0]), ref) <= TOL["f32"]
+        got = to_numpy64(b[0, 0])
+        assert rel_err(got[:at], ref[:at]) <= TOL["f32"]
+        # from the gate on λ itself is near -10000, an fp32 number with steps of 2^-10: each of the two λ of a factor
+        # exp(λ_i - λ_j) is off by up to half a step
+        assert rel_err(got[at:], ref[at:]) <= 2.0 ** -10 + TOL["f32"]
