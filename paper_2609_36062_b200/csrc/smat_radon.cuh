@@ -114,4 +114,5 @@ inline StageSpec stage(const RadonSide& in, const RadonSide& out, int images, co
 
 // One stage with the Radon matrix generated beside the image stream (smat_radon_wide.cu); tables only, no exchange buffer.
 bool radon_wide_fits(int q, const StageSpec& sp);   // whether a stage's slots, tiles and tables fit (host only)
+bool radon_wide_layout_ok(int q, const StageSpec& sp);
 cudaError_t launch_radon_wide(int q, int transpose, const StageSpec& sp, int64_t rp, int bh, int* status, cudaStream_t st);

@@ -960,29 +960,6 @@ int smat_tabulate_tc_supported(const SmatGeo& geo, int64_t state_elems) {
   return 1;
 }
 
-// Host-only: 1 when the shared-memory map of every launch shape this prime can take (both directions, with and without
-// the extra class on the input, with the tile-store variant where the launcher would pick it) passes radon_layout_ok.
-int smat_tabulate_tc_layout_ok(int q) {
-  const int qq = q * q;
-  for (int transpose = 0; transpose < 2; ++transpose)
-    for (int extra = 0; extra < 2; ++extra) {
-      RadonShape sh;
-      const int count_out = (transpose ? !extra : extra) ? qq + q : qq;   // forward stages grow, transposed ones shrink
-      for (int co : {count_out, qq, qq + q}) {
-        if (!radon_shape(q, transpose, extra, co, &sh)) continue;
-        if (!radon_layout_ok(q, sh, sh.ring, 0, 0, extra, sh.smem)) return 0;
-        if (!transpose && sh.nslots == 1 && sh.sr == TILE_ROWS && sh.parts == 1) {
-          const int mini = 2 * ((q + 7) & ~7) * 128, slot = sh.sr * 256;
-          int ring = (227 * 1024 - 1024 - 512 - TILE_ROWS * 8) / (slot + mini);
-          if (ring > sh.ring) ring = sh.ring;
-          if (ring >= 4 && !radon_layout_ok(q, sh, ring, mini, 1, extra, ring * (slot + mini) + TILE_ROWS * 8 + 512 + 1024))
-            return 0;
-        }
-      }
-    }
-  return 1;
-}
-
 // Rows (of state_elems bf16 each, per head) of the intermediate table the d = 4 stages exchange.
 int64_t smat_tabulate_tc_scratch_rows(const SmatGeo& geo) {
   return geo.D == 3 ? (int64_t)geo.q * geo.q * geo.q + (int64_t)geo.q * geo.q : 0;
@@ -999,6 +976,39 @@ int64_t smat_tabulate_tc_scratch_elems(const SmatGeo& geo, int64_t state_elems, 
     return ctas * rows * 128;
   }
   return (int64_t)bh * rows * state_elems;
+}
+
+// Host-only: 1 when every stage of a tabulation of prime q has a kernel whose shared-memory map holds: the resident matrix
+// (with the tile-store variant where the launcher would pick it), the generated one, or, for d = 3 alone, its forward
+// stage.  (The both-stages kernel of smat_radon_slab.cu has one map, asserted where it is compiled.)
+int smat_tabulate_tc_layout_ok(int q) {
+  StageSpec sp[2];
+  if (q >= 19) {
+    radon_stages(q, 2, 0, false, sp);
+    return radon_wide_layout_ok(q, sp[0]) ? 1 : 0;
+  }
+  for (int D = 2; D <= 3; ++D)
+    for (int transpose = 0; transpose < 2; ++transpose) {
+      const int stages = radon_stages(q, D, transpose, false, sp);
+      for (int i = 0; i < stages; ++i) {
+        if (generates_matrix(q, D, transpose)) {
+          if (!radon_wide_layout_ok(q, sp[i])) return 0;
+          continue;
+        }
+        const int extra = sp[i].in.count > q * q;
+        RadonShape sh;
+        if (!radon_shape(q, transpose, extra, sp[i].out.count, &sh)) return 0;
+        if (!radon_layout_ok(q, sh, sh.ring, 0, 0, extra, sh.smem)) return 0;
+        if (!transpose && sh.nslots == 1 && sh.sr == TILE_ROWS && sh.parts == 1) {
+          const int mini = 2 * ((q + 7) & ~7) * 128, slot = sh.sr * 256;
+          int ring = (227 * 1024 - 1024 - 512 - TILE_ROWS * 8) / (slot + mini);
+          if (ring > sh.ring) ring = sh.ring;
+          if (ring >= 4 && !radon_layout_ok(q, sh, ring, mini, 1, extra, ring * (slot + mini) + TILE_ROWS * 8 + 512 + 1024))
+            return 0;
+        }
+      }
+    }
+  return 1;
 }
 
 // transpose = 0: in = F [bh][P][rp] bf16, out = U [bh][B][rp] bf16.  transpose = 1: in = Ū [bh][B][rp], out = F̄ [bh][P][rp].

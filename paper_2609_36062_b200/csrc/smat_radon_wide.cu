@@ -408,7 +408,29 @@ bool wide_shape(int q, const StageSpec& sp, WideShape* w) {
   return w->ring >= 4;
 }
 
+// The shared-memory map of radon_wide_kernel for a shape, checked on the host before every launch: what follows the ring
+// must end inside the allocation, no box may write past its slot, and a slot's inputs must fit the masks.
+//   [0, ring * B_SLOT)                                      ring slots: two halves of SLOT rows x 128 bytes
+//   [.., + (2 MAX_BBUF + 2 A_BARS + 2 MT) * 8 + 8)          barriers, the tensor-memory slot word, the abort flag
+//   [.., + MT * ROWS * 4)                                   output-row table
+//   [.., + nslots * widest * ROWS * 8)                      masks of the widest group's tiles
+bool wide_layout_ok(int q, const StageSpec& sp, const WideShape& w) {
+  const int widest = (w.tiles + w.groups - 1) / w.groups, qq = q * q;
+  bool ok = widest <= MT && w.ring >= 1 && w.ring <= MAX_BBUF && B_SLOT == 2 * SLOT * 128 && B_SLOT % 1024 == 0;
+  ok = ok && w.span <= SLOT && w.nreg * w.span >= w.n_reg && (w.flat || (w.lines * q == w.span && w.n_reg == qq));
+  ok = ok && (w.nslots == w.nreg || (w.nslots == w.nreg + 1 && sp.in.count == qq + q && q <= SLOT));   // the extra class
+  ok = ok && (SLOT + q - 2) / q + 1 <= 6;                                                // lines a slot touches (row_mask)
+  ok = ok && w.tiles * ROWS >= sp.out.count && qq + q < (1 << 16);                       // index arithmetic by umulhi
+  const int end = w.ring * B_SLOT + (2 * MAX_BBUF + 2 * A_BARS + 2 * MT) * 8 + 8 + MT * ROWS * 4 + w.nslots * widest * ROWS * 8;
+  return ok && 1023 + end <= w.smem && w.smem <= 227 * 1024;
+}
+
 }  // namespace
+
+bool radon_wide_layout_ok(int q, const StageSpec& sp) {
+  WideShape w;
+  return wide_shape(q, sp, &w) && wide_layout_ok(q, sp, w);
+}
 
 bool radon_wide_fits(int q, const StageSpec& sp) {
   WideShape w;
@@ -419,6 +441,7 @@ cudaError_t launch_radon_wide(int q, int transpose, const StageSpec& sp, int64_t
   const RadonSide& in = sp.in;
   WideShape w;
   if (!wide_shape(q, sp, &w) || rp % NE) return cudaErrorInvalidValue;
+  if (!wide_layout_ok(q, sp, w)) return cudaErrorInvalidConfiguration;
   WideParams prm;
   prm.q = q; prm.transpose = transpose;
   prm.inv_q = (uint32_t)((1ULL << 32) / (uint32_t)q) + 1;

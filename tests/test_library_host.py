@@ -138,11 +138,17 @@ def test_launching_calls_report_a_missing_sm100_device():
     lib.smat_plan_destroy(h)
 
 
-@pytest.mark.parametrize("q", [2, 3, 5, 7, 11, 13, 17, 19, 23])
+@pytest.mark.parametrize("q", [2, 3, 5, 7, 11, 13, 17, 19, 23, 29, 31, 37, 41, 43, 47, 53])
 def test_tabulation_kernel_shared_memory_map_is_disjoint(q):
-    """Ring slots, per-slot extra rows, the output-row table and the barrier words of the tensor-core tabulation kernel
-    never overlap and no load box or staged tile leaves its slot, for every launch shape of every prime it accepts."""
+    """Ring slots, per-slot extra rows, the output-row table, masks and the barrier words of the tensor-core tabulation
+    kernels never overlap and no load box or staged tile leaves its slot, for every stage of every prime they take."""
     assert binding.load_library().smat_debug_tabulation_layout_ok(q) == 1
+
+
+@pytest.mark.parametrize("q", [59, 61, 241])
+def test_no_tabulation_kernel_claims_a_prime_that_does_not_fit(q):
+    """Their masks leave no room for a ring of image slots: the sums are formed on the fp32 ALUs."""
+    assert binding.load_library().smat_debug_tabulation_layout_ok(q) == 0
 
 
 def test_gated_plans_size_their_inner_plan_and_decode_cache():
