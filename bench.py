@@ -387,6 +387,11 @@ def table_bytes(plan):
     return plan.type_table_element_bytes(), plan.profile_table_element_bytes()
 
 
+def on_alus(plan) -> bool:
+    """Whether the plan's passes run on the fp32-ALU kernels."""
+    return not plan.uses_tensor_cores() and not plan.gated_forward_uses_tensor_cores()
+
+
 def gated_tc_mode(plan) -> int:
     """0: not a gated plan on the tensor cores; 1: its forward only; 2: forward and backward."""
     if not plan.gated_forward_uses_tensor_cores():
@@ -432,7 +437,7 @@ def path_report(w, geo, seconds_per_step, peaks, u_bytes=4, f_bytes=4, gated_tc_
     }
 
 
-def dominant_kernel_report(w, geo, stages, peaks, u_bytes=4, f_bytes=4):
+def dominant_kernel_report(w, geo, stages, peaks, u_bytes=4, f_bytes=4, alu_path=False):
     """Roofline of the stage that takes the longest.  Its bound is the slower of its bytes at the HBM peak and its
     operations (contraction flop plus Algorithm 2's additions, one flop each) at the tensor peak; a tabulation that
     adds on the fp32 ALUs is held against the measured fp32-add rate instead when that is the slower term."""
@@ -440,7 +445,7 @@ def dominant_kernel_report(w, geo, stages, peaks, u_bytes=4, f_bytes=4):
     total = sum(t for _, t in stages)
     name, ms = max(stages, key=lambda s: s[1])
     base = name[len("bwd_fwd_"):] if name.startswith("bwd_fwd_") else name   # a forward stage re-run by the backward
-    work = roofline.stage_work(base, w.T, w.chunk, w.d_k, w.d_v, e, geo, u_bytes, f_bytes).scaled(w.bh)
+    work = roofline.stage_work(base, w.T, w.chunk, w.d_k, w.d_v, e, geo, u_bytes, f_bytes, alu_path).scaled(w.bh)
     t = roofline.roofline_times(work, peaks, sustained=True)
     ops = work.flops + work.adds
     t_ops = ops / (peaks["bf16_tflops_sustained"] * 1e12)
@@ -551,7 +556,7 @@ def run_native(args):
                     "d2h_bytes_per_step": d2h},
             "gpu_launches": launches * steps,
             "clocks": clocks,
-            "roofline": dominant_kernel_report(w, g, stages, peaks, ub, fb),
+            "roofline": dominant_kernel_report(w, g, stages, peaks, ub, fb, on_alus(runner.plan)),
             "path_roofline": path_report(w, g, per_step, peaks, ub, fb, gated_tc_mode(runner.plan)),
             "tables": {"profile_states_P": g.P, "cached_subset_states_B": g.B, "nnzC": g.nnzC, "q": g.q},
             "fadd_rates_adds_per_s": peaks.get("fadd_rates"),
@@ -572,7 +577,7 @@ def run_native(args):
             rep = path_report(ws_, gg, s, peaks, r.plan.type_table_element_bytes(), r.plan.profile_table_element_bytes(),
                               gated_tc_mode(r.plan))
             st_ = r.stage_profile(3)
-            dom = dominant_kernel_report(ws_, gg, st_, peaks, *table_bytes(r.plan))
+            dom = dominant_kernel_report(ws_, gg, st_, peaks, *table_bytes(r.plan), on_alus(r.plan))
             sweep.append({"workload": name, "dominant": {k: dom[k] for k in ("kernel", "bound", "achieved", "peak", "unit",
                                                                               "frac", "ms", "share")}, "value": ws_.tokens / s, "unit": "tokens/s", "ms_per_step": 1e3 * s,
                           "timing": "median of 15 steps after 5 warm-ups, one CUDA event pair per step",

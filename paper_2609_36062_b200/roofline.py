@@ -98,50 +98,94 @@ def roofline_times(work: Work, peaks: dict, sustained: bool = True) -> dict:
 
 
 # Per-kernel algorithmic traffic (bytes), adds and flop, keyed by the stage names the library reports.
-def stage_work(name: str, T, c, r, p, e, geo, u_bytes=4, f_bytes=4) -> Work:
-    """What one forward stage has to do at the least: its contraction flop, Algorithm 2's additions where it
-    tabulates, and the bytes of its inputs and outputs (scratch the stage exchanges with itself is not counted)."""
+def stage_table(T, c, r, p, e, geo, u_bytes=4, f_bytes=4, alu_path=False) -> dict[str, Work]:
+    """What one stage has to do at the least: its contraction flop, Algorithm 2's additions where it tabulates, and the
+    bytes of its inputs and outputs (scratch the stage exchanges with itself is not counted).  alu_path: the plan's passes
+    run on the fp32 ALUs, where chunk states are pooled together with the tables."""
     rp, NC = r * p, T // c
-    n, m, P, B = geo.n, geo.m, geo.P, geo.B
+    lr = geo.d > 1
+    n, m, P, B = (geo.n, geo.m, geo.P, geo.B) if lr else (0, 0, 0, 0)
     st = 4 * rp
     su = u_bytes * rp
     sf = f_bytes * rp
     tc_tiles = T // 128
+    # long-range rows of the two-level output kernel: bf16, but fp32 where blocks are not whole 128-token tiles
+    row = 4 if geo.n % 128 or geo.m % 128 else 2
+    chunks = Work(2 * T * rp, 0, T * (r + p) * e + NC * st)
+    profiles = Work(2 * n * rp, 0, n * (r + p) * e + P * st)
+    dq_tile = Work(T * 129 * (r + p) + 2 * T * rp, 0, T * (2 * p + 2 * r) * e + tc_tiles * rp * 2 + m * r * 2)
+    scaled = lambda dim: Work(0, 0, 2 * T * dim * e + 4 * T)
     table = {
-        "pool":        Work(2 * n * rp, 0, n * (r + p) * e + P * st),
+        # K and V are read once for both sets of states; d = 1 without chunk states: the one state of the decode cache
+        "pool":        Work(2 * (T + n) * rp, 0, T * (r + p) * e + (NC + P) * st) if alu_path else
+                       profiles if lr else Work(2 * geo.n * rp, 0, geo.n * (r + p) * e + st),
         "pool_tc":     Work(2 * n * rp, 0, n * (r + p) * e + P * sf),
         "tabulate":    Work(0, geo.nnzC * rp, P * st + B * su),
         "tabulate_tc": Work(0, geo.nnzC * rp, P * sf + B * su),
         "tabulate_wide": Work(0, geo.nnzC * rp, P * sf + B * su),      # the same on the tensor cores, larger primes
         "tabulate_bf16": Work(0, geo.nnzC * rp, P * sf + B * su),
-        "bwd_tabulate_t_tc": Work(0, geo.nnzC * rp, B * su + P * sf),
+        "read_type":   Work(2 * m * rp, 0, m * r * e + B * st + m * p * 4),
+        "read_type_tc": Work(2 * m * rp, 0, m * r * e + B * su + m * p * 2),
+        # causal branch on the tensor cores
+        "segment_state_tc": Work(2 * T * rp, 0, T * (r + p) * e),
+        "segment_scan": Work(0, 0, 0),                                 # scratch of the branch: totals of whole segments
+        "segment_output_tc": Work(T * 129 * (r + p) + 4 * T * rp, 0, T * (2 * r + 2 * p) * e + m * p * row),
+        "chunk_scan_tc": Work(2 * T * rp, tc_tiles * rp, T * (r + p) * e + tc_tiles * rp * 2),
+        "chunk_output_tc": Work(T * 129 * (r + p) + 2 * T * rp, 0, T * (2 * r + 2 * p) * e + tc_tiles * rp * 2 + m * p * 4),
+        # ... and on the fp32 ALUs
+        "scan":        Work(0, NC * rp, 2 * NC * st),
+        "gated_scan":  Work(0, NC * rp, 2 * NC * st),
+        "tiles":       Work(T * (c + 1) * (r + p) + 2 * T * rp, 0, T * (2 * r + 2 * p) * e + NC * st + m * p * 4),
+        # backward, tables
+        "bwd_pool":    chunks.scaled(2) + profiles + Work(2 * m * rp, 0, B * st - n * (r + p) * e),   # rows read once
+        "bwd_pool_type": Work(2 * m * rp, 0, m * (r + p) * e + B * st),
         "bwd_pool_type_tc": Work(2 * m * rp, 0, m * (r + p) * e + B * su),
+        "bwd_tabulate_t": Work(0, geo.nnzC * rp, B * st + P * sf),
+        "bwd_tabulate_t_tc": Work(0, geo.nnzC * rp, B * su + P * sf),
+        "bwd_dq_type": Work(2 * m * rp, 0, m * p * e + B * st + m * r * 4),
         "bwd_dq_type_tc": Work(2 * m * rp, 0, m * p * e + B * su + m * r * 2),
+        "bwd_dk_profile": Work(2 * n * rp, 0, n * p * e + P * st + n * r * 4),
         "bwd_dk_profile_tc": Work(2 * n * rp, 0, n * p * e + P * sf + n * r * 2),
+        "bwd_dv_profile": Work(2 * n * rp, 0, n * r * e + P * st + n * p * 4),
         "bwd_dv_profile_tc": Work(2 * n * rp, 0, n * r * e + P * sf + n * p * 2),
         "bwd_dkdv_profile_tc": Work(4 * n * rp, 0, n * (r + p) * e + P * sf + n * (r + p) * 2),
+        "bwd_reads":   Work((2 * m + 4 * n) * rp, 0, (m * p + n * (r + p)) * e + (B + P) * st + (m * r + n * (r + p)) * 4),
+        # backward, states and tiles
+        "bwd_scan":    Work(0, 2 * NC * rp, 4 * NC * st),
+        "bwd_gated_scan": Work(0, NC * rp, 2 * NC * st),
         "bwd_suffix_scan_tc": Work(2 * T * rp, tc_tiles * rp, T * (r + p) * e + tc_tiles * rp * 2),
+        "bwd_tiles":   Work(T * (c + 1) * (3 * r + 2 * p) + 6 * T * rp, 0,
+                            T * (4 * r + 3 * p) * e + 2 * NC * st + (m * r + n * (r + p)) * 4),
         # dQ, dK, dV of every 128-token tile: eight 128 x 128 x 128 products per tile; reads Q, K, V, dO, the two
         # per-tile states and the three long-range buffers (bf16), writes the three gradients
         "bwd_tiles_fused_tc": Work(tc_tiles * 8 * 2 * 128 * 128 * 128, 0,
                                    T * (2 * r + 2 * p) * e + T * (2 * r + p) * e + 2 * tc_tiles * rp * 2 +
                                    (m * r + n * r + n * p) * 2),
-        "segment_state_tc": Work(2 * T * rp, 0, T * (r + p) * e),
-        "segment_scan": Work(0, 0, 0),
-        "segment_output_tc": Work(T * 129 * (r + p) + 4 * T * rp, 0, T * (2 * r + 2 * p) * e + m * p * 2),
-        "chunk_state": Work(2 * T * rp, 0, T * (r + p) * e + NC * st),
-        "scan":        Work(0, NC * rp, 2 * NC * st),
-        "scores":      Work(T * (c + 1) * r, 0, 2 * T * r * e + T * c * 4),
-        "read_chunk":  Work(2 * T * rp, 0, T * r * e + NC * st + T * p * 4),
-        "read_type":   Work(2 * m * rp, 0, m * r * e + B * st + 2 * m * p * 4),
-        "read_type_tc": Work(2 * m * rp, 0, m * r * e + B * su + m * p * 2),
-        "chunk_scan_tc": Work(2 * T * rp, tc_tiles * rp, T * (r + p) * e + tc_tiles * rp * 2),
-        "chunk_output_tc": Work(T * 129 * (r + p) + 2 * T * rp, 0, T * (2 * r + 2 * p) * e + tc_tiles * rp * 2 + m * p * 4),
-        "output":      Work(T * (c + 1) * p, 0, T * c * 4 + T * p * e + T * p * 4 + T * p * e),
+        "bwd_dq_tile_tc": dq_tile,
+        "bwd_dk_tile_tc": dq_tile + Work(0, 0, (n - m) * r * 2),
+        "bwd_dv_tile_tc": dq_tile + Work(0, 0, n * p * 2 - m * r * 2),
+        # user-supplied routing: keys in, lists and offsets out; keys of the rows that may need a zero
+        "routing_lists": Work(0, 0, 8 * (n + m) + 4 * (P + B + 2)),
+        "zero_unrouted": Work(0, 0, 4 * max(n, m)),
+        # scalar gates: sums over the log-gates, rescaled copies (pairs of them on the tensor-core path)
+        "gate_prefix": Work(0, T, 8 * T),
+        "bwd_gate_suffix": Work(0, T, 8 * T),
+        "gate_scale":  Work(0, 0, 2 * T * r * e + (T + m) * r * e + 4 * T) if lr else scaled(r),
+        "bwd_gate_scale": Work(0, 0, 2 * T * (r + p) * e + 4 * T) if lr else scaled(r),
+        "gate_scale_q": scaled(r), "gate_scale_k": scaled(r), "gate_scale_lr": scaled(r),
+        "bwd_gate_scale_do": scaled(p), "bwd_gate_scale_v": scaled(p), "bwd_gate_scale_lr": scaled(p),
+        "bwd_gate_dlam": Work(0, 0, 4 * T * r * e + 4 * T),
     }
-    aliases = {"gated_chunk_scan_tc": "chunk_scan_tc", "gated_chunk_output_tc": "chunk_output_tc",
-               "bwd_gated_suffix_scan_tc": "bwd_suffix_scan_tc", "bwd_gated_tiles_fused_tc": "bwd_tiles_fused_tc"}
-    return table.get(aliases.get(name, name), Work(0, 0, 0))
+    for name, like in (("bwd_state_scan_tc", "chunk_scan_tc"), ("gated_chunk_scan_tc", "chunk_scan_tc"),
+                       ("gated_chunk_output_tc", "chunk_output_tc"), ("bwd_gated_suffix_scan_tc", "bwd_suffix_scan_tc"),
+                       ("bwd_gated_tiles_fused_tc", "bwd_tiles_fused_tc")):
+        table[name] = table[like]
+    return table
+
+
+def stage_work(name: str, T, c, r, p, e, geo, u_bytes=4, f_bytes=4, alu_path=False) -> Work:
+    """The stage's entry; a name that the table does not know is an error (KeyError)."""
+    return stage_table(T, c, r, p, e, geo, u_bytes, f_bytes, alu_path)[name]
 
 
 # Stages whose additions run on the fp32 ALUs (the other tabulations form the same sums on the tensor cores).
