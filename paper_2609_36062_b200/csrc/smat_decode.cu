@@ -52,12 +52,14 @@ __device__ __forceinline__ float4 load_state4<__nv_bfloat16>(const __nv_bfloat16
 // a time took 22.1.
 constexpr int DEC_COLS = 32, DEC_ROWS = 32, DEC_THREADS = 256;
 
-template <typename T, typename TU, int PASSES>
+// TOGETHER: the CTAs of a head are a cluster and none writes o or the running gate before all have read q, k and it (gated
+// steps, and o in the place of q or k).
+template <typename T, typename TU, int PASSES, bool TOGETHER>
 __global__ void __launch_bounds__(DEC_THREADS) decode_step_kernel(const T* q, const T* k,
                                                           const T* v, T* o,
                                                           float* S, const TU* U, int64_t type,
                                                           int64_t types, int p, const float* log_a,
-                                                          float* log_g, int together) {
+                                                          float* log_g) {
   constexpr int r = PASSES * DEC_ROWS;
   __shared__ float part[DEC_THREADS / 32][DEC_COLS];
   pdl_trigger();
@@ -87,7 +89,7 @@ __global__ void __launch_bounds__(DEC_THREADS) decode_step_kernel(const T* q, co
   // gated: a = this token's gate, g = the product of the gates since the block boundary (kept as its logarithm)
   float a = 1.f, g = 1.f;
   float lg = 0.f;
-  if (log_a) { lg = log_g[bh] + log_a[bh]; a = __expf(log_a[bh]); g = __expf(lg); }
+  if (TOGETHER && log_a) { lg = log_g[bh] + log_a[bh]; a = __expf(log_a[bh]); g = __expf(lg); }
   float o4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
   for (int n = 0; n < PASSES; ++n) {
@@ -97,8 +99,7 @@ __global__ void __launch_bounds__(DEC_THREADS) decode_step_kernel(const T* q, co
     o4[0] = fmaf(qi[n], fmaf(g, u[n].x, s[n].x), o4[0]); o4[1] = fmaf(qi[n], fmaf(g, u[n].y, s[n].y), o4[1]);
     o4[2] = fmaf(qi[n], fmaf(g, u[n].z, s[n].z), o4[2]); o4[3] = fmaf(qi[n], fmaf(g, u[n].w, s[n].w), o4[3]);
   }
-  // together: the CTAs of a head are a cluster and none writes o or the running gate before all have read q, k and it
-  if (together) asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
+  if (TOGETHER) asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
 #pragma unroll
   for (int c = 0; c < 4; ++c) {   // the four rows a warp holds in each of its passes
     o4[c] += __shfl_xor_sync(0xffffffffu, o4[c], 8);
@@ -106,27 +107,28 @@ __global__ void __launch_bounds__(DEC_THREADS) decode_step_kernel(const T* q, co
   }
   if ((tid & 31) < 8) *reinterpret_cast<float4*>(&part[tid >> 5][(tid & 7) * 4]) = make_float4(o4[0], o4[1], o4[2], o4[3]);
   __syncthreads();
-  if (together) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  if (TOGETHER) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   if (tid < DEC_COLS) {
     float sum = 0.f;
 #pragma unroll
     for (int w = 0; w < DEC_THREADS / 32; ++w) sum += part[w][tid];
     store_out(o + (int64_t)bh * p + j0 + tid, sum);
   }
-  if (log_a && blockIdx.x == 0 && tid == 0) log_g[bh] = lg;
+  if (TOGETHER && log_a && blockIdx.x == 0 && tid == 0) log_g[bh] = lg;
 }
 
 template <typename T, typename TU>
 cudaError_t launch_step(const void* q, const void* k, const void* v, void* o, float* S, const void* U, int64_t type,
                         int64_t types, int r, int p, int bh, cudaStream_t st, const float* log_a, float* log_g) {
-  auto kernel = r == 64 ? decode_step_kernel<T, TU, 2> : decode_step_kernel<T, TU, 4>;
   const unsigned slices = (unsigned)(p / DEC_COLS);
   // o in the place of q or k (o in the place of v needs nothing: a CTA reads just the columns that it writes)
   const size_t in = (size_t)bh * r * sizeof(T), out = (size_t)bh * p * sizeof(T);
-  const int together = log_a || smat_overlap(o, out, q, in) || smat_overlap(o, out, k, in);
+  const bool together = log_a || smat_overlap(o, out, q, in) || smat_overlap(o, out, k, in);
+  auto kernel = r == 64 ? (together ? decode_step_kernel<T, TU, 2, true> : decode_step_kernel<T, TU, 2, false>)
+                        : (together ? decode_step_kernel<T, TU, 4, true> : decode_step_kernel<T, TU, 4, false>);
   return smat_launch_pdl_cluster(kernel, dim3(slices, (unsigned)bh), DEC_THREADS, 0, together ? slices : 1u, st,
                                  static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v),
-                                 static_cast<T*>(o), S, static_cast<const TU*>(U), type, types, p, log_a, log_g, together);
+                                 static_cast<T*>(o), S, static_cast<const TU*>(U), type, types, p, log_a, log_g);
 }
 
 }  // namespace
