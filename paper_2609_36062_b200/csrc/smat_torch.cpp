@@ -10,6 +10,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <exception>
 #include <initializer_list>
 #include <string>
 
@@ -99,6 +100,10 @@ int unlocked(F call) {
 
 // Anything int() takes (a position kept as a float or as an array scalar among it).
 bool token_index(PyObject* o, long long* t) {
+  if (PyLong_CheckExact(o)) {
+    *t = PyLong_AsLongLong(o);
+    return !(*t == -1 && PyErr_Occurred());
+  }
   PyObject* n = PyNumber_Long(o);
   if (!n) return false;
   *t = PyLong_AsLongLong(n);
@@ -141,136 +146,148 @@ PyObject* wrap_all(std::initializer_list<at::Tensor> ts) {
   return tuple;
 }
 
+// The exception in flight as the one torch raises for it (an exhausted device: torch.OutOfMemoryError).
+PyObject* raise() {
+  torch::translate_exception_to_python(std::current_exception());
+  return nullptr;
+}
+
 // forward(kind, Q, K, V, log_a, O, workspace, stream, prof, type): kind 0 plain or routed, 1 gated, 2 normalised
 PyObject* plan_forward(PyObject* self, PyObject* const* a, Py_ssize_t n) {
-  HANDLE_TH_ERRORS   // (an exhausted device arrives as torch.OutOfMemoryError, not as a plain RuntimeError)
-  if (!arity(n, 10, "forward")) return nullptr;
-  const Plan& p = *reinterpret_cast<Plan*>(self);
-  const long kind = PyLong_AsLong(a[0]);
-  const int64_t sk[4] = {p.b, p.h, p.T, p.dk}, sv[4] = {p.b, p.h, p.T, p.dv};
-  const at::Tensor *Q = tensor(a[1], "Q", p.dtype, sk), *K = Q ? tensor(a[2], "K", p.dtype, sk) : nullptr;
-  const at::Tensor* V = K ? tensor(a[3], "V", p.dtype, sv) : nullptr;
-  if (!V) return nullptr;
-  const int64_t sg[2] = {p.b * p.h, p.T};
-  const at::Tensor* la = kind == 1 ? tensor(a[4], "log_a", at::kFloat, sg) : nullptr;
-  if (kind == 1 && !la) return nullptr;
-  at::Tensor O;
-  void *ws, *st;
-  size_t bytes;
-  if (kind == 0 && a[5] != Py_None && !tensor(a[5], "O", p.dtype, sv)) return nullptr;
-  if (!output(a[5], "O", *V, &O) || !workspace(a[6], "workspace", &ws, &bytes) || !stream(a[7], &st)) return nullptr;
-  const void *q = Q->data_ptr(), *k = K->data_ptr(), *v = V->data_ptr();
-  void* o = O.data_ptr();
-  int rc;
-  const char* what;
-  if (kind == 1) {
-    what = "smat_forward_gated";
-    const float* log_a = la->data_ptr<float>();
-    rc = unlocked([&] { return smat_forward_gated(p.handle, q, k, v, log_a, o, ws, bytes, st); });
-  } else if (kind == 2) {
-    what = "smat_forward_normalized";
-    rc = unlocked([&] { return smat_forward_normalized(p.handle, q, k, v, o, ws, bytes, st); });
-  } else if (a[8] != Py_None || a[9] != Py_None) {
-    const int64_t sp[2] = {p.b * p.h, p.n}, stp[2] = {p.b * p.h, p.m};
-    const at::Tensor *prof = tensor(a[8], "prof", at::kInt, sp), *type = prof ? tensor(a[9], "type", at::kInt, stp) : nullptr;
-    if (!type) return nullptr;
-    what = "smat_forward_routed";
-    const int32_t *cells = prof->data_ptr<int>(), *types = type->data_ptr<int>();
-    rc = unlocked([&] { return smat_forward_routed(p.handle, q, k, v, o, cells, types, ws, bytes, st); });
-  } else {
-    what = "smat_forward";
-    rc = unlocked([&] { return smat_forward(p.handle, q, k, v, o, ws, bytes, st); });
+  try {
+    if (!arity(n, 10, "forward")) return nullptr;
+    const Plan& p = *reinterpret_cast<Plan*>(self);
+    const long kind = PyLong_AsLong(a[0]);
+    const int64_t sk[4] = {p.b, p.h, p.T, p.dk}, sv[4] = {p.b, p.h, p.T, p.dv};
+    const at::Tensor *Q = tensor(a[1], "Q", p.dtype, sk), *K = Q ? tensor(a[2], "K", p.dtype, sk) : nullptr;
+    const at::Tensor* V = K ? tensor(a[3], "V", p.dtype, sv) : nullptr;
+    if (!V) return nullptr;
+    const int64_t sg[2] = {p.b * p.h, p.T};
+    const at::Tensor* la = kind == 1 ? tensor(a[4], "log_a", at::kFloat, sg) : nullptr;
+    if (kind == 1 && !la) return nullptr;
+    at::Tensor O;
+    void *ws, *st;
+    size_t bytes;
+    if (kind == 0 && a[5] != Py_None && !tensor(a[5], "O", p.dtype, sv)) return nullptr;
+    if (!output(a[5], "O", *V, &O) || !workspace(a[6], "workspace", &ws, &bytes) || !stream(a[7], &st)) return nullptr;
+    const void *q = Q->data_ptr(), *k = K->data_ptr(), *v = V->data_ptr();
+    void* o = O.data_ptr();
+    int rc;
+    const char* what;
+    if (kind == 1) {
+      what = "smat_forward_gated";
+      const float* log_a = la->data_ptr<float>();
+      rc = unlocked([&] { return smat_forward_gated(p.handle, q, k, v, log_a, o, ws, bytes, st); });
+    } else if (kind == 2) {
+      what = "smat_forward_normalized";
+      rc = unlocked([&] { return smat_forward_normalized(p.handle, q, k, v, o, ws, bytes, st); });
+    } else if (a[8] != Py_None || a[9] != Py_None) {
+      const int64_t sp[2] = {p.b * p.h, p.n}, stp[2] = {p.b * p.h, p.m};
+      const at::Tensor *prof = tensor(a[8], "prof", at::kInt, sp), *type = prof ? tensor(a[9], "type", at::kInt, stp) : nullptr;
+      if (!type) return nullptr;
+      what = "smat_forward_routed";
+      const int32_t *cells = prof->data_ptr<int>(), *types = type->data_ptr<int>();
+      rc = unlocked([&] { return smat_forward_routed(p.handle, q, k, v, o, cells, types, ws, bytes, st); });
+    } else {
+      what = "smat_forward";
+      rc = unlocked([&] { return smat_forward(p.handle, q, k, v, o, ws, bytes, st); });
+    }
+    return fail_status(rc, what) ? wrap(O) : nullptr;
+  } catch (...) {
+    return raise();
   }
-  return fail_status(rc, what) ? wrap(O) : nullptr;
-  END_HANDLE_TH_ERRORS
 }
 
 // backward(kind, Q, K, V, log_a, O, dO, dQ, dK, dV, dlog_a, workspace, stream, prof, type)
 PyObject* plan_backward(PyObject* self, PyObject* const* a, Py_ssize_t n) {
-  HANDLE_TH_ERRORS
-  if (!arity(n, 15, "backward")) return nullptr;
-  const Plan& p = *reinterpret_cast<Plan*>(self);
-  const long kind = PyLong_AsLong(a[0]);
-  const int64_t sk[4] = {p.b, p.h, p.T, p.dk}, sv[4] = {p.b, p.h, p.T, p.dv};
-  const at::Tensor *Q = tensor(a[1], "Q", p.dtype, sk), *K = Q ? tensor(a[2], "K", p.dtype, sk) : nullptr;
-  const at::Tensor* V = K ? tensor(a[3], "V", p.dtype, sv) : nullptr;
-  const at::Tensor* O = V && kind == 2 ? tensor(a[5], "O", p.dtype, sv) : V;
-  const at::Tensor* dO = O ? tensor(a[6], "dO", p.dtype, sv) : nullptr;
-  if (!dO) return nullptr;
-  const int64_t sg[2] = {p.b * p.h, p.T};
-  const at::Tensor* la = kind == 1 ? tensor(a[4], "log_a", at::kFloat, sg) : nullptr;
-  if (kind == 1 && !la) return nullptr;
-  at::Tensor dQ, dK, dV, dla;
-  void *ws, *st;
-  size_t bytes;
-  if (!output(a[7], "dQ", *Q, &dQ) || !output(a[8], "dK", *K, &dK) || !output(a[9], "dV", *V, &dV) ||
-      (la && !output(a[10], "dlog_a", *la, &dla)) || !workspace(a[11], "workspace", &ws, &bytes) || !stream(a[12], &st))
-    return nullptr;
-  const void *q = Q->data_ptr(), *k = K->data_ptr(), *v = V->data_ptr(), *go = dO->data_ptr();
-  void *gq = dQ.data_ptr(), *gk = dK.data_ptr(), *gv = dV.data_ptr();
-  int rc;
-  const char* what;
-  if (kind == 1) {
-    what = "smat_backward_gated";
-    const float* log_a = la->data_ptr<float>();
-    float* glog_a = dla.data_ptr<float>();
-    rc = unlocked([&] { return smat_backward_gated(p.handle, q, k, v, log_a, go, gq, gk, gv, glog_a, ws, bytes, st); });
-  } else if (kind == 2) {
-    what = "smat_backward_normalized";
-    const void* o = O->data_ptr();
-    rc = unlocked([&] { return smat_backward_normalized(p.handle, q, k, v, o, go, gq, gk, gv, ws, bytes, st); });
-  } else if (a[13] != Py_None || a[14] != Py_None) {
-    const int64_t sp[2] = {p.b * p.h, p.n}, stp[2] = {p.b * p.h, p.m};
-    const at::Tensor *prof = tensor(a[13], "prof", at::kInt, sp), *type = prof ? tensor(a[14], "type", at::kInt, stp) : nullptr;
-    if (!type) return nullptr;
-    what = "smat_backward_routed";
-    const int32_t *cells = prof->data_ptr<int>(), *types = type->data_ptr<int>();
-    rc = unlocked([&] { return smat_backward_routed(p.handle, q, k, v, go, gq, gk, gv, cells, types, ws, bytes, st); });
-  } else {
-    what = "smat_backward";
-    rc = unlocked([&] { return smat_backward(p.handle, q, k, v, go, gq, gk, gv, ws, bytes, st); });
+  try {
+    if (!arity(n, 15, "backward")) return nullptr;
+    const Plan& p = *reinterpret_cast<Plan*>(self);
+    const long kind = PyLong_AsLong(a[0]);
+    const int64_t sk[4] = {p.b, p.h, p.T, p.dk}, sv[4] = {p.b, p.h, p.T, p.dv};
+    const at::Tensor *Q = tensor(a[1], "Q", p.dtype, sk), *K = Q ? tensor(a[2], "K", p.dtype, sk) : nullptr;
+    const at::Tensor* V = K ? tensor(a[3], "V", p.dtype, sv) : nullptr;
+    const at::Tensor* O = V && kind == 2 ? tensor(a[5], "O", p.dtype, sv) : V;
+    const at::Tensor* dO = O ? tensor(a[6], "dO", p.dtype, sv) : nullptr;
+    if (!dO) return nullptr;
+    const int64_t sg[2] = {p.b * p.h, p.T};
+    const at::Tensor* la = kind == 1 ? tensor(a[4], "log_a", at::kFloat, sg) : nullptr;
+    if (kind == 1 && !la) return nullptr;
+    at::Tensor dQ, dK, dV, dla;
+    void *ws, *st;
+    size_t bytes;
+    if (!output(a[7], "dQ", *Q, &dQ) || !output(a[8], "dK", *K, &dK) || !output(a[9], "dV", *V, &dV) ||
+        (la && !output(a[10], "dlog_a", *la, &dla)) || !workspace(a[11], "workspace", &ws, &bytes) || !stream(a[12], &st))
+      return nullptr;
+    const void *q = Q->data_ptr(), *k = K->data_ptr(), *v = V->data_ptr(), *go = dO->data_ptr();
+    void *gq = dQ.data_ptr(), *gk = dK.data_ptr(), *gv = dV.data_ptr();
+    int rc;
+    const char* what;
+    if (kind == 1) {
+      what = "smat_backward_gated";
+      const float* log_a = la->data_ptr<float>();
+      float* glog_a = dla.data_ptr<float>();
+      rc = unlocked([&] { return smat_backward_gated(p.handle, q, k, v, log_a, go, gq, gk, gv, glog_a, ws, bytes, st); });
+    } else if (kind == 2) {
+      what = "smat_backward_normalized";
+      const void* o = O->data_ptr();
+      rc = unlocked([&] { return smat_backward_normalized(p.handle, q, k, v, o, go, gq, gk, gv, ws, bytes, st); });
+    } else if (a[13] != Py_None || a[14] != Py_None) {
+      const int64_t sp[2] = {p.b * p.h, p.n}, stp[2] = {p.b * p.h, p.m};
+      const at::Tensor *prof = tensor(a[13], "prof", at::kInt, sp), *type = prof ? tensor(a[14], "type", at::kInt, stp) : nullptr;
+      if (!type) return nullptr;
+      what = "smat_backward_routed";
+      const int32_t *cells = prof->data_ptr<int>(), *types = type->data_ptr<int>();
+      rc = unlocked([&] { return smat_backward_routed(p.handle, q, k, v, go, gq, gk, gv, cells, types, ws, bytes, st); });
+    } else {
+      what = "smat_backward";
+      rc = unlocked([&] { return smat_backward(p.handle, q, k, v, go, gq, gk, gv, ws, bytes, st); });
+    }
+    if (!fail_status(rc, what)) return nullptr;
+    return la ? wrap_all({dQ, dK, dV, dla}) : wrap_all({dQ, dK, dV});
+  } catch (...) {
+    return raise();
   }
-  if (!fail_status(rc, what)) return nullptr;
-  return la ? wrap_all({dQ, dK, dV, dla}) : wrap_all({dQ, dK, dV});
-  END_HANDLE_TH_ERRORS
 }
 
 // decode_step(q, k, v, log_a_t, t, cache, o, stream): log_a_t None for the ungated step
 PyObject* plan_decode_step(PyObject* self, PyObject* const* a, Py_ssize_t n) {
-  HANDLE_TH_ERRORS
-  if (!arity(n, 8, "decode_step")) return nullptr;
-  const Plan& p = *reinterpret_cast<Plan*>(self);
-  const int64_t sk[3] = {p.b, p.h, p.dk}, sv[3] = {p.b, p.h, p.dv};
-  const at::Tensor *q = tensor(a[0], "q", p.dtype, sk), *k = q ? tensor(a[1], "k", p.dtype, sk) : nullptr;
-  const at::Tensor* v = k ? tensor(a[2], "v", p.dtype, sv) : nullptr;
-  if (!v) return nullptr;
-  const at::Tensor* la = nullptr;
-  if (a[3] != Py_None) {
-    if (!THPVariable_Check(a[3])) {
-      PyErr_SetString(PyExc_ValueError, "log_a_t: expected a tensor");
-      return nullptr;
+  try {
+    if (!arity(n, 8, "decode_step")) return nullptr;
+    const Plan& p = *reinterpret_cast<Plan*>(self);
+    const int64_t sk[3] = {p.b, p.h, p.dk}, sv[3] = {p.b, p.h, p.dv};
+    const at::Tensor *q = tensor(a[0], "q", p.dtype, sk), *k = q ? tensor(a[1], "k", p.dtype, sk) : nullptr;
+    const at::Tensor* v = k ? tensor(a[2], "v", p.dtype, sv) : nullptr;
+    if (!v) return nullptr;
+    const at::Tensor* la = nullptr;
+    if (a[3] != Py_None) {
+      if (!THPVariable_Check(a[3])) {
+        PyErr_SetString(PyExc_ValueError, "log_a_t: expected a tensor");
+        return nullptr;
+      }
+      la = &THPVariable_Unpack(a[3]);
+      if (!la->is_cuda() || !la->is_contiguous() || la->scalar_type() != at::kFloat || la->numel() != p.b * p.h) {
+        PyErr_Format(PyExc_ValueError, "log_a_t: expected a contiguous CUDA fp32 tensor of %lld log-gates", (long long)(p.b * p.h));
+        return nullptr;
+      }
     }
-    la = &THPVariable_Unpack(a[3]);
-    if (!la->is_cuda() || !la->is_contiguous() || la->scalar_type() != at::kFloat || la->numel() != p.b * p.h) {
-      PyErr_Format(PyExc_ValueError, "log_a_t: expected a contiguous CUDA fp32 tensor of %lld log-gates", (long long)(p.b * p.h));
-      return nullptr;
-    }
+    long long t;
+    if (!token_index(a[4], &t)) return nullptr;
+    at::Tensor o;
+    void *cache, *st;
+    size_t bytes;
+    if (!workspace(a[5], "cache", &cache, &bytes) || !output(a[6], "o", *v, &o) || !stream(a[7], &st)) return nullptr;
+    const void *qp = q->data_ptr(), *kp = k->data_ptr(), *vp = v->data_ptr();
+    void* op = o.data_ptr();
+    const float* log_a = la ? la->data_ptr<float>() : nullptr;
+    const int rc = unlocked([&] {
+      return la ? smat_decode_step_gated(p.handle, qp, kp, vp, log_a, t, op, cache, bytes, st)
+                : smat_decode_step(p.handle, qp, kp, vp, t, op, cache, bytes, st);
+    });
+    return fail_status(rc, la ? "smat_decode_step_gated" : "smat_decode_step") ? wrap(o) : nullptr;
+  } catch (...) {
+    return raise();
   }
-  long long t;
-  if (!token_index(a[4], &t)) return nullptr;
-  at::Tensor o;
-  void *cache, *st;
-  size_t bytes;
-  if (!workspace(a[5], "cache", &cache, &bytes) || !output(a[6], "o", *v, &o) || !stream(a[7], &st)) return nullptr;
-  const void *qp = q->data_ptr(), *kp = k->data_ptr(), *vp = v->data_ptr();
-  void* op = o.data_ptr();
-  const float* log_a = la ? la->data_ptr<float>() : nullptr;
-  const int rc = unlocked([&] {
-    return la ? smat_decode_step_gated(p.handle, qp, kp, vp, log_a, t, op, cache, bytes, st)
-              : smat_decode_step(p.handle, qp, kp, vp, t, op, cache, bytes, st);
-  });
-  return fail_status(rc, la ? "smat_decode_step_gated" : "smat_decode_step") ? wrap(o) : nullptr;
-  END_HANDLE_TH_ERRORS
 }
 
 // Plan(handle, batch, heads, T, d_k, d_v, bf16)
