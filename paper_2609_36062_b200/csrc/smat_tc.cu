@@ -450,14 +450,6 @@ struct FusedParams {
   int* status;
 };
 
-__device__ __forceinline__ bool elect_one() {
-  uint32_t pred;
-  asm volatile(
-      "{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(pred));
-  return pred != 0;
-}
-
 // GATED (Lemma "Gated SMat", adjoint side): both score tiles are multiplied by exp(λ_i - λ_j) as they are rounded, and
 // the three state products are scaled row by row in tensor memory before the score products are added to them — row i
 // of dO S_inᵀ by exp(λ_i - λ_{last token before the tile}), row j of V D̄ᵀ and of K D̄ by exp(λ_{last token of the
@@ -1312,10 +1304,6 @@ struct ReadParams {
   int* status;
 };
 
-__device__ __forceinline__ void cp_async16_tc(uint32_t smem_addr, const void* gmem) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr), "l"(gmem) : "memory");
-}
-
 // TRANS = 0: out[t][j] = Σ_i x_t[i] St[i][j]  (state as MN-major B);  TRANS = 1: out[t][i] = Σ_j x_t[j] St[i][j]
 // (the same two boxes read as a K-major B).
 // One pass of state_read_tc_kernel: up to 128 tokens of one (state, head) item; states without tokens are skipped.
@@ -1391,8 +1379,8 @@ __global__ void __launch_bounds__(160) state_read_tc_kernel(const __grid_constan
         const int m = idx >> 4, gc = idx & 15;
         const int64_t row = (ps.bh * prm.T + ps.token(m)) * TILE + gc * 8;
         const uint32_t off = (gc >> 3) * BOX_BYTES + m * 128 + (((gc & 7) ^ (m & 7)) << 4);
-        cp_async16_tc(a_base + off, prm.X + row);
-        if (DUAL) cp_async16_tc(a2_base + off, prm.X2 + row);
+        cp_async16(a_base + off, prm.X + row);
+        if (DUAL) cp_async16(a2_base + off, prm.X2 + row);
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -1594,7 +1582,7 @@ __global__ void __launch_bounds__(160) pool_tc_kernel(const __grid_constant__ Po
         const uint32_t dst = (w < 16 ? a_base : b_base) + (gc >> 3) * (TOK * 128) + k * 128 + (((gc & 7) ^ (k & 7)) << 4);
         if (k < kn) {
           const __nv_bfloat16* src = (w < 16 ? prm.K : prm.V) + ((ps.bh * prm.T + ps.token(k)) * TILE + gc * 8);
-          cp_async16_tc(dst, src);
+          cp_async16(dst, src);
         } else {
           asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0u) : "memory");
         }
