@@ -174,17 +174,21 @@ __global__ void __launch_bounds__(192) chunk_scan_tc_kernel(const __grid_constan
 //        dK_b = tril(dO Vᵀ)ᵀ Q  + V  D̄ᵀ        P1 = dO, P2 = V, P3 = Q,  P4 = V  (= P2), St = D̄ᵀ  : K-major rows i
 //        dV_b = tril(Q Kᵀ)ᵀ  dO + K  D̄         P1 = Q,  P2 = K, P3 = dO, P4 = K  (= P2), St = D̄    as [k = i][n = j]
 // All operands are the natural row-major tiles; transposes are expressed through the operand-major bits of the MMA.
-//   warp 8 lane 0 : TMA loads (P1, P2: two boxes each; P3[:, half]; state half), then
+//   last warp, lane 0 : TMA loads (P1, P2: two boxes each; P3[:, half]; state half), then
 //        MMA1  Sc = P1 P2ᵀ                                     -> TMEM columns [0, 128)
 //        MMA2  Oh = P4 · St half          (M = 128, N = 64)    -> TMEM columns [128, 192)
 //        MMA3  Oh += X(ᵀ) · P3[:, half]   (X = masked, rounded Sc, written over the score operand that P4 is not)
-//   warps 0-7     : 32 rows each, two warps to a row quarter: mask and round the scores into the swizzled layout (blocks
-//                   above the diagonal are zeros without being read), later read 32 columns of Oh, add the long-range
-//                   rows and store
-// Gated, 32 heads of 4096 tokens: 0.068 ms (168 MB, 0.026 at the HBM rate; Q and K are loaded, and the scores formed, by
-// both CTAs of a tile).  With four warps and every block unrolled, 1,500 instructions a thread that each CTA ran once, 0.082.
+//   the others        : 32 rows each: mask and round the scores into the swizzled layout (blocks above the diagonal are
+//                       zeros without being read), fetch the long-range rows while the products are formed, read Oh, add
+//                       and store
+// Four such warps, the blocks of 32 keys unrolled; gated eight, two to a row quarter, and the loop kept rolled: with the
+// decays the unrolled form is 1,500 instructions a thread that each CTA runs once (32 heads of 4096 tokens, the kernel
+// alone: 0.068 ms, with four warps 0.082; its 168 MB take 0.026 at the HBM rate, but Q and K are loaded, and the scores
+// formed, by both CTAs of a tile).  Without decays eight are slower: d = 1, 32 heads of 16,512 tokens, the pass 232 us
+// against 228.  The long-range rows fetched only after the products: d = 2, 32 heads of 4480 tokens 120 us against 113,
+// of 18,688 tokens 405 against 394.
 // ---------------------------------------------------------------------------------------------------------------
-constexpr int TILE_EPI_WARPS = 8, TILE_THREADS = 32 * (TILE_EPI_WARPS + 1);
+__host__ __device__ constexpr int tile_epi_warps(bool gated) { return gated ? 8 : 4; }
 constexpr int OUT_SMEM = 6 * BOX_BYTES + 1024 + 256 + TILE * 4;   // operands, alignment, barriers, the tile's λ (gated)
 
 struct TileParams {
@@ -202,11 +206,12 @@ struct TileParams {
 // rounded, and the state product keeps an accumulator of its own so that row i can be scaled by
 // exp(λ_i - λ_{last token before the tile}) when the two are added.
 template <bool P4_IS_P1, bool XT, bool ST_KMAJOR, bool GATED = false>
-__global__ void __launch_bounds__(TILE_THREADS, 2) tile_product_tc_kernel(const __grid_constant__ CUtensorMap tm1,
+__global__ void __launch_bounds__(32 * (tile_epi_warps(GATED) + 1), 2) tile_product_tc_kernel(const __grid_constant__ CUtensorMap tm1,
                                                               const __grid_constant__ CUtensorMap tm2,
                                                               const __grid_constant__ CUtensorMap tm3,
                                                               const __grid_constant__ CUtensorMap tmSt,
                                                               const TileParams prm) {
+  constexpr int EPI = tile_epi_warps(GATED), PARTS = EPI / 4;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* s1 = smem;                    // P1: 2 boxes (K-major, k-blocks 0 and 1)
@@ -233,10 +238,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) tile_product_tc_kernel(const 
 
   if (threadIdx.x == 0) {
     *cta_abort = 0;
-    mbar_init(bar_qk, 1); mbar_init(bar_vs, 1); mbar_init(bar_sc, 1); mbar_init(bar_p, TILE_EPI_WARPS); mbar_init(bar_o, 1);
+    mbar_init(bar_qk, 1); mbar_init(bar_vs, 1); mbar_init(bar_sc, 1); mbar_init(bar_p, EPI); mbar_init(bar_o, 1);
     fence_barrier_init();
   }
-  if (warp == TILE_EPI_WARPS) tmem_alloc(tmem_slot, 256);
+  if (warp == EPI) tmem_alloc(tmem_slot, 256);
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
@@ -250,7 +255,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) tile_product_tc_kernel(const 
   const uint32_t tmem_sc = tmem_base, tmem_o = tmem_base + TILE;
   const uint32_t tmem_st = GATED ? tmem_base + TILE + HALF : tmem_o;   // accumulator of the state product
 
-  if (warp == TILE_EPI_WARPS && lane == 0) {
+  if (warp == EPI && lane == 0) {
     mbar_expect_tx(bar_qk, 4 * BOX_BYTES);
     tma_load_2d(s1, &tm1, 0, (int)row0, bar_qk);
     tma_load_2d(s1 + BOX_BYTES, &tm1, HALF, (int)row0, bar_qk);
@@ -307,15 +312,15 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) tile_product_tc_kernel(const 
     }
     landed(bar_qk, 0, wc);
     landed(bar_vs, 0, wc);
-  } else if (warp < TILE_EPI_WARPS) {
+  } else if (warp < EPI) {
     const int qd = warp & 3, part = warp >> 2;
     const int m = qd * 32 + lane;    // row inside the tile = TMEM lane
     const uint32_t lane_base = (uint32_t)(qd * 32) << 16;
     if (mbar_wait_warp(bar_sc, 0, wc)) {
       fence_after_sync();
       const float lam_m = GATED ? sLam[m] : 0.f;
-#pragma unroll 1
-      for (int cb = part; cb < 4; cb += TILE_EPI_WARPS / 4) {   // blocks of 32 keys
+#pragma unroll (GATED ? 1 : 4)
+      for (int cb = part; cb < 4; cb += PARTS) {   // blocks of 32 keys
         if (cb > qd) {   // wholly above the diagonal
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
@@ -356,24 +361,35 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) tile_product_tc_kernel(const 
       fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_p);   // one arrival per warp
+      // the rows to be added travel while the products are formed: 32 columns are eight (fp32) or four (bf16) pieces
+      const int64_t t = (int64_t)b * TILE + m, at = ((int64_t)bh * prm.T + t) * TILE + half * HALF;
+      const bool add_lr = t >= prm.add_lo && t < prm.add_hi;
+      uint4 y[2 / PARTS][8];
+      if (add_lr) {
+#pragma unroll
+        for (int c = 0; c < 2 / PARTS; ++c) {
+          const int col = (part + c * PARTS) * 32;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            if (!prm.addend16) y[c][i] = reinterpret_cast<const uint4*>(prm.addend + at + col)[i];
+            else if (i < 4) y[c][i] = reinterpret_cast<const uint4*>(prm.addend16 + at + col)[i];
+          }
+        }
+      }
       if (mbar_wait_warp(bar_o, 0, wc)) {
         fence_after_sync();
-        const int64_t t = (int64_t)b * TILE + m;
-        const bool add_lr = t >= prm.add_lo && t < prm.add_hi;
         float row_scale = 1.f;   // GATED: exp(λ_i - λ of the last token before the tile)
         if (GATED) row_scale = __expf(lam_m - (b > 0 ? prm.lam[row0 - 1] : 0.f));
-        const float4* y4 = reinterpret_cast<const float4*>(prm.addend + ((int64_t)bh * prm.T + t) * TILE + half * HALF);
-        const uint4* y16 = reinterpret_cast<const uint4*>(prm.addend16 + ((int64_t)bh * prm.T + t) * TILE + half * HALF);
-        uint4* dst = reinterpret_cast<uint4*>(prm.Out + ((int64_t)bh * prm.T + t) * TILE + half * HALF);
         const bool wide = rows_are_wide(prm.Out);
-        {
-          const int cb = part;   // 32 of the 64 output columns
+#pragma unroll
+        for (int c = 0; c < 2 / PARTS; ++c) {   // 32 of the 64 output columns
+          const int col = (part + c * PARTS) * 32;
           uint32_t v[32];
-          tmem_ld32(tmem_o + lane_base + cb * 32, v);
+          tmem_ld32(tmem_o + lane_base + col, v);
           tmem_ld_wait();
           if (GATED) {
             uint32_t vs[32];
-            tmem_ld32(tmem_st + lane_base + cb * 32, vs);
+            tmem_ld32(tmem_st + lane_base + col, vs);
             tmem_ld_wait();
 #pragma unroll
             for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(fmaf(row_scale, __uint_as_float(vs[e]), __uint_as_float(v[e])));
@@ -385,24 +401,24 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) tile_product_tc_kernel(const 
 #pragma unroll
             for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[i * 8 + e]);
             if (add_lr && prm.addend16) {
-              const uint4 a = *(y16 + cb * 4 + i);   // 8 bf16 values
-              const uint32_t yy[4] = {a.x, a.y, a.z, a.w};
+              const uint32_t yy[4] = {y[c][i].x, y[c][i].y, y[c][i].z, y[c][i].w};   // 8 bf16 values
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
                 f[2 * e] += __uint_as_float(yy[e] << 16);
                 f[2 * e + 1] += __uint_as_float(yy[e] & 0xffff0000u);
               }
             } else if (add_lr) {
-              const float4 a = *(y4 + cb * 8 + i * 2), c = *(y4 + cb * 8 + i * 2 + 1);
-              f[0] += a.x; f[1] += a.y; f[2] += a.z; f[3] += a.w;
-              f[4] += c.x; f[5] += c.y; f[6] += c.z; f[7] += c.w;
+              const uint4 a = y[c][2 * i], d = y[c][2 * i + 1];
+              f[0] += __uint_as_float(a.x); f[1] += __uint_as_float(a.y); f[2] += __uint_as_float(a.z); f[3] += __uint_as_float(a.w);
+              f[4] += __uint_as_float(d.x); f[5] += __uint_as_float(d.y); f[6] += __uint_as_float(d.z); f[7] += __uint_as_float(d.w);
             }
             w[4 * i] = pack_bf16(f[0], f[1]); w[4 * i + 1] = pack_bf16(f[2], f[3]);
             w[4 * i + 2] = pack_bf16(f[4], f[5]); w[4 * i + 3] = pack_bf16(f[6], f[7]);
           }
+          __nv_bfloat16* dst = prm.Out + at + col;
 #pragma unroll
           for (int h8 = 0; h8 < 2; ++h8)   // whole 32-byte sectors
-            st_global_32(dst + cb * 4 + 2 * h8, wide, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
+            st_global_32(dst + 16 * h8, wide, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
                          w[8 * h8 + 5], w[8 * h8 + 6], w[8 * h8 + 7]);
         }
       }
@@ -410,7 +426,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) tile_product_tc_kernel(const 
   }
   fence_before_sync();
   __syncthreads();
-  if (warp == TILE_EPI_WARPS) {
+  if (warp == EPI) {
     fence_after_sync();
     tmem_dealloc(tmem_base, 256);
   }
@@ -1792,7 +1808,7 @@ static cudaError_t launch_tile_product(const void* P1, const void* P2, const voi
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, OUT_SMEM);
   if (err != cudaSuccess) return err;
   dim3 grid((unsigned)(NC * 2), (unsigned)bh);
-  return smat_launch_pdl(tile_product_tc_kernel<P4_IS_P1, XT, ST_KMAJOR, GATED>, grid, TILE_THREADS, OUT_SMEM, st, tm1, tm2, tm3, tmS, prm);
+  return smat_launch_pdl(tile_product_tc_kernel<P4_IS_P1, XT, ST_KMAJOR, GATED>, grid, 32 * (tile_epi_warps(GATED) + 1), OUT_SMEM, st, tm1, tm2, tm3, tmS, prm);
 }
 
 cudaError_t smat_launch_chunk_output_tc(const void* Q, const void* K, const void* V, const void* Sin_bf16,
