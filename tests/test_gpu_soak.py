@@ -10,8 +10,8 @@ from tests.helpers import device_inputs
 
 pytestmark = pytest.mark.gpu
 
-# d, batch, heads, T, d_v, chunk, passes: q = 13 with two CTAs per image and two issuing threads; q = 11 with both
-# Radon stages in one launch; q = 17 with three slots per image
+# d, batch, heads, T, d_v, chunk, passes: q = 13 with the matrix generated beside the image stream; q = 11 with both Radon
+# stages of a slab in one CTA; q = 17 with three slots per image
 CASES = [(3, 4, 8, 4096, 128, 64, 300), (4, 1, 8, 16384, 128, 128, 100), (4, 1, 2, 65536, 128, 128, 40)]
 
 
@@ -29,7 +29,7 @@ def test_repeated_forward_passes_leave_the_status_clean(d, batch, heads, T, dv, 
     assert torch.equal(out, first)
 
 
-# d = 3 (q = 13, transposed Radon stage with three slots per image) and d = 4 (q = 11, both transposed stages in one launch)
+# d = 3 (q = 13, transposed, the matrix generated) and d = 4 (q = 11, both transposed stages in one launch)
 @pytest.mark.parametrize("d,batch,heads,T,c,passes", [(3, 2, 8, 4096, 64, 100), (4, 1, 4, 16384, 128, 40)])
 def test_repeated_backward_passes_leave_the_status_clean(d, batch, heads, T, c, passes):
     w = synth.Workload("soak", d, batch, heads, T, 128, 128, c, "bf16", "normalised", 311)
