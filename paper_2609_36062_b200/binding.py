@@ -17,6 +17,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libsmat.so")
 
 SMAT_F32, SMAT_BF16 = 0, 1
+SMAT_ERR_UNSUPPORTED = 10
 FLAG_SIMT_ONLY = 1
 FLAG_ALG2_TABULATION = 2
 FLAG_PER_TILE_STATES = 4
@@ -387,19 +388,24 @@ class SmatPlan:
         return mask
 
     def debug_tables(self, workspace=None, stream=None):
+        """F, U and the states entering every chunk (or 128-token tile); what the last call did not leave is None."""
         b, h, T, dk, dv = self.shape
         g = self.geometry()
         ws = self._ws if workspace is None else workspace
         tc = self.uses_tensor_cores()
         tiles = tc and bool(self.flags & FLAG_PER_TILE_STATES)   # per-tile states exist on tensor-core plans only then
-        F = U = Sin = None
-        if not (tc and g.d == 1 and not tiles):
-            F = torch.empty((b * h, g.P, dk, dv), dtype=torch.float32, device=ws.device)
-            U = torch.empty((b * h, g.B, dk, dv), dtype=torch.float32, device=ws.device)
-        if not tc or tiles:
-            Sin = torch.empty((b * h, T // (128 if tc else g.c), dk, dv), dtype=torch.float32, device=ws.device)
-        _check(self.lib.smat_debug_tables(self.handle, _ptr(ws), _ptr(F), _ptr(U), _ptr(Sin), _stream(stream)),
-               "smat_debug_tables")
+        partial = tc and not tiles and bool(g.n % 128 or g.m % 128 or g.n < 128)   # states per chunk, after a backward
+        new = lambda count: torch.empty((b * h, count, dk, dv), dtype=torch.float32, device=ws.device)
+        for states in ((True, False) if partial else (not tc or tiles,)):
+            F = U = Sin = None
+            if states or g.d > 1:
+                F, U = new(g.P), new(g.B)
+            if states:
+                Sin = new(T // (128 if tiles else g.c))
+            code = self.lib.smat_debug_tables(self.handle, _ptr(ws), _ptr(F), _ptr(U), _ptr(Sin), _stream(stream))
+            if not (partial and states and code == SMAT_ERR_UNSUPPORTED):
+                break
+        _check(code, "smat_debug_tables")
         return F, U, Sin
 
     def check_status(self, workspace=None, stream=None) -> None:

@@ -10,8 +10,9 @@ from tests.helpers import device_inputs, rel_err, to_numpy64
 
 pytestmark = pytest.mark.gpu
 
-# (d, T, chunk): last tiles of 16, 32, 64, 112 and 127-odd rows, one-tile blocks, blocks longer and shorter than a tile,
-# a whole first block with a partial second one, several segments per block, d = 1 with a partial last tile
+# (d, T, chunk): last tiles of 16, 32, 48, 64, 80 and 112 rows, one-tile blocks, blocks longer and shorter than a tile,
+# a whole first block with a partial second one and the other way round, several segments per block, d = 1 with a partial
+# last tile
 CASES = [(2, 32, 16), (1, 16, 16), (2, 128, 64), (3, 224, 16), (3, 320, 32), (1, 336, 16), (2, 320, 64), (4, 1120, 16),
          (3, 1472, 64), (2, 2368, 64), (1, 2624, 64), (3, 4288, 64)]
 
@@ -69,3 +70,28 @@ def test_routed_tokens_of_no_group_add_nothing():
         Q64, K64, V64 = (synth.as_float64(w, host[x][h]) for x in ("q", "k", "v"))
         ref = so.routed_forward_rows(Q64, K64, V64, geo, prof[h], typ[h], rows)
         assert rel_err(to_numpy64(O[0, h]), ref) <= 2.0 ** -8
+
+
+@pytest.mark.parametrize("d", [3, 1])
+def test_chunk_states_are_exported_where_a_pass_leaves_them(d):
+    """The two-level forward keeps no state per chunk; a backward does, and so does the forward under PER_TILE_STATES."""
+    w, host, dev = _case(d, 1472, 64)
+    plain = binding.SmatPlan(1, 3, w.T, 128, 128, d, 64, "bf16")
+    plain.forward(dev["q"], dev["k"], dev["v"])
+    F, U, Sin = plain.debug_tables()
+    assert Sin is None and (F is None) == (U is None) == (d == 1)
+    plain.backward(dev["q"], dev["k"], dev["v"], dev["v"])
+    states = binding.SmatPlan(1, 3, w.T, 128, 128, d, 64, "bf16", flags=binding.FLAG_PER_TILE_STATES)
+    states.forward(dev["q"], dev["k"], dev["v"])
+    n = plain.geometry().n
+    tables = [p.debug_tables() for p in (plain, states)]
+    for h in range(3):
+        K64, V64 = (synth.as_float64(w, host[x][h]) for x in ("k", "v"))
+        for chunk in (0, 1, n // 64 - 1, n // 64, n // 64 + 1, w.T // 64 - 1):
+            lo = 0 if chunk * 64 < n or d == 1 else n
+            ref = K64[lo:chunk * 64].T @ V64[lo:chunk * 64]
+            for F, U, Sin in tables:
+                e = np.abs(to_numpy64(Sin[h, chunk]) - ref).max()
+                assert e <= 1e-5 * np.abs(ref).max(), (h, chunk, e)
+                if d == 1 and chunk == n // 64:
+                    assert torch.equal(F[h, 0], Sin[h, chunk]) and torch.equal(U[h, 0], Sin[h, chunk])
