@@ -110,7 +110,7 @@ def stage_table(T, c, r, p, e, geo, u_bytes=4, f_bytes=4, alu_path=False) -> dic
     sf = f_bytes * rp
     tc_tiles = T // 128
     # long-range rows of the two-level output kernel: bf16, but fp32 where blocks are not whole 128-token tiles
-    row = 4 if geo.n % 128 or geo.m % 128 else 2
+    row = 4 if geo.n % 128 or geo.m % 128 or geo.n < 128 else 2
     chunks = Work(2 * T * rp, 0, T * (r + p) * e + NC * st)
     profiles = Work(2 * n * rp, 0, n * (r + p) * e + P * st)
     dq_tile = Work(T * 129 * (r + p) + 2 * T * rp, 0, T * (2 * p + 2 * r) * e + tc_tiles * rp * 2 + m * r * 2)
