@@ -20,9 +20,10 @@
 // One persistent CTA per SM, 32 EPT entries of every point per slab, as many slabs in shared memory as fit (at most four);
 // slabs arrive by TMA, and the warp that finishes the last task of a slab starts the next load into the freed buffer.
 // Warps take (slab, task) pairs from a shared counter and write whole rows of 128 EPT bytes.  The least time is the
-// tables' bytes: 32 heads of 16,384 entries at q = 17, 1.25 GB, 0.19 ms.  Measured there: 0.257 ms with three slabs,
-// 0.352 with two, 0.425 for the staged kernel, which keeps its sums in shared memory.  16 heads: q = 11 0.091 -> 0.064,
-// q = 13 0.121 -> 0.087, q = 19 0.299 -> 0.206; 8 heads, q = 23: 0.260 -> 0.218.
+// tables' bytes: 32 heads of 16,384 entries at q = 17, 1.25 GB, 0.19 ms.  Measured there: 0.229 ms with three slabs (0.257
+// while lane 0 alone looked at a slab's barrier; then 0.352 with two slabs), 0.425 for the staged kernel, which keeps its
+// sums in shared memory.  16 heads, staged and here: q = 11 0.091, 0.052; q = 13 0.121, 0.070; q = 19 0.299, 0.145;
+// 8 heads, q = 23: 0.260, 0.150.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -53,7 +54,7 @@ __host__ __device__ constexpr bool is_primitive_root(int r, int q) {
 // bytes must fit shared memory) and the warps.  EPT K q accumulators and 25 other registers a thread have to leave room
 // for enough warps to hide the loads; small primes have the shared-memory bandwidth for K = 2 and twenty warps (q = 11:
 // 0.064 ms against 0.075 at K = 5 and sixteen, q = 13: 0.087 against 0.091 at K = 4), large ones do not (q = 17: 0.299
-// against 0.257 at K = 4 and twelve, q = 19: 0.275 against 0.206 at K = 3).
+// against 0.257 at K = 4 and twelve, q = 19: 0.275 against 0.206 at K = 3; all of these while lane 0 alone waited).
 template <int Q> struct D3Cfg;
 template <> struct D3Cfg<11> { static constexpr int K = 2, ROOT = 2, EPT = 2, WARPS = 20; };
 template <> struct D3Cfg<13> { static constexpr int K = 2, ROOT = 2, EPT = 2, WARPS = 20; };

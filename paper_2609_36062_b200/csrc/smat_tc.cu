@@ -183,8 +183,8 @@ __global__ void __launch_bounds__(192) chunk_scan_tc_kernel(const __grid_constan
 //                       and store
 // Four such warps, the blocks of 32 keys unrolled; gated eight, two to a row quarter, and the loop kept rolled: with the
 // decays the unrolled form is 1,500 instructions a thread that each CTA runs once (32 heads of 4096 tokens, the kernel
-// alone: 0.068 ms, with four warps 0.082; its 168 MB take 0.026 at the HBM rate, but Q and K are loaded, and the scores
-// formed, by both CTAs of a tile).  Without decays eight are slower: d = 1, 32 heads of 16,512 tokens, the pass 232 us
+// alone: 0.062 ms, 0.068 with the long-range rows fetched late, 0.082 then with four warps; its 168 MB take 0.026 at the
+// HBM rate, but Q and K are loaded, and the scores formed, by both CTAs of a tile).  Without decays eight are slower: d = 1, 32 heads of 16,512 tokens, the pass 232 us
 // against 228.  The long-range rows fetched only after the products: d = 2, 32 heads of 4480 tokens 120 us against 113,
 // of 18,688 tokens 405 against 394.
 // ---------------------------------------------------------------------------------------------------------------
