@@ -116,3 +116,7 @@ inline StageSpec stage(const RadonSide& in, const RadonSide& out, int images, co
 bool radon_wide_fits(int q, const StageSpec& sp);   // whether a stage's slots, tiles and tables fit (host only)
 bool radon_wide_layout_ok(int q, const StageSpec& sp);
 cudaError_t launch_radon_wide(int q, int transpose, const StageSpec& sp, int64_t rp, int bh, int* status, cudaStream_t st);
+
+// One stage with the whole matrix in tensor memory as a sparse operand (smat_radon_sparse.cu).
+bool radon_sparse_fits(int q);
+cudaError_t launch_radon_sparse(int q, int transpose, const StageSpec& sp, int64_t rp, int bh, int* status, cudaStream_t st);

@@ -16,9 +16,8 @@
 // traffic.
 //
 // radon_tc_kernel, persistent, one CTA per SM.  An item is one image restricted to 128 consecutive state entries;
-// a CTA owns up to 128 output indices (its part of R; the output indices are split over `parts` CTAs, in whole
-// lines where these fit, that then share every image) and applies them to every item it is given:
-//   warps 0-3      : build the CTA's part of R once and move it to tensor memory (lane = output index, one column
+// R has up to 128 output indices (and for q = 11 four more, below), so one CTA covers an image:
+//   warps 0-3      : build R once and move it to tensor memory (lane = output index, one column
 //                    per two operand rows), where the MMAs read it as their A operand
 //   warp 16 lane 0 : TMA producer; a ring slot holds `sps` lines (fixed hi, all lo) of the image x 128 state entries
 //                    (MN-major B operand, two boxes of 64 entries); the extra class travels in a slot of its own
@@ -28,7 +27,7 @@
 //                    round to bf16 and store 64 contiguous bytes of the output row as two 32-byte sectors
 //   warps 19, 20   : q = 11 only.  q^2 + q = 132 output indices are one tile of 128 and 4 left over, all of the extra
 //                    class (the sum of one line's q rows): these warps add them up from the ring slot itself, so
-//                    that one CTA covers an image instead of two CTAs loading it twice
+//                    that one CTA covers an image
 // d = 4 with q <= 11 (forward with q = 11: smat_radon_slab.cu instead): both stages in ONE launch, slab by slab.  Stage 2
 // of a slab needs stage 1 of every image of the same slab and nothing else, so a CTA keeps the slab's W rows in a private exchange buffer (q^3 + q^2 rows of 128
 // entries, rewritten for every slab, stored and loaded with the L2 evict-last priority while F and U stream with
@@ -37,11 +36,10 @@
 // q = 11 also sends its output tiles off by TMA: the epilogue writes the rounded tile into the item's own ring slot
 // (as large as a tile, and dead once the MMAs have read it) in the box layout, and lane 0 of warp 18 issues the tile
 // stores and frees the slot; the bulk of the stores bypasses the LSU.
-// The kernel exists twice: radon_tc_kernel<false, .> for one stage per launch with every index through the MMAs (q = 17
-// and the small primes), without cache hints, phase tables or ALU warps; radon_tc_kernel<true, .> with them.
-// (The tile-store path is written for several slots per item and several parts and is compiled into both, but the
-// launcher switches it on for q = 11 only: it was measured slower than the direct stores for q = 17.  q = 13 and the
-// transposed q = 17 of d = 3 do not come here: see generates_matrix.)
+// The kernel exists twice: radon_tc_kernel<false> for one stage per launch with every index through the MMAs (small
+// primes), without cache hints, phase tables or ALU warps; radon_tc_kernel<true> with them.
+// (The tile-store path is written for several slots per item and is compiled into both, but the launcher switches it on
+// for q = 11 only.)
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -84,14 +82,14 @@ struct RadonParams {
   int32_t q, transpose;
   int32_t sps, sr;                 // lines (hi values) per ring slot; rows of a slot = sps*q rounded up to 16
   int32_t nreg, nslots;            // slots of regular lines per image; plus one when the input has the extra class
-  int32_t parts, rows_pp;          // CTAs sharing an image, and output indices per CTA (<= 128)
-  int32_t alu_rows;                // output indices parts*rows_pp .. (all of the extra class) summed on the ALUs by the
-                                   // last part, straight from the ring slot; 0: every index goes through the MMAs
+  int32_t rows_mma;                // output indices of the MMA tile (<= 128)
+  int32_t alu_rows;                // output indices rows_mma .. (all of the extra class) summed on the ALUs, straight from
+                                   // the ring slot; 0: every index goes through the MMAs
   int32_t ring;                    // ring slots
   int32_t tma_out;                 // the output tile leaves through the item's own ring slot and TMA stores (q = 11)
   int32_t mini_bytes;              // tma_out: per slot, room for the extra-class rows of the tile (two halves); 0: the
-                                   // extra-class rows of a part sit in the tile itself, after its regular lines
-  int32_t lines_pp;                // tma_out: regular lines per tile (the store box; lines past q - 1 are clipped)
+                                   // extra-class rows sit in the tile itself, after its regular lines
+  int32_t lines_out;               // tma_out: regular lines of the tile (the store box)
   int32_t nph;                     // 1, or 2: both stages of the d = 4 tabulation, slab by slab
   int32_t slabs_per_head;          // rp / 128
   int64_t slabs;                   // heads * slabs_per_head
@@ -248,10 +246,7 @@ __device__ __forceinline__ void issue_slot_steps(int steps, uint32_t tmem_d, uin
 
 // FEAT = false is the plain instantiation (one stage per launch, every index through the MMAs, direct stores, no cache
 // hints): the single-thread roles pay for every instruction, and the prime-specific paths would cost the others time.
-// EARLY: launched to overlap with the kernel before it (see smat_launch.cuh).  q = 17 does without: its launches take
-// hundreds of microseconds, and with the waits compiled in they ran 1 % slower (16 heads of 64 K tokens, d = 4: the pass
-// 4166 us against 4126).
-template <bool FEAT, bool EARLY>
+template <bool FEAT>
 __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid_constant__ CUtensorMap tm_reg0,
                                                                     const __grid_constant__ CUtensorMap tm_vert0,
                                                                     const __grid_constant__ CUtensorMap tm_reg1,
@@ -282,8 +277,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
   volatile int* cta_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WaitCtx wc{cta_abort, prm.status};
-  const int part = blockIdx.x % prm.parts;
-  const bool alu_here = FEAT && prm.alu_rows > 0 && part == prm.parts - 1;
+  const bool alu_here = FEAT && prm.alu_rows > 0;
   const bool tma_out = prm.tma_out != 0;
   const uint32_t nph = FEAT ? (uint32_t)prm.nph : 1u;
 
@@ -304,14 +298,14 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
     if (nph > 1) { prefetch_tmap(&tm_reg1); prefetch_tmap(&tm_vert1); }
   }
   if (warp == MMA_WARP) tmem_alloc(tmem_slot, 512);
-  // This CTA's part of R, built row by row in the (still unused) ring and moved to tensor memory: lane = output
+  // R, built row by row in the (still unused) ring and moved to tensor memory: lane = output
   // index, one column per two operand rows.  The launcher guarantees ring * slot_bytes >= 128 * kt * 2.
   __nv_bfloat16* scratch = reinterpret_cast<__nv_bfloat16*>(sRing);
   for (int c = threadIdx.x; c < prm.ring * (slot_bytes + prm.mini_bytes) / 16; c += blockDim.x)
     reinterpret_cast<uint4*>(sRing)[c] = make_uint4(0u, 0u, 0u, 0u);
   for (int n = threadIdx.x; n < TILE_ROWS; n += blockDim.x)
     for (int h = 0; h < (int)nph; ++h)
-      out_tab[h * TILE_ROWS + n] = n < prm.rows_pp ? side_row(prm.ph[h].out, part * prm.rows_pp + n, q) : ROW_INVALID;
+      out_tab[h * TILE_ROWS + n] = n < prm.rows_mma ? side_row(prm.ph[h].out, n, q) : ROW_INVALID;
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
@@ -321,7 +315,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
   if (warp < 4) {
     const int n = warp * 32 + lane;
     __nv_bfloat16* row = scratch + (size_t)n * kt;
-    if (n < prm.rows_pp && part * prm.rows_pp + n < prm.ph[0].out.count) mark_incident(prm, part * prm.rows_pp + n, row);
+    if (n < prm.rows_mma && n < prm.ph[0].out.count) mark_incident(prm, n, row);
     __syncwarp();
     const uint32_t* roww = reinterpret_cast<const uint32_t*>(row);
     for (int c0 = 0; c0 < (int)r_cols; c0 += 32) {
@@ -338,7 +332,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
-  if (EARLY) pdl_trigger();
+  pdl_trigger();
   const uint32_t tmem_acc = tmem_base + r_cols;
 
   // per phase: streaming tables, or the exchange rows (two-stage kernel only)
@@ -346,21 +340,19 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
   const uint64_t pol_src1 = l2_policy(nph > 1 ? (prm.ph[1].src_private ? POLICY_LAST : POLICY_FIRST) : POLICY_NORMAL);
   const uint64_t pol_dst0 = l2_policy(nph > 1 ? (prm.ph[0].dst_private ? POLICY_LAST : POLICY_FIRST) : POLICY_NORMAL);
   const uint64_t pol_dst1 = l2_policy(nph > 1 ? (prm.ph[1].dst_private ? POLICY_LAST : POLICY_FIRST) : POLICY_NORMAL);
-  // items of this CTA: same part always
-  const uint32_t first = blockIdx.x / prm.parts, step = gridDim.x / prm.parts;
+  const uint32_t first = blockIdx.x, step = gridDim.x;
   const uint32_t sph = (uint32_t)prm.slabs_per_head;
 
   // ---- storing thread (tma_out): one bulk group of tile stores per item; the item's first slot, which holds the tile,
   // goes back to the producer when the stores have read it.  Lane 0 of the second MMA warp when every item is one
   // slot (that warp has no items then), else lane 0 of warp 19.
   auto store_role = [&]() {
-    if (EARLY) pdl_wait();
+    pdl_wait();
     const uint32_t ring = (uint32_t)prm.ring;
     uint32_t slot = 0, prev_slot = 0;
     uint32_t sidx = 0, spar = 0;                                // the item's "staged" barrier (items mod ring) and its parity
     bool have_prev = false;
-    const int hi0 = part * prm.lines_pp;                        // first regular line of this CTA's tiles
-    const int xrow0 = q * q - part * prm.rows_pp;               // tile row of the first extra-class index
+    const int xrow0 = q * q;                                    // tile row of the first extra-class index
     for (ItemIter it(prm, first, step, nph); it.left; it.next()) {
       const RadonPhase& ph = FEAT ? prm.ph[it.ph] : prm.ph[0];
       const CUtensorMap* oreg = FEAT && it.ph ? &tm_oreg1 : &tm_oreg0;
@@ -372,11 +364,9 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
       if (!mbar_wait(staged + sidx, spar, wc)) break;
       if (++sidx == ring) { sidx = 0; spar ^= 1; }
       const uint8_t* tile = sRing + slot * slot_bytes;
-      if (hi0 < q) {
-        tma_store_5d(oreg, tile, e0, 0, hi0, (int)it.img, hc, pol);
-        tma_store_5d(oreg, tile + prm.sr * 128, e0 + 64, 0, hi0, (int)it.img, hc, pol);
-      }
-      if (ph.out.count > q * q && xrow0 < prm.rows_pp && (int)it.img >= ph.out.vert_from) {
+      tma_store_5d(oreg, tile, e0, 0, 0, (int)it.img, hc, pol);
+      tma_store_5d(oreg, tile + prm.sr * 128, e0 + 64, 0, 0, (int)it.img, hc, pol);
+      if (ph.out.count > q * q && xrow0 < prm.rows_mma && (int)it.img >= ph.out.vert_from) {
         const int ci = ph.out.sv_img != 0 ? (int)it.img : 0;   // the map's image stride is sv_img rows
         if (prm.mini_bytes) {
           const uint8_t* mini = sMini + slot * prm.mini_bytes;
@@ -411,7 +401,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
 
   if (warp == PROD_WARP && lane == 0) {
     // ---- TMA producer -----------------------------------------------------------------------------------------
-    if (EARLY) pdl_wait();
+    pdl_wait();
     // The two single-thread roles keep running slot / parity counters: a lone thread pays the full latency of every
     // instruction, so divisions by the ring size inside the loop would show in the kernel time.
     uint32_t slot = 0, par = 0;                               // ring position; parity of the empty barrier's phase to wait for
@@ -468,7 +458,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
     // ---- MMA issuers: the two threads take the items alternately, so that the issue latency of one item (waits,
     // MMAs, commits: more than the tensor pipe needs for it) overlaps with the other thread's item.  Both phases
     // share R and the slot layout, so the issuers only count items. ---------------------------------------------
-    if (EARLY) pdl_wait();
+    pdl_wait();
     const uint32_t me = (uint32_t)(warp - MMA_WARP);
     if (tma_out && me == 1 && prm.nslots == 1) store_role();
     constexpr uint32_t idesc = make_idesc(TILE_ROWS, 128, 0, 1);   // A from tensor memory (R), B MN-major (image rows)
@@ -536,7 +526,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
     // instead of a second, nearly empty tile paying for every MMA again.  A task is one leftover index and 8 state
     // entries (one 16-byte chunk of the swizzled slot); 16 neighbouring tasks store 256 contiguous bytes.
     if (alu_here) {
-      if (EARLY) pdl_wait();
+      pdl_wait();
       const int tid_a = (warp - ALU_WARP) * 32 + lane, tasks = prm.alu_rows * 16;
       const uint32_t ring = (uint32_t)prm.ring;
       uint32_t slot = 0, par = 0;
@@ -549,7 +539,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
         if ((int)it.img >= ph.out.vert_from) {
           const uint8_t* sl = sRing + slot * slot_bytes;
           for (int task = tid_a; task < tasks; task += 32 * ALU_WARPS) {
-            const int u = prm.parts * prm.rows_pp + (task >> 4) - q * q, ch = task & 15;
+            const int u = prm.rows_mma + (task >> 4) - q * q, ch = task & 15;
             const uint8_t* blk = sl + (ch >> 3) * prm.sr * 128;
             float acc[8];
 #pragma unroll
@@ -595,17 +585,17 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
     }
   } else if (warp < EPI_WARPS) {
     // ---- epilogue ---------------------------------------------------------------------------------------------
-    if (EARLY) pdl_wait();
+    pdl_wait();
     // Warp w reads lane quarter w % 4 (32 output indices) and the 32-entry column chunk w / 4 of every item.
     const int qd = warp & 3, cb = warp >> 2;
     const int orow = qd * 32 + lane;                            // output index of this CTA = TMEM lane
     const uint32_t lane_base = (uint32_t)(qd * 32) << 16;
     const int tv0 = out_tab[orow], tv1 = nph > 1 ? out_tab[TILE_ROWS + orow] : ROW_INVALID;
-    const bool active = qd * 32 < prm.rows_pp;                  // warp-uniform: some output index in these lanes
+    const bool active = qd * 32 < prm.rows_mma;                 // warp-uniform: some output index in these lanes
     uint32_t buf = 0, apar = 0, eslot = 0, epar = 0, sidx = 0;
     // tma_out: where this thread's 64 bytes go inside the slot (or inside the slot's extra rows)
-    const bool st_mini = prm.mini_bytes != 0 && part * prm.rows_pp + orow >= q * q;
-    const int st_idx = st_mini ? part * prm.rows_pp + orow - q * q : orow;
+    const bool st_mini = prm.mini_bytes != 0 && orow >= q * q;
+    const int st_idx = st_mini ? orow - q * q : orow;
     const int st_off = (cb >> 1) * (st_mini ? prm.mini_bytes / 2 : prm.sr * 128) + st_idx * 128;
     for (ItemIter it(prm, first, step, nph); it.left; it.next()) {
       const RadonPhase& ph = FEAT ? prm.ph[it.ph] : prm.ph[0];
@@ -636,7 +626,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
           __syncwarp();
         }
         if (tv != ROW_INVALID) {
-          // regular indices and, without extra rows of their own, the extra-class indices of the part: tile row =
+          // regular indices and, without extra rows of their own, the extra-class indices: tile row =
           // TMEM lane; with extra rows per slot (q = 11) the extra-class indices go there
           const int idx = st_idx;
           uint8_t* trow = (st_mini ? sMini + eslot * prm.mini_bytes : sRing + eslot * slot_bytes) + st_off;
@@ -707,18 +697,19 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
 }
 
 struct RadonShape {
-  int sps, sr, nreg, nslots, parts, rows_pp, alu_rows, ring, smem;
+  int sps, sr, nreg, nslots, rows_mma, alu_rows, ring, smem;
 };
 
-// Ring slots of `sps` lines (sps*q rows, rounded up to 16), chosen for the least MMA work; the output indices are
-// split evenly over `parts` CTAs of at most 128 each.  R (128 lanes x one column per two operand rows) and at least
+// Ring slots of `sps` lines (sps*q rows, rounded up to 16), chosen for the least MMA work.  R (128 lanes x one column per two operand rows) and at least
 // two accumulators of 128 columns must fit the 512 columns of tensor memory, and the ring must be able to hold the
 // scratch copy of R while it is built.  Returns false when q is too large for this kernel.
 bool radon_shape(int q, int transpose, int in_has_extra, int count_out, RadonShape* s) {
   const int budget = 227 * 1024 - 1024 - 512 - TILE_ROWS * 8;
   if (q < 2 || q > 64) return false;
-  const int parts = (count_out + TILE_ROWS - 1) / TILE_ROWS;
-  if (parts > 8) return false;
+  // A few indices past a full tile, all of the extra class, with every line in one slot, are left to the ALUs (q = 11:
+  // 132 = 128 + 4 indices).
+  const int left = count_out > TILE_ROWS ? count_out - TILE_ROWS : 0;
+  if (left > 0 && (left > ALU_MAX_ROWS || transpose || in_has_extra || TILE_ROWS < q * q)) return false;
   int best = 1 << 30;
   for (int sps = 1; sps <= q; ++sps) {
     const int sr = (sps * q + 15) & ~15;
@@ -734,24 +725,13 @@ bool radon_shape(int q, int transpose, int in_has_extra, int count_out, RadonSha
     const int cost = nslots * (sr + 48);   // operand rows per image, plus a charge per slot for its hand-over
     if (cost < best) {
       best = cost;
-      s->sps = sps; s->sr = sr; s->nreg = nreg; s->nslots = nslots; s->parts = parts;
-      s->rows_pp = (count_out + parts - 1) / parts; s->alu_rows = 0; s->ring = ring;
+      s->sps = sps; s->sr = sr; s->nreg = nreg; s->nslots = nslots;
+      s->rows_mma = count_out - left; s->alu_rows = left; s->ring = ring;
       s->smem = ring * slot_bytes + TILE_ROWS * 8 + 512 + 1024;
     }
   }
   if (best == (1 << 30)) return false;
-  {   // whole lines per part where they fit: a part's tile can then leave as one box of lines
-    const int lines = count_out / q, lpp = (lines + s->parts - 1) / s->parts;
-    if (count_out % q == 0 && lpp * q <= TILE_ROWS) s->rows_pp = lpp * q;
-  }
-  // A few indices past the last full tile, all of the extra class, with every line in one slot: full tiles for the
-  // MMAs and the rest on the ALUs (q = 11: 132 = 128 + 4 indices, one CTA per image instead of two).
-  const int left = count_out % TILE_ROWS, whole = count_out - left;
-  if (!transpose && !in_has_extra && s->nslots == 1 && s->sps >= q && whole > 0 && left > 0 && left <= ALU_MAX_ROWS &&
-      whole >= q * q) {
-    s->parts = whole / TILE_ROWS; s->rows_pp = TILE_ROWS; s->alu_rows = left;
-  }
-  return true;
+  return left == 0 || (s->nslots == 1 && s->sps >= q);
 }
 
 // The shared-memory map of radon_tc_kernel for a shape, checked on the host before every launch: ring slots, the
@@ -768,9 +748,9 @@ bool radon_layout_ok(int q, const RadonShape& sh, int ring, int mini_bytes, int 
   ok = ok && sh.nslots == sh.nreg + (in_has_extra ? 1 : 0) && sh.nreg * sh.sps >= q;
   ok = ok && q * sh.sps * 128 <= half && q * 128 <= half;                         // a load box (lines or extra class) per half
   ok = ok && ((sh.nslots * sh.sr / 2 + 31) & ~31) + 2 * 128 <= 512;               // R columns and two accumulators
-  ok = ok && sh.rows_pp <= TILE_ROWS && sh.parts * sh.rows_pp + sh.alu_rows >= 0;
-  if (tma_out) {   // the tile is written into the item's first slot: one 128-byte row per output index of the part
-    ok = ok && sh.rows_pp <= sh.sr;
+  ok = ok && sh.rows_mma <= TILE_ROWS;
+  if (tma_out) {   // the tile is written into the item's first slot: one 128-byte row per output index
+    ok = ok && sh.rows_mma <= sh.sr;
     ok = ok && (mini_bytes == 0 || (mini_bytes % 2048 == 0 && mini_bytes / 2 >= q * 128));
   }
   ok = ok && 1023 + ring * (slot + mini_bytes) + 2 * TILE_ROWS * 4 + bars <= smem && smem <= 227 * 1024;
@@ -788,21 +768,19 @@ cudaError_t launch_radon(int q, int transpose, int nph, const StageSpec* sp, int
   if (!radon_shape(q, transpose, in_has_extra, sp[0].out.count, &sh) || rp % 128 ||
       (int64_t)bh * (rp / 128) * max_images * 2 >= (1LL << 31))
     return cudaErrorInvalidValue;
-  if (nph == 2 && (sh.parts != 1 || sp[1].in.count != sp[0].in.count || sp[1].out.count != sp[0].out.count))
+  if (nph == 2 && (sp[1].in.count != sp[0].in.count || sp[1].out.count != sp[0].out.count))
     return cudaErrorInvalidValue;
   RadonParams prm;
   prm.q = q; prm.transpose = transpose; prm.sps = sh.sps; prm.sr = sh.sr; prm.nreg = sh.nreg; prm.nslots = sh.nslots;
-  prm.parts = sh.parts; prm.rows_pp = sh.rows_pp; prm.alu_rows = sh.alu_rows;
+  prm.rows_mma = sh.rows_mma; prm.alu_rows = sh.alu_rows;
   prm.ring = sh.ring; prm.nph = nph; prm.slabs_per_head = (int)(rp / 128); prm.slabs = (int64_t)bh * (rp / 128);
   prm.status = status;
   // One slot per item, as large as an output tile, one CTA per image (q = 11, forward): the tile is stored by TMA
   // from the item's own slot; every slot gets room for the q extra-class rows of its tile (two 64-entry halves).
   int smem = sh.smem;
   prm.tma_out = 0; prm.mini_bytes = 0;
-  prm.lines_pp = sh.rows_pp / q < q ? sh.rows_pp / q : q;
-  // (Tiles of whole lines could leave the same way for q = 17 — the kernel handles several slots per item and several
-  // parts — but there the tile stores were measured 1.6 to 2 times slower than the direct stores.)
-  if (!transpose && sh.nslots == 1 && sh.sr == TILE_ROWS && sh.parts == 1) {
+  prm.lines_out = sh.rows_mma / q < q ? sh.rows_mma / q : q;
+  if (!transpose && sh.nslots == 1 && sh.sr == TILE_ROWS) {
     const int mini = 2 * ((q + 7) & ~7) * 128, slot = sh.sr * 256;
     int ring = (227 * 1024 - 1024 - 512 - TILE_ROWS * 8) / (slot + mini);
     if (ring > sh.ring) ring = sh.ring;
@@ -816,8 +794,8 @@ cudaError_t launch_radon(int q, int transpose, int nph, const StageSpec* sp, int
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (nph == 2 && sms > RADON_EXCHANGE_CTAS) sms = RADON_EXCHANGE_CTAS;  // one private exchange slab per CTA was sized for
-  int64_t ctas = (int64_t)(sms / sh.parts) * sh.parts;
-  const int64_t items = nph == 1 ? prm.slabs * sp[0].images * sh.parts : prm.slabs;
+  int64_t ctas = sms;
+  const int64_t items = nph == 1 ? prm.slabs * sp[0].images : prm.slabs;
   if (items < ctas) ctas = items;
   CUtensorMap tm_reg[2], tm_vert[2], tm_oreg[2], tm_overt[2];
   for (int i = 0; i < nph; ++i) {
@@ -854,7 +832,7 @@ cudaError_t launch_radon(int q, int transpose, int nph, const StageSpec* sp, int
       const int64_t dst_rp = sp[i].dst_private ? 128 : rp, dst_heads = sp[i].dst_private ? ctas : bh;
       const int64_t sizes[4] = {q, q, images, dst_heads};
       const int64_t strides[4] = {out.s_lo, out.s_hi, images > 1 ? out.s_img : out.rows_per_head, out.rows_per_head};
-      const int box[4] = {q, prm.lines_pp, 1, 1};
+      const int box[4] = {q, prm.lines_out, 1, 1};
       if (!radon_map(&tm_oreg[i], sp[i].dst, dst_rp, 5, sizes, strides, box)) return cudaErrorInvalidValue;
       if (out.count > q * q) {
         const bool per_image = out.sv_img != 0;
@@ -873,16 +851,11 @@ cudaError_t launch_radon(int q, int transpose, int nph, const StageSpec* sp, int
   const bool feat = nph > 1 || prm.alu_rows > 0;
   // the plain instantiation has no use for the two ALU warps
   const unsigned threads = feat ? RADON_THREADS : 32 * (ALU_WARP + (prm.tma_out ? 1 : 0));
-  const bool early = feat || q < 17;
-  auto kernel = feat ? radon_tc_kernel<true, true> : (early ? radon_tc_kernel<false, true> : radon_tc_kernel<false, false>);
+  auto kernel = feat ? radon_tc_kernel<true> : radon_tc_kernel<false>;
   cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
-  if (early)
-    return smat_launch_pdl(kernel, dim3((unsigned)ctas), threads, smem, st, tm_reg[0], tm_vert[0], tm_reg[1], tm_vert[1],
-                           tm_oreg[0], tm_overt[0], tm_oreg[1], tm_overt[1], prm);
-  kernel<<<(unsigned)ctas, threads, smem, st>>>(tm_reg[0], tm_vert[0], tm_reg[1], tm_vert[1], tm_oreg[0], tm_overt[0],
-                                                tm_oreg[1], tm_overt[1], prm);
-  return cudaGetLastError();
+  return smat_launch_pdl(kernel, dim3((unsigned)ctas), threads, smem, st, tm_reg[0], tm_vert[0], tm_reg[1], tm_vert[1],
+                         tm_oreg[0], tm_overt[0], tm_oreg[1], tm_overt[1], prm);
 }
 
 // The two stages of d = 4 run as one launch when a CTA's exchange rows (q^3 + q^2 rows of 128 entries), times the
@@ -890,18 +863,19 @@ cudaError_t launch_radon(int q, int transpose, int nph, const StageSpec* sp, int
 bool radon_two_stage_fits(int q, int transpose) {
   RadonShape sh;
   const int qq = q * q;
-  if (!radon_shape(q, transpose, transpose ? 1 : 0, transpose ? qq : qq + q, &sh) || sh.parts != 1) return false;
+  if (!radon_shape(q, transpose, transpose ? 1 : 0, transpose ? qq : qq + q, &sh)) return false;
   return ((int64_t)qq * q + qq) * 256 * RADON_EXCHANGE_CTAS <= (64LL << 20);
 }
 
 }  // namespace
 
-// Which of the two kernels runs a stage.  The one that generates R loads an image once where the resident one has two or
-// three CTAs load it, but shares its issue slots and tensor memory with the generators.  Measured (ms, resident against
-// generated): q = 13, d = 3, 32 heads 0.077 / 0.069, transposed 0.089 / 0.072; q = 13, d = 4, 8 heads 0.425 / 0.405,
-// transposed (4 heads) 0.278 / 0.254; q = 17, d = 3, 64 heads 0.256 / 0.272, transposed 0.312 / 0.269; q = 17, d = 4,
-// 8 heads 1.11 / 1.22.  At q <= 11 one CTA covers an image either way.
-static bool generates_matrix(int q, int D, int transpose) { return q == 13 || (q == 17 && D == 2 && transpose); }
+// Which kernel runs a stage: q = 17 the one with the sparse form of the matrix in tensor memory (smat_radon_sparse.cu), q = 13
+// (and d = 3 beyond) the one that generates it, smaller primes, whose outputs are one tile, the kernel above.  Measured (ms):
+// q = 17, 64 heads of 8192 tokens, d = 3, three CTAs of the kernel above sharing every image 0.257, sparse 0.204; transposed,
+// generated 0.270, sparse 0.206; d = 4, 2 heads of 64 K tokens, three CTAs 0.302, sparse 0.241.  q = 13, d = 3, 32 heads of 4096
+// tokens, generated 0.071, sparse 0.071; d = 4, 4 heads of 40960 tokens 0.211, sparse 0.220.
+static bool sparse_matrix(int q) { return radon_sparse_fits(q); }
+static bool generates_matrix(int q) { return q == 13; }
 
 // The stages of a tabulation of prime q, D = 2 or 3, without their tables.  fused: those of D = 3 run as one launch with
 // the table between them in the private exchange buffer.
@@ -933,14 +907,12 @@ static int radon_stages(int q, int D, int transpose, bool fused, StageSpec (&sp)
 int smat_tabulate_tc_supported(const SmatGeo& geo, int64_t state_elems) {
   if ((geo.D != 2 && geo.D != 3) || state_elems % 128) return 0;
   const int q = geo.q;
-  if (q > 64) return 0;
   for (int transpose = 0; transpose < 2; ++transpose) {
     StageSpec sp[2];
     const int stages = radon_stages(q, geo.D, transpose, false, sp);
     for (int i = 0; i < stages; ++i) {
       RadonShape sh;
-      if (!(generates_matrix(q, geo.D, transpose) ? radon_wide_fits(q, sp[i])
-                                                  : radon_shape(q, transpose, sp[i].in.count > q * q, sp[i].out.count, &sh)))
+      if (!(sparse_matrix(q) || (generates_matrix(q) && radon_wide_fits(q, sp[i])) || radon_shape(q, transpose, sp[i].in.count > q * q, sp[i].out.count, &sh)))
         return 0;
     }
   }
@@ -978,7 +950,8 @@ int smat_tabulate_tc_layout_ok(int q) {
     for (int transpose = 0; transpose < 2; ++transpose) {
       const int stages = radon_stages(q, D, transpose, false, sp);
       for (int i = 0; i < stages; ++i) {
-        if (generates_matrix(q, D, transpose)) {
+        if (sparse_matrix(q)) continue;   // (its maps are asserted where it is compiled)
+        if (generates_matrix(q)) {
           if (!radon_wide_layout_ok(q, sp[i])) return 0;
           continue;
         }
@@ -986,7 +959,7 @@ int smat_tabulate_tc_layout_ok(int q) {
         RadonShape sh;
         if (!radon_shape(q, transpose, extra, sp[i].out.count, &sh)) return 0;
         if (!radon_layout_ok(q, sh, sh.ring, 0, 0, extra, sh.smem)) return 0;
-        if (!transpose && sh.nslots == 1 && sh.sr == TILE_ROWS && sh.parts == 1) {
+        if (!transpose && sh.nslots == 1 && sh.sr == TILE_ROWS) {
           const int mini = 2 * ((q + 7) & ~7) * 128, slot = sh.sr * 256;
           int ring = (227 * 1024 - 1024 - 512 - TILE_ROWS * 8) / (slot + mini);
           if (ring > sh.ring) ring = sh.ring;
@@ -1021,9 +994,9 @@ cudaError_t smat_launch_tabulate_tc(const void* in, void* out, void* scratch, co
   }
   *launches = stages;
   for (int i = 0; i < stages; ++i) {
-    const cudaError_t err = generates_matrix(q, geo.D, transpose)
-                                ? launch_radon_wide(q, transpose, sp[i], state_elems, bh, status, st)
-                                : launch_radon(q, transpose, 1, &sp[i], state_elems, bh, status, st);
+    const cudaError_t err = sparse_matrix(q)      ? launch_radon_sparse(q, transpose, sp[i], state_elems, bh, status, st)
+                            : generates_matrix(q) ? launch_radon_wide(q, transpose, sp[i], state_elems, bh, status, st)
+                                                  : launch_radon(q, transpose, 1, &sp[i], state_elems, bh, status, st);
     if (err != cudaSuccess) return err;
   }
   return cudaSuccess;

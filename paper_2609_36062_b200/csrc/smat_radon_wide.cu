@@ -1,11 +1,11 @@
 // Tabulation stages (see smat_radon_tc.cu for the transform) for primes whose Radon matrix fills more than one MMA tile
-// of 128 output indices: q = 13 (182 indices), 17 (306; d = 3 transposed) and, for d = 3, 19 to 53 (380 to 2862).
+// of 128 output indices: q = 13 (182 indices) and, for d = 3, 19 to 53 (380 to 2862).  (q = 17: smat_radon_sparse.cu.)
 //
 // radon_wide_kernel, persistent, one CTA per SM.  An item is one image restricted to 128 consecutive state entries and
 // up to three tiles of outputs, each with an accumulator of 128 columns in tensor memory; the image streams through a
 // ring of 64-row slots (MN-major B operand) and every slot is applied to all the tiles before it is released.  So an
 // image of q <= 19 is loaded by one CTA once, where the kernel with the matrix resident in tensor memory splits the
-// outputs over two or three CTAs that all load it.  The matrix is neither loaded nor kept (3 x 128 x 304 bf16 at q = 17
+// outputs over two or three CTAs that all load it.  The matrix is neither loaded nor kept (3 x 128 x 368 bf16 at q = 19
 // would not fit beside anything else): a row of R has one nonzero per input line, (u - a hi) mod q or (lo + a hi) mod q,
 // which a bit mask of 64 inputs per row and slot holds (worked out once per launch: 1 KB per tile and slot); a thread per
 // output index spreads the mask over 32 columns of the ring of four A tiles that the remaining 128 columns of tensor
