@@ -75,7 +75,7 @@ struct WideItem {
   uint32_t slab, img;
   __device__ __forceinline__ WideItem(const WideParams& p, uint32_t item) {
     img = item / p.slabs;
-    slab = item - img * p.slabs;
+    slab = p.slabs - 1 - (item - img * p.slabs);   // the last heads first: the kernel before has just written them
   }
 };
 

@@ -182,7 +182,8 @@ __global__ void __launch_bounds__(D3Layout<Q>::THREADS, 1) tabulate_d3_f32_kerne
   const WaitCtx wc{cta_abort, prm.status};
   const uint32_t my_slabs = prm.slabs > blockIdx.x ? (prm.slabs - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
   auto start_load = [&](uint32_t ks) {   // slab ks of this CTA into buffer ks % NBUF; one thread calls this
-    const uint32_t buf = ks % NBUF, slab = blockIdx.x + ks * gridDim.x, head = slab / (uint32_t)prm.slabs_per_head;
+    // (the last heads first: the kernel before has just written them)
+    const uint32_t buf = ks % NBUF, slab = prm.slabs - 1 - (blockIdx.x + ks * gridDim.x), head = slab / (uint32_t)prm.slabs_per_head;
     const int e0 = (int)(slab - head * prm.slabs_per_head) * L::ENTRIES;
     started[buf] = ks;
     mbar_expect_tx(slab_full + buf, L::SLAB_BYTES);   // (rows past the last point arrive as zeros)
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(D3Layout<Q>::THREADS, 1) tabulate_d3_f32_kerne
     if (id >= total) break;
     const uint32_t ks = id / L::TASKS, buf = ks % NBUF;
     const int task = (int)(id - ks * L::TASKS);
-    const uint32_t slab = blockIdx.x + ks * gridDim.x, head = slab / (uint32_t)prm.slabs_per_head;
+    const uint32_t slab = prm.slabs - 1 - (blockIdx.x + ks * gridDim.x), head = slab / (uint32_t)prm.slabs_per_head;
     const int64_t e0 = (int64_t)(slab - head * prm.slabs_per_head) * L::ENTRIES + lane * L::EPT;
     float* u = prm.U + (int64_t)head * prm.B * prm.rp + e0;
     // Loads land out of order, and the warps can hold tasks of more than two slabs: a warp may come to wait for a slab
