@@ -293,13 +293,27 @@ void scan_states(Ctx& cx, const char* name, std::initializer_list<SmatScanJob> j
   for (const SmatScanJob& j : jobs) a.job[a.jobs++] = j;
   SMAT_TRY(cx, name, smat_launch_scan(a, pl->rp, pl->NC, pl->bh, cx.st));
 }
-// Exclusive prefix sums of the segment totals of both blocks.
-void scan_segments(Ctx& cx, float* seg, int64_t nseg0, int64_t nseg) {
+// The two-level causal branch's cut into segments, and its first half: the totals of the segments (none where every block
+// is one segment), and their exclusive prefix sums where a block has more than two.
+struct Segments {
+  int nseg0 = 0, nseg1 = 0;
+};
+Segments segment_totals(Ctx& cx, const void* K, const void* V, int64_t rows0, int64_t rows1, int L) {
   const smat_plan* pl = cx.pl;
-  SmatScanArgs a{};
-  a.jobs = 1;
-  a.job[0] = SmatScanJob{seg, 0, nseg0, nseg0, nseg, 0};
-  SMAT_TRY(cx, "segment_scan", smat_launch_scan(a, pl->rp, nseg, pl->bh, cx.st));
+  const int64_t tiles0 = (rows0 + 127) / 128, tiles1 = (rows1 + 127) / 128;
+  float* seg = cx.f(pl->off_sin);
+  Segments s;
+  smat_segment_counts(tiles0, tiles1, pl->bh, L, &s.nseg0, &s.nseg1);
+  if (s.nseg0 > 1 || s.nseg1 > 1)
+    SMAT_TRY(cx, "segment_state_tc", smat_launch_segment_state_tc(K, V, seg, rows0, rows1, s.nseg0, s.nseg1, pl->bh,
+                                                                  reinterpret_cast<int*>(cx.ws + pl->off_status), cx.st));
+  if (smat_segments_need_scan(s.nseg0, s.nseg1)) {
+    SmatScanArgs a{};
+    a.jobs = 1;
+    a.job[0] = SmatScanJob{seg, 0, s.nseg0, s.nseg0, s.nseg0 + s.nseg1, 0};
+    SMAT_TRY(cx, "segment_scan", smat_launch_scan(a, pl->rp, s.nseg0 + s.nseg1, pl->bh, cx.st));
+  }
+  return s;
 }
 
 smat_status check_common(const smat_plan* pl, const void* ws, size_t ws_bytes, int for_backward) {
@@ -620,16 +634,11 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     pl->tile_states = L < 2;
     pl->kept_tile_states = false;
     if (L >= 2) {  // steps 5-7, two-level: segment totals, scan of the totals, fused per-segment output
-      float* seg = cx.f(pl->off_sin);
-      int nseg0 = 0, nseg1 = 0;
-      smat_segment_counts(tiles0, tiles1, pl->bh, L, &nseg0, &nseg1);
-      const int64_t nseg = nseg0 + nseg1;
       const int64_t rows0 = tiles0 * 128, rows1 = tiles1 * 128;
-      SMAT_TRY(cx, "segment_state_tc", smat_launch_segment_state_tc(K, V, seg, rows0, rows1, nseg0, nseg1, pl->bh, status, cx.st));
-      scan_segments(cx, seg, nseg0, nseg);
+      const Segments sg = segment_totals(cx, K, V, rows0, rows1, L);
       const bool keep = (pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES) != 0;   // a backward will want the per-tile states
-      SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, seg, ylr, 0, lr ? pl->geo.n : pl->T, O,
-                                                                       rows0, rows1, nseg0, nseg1, pl->bh, status, cx.st,
+      SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, cx.f(pl->off_sin), ylr, 0, lr ? pl->geo.n : pl->T, O,
+                                                                       rows0, rows1, sg.nseg0, sg.nseg1, pl->bh, status, cx.st,
                                                                        keep ? cx.ws + pl->off_sin_tiles : nullptr));
       pl->kept_tile_states = keep;
     } else {
@@ -648,7 +657,6 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     // form over tiles of which the last of a block is partial.
     int* status = reinterpret_cast<int*>(cx.ws + pl->off_status);
     float* ylr = cx.f(pl->off_acc);
-    float* seg = cx.f(pl->off_sin);
     const bool lr = !pl->geo.dense_G;
     const int64_t rows0 = lr ? pl->geo.n : pl->T, rows1 = lr ? pl->geo.m : 0;
     if (lr) {
@@ -656,13 +664,9 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
       zero_unrouted(cx, SMAT_GM_TYPE, ylr, 512);
       state_read(cx, "read_type", {read_job(cx, SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, ylr)});
     }
-    int nseg0 = 0, nseg1 = 0;
-    smat_segment_counts((rows0 + 127) / 128, (rows1 + 127) / 128, pl->bh, 2, &nseg0, &nseg1);
-    const int64_t nseg = nseg0 + nseg1;
-    SMAT_TRY(cx, "segment_state_tc", smat_launch_segment_state_tc(K, V, seg, rows0, rows1, nseg0, nseg1, pl->bh, status, cx.st));
-    scan_segments(cx, seg, nseg0, nseg);
-    SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, seg, ylr, 1, lr ? pl->geo.n : pl->T, O, rows0,
-                                                                     rows1, nseg0, nseg1, pl->bh, status, cx.st));
+    const Segments sg = segment_totals(cx, K, V, rows0, rows1, 2);
+    SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, cx.f(pl->off_sin), ylr, 1, lr ? pl->geo.n : pl->T, O, rows0,
+                                                                     rows1, sg.nseg0, sg.nseg1, pl->bh, status, cx.st));
     pl->launches = cx.launches;
     return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;
   }

@@ -240,11 +240,13 @@ cudaError_t smat_launch_routing_lists(const int32_t* prof, const int32_t* type, 
 // Zeroes the row (row_bytes bytes at rows + (bh*T + first + i) * row_bytes) of every token i whose key lies outside [0, G).
 cudaError_t smat_launch_zero_unrouted(const int32_t* key, int64_t count, int64_t G, int64_t first, void* rows, int64_t T,
                                       int row_bytes, int bh, cudaStream_t st);
-// Two-level causal branch: segment totals, then (after an exclusive scan of the totals) per-segment fused output.
+// Two-level causal branch: segment totals, then (after an exclusive scan of the totals, where a block has more than two)
+// per-segment fused output.
 // Block 0 holds rows0 tokens of every head and block 1 the rows1 after them (0: one block, d = 1); the last tile of a
 // block may be partial.
 int smat_segment_tiles(int64_t tiles_block0, int64_t tiles_block1, int bh);
 void smat_segment_counts(int64_t tiles0, int64_t tiles1, int bh, int L, int* nseg0, int* nseg1);
+bool smat_segments_need_scan(int nseg0, int nseg1);
 cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* totals, int64_t rows0, int64_t rows1,
                                          int nseg0, int nseg1, int bh, int* status, cudaStream_t st);
 // ylr_f32 = 0: long-range rows in bf16, blocks of whole tiles.  ylr_f32 = 1: fp32 rows, any blocks, and the state and

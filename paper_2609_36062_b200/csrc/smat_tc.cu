@@ -854,15 +854,9 @@ __global__ void __launch_bounds__(192) segment_state_tc_kernel(const __grid_cons
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int seg = blockIdx.x, bh = blockIdx.y;
-  // The scan is exclusive: nobody reads the total of a block's last segment (the scan loads it after its last store).
-  // Such a CTA still waits for the kernel before: where every block is one segment no other CTA of the launch does, and
-  // the kernels after this one would run beside that kernel.
-  if (seg == prm.cut.nseg0 - 1 || seg == prm.cut.nseg - 1) {
-    pdl_trigger();
-    pdl_wait();
-    return;
-  }
+  // Nobody reads the total of a block's last segment: the launch has no CTAs for it.
+  const int bh = blockIdx.y;
+  const int seg = (int)blockIdx.x < prm.cut.nseg0 - 1 ? blockIdx.x : blockIdx.x + 1;
   int64_t tile0;
   int Lc;
   seg_range(prm.cut, seg, &tile0, &Lc);
@@ -955,7 +949,8 @@ struct SegOutParams {
   int64_t T;
   SegCut cut;
   int nseg;
-  const float* seg_in;   // [bh][nseg][128][128] state entering each segment
+  const float* seg_in;   // [bh][nseg][128][128]: the state entering each segment, or (totals) the segments' totals
+  int totals;            // a block has two segments at most: its second is entered with the first one's total
   int64_t n_lr;
   const __nv_bfloat16* ylr;   // plain: [bh][T][128] long-range rows, bf16 (rows t >= n_lr are added)
   const float* ylr32;         // SPLIT: the same rows in fp32
@@ -1194,11 +1189,17 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
     };
     {  // state entering the segment: global fp32 -> TMEM (accumulator) and the shared tile
       uint32_t v[32];
-      const uint4* src = reinterpret_cast<const uint4*>(prm.seg_in + (((int64_t)bh * prm.nseg + seg) * TILE + m) * TILE + col0);
+      const int from = prm.totals ? seg - 1 : seg;
+      if (prm.totals && (seg == 0 || seg == prm.cut.nseg0)) {
 #pragma unroll
-      for (int q4 = 0; q4 < 8; ++q4) {
-        const uint4 a = *(src + q4);
-        v[4 * q4] = a.x; v[4 * q4 + 1] = a.y; v[4 * q4 + 2] = a.z; v[4 * q4 + 3] = a.w;
+        for (int e = 0; e < 32; ++e) v[e] = 0u;
+      } else {
+        const uint4* src = reinterpret_cast<const uint4*>(prm.seg_in + (((int64_t)bh * prm.nseg + from) * TILE + m) * TILE + col0);
+#pragma unroll
+        for (int q4 = 0; q4 < 8; ++q4) {
+          const uint4 a = *(src + q4);
+          v[4 * q4] = a.x; v[4 * q4 + 1] = a.y; v[4 * q4 + 2] = a.z; v[4 * q4 + 3] = a.w;
+        }
       }
       tmem_st32(tmem_s + lane_base + col0, v);
       tmem_st_wait();
@@ -1987,6 +1988,11 @@ static SegCut segment_cut(int64_t rows0, int64_t rows1, int nseg0, int nseg1) {
   return c;
 }
 
+// Up to two segments per block: the output CTA of the second reads the first one's total, and there is nothing to scan (the
+// pass, 32 heads of 4096 tokens, d = 3: 206 -> 199 us; 128 heads of 8192: the scan's 21 us).  With four segments the sums at
+// the head of the output CTAs take longer than the scan (32 heads of 16 K tokens: output 141 -> 160 us, scan 10).
+bool smat_segments_need_scan(int nseg0, int nseg1) { return nseg0 > 2 || nseg1 > 2; }
+
 cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* totals, int64_t rows0, int64_t rows1,
                                          int nseg0, int nseg1, int bh, int* status, cudaStream_t st) {
   const int64_t T = rows0 + rows1;
@@ -1998,7 +2004,7 @@ cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* to
   cudaError_t err =
       cudaFuncSetAttribute(segment_state_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SEG_STATE_SMEM);
   if (err != cudaSuccess) return err;
-  dim3 grid((unsigned)prm.nseg, (unsigned)bh);
+  dim3 grid((unsigned)(nseg0 - 1 + (nseg1 > 0 ? nseg1 - 1 : 0)), (unsigned)bh);
   return smat_launch_pdl(segment_state_tc_kernel, grid, 192, SEG_STATE_SMEM, st, tmK, tmV, prm);
 }
 
@@ -2016,7 +2022,7 @@ cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const vo
     if (rows1 && !make_block_map(&dst[i][1], base + rows0 * TILE, (uint64_t)rows1, (uint64_t)T, (uint64_t)bh)) return cudaErrorInvalidValue;
   }
   SegOutParams prm;
-  prm.T = T; prm.nseg = nseg0 + nseg1; prm.seg_in = seg_in; prm.n_lr = n_lr;
+  prm.T = T; prm.nseg = nseg0 + nseg1; prm.seg_in = seg_in; prm.totals = !smat_segments_need_scan(nseg0, nseg1); prm.n_lr = n_lr;
   prm.ylr = static_cast<const __nv_bfloat16*>(ylr);
   prm.ylr32 = static_cast<const float*>(ylr);
   prm.cut = segment_cut(rows0, rows1, nseg0, nseg1);
