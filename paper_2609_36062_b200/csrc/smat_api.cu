@@ -122,6 +122,8 @@ smat_status build_geometry(SmatGeo* g, int64_t T, int64_t c, int d, int q_overri
 SmatGroupSpec group(const smat_plan* pl, int mode) {
   SmatGroupSpec s; s.mode = mode; s.n = pl->geo.n; s.T = pl->T; s.c = pl->c;
   s.period = mode == SMAT_GM_PROFILE ? pl->geo.P : pl->geo.B;
+  const int64_t tokens = mode == SMAT_GM_PROFILE ? s.n : s.T - s.n;
+  s.base = tokens / s.period; s.rem = tokens % s.period;
   s.list = nullptr; s.offs = nullptr; s.list_stride = 0; s.offs_stride = 0;
   return s;
 }

@@ -16,6 +16,7 @@ enum SmatGroupMode { SMAT_GM_NONE = 0, SMAT_GM_CHUNK = 1, SMAT_GM_PROFILE = 2, S
 struct SmatGroupSpec {
   int mode;
   int64_t n, T, c, period;  // period = P (PROFILE) or B (TYPE)
+  int64_t base, rem;        // the block's tokens = base * period + rem: a group has base or base + 1 of them
   // User-supplied routing (content-based assignment, Sec. 3): when `list` is non-null the tokens of PROFILE / TYPE
   // group g of head bh are list[bh * list_stride + offs[bh * offs_stride + g] ...  offs[... + g + 1]) (token positions
   // in [0, T), ascending inside a group) instead of the positional strides.
@@ -23,6 +24,12 @@ struct SmatGroupSpec {
   const int32_t* offs;
   int64_t list_stride, offs_stride;
 };
+
+// a / b of non-negative numbers; a 64-bit division takes the device several hundred cycles, and every role of a persistent
+// kernel makes one per item.
+SMAT_HD int64_t smat_div(int64_t a, int64_t b) {
+  return ((uint64_t)(a | b) >> 32) == 0 ? (int64_t)((uint32_t)a / (uint32_t)b) : a / b;
+}
 
 // The tokens of one group: position of the k-th one is at(k).
 struct SmatTokens {
@@ -45,12 +52,11 @@ SMAT_HD SmatTokens smat_group_tokens(const SmatGroupSpec& s, int64_t bh, int64_t
       r.t0 = g * s.c; r.ts = 1; r.cnt = s.c;
       break;
     case SMAT_GM_PROFILE:
-      r.t0 = g; r.ts = s.period; r.cnt = g < s.n ? (s.n - g + s.period - 1) / s.period : 0;
+      r.t0 = g; r.ts = s.period; r.cnt = s.base + (g < s.rem);
       break;
     case SMAT_GM_TYPE: {
       int64_t i0 = g ? g : s.period;  // paper's 1-based recent index of the first token of this type
-      int64_t m = s.T - s.n;
-      r.t0 = s.n + i0 - 1; r.ts = s.period; r.cnt = i0 <= m ? (m - i0) / s.period + 1 : 0;
+      r.t0 = s.n + i0 - 1; r.ts = s.period; r.cnt = s.base + (i0 <= s.rem);
       break;
     }
     default:

@@ -67,7 +67,7 @@ struct PoolCursor {
     if (!valid()) return;
     while (item >= l->first[job + 1]) ++job;
     const int64_t at = item - l->first[job];
-    bh = at / l->a.job[job].groups;
+    bh = smat_div(at, l->a.job[job].groups);
     tk = smat_group_tokens(l->a.job[job].grp, bh, at - bh * l->a.job[job].groups);
     cnt = tk.cnt;
   }
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
   };
   auto tokens_of = [&](int64_t item, int j, int64_t* bh) {
     const int64_t at = item - list.first[j];
-    *bh = at / list.a.job[j].groups;
+    *bh = smat_div(at, list.a.job[j].groups);
     return smat_group_tokens(list.a.job[j].grp, *bh, at - *bh * list.a.job[j].groups);
   };
   auto state_of = [&](int64_t item) {

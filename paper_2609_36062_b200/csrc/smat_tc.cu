@@ -1334,7 +1334,7 @@ struct ReadPass {
   __device__ void load() {
     k0 = 0;
     for (; item < pp->items; item += stride) {
-      bh = item / pp->groups;
+      bh = smat_div(item, pp->groups);
       tk = smat_group_tokens(pp->grp, bh, item - bh * pp->groups);
       cnt = tk.cnt;
       if (cnt > 0) break;
@@ -1536,7 +1536,7 @@ struct PoolPass {
   __device__ void load() {
     k0 = 0;
     if (item < pp->items) {
-      bh = item / pp->groups;
+      bh = smat_div(item, pp->groups);
       tk = smat_group_tokens(pp->grp, bh, item - bh * pp->groups);
       cnt = tk.cnt;
     }
