@@ -138,6 +138,7 @@ struct Ctx {
   cudaError_t err;
   int launches;
   const smat_plan* rec = nullptr;   // plan whose stage timer records the launches (default: pl)
+  int* clear = nullptr;   // status word that the first pooling launch of the pass sets to zero (see begin_pass)
   bool routed = false;   // profile / type groups come from the token lists in the workspace, not from positions
   const int32_t* prof = nullptr;   // the caller's arrays of a routed call
   const int32_t* type = nullptr;
@@ -166,6 +167,17 @@ cudaError_t clear_status(const Ctx& cx) {
   if (err == cudaSuccess && pl->inner)
     err = cudaMemsetAsync(cx.ws + pl->off_inner + pl->inner->off_status, 0, 256, cx.st);
   return err;
+}
+
+// The same, left to the pooling launch where the pass begins with it (a memset among a few short launches costs as much as
+// one of them).
+void begin_pass(Ctx& cx, bool pools_first) {
+  if (pools_first && !cx.pl->inner) {
+    cx.pl->kept_gated_forward = false;
+    cx.clear = reinterpret_cast<int*>(cx.ws + cx.pl->off_status);
+  } else {
+    cx.err = clear_status(cx);
+  }
 }
 
 void mark_stage(const smat_plan* pl, cudaStream_t st, const char* name) {
@@ -217,7 +229,8 @@ void pool(Ctx& cx, const char* name, std::initializer_list<SmatPoolJob> jobs) {
   const smat_plan* pl = cx.pl;
   SmatPoolArgs a{};
   for (const SmatPoolJob& j : jobs) a.job[a.jobs++] = j;
-  SMAT_TRY(cx, name, smat_launch_pool(a, pl->dtype == SMAT_BF16, pl->T, pl->bh, pl->r, pl->p, cx.st));
+  SMAT_TRY(cx, name, smat_launch_pool(a, pl->dtype == SMAT_BF16, pl->T, pl->bh, pl->r, pl->p, cx.clear, cx.st));
+  cx.clear = nullptr;
 }
 void outer_sum(Ctx& cx, const char* name, int mode, const void* a, const void* b, float* state) {
   pool(cx, name, {pool_job(cx, mode, a, b, state)});
@@ -230,12 +243,16 @@ SmatReadJob read_job(const Ctx& cx, int mode, const void* x, const float* state,
   j.x = x; j.state = state; j.out = out; j.grp = group(cx, mode); j.groups = group_count(cx.pl, mode); j.trans = transposed;
   return j;
 }
-void state_read(Ctx& cx, const char* name, std::initializer_list<SmatReadJob> jobs) {
+// scans: chunk states that the same launch scans
+void state_read(Ctx& cx, const char* name, std::initializer_list<SmatReadJob> jobs, std::initializer_list<SmatScanJob> scans = {}) {
   const smat_plan* pl = cx.pl;
   SmatReadArgs a{};
+  SmatScanArgs sc{};
   for (const SmatReadJob& j : jobs) a.job[a.jobs++] = j;
+  for (const SmatScanJob& j : scans) sc.job[sc.jobs++] = j;
   SMAT_TRY(cx, name, smat_launch_state_read(a, pl->dtype == SMAT_BF16, pl->T, pl->bh, pl->r, pl->p,
-                                            reinterpret_cast<int*>(cx.ws + pl->off_status), cx.st));
+                                            reinterpret_cast<int*>(cx.ws + pl->off_status), cx.st, sc.jobs ? &sc : nullptr,
+                                            pl->NC));
 }
 
 // The within-chunk tiles of one output (see tile_rows_kernel); acc rows acc_lo <= t < acc_hi are added.
@@ -612,7 +629,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
   if (!device_ok()) return SMAT_ERR_ARCH;
   Ctx cx{pl, static_cast<cudaStream_t>(cuda_stream), static_cast<char*>(workspace), cudaSuccess, 0};
   pl->stages = 0;
-  cx.err = clear_status(cx);
+  begin_pass(cx, !prof && !type && !pl->tc && !(pl->ragged_tc && pl->geo.dense_G));
   s = begin_routing(cx, prof, type);
   if (s != SMAT_OK) return s;
   if (pl->tc) {
@@ -678,11 +695,12 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
   const SmatPoolJob chunks = pool_job(cx, SMAT_GM_CHUNK, K, V, sin);
   if (lr) pool(cx, "pool", {pool_job(cx, SMAT_GM_PROFILE, K, V, cx.f(pl->off_F)), chunks});           // steps 2, 5
   else pool(cx, "pool", {chunks});
-  scan_states(cx, "scan", {scan_job(cx, sin, 0)});                                                   // step 6
   if (lr) {
     tabulate(cx, "tabulate", cx.f(pl->off_F), cx.f(pl->off_U), 0);                                   // step 3
     zero_unrouted(cx, SMAT_GM_TYPE, acc, pl->p * 4);
-    state_read(cx, "read_type", {read_job(cx, SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, acc)});           // step 4
+    state_read(cx, "read_type", {read_job(cx, SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, acc)}, {scan_job(cx, sin, 0)});   // steps 4, 6
+  } else {
+    scan_states(cx, "scan", {scan_job(cx, sin, 0)});                                                 // step 6
   }
   tile_rows(cx, "tiles", pl->r, pl->p, {tile_job(Q, K, V, Q, sin, 0, 0, acc, lr ? pl->geo.n : pl->T, pl->T, O)}, nullptr);   // step 7
   pl->launches = cx.launches;
@@ -701,7 +719,7 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
   if (!device_ok()) return SMAT_ERR_ARCH;
   Ctx cx{pl, static_cast<cudaStream_t>(cuda_stream), static_cast<char*>(workspace), cudaSuccess, 0};
   pl->stages = 0;
-  cx.err = clear_status(cx);
+  begin_pass(cx, !prof && !type && !pl->tc);
   s = begin_routing(cx, prof, type);
   if (s != SMAT_OK) return s;
   const bool lr = !pl->geo.dense_G;
@@ -815,8 +833,9 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
   if (lr) pool(cx, "bwd_pool", {pool_job(cx, SMAT_GM_PROFILE, K, V, cx.f(pl->off_F)), cf, cb,
                                 pool_job(cx, SMAT_GM_TYPE, Q, dO, cx.f(pl->off_ubar))});
   else pool(cx, "bwd_pool", {cf, cb});
-  scan_states(cx, "bwd_scan", {scan_job(cx, sin, 0), scan_job(cx, dbar, 1)});
-  if (lr) {
+  if (!lr) {
+    scan_states(cx, "bwd_scan", {scan_job(cx, sin, 0), scan_job(cx, dbar, 1)});
+  } else {
     tabulate(cx, "tabulate", cx.f(pl->off_F), cx.f(pl->off_U), 0);
     tabulate(cx, "bwd_tabulate_t", cx.f(pl->off_ubar), cx.f(pl->off_fbar), 1);
     // dQ's long-range rows are recent and dK's distant: they share a buffer
@@ -825,7 +844,8 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
     zero_unrouted(cx, SMAT_GM_PROFILE, acc_v, pl->p * 4);
     state_read(cx, "bwd_reads", {read_job(cx, SMAT_GM_TYPE, dO, cx.f(pl->off_U), 1, acc),
                                  read_job(cx, SMAT_GM_PROFILE, V, cx.f(pl->off_fbar), 1, acc),
-                                 read_job(cx, SMAT_GM_PROFILE, K, cx.f(pl->off_fbar), 0, acc_v)});
+                                 read_job(cx, SMAT_GM_PROFILE, K, cx.f(pl->off_fbar), 0, acc_v)},
+               {scan_job(cx, sin, 0), scan_job(cx, dbar, 1)});
   }
   const int64_t n = lr ? pl->geo.n : 0, from = lr ? n : pl->T;
   adjoint_tiles(cx, "bwd_tiles", tile_job(dO, V, K, dO, sin, 1, 0, acc, from, pl->T, dQ),

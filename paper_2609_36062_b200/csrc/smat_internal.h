@@ -129,7 +129,8 @@ struct SmatPoolArgs {
   SmatPoolJob job[4];
   int jobs;
 };
-cudaError_t smat_launch_pool(const SmatPoolArgs& a, int bf16, int64_t Tlen, int bh, int r, int p, cudaStream_t st);
+// clear (or null): status word that the launch sets to zero.
+cudaError_t smat_launch_pool(const SmatPoolArgs& a, int bf16, int64_t Tlen, int bh, int r, int p, int* clear, cudaStream_t st);
 
 // Routed reads of per-group fp32 states [r][p]: out[t] = x_t · state[g(t)] for the tokens of every group (trans: the
 // second state index is contracted), fp32 rows, for up to three sets in one launch.
@@ -145,8 +146,9 @@ struct SmatReadArgs {
   SmatReadJob job[3];
   int jobs;
 };
+// scan (or null): chunk states, NC of r x p to a head, that CTAs of the same launch scan (as smat_launch_scan would).
 cudaError_t smat_launch_state_read(const SmatReadArgs& a, int bf16, int64_t Tlen, int bh, int r, int p, int* status,
-                                   cudaStream_t st);
+                                   cudaStream_t st, const SmatScanArgs* scan = nullptr, int64_t NC = 0);
 
 // Both stages of the d = 4 tabulation with the table between them in shared memory (the primes for which it fits).
 int smat_tabulate_slab_supported(int q, int64_t state_elems);

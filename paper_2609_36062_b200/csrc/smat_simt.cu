@@ -5,6 +5,7 @@
 
 #include "smat_internal.h"
 #include "smat_launch.cuh"
+#include "smat_scan.cuh"
 #include "smat_tc.cuh"
 
 namespace {
@@ -226,37 +227,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) tile_rows_kernel(const __grid
 }
 
 // ---- scan --------------------------------------------------------------------------------------
-// Each thread owns four consecutive state entries and walks the chunks of its range in order.
-// Loads are issued sixteen chunks ahead of the dependent additions.
 __global__ void __launch_bounds__(256) scan_kernel(const __grid_constant__ SmatScanArgs a, int64_t state_elems, int64_t NC) {
   pdl_trigger();
-  const int64_t e4 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e4 * 4 >= state_elems) return;
-  const int64_t bh = blockIdx.y;
-  const SmatScanJob& job = a.job[blockIdx.z >> 1];
-  const int range = blockIdx.z & 1, reverse = job.reverse;
-  const int64_t lo = range ? job.lo1 : job.lo0, hi = range ? job.hi1 : job.hi0;
-  float4* base = reinterpret_cast<float4*>(job.S + bh * NC * state_elems) + e4;
-  const int64_t stride4 = state_elems / 4;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  constexpr int AHEAD = 16;
   pdl_wait();
-  for (int64_t s = 0; s < hi - lo; s += AHEAD) {
-    float4 v[AHEAD];
-#pragma unroll
-    for (int u = 0; u < AHEAD; ++u) {
-      const int64_t k = s + u;
-      if (k < hi - lo) v[u] = base[(reverse ? hi - 1 - k : lo + k) * stride4];
-    }
-#pragma unroll
-    for (int u = 0; u < AHEAD; ++u) {
-      const int64_t k = s + u;
-      if (k < hi - lo) {
-        base[(reverse ? hi - 1 - k : lo + k) * stride4] = acc;
-        acc.x += v[u].x; acc.y += v[u].y; acc.z += v[u].z; acc.w += v[u].w;
-      }
-    }
-  }
+  smat_scan_entries(a, state_elems, NC, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y, blockIdx.z);
 }
 
 // ---- Algorithm 2, direct form ------------------------------------------------------------------------

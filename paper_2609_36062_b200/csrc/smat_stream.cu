@@ -11,6 +11,7 @@
 
 #include "smat_internal.h"
 #include "smat_launch.cuh"
+#include "smat_scan.cuh"
 #include "smat_tc.cuh"
 
 namespace {
@@ -93,8 +94,9 @@ struct PoolCursor {
 
 // Two token buffers alternate over the passes, also inside a group of many tokens: the next pass's rows (of the same
 // group or of the next item) travel while this pass is summed.
+// clear (or null): the status word of a pass that begins with this launch, which waits for nothing that could fail.
 template <int R, int PD, typename T>
-__global__ void __launch_bounds__(256) pool_stream_kernel(const __grid_constant__ PoolList list, int64_t Tlen) {
+__global__ void __launch_bounds__(256) pool_stream_kernel(const __grid_constant__ PoolList list, int64_t Tlen, int* clear) {
   constexpr int TK = sizeof(T) == 2 ? 32 : 16;  // tokens staged per pass
   constexpr int NJ4 = PD / 4;
   constexpr int NG = 256 / NJ4;
@@ -128,6 +130,7 @@ __global__ void __launch_bounds__(256) pool_stream_kernel(const __grid_constant_
   };
 
   pdl_wait();   // (the token lists of a routed call come from the kernel before)
+  if (clear && blockIdx.x == 0 && tid == 0) *clear = 0;
   PoolCursor<TK> cur(list, blockIdx.x, gridDim.x);
   fetch(cur, 0);
   float4 acc[NS];
@@ -179,6 +182,11 @@ __global__ void __launch_bounds__(256) pool_stream_kernel(const __grid_constant_
 struct ReadList {
   SmatReadArgs a;
   int64_t first[4];
+  // Chunk states that the tile kernel behind the read will want scanned: the first scan_ctas CTAs of the launch do that
+  // (a sequence of launches of a few CTAs each is bound by their number).
+  SmatScanArgs scan;
+  int64_t NC;
+  int32_t scan_x, scan_y, scan_ctas;   // CTAs per head and (job, range); heads; all of them
 };
 
 // Two CTAs share an SM; each owns one 64 KB state buffer in two halves of rows: the next item's first half is under way
@@ -210,9 +218,15 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
   pdl_trigger();
   const tc::WaitCtx wc{cta_abort, status};
   const int tid = threadIdx.x;
+  if ((int)blockIdx.x < list.scan_ctas) {
+    pdl_wait();
+    const int x = blockIdx.x % list.scan_x, yz = blockIdx.x / list.scan_x;
+    smat_scan_entries(list.scan, R * PD, list.NC, x * 256 + tid, yz % list.scan_y, yz / list.scan_y);
+    return;
+  }
   const int j4 = tid % NJ4, ig = tid / NJ4;
   constexpr uint32_t HBYTES = R * PD * 2;   // half a state
-  const int64_t items = list.first[list.a.jobs], cta = blockIdx.x, ctas = gridDim.x;
+  const int64_t items = list.first[list.a.jobs], cta = blockIdx.x - list.scan_ctas, ctas = gridDim.x - list.scan_ctas;
   auto job_of = [&](int64_t item) {
     int j = 0;
     while (item >= list.first[j + 1]) ++j;
@@ -396,7 +410,7 @@ int sm_count() {
 }
 
 template <int R, int PD, typename T>
-cudaError_t launch_pool(const PoolList& list, int64_t Tlen, cudaStream_t st) {
+cudaError_t launch_pool(const PoolList& list, int64_t Tlen, int* clear, cudaStream_t st) {
   constexpr int TK = sizeof(T) == 2 ? 32 : 16;
   const size_t smem = R * PD * 4 + 2 * TK * (R + PD) * sizeof(T);
   cudaError_t err = set_smem(pool_stream_kernel<R, PD, T>, smem);
@@ -404,7 +418,7 @@ cudaError_t launch_pool(const PoolList& list, int64_t Tlen, cudaStream_t st) {
   const int64_t items = list.first[list.a.jobs];
   const int per_sm = smem <= 110 * 1024 ? 2 : 1;
   const int64_t grid = items < (int64_t)sm_count() * per_sm ? items : (int64_t)sm_count() * per_sm;
-  return smat_launch_pdl(pool_stream_kernel<R, PD, T>, dim3((unsigned)grid), 256, smem, st, list, Tlen);
+  return smat_launch_pdl(pool_stream_kernel<R, PD, T>, dim3((unsigned)grid), 256, smem, st, list, Tlen, clear);
 }
 
 template <int R, int PD, typename T>
@@ -415,28 +429,33 @@ cudaError_t launch_read(const ReadList& list, int64_t Tlen, int* status, cudaStr
   const int64_t items = list.first[list.a.jobs];
   const int per_sm = smem <= 112 * 1024 ? 2 : 1;
   const int64_t grid = items < (int64_t)sm_count() * per_sm ? items : (int64_t)sm_count() * per_sm;
-  return smat_launch_pdl(state_read_stream_kernel<R, PD, T>, dim3((unsigned)grid), 256, smem, st, list, Tlen, status);
+  return smat_launch_pdl(state_read_stream_kernel<R, PD, T>, dim3((unsigned)(grid + list.scan_ctas)), 256, smem, st, list, Tlen, status);
 }
 
 }  // namespace
 
-cudaError_t smat_launch_pool(const SmatPoolArgs& a, int bf16, int64_t Tlen, int bh, int r, int p, cudaStream_t st) {
+cudaError_t smat_launch_pool(const SmatPoolArgs& a, int bf16, int64_t Tlen, int bh, int r, int p, int* clear, cudaStream_t st) {
   PoolList list;
   list.a = a;
   list.first[0] = 0;
   for (int j = 0; j < a.jobs; ++j) list.first[j + 1] = list.first[j] + a.job[j].groups * bh;
 #define SMAT_POOL(RV, PV)                                                                                          \
   if (r == RV && p == PV)                                                                                          \
-    return bf16 ? launch_pool<RV, PV, __nv_bfloat16>(list, Tlen, st) : launch_pool<RV, PV, float>(list, Tlen, st);
+    return bf16 ? launch_pool<RV, PV, __nv_bfloat16>(list, Tlen, clear, st) : launch_pool<RV, PV, float>(list, Tlen, clear, st);
   SMAT_POOL(128, 128) SMAT_POOL(64, 64) SMAT_POOL(64, 128) SMAT_POOL(128, 64)
 #undef SMAT_POOL
   return cudaErrorInvalidValue;
 }
 
 cudaError_t smat_launch_state_read(const SmatReadArgs& a, int bf16, int64_t Tlen, int bh, int r, int p, int* status,
-                                   cudaStream_t st) {
-  ReadList list;
+                                   cudaStream_t st, const SmatScanArgs* scan, int64_t NC) {
+  ReadList list{};
   list.a = a;
+  if (scan) {
+    list.scan = *scan; list.NC = NC;
+    list.scan_x = (r * p / 4 + 255) / 256; list.scan_y = bh;
+    list.scan_ctas = list.scan_x * bh * 2 * scan->jobs;
+  }
   list.first[0] = 0;
   for (int j = 0; j < a.jobs; ++j) list.first[j + 1] = list.first[j] + a.job[j].groups * bh;
 #define SMAT_READ(RV, PV)                                                                        \
