@@ -169,10 +169,12 @@ cudaError_t clear_status(const Ctx& cx) {
   return err;
 }
 
-// The same, left to the pooling launch where the pass begins with it (a memset among a few short launches costs as much as
-// one of them).
-void begin_pass(Ctx& cx, bool pools_first) {
-  if (pools_first && !cx.pl->inner) {
+// The same, left to the pooling launch where the pass begins with it and has an SM for each of its `pooled` states per head:
+// a memset among a few short launches costs as much as one of them.  (More CTAs than SMs are better placed after it: those
+// that start while the pass before drains crowd the SMs that are free first.  d = 1, 8 heads of 2048 tokens, 64 wide, chunk
+// 32, forward and backward: 119 us with the memset, 133 without.)
+void begin_pass(Ctx& cx, bool pools_first, int64_t pooled) {
+  if (pools_first && !cx.pl->inner && smat_pool_one_round(pooled * cx.pl->bh)) {
     cx.pl->kept_gated_forward = false;
     cx.clear = reinterpret_cast<int*>(cx.ws + cx.pl->off_status);
   } else {
@@ -629,7 +631,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
   if (!device_ok()) return SMAT_ERR_ARCH;
   Ctx cx{pl, static_cast<cudaStream_t>(cuda_stream), static_cast<char*>(workspace), cudaSuccess, 0};
   pl->stages = 0;
-  begin_pass(cx, !prof && !type && !pl->tc && !(pl->ragged_tc && pl->geo.dense_G));
+  begin_pass(cx, !prof && !type && !pl->tc && !(pl->ragged_tc && pl->geo.dense_G), pl->NC + (pl->geo.dense_G ? 0 : pl->geo.P));
   s = begin_routing(cx, prof, type);
   if (s != SMAT_OK) return s;
   if (pl->tc) {
@@ -719,7 +721,7 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
   if (!device_ok()) return SMAT_ERR_ARCH;
   Ctx cx{pl, static_cast<cudaStream_t>(cuda_stream), static_cast<char*>(workspace), cudaSuccess, 0};
   pl->stages = 0;
-  begin_pass(cx, !prof && !type && !pl->tc);
+  begin_pass(cx, !prof && !type && !pl->tc, 2 * pl->NC + (pl->geo.dense_G ? 0 : pl->geo.P + pl->geo.B));
   s = begin_routing(cx, prof, type);
   if (s != SMAT_OK) return s;
   const bool lr = !pl->geo.dense_G;

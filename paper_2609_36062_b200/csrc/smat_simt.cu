@@ -18,17 +18,16 @@ using tc::cp_async_wait;
 // Out[i] = Σ_j X_ij P3_j + P4_i · St (+ addend row),   X_ij = P1_i · P2_j where j <= i (upper: j >= i) in i's chunk:
 //     O  : P1 = Q,  P2 = K,  P3 = V,  P4 = Q,  St = S_in              dQ : P1 = dO, P2 = V,  P3 = K,  P4 = dO, St = S_inᵀ
 //     dK : P1 = V,  P2 = dO, P3 = Q,  P4 = V,  St = D̄ᵀ (upper)        dV : P1 = K,  P2 = Q,  P3 = dO, P4 = K,  St = D̄ (upper)
-// (Eq. "local", Eq. "local-adjoint" with the broadcast of the scanned states.)  A CTA takes 32 rows of one chunk: the
+// (Eq. "local", Eq. "local-adjoint" with the broadcast of the scanned states.)  A CTA takes 32 or 16 rows of one chunk: the
 // scores of 64 columns at a time go through shared memory, two operand buffers alternate between the next columns'
 // P2 / P3 and the 64-row pieces of the state, fetched while the other one is used.  Everything is fp32.
 // One launch serves the forward tile, or the three adjoints (jobs).  What it replaces — scores, state product and
 // tile product as separate launches of a general 64 x 64 product, with the score tiles in memory — took 21 launches
 // and 259 us for forward + backward of one 512-token head (64 wide, chunk 64).
-constexpr int ROWS = 32;      // rows per CTA
 constexpr int COLS = 64;      // score columns per step, and rows of a state piece
 constexpr int TILE_THREADS = 256;
 
-template <typename T, int SD, int OD>
+template <typename T, int SD, int OD, int ROWS>
 struct TileLayout {
   static constexpr int SROW = SD * (int)sizeof(T) + 16;   // bytes per staged row (padded by one 16-byte chunk)
   static constexpr int OROW = OD * (int)sizeof(T) + 16;
@@ -60,9 +59,10 @@ __device__ __forceinline__ float4 fma4(float s, const float4 b, float4 a) {
   return a;
 }
 
-template <typename T, int SD, int OD>
+template <typename T, int SD, int OD, int ROWS>
 __global__ void __launch_bounds__(TILE_THREADS, 2) tile_rows_kernel(const __grid_constant__ SmatTileArgs a) {
-  using L = TileLayout<T, SD, OD>;
+  using L = TileLayout<T, SD, OD, ROWS>;
+  constexpr int SR = ROWS / 16;   // score rows per thread
   extern __shared__ __align__(16) uint8_t smem[];
   pdl_trigger();
   uint8_t *s1 = smem, *s4 = smem + L::OFF_P4, *sA = smem + L::OFF_A, *sB = smem + L::OFF_B;
@@ -132,37 +132,37 @@ __global__ void __launch_bounds__(TILE_THREADS, 2) tile_rows_kernel(const __grid
     const int cols = cols_of(kb);
     cp_async_wait<1>();
     __syncthreads();
-    {   // scores: two rows x four columns per thread
+    {   // scores: SR rows x four columns per thread
       const int ty = tid >> 4, tx = tid & 15;
-      float x[2][4];
+      float x[SR][4];
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
+      for (int i = 0; i < SR; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) x[i][j] = 0.f;
 #pragma unroll 4
       for (int k = 0; k < SD; k += 4) {
-        float4 av[2], bv[4];
+        float4 av[SR], bv[4];
 #pragma unroll
-        for (int i = 0; i < 2; ++i) av[i] = ld4(reinterpret_cast<const T*>(s1 + (ty * 2 + i) * L::SROW) + k);
+        for (int i = 0; i < SR; ++i) av[i] = ld4(reinterpret_cast<const T*>(s1 + (ty * SR + i) * L::SROW) + k);
 #pragma unroll
         for (int j = 0; j < 4; ++j) bv[j] = ld4(reinterpret_cast<const T*>(sA + (tx + 16 * j) * L::SROW) + k);
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
+        for (int i = 0; i < SR; ++i)
 #pragma unroll
           for (int j = 0; j < 4; ++j) x[i][j] = dot4(av[i], bv[j], x[i][j]);
       }
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
+      for (int i = 0; i < SR; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const int m = m0 + ty * 2 + i, n = kb * COLS + tx + 16 * j;   // positions inside the chunk
+          const int m = m0 + ty * SR + i, n = kb * COLS + tx + 16 * j;   // positions inside the chunk
           const bool in = m < a.c && n < a.c && (job.upper ? n >= m : n <= m);
           float v = in ? x[i][j] : 0.f;
           if (a.lam && in) {   // gated: decay between the key's and the query's position
             const float* l = a.lam + row0;
             v *= job.upper ? __expf(l[n] - l[m]) : __expf(l[m] - l[n]);
           }
-          sX[(ty * 2 + i) * L::XROW + tx + 16 * j] = v;
+          sX[(ty * SR + i) * L::XROW + tx + 16 * j] = v;
         }
     }
     __syncthreads();
@@ -319,10 +319,10 @@ __global__ void mask_kernel(uint8_t* mask, const SmatGeo geo) {
 
 }  // namespace
 
-template <typename T, int SD, int OD>
-static cudaError_t launch_tile_rows(SmatTileArgs a, int bh, cudaStream_t st) {
-  constexpr int smem = TileLayout<T, SD, OD>::SMEM;
-  cudaError_t err = cudaFuncSetAttribute(tile_rows_kernel<T, SD, OD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+template <typename T, int SD, int OD, int ROWS>
+static cudaError_t launch_tile_rows_of(SmatTileArgs a, int bh, cudaStream_t st) {
+  constexpr int smem = TileLayout<T, SD, OD, ROWS>::SMEM;
+  cudaError_t err = cudaFuncSetAttribute(tile_rows_kernel<T, SD, OD, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
   const unsigned blocks = (unsigned)((a.c + ROWS - 1) / ROWS);
   const size_t rows = (size_t)bh * a.T * sizeof(T);
@@ -331,7 +331,14 @@ static cudaError_t launch_tile_rows(SmatTileArgs a, int bh, cudaStream_t st) {
     if (smat_overlap(a.job[j].out, rows * OD, a.job[j].p2, rows * SD) || smat_overlap(a.job[j].out, rows * OD, a.job[j].p3, rows * OD))
       a.together = 1;
   const dim3 grid((unsigned)(a.jobs * a.NC) * blocks, (unsigned)bh);
-  return smat_launch_pdl_cluster(tile_rows_kernel<T, SD, OD>, grid, TILE_THREADS, smem, a.together ? blocks : 1u, st, a);
+  return smat_launch_pdl_cluster(tile_rows_kernel<T, SD, OD, ROWS>, grid, TILE_THREADS, smem, a.together ? blocks : 1u, st, a);
+}
+
+// 32 rows to a CTA, or 16 while that leaves SMs idle: half the work on the path of a launch that is one round of CTAs.
+template <typename T, int SD, int OD>
+static cudaError_t launch_tile_rows(const SmatTileArgs& a, int bh, cudaStream_t st) {
+  const int64_t ctas = (int64_t)a.jobs * a.NC * ((a.c + 15) / 16) * bh;
+  return ctas <= 148 ? launch_tile_rows_of<T, SD, OD, 16>(a, bh, st) : launch_tile_rows_of<T, SD, OD, 32>(a, bh, st);
 }
 
 cudaError_t smat_launch_tile_rows(const SmatTileArgs& a, int bf16, int score_dim, int out_dim, int bh, cudaStream_t st) {

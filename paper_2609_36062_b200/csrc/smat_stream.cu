@@ -95,9 +95,9 @@ struct PoolCursor {
 // Two token buffers alternate over the passes, also inside a group of many tokens: the next pass's rows (of the same
 // group or of the next item) travel while this pass is summed.
 // clear (or null): the status word of a pass that begins with this launch, which waits for nothing that could fail.
-template <int R, int PD, typename T>
+// TK: tokens staged per pass.
+template <int R, int PD, typename T, int TK>
 __global__ void __launch_bounds__(256) pool_stream_kernel(const __grid_constant__ PoolList list, int64_t Tlen, int* clear) {
-  constexpr int TK = sizeof(T) == 2 ? 32 : 16;  // tokens staged per pass
   constexpr int NJ4 = PD / 4;
   constexpr int NG = 256 / NJ4;
   constexpr int NS = R / NG;
@@ -409,16 +409,30 @@ int sm_count() {
   return sms;
 }
 
-template <int R, int PD, typename T>
-cudaError_t launch_pool(const PoolList& list, int64_t Tlen, int* clear, cudaStream_t st) {
-  constexpr int TK = sizeof(T) == 2 ? 32 : 16;
+}  // namespace
+
+bool smat_pool_one_round(int64_t states) { return states <= sm_count(); }
+
+namespace {
+
+template <int R, int PD, typename T, int TK>
+cudaError_t launch_pool_tk(const PoolList& list, int64_t Tlen, int* clear, cudaStream_t st) {
   const size_t smem = R * PD * 4 + 2 * TK * (R + PD) * sizeof(T);
-  cudaError_t err = set_smem(pool_stream_kernel<R, PD, T>, smem);
+  cudaError_t err = set_smem(pool_stream_kernel<R, PD, T, TK>, smem);
   if (err != cudaSuccess) return err;
   const int64_t items = list.first[list.a.jobs];
   const int per_sm = smem <= 110 * 1024 ? 2 : 1;
   const int64_t grid = items < (int64_t)sm_count() * per_sm ? items : (int64_t)sm_count() * per_sm;
-  return smat_launch_pdl(pool_stream_kernel<R, PD, T>, dim3((unsigned)grid), 256, smem, st, list, Tlen, clear);
+  return smat_launch_pdl(pool_stream_kernel<R, PD, T, TK>, dim3((unsigned)grid), 256, smem, st, list, Tlen, clear);
+}
+
+// As long as every item has an SM of its own the time is one item's way through the passes: 64 tokens to a pass there (a
+// chunk of 64 is one round of loads instead of four: forward and backward of one 512-token head, d = 2, fp32, 45.9 -> 37.2 us
+// together with the 16-row tiles); else few, so that two CTAs share an SM.
+template <int R, int PD, typename T>
+cudaError_t launch_pool(const PoolList& list, int64_t Tlen, int* clear, cudaStream_t st) {
+  if (smat_pool_one_round(list.first[list.a.jobs])) return launch_pool_tk<R, PD, T, 64>(list, Tlen, clear, st);
+  return launch_pool_tk<R, PD, T, sizeof(T) == 2 ? 32 : 16>(list, Tlen, clear, st);
 }
 
 template <int R, int PD, typename T>

@@ -1,0 +1,29 @@
+"""The fp32 path where its launches have an SM for every piece of work (16-row tiles, 64 tokens to a pooling pass, the status
+word cleared by the pooling launch) against the same head among enough copies of itself that none of that applies: every sum
+has the same terms in the same order, so the results are equal bit for bit."""
+import pytest
+import torch
+
+from paper_2609_36062_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d,T,chunk,dk,dv,many", [(1, 256, 32, 64, 64, 48), (2, 512, 64, 64, 128, 32), (3, 288, 16, 128, 64, 24),
+                                                  (2, 640, 128, 128, 128, 40)])
+def test_one_head_equals_one_of_many(d, T, chunk, dk, dv, many):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(T)
+    q, k, v, do = (torch.randn(1, 1, T, n, generator=g, device="cuda") / n ** 0.5 for n in (dk, dk, dv, dv))
+    results = []
+    for heads in (1, many):
+        x = [t.expand(1, heads, T, t.shape[-1]).contiguous() for t in (q, k, v, do)]
+        plan = binding.SmatPlan(1, heads, T, dk, dv, d, chunk, "f32")
+        ws = plan.workspace(for_backward=True)
+        ws.fill_(0x55)                                            # the status word starts as anything
+        out = [plan.forward(*x[:3], workspace=ws)]
+        plan.check_status(ws)
+        out += plan.backward(*x, workspace=ws)
+        results.append([o[:, -1].clone() for o in out])
+    for a, b in zip(*results):
+        assert torch.equal(a, b)
