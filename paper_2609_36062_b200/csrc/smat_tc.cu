@@ -1304,9 +1304,21 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
 //                   Y = Q_h U_h   (M = up to 128 queries of the type, N = 128, K = 128)
 //   warps 0-3     : gather the queries of the type (token stride B) into the swizzled K-major A tile with
 //                   cp.async, later read the rows of Y from TMEM and scatter them to their tokens
-// Types with more than 128 queries take several passes over the same state.
+// Types with more than TOK queries take several passes over the same state.
+// TOK = 32, where the groups are that small (d >= 3: 6 to 24 tokens): the query tile has 32 rows of its own and the MMA's other
+// rows read whatever follows (their sums are never read), which leaves room for two states per CTA: the next one travels
+// while this one is multiplied and its rows are written, and six are on their way to an SM (dual: four).
+// TOK = 128 (d = 2): one state per CTA.
 // ---------------------------------------------------------------------------------------------------------------
-constexpr int READ_SMEM = 4 * BOX_BYTES + 1024 + 256;
+template <int DUAL, int TOK>
+struct ReadTcLayout {
+  static constexpr int NB = TOK == 32 ? 2 : 1;              // states in shared memory
+  static constexpr int A_BYTES = 2 * TOK * 128;             // a query tile: two 64-column blocks of TOK rows
+  static constexpr int B = (DUAL ? 2 : 1) * A_BYTES;        // first state
+  static constexpr int BARS = B + NB * 2 * BOX_BYTES;
+  static constexpr int SMEM = BARS + 1024 + 128;
+  static_assert(A_BYTES % 1024 == 0 && B - A_BYTES / 2 + BOX_BYTES <= BARS, "an MMA reads 128 rows from either block of a tile");
+};
 
 struct ReadParams {
   int64_t T;             // tokens per head
@@ -1323,8 +1335,9 @@ struct ReadParams {
 
 // TRANS = 0: out[t][j] = Σ_i x_t[i] St[i][j]  (state as MN-major B);  TRANS = 1: out[t][i] = Σ_j x_t[j] St[i][j]
 // (the same two boxes read as a K-major B).
-// One pass of state_read_tc_kernel: up to 128 tokens of one (state, head) item; states without tokens are skipped.
+// One pass of state_read_tc_kernel: up to TOK tokens of one (state, head) item; states without tokens are skipped.
 // Every role walks the same sequence.
+template <int TOK>
 struct ReadPass {
   const ReadParams* pp;
   int64_t item, stride;
@@ -1343,37 +1356,41 @@ struct ReadPass {
   __device__ int64_t token(int m) const { return tk.at(k0 + m); }   // position of row m of this pass
   __device__ bool valid() const { return item < pp->items; }
   __device__ bool first() const { return k0 == 0; }
-  __device__ bool last() const { return k0 + TILE >= cnt; }
-  __device__ int tokens() const { const int64_t left = cnt - k0; return (int)(left < TILE ? left : TILE); }
+  __device__ bool last() const { return k0 + TOK >= cnt; }
+  __device__ int tokens() const { const int64_t left = cnt - k0; return (int)(left < TOK ? left : TOK); }
+  __device__ void next_item() { item += stride; load(); }
   __device__ void next() {
-    if (last()) { item += stride; load(); } else k0 += TILE;
+    if (last()) next_item(); else k0 += TOK;
   }
 };
 
 // DUAL (with TRANS = 1): both adjoint reads of a profile's tokens from one load of the state F̄_x —
 // out[t] = F̄_x x_t (rows X, e.g. dK from v) and out2[t] = F̄_xᵀ x2_t (rows X2, e.g. dV from k) — two operand tiles, two
 // accumulators, bf16 results.
-template <int TRANS, int DUAL = 0>
+template <int TRANS, int DUAL, int TOK>
 __global__ void __launch_bounds__(160) state_read_tc_kernel(const __grid_constant__ CUtensorMap tmU,
                                                             const ReadParams prm) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  using L = ReadTcLayout<DUAL, TOK>;
+  constexpr int NB = L::NB;
   uint8_t* sA = smem;                    // queries, K-major, two 64-column blocks
-  uint8_t* sB = smem + 2 * BOX_BYTES;    // state, MN-major, two 64-column blocks
-  uint8_t* sA2 = smem + 4 * BOX_BYTES;   // DUAL: the second rows
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (DUAL ? 6 : 4) * BOX_BYTES);
-  uint64_t* bar_u = bars + 0;   // state landed (TMA)
-  uint64_t* bar_a = bars + 1;   // queries landed (one arrival per warp)
-  uint64_t* bar_d = bars + 2;   // product in TMEM
-  uint64_t* bar_e = bars + 3;   // TMEM read out (4 arrivals)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 4);
+  uint8_t* sA2 = smem + L::A_BYTES;      // DUAL: the second rows
+  uint8_t* sB = smem + L::B;             // [NB] states, MN-major, two 64-column blocks each
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::BARS);
+  uint64_t* bar_u = bars + 0;   // [NB] state landed (TMA)
+  uint64_t* bar_a = bars + 2;   // queries landed (one arrival per warp)
+  uint64_t* bar_d = bars + 3;   // product in TMEM
+  uint64_t* bar_e = bars + 4;   // TMEM read out (4 arrivals)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 5);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WaitCtx wc{cta_abort, prm.status};
 
   if (threadIdx.x == 0) {
     *cta_abort = 0;
-    mbar_init(bar_u, 1); mbar_init(bar_a, 4); mbar_init(bar_d, 1); mbar_init(bar_e, 4);
+    for (int b = 0; b < NB; ++b) mbar_init(bar_u + b, 1);
+    mbar_init(bar_a, 4); mbar_init(bar_d, 1); mbar_init(bar_e, 4);
     fence_barrier_init();
   }
   if (warp == 4) tmem_alloc(tmem_slot, DUAL ? 2 * TILE : TILE);
@@ -1385,17 +1402,17 @@ __global__ void __launch_bounds__(160) state_read_tc_kernel(const __grid_constan
   const uint32_t tmem_d = *tmem_slot;
   constexpr uint32_t idesc = make_idesc(TILE, TILE, 0, TRANS ? 0 : 1);
   constexpr uint32_t idesc2 = make_idesc(TILE, TILE, 0, 1);
-  ReadPass cur(prm, blockIdx.x, gridDim.x);
+  ReadPass<TOK> cur(prm, blockIdx.x, gridDim.x);
 
   if (warp < 4) {
     const int tid = threadIdx.x;
     const uint32_t a_base = smem_u32(sA), a2_base = smem_u32(sA2);
-    auto gather = [&](const ReadPass& ps) {
+    auto gather = [&](const ReadPass<TOK>& ps) {
       const int kn = ps.tokens();
       for (int idx = tid; idx < kn * 16; idx += 128) {
         const int m = idx >> 4, gc = idx & 15;
         const int64_t row = (ps.bh * prm.T + ps.token(m)) * TILE + gc * 8;
-        const uint32_t off = (gc >> 3) * BOX_BYTES + m * 128 + (((gc & 7) ^ (m & 7)) << 4);
+        const uint32_t off = (gc >> 3) * (TOK * 128) + m * 128 + (((gc & 7) ^ (m & 7)) << 4);
         cp_async16(a_base + off, prm.X + row);
         if (DUAL) cp_async16(a2_base + off, prm.X2 + row);
       }
@@ -1408,7 +1425,7 @@ __global__ void __launch_bounds__(160) state_read_tc_kernel(const __grid_constan
       fence_proxy_async();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_a);   // one arrival per warp
-      ReadPass nxt = cur;
+      ReadPass<TOK> nxt = cur;
       nxt.next();
       bool ok = mbar_wait(bar_d, n_pass & 1, wc);            // the MMAs have read the query tile; the product is in TMEM
       ok = __all_sync(0xffffffffu, ok);
@@ -1420,6 +1437,7 @@ __global__ void __launch_bounds__(160) state_read_tc_kernel(const __grid_constan
       float4* dst = reinterpret_cast<float4*>(prm.out + row);
 #pragma unroll
       for (int cbo = 0; cbo < (DUAL ? 8 : 4); ++cbo) {
+        if (warp * 32 >= kn) break;                          // (warp-uniform) no tokens in these lanes
         const int cb = cbo & 3;
         __nv_bfloat16* dst16 = (cbo < 4 ? prm.out_bf16 : prm.out2_bf16) + row;
         uint32_t v[32];
@@ -1452,49 +1470,57 @@ __global__ void __launch_bounds__(160) state_read_tc_kernel(const __grid_constan
     asm volatile("cp.async.wait_group 0;" ::: "memory");
   } else if (lane == 0) {
     (void)idesc2;
-    auto load_state = [&](int64_t item) {
-      mbar_expect_tx(bar_u, 2 * BOX_BYTES);
-      const int row = (int)(item * TILE);
-      tma_load_2d(sB, &tmU, 0, row, bar_u);
-      tma_load_2d(sB + BOX_BYTES, &tmU, HALF, row, bar_u);
-    };
-    uint32_t n_item = 0, n_pass = 0;  // completed uses of bar_u and of bar_a / bar_d / bar_e
+    uint32_t n_item = 0, n_pass = 0;  // completed items, and uses of bar_a / bar_d / bar_e
     uint32_t loads = 0;               // started states
+    ReadPass<TOK> ahead = cur;        // the item whose state is loaded next
+    auto load_state = [&] {
+      if (!ahead.valid()) return;
+      const uint32_t b = loads % NB;
+      uint8_t* dst = sB + b * 2 * BOX_BYTES;
+      const int row = (int)(ahead.item * TILE);
+      mbar_expect_tx(bar_u + b, 2 * BOX_BYTES);
+      tma_load_2d(dst, &tmU, 0, row, bar_u + b);
+      tma_load_2d(dst + BOX_BYTES, &tmU, HALF, row, bar_u + b);
+      ++loads;
+      ahead.next_item();
+    };
     bool ok = true;
-    if (cur.valid()) { load_state(cur.item); ++loads; }
+    for (int b = 0; b < NB; ++b) load_state();
     while (cur.valid() && ok) {
-      if (cur.first()) ok = mbar_wait(bar_u, n_item & 1, wc);
+      const uint32_t b = n_item % NB;
+      if (cur.first()) ok = mbar_wait(bar_u + b, (n_item / NB) & 1, wc);
       if (ok) ok = mbar_wait(bar_a, n_pass & 1, wc);
       if (ok && n_pass > 0) ok = mbar_wait(bar_e, (n_pass - 1) & 1, wc);  // previous product has been read out
       if (!ok) break;
       fence_after_sync();
+      const uint32_t a0 = smem_u32(sA), a2 = smem_u32(sA2), b0 = smem_u32(sB) + b * 2 * BOX_BYTES;
 #pragma unroll
       for (int kk = 0; kk < TILE / 16; ++kk) {
-        const uint64_t dA = make_desc(smem_u32(sA) + (kk >> 2) * BOX_BYTES + (kk & 3) * 32, 16, 1024);
-        const uint64_t dB = TRANS ? make_desc(smem_u32(sB) + (kk >> 2) * BOX_BYTES + (kk & 3) * 32, 16, 1024)
-                                  : make_desc(smem_u32(sB) + kk * 2048, BOX_BYTES, 1024);
+        const uint64_t dA = make_desc(a0 + (kk >> 2) * (TOK * 128) + (kk & 3) * 32, 16, 1024);
+        const uint64_t dB = TRANS ? make_desc(b0 + (kk >> 2) * BOX_BYTES + (kk & 3) * 32, 16, 1024)
+                                  : make_desc(b0 + kk * 2048, BOX_BYTES, 1024);
         mma_bf16(tmem_d, dA, dB, idesc, kk != 0);
       }
       if (DUAL) {
 #pragma unroll
         for (int kk = 0; kk < TILE / 16; ++kk) {   // the second rows against the state as it lies (MN-major B)
-          const uint64_t dA = make_desc(smem_u32(sA2) + (kk >> 2) * BOX_BYTES + (kk & 3) * 32, 16, 1024);
-          const uint64_t dB = make_desc(smem_u32(sB) + kk * 2048, BOX_BYTES, 1024);
+          const uint64_t dA = make_desc(a2 + (kk >> 2) * (TOK * 128) + (kk & 3) * 32, 16, 1024);
+          const uint64_t dB = make_desc(b0 + kk * 2048, BOX_BYTES, 1024);
           mma_bf16(tmem_d + TILE, dA, dB, idesc2, kk != 0);
         }
       }
       mma_commit(bar_d);
-      // the state tile may be overwritten (next item) only after the MMAs have read it
+      // the state tile may be overwritten (a later item) only after the MMAs have read it
       ok = mbar_wait(bar_d, n_pass & 1, wc);
-      const bool was_last = cur.last();
+      if (cur.last()) {
+        ++n_item;
+        if (ok) load_state();   // travels while the product is written out
+      }
       cur.next();
       ++n_pass;
-      if (was_last) {
-        ++n_item;
-        if (ok && cur.valid()) { load_state(cur.item); ++loads; }   // travels while the product is written out
-      }
     }
-    landed(bar_u, (loads + 1) & 1, wc);
+    for (uint32_t b = 0; b < (uint32_t)NB; ++b)   // (a barrier that never saw a load lets parity 1 pass)
+      landed(bar_u + b, ((loads > b ? (loads - 1 - b) / NB + 1 : 0) + 1) & 1, wc);
   }
   fence_before_sync();
   __syncthreads();
@@ -1865,6 +1891,10 @@ cudaError_t smat_launch_bwd_tiles_fused_tc(const void* Q, const void* K, const v
 
 // Both adjoint reads of the profile states in one launch: out_t[t] = St x_t (rows Xt, the second state index
 // contracted) and out_n[t] = Stᵀ x_t (rows Xn, the first one), bf16 rows; every state is loaded once.
+// Whether a group's tokens fit the 32-row query tile: always for positional groups, on average (and half of it) for listed
+// ones, whose heavy groups take more passes.
+static bool read_groups_small(const SmatGroupSpec& grp) { return grp.list ? grp.base < 16 : grp.base < 32; }
+
 cudaError_t smat_launch_state_read_dual_tc(const void* Xt, const void* Xn, const void* state_bf16, void* out_t_bf16,
                                            void* out_n_bf16, const SmatGroupSpec& grp, int64_t groups, int64_t T, int bh,
                                            int* status, cudaStream_t st) {
@@ -1881,11 +1911,13 @@ cudaError_t smat_launch_state_read_dual_tc(const void* Xt, const void* Xn, const
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int smem = READ_SMEM + 2 * BOX_BYTES;
-  const int64_t grid = prm.items < 2LL * sms ? prm.items : 2LL * sms;   // 256 columns of tensor memory and 97 KB each
-  cudaError_t err = cudaFuncSetAttribute(state_read_tc_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const bool small = read_groups_small(grp);
+  const int smem = small ? ReadTcLayout<1, 32>::SMEM : ReadTcLayout<1, 128>::SMEM;
+  const int64_t grid = prm.items < 2LL * sms ? prm.items : 2LL * sms;   // 256 columns of tensor memory and up to 97 KB each
+  auto kernel = small ? state_read_tc_kernel<1, 1, 32> : state_read_tc_kernel<1, 1, 128>;
+  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
-  return smat_launch_pdl(state_read_tc_kernel<1, 1>, dim3((unsigned)grid), 160, smem, st, tmU, prm);
+  return smat_launch_pdl(kernel, dim3((unsigned)grid), 160, smem, st, tmU, prm);
 }
 
 cudaError_t smat_launch_state_read_tc(const void* X, const void* state_bf16, float* out, void* out_bf16, int transposed,
@@ -1904,10 +1936,13 @@ cudaError_t smat_launch_state_read_tc(const void* X, const void* state_bf16, flo
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t grid = prm.items < 3LL * sms ? prm.items : 3LL * sms;
-  auto kernel = transposed ? state_read_tc_kernel<1> : state_read_tc_kernel<0>;
-  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, READ_SMEM);
+  const bool small = read_groups_small(grp);
+  const int smem = small ? ReadTcLayout<0, 32>::SMEM : ReadTcLayout<0, 128>::SMEM;
+  auto kernel = small ? (transposed ? state_read_tc_kernel<1, 0, 32> : state_read_tc_kernel<0, 0, 32>)
+                      : (transposed ? state_read_tc_kernel<1, 0, 128> : state_read_tc_kernel<0, 0, 128>);
+  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
-  return smat_launch_pdl(kernel, dim3((unsigned)grid), 160, READ_SMEM, st, tmU, prm);
+  return smat_launch_pdl(kernel, dim3((unsigned)grid), 160, smem, st, tmU, prm);
 }
 
 template <int TOK, int OUT_BF16>
