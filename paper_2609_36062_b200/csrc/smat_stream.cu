@@ -3,7 +3,7 @@
 //   pool_stream_kernel       : state[g] = Σ_{tokens of g} a_tᵀ b_t ; each finished 64 KB state leaves through a
 //                              bulk store while the next group's tokens are already in flight        (Algorithm 1, step 2)
 //   state_read_stream_kernel : out[t] = x_t · state[g(t)] for the few tokens of every group; states arrive through
-//                              bulk loads, half a state at a time                                          (Algorithm 1, step 4)
+//                              bulk loads                                                             (Algorithm 1, step 4)
 // Both are bound by the one pass over the table they write or read.
 #include <cuda_bf16.h>
 
@@ -26,17 +26,6 @@ __device__ __forceinline__ float4 fma4(float s, const float4 b, float4 a) {
   return a;
 }
 __device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-template <int N>
-__device__ __forceinline__ void load_row(const float* p, float (&x)[N]) {
-  static_assert(N == 2 || N == 4, "one load");
-  if (N == 4) {
-    const float4 v = *reinterpret_cast<const float4*>(p);
-    x[0] = v.x; x[1] = v.y; x[N - 2] = v.z; x[N - 1] = v.w;
-  } else {
-    const float2 v = *reinterpret_cast<const float2*>(p);
-    x[0] = v.x; x[1] = v.y;
-  }
-}
 __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
   const uint2 raw = *reinterpret_cast<const uint2*>(p);
   const __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162*>(&raw.x);
@@ -189,10 +178,10 @@ struct ReadList {
   int32_t scan_x, scan_y, scan_ctas;   // CTAs per head and (job, range); heads; all of them
 };
 
-// Two CTAs share an SM; each owns one 64 KB state buffer in two halves of rows: the next item's first half is under way
-// while the second half is contracted, and its second half while the rows are reduced and stored.  32 heads of 5056 tokens,
-// d = 3 (306 states a head, 642 MB, 0.098 ms at the HBM rate): 0.160 ms, 0.178 with one load per state and eight tokens to
-// every pass; one CTA of sixteen warps with a ring of five halves 0.203 (its barriers are on the path of every pass).
+// Two CTAs share an SM; each owns one 64 KB state buffer, so one CTA's contraction overlaps the other's bulk load.  (A state
+// in two halves, the first one fetched again while the second is contracted: nothing gained where a group is one pass, and a
+// barrier more to each where it is many.  8 heads of 2048 tokens, d = 2, fp32, half of them in one group, forward and
+// backward: 1980 us so, 2100 in halves.)
 template <int R, int PD, typename T>
 struct ReadLayout {
   static constexpr int KT = 8;                              // tokens per pass over a state
@@ -207,14 +196,14 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
                                                                    int* status) {
   using L = ReadLayout<R, PD, T>;
   constexpr int KT = L::KT, NJ4 = L::NJ4, NG = L::NG;
-  constexpr int RPH = R / NG / 2, VR = RPH < 4 ? RPH : 4;   // a thread's rows of a half
+  constexpr int RPG = R / NG;
   extern __shared__ __align__(128) uint8_t smem_raw[];
   float* Sb = reinterpret_cast<float*>(smem_raw);        // [R*PD]
   float* red = Sb + R * PD;                              // [RED]
   T* Xraw = reinterpret_cast<T*>(red + L::RED);          // [2][KT][XM] raw rows of the first KT tokens of an item
   float* Xs = reinterpret_cast<float*>(Xraw + 2 * KT * L::XM);  // [KT][XM]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(Xs + KT * L::XM);   // [2] a half of the state has landed
-  volatile int* cta_abort = reinterpret_cast<volatile int*>(bar + 2);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(Xs + KT * L::XM);
+  volatile int* cta_abort = reinterpret_cast<volatile int*>(bar + 1);
   pdl_trigger();
   const tc::WaitCtx wc{cta_abort, status};
   const int tid = threadIdx.x;
@@ -225,7 +214,7 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
     return;
   }
   const int j4 = tid % NJ4, ig = tid / NJ4;
-  constexpr uint32_t HBYTES = R * PD * 2;   // half a state
+  constexpr uint32_t SBYTES = R * PD * 4;
   const int64_t items = list.first[list.a.jobs], cta = blockIdx.x - list.scan_ctas, ctas = gridDim.x - list.scan_ctas;
   auto job_of = [&](int64_t item) {
     int j = 0;
@@ -261,22 +250,20 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
   if (tid == 0) {
     *cta_abort = 0;
     tc::mbar_init(bar, 1);
-    tc::mbar_init(bar + 1, 1);
     tc::fence_barrier_init();
   }
-  uint32_t loads[2] = {0, 0};   // started halves (thread 0)
-  auto load_half = [&](int64_t item, int h) {
-    tc::mbar_expect_tx(bar + h, HBYTES);
-    bulk_load(Sb + h * (R * PD / 2), state_of(item) + h * (R * PD / 2), HBYTES, bar + h);
-    ++loads[h];
+  uint32_t loads = 0;   // started states (thread 0)
+  auto load_state = [&](int64_t item) {
+    tc::mbar_expect_tx(bar, SBYTES);
+    bulk_load(Sb, state_of(item), SBYTES, bar);
+    ++loads;
   };
   pdl_wait();
-  if (tid == 0 && cta < items) { load_half(cta, 0); load_half(cta, 1); }
+  if (tid == 0 && cta < items) load_state(cta);
   prefetch_x(cta, 0);
   __syncthreads();
   int n = 0;
-  bool ok = true;
-  for (int64_t item = cta; item < items && ok; item += ctas, ++n) {
+  for (int64_t item = cta; item < items; item += ctas, ++n) {
     const int buf = n & 1;
     const int j = job_of(item);
     int64_t bh;
@@ -289,50 +276,34 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
     prefetch_x(nxt, buf ^ 1);
     cp_async_wait<1>();
     __syncthreads();
-    int64_t k0 = 0;
-    do {   // (a state without tokens is waited for and passed over)
+    for (int64_t k0 = 0; k0 == 0 || k0 < cnt; k0 += KT) {   // (a state without tokens is waited for and passed over)
       const int kn = (int)((cnt - k0) < KT ? (cnt - k0) : KT);
-      const bool last = k0 + KT >= cnt;
       for (int idx = tid; idx < KT * xd; idx += 256) {
         const int k = idx / xd, i = idx - k * xd;
         float v = 0.f;
         if (k < kn) v = k0 == 0 ? to_float(Xraw[(buf * KT + k) * L::XM + i]) : to_float(Xb[tk.at(k0 + k) * xd + i]);
         Xs[k * L::XM + i] = v;
       }
-      // Block-wide barriers follow: all go on, or none.  After the second one every thread is past its reads of the first
-      // half, after the one behind the contraction past those of the second.
-      auto half_landed = [&](int h) {
-        ok = __syncthreads_and(tc::mbar_wait(bar + h, n & 1, wc)) != 0;
-        if (ok && h == 1 && last && tid == 0 && nxt < items) load_half(nxt, 0);
-        return ok;
-      };
-      auto both_read = [&] {
-        __syncthreads();
-        if (last && tid == 0 && nxt < items) load_half(nxt, 1);
-      };
+      const bool ok = __syncthreads_and(k0 > 0 || tc::mbar_wait(bar, n & 1, wc)) != 0;   // (block-wide barriers follow: all go on, or none)
+      if (!ok || cnt == 0) break;
       if (!trans) {
-        // KK: tokens of the pass, rounded up: nine tokens are a pass of eight and one of two
+        // KK: tokens of the pass, rounded up: nine tokens are a pass of eight and one of two (32 heads of 5056 tokens, d = 3,
+        // normalised: the pass 651 us with eight to every one, 615 so)
         auto contract = [&](auto tokens) {
           constexpr int KK = decltype(tokens)::value;
           float4 acc[KK];
 #pragma unroll
           for (int k = 0; k < KK; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-          for (int h = 0; h < 2; ++h) {
-            if (!half_landed(h)) return;
-            // VR rows at a time, so that a token's factors are one load
+          // four rows at a time, so that a token's factors are one load (32 heads, 307 states, bf16: 0.185 -> 0.177 ms)
 #pragma unroll 2
-            for (int s = 0; s < RPH; s += VR) {
-              const int i = h * (R / 2) + ig * RPH + s;
-              float4 u[VR];
+          for (int s = 0; s < RPG; s += 4) {
+            const int i = ig * RPG + s;
+            const float4 u0 = S4[i * NJ4 + j4], u1 = S4[(i + 1) * NJ4 + j4], u2 = S4[(i + 2) * NJ4 + j4], u3 = S4[(i + 3) * NJ4 + j4];
 #pragma unroll
-              for (int e = 0; e < VR; ++e) u[e] = S4[(i + e) * NJ4 + j4];
-#pragma unroll
-              for (int k = 0; k < KK; ++k) {
-                float x[VR];
-                load_row<VR>(Xs + k * L::XM + i, x);
-#pragma unroll
-                for (int e = 0; e < VR; ++e) acc[k] = fma4(x[e], u[e], acc[k]);
-              }
+            for (int k = 0; k < KK; ++k) {
+              const float4 x = *reinterpret_cast<const float4*>(Xs + k * L::XM + i);
+              acc[k] = fma4(x.x, u0, acc[k]); acc[k] = fma4(x.y, u1, acc[k]);
+              acc[k] = fma4(x.z, u2, acc[k]); acc[k] = fma4(x.w, u3, acc[k]);
             }
           }
 #pragma unroll
@@ -341,8 +312,7 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
         if (kn > 4) contract(std::integral_constant<int, 8>{});
         else if (kn > 2) contract(std::integral_constant<int, 4>{});
         else contract(std::integral_constant<int, 2>{});
-        if (!ok) break;
-        both_read();
+        __syncthreads();
         for (int idx = tid; idx < kn * NJ4; idx += 256) {   // the row groups' partial rows meet in shared memory
           const int k = idx / NJ4, c = idx - k * NJ4;
           float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -354,42 +324,36 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
           *reinterpret_cast<float4*>(out + tk.at(k0 + k) * PD + c * 4) = v;
         }
       } else {
-        for (int h = 0; h < 2; ++h) {
-          if (!half_landed(h)) break;
 #pragma unroll 2
-          for (int s = 0; s < RPH; ++s) {
-            const int i = h * (R / 2) + ig * RPH + s;
-            const float4 u = S4[i * NJ4 + j4];
-            float part[KT];
+        for (int s = 0; s < RPG; ++s) {
+          const int i = ig * RPG + s;
+          const float4 u = S4[i * NJ4 + j4];
+          float part[KT];
 #pragma unroll
-            for (int k = 0; k < KT; ++k) {
-              const float4 x4 = *reinterpret_cast<const float4*>(Xs + k * L::XM + j4 * 4);
-              part[k] = u.x * x4.x + u.y * x4.y + u.z * x4.z + u.w * x4.w;
-            }
-#pragma unroll
-            for (int off = NJ4 / 2; off > 0; off >>= 1)
-#pragma unroll
-              for (int k = 0; k < KT; ++k) part[k] += __shfl_xor_sync(0xffffffffu, part[k], off);
-            if (j4 == 0)
-#pragma unroll
-              for (int k = 0; k < KT; ++k) red[k * R + i] = part[k];
+          for (int k = 0; k < KT; ++k) {
+            const float4 x4 = *reinterpret_cast<const float4*>(Xs + k * L::XM + j4 * 4);
+            part[k] = u.x * x4.x + u.y * x4.y + u.z * x4.z + u.w * x4.w;
           }
+#pragma unroll
+          for (int off = NJ4 / 2; off > 0; off >>= 1)
+#pragma unroll
+            for (int k = 0; k < KT; ++k) part[k] += __shfl_xor_sync(0xffffffffu, part[k], off);
+          if (j4 == 0)
+#pragma unroll
+            for (int k = 0; k < KT; ++k) red[k * R + i] = part[k];
         }
-        if (!ok) break;
-        both_read();
+        __syncthreads();
         for (int idx = tid; idx < kn * R; idx += 256) {
           const int k = idx / R, i = idx % R;
           out[tk.at(k0 + k) * R + i] = red[k * R + i];
         }
       }
       __syncthreads();
-      k0 += KT;
-    } while (k0 < cnt);
+    }
+    // every thread is past its reads of the state buffer: fetch the next item's state
+    if (tid == 0 && nxt < items && !*cta_abort) load_state(nxt);
   }
-  if (tid == 0) {
-    tc::landed(bar, (loads[0] + 1) & 1, wc);
-    tc::landed(bar + 1, (loads[1] + 1) & 1, wc);
-  }
+  if (tid == 0) tc::landed(bar, (loads + 1) & 1, wc);
   cp_async_wait<0>();
 }
 

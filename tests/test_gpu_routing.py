@@ -121,3 +121,39 @@ def test_one_type_takes_every_query_of_a_short_batch():
     for h in (0, 77, w.bh - 1):
         Q64, K64, V64 = (synth.as_float64(w, host[x][h]) for x in ("q", "k", "v"))
         assert rel_err(to_numpy64(O.reshape(w.bh, w.T, -1)[h]), so.forward_dense(Q64, K64, V64, M)) <= TOL["bf16"]
+
+
+def _sizes_to_keys(sizes, count, groups, rng):
+    """`count` keys in random order: group g gets sizes[g] of them, the groups behind those what is left, one each in turn."""
+    keys = [g for g, s in enumerate(sizes) for _ in range(s)]
+    rest = np.arange(count - len(keys)) % (groups - len(sizes)) + len(sizes)
+    return rng.permutation(np.concatenate([np.array(keys, dtype=np.int64), rest])).astype(np.int32)
+
+
+# Group sizes at the edges of the passes and of the parts that a heavy group is handed out in: fp32 passes of 8 with
+# remainders of 2, 4 and 8; bf16 query tiles of 32 rows, parts of 128
+@pytest.mark.parametrize("dtype,d,T,c,sizes", [
+    ("f32", 2, 512, 32, (0, 1, 2, 3, 4, 5, 7, 8, 9, 10, 12, 15, 16, 17, 33)),
+    ("bf16", 3, 2048, 128, (0, 1, 31, 32, 33, 127, 128, 129, 160, 257)),
+    ("bf16", 3, 2048, 64, (0, 640, 5, 256)),
+    ("bf16", 3, 1088, 64, (0, 1, 7, 8, 9, 140)),                 # blocks that are not whole tiles: fp32 tables and reads
+])
+def test_group_sizes_at_the_edges_of_passes_and_parts(dtype, d, T, c, sizes):
+    dk = 128 if dtype == "bf16" else 64
+    w = synth.Workload("edges", d, 1, 2, T, dk, dk, c, dtype, "normalised", 91)
+    host, dev = device_inputs(w, ("q", "k", "v", "do"))
+    geo = so.geometry(T, c, d)
+    rng = np.random.default_rng(T)
+    cells = np.stack([_sizes_to_keys(sizes[::s], geo.n, geo.P, rng) for s in (1, -1)])   # (the heads differ)
+    types = np.stack([_sizes_to_keys(sizes[::s], geo.m, geo.B, rng) for s in (-1, 1)])
+    prof, typ = torch.from_numpy(cells).cuda(), torch.from_numpy(types).cuda()
+    plan = binding.SmatPlan(w.batch, w.heads, w.T, w.d_k, w.d_v, w.d, w.chunk, w.dtype)
+    for _ in range(2):                                           # the second pass starts from what the first one left
+        O = plan.forward(dev["q"], dev["k"], dev["v"], prof=prof, type=typ)
+        grads = plan.backward(dev["q"], dev["k"], dev["v"], dev["do"], prof=prof, type=typ)
+    plan.check_status()
+    for h in range(w.bh):
+        Q64, K64, V64, G64 = (synth.as_float64(w, host[x][h]) for x in ("q", "k", "v", "do"))
+        M = so.routed_dense_mask(geo, cells[h], types[h])
+        for got, ref in zip((O, *grads), (so.forward_dense(Q64, K64, V64, M), *so.backward_dense(Q64, K64, V64, G64, M))):
+            assert rel_err(to_numpy64(got[0, h]), ref) <= TOL[dtype]
