@@ -174,7 +174,7 @@ cudaError_t clear_status(const Ctx& cx) {
 // that start while the pass before drains crowd the SMs that are free first.  d = 1, 8 heads of 2048 tokens, 64 wide, chunk
 // 32, forward and backward: 119 us with the memset, 133 without.)
 void begin_pass(Ctx& cx, bool pools_first, int64_t pooled) {
-  if (pools_first && !cx.pl->inner && smat_pool_one_round(pooled * cx.pl->bh)) {
+  if (pools_first && !cx.pl->inner && pooled * cx.pl->bh <= smat_sm_count()) {
     cx.pl->kept_gated_forward = false;
     cx.clear = reinterpret_cast<int*>(cx.ws + cx.pl->off_status);
   } else {
@@ -313,6 +313,19 @@ void scan_states(Ctx& cx, const char* name, std::initializer_list<SmatScanJob> j
   SmatScanArgs a{};
   for (const SmatScanJob& j : jobs) a.job[a.jobs++] = j;
   SMAT_TRY(cx, name, smat_launch_scan(a, pl->rp, pl->NC, pl->bh, cx.st));
+}
+// Whether the routed read's launch scans the chunk states, instead of a launch of its own behind the pooling.  That saves a
+// launch, but its CTAs share an SM with one other (they carry the read's shared memory) where eight of the scan kernel do,
+// they stand in front of the read's, and behind a tabulation they find less of the states in the L2 cache.  So only while a
+// direction's CTAs are one round of the launch, at d >= 3 while the states are small, and not where a heavy group of a routed
+// call is what the launch takes.  Forward and backward in us, scanned apart / beside the read: d = 3, one 512-token head, 64
+// wide, 57 / 53; d = 2, 128 wide, 8 heads of 2048 tokens 409 / 406, 32 of 512 415 / 423, 128 of 512 1506 / 1583; d = 3, 64
+// wide, 16 heads of 2048 (8 MB) 386 / 386, 8 of 8192 (17 MB, forward alone) 188 / 190; 128 wide, 8 of 5056 (41 MB, normalised)
+// 1214 / 1260; d = 2, routed, 8 heads of 2048, all tokens in one group, 3469 / 3555.
+bool scan_beside_read(const Ctx& cx) {
+  const smat_plan* pl = cx.pl;
+  const int64_t ctas = 2 * (int64_t)pl->bh * ((pl->rp / 4 + 255) / 256);
+  return !cx.routed && ctas <= 2 * smat_sm_count() && (pl->geo.D == 1 || pl->bh * pl->NC * pl->rp * 4 <= (12LL << 20));
 }
 // The two-level causal branch's cut into segments, and its first half: the totals of the segments (none where every block
 // is one segment), and their exclusive prefix sums where a block has more than two.
@@ -697,12 +710,14 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
   const SmatPoolJob chunks = pool_job(cx, SMAT_GM_CHUNK, K, V, sin);
   if (lr) pool(cx, "pool", {pool_job(cx, SMAT_GM_PROFILE, K, V, cx.f(pl->off_F)), chunks});           // steps 2, 5
   else pool(cx, "pool", {chunks});
+  const bool beside = lr && scan_beside_read(cx);
+  if (!beside) scan_states(cx, "scan", {scan_job(cx, sin, 0)});                                      // step 6
   if (lr) {
     tabulate(cx, "tabulate", cx.f(pl->off_F), cx.f(pl->off_U), 0);                                   // step 3
     zero_unrouted(cx, SMAT_GM_TYPE, acc, pl->p * 4);
-    state_read(cx, "read_type", {read_job(cx, SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, acc)}, {scan_job(cx, sin, 0)});   // steps 4, 6
-  } else {
-    scan_states(cx, "scan", {scan_job(cx, sin, 0)});                                                 // step 6
+    const SmatReadJob read = read_job(cx, SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, acc);                 // step 4
+    if (beside) state_read(cx, "read_type", {read}, {scan_job(cx, sin, 0)});
+    else state_read(cx, "read_type", {read});
   }
   tile_rows(cx, "tiles", pl->r, pl->p, {tile_job(Q, K, V, Q, sin, 0, 0, acc, lr ? pl->geo.n : pl->T, pl->T, O)}, nullptr);   // step 7
   pl->launches = cx.launches;
@@ -835,19 +850,21 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
   if (lr) pool(cx, "bwd_pool", {pool_job(cx, SMAT_GM_PROFILE, K, V, cx.f(pl->off_F)), cf, cb,
                                 pool_job(cx, SMAT_GM_TYPE, Q, dO, cx.f(pl->off_ubar))});
   else pool(cx, "bwd_pool", {cf, cb});
-  if (!lr) {
-    scan_states(cx, "bwd_scan", {scan_job(cx, sin, 0), scan_job(cx, dbar, 1)});
-  } else {
+  const SmatScanJob prefix = scan_job(cx, sin, 0), suffix = scan_job(cx, dbar, 1);
+  const bool beside = lr && scan_beside_read(cx);
+  if (!beside) scan_states(cx, "bwd_scan", {prefix, suffix});
+  if (lr) {
     tabulate(cx, "tabulate", cx.f(pl->off_F), cx.f(pl->off_U), 0);
     tabulate(cx, "bwd_tabulate_t", cx.f(pl->off_ubar), cx.f(pl->off_fbar), 1);
     // dQ's long-range rows are recent and dK's distant: they share a buffer
     zero_unrouted(cx, SMAT_GM_TYPE, acc, pl->r * 4);
     zero_unrouted(cx, SMAT_GM_PROFILE, acc, pl->r * 4);
     zero_unrouted(cx, SMAT_GM_PROFILE, acc_v, pl->p * 4);
-    state_read(cx, "bwd_reads", {read_job(cx, SMAT_GM_TYPE, dO, cx.f(pl->off_U), 1, acc),
-                                 read_job(cx, SMAT_GM_PROFILE, V, cx.f(pl->off_fbar), 1, acc),
-                                 read_job(cx, SMAT_GM_PROFILE, K, cx.f(pl->off_fbar), 0, acc_v)},
-               {scan_job(cx, sin, 0), scan_job(cx, dbar, 1)});
+    const SmatReadJob rq = read_job(cx, SMAT_GM_TYPE, dO, cx.f(pl->off_U), 1, acc);
+    const SmatReadJob rk = read_job(cx, SMAT_GM_PROFILE, V, cx.f(pl->off_fbar), 1, acc);
+    const SmatReadJob rv = read_job(cx, SMAT_GM_PROFILE, K, cx.f(pl->off_fbar), 0, acc_v);
+    if (beside) state_read(cx, "bwd_reads", {rq, rk, rv}, {prefix, suffix});
+    else state_read(cx, "bwd_reads", {rq, rk, rv});
   }
   const int64_t n = lr ? pl->geo.n : 0, from = lr ? n : pl->T;
   adjoint_tiles(cx, "bwd_tiles", tile_job(dO, V, K, dO, sin, 1, 0, acc, from, pl->T, dQ),

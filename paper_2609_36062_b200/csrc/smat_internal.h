@@ -129,8 +129,7 @@ struct SmatPoolArgs {
   SmatPoolJob job[4];
   int jobs;
 };
-// Whether a pooling launch of that many states has an SM for each.
-bool smat_pool_one_round(int64_t states);
+int smat_sm_count();   // SMs of the device
 // clear (or null): status word that the launch sets to zero.
 cudaError_t smat_launch_pool(const SmatPoolArgs& a, int bf16, int64_t Tlen, int bh, int r, int p, int* clear, cudaStream_t st);
 

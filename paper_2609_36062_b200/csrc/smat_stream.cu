@@ -171,8 +171,8 @@ __global__ void __launch_bounds__(256) pool_stream_kernel(const __grid_constant_
 struct ReadList {
   SmatReadArgs a;
   int64_t first[4];
-  // Chunk states that the tile kernel behind the read will want scanned: the first scan_ctas CTAs of the launch do that
-  // (a sequence of launches of a few CTAs each is bound by their number).
+  // Chunk states that the tile kernel behind the read will want scanned: the first scan_ctas CTAs of the launch do that, where
+  // the pass is a sequence of launches of a few CTAs each and bound by their number.
   SmatScanArgs scan;
   int64_t NC;
   int32_t scan_x, scan_y, scan_ctas;   // CTAs per head and (job, range); heads; all of them
@@ -362,7 +362,9 @@ cudaError_t set_smem(K kernel, size_t bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-int sm_count() {
+}  // namespace
+
+int smat_sm_count() {
   static int sms = 0;
   if (!sms) {
     int dev = 0;
@@ -373,10 +375,6 @@ int sm_count() {
   return sms;
 }
 
-}  // namespace
-
-bool smat_pool_one_round(int64_t states) { return states <= sm_count(); }
-
 namespace {
 
 template <int R, int PD, typename T, int TK>
@@ -386,7 +384,7 @@ cudaError_t launch_pool_tk(const PoolList& list, int64_t Tlen, int* clear, cudaS
   if (err != cudaSuccess) return err;
   const int64_t items = list.first[list.a.jobs];
   const int per_sm = smem <= 110 * 1024 ? 2 : 1;
-  const int64_t grid = items < (int64_t)sm_count() * per_sm ? items : (int64_t)sm_count() * per_sm;
+  const int64_t grid = items < (int64_t)smat_sm_count() * per_sm ? items : (int64_t)smat_sm_count() * per_sm;
   return smat_launch_pdl(pool_stream_kernel<R, PD, T, TK>, dim3((unsigned)grid), 256, smem, st, list, Tlen, clear);
 }
 
@@ -395,7 +393,7 @@ cudaError_t launch_pool_tk(const PoolList& list, int64_t Tlen, int* clear, cudaS
 // together with the 16-row tiles); else few, so that two CTAs share an SM.
 template <int R, int PD, typename T>
 cudaError_t launch_pool(const PoolList& list, int64_t Tlen, int* clear, cudaStream_t st) {
-  if (smat_pool_one_round(list.first[list.a.jobs])) return launch_pool_tk<R, PD, T, 64>(list, Tlen, clear, st);
+  if (list.first[list.a.jobs] <= smat_sm_count()) return launch_pool_tk<R, PD, T, 64>(list, Tlen, clear, st);
   return launch_pool_tk<R, PD, T, sizeof(T) == 2 ? 32 : 16>(list, Tlen, clear, st);
 }
 
@@ -406,7 +404,7 @@ cudaError_t launch_read(const ReadList& list, int64_t Tlen, int* status, cudaStr
   if (err != cudaSuccess) return err;
   const int64_t items = list.first[list.a.jobs];
   const int per_sm = smem <= 112 * 1024 ? 2 : 1;
-  const int64_t grid = items < (int64_t)sm_count() * per_sm ? items : (int64_t)sm_count() * per_sm;
+  const int64_t grid = items < (int64_t)smat_sm_count() * per_sm ? items : (int64_t)smat_sm_count() * per_sm;
   return smat_launch_pdl(state_read_stream_kernel<R, PD, T>, dim3((unsigned)(grid + list.scan_ctas)), 256, smem, st, list, Tlen, status);
 }
 

@@ -27,3 +27,28 @@ def test_one_head_equals_one_of_many(d, T, chunk, dk, dv, many):
         results.append([o[:, -1].clone() for o in out])
     for a, b in zip(*results):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("d,heads,T,width,apart", [(2, 1, 512, 64, False), (2, 9, 512, 128, False), (2, 10, 512, 128, True),
+                                                   (2, 37, 512, 64, False), (2, 38, 512, 64, True), (2, 128, 512, 128, True),
+                                                   (3, 8, 1024, 128, False), (3, 8, 2048, 128, True), (1, 1, 512, 64, True)])
+def test_where_the_chunk_scan_runs(d, heads, T, width, apart):
+    """A launch of its own from the size on where its CTAs would hold up the routed read (148 SMs); results do not depend on it."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(heads)
+    x = [torch.randn(1, heads, T, width, generator=g, device="cuda") / width ** 0.5 for _ in range(4)]
+    plan = binding.SmatPlan(1, heads, T, width, width, d, 64, "f32")
+    ref = binding.SmatPlan(1, 1, T, width, width, d, 64, "f32")   # one head: beside the read
+    plan.profile_enable(True)
+    stages = []
+    O = plan.forward(*x[:3])
+    torch.cuda.synchronize()
+    stages += [name for name, _ in plan.profile_read()]
+    grads = plan.backward(*x)
+    torch.cuda.synchronize()
+    stages += [name for name, _ in plan.profile_read()]
+    plan.profile_enable(False)
+    assert ("scan" in stages, "bwd_scan" in stages) == (apart, apart)
+    last = [t[:, -1:].contiguous() for t in x]
+    for a, b in zip((O, *grads), (ref.forward(*last[:3]), *ref.backward(*last))):
+        assert torch.equal(a[:, -1:], b)
