@@ -321,10 +321,10 @@ __global__ void mask_kernel(uint8_t* mask, const SmatGeo geo) {
 
 template <typename T, int SD, int OD, int ROWS>
 static cudaError_t launch_tile_rows_of(SmatTileArgs a, int bh, cudaStream_t st) {
-  constexpr int smem = TileLayout<T, SD, OD, ROWS>::SMEM;
+  const unsigned blocks = (unsigned)((a.c + ROWS - 1) / ROWS);
+  const int smem = smat_smem_alone((int64_t)a.jobs * a.NC * blocks * bh, TileLayout<T, SD, OD, ROWS>::SMEM);
   cudaError_t err = cudaFuncSetAttribute(tile_rows_kernel<T, SD, OD, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
-  const unsigned blocks = (unsigned)((a.c + ROWS - 1) / ROWS);
   const size_t rows = (size_t)bh * a.T * sizeof(T);
   a.together = 0;
   for (int j = 0; j < a.jobs; ++j)
@@ -338,7 +338,7 @@ static cudaError_t launch_tile_rows_of(SmatTileArgs a, int bh, cudaStream_t st) 
 template <typename T, int SD, int OD>
 static cudaError_t launch_tile_rows(const SmatTileArgs& a, int bh, cudaStream_t st) {
   const int64_t ctas = (int64_t)a.jobs * a.NC * ((a.c + 15) / 16) * bh;
-  return ctas <= 148 ? launch_tile_rows_of<T, SD, OD, 16>(a, bh, st) : launch_tile_rows_of<T, SD, OD, 32>(a, bh, st);
+  return ctas <= smat_sm_count() ? launch_tile_rows_of<T, SD, OD, 16>(a, bh, st) : launch_tile_rows_of<T, SD, OD, 32>(a, bh, st);
 }
 
 cudaError_t smat_launch_tile_rows(const SmatTileArgs& a, int bf16, int score_dim, int out_dim, int bh, cudaStream_t st) {

@@ -379,10 +379,10 @@ namespace {
 
 template <int R, int PD, typename T, int TK>
 cudaError_t launch_pool_tk(const PoolList& list, int64_t Tlen, int* clear, cudaStream_t st) {
-  const size_t smem = R * PD * 4 + 2 * TK * (R + PD) * sizeof(T);
+  const int64_t items = list.first[list.a.jobs];
+  const size_t smem = smat_smem_alone(items, R * PD * 4 + 2 * TK * (R + PD) * (int)sizeof(T));
   cudaError_t err = set_smem(pool_stream_kernel<R, PD, T, TK>, smem);
   if (err != cudaSuccess) return err;
-  const int64_t items = list.first[list.a.jobs];
   const int per_sm = smem <= 110 * 1024 ? 2 : 1;
   const int64_t grid = items < (int64_t)smat_sm_count() * per_sm ? items : (int64_t)smat_sm_count() * per_sm;
   return smat_launch_pdl(pool_stream_kernel<R, PD, T, TK>, dim3((unsigned)grid), 256, smem, st, list, Tlen, clear);
