@@ -24,6 +24,7 @@ struct smat_plan {
   size_t off_status, off_sin, off_F, off_U, off_acc, off_W, off_fwd_end;
   size_t off_dbar, off_ubar, off_fbar, off_acc2, off_bwd_end;
   size_t off_plist, off_poffs, off_tlist, off_toffs;   // token lists of user-supplied routing (int32)
+  size_t off_pheavy, off_theavy;                       // ... and parts of their heavy groups
   size_t off_lr3;         // tensor-core backward: third buffer of bf16 long-range rows (the first two share off_acc)
   size_t off_sin_tiles;   // KEEP_FORWARD_TABLES on tensor-core plans: the bf16 state entering every tile, left by the forward
   size_t off_lam, off_dlam, off_gq, off_gk, off_glr, off_gdo, off_gv, off_gvlr;   // gated variant (SMAT_FLAG_GATED)
@@ -125,6 +126,7 @@ SmatGroupSpec group(const smat_plan* pl, int mode) {
   const int64_t tokens = mode == SMAT_GM_PROFILE ? s.n : s.T - s.n;
   s.base = tokens / s.period; s.rem = tokens % s.period;
   s.list = nullptr; s.offs = nullptr; s.list_stride = 0; s.offs_stride = 0;
+  s.heavy = nullptr; s.heavy_count = nullptr;
   return s;
 }
 
@@ -145,15 +147,26 @@ struct Ctx {
   float* f(size_t off) const { return reinterpret_cast<float*>(ws + off); }
 };
 
+// The 256 bytes at off_status: the status word, and at these offsets the numbers of heavy parts of a routed pass.
+constexpr size_t PROF_HEAVY_COUNT = 128, TYPE_HEAVY_COUNT = 192;
+
+SmatRouteLists route_lists(const Ctx& cx, bool prof) {
+  const smat_plan* pl = cx.pl;
+  auto i32 = [&](size_t off) { return reinterpret_cast<int32_t*>(cx.ws + off); };
+  return SmatRouteLists{i32(prof ? pl->off_plist : pl->off_tlist), i32(prof ? pl->off_poffs : pl->off_toffs),
+                        reinterpret_cast<SmatHeavyPart*>(cx.ws + (prof ? pl->off_pheavy : pl->off_theavy)),
+                        i32(pl->off_status + (prof ? PROF_HEAVY_COUNT : TYPE_HEAVY_COUNT))};
+}
+
 SmatGroupSpec group(const Ctx& cx, int mode) {
   const smat_plan* pl = cx.pl;
   SmatGroupSpec s = group(pl, mode);
   if (cx.routed && mode != SMAT_GM_CHUNK) {
     const bool prof = mode == SMAT_GM_PROFILE;
-    s.list = reinterpret_cast<const int32_t*>(cx.ws + (prof ? pl->off_plist : pl->off_tlist));
-    s.offs = reinterpret_cast<const int32_t*>(cx.ws + (prof ? pl->off_poffs : pl->off_toffs));
     s.list_stride = prof ? pl->geo.n : pl->geo.m;
     s.offs_stride = (prof ? pl->geo.P : pl->geo.B) + 1;
+    const SmatRouteLists to = route_lists(cx, prof);
+    s.list = to.list; s.offs = to.offs; s.heavy = to.heavy; s.heavy_count = to.heavy_count;
   }
   return s;
 }
@@ -504,6 +517,8 @@ smat_status smat_plan_create(smat_plan** out, int batch, int heads, int64_t T, i
   pl->off_poffs = off;  off = align_up(off + (lists ? (size_t)pl->bh * (g.P + 1) * 4 : 0));
   pl->off_tlist = off;  off = align_up(off + (lists ? (size_t)pl->bh * g.m * 4 : 0));
   pl->off_toffs = off;  off = align_up(off + (lists ? (size_t)pl->bh * (g.B + 1) * 4 : 0));
+  pl->off_pheavy = off; off = align_up(off + (lists ? (size_t)pl->bh * (g.n / SMAT_HEAVY_TOKENS) * sizeof(SmatHeavyPart) : 0));
+  pl->off_theavy = off; off = align_up(off + (lists ? (size_t)pl->bh * (g.m / SMAT_HEAVY_TOKENS) * sizeof(SmatHeavyPart) : 0));
   // gated variant: λ and the rescaled copies of Q, K (forward) and dO, V (backward), in the plan's dtype
   const size_t esz = dtype == SMAT_BF16 ? 2 : 4;
   const size_t gated = (flags & SMAT_FLAG_GATED) ? 1 : 0;
@@ -616,9 +631,8 @@ smat_status begin_routing(Ctx& cx, const int32_t* prof, const int32_t* type) {
   if ((reinterpret_cast<uintptr_t>(prof) | reinterpret_cast<uintptr_t>(type)) & 3) return SMAT_ERR_ALIGN;
   const int64_t gmax = pl->geo.P > pl->geo.B ? pl->geo.P : pl->geo.B;
   if (gmax > smat_routing_max_groups()) return SMAT_ERR_UNSUPPORTED;
-  auto i32 = [&](size_t off) { return reinterpret_cast<int32_t*>(cx.ws + off); };
-  SMAT_TRY(cx, "routing_lists", smat_launch_routing_lists(prof, type, i32(pl->off_plist), i32(pl->off_poffs),
-                                                          i32(pl->off_tlist), i32(pl->off_toffs), pl->geo, pl->bh, cx.st));
+  SMAT_TRY(cx, "routing_lists", smat_launch_routing_lists(prof, type, route_lists(cx, true), route_lists(cx, false), pl->geo,
+                                                          pl->bh, cx.st));
   cx.routed = true;
   cx.prof = prof; cx.type = type;
   return SMAT_OK;

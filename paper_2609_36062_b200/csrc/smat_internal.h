@@ -13,6 +13,13 @@
 //   TYPE    g = type h             recent tokens with (t-n+1) ≡ h (mod B), t < T  (Eq. "schedule", U_h)
 enum SmatGroupMode { SMAT_GM_NONE = 0, SMAT_GM_CHUNK = 1, SMAT_GM_PROFILE = 2, SMAT_GM_TYPE = 3 };
 
+// A listed group may hold any number of tokens: what it has behind its first SMAT_HEAVY_TOKENS is cut into parts of at most
+// as many, for kernels that hand these out to several CTAs.
+constexpr int SMAT_HEAVY_TOKENS = 128;
+struct SmatHeavyPart {
+  uint16_t bh, group;   // (a plan has at most 65535 heads, a routed call 27000 groups)
+  int32_t first;        // tokens of the group in front of the part
+};
 struct SmatGroupSpec {
   int mode;
   int64_t n, T, c, period;  // period = P (PROFILE) or B (TYPE)
@@ -23,6 +30,8 @@ struct SmatGroupSpec {
   const int32_t* list;
   const int32_t* offs;
   int64_t list_stride, offs_stride;
+  const SmatHeavyPart* heavy;   // the parts of all heads, *heavy_count of them in any order (null: positional groups)
+  const int32_t* heavy_count;
 };
 
 // a / b of non-negative numbers; a 64-bit division takes the device several hundred cycles, and every role of a persistent
@@ -249,11 +258,17 @@ cudaError_t smat_launch_gate_dlam(const void* Q, const void* dQ, const void* K, 
 cudaError_t smat_launch_normalize_step(int step, const void* a, const void* b, void* out, int bf16, int p, int64_t rows,
                                        cudaStream_t st);
 // Token lists of user-supplied routing: prof [bh][n] (cells in [0, P)) and type [bh][m] (types in [0, B)) -> CSR lists
-// (offsets [bh][G + 1], token positions [bh][count], ascending inside a group).  Keys out of range are dropped.
+// (offsets [bh][G + 1], token positions [bh][count], ascending inside a group).  Keys out of range are dropped.  Parts of
+// heavy groups are appended at heavy (room for bh * (count / SMAT_HEAVY_TOKENS)) and added to *heavy_count, zero before.
+struct SmatRouteLists {
+  int32_t* list;
+  int32_t* offs;
+  SmatHeavyPart* heavy;
+  int32_t* heavy_count;
+};
 int64_t smat_routing_max_groups();
-cudaError_t smat_launch_routing_lists(const int32_t* prof, const int32_t* type, int32_t* prof_list, int32_t* prof_offs,
-                                      int32_t* type_list, int32_t* type_offs, const SmatGeo& geo, int bh,
-                                      cudaStream_t st);
+cudaError_t smat_launch_routing_lists(const int32_t* prof, const int32_t* type, const SmatRouteLists& prof_to,
+                                      const SmatRouteLists& type_to, const SmatGeo& geo, int bh, cudaStream_t st);
 // Zeroes the row (row_bytes bytes at rows + (bh*T + first + i) * row_bytes) of every token i whose key lies outside [0, G).
 cudaError_t smat_launch_zero_unrouted(const int32_t* key, int64_t count, int64_t G, int64_t first, void* rows, int64_t T,
                                       int row_bytes, int bh, cudaStream_t st);

@@ -17,15 +17,15 @@ constexpr int ROUTE_THREADS = 256;
 //   1. every warp histograms the keys of its range in its own row of counters (keys outside [0, G) are dropped:
 //      such a token belongs to no group)
 //   2. totals per group, exclusive scan -> offs[0 .. G]; row w then becomes the first slot of group g for warp w's
-//      tokens: offs[g] + the counts of the warps before it
+//      tokens: offs[g] + the counts of the warps before it; a heavy group's parts are noted (their order depends on thread
+//      timing, but each is a set of rows that some CTA reads on their own)
 //   3. stable placement: every warp walks ITS range in order, 32 tokens at a time; lanes with equal keys find each other
 //      with match.any, the lowest such lane advances the warp's cursor of the group, every lane writes its token's
 //      position.  Ranges are in token order and each warp's slots follow those of the warps before it, so the list of
 //      a group is ascending.
 struct RouteParams {
   const int32_t* key[2];   // [bh][count]
-  int32_t* list[2];        // [bh][count]
-  int32_t* offs[2];        // [bh][G + 1]
+  SmatRouteLists to[2];    // lists [bh][count], offsets [bh][G + 1]
   int64_t count[2], G[2], first[2];   // tokens per head, groups, position of the first token of the kind
   int warps;               // W: rows of per-warp counters in shared memory
 };
@@ -38,8 +38,9 @@ __global__ void __launch_bounds__(ROUTE_THREADS) routing_lists_kernel(const __gr
   const int64_t bh = blockIdx.x, n = prm.count[kind], G = prm.G[kind], pitch = G + 1;
   const int W = prm.warps;
   const int32_t* key = prm.key[kind] + bh * n;
-  int32_t* list = prm.list[kind] + bh * n;
-  int32_t* offs = prm.offs[kind] + bh * pitch;
+  const SmatRouteLists& to = prm.to[kind];
+  int32_t* list = to.list + bh * n;
+  int32_t* offs = to.offs + bh * pitch;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int32_t* total = rows;
   for (int64_t i = tid; i < (1 + W) * pitch; i += ROUTE_THREADS) rows[i] = 0;
@@ -89,6 +90,12 @@ __global__ void __launch_bounds__(ROUTE_THREADS) routing_lists_kernel(const __gr
       const int32_t c = rows[(1 + w) * pitch + g];
       rows[(1 + w) * pitch + g] = slot;
       slot += c;
+    }
+    const int32_t parts = (total[g + 1] - total[g] - 1) / SMAT_HEAVY_TOKENS;   // (behind the first; none of an empty group)
+    if (parts > 0) {
+      const int32_t at = atomicAdd(to.heavy_count, parts);
+      for (int32_t i = 0; i < parts; ++i)
+        to.heavy[at + i] = SmatHeavyPart{(uint16_t)bh, (uint16_t)g, (i + 1) * SMAT_HEAVY_TOKENS};
     }
   }
   __syncthreads();
@@ -142,12 +149,11 @@ cudaError_t smat_launch_zero_unrouted(const int32_t* key, int64_t count, int64_t
 // Largest group count the list builder handles (its cursors live in shared memory).
 int64_t smat_routing_max_groups() { return 27000; }
 
-cudaError_t smat_launch_routing_lists(const int32_t* prof, const int32_t* type, int32_t* prof_list, int32_t* prof_offs,
-                                      int32_t* type_list, int32_t* type_offs, const SmatGeo& geo, int bh,
-                                      cudaStream_t st) {
+cudaError_t smat_launch_routing_lists(const int32_t* prof, const int32_t* type, const SmatRouteLists& prof_to,
+                                      const SmatRouteLists& type_to, const SmatGeo& geo, int bh, cudaStream_t st) {
   RouteParams prm;
-  prm.key[0] = prof; prm.list[0] = prof_list; prm.offs[0] = prof_offs; prm.count[0] = geo.n; prm.G[0] = geo.P; prm.first[0] = 0;
-  prm.key[1] = type; prm.list[1] = type_list; prm.offs[1] = type_offs; prm.count[1] = geo.m; prm.G[1] = geo.B; prm.first[1] = geo.n;
+  prm.key[0] = prof; prm.to[0] = prof_to; prm.count[0] = geo.n; prm.G[0] = geo.P; prm.first[0] = 0;
+  prm.key[1] = type; prm.to[1] = type_to; prm.count[1] = geo.m; prm.G[1] = geo.B; prm.first[1] = geo.n;
   const int64_t gmax = geo.P > geo.B ? geo.P : geo.B;
   if (gmax > smat_routing_max_groups()) return cudaErrorInvalidConfiguration;
   int64_t warps = (int64_t)(220 * 1024 / sizeof(int32_t)) / (gmax + 1) - 1;

@@ -1324,7 +1324,7 @@ struct ReadParams {
   int64_t T;             // tokens per head
   SmatGroupSpec grp;     // which tokens share a state: types (recent tokens) or profiles (distant tokens)
   int64_t groups;        // states per head
-  int64_t items;         // heads * groups
+  int64_t states;        // heads * groups
   const __nv_bfloat16* X;  // [bh][T][128] rows contracted against the state
   float* out;            // [bh][T][128] fp32 rows, or
   __nv_bfloat16* out_bf16;  // bf16 rows (when non-null)
@@ -1335,26 +1335,38 @@ struct ReadParams {
 
 // TRANS = 0: out[t][j] = Σ_i x_t[i] St[i][j]  (state as MN-major B);  TRANS = 1: out[t][i] = Σ_j x_t[j] St[i][j]
 // (the same two boxes read as a K-major B).
-// One pass of state_read_tc_kernel: up to TOK tokens of one (state, head) item; states without tokens are skipped.
-// Every role walks the same sequence.
+// One pass of state_read_tc_kernel: up to TOK tokens of one item, a (state, head) or, in front of these, a part of a heavy
+// group; states without tokens are skipped.  Every role walks the same sequence.
 template <int TOK>
 struct ReadPass {
   const ReadParams* pp;
-  int64_t item, stride;
-  int64_t bh, cnt, k0;
+  int64_t item, stride, parts;
+  int64_t state, bh, cnt, k0;
   SmatTokens tk;
-  __device__ ReadPass(const ReadParams& p, int64_t first, int64_t stride_) : pp(&p), item(first), stride(stride_) { load(); }
+  __device__ ReadPass(const ReadParams& p, int64_t first, int64_t stride_)
+      : pp(&p), item(first), stride(stride_), parts(p.grp.heavy ? *p.grp.heavy_count : 0) { load(); }
   __device__ void load() {
     k0 = 0;
-    for (; item < pp->items; item += stride) {
-      bh = smat_div(item, pp->groups);
-      tk = smat_group_tokens(pp->grp, bh, item - bh * pp->groups);
-      cnt = tk.cnt;
+    for (; valid(); item += stride) {
+      if (item < parts) {
+        const SmatHeavyPart part = pp->grp.heavy[item];
+        bh = part.bh;
+        state = bh * pp->groups + part.group;
+        tk = smat_group_tokens(pp->grp, bh, part.group);
+        tk.lst += part.first;
+        cnt = tk.cnt - part.first;
+      } else {
+        state = item - parts;
+        bh = smat_div(state, pp->groups);
+        tk = smat_group_tokens(pp->grp, bh, state - bh * pp->groups);
+        cnt = tk.cnt;
+      }
+      if (pp->grp.heavy && cnt > SMAT_HEAVY_TOKENS) cnt = SMAT_HEAVY_TOKENS;
       if (cnt > 0) break;
     }
   }
   __device__ int64_t token(int m) const { return tk.at(k0 + m); }   // position of row m of this pass
-  __device__ bool valid() const { return item < pp->items; }
+  __device__ bool valid() const { return item < parts + pp->states; }
   __device__ bool first() const { return k0 == 0; }
   __device__ bool last() const { return k0 + TOK >= cnt; }
   __device__ int tokens() const { const int64_t left = cnt - k0; return (int)(left < TOK ? left : TOK); }
@@ -1477,7 +1489,7 @@ __global__ void __launch_bounds__(160) state_read_tc_kernel(const __grid_constan
       if (!ahead.valid()) return;
       const uint32_t b = loads % NB;
       uint8_t* dst = sB + b * 2 * BOX_BYTES;
-      const int row = (int)(ahead.item * TILE);
+      const int row = (int)(ahead.state * TILE);
       mbar_expect_tx(bar_u + b, 2 * BOX_BYTES);
       tma_load_2d(dst, &tmU, 0, row, bar_u + b);
       tma_load_2d(dst + BOX_BYTES, &tmU, HALF, row, bar_u + b);
@@ -1889,31 +1901,39 @@ cudaError_t smat_launch_bwd_tiles_fused_tc(const void* Q, const void* K, const v
   return smat_launch_pdl(kernel, dim3(grid), FUSED_THREADS, FUSED_SMEM, st, tmQ, tmK, tmV, tmG, tmS, tmD, prm);
 }
 
+// Whether the read takes 32-row query tiles: where the tokens of every positional group fit one, and where listed groups have
+// fewer than 16 on average (their sizes are known to the device alone).  A listed group of more than SMAT_HEAVY_TOKENS is
+// then handed out in parts of four tiles, where one CTA walking it 32 tokens at a time is slower than 128 at a time.  Routed
+// pass, d = 3, 16 heads of 16 K tokens, uniform / half of the tokens in one group / all of them: 442 / 1149 / 1830 us with
+// 128-row tiles, 439 / 1276 / 2095 with 32-row ones and whole groups, 434 / 905 / 1311 with parts.
+static bool read_groups_small(const SmatGroupSpec& grp) { return grp.list ? grp.base < 16 : grp.base < 32; }
+// What a launch of the read walks, and its CTAs, `resident` of which share an SM.
+static int64_t read_items(ReadParams& prm, const SmatGroupSpec& grp, int64_t groups, int bh, int resident) {
+  prm.grp = grp; prm.groups = groups; prm.states = (int64_t)bh * groups;
+  if (!read_groups_small(grp)) prm.grp.heavy = nullptr;
+  const int64_t most = prm.states + (prm.grp.heavy ? bh * ((grp.mode == SMAT_GM_PROFILE ? grp.n : grp.T - grp.n) / SMAT_HEAVY_TOKENS) : 0);
+  const int64_t slots = (int64_t)resident * smat_sm_count();
+  return most < slots ? most : slots;
+}
+
 // Both adjoint reads of the profile states in one launch: out_t[t] = St x_t (rows Xt, the second state index
 // contracted) and out_n[t] = Stᵀ x_t (rows Xn, the first one), bf16 rows; every state is loaded once.
-// Whether a group's tokens fit the 32-row query tile: always for positional groups, on average (and half of it) for listed
-// ones, whose heavy groups take more passes.
-static bool read_groups_small(const SmatGroupSpec& grp) { return grp.list ? grp.base < 16 : grp.base < 32; }
-
 cudaError_t smat_launch_state_read_dual_tc(const void* Xt, const void* Xn, const void* state_bf16, void* out_t_bf16,
                                            void* out_n_bf16, const SmatGroupSpec& grp, int64_t groups, int64_t T, int bh,
                                            int* status, cudaStream_t st) {
   CUtensorMap tmU;
   if (!make_map(&tmU, state_bf16, (uint64_t)bh * groups * TILE)) return cudaErrorInvalidValue;
   ReadParams prm;
-  prm.T = T; prm.grp = grp; prm.groups = groups; prm.items = (int64_t)bh * groups;
+  prm.T = T;
   prm.X = static_cast<const __nv_bfloat16*>(Xt);
   prm.X2 = static_cast<const __nv_bfloat16*>(Xn);
   prm.out = nullptr;
   prm.out_bf16 = static_cast<__nv_bfloat16*>(out_t_bf16);
   prm.out2_bf16 = static_cast<__nv_bfloat16*>(out_n_bf16);
   prm.status = status;
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const bool small = read_groups_small(grp);
   const int smem = small ? ReadTcLayout<1, 32>::SMEM : ReadTcLayout<1, 128>::SMEM;
-  const int64_t grid = prm.items < 2LL * sms ? prm.items : 2LL * sms;   // 256 columns of tensor memory and up to 97 KB each
+  const int64_t grid = read_items(prm, grp, groups, bh, 2);   // 256 columns of tensor memory and up to 97 KB each
   auto kernel = small ? state_read_tc_kernel<1, 1, 32> : state_read_tc_kernel<1, 1, 128>;
   cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
@@ -1926,16 +1946,13 @@ cudaError_t smat_launch_state_read_tc(const void* X, const void* state_bf16, flo
   CUtensorMap tmU;
   if (!make_map(&tmU, state_bf16, (uint64_t)bh * groups * TILE)) return cudaErrorInvalidValue;
   ReadParams prm;
-  prm.T = T; prm.grp = grp; prm.groups = groups; prm.items = (int64_t)bh * groups;
+  prm.T = T;
   prm.X = static_cast<const __nv_bfloat16*>(X);
   prm.X2 = nullptr; prm.out2_bf16 = nullptr;
   prm.out = out;
   prm.out_bf16 = static_cast<__nv_bfloat16*>(out_bf16);
   prm.status = status;
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t grid = prm.items < 3LL * sms ? prm.items : 3LL * sms;
+  const int64_t grid = read_items(prm, grp, groups, bh, 3);
   const bool small = read_groups_small(grp);
   const int smem = small ? ReadTcLayout<0, 32>::SMEM : ReadTcLayout<0, 128>::SMEM;
   auto kernel = small ? (transposed ? state_read_tc_kernel<1, 0, 32> : state_read_tc_kernel<0, 0, 32>)

@@ -157,3 +157,25 @@ def test_group_sizes_at_the_edges_of_passes_and_parts(dtype, d, T, c, sizes):
         M = so.routed_dense_mask(geo, cells[h], types[h])
         for got, ref in zip((O, *grads), (so.forward_dense(Q64, K64, V64, M), *so.backward_dense(Q64, K64, V64, G64, M))):
             assert rel_err(to_numpy64(got[0, h]), ref) <= TOL[dtype]
+
+
+def test_a_heavy_type_is_read_by_many_ctas():
+    """All queries of a head share one type: the read takes no longer than a uniform one (twice: the slack), where one CTA per
+    head walking all of them takes several times as long."""
+    w = synth.Workload("heavy", 3, 1, 16, 16384, 128, 128, 128, "bf16", "normalised", 17)
+    _, dev = device_inputs(w)
+    plan = binding.SmatPlan(w.batch, w.heads, w.T, w.d_k, w.d_v, w.d, w.chunk, w.dtype)
+    geo = plan.geometry()
+    prof = torch.randint(geo.P, (w.bh, geo.n), device="cuda", dtype=torch.int32)
+    uniform = torch.randint(geo.B, (w.bh, geo.m), device="cuda", dtype=torch.int32)
+    plan.profile_enable(True)
+    took = []
+    for typ in (uniform, torch.full_like(uniform, 5)):
+        times = []
+        for _ in range(9):
+            plan.forward(dev["q"], dev["k"], dev["v"], prof=prof, type=typ)
+            torch.cuda.synchronize()
+            times.append(dict(plan.profile_read())["read_type_tc"])
+        took.append(sorted(times)[4])
+    plan.profile_enable(False)
+    assert took[1] <= 2 * took[0], took
