@@ -85,13 +85,14 @@ __global__ void __launch_bounds__(ROUTE_THREADS) routing_lists_kernel(const __gr
   // total[g] = tokens in groups < g (total[0] = 0): the offsets; then the per-warp first slots
   for (int64_t g = tid; g <= G; g += ROUTE_THREADS) offs[g] = total[g];
   for (int64_t g = tid; g < G; g += ROUTE_THREADS) {
-    int32_t slot = total[g];
+    const int32_t begin = total[g];
+    int32_t slot = begin;
     for (int w = 0; w < W; ++w) {
       const int32_t c = rows[(1 + w) * pitch + g];
       rows[(1 + w) * pitch + g] = slot;
       slot += c;
     }
-    const int32_t parts = (total[g + 1] - total[g] - 1) / SMAT_HEAVY_TOKENS;   // (behind the first; none of an empty group)
+    const int32_t parts = (slot - begin - 1) / SMAT_HEAVY_TOKENS;   // behind the first; none of an empty group
     if (parts > 0) {
       const int32_t at = atomicAdd(to.heavy_count, parts);
       for (int32_t i = 0; i < parts; ++i)

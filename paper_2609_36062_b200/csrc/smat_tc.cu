@@ -1335,8 +1335,9 @@ struct ReadParams {
 
 // TRANS = 0: out[t][j] = Σ_i x_t[i] St[i][j]  (state as MN-major B);  TRANS = 1: out[t][i] = Σ_j x_t[j] St[i][j]
 // (the same two boxes read as a K-major B).
-// One pass of state_read_tc_kernel: up to TOK tokens of one item, a (state, head) or, in front of these, a part of a heavy
-// group; states without tokens are skipped.  Every role walks the same sequence.
+// One pass of state_read_tc_kernel: up to TOK tokens of one item, a (state, head) or, behind these, a part of a heavy group;
+// states without tokens are skipped.  Every role walks the same sequence.  (Behind, so that the first item does not wait for
+// the number of parts.)
 template <int TOK>
 struct ReadPass {
   const ReadParams* pp;
@@ -1348,25 +1349,25 @@ struct ReadPass {
   __device__ void load() {
     k0 = 0;
     for (; valid(); item += stride) {
-      if (item < parts) {
-        const SmatHeavyPart part = pp->grp.heavy[item];
+      if (item < pp->states) {
+        state = item;
+        bh = smat_div(state, pp->groups);
+        tk = smat_group_tokens(pp->grp, bh, state - bh * pp->groups);
+        cnt = tk.cnt;
+      } else {
+        const SmatHeavyPart part = pp->grp.heavy[item - pp->states];
         bh = part.bh;
         state = bh * pp->groups + part.group;
         tk = smat_group_tokens(pp->grp, bh, part.group);
         tk.lst += part.first;
         cnt = tk.cnt - part.first;
-      } else {
-        state = item - parts;
-        bh = smat_div(state, pp->groups);
-        tk = smat_group_tokens(pp->grp, bh, state - bh * pp->groups);
-        cnt = tk.cnt;
       }
       if (pp->grp.heavy && cnt > SMAT_HEAVY_TOKENS) cnt = SMAT_HEAVY_TOKENS;
       if (cnt > 0) break;
     }
   }
   __device__ int64_t token(int m) const { return tk.at(k0 + m); }   // position of row m of this pass
-  __device__ bool valid() const { return item < parts + pp->states; }
+  __device__ bool valid() const { return item < pp->states || item < pp->states + parts; }
   __device__ bool first() const { return k0 == 0; }
   __device__ bool last() const { return k0 + TOK >= cnt; }
   __device__ int tokens() const { const int64_t left = cnt - k0; return (int)(left < TOK ? left : TOK); }
