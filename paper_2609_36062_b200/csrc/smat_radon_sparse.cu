@@ -78,6 +78,8 @@ constexpr int sparse_smem(const SparseShape& s) { return 1024 + s.ring * s.slot_
 // barriers end inside the allocation; values lie on columns that are multiples of eight, the positions of a pair of steps on
 // multiples of four, all behind the accumulators; the rows of the extra class (whole lines) lie in the dense tile.
 constexpr bool sparse_layout_ok(const SparseShape& s) {
+  for (int t = 0; t < s.tiles; ++t)
+    if (s.col(t) % 8 != 0 || (t < s.dense && (s.col(t) + 8 * s.steps) % 4 != 0)) return false;
   const int in_steps = s.tail >= 0 ? s.rows - 1 : s.rows;
   return s.slot_bytes % 1024 == 0 && s.rows <= s.slot_rows && s.steps * 32 <= s.slot_rows && s.dense_steps * 16 <= s.slot_rows &&
          s.steps * 32 >= in_steps && s.dense_steps * 16 >= in_steps &&

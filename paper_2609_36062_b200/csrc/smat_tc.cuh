@@ -198,7 +198,8 @@ __device__ __forceinline__ void mma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, ui
 // A with two nonzeros at most in every four columns: A (128 x 32) comes from tensor memory as its 16 kept values per row
 // (8 columns) and their positions, 4 bits to a group of four inputs: (index of the second value << 2) | index of the first.
 // The positions of row m, inputs 16 h to 16 h + 15, are half-word (m / 8) % 2 of lane 16 (m / 16) + 8 h + m % 8 in one of
-// the two columns at `tmem_meta` (even); make_idesc_sparse names which.
+// the first two columns at `tmem_meta`; make_idesc_sparse names which (0 or 1).  tmem_a is a multiple of 8 columns, tmem_meta
+// of 4.
 __host__ __device__ constexpr uint32_t make_idesc_sparse(int M, int N, int a_mn_major, int b_mn_major, int meta_column) {
   return make_idesc(M, N, a_mn_major, b_mn_major) | (1u << 2) | (uint32_t)meta_column;
 }
