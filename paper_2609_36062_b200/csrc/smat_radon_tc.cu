@@ -33,13 +33,11 @@
 // entries, rewritten for every slab, stored and loaded with the L2 evict-last priority while F and U stream with
 // evict-first) and the full-size W table is never built.  The storing warps make the slab's rows visible (memory
 // fence, proxy fence) and arrive on a barrier the producer waits on before the first stage-2 load.
-// q = 11 also sends its output tiles off by TMA: the epilogue writes the rounded tile into the item's own ring slot
-// (as large as a tile, and dead once the MMAs have read it) in the box layout, and lane 0 of warp 18 issues the tile
-// stores and frees the slot; the bulk of the stores bypasses the LSU.
-// The kernel exists twice: radon_tc_kernel<false> for one stage per launch with every index through the MMAs (small
-// primes), without cache hints, phase tables or ALU warps; radon_tc_kernel<true> with them.
-// (The tile-store path is written for several slots per item and is compiled into both, but the launcher switches it on
-// for q = 11 only.)
+// That stage (d = 3, q = 11, forward) also sends its output tiles off by TMA: the epilogue writes the rounded tile into the
+// item's own ring slot (as large as a tile, and dead once the MMAs have read it) in the box layout, and lane 0 of warp 18
+// issues the tile stores and frees the slot; the bulk of the stores bypasses the LSU.
+// The kernel exists twice: radon_tc_kernel<false> for one stage per launch with every index through the MMAs and direct
+// stores (small primes), without cache hints or phase tables; radon_tc_kernel<true> with them.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -84,12 +82,10 @@ struct RadonParams {
   int32_t nreg, nslots;            // slots of regular lines per image; plus one when the input has the extra class
   int32_t rows_mma;                // output indices of the MMA tile (<= 128)
   int32_t alu_rows;                // output indices rows_mma .. (all of the extra class) summed on the ALUs, straight from
-                                   // the ring slot; 0: every index goes through the MMAs
+                                   // the ring slot; the tile then leaves through that slot and TMA stores.  0: every index
+                                   // goes through the MMAs, direct stores
   int32_t ring;                    // ring slots
-  int32_t tma_out;                 // the output tile leaves through the item's own ring slot and TMA stores (q = 11)
-  int32_t mini_bytes;              // tma_out: per slot, room for the extra-class rows of the tile (two halves); 0: the
-                                   // extra-class rows sit in the tile itself, after its regular lines
-  int32_t lines_out;               // tma_out: regular lines of the tile (the store box)
+  int32_t mini_bytes;              // alu_rows: per slot, room for the extra-class rows of the tile (two halves)
   int32_t nph;                     // 1, or 2: both stages of the d = 4 tabulation, slab by slab
   int32_t slabs_per_head;          // rp / 128
   int64_t slabs;                   // heads * slabs_per_head
@@ -195,13 +191,6 @@ __device__ __forceinline__ void st_global_v8_hint(void* dst, uint32_t w0, uint32
                "r"(w1), "r"(w2), "r"(w3), "r"(w4), "r"(w5), "r"(w6), "r"(w7), "l"(pol)
                : "memory");
 }
-__device__ __forceinline__ void st_global_v4_hint(void* dst, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3,
-                                                  uint64_t pol) {
-  asm volatile("st.global.L2::cache_hint.v4.b32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(dst), "r"(w0), "r"(w1), "r"(w2),
-               "r"(w3), "l"(pol)
-               : "memory");
-}
-
 // Tile stores: shared memory (box layout, 128-byte swizzle) -> global, as one bulk group per item.
 __device__ __forceinline__ void tma_store_5d(const CUtensorMap* map, const void* smem_src, int c0, int c1, int c2, int c3,
                                              int c4, uint64_t pol) {
@@ -253,8 +242,6 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
                                                                     const __grid_constant__ CUtensorMap tm_vert1,
                                                                     const __grid_constant__ CUtensorMap tm_oreg0,
                                                                     const __grid_constant__ CUtensorMap tm_overt0,
-                                                                    const __grid_constant__ CUtensorMap tm_oreg1,
-                                                                    const __grid_constant__ CUtensorMap tm_overt1,
                                                                     const RadonParams prm) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -270,28 +257,26 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
   uint64_t* acc_full = empty + prm.ring;    // [MAX_ACC] accumulator complete
   uint64_t* acc_empty = acc_full + MAX_ACC; // [MAX_ACC] accumulator read out (one arrival per epilogue warp)
   uint64_t* w_ready = acc_empty + MAX_ACC;  // phase 0 of the current slab written out (one arrival per storing warp)
-  uint64_t* staged = w_ready + 1;           // [ring] tma_out: an item's tile is complete in its first slot (one arrival per
-                                            // epilogue warp); indexed by the item count modulo the ring size
+  uint64_t* staged = w_ready + 1;           // [ring] tma_out: the item's tile is complete in its slot (one arrival per
+                                            // epilogue warp)
   uint64_t* alu_done = staged + prm.ring;   // [ring] tma_out: the ALU warps have read the slot and written their rows
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(alu_done + prm.ring);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WaitCtx wc{cta_abort, prm.status};
-  const bool alu_here = FEAT && prm.alu_rows > 0;
-  const bool tma_out = prm.tma_out != 0;
+  const bool tma_out = FEAT && prm.alu_rows > 0;
   const uint32_t nph = FEAT ? (uint32_t)prm.nph : 1u;
 
   if (threadIdx.x == 0) {
     *cta_abort = 0;
     for (int s = 0; s < prm.ring; ++s) {
       mbar_init(full + s, 1);
-      mbar_init(empty + s, tma_out ? 1 : (alu_here ? 1 + ALU_WARPS : 1));   // tma_out: the storing thread frees the slot
+      mbar_init(empty + s, 1);   // (tma_out: the storing thread frees the slot)
       mbar_init(alu_done + s, ALU_WARPS);
       mbar_init(staged + s, EPI_WARPS);
     }
     for (int b = 0; b < MAX_ACC; ++b) { mbar_init(acc_full + b, 1); mbar_init(acc_empty + b, EPI_WARPS); }
-    mbar_init(w_ready, tma_out ? 1 : (alu_here ? EPI_WARPS + ALU_WARPS : EPI_WARPS));
-
+    mbar_init(w_ready, EPI_WARPS);
     fence_barrier_init();
     prefetch_tmap(&tm_reg0);
     prefetch_tmap(&tm_vert0);
@@ -343,57 +328,34 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
   const uint32_t first = blockIdx.x, step = gridDim.x;
   const uint32_t sph = (uint32_t)prm.slabs_per_head;
 
-  // ---- storing thread (tma_out): one bulk group of tile stores per item; the item's first slot, which holds the tile,
-  // goes back to the producer when the stores have read it.  Lane 0 of the second MMA warp when every item is one
-  // slot (that warp has no items then), else lane 0 of warp 19.
+  // ---- storing thread (tma_out: one stage, one slot per item): one bulk group of tile stores per item; the slot, which holds
+  // the tile, goes back to the producer when the stores have read it.  Lane 0 of the second MMA warp, which has no items then.
   auto store_role = [&]() {
     pdl_wait();
+    const RadonPhase& ph = prm.ph[0];
     const uint32_t ring = (uint32_t)prm.ring;
-    uint32_t slot = 0, prev_slot = 0;
-    uint32_t sidx = 0, spar = 0;                                // the item's "staged" barrier (items mod ring) and its parity
+    uint32_t slot = 0, prev_slot = 0, par = 0;                  // par: what a slot's "staged" barrier shows
     bool have_prev = false;
-    const int xrow0 = q * q;                                    // tile row of the first extra-class index
     for (ItemIter it(prm, first, step, nph); it.left; it.next()) {
-      const RadonPhase& ph = FEAT ? prm.ph[it.ph] : prm.ph[0];
-      const CUtensorMap* oreg = FEAT && it.ph ? &tm_oreg1 : &tm_oreg0;
-      const CUtensorMap* overt = FEAT && it.ph ? &tm_overt1 : &tm_overt0;
       const uint32_t head = it.slab / sph;
-      const int e0 = ph.dst_private ? 0 : (int)(it.slab - head * sph) * 128;
-      const int hc = ph.dst_private ? (int)blockIdx.x : (int)head;
-      const uint64_t pol = it.ph ? pol_dst1 : pol_dst0;
-      if (!mbar_wait(staged + sidx, spar, wc)) break;
-      if (++sidx == ring) { sidx = 0; spar ^= 1; }
-      const uint8_t* tile = sRing + slot * slot_bytes;
-      tma_store_5d(oreg, tile, e0, 0, 0, (int)it.img, hc, pol);
-      tma_store_5d(oreg, tile + prm.sr * 128, e0 + 64, 0, 0, (int)it.img, hc, pol);
-      if (ph.out.count > q * q && xrow0 < prm.rows_mma && (int)it.img >= ph.out.vert_from) {
+      const int e0 = (int)(it.slab - head * sph) * 128;
+      if (!mbar_wait(staged + slot, par, wc)) break;
+      const uint8_t *tile = sRing + slot * slot_bytes, *mini = sMini + slot * prm.mini_bytes;
+      tma_store_5d(&tm_oreg0, tile, e0, 0, 0, (int)it.img, (int)head, pol_dst0);
+      tma_store_5d(&tm_oreg0, tile + prm.sr * 128, e0 + 64, 0, 0, (int)it.img, (int)head, pol_dst0);
+      if ((int)it.img >= ph.out.vert_from) {
         const int ci = ph.out.sv_img != 0 ? (int)it.img : 0;   // the map's image stride is sv_img rows
-        if (prm.mini_bytes) {
-          const uint8_t* mini = sMini + slot * prm.mini_bytes;
-          tma_store_4d(overt, mini, e0, 0, ci, hc, pol);
-          tma_store_4d(overt, mini + prm.mini_bytes / 2, e0 + 64, 0, ci, hc, pol);
-        } else {
-          tma_store_4d(overt, tile + xrow0 * 128, e0, 0, ci, hc, pol);
-          tma_store_4d(overt, tile + prm.sr * 128 + xrow0 * 128, e0 + 64, 0, ci, hc, pol);
-        }
+        tma_store_4d(&tm_overt0, mini, e0, 0, ci, (int)head, pol_dst0);
+        tma_store_4d(&tm_overt0, mini + prm.mini_bytes / 2, e0 + 64, 0, ci, (int)head, pol_dst0);
       }
       bulk_commit();
       if (have_prev) {
         bulk_wait_read<1>();
         mbar_arrive(empty + prev_slot);
       }
-      if (it.closes_phase0()) {   // the slab's stage-1 rows are in memory before the producer loads them back
-        bulk_wait_all();
-        fence_proxy_async_all();
-        mbar_arrive(empty + slot);
-        mbar_arrive(w_ready);
-        have_prev = false;
-      } else {
-        prev_slot = slot;
-        have_prev = true;
-      }
-      slot += (uint32_t)prm.nslots;
-      if (slot >= ring) slot -= ring;
+      prev_slot = slot;
+      have_prev = true;
+      if (++slot == ring) { slot = 0; par ^= 1; }
     }
     if (have_prev) { bulk_wait_read<0>(); mbar_arrive(empty + prev_slot); }
     bulk_wait_all();
@@ -460,7 +422,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
     // share R and the slot layout, so the issuers only count items. ---------------------------------------------
     pdl_wait();
     const uint32_t me = (uint32_t)(warp - MMA_WARP);
-    if (tma_out && me == 1 && prm.nslots == 1) store_role();
+    if (tma_out && me == 1) store_role();
     constexpr uint32_t idesc = make_idesc(TILE_ROWS, 128, 0, 1);   // A from tensor memory (R), B MN-major (image rows)
     const uint64_t dB0 = make_desc(smem_u32(sRing), prm.sr * 128, 1024);
     const uint32_t slot16 = (uint32_t)slot_bytes >> 4;            // descriptor address units are 16 bytes
@@ -517,26 +479,20 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
         if (++buf == nacc) { buf = 0; if (n_item >= nacc) apar ^= 1; }
       }
     }
-  } else if (tma_out && prm.nslots > 1 && warp == ALU_WARP) {
-    if (lane == 0) store_role();
   } else if (FEAT && warp >= ALU_WARP) {
     // ---- leftover rows on the ALUs ----------------------------------------------------------------------------
     // q*q + q output indices rarely fill whole tiles of 128.  When only a few are left over, and they belong to the
     // extra class (index q*q + u = the sum of line u's q rows), these warps add the rows up from the slot itself
     // instead of a second, nearly empty tile paying for every MMA again.  A task is one leftover index and 8 state
-    // entries (one 16-byte chunk of the swizzled slot); 16 neighbouring tasks store 256 contiguous bytes.
-    if (alu_here) {
+    // entries (one 16-byte chunk of the swizzled slot).
+    if (tma_out) {
       pdl_wait();
       const int tid_a = (warp - ALU_WARP) * 32 + lane, tasks = prm.alu_rows * 16;
       const uint32_t ring = (uint32_t)prm.ring;
       uint32_t slot = 0, par = 0;
       for (ItemIter it(prm, first, step, nph); it.left; it.next()) {
-        const RadonPhase& ph = FEAT ? prm.ph[it.ph] : prm.ph[0];
-        const uint32_t head = it.slab / sph;
-        const int e0 = ph.dst_private ? 0 : (int)(it.slab - head * sph) * 128;
-        const int64_t hrow = (int64_t)(ph.dst_private ? blockIdx.x : head) * ph.out.rows_per_head;
         if (!mbar_wait_warp(full + slot, par, wc)) break;
-        if ((int)it.img >= ph.out.vert_from) {
+        if ((int)it.img >= prm.ph[0].out.vert_from) {
           const uint8_t* sl = sRing + slot * slot_bytes;
           for (int task = tid_a; task < tasks; task += 32 * ALU_WARPS) {
             const int u = prm.rows_mma + (task >> 4) - q * q, ch = task & 15;
@@ -552,34 +508,16 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
               acc[4] += __uint_as_float(w.z << 16); acc[5] += __uint_as_float(w.z & 0xffff0000u);
               acc[6] += __uint_as_float(w.w << 16); acc[7] += __uint_as_float(w.w & 0xffff0000u);
             }
-            if (tma_out) {   // into the slot's extra-class rows, from where the storing thread sends them with the tile
-              uint8_t* mrow = sMini + slot * prm.mini_bytes + (ch >> 3) * (prm.mini_bytes / 2) + u * 128;
-              *reinterpret_cast<uint4*>(mrow + (((ch & 7) ^ (u & 7)) << 4)) =
-                  make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]),
-                             pack_bf16(acc[6], acc[7]));
-            } else {
-              const int row = ph.out.v0 + (int)it.img * ph.out.sv_img + u * ph.out.sv_lo;
-              __nv_bfloat16* dst = ph.dst + (hrow + row) * ph.dst_pitch + e0 + ch * 8;
-              st_global_v4_hint(dst, pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]),
-                                pack_bf16(acc[6], acc[7]), it.ph ? pol_dst1 : pol_dst0);
-            }
+            // into the slot's extra-class rows, from where the storing thread sends them with the tile
+            uint8_t* mrow = sMini + slot * prm.mini_bytes + (ch >> 3) * (prm.mini_bytes / 2) + u * 128;
+            *reinterpret_cast<uint4*>(mrow + (((ch & 7) ^ (u & 7)) << 4)) =
+                make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]),
+                           pack_bf16(acc[6], acc[7]));
           }
         }
-        if (tma_out) {
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(alu_done + slot);
-          if (++slot == ring) { slot = 0; par ^= 1; }
-          continue;
-        }
+        fence_proxy_async();
         __syncwarp();
-        if (lane == 0) mbar_arrive(empty + slot);
-        if (it.closes_phase0()) {   // what this warp stored for the slab is ordered before the copy engine's reads
-          __threadfence();
-          fence_proxy_async_all();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(w_ready);
-        }
+        if (lane == 0) mbar_arrive(alu_done + slot);
         if (++slot == ring) { slot = 0; par ^= 1; }
       }
     }
@@ -592,9 +530,9 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
     const uint32_t lane_base = (uint32_t)(qd * 32) << 16;
     const int tv0 = out_tab[orow], tv1 = nph > 1 ? out_tab[TILE_ROWS + orow] : ROW_INVALID;
     const bool active = qd * 32 < prm.rows_mma;                 // warp-uniform: some output index in these lanes
-    uint32_t buf = 0, apar = 0, eslot = 0, epar = 0, sidx = 0;
+    uint32_t buf = 0, apar = 0, eslot = 0, epar = 0;
     // tma_out: where this thread's 64 bytes go inside the slot (or inside the slot's extra rows)
-    const bool st_mini = prm.mini_bytes != 0 && orow >= q * q;
+    const bool st_mini = orow >= q * q;
     const int st_idx = st_mini ? orow - q * q : orow;
     const int st_off = (cb >> 1) * (st_mini ? prm.mini_bytes / 2 : prm.sr * 128) + st_idx * 128;
     for (ItemIter it(prm, first, step, nph); it.left; it.next()) {
@@ -616,18 +554,8 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
         fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(acc_empty + buf);             // the accumulator is in registers
-        if (alu_here && !mbar_wait_warp(alu_done + eslot, epar, wc)) break;   // the ALU warps have read the image
-        if (prm.nslots > 1) {                                     // the item's other slots are free already
-          if (warp == 0 && lane == 0)
-            for (int g = 1; g < prm.nslots; ++g) {
-              uint32_t sl = eslot + g; if (sl >= (uint32_t)prm.ring) sl -= (uint32_t)prm.ring;
-              mbar_arrive(empty + sl);
-            }
-          __syncwarp();
-        }
+        if (!mbar_wait_warp(alu_done + eslot, epar, wc)) break;   // the ALU warps have read the image
         if (tv != ROW_INVALID) {
-          // regular indices and, without extra rows of their own, the extra-class indices: tile row =
-          // TMEM lane; with extra rows per slot (q = 11) the extra-class indices go there
           const int idx = st_idx;
           uint8_t* trow = (st_mini ? sMini + eslot * prm.mini_bytes : sRing + eslot * slot_bytes) + st_off;
 #pragma unroll
@@ -640,10 +568,8 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
         }
         fence_proxy_async();
         __syncwarp();
-        if (lane == 0) mbar_arrive(staged + sidx);   // one barrier per item in flight: at most `ring` of them
-        if (++sidx == (uint32_t)prm.ring) sidx = 0;
-        eslot += (uint32_t)prm.nslots;
-        if (eslot >= (uint32_t)prm.ring) { eslot -= (uint32_t)prm.ring; epar ^= 1; }
+        if (lane == 0) mbar_arrive(staged + eslot);
+        if (++eslot == (uint32_t)prm.ring) { eslot = 0; epar ^= 1; }
         if (++buf == nacc) { buf = 0; apar ^= 1; }
         continue;
       }
@@ -679,7 +605,7 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
       fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(acc_empty + buf);
-      if (it.closes_phase0()) {   // as for the ALU warps: the slab's phase 0 rows before the copy engine reads them
+      if (it.closes_phase0()) {   // the slab's phase 0 rows before the copy engine reads them
         __threadfence();
         fence_proxy_async_all();
         __syncwarp();
@@ -697,12 +623,12 @@ __global__ void __launch_bounds__(RADON_THREADS, 1) radon_tc_kernel(const __grid
 }
 
 struct RadonShape {
-  int sps, sr, nreg, nslots, rows_mma, alu_rows, ring, smem;
+  int sps, sr, nreg, nslots, rows_mma, alu_rows, ring, mini_bytes, smem;
 };
 
-// Ring slots of `sps` lines (sps*q rows, rounded up to 16), chosen for the least MMA work.  R (128 lanes x one column per two operand rows) and at least
-// two accumulators of 128 columns must fit the 512 columns of tensor memory, and the ring must be able to hold the
-// scratch copy of R while it is built.  Returns false when q is too large for this kernel.
+// Ring slots of `sps` lines (sps*q rows, rounded up to 16), chosen for the least MMA work.  R (128 lanes x one column per two
+// operand rows) and at least two accumulators of 128 columns must fit the 512 columns of tensor memory, and the ring must be
+// able to hold the scratch copy of R while it is built.  Returns false when q is too large for this kernel.
 bool radon_shape(int q, int transpose, int in_has_extra, int count_out, RadonShape* s) {
   const int budget = 227 * 1024 - 1024 - 512 - TILE_ROWS * 8;
   if (q < 2 || q > 64) return false;
@@ -726,12 +652,20 @@ bool radon_shape(int q, int transpose, int in_has_extra, int count_out, RadonSha
     if (cost < best) {
       best = cost;
       s->sps = sps; s->sr = sr; s->nreg = nreg; s->nslots = nslots;
-      s->rows_mma = count_out - left; s->alu_rows = left; s->ring = ring;
+      s->rows_mma = count_out - left; s->alu_rows = left; s->ring = ring; s->mini_bytes = 0;
       s->smem = ring * slot_bytes + TILE_ROWS * 8 + 512 + 1024;
     }
   }
   if (best == (1 << 30)) return false;
-  return left == 0 || (s->nslots == 1 && s->sps >= q);
+  if (left == 0) return true;
+  // The tile is stored by TMA from the item's own slot, which is as large; every slot gets room for the q extra-class rows of
+  // its tile (two 64-entry halves).
+  if (s->nslots != 1 || s->sps < q || s->sr != TILE_ROWS) return false;
+  s->mini_bytes = 2 * ((q + 7) & ~7) * 128;
+  const int slot_bytes = s->sr * 256 + s->mini_bytes, ring = budget / slot_bytes;
+  if (ring < s->ring) s->ring = ring;
+  s->smem = s->ring * slot_bytes + TILE_ROWS * 8 + 512 + 1024;
+  return s->ring >= 4;
 }
 
 // The shared-memory map of radon_tc_kernel for a shape, checked on the host before every launch: ring slots, the
@@ -741,19 +675,17 @@ bool radon_shape(int q, int transpose, int in_has_extra, int count_out, RadonSha
 //   [.., + ring * mini)                   extra-class rows per slot (two halves of mini / 2)
 //   [.., + 2 * 128 * 4)                   output-row table
 //   [.., + (4 ring + 2 MAX_ACC + 1) * 8 + 8)   barriers, the tensor-memory slot word, the abort flag
-bool radon_layout_ok(int q, const RadonShape& sh, int ring, int mini_bytes, int tma_out, int in_has_extra, int smem) {
+bool radon_layout_ok(int q, const RadonShape& sh, int in_has_extra) {
   const int slot = sh.sr * 256, half = sh.sr * 128;
-  const int bars = (4 * ring + 2 * MAX_ACC + 1) * 8 + 8;
-  bool ok = sh.sr % 16 == 0 && sh.sr <= TILE_ROWS && ring >= sh.nslots;           // the scratch copy of R: 128 rows x kt bf16
+  const int bars = (4 * sh.ring + 2 * MAX_ACC + 1) * 8 + 8;
+  bool ok = sh.sr % 16 == 0 && sh.sr <= TILE_ROWS && sh.ring >= sh.nslots;        // the scratch copy of R: 128 rows x kt bf16
   ok = ok && sh.nslots == sh.nreg + (in_has_extra ? 1 : 0) && sh.nreg * sh.sps >= q;
   ok = ok && q * sh.sps * 128 <= half && q * 128 <= half;                         // a load box (lines or extra class) per half
   ok = ok && ((sh.nslots * sh.sr / 2 + 31) & ~31) + 2 * 128 <= 512;               // R columns and two accumulators
   ok = ok && sh.rows_mma <= TILE_ROWS;
-  if (tma_out) {   // the tile is written into the item's first slot: one 128-byte row per output index
-    ok = ok && sh.rows_mma <= sh.sr;
-    ok = ok && (mini_bytes == 0 || (mini_bytes % 2048 == 0 && mini_bytes / 2 >= q * 128));
-  }
-  ok = ok && 1023 + ring * (slot + mini_bytes) + 2 * TILE_ROWS * 4 + bars <= smem && smem <= 227 * 1024;
+  if (sh.alu_rows)   // the tile is written into the item's slot: one 128-byte row per regular output index, the others behind
+    ok = ok && sh.nslots == 1 && q * q <= sh.sr && sh.rows_mma >= q * q && sh.mini_bytes % 2048 == 0 && sh.mini_bytes / 2 >= q * 128;
+  ok = ok && 1023 + sh.ring * (slot + sh.mini_bytes) + 2 * TILE_ROWS * 4 + bars <= sh.smem && sh.smem <= 227 * 1024;
   return ok;
 }
 
@@ -768,28 +700,15 @@ cudaError_t launch_radon(int q, int transpose, int nph, const StageSpec* sp, int
   if (!radon_shape(q, transpose, in_has_extra, sp[0].out.count, &sh) || rp % 128 ||
       (int64_t)bh * (rp / 128) * max_images * 2 >= (1LL << 31))
     return cudaErrorInvalidValue;
-  if (nph == 2 && (sp[1].in.count != sp[0].in.count || sp[1].out.count != sp[0].out.count))
+  if (nph == 2 && (sp[1].in.count != sp[0].in.count || sp[1].out.count != sp[0].out.count || sh.alu_rows > 0))
     return cudaErrorInvalidValue;
   RadonParams prm;
   prm.q = q; prm.transpose = transpose; prm.sps = sh.sps; prm.sr = sh.sr; prm.nreg = sh.nreg; prm.nslots = sh.nslots;
   prm.rows_mma = sh.rows_mma; prm.alu_rows = sh.alu_rows;
   prm.ring = sh.ring; prm.nph = nph; prm.slabs_per_head = (int)(rp / 128); prm.slabs = (int64_t)bh * (rp / 128);
   prm.status = status;
-  // One slot per item, as large as an output tile, one CTA per image (q = 11, forward): the tile is stored by TMA
-  // from the item's own slot; every slot gets room for the q extra-class rows of its tile (two 64-entry halves).
-  int smem = sh.smem;
-  prm.tma_out = 0; prm.mini_bytes = 0;
-  prm.lines_out = sh.rows_mma / q < q ? sh.rows_mma / q : q;
-  if (!transpose && sh.nslots == 1 && sh.sr == TILE_ROWS) {
-    const int mini = 2 * ((q + 7) & ~7) * 128, slot = sh.sr * 256;
-    int ring = (227 * 1024 - 1024 - 512 - TILE_ROWS * 8) / (slot + mini);
-    if (ring > sh.ring) ring = sh.ring;
-    if (ring >= 4) {
-      prm.tma_out = 1; prm.mini_bytes = mini; prm.ring = ring;
-      smem = ring * (slot + mini) + TILE_ROWS * 8 + 512 + 1024;
-    }
-  }
-  if (!radon_layout_ok(q, sh, prm.ring, prm.mini_bytes, prm.tma_out, in_has_extra, smem)) return cudaErrorInvalidConfiguration;
+  prm.mini_bytes = sh.mini_bytes;
+  if (!radon_layout_ok(q, sh, in_has_extra)) return cudaErrorInvalidConfiguration;
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -797,7 +716,7 @@ cudaError_t launch_radon(int q, int transpose, int nph, const StageSpec* sp, int
   int64_t ctas = sms;
   const int64_t items = nph == 1 ? prm.slabs * sp[0].images : prm.slabs;
   if (items < ctas) ctas = items;
-  CUtensorMap tm_reg[2], tm_vert[2], tm_oreg[2], tm_overt[2];
+  CUtensorMap tm_reg[2], tm_vert[2];
   for (int i = 0; i < nph; ++i) {
     RadonPhase& ph = prm.ph[i];
     const RadonSide& in = sp[i].in;
@@ -826,36 +745,31 @@ cudaError_t launch_radon(int q, int transpose, int nph, const StageSpec* sp, int
     } else {
       tm_vert[i] = tm_reg[i];
     }
-    tm_oreg[i] = tm_reg[i]; tm_overt[i] = tm_reg[i];
-    if (prm.tma_out) {   // the same two shapes over the output rows: boxes of q lines, and of the extra class
-      const RadonSide& out = sp[i].out;
-      const int64_t dst_rp = sp[i].dst_private ? 128 : rp, dst_heads = sp[i].dst_private ? ctas : bh;
-      const int64_t sizes[4] = {q, q, images, dst_heads};
-      const int64_t strides[4] = {out.s_lo, out.s_hi, images > 1 ? out.s_img : out.rows_per_head, out.rows_per_head};
-      const int box[4] = {q, prm.lines_out, 1, 1};
-      if (!radon_map(&tm_oreg[i], sp[i].dst, dst_rp, 5, sizes, strides, box)) return cudaErrorInvalidValue;
-      if (out.count > q * q) {
-        const bool per_image = out.sv_img != 0;
-        const int64_t vsizes[3] = {q, per_image ? images : 1, dst_heads};
-        const int64_t vstrides[3] = {out.sv_lo, per_image ? out.sv_img : out.rows_per_head, out.rows_per_head};
-        const int vbox[3] = {q, 1, 1};
-        if (!radon_map(&tm_overt[i], static_cast<__nv_bfloat16*>(sp[i].dst) + (int64_t)out.v0 * dst_rp, dst_rp, 4, vsizes,
-                       vstrides, vbox))
-          return cudaErrorInvalidValue;
-      }
-    }
+  }
+  CUtensorMap tm_oreg = tm_reg[0], tm_overt = tm_reg[0];
+  if (prm.alu_rows > 0) {   // the same two shapes over the output rows: boxes of q lines, and of the extra class
+    const RadonSide& out = sp[0].out;
+    const int images = sp[0].images;
+    const bool per_image = out.sv_img != 0;
+    const int64_t sizes[4] = {q, q, images, bh}, vsizes[3] = {q, per_image ? images : 1, bh};
+    const int64_t strides[4] = {out.s_lo, out.s_hi, images > 1 ? out.s_img : out.rows_per_head, out.rows_per_head};
+    const int64_t vstrides[3] = {out.sv_lo, per_image ? out.sv_img : out.rows_per_head, out.rows_per_head};
+    const int box[4] = {q, q, 1, 1}, vbox[3] = {q, 1, 1};
+    if (!radon_map(&tm_oreg, sp[0].dst, rp, 5, sizes, strides, box) ||
+        !radon_map(&tm_overt, static_cast<__nv_bfloat16*>(sp[0].dst) + (int64_t)out.v0 * rp, rp, 4, vsizes, vstrides, vbox))
+      return cudaErrorInvalidValue;
   }
   if (nph == 1) {
-    prm.ph[1] = prm.ph[0]; tm_reg[1] = tm_reg[0]; tm_vert[1] = tm_vert[0]; tm_oreg[1] = tm_oreg[0]; tm_overt[1] = tm_overt[0];
+    prm.ph[1] = prm.ph[0]; tm_reg[1] = tm_reg[0]; tm_vert[1] = tm_vert[0];
   }
   const bool feat = nph > 1 || prm.alu_rows > 0;
   // the plain instantiation has no use for the two ALU warps
-  const unsigned threads = feat ? RADON_THREADS : 32 * (ALU_WARP + (prm.tma_out ? 1 : 0));
+  const unsigned threads = feat ? RADON_THREADS : 32 * ALU_WARP;
   auto kernel = feat ? radon_tc_kernel<true> : radon_tc_kernel<false>;
-  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sh.smem);
   if (err != cudaSuccess) return err;
-  return smat_launch_pdl(kernel, dim3((unsigned)ctas), threads, smem, st, tm_reg[0], tm_vert[0], tm_reg[1], tm_vert[1],
-                         tm_oreg[0], tm_overt[0], tm_oreg[1], tm_overt[1], prm);
+  return smat_launch_pdl(kernel, dim3((unsigned)ctas), threads, sh.smem, st, tm_reg[0], tm_vert[0], tm_reg[1], tm_vert[1], tm_oreg,
+                         tm_overt, prm);
 }
 
 // The two stages of d = 4 run as one launch when a CTA's exchange rows (q^3 + q^2 rows of 128 entries), times the
@@ -938,7 +852,7 @@ int64_t smat_tabulate_tc_scratch_elems(const SmatGeo& geo, int64_t state_elems, 
 }
 
 // Host-only: 1 when every stage of a tabulation of prime q has a kernel whose shared-memory map holds: the resident matrix
-// (with the tile-store variant where the launcher would pick it), the generated one, or, for d = 3 alone, its forward
+// (with its tile stores at q = 11), the generated one, or, for d = 3 alone, its forward
 // stage.  (The both-stages kernel of smat_radon_slab.cu has one map, asserted where it is compiled.)
 int smat_tabulate_tc_layout_ok(int q) {
   StageSpec sp[2];
@@ -958,14 +872,7 @@ int smat_tabulate_tc_layout_ok(int q) {
         const int extra = sp[i].in.count > q * q;
         RadonShape sh;
         if (!radon_shape(q, transpose, extra, sp[i].out.count, &sh)) return 0;
-        if (!radon_layout_ok(q, sh, sh.ring, 0, 0, extra, sh.smem)) return 0;
-        if (!transpose && sh.nslots == 1 && sh.sr == TILE_ROWS) {
-          const int mini = 2 * ((q + 7) & ~7) * 128, slot = sh.sr * 256;
-          int ring = (227 * 1024 - 1024 - 512 - TILE_ROWS * 8) / (slot + mini);
-          if (ring > sh.ring) ring = sh.ring;
-          if (ring >= 4 && !radon_layout_ok(q, sh, ring, mini, 1, extra, ring * (slot + mini) + TILE_ROWS * 8 + 512 + 1024))
-            return 0;
-        }
+        if (!radon_layout_ok(q, sh, extra)) return 0;
       }
     }
   return 1;
