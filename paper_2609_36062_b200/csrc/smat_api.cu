@@ -150,11 +150,16 @@ struct Ctx {
 // The 256 bytes at off_status: the status word, and at these offsets the numbers of heavy parts of a routed pass.
 constexpr size_t PROF_HEAVY_COUNT = 128, TYPE_HEAVY_COUNT = 192;
 
+// Parts of heavy groups that a head may have; none where no kernel asks for them.
+int64_t heavy_parts(const smat_plan* pl, bool prof) {
+  const int64_t tokens = prof ? pl->geo.n : pl->geo.m, groups = prof ? pl->geo.P : pl->geo.B;
+  return pl->tc && !pl->geo.dense_G && tokens < SMAT_LISTED_SMALL * groups ? tokens / SMAT_HEAVY_TOKENS : 0;
+}
 SmatRouteLists route_lists(const Ctx& cx, bool prof) {
   const smat_plan* pl = cx.pl;
   auto i32 = [&](size_t off) { return reinterpret_cast<int32_t*>(cx.ws + off); };
   return SmatRouteLists{i32(prof ? pl->off_plist : pl->off_tlist), i32(prof ? pl->off_poffs : pl->off_toffs),
-                        reinterpret_cast<SmatHeavyPart*>(cx.ws + (prof ? pl->off_pheavy : pl->off_theavy)),
+                        heavy_parts(pl, prof) ? reinterpret_cast<SmatHeavyPart*>(cx.ws + (prof ? pl->off_pheavy : pl->off_theavy)) : nullptr,
                         i32(pl->off_status + (prof ? PROF_HEAVY_COUNT : TYPE_HEAVY_COUNT))};
 }
 
@@ -517,8 +522,8 @@ smat_status smat_plan_create(smat_plan** out, int batch, int heads, int64_t T, i
   pl->off_poffs = off;  off = align_up(off + (lists ? (size_t)pl->bh * (g.P + 1) * 4 : 0));
   pl->off_tlist = off;  off = align_up(off + (lists ? (size_t)pl->bh * g.m * 4 : 0));
   pl->off_toffs = off;  off = align_up(off + (lists ? (size_t)pl->bh * (g.B + 1) * 4 : 0));
-  pl->off_pheavy = off; off = align_up(off + (lists ? (size_t)pl->bh * (g.n / SMAT_HEAVY_TOKENS) * sizeof(SmatHeavyPart) : 0));
-  pl->off_theavy = off; off = align_up(off + (lists ? (size_t)pl->bh * (g.m / SMAT_HEAVY_TOKENS) * sizeof(SmatHeavyPart) : 0));
+  pl->off_pheavy = off; off = align_up(off + (size_t)pl->bh * heavy_parts(pl, true) * sizeof(SmatHeavyPart));
+  pl->off_theavy = off; off = align_up(off + (size_t)pl->bh * heavy_parts(pl, false) * sizeof(SmatHeavyPart));
   // gated variant: λ and the rescaled copies of Q, K (forward) and dO, V (backward), in the plan's dtype
   const size_t esz = dtype == SMAT_BF16 ? 2 : 4;
   const size_t gated = (flags & SMAT_FLAG_GATED) ? 1 : 0;

@@ -14,11 +14,10 @@
 enum SmatGroupMode { SMAT_GM_NONE = 0, SMAT_GM_CHUNK = 1, SMAT_GM_PROFILE = 2, SMAT_GM_TYPE = 3 };
 
 // A listed group may hold any number of tokens: what it has behind its first SMAT_HEAVY_TOKENS is cut into parts of at most
-// as many, for kernels that hand these out to several CTAs.
-constexpr int SMAT_HEAVY_TOKENS = 128;
+// as many, for kernels that hand these out to several CTAs (where groups hold fewer than SMAT_LISTED_SMALL on average).
+constexpr int SMAT_HEAVY_TOKENS = 128, SMAT_LISTED_SMALL = 16;
 struct SmatHeavyPart {
-  uint16_t bh, group;   // (a plan has at most 65535 heads, a routed call 27000 groups)
-  int32_t first;        // tokens of the group in front of the part
+  uint16_t bh, group, number;   // (at most 65535 heads, 27000 groups of a routed call, 65535 * 128 tokens); the first part is 1
 };
 struct SmatGroupSpec {
   int mode;
@@ -30,7 +29,7 @@ struct SmatGroupSpec {
   const int32_t* list;
   const int32_t* offs;
   int64_t list_stride, offs_stride;
-  const SmatHeavyPart* heavy;   // the parts of all heads, *heavy_count of them in any order (null: positional groups)
+  const SmatHeavyPart* heavy;   // the parts of all heads, *heavy_count of them in any order (null: not made)
   const int32_t* heavy_count;
 };
 
@@ -259,7 +258,7 @@ cudaError_t smat_launch_normalize_step(int step, const void* a, const void* b, v
                                        cudaStream_t st);
 // Token lists of user-supplied routing: prof [bh][n] (cells in [0, P)) and type [bh][m] (types in [0, B)) -> CSR lists
 // (offsets [bh][G + 1], token positions [bh][count], ascending inside a group).  Keys out of range are dropped.  Parts of
-// heavy groups are appended at heavy (room for bh * (count / SMAT_HEAVY_TOKENS)) and added to *heavy_count, zero before.
+// heavy groups are appended at heavy (null, or room for bh * (count / SMAT_HEAVY_TOKENS)) and added to *heavy_count, zero before.
 struct SmatRouteLists {
   int32_t* list;
   int32_t* offs;

@@ -16,9 +16,9 @@ constexpr int ROUTE_THREADS = 256;
 // The tokens are cut into W contiguous ranges, one per warp (W as large as shared memory allows, at most 8):
 //   1. every warp histograms the keys of its range in its own row of counters (keys outside [0, G) are dropped:
 //      such a token belongs to no group)
-//   2. totals per group, exclusive scan -> offs[0 .. G]; row w then becomes the first slot of group g for warp w's
-//      tokens: offs[g] + the counts of the warps before it; a heavy group's parts are noted (their order depends on thread
-//      timing, but each is a set of rows that some CTA reads on their own)
+//   2. totals per group (a heavy group's parts are noted: their order depends on thread timing, but each is a set of rows that
+//      some CTA reads on its own), exclusive scan -> offs[0 .. G]; row w then becomes the first slot of group g for warp w's
+//      tokens: offs[g] + the counts of the warps before it
 //   3. stable placement: every warp walks ITS range in order, 32 tokens at a time; lanes with equal keys find each other
 //      with match.any, the lowest such lane advances the warp's cursor of the group, every lane writes its token's
 //      position.  Ranges are in token order and each warp's slots follow those of the warps before it, so the list of
@@ -59,6 +59,10 @@ __global__ void __launch_bounds__(ROUTE_THREADS) routing_lists_kernel(const __gr
     int32_t sum = 0;
     for (int w = 0; w < W; ++w) sum += rows[(1 + w) * pitch + g];
     total[g + 1] = sum;          // shifted by one: the inclusive scan below leaves the first slot of group g at index g
+    if (sum > SMAT_HEAVY_TOKENS && to.heavy) {
+      const int32_t parts = (sum - 1) / SMAT_HEAVY_TOKENS, at = atomicAdd(to.heavy_count, parts);   // behind the first
+      for (int32_t i = 0; i < parts; ++i) to.heavy[at + i] = SmatHeavyPart{(uint16_t)bh, (uint16_t)g, (uint16_t)(i + 1)};
+    }
   }
   __syncthreads();
   __shared__ int32_t warp_sum[ROUTE_THREADS / 32];
@@ -85,18 +89,11 @@ __global__ void __launch_bounds__(ROUTE_THREADS) routing_lists_kernel(const __gr
   // total[g] = tokens in groups < g (total[0] = 0): the offsets; then the per-warp first slots
   for (int64_t g = tid; g <= G; g += ROUTE_THREADS) offs[g] = total[g];
   for (int64_t g = tid; g < G; g += ROUTE_THREADS) {
-    const int32_t begin = total[g];
-    int32_t slot = begin;
+    int32_t slot = total[g];
     for (int w = 0; w < W; ++w) {
       const int32_t c = rows[(1 + w) * pitch + g];
       rows[(1 + w) * pitch + g] = slot;
       slot += c;
-    }
-    const int32_t parts = (slot - begin - 1) / SMAT_HEAVY_TOKENS;   // behind the first; none of an empty group
-    if (parts > 0) {
-      const int32_t at = atomicAdd(to.heavy_count, parts);
-      for (int32_t i = 0; i < parts; ++i)
-        to.heavy[at + i] = SmatHeavyPart{(uint16_t)bh, (uint16_t)g, (i + 1) * SMAT_HEAVY_TOKENS};
     }
   }
   __syncthreads();

@@ -1359,8 +1359,8 @@ struct ReadPass {
         bh = part.bh;
         state = bh * pp->groups + part.group;
         tk = smat_group_tokens(pp->grp, bh, part.group);
-        tk.lst += part.first;
-        cnt = tk.cnt - part.first;
+        tk.lst += part.number * SMAT_HEAVY_TOKENS;
+        cnt = tk.cnt - part.number * SMAT_HEAVY_TOKENS;
       }
       if (pp->grp.heavy && cnt > SMAT_HEAVY_TOKENS) cnt = SMAT_HEAVY_TOKENS;
       if (cnt > 0) break;
@@ -1907,7 +1907,7 @@ cudaError_t smat_launch_bwd_tiles_fused_tc(const void* Q, const void* K, const v
 // then handed out in parts of four tiles, where one CTA walking it 32 tokens at a time is slower than 128 at a time.  Routed
 // pass, d = 3, 16 heads of 16 K tokens, uniform / half of the tokens in one group / all of them: 442 / 1149 / 1830 us with
 // 128-row tiles, 439 / 1276 / 2095 with 32-row ones and whole groups, 434 / 905 / 1311 with parts.
-static bool read_groups_small(const SmatGroupSpec& grp) { return grp.list ? grp.base < 16 : grp.base < 32; }
+static bool read_groups_small(const SmatGroupSpec& grp) { return grp.list ? grp.base < SMAT_LISTED_SMALL : grp.base < 32; }
 // What a launch of the read walks, and its CTAs, `resident` of which share an SM.
 static int64_t read_items(ReadParams& prm, const SmatGroupSpec& grp, int64_t groups, int bh, int resident) {
   prm.grp = grp; prm.groups = groups; prm.states = (int64_t)bh * groups;
