@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(THREADS, 1) radon_sparse_kernel(const __grid_c
     // How fast the instructions follow one another, by unrolling.  A sparse one of 64 columns reads shared memory at its full
     // rate; in one burst per item they hold up the boxes that arrive.  64 heads of 8192 tokens, forward / transposed:
     // fully unrolled 0.234 / 0.230 ms, by two 0.204 / 0.230, not at all 0.232 (36 instructions of about 100 cycles are an
-    // item's time) / 0.206.
+    // item's time) / 0.206.  d = 4, 4 heads of 64 K tokens, both stages: 0.51 / 0.51, 0.47 / 0.51, 0.49 / 0.48.
     constexpr int PACE = TRANSPOSE ? 1 : 2;
     constexpr uint32_t id_dense = make_idesc(ROWS, NE, 0, 1);    // R from tensor memory, image rows MN-major
     constexpr uint32_t id_even = make_idesc_sparse(ROWS, NE, 0, 1, 0), id_odd = make_idesc_sparse(ROWS, NE, 0, 1, 1);

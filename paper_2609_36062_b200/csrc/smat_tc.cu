@@ -2042,7 +2042,7 @@ static SegCut segment_cut(int64_t rows0, int64_t rows1, int nseg0, int nseg1) {
 }
 
 // Up to two segments per block: the output CTA of the second reads the first one's total, and there is nothing to scan (the
-// pass, 32 heads of 4096 tokens, d = 3: 206 -> 199 us; 128 heads of 8192: the scan's 21 us).  With four segments the sums at
+// pass, 32 heads of 4096 tokens, d = 3: 201 -> 199 us; 128 heads of 8192: the scan's 21 us).  With four segments the sums at
 // the head of the output CTAs take longer than the scan (32 heads of 16 K tokens: output 141 -> 160 us, scan 10).
 bool smat_segments_need_scan(int nseg0, int nseg1) { return nseg0 > 2 || nseg1 > 2; }
 
