@@ -178,10 +178,12 @@ struct ReadList {
   int32_t scan_x, scan_y, scan_ctas;   // CTAs per head and (job, range); heads; all of them
 };
 
-// Two CTAs share an SM; each owns one 64 KB state buffer, so one CTA's contraction overlaps the other's bulk load.  (A state
-// in two halves, the first one fetched again while the second is contracted: nothing gained where a group is one pass, and a
-// barrier more to each where it is many.  8 heads of 2048 tokens, d = 2, fp32, half of them in one group, forward and
-// backward: 1980 us so, 2100 in halves.)
+// Two CTAs share an SM; each owns one 64 KB state buffer, so one CTA's contraction overlaps the other's bulk load.  A state
+// of 32 KB or more arrives in two halves of rows.  Where a group is one pass of five to eight tokens they are contracted one
+// after the other, and the next state's first half is fetched in between (d = 3, seven or eight tokens to a group, bf16 with
+// fp32 tables, heads of 2688 tokens: 24 of them 263 -> 258 us a pass, 8 of them 116.5 -> 112.6).  That costs a barrier, which
+// shorter passes do not earn back and groups of several passes would pay in each (8 heads of 2048, d = 2, fp32, half of the
+// tokens in one group, forward and backward: 2000 us so, 2100 with every pass in halves).
 template <int R, int PD, typename T>
 struct ReadLayout {
   static constexpr int KT = 8;                              // tokens per pass over a state
@@ -196,14 +198,15 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
                                                                    int* status) {
   using L = ReadLayout<R, PD, T>;
   constexpr int KT = L::KT, NJ4 = L::NJ4, NG = L::NG;
-  constexpr int RPG = R / NG;
+  constexpr int RPG = R / NG, RPH = RPG / 2;   // a thread's rows of a state, and of a half
+  constexpr bool HALVES = RPH >= 4;
   extern __shared__ __align__(128) uint8_t smem_raw[];
   float* Sb = reinterpret_cast<float*>(smem_raw);        // [R*PD]
   float* red = Sb + R * PD;                              // [RED]
   T* Xraw = reinterpret_cast<T*>(red + L::RED);          // [2][KT][XM] raw rows of the first KT tokens of an item
   float* Xs = reinterpret_cast<float*>(Xraw + 2 * KT * L::XM);  // [KT][XM]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(Xs + KT * L::XM);
-  volatile int* cta_abort = reinterpret_cast<volatile int*>(bar + 1);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(Xs + KT * L::XM);   // [2] a half of the state has landed
+  volatile int* cta_abort = reinterpret_cast<volatile int*>(bar + 2);
   pdl_trigger();
   const tc::WaitCtx wc{cta_abort, status};
   const int tid = threadIdx.x;
@@ -214,7 +217,7 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
     return;
   }
   const int j4 = tid % NJ4, ig = tid / NJ4;
-  constexpr uint32_t SBYTES = R * PD * 4;
+  constexpr uint32_t LBYTES = HALVES ? R * PD * 2 : R * PD * 4;   // a load: half a state, or all of it
   const int64_t items = list.first[list.a.jobs], cta = blockIdx.x - list.scan_ctas, ctas = gridDim.x - list.scan_ctas;
   auto job_of = [&](int64_t item) {
     int j = 0;
@@ -250,13 +253,18 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
   if (tid == 0) {
     *cta_abort = 0;
     tc::mbar_init(bar, 1);
+    tc::mbar_init(bar + 1, 1);
     tc::fence_barrier_init();
   }
-  uint32_t loads = 0;   // started states (thread 0)
+  uint32_t loads[2] = {0, 0};   // started ones (thread 0)
+  auto load_half = [&](int64_t item, int h) {
+    tc::mbar_expect_tx(bar + h, LBYTES);
+    bulk_load(Sb + h * (R * PD / 2), state_of(item) + h * (R * PD / 2), LBYTES, bar + h);
+    ++loads[h];
+  };
   auto load_state = [&](int64_t item) {
-    tc::mbar_expect_tx(bar, SBYTES);
-    bulk_load(Sb, state_of(item), SBYTES, bar);
-    ++loads;
+    load_half(item, 0);
+    if (HALVES) load_half(item, 1);
   };
   pdl_wait();
   if (tid == 0 && cta < items) load_state(cta);
@@ -273,6 +281,7 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
     const T* Xb = static_cast<const T*>(list.a.job[j].x) + bh * Tlen * xd;
     float* out = list.a.job[j].out + bh * Tlen * od;
     const float4* S4 = reinterpret_cast<const float4*>(Sb);
+    const bool split = HALVES && !trans && cnt > 4 && cnt <= KT;
     prefetch_x(nxt, buf ^ 1);
     cp_async_wait<1>();
     __syncthreads();
@@ -284,7 +293,8 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
         if (k < kn) v = k0 == 0 ? to_float(Xraw[(buf * KT + k) * L::XM + i]) : to_float(Xb[tk.at(k0 + k) * xd + i]);
         Xs[k * L::XM + i] = v;
       }
-      const bool ok = __syncthreads_and(k0 > 0 || tc::mbar_wait(bar, n & 1, wc)) != 0;   // (block-wide barriers follow: all go on, or none)
+      // (block-wide barriers follow: all go on, or none)
+      const bool ok = __syncthreads_and(k0 > 0 || (tc::mbar_wait(bar, n & 1, wc) && (split || !HALVES || tc::mbar_wait(bar + 1, n & 1, wc)))) != 0;
       if (!ok || cnt == 0) break;
       if (!trans) {
         // KK: tokens of the pass, rounded up: nine tokens are a pass of eight and one of two (32 heads of 5056 tokens, d = 3,
@@ -295,24 +305,36 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
 #pragma unroll
           for (int k = 0; k < KK; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
           // four rows at a time, so that a token's factors are one load (32 heads, 307 states, bf16: 0.185 -> 0.177 ms)
+          auto rows = [&](int first, int count) {
 #pragma unroll 2
-          for (int s = 0; s < RPG; s += 4) {
-            const int i = ig * RPG + s;
-            const float4 u0 = S4[i * NJ4 + j4], u1 = S4[(i + 1) * NJ4 + j4], u2 = S4[(i + 2) * NJ4 + j4], u3 = S4[(i + 3) * NJ4 + j4];
+            for (int s = 0; s < count; s += 4) {
+              const int i = first + s;
+              const float4 u0 = S4[i * NJ4 + j4], u1 = S4[(i + 1) * NJ4 + j4], u2 = S4[(i + 2) * NJ4 + j4], u3 = S4[(i + 3) * NJ4 + j4];
 #pragma unroll
-            for (int k = 0; k < KK; ++k) {
-              const float4 x = *reinterpret_cast<const float4*>(Xs + k * L::XM + i);
-              acc[k] = fma4(x.x, u0, acc[k]); acc[k] = fma4(x.y, u1, acc[k]);
-              acc[k] = fma4(x.z, u2, acc[k]); acc[k] = fma4(x.w, u3, acc[k]);
+              for (int k = 0; k < KK; ++k) {
+                const float4 x = *reinterpret_cast<const float4*>(Xs + k * L::XM + i);
+                acc[k] = fma4(x.x, u0, acc[k]); acc[k] = fma4(x.y, u1, acc[k]);
+                acc[k] = fma4(x.z, u2, acc[k]); acc[k] = fma4(x.w, u3, acc[k]);
+              }
             }
+          };
+          if (HALVES && KK == KT && split) {
+            rows(ig * RPH, RPH);
+            if (!__syncthreads_and(tc::mbar_wait(bar + 1, n & 1, wc))) return false;
+            if (tid == 0 && nxt < items) load_half(nxt, 0);   // every thread is past its reads of the first half
+            rows(R / 2 + ig * RPH, RPH);
+          } else {
+            rows(ig * RPG, RPG);
           }
 #pragma unroll
           for (int k = 0; k < KK; ++k) *reinterpret_cast<float4*>(red + (ig * KT + k) * PD + j4 * 4) = acc[k];
+          return true;
         };
-        if (kn > 4) contract(std::integral_constant<int, 8>{});
-        else if (kn > 2) contract(std::integral_constant<int, 4>{});
-        else contract(std::integral_constant<int, 2>{});
+        const bool done = kn > 4 ? contract(std::integral_constant<int, 8>{})
+                                 : (kn > 2 ? contract(std::integral_constant<int, 4>{}) : contract(std::integral_constant<int, 2>{}));
+        if (!done) break;
         __syncthreads();
+        if (split && tid == 0 && nxt < items) load_half(nxt, 1);
         for (int idx = tid; idx < kn * NJ4; idx += 256) {   // the row groups' partial rows meet in shared memory
           const int k = idx / NJ4, c = idx - k * NJ4;
           float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -351,9 +373,12 @@ __global__ void __launch_bounds__(256, 2) state_read_stream_kernel(const __grid_
       __syncthreads();
     }
     // every thread is past its reads of the state buffer: fetch the next item's state
-    if (tid == 0 && nxt < items && !*cta_abort) load_state(nxt);
+    if (!split && tid == 0 && nxt < items && !*cta_abort) load_state(nxt);
   }
-  if (tid == 0) tc::landed(bar, (loads + 1) & 1, wc);
+  if (tid == 0) {   // (a barrier that never saw a load lets parity 1 pass)
+    tc::landed(bar, (loads[0] + 1) & 1, wc);
+    tc::landed(bar + 1, (loads[1] + 1) & 1, wc);
+  }
   cp_async_wait<0>();
 }
 
