@@ -408,6 +408,14 @@ void tabulate_tc(Ctx& cx, const char* name, const void* in, void* out, int trans
   cx.launches += launches - 1;
 }
 
+// Whether the tensor-core forward's long-range rows travel in fp32: in the per-tile form, where the type table is fp32, and where
+// blocks are odd numbers of tiles.
+bool forward_rows_f32(const smat_plan* pl) {
+  const bool lr = !pl->geo.dense_G;
+  return (pl->flags & SMAT_FLAG_PER_TILE_STATES) || (lr && !pl->u_bf16) ||
+         smat_segment_tiles(lr ? pl->geo.n / 128 : pl->T / 128, lr ? pl->geo.m / 128 : 0, pl->bh) < 2;
+}
+
 // Steps 2-3 of Algorithm 1 alone, as the plan's forward runs them: the type table U ends in the workspace at the
 // returned offset (d = 1: the single state U_0 = F_0, fp32).
 size_t build_type_table(Ctx& cx, const void* K, const void* V) {
@@ -671,26 +679,29 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     float* ylr = cx.f(pl->off_acc);
     const bool lr = !pl->geo.dense_G;
     if (lr) build_type_table(cx, K, V);                                                      // steps 2-3
-    // The two-level causal branch takes the long-range rows as bf16 (half the bytes for the typed read to write and
-    // for the output kernel to fetch); plans whose type table is fp32 use the per-tile form.
+    // The causal branch is the two-level one wherever the plan does not ask for per-tile states: blocks of any number of tiles
+    // are cut into segments that differ by a tile at most (odd numbers took the per-tile form: d = 2, 16 heads of 13,056 tokens
+    // 155 -> 146 us, of 23,296 259 -> 239; d = 4, 8 heads of 22,912 423 -> 376; d = 1, 16 heads of 3200 36 -> 30).  It takes the
+    // long-range rows as bf16 (half the bytes to write and to fetch) where blocks are even numbers of tiles, else in fp32.
     const int64_t tiles0 = lr ? pl->geo.n / 128 : pl->T / 128, tiles1 = lr ? pl->geo.m / 128 : 0;
-    const int L = ((pl->flags & SMAT_FLAG_PER_TILE_STATES) || (lr && !pl->u_bf16)) ? 1 : smat_segment_tiles(tiles0, tiles1, pl->bh);
+    const bool per_tile = (pl->flags & SMAT_FLAG_PER_TILE_STATES) != 0, f32 = forward_rows_f32(pl);
     if (lr) {                                                                                // step 4
-      zero_unrouted(cx, SMAT_GM_TYPE, ylr, L >= 2 && pl->u_bf16 ? 256 : 512);
+      zero_unrouted(cx, SMAT_GM_TYPE, ylr, f32 ? 512 : 256);
       if (pl->u_bf16)
-        SMAT_TRY(cx, "read_type_tc", smat_launch_state_read_tc(Q, cx.ws + pl->off_U, ylr, L >= 2 ? ylr : nullptr, 0,
+        SMAT_TRY(cx, "read_type_tc", smat_launch_state_read_tc(Q, cx.ws + pl->off_U, ylr, f32 ? nullptr : ylr, 0,
                                                                group(cx, SMAT_GM_TYPE), pl->geo.B, pl->T, pl->bh, status,
                                                                cx.st));
       else
         state_read(cx, "read_type", {read_job(cx, SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, ylr)});
     }
-    pl->tile_states = L < 2;
+    pl->tile_states = per_tile;
     pl->kept_tile_states = false;
-    if (L >= 2) {  // steps 5-7, two-level: segment totals, scan of the totals, fused per-segment output
+    if (!per_tile) {  // steps 5-7, two-level: segment totals, scan of the totals, fused per-segment output
       const int64_t rows0 = tiles0 * 128, rows1 = tiles1 * 128;
-      const Segments sg = segment_totals(cx, K, V, rows0, rows1, L);
+      const int L = smat_segment_tiles(tiles0, tiles1, pl->bh);
+      const Segments sg = segment_totals(cx, K, V, rows0, rows1, L < 2 ? 2 : L);
       const bool keep = (pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES) != 0;   // a backward will want the per-tile states
-      SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, cx.f(pl->off_sin), ylr, 0, lr ? pl->geo.n : pl->T, O,
+      SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, cx.f(pl->off_sin), ylr, f32, 0, lr ? pl->geo.n : pl->T, O,
                                                                        rows0, rows1, sg.nseg0, sg.nseg1, pl->bh, status, cx.st,
                                                                        keep ? cx.ws + pl->off_sin_tiles : nullptr));
       pl->kept_tile_states = keep;
@@ -718,7 +729,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
       state_read(cx, "read_type", {read_job(cx, SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, ylr)});
     }
     const Segments sg = segment_totals(cx, K, V, rows0, rows1, 2);
-    SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, cx.f(pl->off_sin), ylr, 1, lr ? pl->geo.n : pl->T, O, rows0,
+    SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, cx.f(pl->off_sin), ylr, 1, 1, lr ? pl->geo.n : pl->T, O, rows0,
                                                                      rows1, sg.nseg0, sg.nseg1, pl->bh, status, cx.st));
     pl->launches = cx.launches;
     return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;

@@ -280,9 +280,9 @@ void smat_segment_counts(int64_t tiles0, int64_t tiles1, int bh, int L, int* nse
 bool smat_segments_need_scan(int nseg0, int nseg1);
 cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* totals, int64_t rows0, int64_t rows1,
                                          int nseg0, int nseg1, int bh, int* status, cudaStream_t st);
-// ylr_f32 = 0: long-range rows in bf16, blocks of whole tiles.  ylr_f32 = 1: fp32 rows, any blocks, and the state and
-// the scores enter their products as a bf16 part plus a bf16 remainder.
+// ylr_f32: the long-range rows are fp32 (else bf16).  split: any blocks (else of whole tiles), and the state and the scores enter
+// their products as a bf16 part plus a bf16 remainder (with fp32 rows only).
 cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const void* V, const float* seg_in,
-                                          const void* ylr, int ylr_f32, int64_t n_lr, void* O, int64_t rows0, int64_t rows1,
+                                          const void* ylr, int ylr_f32, int split, int64_t n_lr, void* O, int64_t rows0, int64_t rows1,
                                           int nseg0, int nseg1, int bh, int* status, cudaStream_t st,
                                           void* sin_tiles = nullptr);

@@ -952,8 +952,8 @@ struct SegOutParams {
   const float* seg_in;   // [bh][nseg][128][128]: the state entering each segment, or (totals) the segments' totals
   int totals;            // a block has two segments at most: its second is entered with the first one's total
   int64_t n_lr;
-  const __nv_bfloat16* ylr;   // plain: [bh][T][128] long-range rows, bf16 (rows t >= n_lr are added)
-  const float* ylr32;         // SPLIT: the same rows in fp32
+  const __nv_bfloat16* ylr;   // [bh][T][128] long-range rows, bf16 (rows t >= n_lr are added)
+  const float* ylr32;         // Y32: the same rows in fp32
   __nv_bfloat16* O;
   __nv_bfloat16* sin_tiles;   // plain, optional [bh][T/128][128][128]: the bf16 state entering every tile, for a later backward
   int* status;
@@ -982,7 +982,7 @@ struct SegOutMaps {
   CUtensorMap q[2], k[2], v[2];
 };
 
-template <bool SPLIT>
+template <bool SPLIT, bool Y32>
 __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(const __grid_constant__ SegOutMaps maps,
                                                                             const SegOutParams prm) {
   using Lay = SegOutLayout<SPLIT>;
@@ -1244,12 +1244,12 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
       const int64_t t = row_first + (int64_t)it * TILE + m;
       const bool live = !SPLIT || t < row_end;
       const bool add_lr = live && t >= prm.n_lr;
-      uint4 y[SPLIT ? 8 : 4];                        // 32 bf16 or fp32 values
+      uint4 y[Y32 ? 8 : 4];                        // 32 bf16 or fp32 values
       if (add_lr) {
-        const uint4* y4 = SPLIT ? reinterpret_cast<const uint4*>(prm.ylr32 + ((int64_t)bh * prm.T + t) * TILE + col0)
-                                : reinterpret_cast<const uint4*>(prm.ylr + ((int64_t)bh * prm.T + t) * TILE + col0);
+        const uint4* y4 = Y32 ? reinterpret_cast<const uint4*>(prm.ylr32 + ((int64_t)bh * prm.T + t) * TILE + col0)
+                              : reinterpret_cast<const uint4*>(prm.ylr + ((int64_t)bh * prm.T + t) * TILE + col0);
 #pragma unroll
-        for (int i = 0; i < (SPLIT ? 8 : 4); ++i) y[i] = *(y4 + i);
+        for (int i = 0; i < (Y32 ? 8 : 4); ++i) y[i] = *(y4 + i);
       }
       if (!mbar_wait_warp(bar_o, it & 1, wc)) break;
       fence_after_sync();
@@ -1265,8 +1265,8 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
 #pragma unroll
         for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[i * 8 + e]);
         if (add_lr) {
-          if (SPLIT) {
-            const uint4 a = y[2 * i], c = y[SPLIT ? 2 * i + 1 : 0];
+          if (Y32) {
+            const uint4 a = y[Y32 ? 2 * i : 0], c = y[Y32 ? 2 * i + 1 : 0];
             f[0] += __uint_as_float(a.x); f[1] += __uint_as_float(a.y); f[2] += __uint_as_float(a.z); f[3] += __uint_as_float(a.w);
             f[4] += __uint_as_float(c.x); f[5] += __uint_as_float(c.y); f[6] += __uint_as_float(c.z); f[7] += __uint_as_float(c.w);
           } else {
@@ -2062,7 +2062,7 @@ cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* to
 }
 
 cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const void* V, const float* seg_in,
-                                          const void* ylr, int ylr_f32, int64_t n_lr, void* O, int64_t rows0, int64_t rows1,
+                                          const void* ylr, int ylr_f32, int split, int64_t n_lr, void* O, int64_t rows0, int64_t rows1,
                                           int nseg0, int nseg1, int bh, int* status, cudaStream_t st, void* sin_tiles) {
   const int64_t T = rows0 + rows1;
   SegOutMaps maps;
@@ -2082,8 +2082,10 @@ cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const vo
   prm.O = static_cast<__nv_bfloat16*>(O);
   prm.sin_tiles = static_cast<__nv_bfloat16*>(sin_tiles);
   prm.status = status;
-  auto kernel = ylr_f32 ? segment_output_tc_kernel<true> : segment_output_tc_kernel<false>;
-  const int smem = ylr_f32 ? SegOutLayout<true>::SMEM : SegOutLayout<false>::SMEM;
+  if (split && !ylr_f32) return cudaErrorInvalidValue;
+  auto kernel = split ? segment_output_tc_kernel<true, true>
+                      : ylr_f32 ? segment_output_tc_kernel<false, true> : segment_output_tc_kernel<false, false>;
+  const int smem = split ? SegOutLayout<true>::SMEM : SegOutLayout<false>::SMEM;
   cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
   dim3 grid((unsigned)prm.nseg, (unsigned)bh);
