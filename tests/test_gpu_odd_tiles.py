@@ -25,6 +25,7 @@ def test_blocks_of_odd_numbers_of_tiles(d, heads, T):
         assert ("segment_output_tc" in stages) == (plan is plans[0])
         got.append([O, *plan.backward(dev["q"], dev["k"], dev["v"], dev["do"], workspace=ws)])
         plan.check_status(ws)
-    # the same sums of the same rounded operands in another order, and the tile's state rounded to bf16 once either way
+    # The same sums in another order.  Either side's value is rounded to bf16 when it is stored, half a unit in the last place,
+    # 2^-8 of the largest at most; operands (state, scores) on a rounding boundary may fall to different sides, another 2^-8.
     for a, b in zip(*got):
-        assert rel_err(to_numpy64(a), to_numpy64(b)) <= 4e-3     # (as kept against rebuilt states in test_gpu_parity.py)
+        assert rel_err(to_numpy64(a), to_numpy64(b)) <= 3 * 2.0 ** -8
