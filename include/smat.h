@@ -144,21 +144,23 @@ size_t smat_workspace_bytes(const smat_plan* plan, int for_backward);
 
 /*
  * Forward pass, Algorithm 1 steps 2-7 (step 1 is implicit: φ = q_i, ψ = k_j, Z_j = k_j v_jᵀ).
- * Reads Q, K, V; writes O (plan dtype).  The profile table F and the type table U ("cached subset
- * states") are left in the workspace in the element type the plan keeps them in (fp32, or bf16: see
- * smat_profile_table_element_bytes / smat_type_table_element_bytes), the incoming states S_in as fp32 per
+ * Reads Q, K, V; writes O (plan dtype).  Where a type's tokens and the keys that it sees are few (short contexts, bf16,
+ * d_k = d_v = 128, positional routing), the long-range rows are formed from Q, K and V alone, and K and V of the distant
+ * tokens are left in the workspace, from which smat_debug_tables forms the tables.  Else the profile table F and the
+ * type table U ("cached subset states") are left there in the element type the plan keeps them in (fp32, or bf16: see
+ * smat_profile_table_element_bytes / smat_type_table_element_bytes).  The incoming states S_in are left as fp32 per
  * chunk (fp32-ALU plans) or as bf16 per 128-token tile (tensor-core plans with SMAT_FLAG_PER_TILE_STATES);
- * smat_debug_tables reads them back widened to fp32.  Asynchronous on `cuda_stream`.
+ * smat_debug_tables reads all of these back widened to fp32.  Asynchronous on `cuda_stream`.
  */
 smat_status smat_forward(const smat_plan* plan, const void* Q, const void* K, const void* V, void* O, void* workspace,
                          size_t workspace_bytes, void* cuda_stream);
 
 /*
  * Backward pass (chunking proof, "Backward Pass"): given dO = ∂L/∂O writes dQ, dK, dV (plan dtype).
- * It rebuilds the forward tables it needs (S_in, F, U) inside the workspace, so it does not
+ * It rebuilds what it needs of the forward (S_in; F and U, where the plan forms tables) inside the workspace, so it does not
  * depend on an earlier smat_forward call — unless the plan was created with SMAT_FLAG_KEEP_FORWARD_TABLES
- * (tensor-core plans only), in which case F and U are taken from the workspace as the preceding smat_forward
- * left them.  Asynchronous on `cuda_stream`.
+ * (tensor-core plans only), in which case it takes them from the workspace as the preceding smat_forward left them (F and U
+ * where that formed them).  Asynchronous on `cuda_stream`.
  */
 smat_status smat_backward(const smat_plan* plan, const void* Q, const void* K, const void* V, const void* dO, void* dQ,
                           void* dK, void* dV, void* workspace, size_t workspace_bytes, void* cuda_stream);

@@ -45,12 +45,14 @@ struct smat_plan {
   bool ubar_tc;        // backward pools the per-type adjoint states on the tensor cores
   bool ubar_bf16;      // ... and keeps them in bf16
   bool fbar_bf16;      // the per-profile adjoint states (transposed tabulation) are kept in bf16
+  bool lines;          // positional passes on the tensor cores form the long-range rows without tables (smat_lines.cu)
   mutable int launches;
   mutable bool tile_states;       // the last call left its incoming states at off_sin (bf16 per 128-token tile; on plans
                                   // with ragged_tc fp32 per chunk)
   mutable bool kept_tile_states;  // the last forward left them at off_sin_tiles for the backward (KEEP_FORWARD_TABLES)
   mutable bool kept_gated_forward;  // the last call was the tensor-core gated forward: λ, the rescaled K copies, U and the
                                     // per-tile states are still in the workspace (used under KEEP_FORWARD_TABLES)
+  mutable int forward_left;         // LineCopy: what the last forward left in the tables' place (0: it formed the tables)
   // optional per-launch timing (smat_profile_enable): event k is recorded before launch k
   mutable bool profiling;
   mutable cudaEvent_t events[SMAT_MAX_STAGES + 1];
@@ -148,7 +150,8 @@ struct Ctx {
 };
 
 // The 256 bytes at off_status: the status word, and at these offsets the numbers of heavy parts of a routed pass.
-constexpr size_t PROF_HEAVY_COUNT = 128, TYPE_HEAVY_COUNT = 192;
+// The word behind the status word says what a pass without tables left in their place (LineCopy).
+constexpr size_t PROF_HEAVY_COUNT = 128, TYPE_HEAVY_COUNT = 192, LINE_MARK = 4;
 
 // Parts of heavy groups that a head may have; none where no kernel asks for them.
 int64_t heavy_parts(const smat_plan* pl, bool prof) {
@@ -416,6 +419,33 @@ bool forward_rows_f32(const smat_plan* pl) {
          smat_segment_tiles(lr ? pl->geo.n / 128 : pl->T / 128, lr ? pl->geo.m / 128 : 0, pl->bh) < 2;
 }
 
+// Passes that form no tables leave K and V of the distant tokens in their place, for smat_debug_tables: in the long-range
+// buffer, beside the fp32 rows of the recent tokens (mark 1) or behind the bf16 rows of all (mark 2).
+enum LineCopy { LINE_COPY_NONE = 0, LINE_COPY_BESIDE = 1, LINE_COPY_BEHIND = 2 };
+size_t line_copy_offset(const smat_plan* pl, int where) {
+  return pl->off_acc + (where == LINE_COPY_BEHIND ? (size_t)pl->bh * pl->T * 256 : 0);
+}
+
+// Long-range rows of the recent tokens (types = 1) or of the distant ones, without tables; see SmatLineArgs.
+SmatLineArgs line_job(int types, const void* x, const void* y, const void* z, void* out, int out_f32, const float* lam = nullptr) {
+  SmatLineArgs a{};
+  a.rows_are_types = types; a.x1 = x; a.y = y; a.z = z; a.out1 = out; a.out_f32 = out_f32; a.lam = lam;
+  return a;
+}
+void line_copy(const Ctx& cx, SmatLineArgs* a, int where, bool y_is_v) {
+  const smat_plan* pl = cx.pl;
+  a->copy = cx.ws + line_copy_offset(pl, where);
+  a->copy_head = where == LINE_COPY_BEHIND ? pl->geo.n : pl->T;
+  a->copy_swap = y_is_v;
+}
+void line_mark(const Ctx& cx, SmatLineArgs* a, int where) {
+  a->mark = reinterpret_cast<int*>(cx.ws + cx.pl->off_status + LINE_MARK);
+  a->mark_value = where;
+}
+void line_rows(Ctx& cx, const char* name, const SmatLineArgs& a) {
+  SMAT_TRY(cx, name, smat_launch_line_products(a, cx.pl->geo, cx.pl->bh, cx.st));
+}
+
 // Steps 2-3 of Algorithm 1 alone, as the plan's forward runs them: the type table U ends in the workspace at the
 // returned offset (d = 1: the single state U_0 = F_0, fp32).
 size_t build_type_table(Ctx& cx, const void* K, const void* V) {
@@ -479,7 +509,7 @@ smat_status smat_plan_create(smat_plan** out, int batch, int heads, int64_t T, i
   pl->r = d_k; pl->p = d_v; pl->T = T; pl->c = chunk; pl->NC = T / chunk;
   pl->dtype = dtype; pl->flags = flags; pl->rp = (int64_t)d_k * d_v; pl->launches = 0;
   pl->profiling = false; pl->stages = 0; pl->tile_states = false; pl->kept_tile_states = false;
-  pl->kept_gated_forward = false;
+  pl->kept_gated_forward = false; pl->forward_left = 0;
   smat_status s = build_geometry(&pl->geo, T, chunk, d, q_override);
   if (s != SMAT_OK) { delete pl; return s; }
   const SmatGeo& g = pl->geo;
@@ -508,6 +538,10 @@ smat_status smat_plan_create(smat_plan** out, int batch, int heads, int64_t T, i
   pl->ubar_tc = pl->tc && !g.dense_G && (pl->tab_tc || g.m / g.B >= 12);
   pl->ubar_bf16 = pl->ubar_tc && ((g.D == 1 && fbar_by_read) || pl->tab_tc);   // d = 2: F̄ is Ū itself
   pl->fbar_bf16 = pl->tc && !g.dense_G && (pl->tab_tc || (g.D == 1 ? pl->ubar_bf16 : fbar_by_read));
+  // The flags that ask for a tabulation ask for tables.
+  const bool lines_by_flag = !(flags & (SMAT_FLAG_ALG2_TABULATION | SMAT_FLAG_ALU_TABULATION | SMAT_FLAG_D3_SHARED_SUMS));
+  pl->lines = lines_by_flag && ((pl->tc && pl->u_bf16 && pl->fbar_bf16) || pl->ragged_tc) &&
+              smat_lines_pay(g, pl->bh, pl->ragged_tc ? 4 : 2);
   // Workspace regions, each sized for the element type the plan stores there.  Tensor-core plans keep the causal
   // states per 128-token tile in bf16 (or, in the two-level form, fewer fp32 segment states in the same region); the
   // fp32-ALU plans keep one fp32 state per chunk.
@@ -678,14 +712,22 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     int* status = reinterpret_cast<int*>(cx.ws + pl->off_status);
     float* ylr = cx.f(pl->off_acc);
     const bool lr = !pl->geo.dense_G;
-    if (lr) build_type_table(cx, K, V);                                                      // steps 2-3
+    const bool lines = pl->lines && !cx.routed;
+    pl->forward_left = LINE_COPY_NONE;
+    if (lr && !lines) build_type_table(cx, K, V);                                            // steps 2-3
     // The causal branch is the two-level one wherever the plan does not ask for per-tile states: blocks of any number of tiles
     // are cut into segments that differ by a tile at most (odd numbers took the per-tile form: d = 2, 16 heads of 13,056 tokens
     // 155 -> 146 us, of 23,296 259 -> 239; d = 4, 8 heads of 22,912 423 -> 376; d = 1, 16 heads of 3200 36 -> 30).  It takes the
     // long-range rows as bf16 (half the bytes to write and to fetch) where blocks are even numbers of tiles, else in fp32.
     const int64_t tiles0 = lr ? pl->geo.n / 128 : pl->T / 128, tiles1 = lr ? pl->geo.m / 128 : 0;
     const bool per_tile = (pl->flags & SMAT_FLAG_PER_TILE_STATES) != 0, f32 = forward_rows_f32(pl);
-    if (lr) {                                                                                // step 4
+    if (lines) {                                                                             // steps 2-4 in one
+      SmatLineArgs a = line_job(1, Q, K, V, ylr, f32);
+      pl->forward_left = f32 ? LINE_COPY_BESIDE : LINE_COPY_BEHIND;
+      line_copy(cx, &a, pl->forward_left, false);
+      line_mark(cx, &a, pl->forward_left);
+      line_rows(cx, "read_lines", a);
+    } else if (lr) {                                                                         // step 4
       zero_unrouted(cx, SMAT_GM_TYPE, ylr, f32 ? 512 : 256);
       if (pl->u_bf16)
         SMAT_TRY(cx, "read_type_tc", smat_launch_state_read_tc(Q, cx.ws + pl->off_U, ylr, f32 ? nullptr : ylr, 0,
@@ -723,7 +765,12 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     float* ylr = cx.f(pl->off_acc);
     const bool lr = !pl->geo.dense_G;
     const int64_t rows0 = lr ? pl->geo.n : pl->T, rows1 = lr ? pl->geo.m : 0;
-    if (lr) {
+    if (pl->lines && !cx.routed) {
+      SmatLineArgs a = line_job(1, Q, K, V, ylr, 1);
+      line_copy(cx, &a, LINE_COPY_BESIDE, false);
+      line_mark(cx, &a, LINE_COPY_BESIDE);
+      line_rows(cx, "read_lines", a);
+    } else if (lr) {
       build_type_table(cx, K, V);
       zero_unrouted(cx, SMAT_GM_TYPE, ylr, 512);
       state_read(cx, "read_type", {read_job(cx, SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, ylr)});
@@ -783,20 +830,28 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
     const SmatGroupSpec types = group(cx, SMAT_GM_TYPE), profs = group(cx, SMAT_GM_PROFILE);
     const int64_t n = pl->geo.n;
     if (lr) {
-      if (!(pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES)) build_type_table(cx, K, V);
+      const bool lines = pl->lines && !cx.routed;
+      const bool after_forward = (pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES) != 0;
+      if (!lines && !(after_forward && pl->forward_left == LINE_COPY_NONE)) build_type_table(cx, K, V);
       // Ū_h = Σ q dOᵀ over the type (Eq. "lr-adjoint"), then F̄ = Cᵀ Ū
       const bool ubar_tc = pl->ubar_tc, ubar_bf16 = pl->ubar_bf16;
-      if (ubar_tc)
+      if (lines) {
+      } else if (ubar_tc)
         SMAT_TRY(cx, "bwd_pool_type_tc", smat_launch_pool_tc(Q, dO, cx.ws + pl->off_ubar, ubar_bf16, types, pl->geo.B,
                                                              max_group_tokens(pl, SMAT_GM_TYPE, cx.routed), pl->T, pl->bh,
                                                              status, cx.st));
       else
         outer_sum(cx, "bwd_pool_type", SMAT_GM_TYPE, Q, dO, cx.f(pl->off_ubar));
       const bool fbar_is_bf16 = pl->fbar_bf16;
-      if (pl->tab_tc)
+      if (lines) {
+      } else if (pl->tab_tc)
         tabulate_tc(cx, "bwd_tabulate_t_tc", cx.ws + pl->off_ubar, cx.ws + pl->off_fbar, 1);
       else
         tabulate(cx, "bwd_tabulate_t", cx.f(pl->off_ubar), cx.f(pl->off_fbar), 1, pl->geo.D == 2 && pl->fbar_bf16);
+      // dQ's long-range rows without tables; K and V of the distant tokens are behind them already where the forward left them
+      SmatLineArgs dq_lines = line_job(1, dO, V, K, lrbuf, 0);
+      if (!(after_forward && pl->forward_left == LINE_COPY_BEHIND)) line_copy(cx, &dq_lines, LINE_COPY_BEHIND, true);
+      line_mark(cx, &dq_lines, LINE_COPY_BEHIND);
       // per-tile states
       if (!kept)
         SMAT_TRY(cx, "bwd_state_scan_tc", smat_launch_chunk_scan_tc(K, V, sin_tiles, pl->T, pl->bh, n, 0, 0, status, cx.st));
@@ -805,8 +860,19 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
         // All three long-range terms come from the tensor-core read as bf16 rows: one buffer each, then ONE kernel for
         // the three within-chunk adjoints (every operand of a tile loaded once, both score tiles formed once).
         char* lr_q = cx.ws + pl->off_acc;
-        char* lr_k = lr_q + (size_t)pl->bh * pl->T * 128 * 2;
+        char* lr_k = lines ? lr_q : lr_q + (size_t)pl->bh * pl->T * 128 * 2;   // (dQ's rows are recent, dK's distant)
         char* lr_v = cx.ws + pl->off_lr3;
+        if (lines) {
+          line_rows(cx, "bwd_dq_lines", dq_lines);
+          SmatLineArgs a = line_job(0, K, Q, dO, lr_v, 0);
+          a.x2 = V; a.out2 = lr_k;
+          line_rows(cx, "bwd_dkdv_lines", a);
+          SMAT_TRY(cx, "bwd_tiles_fused_tc", smat_launch_bwd_tiles_fused_tc(Q, K, V, dO, sin_tiles, cx.ws + pl->off_dbar, lr_q,
+                                                                             lr_k, lr_v, n, dQ, dK, dV, pl->T, pl->bh, status,
+                                                                             cx.st));
+          pl->launches = cx.launches;
+          return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;
+        }
         zero_unrouted(cx, SMAT_GM_TYPE, lr_q, 256);
         SMAT_TRY(cx, "bwd_dq_type_tc", smat_launch_state_read_tc(dO, cx.ws + pl->off_U, nullptr, lr_q, 1, types, pl->geo.B,
                                                                  pl->T, pl->bh, status, cx.st));
@@ -823,8 +889,10 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
       }
       // dQ: recent rows add U_type dO
       // (the rows travel as bf16 where the tensor-core read writes them: rounded once, added in fp32 by the tile kernel)
-      zero_unrouted(cx, SMAT_GM_TYPE, lrbuf, pl->u_bf16 ? 256 : 512);
-      if (pl->u_bf16)
+      if (!lines) zero_unrouted(cx, SMAT_GM_TYPE, lrbuf, pl->u_bf16 ? 256 : 512);
+      if (lines)
+        line_rows(cx, "bwd_dq_lines", dq_lines);
+      else if (pl->u_bf16)
         SMAT_TRY(cx, "bwd_dq_type_tc", smat_launch_state_read_tc(dO, cx.ws + pl->off_U, lrbuf, lrbuf, 1, types, pl->geo.B,
                                                                  pl->T, pl->bh, status, cx.st));
       else
@@ -833,8 +901,10 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
                                                                   lrbuf, n, pl->T, dQ, pl->T, pl->bh, status, cx.st,
                                                                   pl->u_bf16 ? 1 : 0));
       // dK: distant rows add F̄_prof v
-      zero_unrouted(cx, SMAT_GM_PROFILE, lrbuf, fbar_is_bf16 ? 256 : 512);
-      if (fbar_is_bf16)
+      if (!lines) zero_unrouted(cx, SMAT_GM_PROFILE, lrbuf, fbar_is_bf16 ? 256 : 512);
+      if (lines)
+        line_rows(cx, "bwd_dk_lines", line_job(0, V, dO, Q, lrbuf, 0));
+      else if (fbar_is_bf16)
         SMAT_TRY(cx, "bwd_dk_profile_tc", smat_launch_state_read_tc(V, cx.ws + pl->off_fbar, lrbuf, lrbuf, 1, profs, pl->geo.P,
                                                                     pl->T, pl->bh, status, cx.st));
       else
@@ -843,8 +913,10 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
                                                                   lrbuf, 0, n, dK, pl->T, pl->bh, status, cx.st,
                                                                   fbar_is_bf16 ? 1 : 0));
       // dV: distant rows add F̄_profᵀ k
-      zero_unrouted(cx, SMAT_GM_PROFILE, lrbuf, fbar_is_bf16 ? 256 : 512);
-      if (fbar_is_bf16)
+      if (!lines) zero_unrouted(cx, SMAT_GM_PROFILE, lrbuf, fbar_is_bf16 ? 256 : 512);
+      if (lines)
+        line_rows(cx, "bwd_dv_lines", line_job(0, K, Q, dO, lrbuf, 0));
+      else if (fbar_is_bf16)
         SMAT_TRY(cx, "bwd_dv_profile_tc", smat_launch_state_read_tc(K, cx.ws + pl->off_fbar, lrbuf, lrbuf, 0, profs, pl->geo.P,
                                                                     pl->T, pl->bh, status, cx.st));
       else
@@ -954,11 +1026,13 @@ smat_status forward_gated_tc(Ctx& cx, const Gated& gt, const void* Q, const void
   int* status = reinterpret_cast<int*>(ci.ws + in->off_status);
   SMAT_TRY(cx, "gate_prefix", smat_launch_head_scan(log_a, gt.lam, pl->T, pl->bh, 0, cx.st));
   // exp(λ_{tile end} - λ_j) k_j, and keys and queries split at the boundary
-  SMAT_TRY(cx, "gate_scale", smat_launch_gate_scale_pair(K, K, Q, gt.kc, lr ? gt.lr : nullptr, gt.lam, 1, pl->geo.n, pl->T,
-                                                         pl->bh, cx.st));
+  SMAT_TRY(cx, "gate_scale", smat_launch_gate_scale_pair(K, K, Q, gt.kc, lr && !in->lines ? gt.lr : nullptr, gt.lam, 1, pl->geo.n,
+                                                         pl->T, pl->bh, cx.st));
   ci.err = cx.err;
   float* ylr = ci.f(in->off_acc);
-  if (lr) {
+  if (in->lines) {   // the factors at the boundary enter the scores and the rows
+    line_rows(ci, "read_lines", line_job(1, Q, K, V, ylr, 1, gt.lam));
+  } else if (lr) {
     build_type_table(ci, gt.lr, V);                                                          // steps 2-3 on the rescaled keys
     if (in->u_bf16)
       SMAT_TRY(ci, "read_type_tc", smat_launch_state_read_tc(gt.lr, ci.ws + in->off_U, ylr, nullptr, 0,
@@ -1001,17 +1075,24 @@ smat_status backward_gated_tc(Ctx& cx, const Gated& gt, const void* Q, const voi
   const bool kept = (pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES) && after_gated_forward;
   if (!kept) {
     SMAT_TRY(cx, "gate_prefix", smat_launch_head_scan(log_a, gt.lam, pl->T, pl->bh, 0, cx.st));
-    SMAT_TRY(cx, "gate_scale", smat_launch_gate_scale_pair(K, K, Q, gt.kc, lr ? gt.lr : nullptr, gt.lam, 1, n, pl->T, pl->bh,
-                                                           cx.st));
+    SMAT_TRY(cx, "gate_scale", smat_launch_gate_scale_pair(K, K, Q, gt.kc, lr && !in->lines ? gt.lr : nullptr, gt.lam, 1, n, pl->T,
+                                                           pl->bh, cx.st));
   }
-  SMAT_TRY(cx, "bwd_gate_scale", smat_launch_gate_scale_pair(Q, V, dO, gt.qc, lr ? gt.vlr : nullptr, gt.lam, 0, n, pl->T,
-                                                             pl->bh, cx.st));
+  SMAT_TRY(cx, "bwd_gate_scale", smat_launch_gate_scale_pair(Q, V, dO, gt.qc, lr && !in->lines ? gt.vlr : nullptr, gt.lam, 0, n,
+                                                             pl->T, pl->bh, cx.st));
   ci.err = cx.err;
   char* sin = ci.ws + in->off_sin;
   char* dbar = ci.ws + in->off_dbar;
   float* dlam = cx.f(pl->off_dlam);
   char *lr_q = nullptr, *lr_k = nullptr, *lr_v = nullptr;
-  if (lr) {
+  if (in->lines) {
+    lr_q = lr_k = ci.ws + in->off_acc;
+    lr_v = ci.ws + in->off_lr3;
+    line_rows(ci, "bwd_dq_lines", line_job(1, dO, V, K, lr_q, 0, gt.lam));
+    SmatLineArgs a = line_job(0, K, Q, dO, lr_v, 0, gt.lam);
+    a.x2 = V; a.out2 = lr_k;
+    line_rows(ci, "bwd_dkdv_lines", a);
+  } else if (lr) {
     const SmatGroupSpec types = group(ci, SMAT_GM_TYPE), profs = group(ci, SMAT_GM_PROFILE);
     if (!kept) build_type_table(ci, gt.lr, V);
     if (in->ubar_tc)
@@ -1281,6 +1362,13 @@ smat_status smat_debug_tables(const smat_plan* pl, const void* workspace, float*
       err = cudaMemcpy2DAsync(dst, state, ws + pl->off_sin + (size_t)first_recent * state, (size_t)pl->NC * state,
                               state, pl->bh, cudaMemcpyDeviceToDevice, st);
     }
+  } else if (pl->lines) {
+    const int* mark = reinterpret_cast<const int*>(ws + pl->off_status + LINE_MARK);
+    const void *beside = ws + line_copy_offset(pl, LINE_COPY_BESIDE), *behind = ws + line_copy_offset(pl, LINE_COPY_BEHIND);
+    if (F && err == cudaSuccess)
+      err = smat_launch_line_tables(pl->geo, pl->bh, mark, beside, behind, ws + pl->off_F, pl->f_bf16, pl->f_bf16, 0, F, st);
+    if (U && err == cudaSuccess)
+      err = smat_launch_line_tables(pl->geo, pl->bh, mark, beside, behind, ws + pl->off_U, pl->u_bf16, pl->f_bf16, 1, U, st);
   } else {
     if (F && err == cudaSuccess) {
       if (pl->f_bf16)

@@ -286,3 +286,25 @@ cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const vo
                                           const void* ylr, int ylr_f32, int split, int64_t n_lr, void* O, int64_t rows0, int64_t rows1,
                                           int nseg0, int nseg1, int bh, int* status, cudaStream_t st,
                                           void* sin_tiles = nullptr);
+// Long-range rows without tables (see smat_lines.cu), positional routing, bf16 rows of 128: for every token t of a type (or,
+// rows_are_types = 0, of a cell) out1_t = Σ_s (x1_t · y_s) z_s over the tokens s of the cells of its hyperplane (of the types
+// through the cell), and with out2 also out2_t = Σ_s (x2_t · z_s) y_s.
+struct SmatLineArgs {
+  const void *x1, *x2, *y, *z;
+  void *out1, *out2;
+  int out_f32, rows_are_types;
+  const float* lam;      // gated: prefix sums of the log-gates; terms are multiplied by exp(λ_recent - λ_distant)
+  void* copy;            // null, or where K and V of every distant token are left side by side: token t of head b at
+  int64_t copy_head;     // row b * copy_head + t of 512 bytes
+  int copy_swap;         // y is V and z is K
+  int* mark;             // null, or a word that is set to mark_value
+  int mark_value;
+};
+// Whether the kernel takes the shape, and whether it is the faster way (table_bytes: of an entry of the tables otherwise).
+bool smat_lines_supported(const SmatGeo& geo, int bh);
+bool smat_lines_pay(const SmatGeo& geo, int bh, int table_bytes);
+// F (types = 0) or U of a pass of a plan that may have formed no tables, as fp32: from K and V that it left where *mark says (1:
+// beside, 2: behind), or from `table` where *mark is zero.
+cudaError_t smat_launch_line_tables(const SmatGeo& geo, int bh, const int* mark, const void* beside, const void* behind,
+                                    const void* table, int table_bf16, int profile_bf16, int types, float* dst, cudaStream_t st);
+cudaError_t smat_launch_line_products(const SmatLineArgs& a, const SmatGeo& geo, int bh, cudaStream_t st);

@@ -83,7 +83,7 @@ struct PoolCursor {
 
 // Two token buffers alternate over the passes, also inside a group of many tokens: the next pass's rows (of the same
 // group or of the next item) travel while this pass is summed.
-// clear (or null): the status word of a pass that begins with this launch, which waits for nothing that could fail.
+// clear (or null): the status word (and the mark behind it) of a pass that begins with this launch, which waits for nothing that could fail.
 // TK: tokens staged per pass.
 template <int R, int PD, typename T, int TK>
 __global__ void __launch_bounds__(256) pool_stream_kernel(const __grid_constant__ PoolList list, int64_t Tlen, int* clear) {
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(256) pool_stream_kernel(const __grid_constant_
   };
 
   pdl_wait();   // (the token lists of a routed call come from the kernel before)
-  if (clear && blockIdx.x == 0 && tid == 0) *clear = 0;
+  if (clear && blockIdx.x == 0 && tid == 0) clear[0] = clear[1] = 0;
   PoolCursor<TK> cur(list, blockIdx.x, gridDim.x);
   fetch(cur, 0);
   float4 acc[NS];

@@ -115,6 +115,10 @@ def stage_table(T, c, r, p, e, geo, u_bytes=4, f_bytes=4, alu_path=False) -> dic
     profiles = Work(2 * n * rp, 0, n * (r + p) * e + P * st)
     dq_tile = Work(T * 129 * (r + p) + 2 * T * rp, 0, T * (2 * p + 2 * r) * e + tc_tiles * rp * 2 + m * r * 2)
     scaled = lambda dim: Work(0, 0, 2 * T * dim * e + 4 * T)
+    # long-range rows without tables: a recent and a distant token meet where the type's hyperplane holds the cell, one in q;
+    # operands in and rows out once (between the two, rows are gathered from the L2 cache many times over)
+    pairs = m * n / geo.q if lr else 0
+    lines = lambda dim, operands, out: Work(pairs * 2 * dim, 0, operands + out)
     table = {
         # K and V are read once for both sets of states; d = 1 without chunk states: the one state of the decode cache
         "pool":        Work(2 * (T + n) * rp, 0, T * (r + p) * e + (NC + P) * st) if alu_path else
@@ -126,6 +130,12 @@ def stage_table(T, c, r, p, e, geo, u_bytes=4, f_bytes=4, alu_path=False) -> dic
         "tabulate_bf16": Work(0, geo.nnzC * rp, P * sf + B * su),
         "read_type":   Work(2 * m * rp, 0, m * r * e + B * st + m * p * 4),
         "read_type_tc": Work(2 * m * rp, 0, m * r * e + B * su + m * p * 2),
+        # ... and without tables
+        "read_lines":  lines(r + p, (m * r + n * (r + p)) * e, m * p * row),
+        "bwd_dq_lines": lines(r + p, (m * p + n * (r + p)) * e, m * r * 2),
+        "bwd_dkdv_lines": lines(2 * (r + p), (n + m) * (r + p) * e, n * (r + p) * 2),
+        "bwd_dk_lines": lines(r + p, (n * p + m * (r + p)) * e, n * r * 2),
+        "bwd_dv_lines": lines(r + p, (n * r + m * (r + p)) * e, n * p * 2),
         # causal branch on the tensor cores
         "segment_state_tc": Work(2 * T * rp, 0, T * (r + p) * e),
         "segment_scan": Work(0, 0, 0),                                 # scratch of the branch: totals of whole segments

@@ -1,0 +1,125 @@
+"""Long-range rows formed without tables (smat_lines.cu) at its edges, against the fp64 dense-mask oracle: 16- and 32-row tiles
+with one row missing, full and one row over, several row blocks, last steps of 1 to 16 slots, every class of direction, blocks
+that are not whole tiles, gates; and the export of tables that the pass has not formed."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import chunkwise_ref as cw
+from oracle import smat_oracle as so
+from paper_2609_36062_b200 import binding, synth
+from tests.helpers import TOL, device_inputs, rel_err, sample_tokens, to_numpy64
+
+pytestmark = pytest.mark.gpu
+
+
+def _plan(w, flags=0, q=0):
+    return binding.SmatPlan(w.batch, w.heads, w.T, w.d_k, w.d_v, w.d, w.chunk, w.dtype, flags=flags, q_override=q)
+
+
+def _stages(plan, call):
+    plan.profile_enable(True)
+    out = call()
+    names = [name for name, _ in plan.profile_read()]
+    plan.profile_enable(False)
+    plan.check_status()
+    return out, names
+
+
+# d, heads, tokens, chunk, field size (0: the default); rows of a type / of a cell, slots of a type / of a cell
+CASES = [
+    (3, 8, 2048, 128, 0),      # q = 11: 7 or 8 / 8 or 9 rows, 99 / 96 slots
+    (3, 20, 2048, 128, 7),     # q = 7: 19 / 21 rows (two tiles, two blocks of one), 147 / 152 slots
+    (4, 4, 2048, 64, 0),       # q = 7: 2 or 3 rows, three classes of direction
+    (4, 32, 1024, 128, 3),     # q = 3: 13 or 14 / 18 or 19 rows
+    (3, 8, 2304, 64, 0),       # odd numbers of tiles: rows in fp32
+    (3, 8, 2240, 64, 0),       # blocks that are not whole tiles (forward alone)
+    (2, 32, 2112, 64, 0),      # ... d = 2: one cell to a type, 32 rows
+    (4, 4, 2240, 64, 0),
+]
+
+
+@pytest.mark.parametrize("d,heads,T,c,q", CASES)
+def test_rows_without_tables_match_the_dense_oracle(d, heads, T, c, q):
+    w = synth.Workload("lines", d, 1, heads, T, 128, 128, c, "bf16", "normalised", 300 + T + d)
+    host, dev = device_inputs(w, ("q", "k", "v", "do"))
+    plan = _plan(w, q=q)
+    O, names = _stages(plan, lambda: plan.forward(dev["q"], dev["k"], dev["v"]))
+    assert "read_lines" in names and "pool_tc" not in names
+    F, U, _ = plan.debug_tables()
+    grads, names = _stages(plan, lambda: plan.backward(dev["q"], dev["k"], dev["v"], dev["do"]))
+    geo = so.geometry(T, c, d, q or None)
+    assert ("bwd_dkdv_lines" in names) == (geo.n % 128 == 0 and (T - geo.n) % 128 == 0)
+    F2, U2, _ = plan.debug_tables()
+    M = so.dense_mask(T, c, d, q or None)
+    tables = 1.0 if plan.profile_table_element_bytes() == 2 else 1e-3   # bf16 tables, or fp32: bounds of test_gpu_parity.py
+    for h in (0, heads - 1):
+        Q64, K64, V64, G64 = (synth.as_float64(w, host[x][h]) for x in ("q", "k", "v", "do"))
+        for got, ref in zip((O, *grads), (so.forward_dense(Q64, K64, V64, M), *so.backward_dense(Q64, K64, V64, G64, M))):
+            assert rel_err(to_numpy64(got[0, h]), ref) <= TOL["bf16"]
+        _, tab = cw.forward(Q64, K64, V64, geo, return_tables=True)
+        for got in (F, F2):
+            assert rel_err(to_numpy64(got[h]), tab["F"]) <= 8e-3 * tables
+        for got in (U, U2):
+            assert rel_err(to_numpy64(got[h]), tab["U"]) <= 1.2e-2 * tables
+
+
+@pytest.mark.parametrize("d,heads,T", [(3, 8, 2048), (4, 4, 2304)])
+def test_gated_rows_without_tables_match_the_dense_oracle(d, heads, T):
+    w = synth.Workload("glines", d, 1, heads, T, 128, 128, 128, "bf16", "normalised", 400 + T)
+    host, dev = device_inputs(w, ("q", "k", "v", "do"))
+    rng = np.random.default_rng(T)
+    la = np.log(rng.uniform(0.99, 1.0, (heads, T))).astype(np.float32)     # the boundary is within reach
+    la_dev = torch.from_numpy(la).cuda()
+    plan = _plan(w, binding.FLAG_GATED | binding.FLAG_KEEP_FORWARD_TABLES)
+    ws = plan.workspace(for_backward=True)
+    plan.profile_enable(True)
+    O = plan.forward_gated(dev["q"], dev["k"], dev["v"], la_dev, workspace=ws)
+    assert "read_lines" in [name for name, _ in plan.profile_read()]
+    grads = plan.backward_gated(dev["q"], dev["k"], dev["v"], la_dev, dev["do"], workspace=ws)
+    assert {"bwd_dq_lines", "bwd_dkdv_lines"} <= {name for name, _ in plan.profile_read()}
+    plan.profile_enable(False)
+    plan.check_status(ws)
+    M = so.dense_mask(T, 128, d)
+    for h in (0, heads - 1):
+        Q64, K64, V64, G64 = (synth.as_float64(w, host[x][h]) for x in ("q", "k", "v", "do"))
+        lah = la[h].astype(np.float64)
+        assert rel_err(to_numpy64(O[0, h]), so.gated_forward_dense(Q64, K64, V64, M, lah)) <= TOL["bf16"]
+        rq, rk, rv, rla = so.gated_backward_dense(Q64, K64, V64, G64, M, lah)
+        for got, ref in zip(grads[:3], (rq, rk, rv)):
+            assert rel_err(to_numpy64(got[0, h]), ref) <= TOL["bf16"]
+        assert rel_err(to_numpy64(grads[3].reshape(heads, T)[h]), rla) <= 5e-2   # (the stated bound of the gate gradient)
+
+
+def test_two_tiles_of_rows_at_full_length():
+    """q = 23, 16 or 17 rows to a type, in two tiles of 16: sampled rows of a long forward pass."""
+    w = synth.Workload("long", 3, 1, 4, 18432, 128, 128, 128, "bf16", "normalised", 77)
+    host, dev = device_inputs(w)
+    plan = _plan(w)
+    O, names = _stages(plan, lambda: plan.forward(dev["q"], dev["k"], dev["v"]))
+    assert "read_lines" in names
+    geo = so.geometry(w.T, w.chunk, w.d)
+    rows = sample_tokens(geo, 64, seed=5)
+    Q64, K64, V64 = (synth.as_float64(w, host[x][3]) for x in ("q", "k", "v"))
+    assert rel_err(to_numpy64(O[0, 3][rows]), so.forward_rows(Q64, K64, V64, geo, rows)) <= TOL["bf16"]
+
+
+def test_non_finite_tokens_reach_no_row_that_does_not_see_them():
+    """An unseen token is never gathered, and a slot without a token gathers one that its rows see: rows whose hyperplane misses
+    the cell keep their bits."""
+    w = synth.Workload("nan", 3, 1, 8, 2048, 128, 128, 128, "bf16", "normalised", 91)
+    _, dev = device_inputs(w)
+    plan = _plan(w)
+    clean = plan.forward(dev["q"], dev["k"], dev["v"])
+    s = 5
+    k, v = dev["k"].clone(), dev["v"].clone()
+    k[0, 3, s], v[0, 3, s] = float("nan"), float("inf")
+    dirty = plan.forward(dev["q"], k, v)
+    plan.check_status()
+    geo = so.geometry(w.T, w.chunk, w.d)
+    unseen = torch.from_numpy(so.mask_col(s, geo)[geo.n:] == 0).cuda()
+    assert unseen.any() and not unseen.all()
+    assert torch.equal(dirty[0, 3, geo.n:][unseen], clean[0, 3, geo.n:][unseen])
+    assert not torch.isfinite(dirty[0, 3, geo.n:][~unseen].float()).any(dim=-1).any()
+    others = [h for h in range(8) if h != 3]
+    assert torch.equal(dirty[0, others], clean[0, others])
