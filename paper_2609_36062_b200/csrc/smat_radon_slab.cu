@@ -178,8 +178,10 @@ __global__ void __launch_bounds__(THREADS, 1) radon_slab_kernel(const __grid_con
   pdl_trigger();
   const uint32_t acc1 = tmem_base + R_COLS, acc2 = acc1 + 64 * ACC1;
   constexpr uint32_t idesc = make_idesc(128, NE, 0, 1);   // R from tensor memory, image rows MN-major
-  auto slab_head = [&](uint32_t k, int& e0) {             // head and first entry of this CTA's slab k
-    const uint32_t slab = blockIdx.x + k * gridDim.x, head = slab / prm.slabs_per_head;
+  // Head and first entry of this CTA's slab k: the last heads first, whose F the pooling has just written, so that the read finds
+  // the first ones' U in the L2 cache (32 heads of 16 K tokens, the pass 1392 -> 1385 us).
+  auto slab_head = [&](uint32_t k, int& e0) {
+    const uint32_t slab = prm.slabs - 1 - (blockIdx.x + k * gridDim.x), head = slab / prm.slabs_per_head;
     e0 = (int)(slab - head * prm.slabs_per_head) * NE;
     return (int)head;
   };
