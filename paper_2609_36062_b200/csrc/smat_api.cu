@@ -697,7 +697,7 @@ void zero_unrouted(Ctx& cx, int mode, void* rows, int row_bytes) {
 }
 
 smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, const void* V, void* O, const int32_t* prof,
-                         const int32_t* type, void* workspace, size_t workspace_bytes, void* cuda_stream) {
+                         const int32_t* type, void* workspace, size_t workspace_bytes, void* cuda_stream, bool divide = false) {
   if (!Q || !K || !V || !O) return SMAT_ERR_NULL;
   smat_status s = check_common(pl, workspace, workspace_bytes, 0);
   if (s != SMAT_OK) return s;
@@ -745,7 +745,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
       const bool keep = (pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES) != 0;   // a backward will want the per-tile states
       SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, cx.f(pl->off_sin), ylr, f32, 0, lr ? pl->geo.n : pl->T, O,
                                                                        rows0, rows1, sg.nseg0, sg.nseg1, pl->bh, status, cx.st,
-                                                                       keep ? cx.ws + pl->off_sin_tiles : nullptr));
+                                                                       keep ? cx.ws + pl->off_sin_tiles : nullptr, divide));
       pl->kept_tile_states = keep;
     } else {
       SMAT_TRY(cx, "chunk_scan_tc", smat_launch_chunk_scan_tc(K, V, cx.ws + pl->off_sin, pl->T, pl->bh, pl->geo.n,
@@ -777,7 +777,8 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     }
     const Segments sg = segment_totals(cx, K, V, rows0, rows1, 2);
     SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, cx.f(pl->off_sin), ylr, 1, 1, lr ? pl->geo.n : pl->T, O, rows0,
-                                                                     rows1, sg.nseg0, sg.nseg1, pl->bh, status, cx.st));
+                                                                     rows1, sg.nseg0, sg.nseg1, pl->bh, status, cx.st, nullptr,
+                                                                     divide));
     pl->launches = cx.launches;
     return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;
   }
@@ -1154,10 +1155,19 @@ smat_status smat_forward_normalized(const smat_plan* pl, const void* Q, const vo
   const int64_t rows = (int64_t)pl->bh * pl->T;
   // v̄ = [v; 1]: the last value column is the normaliser column (Eq. "augmented-kv-state")
   if (smat_launch_normalize_step(0, V, nullptr, ws + pl->off_nv, bf, pl->p, rows, st) != cudaSuccess) return SMAT_ERR_LAUNCH;
-  smat_status s = forward_impl(pl, Q, K, ws + pl->off_nv, ws + pl->off_ny, nullptr, nullptr, workspace, workspace_bytes,
-                               cuda_stream);
+  // The single final division (Eq. "augmented-attention-output"): by the output kernel of the two-level branch, before the rows
+  // are rounded, or by a kernel of its own (32 heads of 5056 tokens, d = 3: 231 us a pass, 248; 16 of 13,056, d = 2: 177,
+  // 209), also where O is an operand's array, which others may still read.
+  const size_t bytes = (size_t)rows * 256;
+  const bool divides = (pl->tc || pl->ragged_tc) && !(pl->flags & SMAT_FLAG_PER_TILE_STATES) && !smat_overlap(O, bytes, Q, bytes) &&
+                       !smat_overlap(O, bytes, K, bytes);
+  smat_status s = forward_impl(pl, Q, K, ws + pl->off_nv, divides ? O : ws + pl->off_ny, nullptr, nullptr, workspace,
+                               workspace_bytes, cuda_stream, divides);
   if (s != SMAT_OK) return s;
-  // the single final division (Eq. "augmented-attention-output")
+  if (divides) {
+    pl->launches += 1;
+    return SMAT_OK;
+  }
   if (smat_launch_normalize_step(1, ws + pl->off_ny, nullptr, O, bf, pl->p, rows, st) != cudaSuccess) return SMAT_ERR_LAUNCH;
   pl->launches += 2;
   return SMAT_OK;

@@ -281,11 +281,12 @@ bool smat_segments_need_scan(int nseg0, int nseg1);
 cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* totals, int64_t rows0, int64_t rows1,
                                          int nseg0, int nseg1, int bh, int* status, cudaStream_t st);
 // ylr_f32: the long-range rows are fp32 (else bf16).  split: any blocks (else of whole tiles), and the state and the scores enter
-// their products as a bf16 part plus a bf16 remainder (with fp32 rows only).
+// their products as a bf16 part plus a bf16 remainder (with fp32 rows only).  divide: the rows leave divided by their last column,
+// which stays as it is.
 cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const void* V, const float* seg_in,
                                           const void* ylr, int ylr_f32, int split, int64_t n_lr, void* O, int64_t rows0, int64_t rows1,
                                           int nseg0, int nseg1, int bh, int* status, cudaStream_t st,
-                                          void* sin_tiles = nullptr);
+                                          void* sin_tiles = nullptr, int divide = 0);
 // Long-range rows without tables (see smat_lines.cu), positional routing, bf16 rows of 128: for every token t of a type (or,
 // rows_are_types = 0, of a cell) out1_t = Σ_s (x1_t · y_s) z_s over the tokens s of the cells of its hyperplane (of the types
 // through the cell), and with out2 also out2_t = Σ_s (x2_t · z_s) y_s.

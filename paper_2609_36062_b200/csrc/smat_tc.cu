@@ -942,7 +942,9 @@ struct SegOutLayout {
   static constexpr int V_STRIDE = SPLIT ? 0 : STAGE;
   static constexpr int STATE = SPLIT ? 2 * STAGE + 2 * BOX_BYTES : 2 * STAGE;
   static constexpr int BARS = STATE + (SPLIT ? 4 : 2) * BOX_BYTES;
-  static constexpr int SMEM = BARS + 1024 + 256;
+  static constexpr int NORM = BARS + 256;                          // two tiles' normalisers
+  static constexpr int SMEM = NORM + 2 * TILE * 4 + 1024;
+  static_assert(SMEM <= 227 * 1024, "shared memory of a CTA");
 };
 
 struct SegOutParams {
@@ -982,7 +984,7 @@ struct SegOutMaps {
   CUtensorMap q[2], k[2], v[2];
 };
 
-template <bool SPLIT, bool Y32>
+template <bool SPLIT, bool Y32, bool DIVIDE>
 __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(const __grid_constant__ SegOutMaps maps,
                                                                             const SegOutParams prm) {
   using Lay = SegOutLayout<SPLIT>;
@@ -1000,8 +1002,10 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
   uint64_t* bar_qk = bars + 9;     // Q S finished and the state updated: Q, K and the shared state may be overwritten
   uint64_t* bar_p = bars + 10;     // P written (one arrival per warp)
   uint64_t* bar_o = bars + 11;     // output complete
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 12);
+  uint64_t* bar_n = bars + 12;     // [4] normalisers of the tile's row quarter written
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  float* norm = reinterpret_cast<float*>(smem + Lay::NORM);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int seg = blockIdx.x, bh = blockIdx.y;
   int64_t tile0;
@@ -1015,6 +1019,7 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
     mbar_init(vfull, 1); mbar_init(vempty, 1);
     mbar_init(bar_s, SEG_EPI_WARPS); mbar_init(bar_sc, 1); mbar_init(bar_scr, SEG_EPI_WARPS); mbar_init(bar_qk, 1);
     mbar_init(bar_p, SEG_EPI_WARPS); mbar_init(bar_o, 1);
+    for (int i = 0; i < 4; ++i) mbar_init(bar_n + i, 1);
     fence_barrier_init();
   }
   if (warp == SEG_EPI_WARPS) tmem_alloc(tmem_slot, 512);
@@ -1258,29 +1263,45 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
       uint32_t v[32];
       tmem_ld32(tmem_o + lane_base + col0, v);
       tmem_ld_wait();
-      uint32_t w[16];
+      float f[32];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        float f[8];
+      for (int e = 0; e < 32; ++e) f[e] = __uint_as_float(v[e]);
+      if (add_lr) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[i * 8 + e]);
-        if (add_lr) {
+        for (int i = 0; i < 4; ++i) {
+          float* fi = f + 8 * i;
           if (Y32) {
             const uint4 a = y[Y32 ? 2 * i : 0], c = y[Y32 ? 2 * i + 1 : 0];
-            f[0] += __uint_as_float(a.x); f[1] += __uint_as_float(a.y); f[2] += __uint_as_float(a.z); f[3] += __uint_as_float(a.w);
-            f[4] += __uint_as_float(c.x); f[5] += __uint_as_float(c.y); f[6] += __uint_as_float(c.z); f[7] += __uint_as_float(c.w);
+            fi[0] += __uint_as_float(a.x); fi[1] += __uint_as_float(a.y); fi[2] += __uint_as_float(a.z); fi[3] += __uint_as_float(a.w);
+            fi[4] += __uint_as_float(c.x); fi[5] += __uint_as_float(c.y); fi[6] += __uint_as_float(c.z); fi[7] += __uint_as_float(c.w);
           } else {
             const uint32_t yy[4] = {y[i].x, y[i].y, y[i].z, y[i].w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              f[2 * e] += __uint_as_float(yy[e] << 16);
-              f[2 * e + 1] += __uint_as_float(yy[e] & 0xffff0000u);
+              fi[2 * e] += __uint_as_float(yy[e] << 16);
+              fi[2 * e + 1] += __uint_as_float(yy[e] & 0xffff0000u);
             }
           }
         }
-        w[4 * i] = pack_bf16(f[0], f[1]); w[4 * i + 1] = pack_bf16(f[2], f[3]);
-        w[4 * i + 2] = pack_bf16(f[4], f[5]); w[4 * i + 3] = pack_bf16(f[6], f[7]);
       }
+      if (DIVIDE) {
+        // The warps of the last column quarter hold the normalisers.  (A tile's are written over those of two tiles before, which
+        // every warp has read by the time it publishes the state in between.)
+        float* at = norm + (it & 1) * TILE + m;
+        if (cq == 3) {
+          *at = f[31];
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_n + (warp & 3));
+        }
+        if (!mbar_wait_warp(bar_n + (warp & 3), it & 1, wc)) break;
+        const float den = *at, inv = 1.0f / den;
+#pragma unroll
+        for (int e = 0; e < 32; ++e) f[e] *= inv;
+        if (cq == 3) f[31] = den;
+      }
+      uint32_t w[16];
+#pragma unroll
+      for (int e = 0; e < 16; ++e) w[e] = pack_bf16(f[2 * e], f[2 * e + 1]);
       if (live) {
 #pragma unroll
         for (int h8 = 0; h8 < 2; ++h8)   // whole 32-byte sectors
@@ -2063,7 +2084,7 @@ cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* to
 
 cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const void* V, const float* seg_in,
                                           const void* ylr, int ylr_f32, int split, int64_t n_lr, void* O, int64_t rows0, int64_t rows1,
-                                          int nseg0, int nseg1, int bh, int* status, cudaStream_t st, void* sin_tiles) {
+                                          int nseg0, int nseg1, int bh, int* status, cudaStream_t st, void* sin_tiles, int divide) {
   const int64_t T = rows0 + rows1;
   SegOutMaps maps;
   const void* src[3] = {Q, K, V};
@@ -2083,8 +2104,9 @@ cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const vo
   prm.sin_tiles = static_cast<__nv_bfloat16*>(sin_tiles);
   prm.status = status;
   if (split && !ylr_f32) return cudaErrorInvalidValue;
-  auto kernel = split ? segment_output_tc_kernel<true, true>
-                      : ylr_f32 ? segment_output_tc_kernel<false, true> : segment_output_tc_kernel<false, false>;
+  auto kernel = split     ? (divide ? segment_output_tc_kernel<true, true, true> : segment_output_tc_kernel<true, true, false>)
+                : ylr_f32 ? (divide ? segment_output_tc_kernel<false, true, true> : segment_output_tc_kernel<false, true, false>)
+                          : (divide ? segment_output_tc_kernel<false, false, true> : segment_output_tc_kernel<false, false, false>);
   const int smem = split ? SegOutLayout<true>::SMEM : SegOutLayout<false>::SMEM;
   cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
