@@ -6,8 +6,8 @@
 // tokens against the tokens of all types through the cell, both products from one gather (DUAL).  The rows come from the L2
 // cache, which holds a head's K and V many times over, and nothing but the outputs goes back to memory.
 //
-// Scores are rounded to bf16 once, as the causal tiles' are (where the plan's tables are fp32, to a leading part and a remainder,
-// 16 bits); the tables were rounded once for F and once or three times for U.
+// Scores are rounded to bf16 once, as the causal tiles' are; tables are rounded once for F and once or three times for U.  Where
+// the plan's tables are fp32, and for d = 2 (one rounding there too), they enter as a leading part and a remainder, 16 bits.
 //
 // The matrix instructions are those of a warp (m16n8k16): a type has 6 to 20 rows, which fill a tile of 16 and would leave most
 // of a 128-row one of tcgen05 empty, and at 545 TFLOP/s measured they are not what the kernel waits for.
@@ -179,11 +179,12 @@ struct LineSmem {
 //   scores   its words of a row are bytes 32 q to 32 q + 31 of either half: the order of the contracted index is free, as
 //            long as X and Y have the same
 //   outputs  the rows of Z transposed on the way from shared memory (ldmatrix)
-// Bound by the instructions that a warp issues for a stage, about 400 one after the other at 12 warps to an SM (8 where a thread's
-// accumulators are 128), not by the gather: 6 to 9 TB/s, where row loads alone reach 16.  Three tables' kernels / this one, us:
-// d = 3, 32 heads of 2048 tokens 137 / 42, of 4096 163 / 77, 128 heads of 8192 917 / 550, 16 heads of 16 K 312 / 186, of 24 K
-// 529 / 333; d = 4, 32 heads of 4096 552 / 236; fp32 tables: d = 3, 32 heads of 5056 503 / 121; d = 2, 32 of 4160 238 / 32.
-// The first form, four warps to an item with the scores exchanged through shared memory, took 156 where this takes 77.
+// Bound by the instructions that a warp issues for a stage, about 300 one after the other at 12 warps to an SM (8 where a thread's
+// accumulators are 128), not by the gather: 7 to 12 TB/s, where row loads alone reach 16.  Three tables' kernels / this one, us:
+// d = 3, 32 heads of 2048 tokens 137 / 35, of 4096 163 / 61, 128 heads of 8192 917 / 420, 16 heads of 16 K 312 / 153, of 24 K
+// 529 / 267; d = 4, 32 heads of 4096 552 / 193; fp32 tables: d = 3, 32 heads of 5056 503 / 103; d = 2, 32 of 4160 238 / 34.
+// The first form, four warps to an item with the scores exchanged through shared memory, took 156 where this takes 61; with a
+// test for every kind of stage in front of each and all of Z in registers (spills) it was 77.
 template <int RT, bool DUAL, bool GATED, bool SPLIT>
 __global__ void __launch_bounds__(32 * LN_WARPS, LineSmem<RT, DUAL>::warps_per_sm / LN_WARPS)
 line_products_kernel(const __grid_constant__ LineParams p) {
@@ -218,10 +219,11 @@ line_products_kernel(const __grid_constant__ LineParams p) {
     return t < (int)p.n ? expf(edge - l[t]) : expf(l[t] - edge);
   };
 
-  // The loads: stage ls of item lit (0: X, then steps of 16 slots) goes to slot lslot of the ring.
-  uint32_t lit = it, ls = 0, lslot = 0;
+  // The loads, two stages ahead of the products: of item `la`, X or a step's 16 slots, into slot lslot of the ring.
+  uint32_t lslot = 0;
   Item la = item_at(it);
   LineOf line = line_of(p, la.g);
+  bool more = true;       // there is such an item
   Slot ntok{0, false};    // the lane's slot of the 32 that are being loaded
   float nfac = 0.f;
   uint32_t to[4];         // where the pieces of rows crow + 2 i go, i mod 4
@@ -229,48 +231,60 @@ line_products_kernel(const __grid_constant__ LineParams p) {
   for (int i = 0; i < 4; ++i) to[i] = ring + piece(crow + 2 * i, cpiece);
   int64_t head = (int64_t)la.bh * p.T * 128 + cpiece * 8;
   const __nv_bfloat16 *ly = p.y + head, *lz = p.z + head;
-  auto load = [&]() {
-    if (lit < p.items) {
-      if (ls == 0) {
-        const __nv_bfloat16 *lx = p.x1 + head, *lx2 = DUAL ? p.x2 + head : nullptr;
-        int mine = row_token(p, la.g, la.rb * (RT * 16) + lane);
-        if (mine < 0) mine = row_token(p, la.g, 0);   // (what comes of it is not stored)
+  auto load_rows = [&]() {
+    if (more) {
+      const __nv_bfloat16 *lx = p.x1 + head, *lx2 = DUAL ? p.x2 + head : nullptr;
+      int mine = row_token(p, la.g, la.rb * (RT * 16) + lane);
+      if (mine < 0) mine = row_token(p, la.g, 0);   // (what comes of it is not stored)
 #pragma unroll
-        for (int i = 0; i < RT * 8; ++i) {
-          const uint32_t t = __shfl_sync(0xffffffffu, mine, crow + 2 * i), dst = to[i & 3] + lslot * LN_STAGE + (i >> 2) * 2048;
-          cp_async16(dst, lx + (uint64_t)t * 128);
-          if (DUAL) cp_async16(dst + 4096, lx2 + (uint64_t)t * 128);
-        }
-      } else {
-        if (ls & 1) {
-          ntok = slot_token(p, line, (ls - 1) * LN_STEP + lane);
-          if (GATED) nfac = ntok.there ? factor(la.bh, (int)ntok.t) : 0.f;
-        }
-        const uint32_t from = crow + (ls & 1 ? 0 : 16);
-#pragma unroll
-        for (int i = 0; i < LN_STEP / 2; ++i) {
-          const uint32_t t = __shfl_sync(0xffffffffu, ntok.t, from + 2 * i), dst = to[i & 3] + lslot * LN_STAGE + (i >> 2) * 2048;
-          cp_async16(dst, ly + (uint64_t)t * 128);
-          cp_async16(dst + 4096, lz + (uint64_t)t * 128);
-        }
-      }
-      if (ls == p.steps) {
-        ls = 0;
-        lit += stride;
-        la = item_at(lit);
-        line = line_of(p, la.g);
-        head = (int64_t)la.bh * p.T * 128 + cpiece * 8;
-        ly = p.y + head;
-        lz = p.z + head;
-      } else {
-        ++ls;
+      for (int i = 0; i < RT * 8; ++i) {
+        const uint32_t t = __shfl_sync(0xffffffffu, mine, crow + 2 * i), dst = to[i & 3] + lslot * LN_STAGE + (i >> 2) * 2048;
+        cp_async16(dst, lx + (uint64_t)t * 128);
+        if (DUAL) cp_async16(dst + 4096, lx2 + (uint64_t)t * 128);
       }
     }
     cp_async_commit();
     lslot ^= 1;
   };
+  auto load_keys = [&](uint32_t step) {
+    if (!(step & 1)) {
+      ntok = slot_token(p, line, step * LN_STEP + lane);
+      if (GATED) nfac = ntok.there ? factor(la.bh, (int)ntok.t) : 0.f;
+    }
+    const uint32_t from = crow + (step & 1) * 16, stage = lslot * LN_STAGE;
 #pragma unroll
-  for (int i = 0; i < LN_STAGES; ++i) load();
+    for (int i = 0; i < LN_STEP / 2; ++i) {
+      const uint32_t t = __shfl_sync(0xffffffffu, ntok.t, from + 2 * i), dst = to[i & 3] + stage + (i >> 2) * 2048;
+      cp_async16(dst, ly + (uint64_t)t * 128);
+      cp_async16(dst + 4096, lz + (uint64_t)t * 128);
+    }
+    cp_async_commit();
+    lslot ^= 1;
+  };
+  // The stage behind step `step` of an item of p.steps: a step of the same one, X of the next one, or that one's first step.
+  auto load_behind = [&](uint32_t step) {
+    if (step < p.steps) {
+      load_keys(step);
+    } else if (step == p.steps) {
+      const uint32_t i = p.groups * p.blocks * la.bh + la.g * p.blocks + la.rb + stride;
+      more = i < p.items;
+      if (more) {
+        la = item_at(i);
+        line = line_of(p, la.g);
+        head = (int64_t)la.bh * p.T * 128 + cpiece * 8;
+        ly = p.y + head;
+        lz = p.z + head;
+      }
+      load_rows();
+    } else if (more) {
+      load_keys(0);
+    } else {
+      cp_async_commit();
+      lslot ^= 1;
+    }
+  };
+  load_rows();
+  load_keys(0);
 
   uint32_t slot = 0;
   // this lane's words for the scores of row g (two pieces in either half), and its row of the transposed tiles
@@ -279,7 +293,7 @@ line_products_kernel(const __grid_constant__ LineParams p) {
     lds16(s_at[i & 1] + off + (i >> 1) * 128, w);
   };
   while (true) {
-    const Item cur = item_at(it);
+    const Item cur = la;
     uint32_t xf[L::x_regs ? 2 : 1][16];
     cp_async_wait<LN_STAGES - 1>();
     __syncwarp();
@@ -302,7 +316,7 @@ line_products_kernel(const __grid_constant__ LineParams p) {
             }
           }
       __syncwarp();
-      load();
+      load_behind(1);
       slot ^= 1;
     }
     float acc[NX][RT][16][4];
@@ -400,29 +414,29 @@ line_products_kernel(const __grid_constant__ LineParams p) {
       }
 #pragma unroll
       for (int o = 0; o < NX; ++o) {
-        uint32_t b[8][4];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) ldsm4_trans((o_at + tile + (1 - o) * 4096) ^ (j << 5), b[j]);
-        if (o + 1 == NX) {
-          __syncwarp();   // every lane has what it needs of the slot
-          load();
-          slot ^= 1;
-        }
+        for (int j = 0; j < 8; j += 4) {   // (half of the columns at a time: all of Z at once would spill)
+          uint32_t b[4][4];
 #pragma unroll
-        for (int j = 0; j < 8; j += 2) {
+          for (int c = 0; c < 4; ++c) ldsm4_trans((o_at + tile + (1 - o) * 4096) ^ ((j + c) << 5), b[c]);
+          if (o + 1 == NX && j == 4) {
+            __syncwarp();   // every lane has what it needs of the slot
+            load_behind(s + 2);
+            slot ^= 1;
+          }
 #pragma unroll
           for (int rt = 0; rt < RT; ++rt)
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
-              mma16816(acc[o][rt][2 * j + c], ph[o][rt][0], ph[o][rt][1], ph[o][rt][2], ph[o][rt][3], b[j + c / 2][2 * (c & 1)],
-                       b[j + c / 2][2 * (c & 1) + 1]);
+            for (int c = 0; c < 8; ++c)
+              mma16816(acc[o][rt][2 * j + c], ph[o][rt][0], ph[o][rt][1], ph[o][rt][2], ph[o][rt][3], b[c / 2][2 * (c & 1)],
+                       b[c / 2][2 * (c & 1) + 1]);
           if (SPLIT)
 #pragma unroll
             for (int rt = 0; rt < RT; ++rt)
 #pragma unroll
-              for (int c = 0; c < 4; ++c)
-                mma16816(acc[o][rt][2 * j + c], pl[o][rt][0], pl[o][rt][1], pl[o][rt][2], pl[o][rt][3], b[j + c / 2][2 * (c & 1)],
-                         b[j + c / 2][2 * (c & 1) + 1]);
+              for (int c = 0; c < 8; ++c)
+                mma16816(acc[o][rt][2 * j + c], pl[o][rt][0], pl[o][rt][1], pl[o][rt][2], pl[o][rt][3], b[c / 2][2 * (c & 1)],
+                         b[c / 2][2 * (c & 1) + 1]);
         }
       }
     }
@@ -593,8 +607,8 @@ cudaError_t smat_launch_line_products(const SmatLineArgs& a, const SmatGeo& geo,
   }
   if (line_shape(geo, bh, a.rows_are_types).rt == 1) {
     if (a.lam) return launch_lines<1, false, true, false>(p, st);
-    return a.out_f32 ? launch_lines<1, false, false, true>(p, st) : launch_lines<1, false, false, false>(p, st);
+    return a.split ? launch_lines<1, false, false, true>(p, st) : launch_lines<1, false, false, false>(p, st);
   }
   if (a.lam) return launch_lines<2, false, true, false>(p, st);
-  return a.out_f32 ? launch_lines<2, false, false, true>(p, st) : launch_lines<2, false, false, false>(p, st);
+  return a.split ? launch_lines<2, false, false, true>(p, st) : launch_lines<2, false, false, false>(p, st);
 }
