@@ -540,10 +540,11 @@ smat_status smat_plan_create(smat_plan** out, int batch, int heads, int64_t T, i
   pl->ubar_tc = pl->tc && !g.dense_G && (pl->tab_tc || g.m / g.B >= 12);
   pl->ubar_bf16 = pl->ubar_tc && ((g.D == 1 && fbar_by_read) || pl->tab_tc);   // d = 2: F̄ is Ū itself
   pl->fbar_bf16 = pl->tc && !g.dense_G && (pl->tab_tc || (g.D == 1 ? pl->ubar_bf16 : fbar_by_read));
-  // The flags that ask for a tabulation ask for tables.
+  // The flags that ask for a tabulation ask for tables; the plan inside a gated one (per-tile states) serves both passes.
   const bool lines_by_flag = !(flags & (SMAT_FLAG_ALG2_TABULATION | SMAT_FLAG_ALU_TABULATION | SMAT_FLAG_D3_SHARED_SUMS));
   pl->lines = lines_by_flag && ((pl->tc && pl->u_bf16 && pl->fbar_bf16) || pl->ragged_tc) &&
-              smat_lines_pay(g, pl->bh, pl->ragged_tc ? 4 : 2);
+              smat_lines_pay(g, pl->bh, pl->ragged_tc ? 4 : 2,
+                             !pl->ragged_tc && (flags & (SMAT_FLAG_KEEP_FORWARD_TABLES | SMAT_FLAG_PER_TILE_STATES)) != 0);
   // Workspace regions, each sized for the element type the plan stores there.  Tensor-core plans keep the causal
   // states per 128-token tile in bf16 (or, in the two-level form, fewer fp32 segment states in the same region); the
   // fp32-ALU plans keep one fp32 state per chunk.

@@ -302,9 +302,10 @@ struct SmatLineArgs {
   int* mark;             // null, or a word that is set to mark_value
   int mark_value;
 };
-// Whether the kernel takes the shape, and whether it is the faster way (table_bytes: of an entry of the tables otherwise).
+// Whether the kernel takes the shape, and whether it is the faster way (table_bytes: of an entry of the tables otherwise; trains: a
+// backward follows every forward).
 bool smat_lines_supported(const SmatGeo& geo, int bh);
-bool smat_lines_pay(const SmatGeo& geo, int bh, int table_bytes);
+bool smat_lines_pay(const SmatGeo& geo, int bh, int table_bytes, bool trains);
 // F (types = 0) or U of a pass of a plan that may have formed no tables, as fp32: from K and V that it left where *mark says (1:
 // beside, 2: behind), or from `table` where *mark is zero.
 cudaError_t smat_launch_line_tables(const SmatGeo& geo, int bh, const int* mark, const void* beside, const void* behind,

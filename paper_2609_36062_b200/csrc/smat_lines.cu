@@ -22,8 +22,8 @@ namespace {
 
 using namespace tc;
 
-constexpr int LN_WARPS = 2, LN_STEP = 16;                          // warps of a CTA; gathered rows per step
-constexpr int LN_STAGES = 2, LN_STAGE = 2 * LN_STEP * 256;         // stages of a warp's ring (line_products_kernel counts on two), their bytes
+constexpr int LN_STEP = 16;                                  // gathered rows per step
+constexpr int LN_STAGES = 2, LN_STAGE = 2 * LN_STEP * 256;   // stages of the ring (line_products_kernel counts on two), their bytes
 
 struct LineParams {
   const __nv_bfloat16 *x1, *x2, *y, *z;   // [bh][T][128]
@@ -163,44 +163,43 @@ __device__ __forceinline__ void mma16816_first(float (&c)[4], uint32_t a0, uint3
 }
 
 // 16-byte piece c of row r in a tile of 256-byte rows: pieces 2 q of rows 2 k and 2 k + 1 lie in different bank groups, and so do
-// piece c of rows 0 to 7
+// piece c of rows 0 to 7.  (Rows 272 bytes apart need no exclusive or, but a sector then lands across two: 109 us for 120.)
 __device__ __forceinline__ uint32_t piece(uint32_t r, uint32_t c) { return r * 256 + ((c ^ (r & 7)) << 4); }
 
 template <int RT, bool DUAL>
 struct LineSmem {
   static constexpr bool x_regs = RT * (1 + DUAL) == 1;
   static constexpr int warps_per_sm = x_regs ? 12 : 8;
-  static constexpr int x_bytes = x_regs ? 0 : RT * (1 + DUAL) * 4096, warp_bytes = LN_STAGES * LN_STAGE + x_bytes;
+  static constexpr int x_bytes = x_regs ? 0 : RT * (1 + DUAL) * 4096, bytes = LN_STAGES * LN_STAGE + x_bytes;
 };
 
-// A warp takes an item (16 RT rows of a row group) from beginning to end, with a ring of its own in shared memory: no barriers.
+// A CTA is one warp (what is the same for all of it stays in uniform registers; with two to a CTA 3 to 5 % more) and takes an item (16 RT
+// rows of a row group) from beginning to end, with a ring of its own in shared memory: no barriers.
 // Stages of the ring: X of an item, then 16 gathered rows of Y and Z after the other.  Lane (g, q) = (lane / 4, lane % 4) of the
 // matrix instructions:
 //   scores   its words of a row are bytes 32 q to 32 q + 31 of either half: the order of the contracted index is free, as
 //            long as X and Y have the same
 //   outputs  the rows of Z transposed on the way from shared memory (ldmatrix)
-// Bound by the instructions that a warp issues for a stage, about 300 one after the other at 12 warps to an SM (8 where a thread's
+// Bound by the instructions that a warp issues for a stage, about 290 one after the other at 12 warps to an SM (8 where a thread's
 // accumulators are 128), not by the gather: 7 to 12 TB/s, where row loads alone reach 16.  Three tables' kernels / this one, us:
-// d = 3, 32 heads of 2048 tokens 137 / 35, of 4096 163 / 61, 128 heads of 8192 917 / 420, 16 heads of 16 K 312 / 153, of 24 K
-// 529 / 267; d = 4, 32 heads of 4096 552 / 193; fp32 tables: d = 3, 32 heads of 5056 503 / 103; d = 2, 32 of 4160 238 / 34.
-// The first form, four warps to an item with the scores exchanged through shared memory, took 156 where this takes 61; with a
+// d = 3, 32 heads of 2048 tokens 137 / 33, of 4096 163 / 57, 128 heads of 8192 917 / 410, 16 heads of 16 K 312 / 147, of 24 K
+// 529 / 255; d = 4, 32 heads of 4096 552 / 190; fp32 tables: d = 3, 32 heads of 5056 503 / 95; d = 2, 32 of 4160 238 / 33.
+// The first form, four warps to an item with the scores exchanged through shared memory, took 156 where this takes 57; with a
 // test for every kind of stage in front of each and all of Z in registers (spills) it was 77.
 template <int RT, bool DUAL, bool GATED, bool SPLIT>
-__global__ void __launch_bounds__(32 * LN_WARPS, LineSmem<RT, DUAL>::warps_per_sm / LN_WARPS)
+__global__ void __launch_bounds__(32, LineSmem<RT, DUAL>::warps_per_sm)
 line_products_kernel(const __grid_constant__ LineParams p) {
   using L = LineSmem<RT, DUAL>;
   constexpr int NX = 1 + DUAL;
   extern __shared__ __align__(1024) uint8_t smem[];
-  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
-  const uint32_t stride = gridDim.x * LN_WARPS;
-  const uint32_t ring = smem_u32(smem) + warp * L::warp_bytes, xs = ring + LN_STAGES * LN_STAGE + lane * 16;
+  const uint32_t lane = threadIdx.x, g = lane >> 2, q = lane & 3;
+  const uint32_t ring = smem_u32(smem), xs = ring + LN_STAGES * LN_STAGE + lane * 16;
   const uint32_t crow = lane >> 4, cpiece = lane & 15;   // pieces that a lane copies: rows crow + 2 i
 
   pdl_trigger();
   pdl_wait();
   if (p.mark && blockIdx.x == 0 && threadIdx.x == 0) *p.mark = p.mark_value;
-  uint32_t it = blockIdx.x * LN_WARPS + warp;
-  if (it >= p.items) return;
+  uint32_t it = blockIdx.x;
 
   struct Item {
     uint32_t g, rb, bh;
@@ -266,7 +265,7 @@ line_products_kernel(const __grid_constant__ LineParams p) {
     if (step < p.steps) {
       load_keys(step);
     } else if (step == p.steps) {
-      const uint32_t i = p.groups * p.blocks * la.bh + la.g * p.blocks + la.rb + stride;
+      const uint32_t i = p.groups * p.blocks * la.bh + la.g * p.blocks + la.rb + gridDim.x;
       more = i < p.items;
       if (more) {
         la = item_at(i);
@@ -465,7 +464,7 @@ line_products_kernel(const __grid_constant__ LineParams p) {
           }
         }
       }
-    it += stride;
+    it += gridDim.x;
     if (it >= p.items) break;
   }
 }
@@ -473,13 +472,12 @@ line_products_kernel(const __grid_constant__ LineParams p) {
 template <int RT, bool DUAL, bool GATED, bool SPLIT>
 cudaError_t launch_lines(const LineParams& p, cudaStream_t st) {
   using L = LineSmem<RT, DUAL>;
-  constexpr int bytes = LN_WARPS * L::warp_bytes;
-  static_assert((L::warps_per_sm / LN_WARPS) * (bytes + 1024) <= 228 * 1024, "the rings of an SM");
+  static_assert(L::warps_per_sm * (L::bytes + 1024) <= 228 * 1024, "the rings of an SM");
   auto* kernel = line_products_kernel<RT, DUAL, GATED, SPLIT>;
-  const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::bytes);
   if (err != cudaSuccess) return err;
-  const uint32_t most = (uint32_t)smat_sm_count() * (L::warps_per_sm / LN_WARPS), ctas = (p.items + LN_WARPS - 1) / LN_WARPS;
-  return smat_launch_pdl(kernel, dim3(ctas < most ? ctas : most), 32 * LN_WARPS, bytes, st, p);
+  const uint32_t most = (uint32_t)smat_sm_count() * L::warps_per_sm;
+  return smat_launch_pdl(kernel, dim3(p.items < most ? p.items : most), 32, (size_t)L::bytes, st, p);
 }
 
 struct LineShape {
@@ -512,20 +510,23 @@ bool smat_lines_supported(const SmatGeo& geo, int bh) {
   return true;
 }
 
-// The line lies where the gathered bytes (from the L2 cache) pass the tables' (to and from memory) by three quarters, long-range
-// stages in us, tables / here: d = 3, q = 29, 16 heads, ratio 1.7 (24 K tokens) 529 / 333, 2.1 (28 K) 535 / 494, 2.3 (32 K) 541 / 553;
-// d = 4, q = 11, 16 heads, 1.5 (7168) 550 / 472, 2.0 (8192) 556 / 624; fp32 tables, d = 4, 1.7 (16,320) 1270 / 1213.  bf16 and d = 2:
-// one table, and its pooling and read are near the memory rate; 32 heads, 0.7 (4096) 41 / 29 and the training step 250 / 235, 16
-// heads, 0.8 (6144), the training step 210.7 / 214.5.  Types of less than two tokens leave the row tile empty: 16 heads of 5376, d = 4
-// (1.8) 587 / 580 for the pass.  And a warp takes an item from beginning to end: there have to be items for half of the chip's
-// warps (d = 3, 2 heads of 4096 tokens, 364 items, 44.4 / 46.1 for the pass; 8 of 2048, 1056 items, 66 / 42).
-bool smat_lines_pay(const SmatGeo& geo, int bh, int table_bytes) {
-  constexpr uint64_t HALF_THE_WARPS = 148 * 6;
+// The line lies where the gathered bytes (from the L2 cache) pass the tables' (to and from memory) by a limit; the pass in us, with
+// tables / without.  Forward 2.3: d = 3, q = 29, 16 heads, ratio 1.7 (24 K tokens) 648 / 387, 2.1 (28 K) 673 / 607, 2.3 (32 K) 696 / 677, 2.9
+// (40 K) 765 / 850; d = 4, q = 11, 16 heads, 2.0 (10,240) 608 / 536, 2.5 (12,288) 615 / 643.  Plans made for training steps 1.75, since dK
+// and dV take two products of a gather: d = 4, 8 heads, 1.5 (7168) 845 / 751, 2.0 (8192) 851 / 876, gated 974 / 1019.  d = 2 with a bf16
+// table 0.75: there is one, and its pooling and read are near the memory rate; 32 heads, 0.7 (4096) 85 / 83 and the training step
+// 250 / 237, 16 heads, 0.8 (6144), the training step 210.7 / 214.5.  Types of less than two tokens leave the row tile empty: 16
+// heads of 5376, d = 4 (1.8) 587 / 580.
+// Items, a warp each: one to an SM, but with bf16 tables half of the warps that the chip runs, for routed calls form tables, and in
+// batches of a few heads positional arrays give the same bits as positions (2 heads of 4096 tokens, d = 3, 45 / 39).
+bool smat_lines_pay(const SmatGeo& geo, int bh, int table_bytes, bool trains) {
+  constexpr uint64_t SMS = 148;
   if (!smat_lines_supported(geo, bh) || 2 * geo.B > geo.m) return false;
   const LineShape s = line_shape(geo, bh, 1);
   const double gathered = (double)s.groups * s.blocks * s.slots * 512;
   const double tables = 2.0 * (double)(geo.P + (geo.D == 1 ? 0 : geo.B)) * 16384 * table_bytes;
-  return (uint64_t)bh * s.groups >= HALF_THE_WARPS && gathered <= (geo.D == 1 && table_bytes == 2 ? 0.75 : 1.75) * tables;
+  const double limit = geo.D == 1 && table_bytes == 2 ? 0.75 : trains ? 1.75 : 2.3;
+  return s.items >= (table_bytes == 2 ? 6 * SMS : SMS) && gathered <= limit * tables;
 }
 
 namespace {
