@@ -353,7 +353,7 @@ bool scan_beside_read(const Ctx& cx) {
 struct Segments {
   int nseg0 = 0, nseg1 = 0;
 };
-Segments segment_totals(Ctx& cx, const void* K, const void* V, int64_t rows0, int64_t rows1, int L) {
+Segments segment_totals(Ctx& cx, const void* K, const void* V, int64_t rows0, int64_t rows1, int L, bool ones = false) {
   const smat_plan* pl = cx.pl;
   const int64_t tiles0 = (rows0 + 127) / 128, tiles1 = (rows1 + 127) / 128;
   float* seg = cx.f(pl->off_sin);
@@ -361,7 +361,7 @@ Segments segment_totals(Ctx& cx, const void* K, const void* V, int64_t rows0, in
   smat_segment_counts(tiles0, tiles1, pl->bh, L, &s.nseg0, &s.nseg1);
   if (s.nseg0 > 1 || s.nseg1 > 1)
     SMAT_TRY(cx, "segment_state_tc", smat_launch_segment_state_tc(K, V, seg, rows0, rows1, s.nseg0, s.nseg1, pl->bh,
-                                                                  reinterpret_cast<int*>(cx.ws + pl->off_status), cx.st));
+                                                                  reinterpret_cast<int*>(cx.ws + pl->off_status), cx.st, ones));
   if (smat_segments_need_scan(s.nseg0, s.nseg1)) {
     SmatScanArgs a{};
     a.jobs = 1;
@@ -726,6 +726,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     const bool per_tile = (pl->flags & SMAT_FLAG_PER_TILE_STATES) != 0, f32 = forward_rows_f32(pl);
     if (lines) {                                                                             // steps 2-4 in one
       SmatLineArgs a = line_job(1, Q, K, V, ylr, f32, pl->geo.D == 1);
+      a.ones = divide;
       pl->forward_left = f32 ? LINE_COPY_BESIDE : LINE_COPY_BEHIND;
       line_copy(cx, &a, pl->forward_left, false);
       line_mark(cx, &a, pl->forward_left);
@@ -744,7 +745,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     if (!per_tile) {  // steps 5-7, two-level: segment totals, scan of the totals, fused per-segment output
       const int64_t rows0 = tiles0 * 128, rows1 = tiles1 * 128;
       const int L = smat_segment_tiles(tiles0, tiles1, pl->bh);
-      const Segments sg = segment_totals(cx, K, V, rows0, rows1, L < 2 ? 2 : L);
+      const Segments sg = segment_totals(cx, K, V, rows0, rows1, L < 2 ? 2 : L, divide);
       const bool keep = (pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES) != 0;   // a backward will want the per-tile states
       SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, cx.f(pl->off_sin), ylr, f32, 0, lr ? pl->geo.n : pl->T, O,
                                                                        rows0, rows1, sg.nseg0, sg.nseg1, pl->bh, status, cx.st,
@@ -770,6 +771,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     const int64_t rows0 = lr ? pl->geo.n : pl->T, rows1 = lr ? pl->geo.m : 0;
     if (pl->lines && !cx.routed) {
       SmatLineArgs a = line_job(1, Q, K, V, ylr, 1, 1);
+      a.ones = divide;
       line_copy(cx, &a, LINE_COPY_BESIDE, false);
       line_mark(cx, &a, LINE_COPY_BESIDE);
       line_rows(cx, "read_lines", a);
@@ -778,7 +780,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
       zero_unrouted(cx, SMAT_GM_TYPE, ylr, 512);
       state_read(cx, "read_type", {read_job(cx, SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, ylr)});
     }
-    const Segments sg = segment_totals(cx, K, V, rows0, rows1, 2);
+    const Segments sg = segment_totals(cx, K, V, rows0, rows1, 2, divide);
     SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, cx.f(pl->off_sin), ylr, 1, 1, lr ? pl->geo.n : pl->T, O, rows0,
                                                                      rows1, sg.nseg0, sg.nseg1, pl->bh, status, cx.st, nullptr,
                                                                      divide));
@@ -1156,19 +1158,22 @@ smat_status smat_forward_normalized(const smat_plan* pl, const void* Q, const vo
   if (!device_ok()) return SMAT_ERR_ARCH;
   const int bf = pl->dtype == SMAT_BF16;
   const int64_t rows = (int64_t)pl->bh * pl->T;
-  // v̄ = [v; 1]: the last value column is the normaliser column (Eq. "augmented-kv-state")
-  if (smat_launch_normalize_step(0, V, nullptr, ws + pl->off_nv, bf, pl->p, rows, st) != cudaSuccess) return SMAT_ERR_LAUNCH;
   // The single final division (Eq. "augmented-attention-output"): by the output kernel of the two-level branch, before the rows
   // are rounded, or by a kernel of its own (32 heads of 5056 tokens, d = 3: 231 us a pass, 248; 16 of 13,056, d = 2: 177,
   // 209), also where O is an operand's array, which others may still read.
   const size_t bytes = (size_t)rows * 256;
   const bool divides = (pl->tc || pl->ragged_tc) && !(pl->flags & SMAT_FLAG_PER_TILE_STATES) && !smat_overlap(O, bytes, Q, bytes) &&
-                       !smat_overlap(O, bytes, K, bytes);
-  smat_status s = forward_impl(pl, Q, K, ws + pl->off_nv, divides ? O : ws + pl->off_ny, nullptr, nullptr, workspace,
+                       !smat_overlap(O, bytes, K, bytes) && !smat_overlap(O, bytes, V, bytes);
+  // v̄ = [v; 1]: the last value column is the normaliser column (Eq. "augmented-kv-state").  The output kernel, the totals and
+  // the rows without tables set it in the tiles that they load; tables are pooled from a copy (the first of these
+  // passes with the copy 199, now 171; d = 1, 16 heads of 32 K, 239, 169).
+  const bool copies = !divides || !(pl->lines || pl->geo.dense_G);
+  if (copies && smat_launch_normalize_step(0, V, nullptr, ws + pl->off_nv, bf, pl->p, rows, st) != cudaSuccess) return SMAT_ERR_LAUNCH;
+  smat_status s = forward_impl(pl, Q, K, copies ? ws + pl->off_nv : V, divides ? O : ws + pl->off_ny, nullptr, nullptr, workspace,
                                workspace_bytes, cuda_stream, divides);
   if (s != SMAT_OK) return s;
   if (divides) {
-    pl->launches += 1;
+    pl->launches += copies;
     return SMAT_OK;
   }
   if (smat_launch_normalize_step(1, ws + pl->off_ny, nullptr, O, bf, pl->p, rows, st) != cudaSuccess) return SMAT_ERR_LAUNCH;

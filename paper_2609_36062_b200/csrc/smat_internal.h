@@ -279,10 +279,10 @@ int smat_segment_tiles(int64_t tiles_block0, int64_t tiles_block1, int bh);
 void smat_segment_counts(int64_t tiles0, int64_t tiles1, int bh, int L, int* nseg0, int* nseg1);
 bool smat_segments_need_scan(int nseg0, int nseg1);
 cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* totals, int64_t rows0, int64_t rows1,
-                                         int nseg0, int nseg1, int bh, int* status, cudaStream_t st);
+                                         int nseg0, int nseg1, int bh, int* status, cudaStream_t st, int ones = 0);
 // ylr_f32: the long-range rows are fp32 (else bf16).  split: any blocks (else of whole tiles), and the state and the scores enter
 // their products as a bf16 part plus a bf16 remainder (with fp32 rows only).  divide: the rows leave divided by their last column,
-// which stays as it is.
+// which stays as it is, and V's last column counts as one (as in the totals with `ones`).
 cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const void* V, const float* seg_in,
                                           const void* ylr, int ylr_f32, int split, int64_t n_lr, void* O, int64_t rows0, int64_t rows1,
                                           int nseg0, int nseg1, int bh, int* status, cudaStream_t st,
@@ -294,6 +294,7 @@ struct SmatLineArgs {
   const void *x1, *x2, *y, *z;
   void *out1, *out2;
   int out_f32, rows_are_types;
+  int ones;              // Z's last column counts as one (one product, ungated)
   int split;             // scores enter their products as a bf16 part plus a bf16 remainder (one product, ungated)
   const float* lam;      // gated: prefix sums of the log-gates; terms are multiplied by exp(λ_recent - λ_distant)
   void* copy;            // null, or where K and V of every distant token are left side by side: token t of head b at

@@ -43,7 +43,7 @@ struct LineParams {
   uint32_t groups, blocks, lines, slots, steps;   // row groups of a head, row blocks of a group, gathered groups of a group
   uint32_t full_steps;                            // steps before the first that has a slot without a token
   uint32_t items;
-  int rows_are_types, out_f32;
+  int rows_are_types, out_f32, ones;
 };
 
 __device__ __forceinline__ uint32_t div_q(const LineParams& p, uint32_t v) { return __umulhi(v, p.q_inv); }
@@ -408,6 +408,7 @@ line_products_kernel(const __grid_constant__ LineParams p) {
           lds16(ring + tile + piece(r, cpiece), w);
           dst[p.copy_swap ? 16 : 0] = make_uint4(w[0], w[1], w[2], w[3]);
           lds16(ring + tile + 4096 + piece(r, cpiece), w);
+          if (p.ones && cpiece == 15) w[3] = __byte_perm(w[3], 0x3f800000u, 0x7610);
           dst[p.copy_swap ? 0 : 16] = make_uint4(w[0], w[1], w[2], w[3]);
         }
       }
@@ -418,6 +419,7 @@ line_products_kernel(const __grid_constant__ LineParams p) {
           uint32_t b[4][4];
 #pragma unroll
           for (int c = 0; c < 4; ++c) ldsm4_trans((o_at + tile + (1 - o) * 4096) ^ ((j + c) << 5), b[c]);
+          if (!DUAL && !GATED && j == 4 && p.ones && g == 7) b[3][2] = b[3][3] = 0x3f803f80u;   // column 127 of both keys of a register
           if (o + 1 == NX && j == 4) {
             __syncwarp();   // every lane has what it needs of the slot
             load_behind(s + 2);
@@ -600,7 +602,7 @@ cudaError_t smat_launch_line_products(const SmatLineArgs& a, const SmatGeo& geo,
   LineParams p = line_geometry(geo, line_shape(geo, bh, a.rows_are_types, a.out2 != nullptr), a.rows_are_types);
   using B16 = const __nv_bfloat16;
   p.x1 = static_cast<B16*>(a.x1); p.x2 = static_cast<B16*>(a.x2); p.y = static_cast<B16*>(a.y); p.z = static_cast<B16*>(a.z);
-  p.out1 = a.out1; p.out2 = a.out2; p.out_f32 = a.out_f32;
+  p.out1 = a.out1; p.out2 = a.out2; p.out_f32 = a.out_f32; p.ones = a.ones;
   p.copy = static_cast<__nv_bfloat16*>(a.copy); p.copy_head = a.copy_head; p.copy_swap = a.copy_swap; p.mark = a.mark; p.mark_value = a.mark_value;
   p.lam = a.lam;
   if (a.out2) {

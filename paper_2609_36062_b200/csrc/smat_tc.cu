@@ -834,7 +834,18 @@ __device__ __forceinline__ void seg_range(const SegCut& c, int seg, int64_t* til
   }
 }
 
+// Normalised output: the last value column is one, whatever the caller left there.  A warp sets it in a V tile that has landed
+// (two 64-column boxes, 128-byte swizzle); the products wait for it.
+__device__ __forceinline__ void set_ones_column(uint8_t* v_tile, int lane) {
+#pragma unroll
+  for (int r = lane; r < TILE; r += 32)
+    *reinterpret_cast<__nv_bfloat16*>(v_tile + BOX_BYTES + r * 128 + ((7 ^ (r & 7)) << 4) + 14) = __float2bfloat16_rn(1.0f);
+  fence_proxy_async();
+  __syncwarp();
+}
+
 struct SegStateParams {
+  int ones;              // V's last column counts as one
   int64_t T;
   SegCut cut;
   int nseg;              // segments per head
@@ -850,7 +861,8 @@ __global__ void __launch_bounds__(192) segment_state_tc_kernel(const __grid_cons
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SEG_STATE_STAGES * 4 * BOX_BYTES);
   uint64_t* full = bars;
   uint64_t* empty = bars + SEG_STATE_STAGES;
-  uint64_t* done = empty + SEG_STATE_STAGES;
+  uint64_t* ones = empty + SEG_STATE_STAGES;   // [SEG_STATE_STAGES] V's last column set (prm.ones)
+  uint64_t* done = ones + SEG_STATE_STAGES;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -863,7 +875,7 @@ __global__ void __launch_bounds__(192) segment_state_tc_kernel(const __grid_cons
   const WaitCtx wc{cta_abort, prm.status};
   if (threadIdx.x == 0) {
     *cta_abort = 0;
-    for (int s = 0; s < SEG_STATE_STAGES; ++s) { mbar_init(full + s, 1); mbar_init(empty + s, 1); }
+    for (int s = 0; s < SEG_STATE_STAGES; ++s) { mbar_init(full + s, 1); mbar_init(empty + s, 1); mbar_init(ones + s, 1); }
     mbar_init(done, 1);
     fence_barrier_init();
   }
@@ -894,7 +906,7 @@ __global__ void __launch_bounds__(192) segment_state_tc_kernel(const __grid_cons
     bool ok = true;
     for (int it = 0; it < Lc && ok; ++it) {
       const int s = it % SEG_STATE_STAGES;
-      ok = mbar_wait(full + s, (it / SEG_STATE_STAGES) & 1, wc);
+      ok = mbar_wait((prm.ones ? ones : full) + s, (it / SEG_STATE_STAGES) & 1, wc);
       if (!ok) break;
       fence_after_sync();
       const uint32_t sK = smem_u32(smem + s * 4 * BOX_BYTES);
@@ -907,6 +919,12 @@ __global__ void __launch_bounds__(192) segment_state_tc_kernel(const __grid_cons
     }
     if (ok) mma_commit(done);
   } else if (warp < 4) {
+    for (int it = 0; prm.ones && warp == 0 && it < Lc; ++it) {
+      const int s = it % SEG_STATE_STAGES;
+      if (!mbar_wait_warp(full + s, (it / SEG_STATE_STAGES) & 1, wc)) break;
+      set_ones_column(smem + s * 4 * BOX_BYTES + 2 * BOX_BYTES, lane);
+      if (lane == 0) mbar_arrive(ones + s);
+    }
     if (mbar_wait_warp(done, 0, wc)) {
       fence_after_sync();
       const int i = warp * 32 + lane;
@@ -963,7 +981,7 @@ struct SegOutParams {
 
 // One CTA per (segment, head), all 128 output columns.
 //   warps 0-15 : each owns 32 rows x 32 columns of every TMEM tile (state, scores, output)
-//   warp 16    : TMA producer;   warp 17 : MMA issuer
+//   warp 16    : TMA producer;   warp 17 : MMA issuer;   warp 18 (DIVIDE) : sets V's last column
 // TMEM columns: running state S [0,128), scores [128,256), two output accumulators [256,384) and [384,512).
 // Per tile b, in issue order:  O = Q S_b ; S += Kᵀ V ; (next tile's) Sc = Q Kᵀ ; O += tril(Sc_b) V.
 // The state's own chain — publish S_b, Q S and Kᵀ V, read S_{b+1} back — does not wait for the score tile: while the
@@ -985,7 +1003,7 @@ struct SegOutMaps {
 };
 
 template <bool SPLIT, bool Y32, bool DIVIDE>
-__global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(const __grid_constant__ SegOutMaps maps,
+__global__ void __launch_bounds__(SEG_OUT_THREADS + 32 * DIVIDE) segment_output_tc_kernel(const __grid_constant__ SegOutMaps maps,
                                                                             const SegOutParams prm) {
   using Lay = SegOutLayout<SPLIT>;
   extern __shared__ uint8_t smem_raw[];
@@ -1003,7 +1021,8 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
   uint64_t* bar_p = bars + 10;     // P written (one arrival per warp)
   uint64_t* bar_o = bars + 11;     // output complete
   uint64_t* bar_n = bars + 12;     // [4] normalisers of the tile's row quarter written
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
+  uint64_t* bar_ones = bars + 16;  // [2] DIVIDE: V's last column set
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 18);
   volatile int* cta_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float* norm = reinterpret_cast<float*>(smem + Lay::NORM);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1020,6 +1039,7 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
     mbar_init(bar_s, SEG_EPI_WARPS); mbar_init(bar_sc, 1); mbar_init(bar_scr, SEG_EPI_WARPS); mbar_init(bar_qk, 1);
     mbar_init(bar_p, SEG_EPI_WARPS); mbar_init(bar_o, 1);
     for (int i = 0; i < 4; ++i) mbar_init(bar_n + i, 1);
+    mbar_init(bar_ones, 1); mbar_init(bar_ones + 1, 1);
     fence_barrier_init();
   }
   if (warp == SEG_EPI_WARPS) tmem_alloc(tmem_slot, 512);
@@ -1102,7 +1122,9 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
 #pragma unroll
         for (int kk = 0; kk < TILE / 16; ++kk)   // ... plus Q times the state's remainder
           mma_bf16(tmem_o, qk + (uint64_t)((kk >> 2) * BOX16 + (kk & 3) * 2), dS_mn + (uint64_t)(2 * BOX16 + kk * 128), idesc_o, 1);
-        ok = mbar_wait(vfull, it & 1, wc);
+      }
+      if (SPLIT || DIVIDE) {
+        ok = SPLIT ? mbar_wait(DIVIDE ? bar_ones : vfull, it & 1, wc) : mbar_wait(bar_ones + s, (it >> 1) & 1, wc);
         if (!ok) break;
         fence_after_sync();
       }
@@ -1133,6 +1155,13 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS) segment_output_tc_kernel(cons
       mma_commit(empty + s);
       mma_commit(bar_o);
       if (it + 1 < Lc && !early) ok = scores(it + 1);
+    }
+  } else if (DIVIDE && warp == SEG_EPI_WARPS + 2) {
+    for (int it = 0; it < Lc; ++it) {
+      const int s = SPLIT ? 0 : it & 1;
+      if (!(SPLIT ? mbar_wait_warp(vfull, it & 1, wc) : mbar_wait_warp(full + s, (it >> 1) & 1, wc))) break;
+      set_ones_column(smem + Lay::V + s * Lay::V_STRIDE, lane);
+      if (lane == 0) mbar_arrive(bar_ones + s);
     }
   } else if (warp < SEG_EPI_WARPS) {
     // Sixteen warps: warp w owns the lane quarter w % 4 (32 rows) and the column quarter w / 4 (32 columns) of every
@@ -2068,12 +2097,12 @@ static SegCut segment_cut(int64_t rows0, int64_t rows1, int nseg0, int nseg1) {
 bool smat_segments_need_scan(int nseg0, int nseg1) { return nseg0 > 2 || nseg1 > 2; }
 
 cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* totals, int64_t rows0, int64_t rows1,
-                                         int nseg0, int nseg1, int bh, int* status, cudaStream_t st) {
+                                         int nseg0, int nseg1, int bh, int* status, cudaStream_t st, int ones) {
   const int64_t T = rows0 + rows1;
   CUtensorMap tmK, tmV;
   if (!make_map(&tmK, K, (uint64_t)bh * T) || !make_map(&tmV, V, (uint64_t)bh * T)) return cudaErrorInvalidValue;
   SegStateParams prm;
-  prm.T = T; prm.nseg = nseg0 + nseg1; prm.totals = totals; prm.status = status;
+  prm.ones = ones; prm.T = T; prm.nseg = nseg0 + nseg1; prm.totals = totals; prm.status = status;
   prm.cut = segment_cut(rows0, rows1, nseg0, nseg1);
   cudaError_t err =
       cudaFuncSetAttribute(segment_state_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SEG_STATE_SMEM);
@@ -2111,5 +2140,5 @@ cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const vo
   cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
   dim3 grid((unsigned)prm.nseg, (unsigned)bh);
-  return smat_launch_pdl(kernel, grid, SEG_OUT_THREADS, smem, st, maps, prm);
+  return smat_launch_pdl(kernel, grid, SEG_OUT_THREADS + (divide ? 32 : 0), smem, st, maps, prm);
 }

@@ -1,6 +1,8 @@
-"""The division of the normalised output by the output kernel, against the fp64 oracle: blocks of one tile, of even and odd numbers
-of tiles, partial last tiles, several segments; and by its own kernel, where O is an operand's array."""
+"""The division of the normalised output by the output kernel, and V's ones column set where V is consumed, against the fp64 oracle:
+blocks of one tile, of even and odd numbers of tiles, partial last tiles, several segments, with tables and without; and by
+kernels of their own, where O is an operand's array."""
 import pytest
+import torch
 
 from oracle import smat_oracle as so
 from paper_2609_36062_b200 import binding, synth
@@ -23,8 +25,17 @@ def test_rows_leave_divided_by_their_normaliser(d, heads, T, c):
         ref, den = so.normalized_forward_dense(Q64, K64, V64[:, :-1], M)
         got = to_numpy64(O[0, h])
         assert rel_err(got[:, :-1], ref) <= 2e-2 and rel_err(got[:, -1], den) <= 2e-2   # the stated bound of bf16 plans
-    # into Q's array: the row kernel divides what has been rounded, so another half unit in the last place (2^-8) for the sum and
+    # what the caller left in the normaliser column does not matter, to the exported tables either
+    tables = plan.debug_tables() if d > 1 else ()
+    v = dev["v"].clone()
+    v[..., -1] = float("nan")
+    assert torch.equal(plan.forward_normalized(dev["q"], dev["k"], v), O)
+    for a, b in zip(tables[:2], plan.debug_tables() if d > 1 else ()):
+        assert torch.equal(a, b)
+    # into an operand's array: the row kernel divides what has been rounded, so another half unit in the last place (2^-8) for the sum and
     # one for the normaliser
-    into = plan.forward_normalized(dev["q"], dev["k"], dev["v"], O=dev["q"])
-    assert into.data_ptr() == dev["q"].data_ptr()
-    assert rel_err(to_numpy64(into), to_numpy64(O)) <= 3 * 2.0 ** -8
+    for place in ("q", "v"):
+        x = {name: t.clone() for name, t in dev.items()}
+        into = plan.forward_normalized(x["q"], x["k"], x["v"], O=x[place])
+        assert into.data_ptr() == x[place].data_ptr()
+        assert rel_err(to_numpy64(into), to_numpy64(O)) <= 3 * 2.0 ** -8
