@@ -399,36 +399,45 @@ def gated_tc_mode(plan) -> int:
     return 2 if plan.gated_backward_uses_tensor_cores() else 1
 
 
-def path_report(w, geo, seconds_per_step, peaks, u_bytes=4, f_bytes=4, gated_tc_forward=0):
+def without_tables(stages) -> bool:
+    """Whether the passes formed their long-range rows without tables."""
+    return any(name == "read_lines" for name, _ in stages)
+
+
+def path_report(w, geo, seconds_per_step, peaks, u_bytes=4, f_bytes=4, gated_tc_forward=0, no_tables=False):
     """Fractions against the path roofline.  The bytes are those of the design that ran: where a table is kept as
     bf16 its round trip is charged at 2 bytes per entry, and the fraction against the roofline with fp32 tables is
     given beside it.  gated_tc_forward: 0 = not a gated tensor-core pass; 1 = a gated plan whose forward runs on the
     tensor cores (bf16 tables) while its backward rebuilds fp32 tables on the ALU kernels; 2 = both passes on the
-    tensor cores.  Each pass is charged with the tables it keeps."""
+    tensor cores.  Each pass is charged with the tables it keeps (no_tables: none)."""
     e = 4 if w.dtype == "f32" else 2
     def total(ub, fb):
         if gated_tc_forward and (ub, fb) != (4, 4):
-            wk = roofline.forward_work(w.T, w.chunk, w.d_k, w.d_v, e, geo, 2, 2)
+            wk = roofline.forward_work(w.T, w.chunk, w.d_k, w.d_v, e, geo, ub, fb)
             if w.backward:   # the gated backward rebuilds the forward tables; fp32 tables where it runs on the ALU kernels
-                tb = 2 if gated_tc_forward == 2 else 4   # the tensor-core backward reuses the forward's tables
+                tb = ub if gated_tc_forward == 2 else 4   # the tensor-core backward reuses the forward's tables
                 wk = wk + roofline.backward_work(w.T, w.chunk, w.d_k, w.d_v, e, geo, tb, tb,
                                                  keep_forward_tables=gated_tc_forward == 2, f_bytes=tb, ubar_bytes=tb)
             return wk.scaled(w.bh)
         wk = roofline.forward_work(w.T, w.chunk, w.d_k, w.d_v, e, geo, ub, fb)
         if w.backward:  # bench.py's fwd+bwd step keeps the forward's tables; the adjoint tables follow the forward's
-            fbar = 2 if (fb == 2 or (ub == 2 and geo.d <= 3)) else 4
-            ubar = 2 if (fb == 2 and geo.d >= 3) or (ub == 2 and geo.d == 2) else 4
+            fbar = 0 if fb == 0 else 2 if (fb == 2 or (ub == 2 and geo.d <= 3)) else 4
+            ubar = 0 if fb == 0 else 2 if (fb == 2 and geo.d >= 3) or (ub == 2 and geo.d == 2) else 4
             wk = wk + roofline.backward_work(w.T, w.chunk, w.d_k, w.d_v, e, geo, ub, fbar, keep_forward_tables=True,
                                              f_bytes=fb, ubar_bytes=ubar)
         return wk.scaled(w.bh)
-    work = total(2, 2) if gated_tc_forward else total(u_bytes, f_bytes)
+    if no_tables:
+        u_bytes = f_bytes = 0
+    elif gated_tc_forward:
+        u_bytes = f_bytes = 2
+    work = total(u_bytes, f_bytes)
     t = roofline.roofline_times(work, peaks)
     t32 = roofline.roofline_times(total(4, 4), peaks)
     return {
         "frac_2term": t["t_2term"] / seconds_per_step, "frac_3term": t["t_3term"] / seconds_per_step,
         "frac_2term_fp32_tables": t32["t_2term"] / seconds_per_step,
-        "type_table_bytes_per_entry": 2 if gated_tc_forward else u_bytes,
-        "profile_table_bytes_per_entry": 2 if gated_tc_forward else f_bytes,
+        "type_table_bytes_per_entry": u_bytes,
+        "profile_table_bytes_per_entry": f_bytes,
         "roofline_ms_2term": 1e3 * t["t_2term"], "roofline_ms_3term": 1e3 * t["t_3term"],
         "t_tensor_ms": 1e3 * t["t_tensor"], "t_alu_ms": 1e3 * t["t_alu"], "t_hbm_ms": 1e3 * t["t_hbm"],
         "alu_peak_adds_per_s": t["alu_peak_adds"], "alu_peak_source": t["alu_peak_source"],
@@ -557,7 +566,7 @@ def run_native(args):
             "gpu_launches": launches * steps,
             "clocks": clocks,
             "roofline": dominant_kernel_report(w, g, stages, peaks, ub, fb, on_alus(runner.plan)),
-            "path_roofline": path_report(w, g, per_step, peaks, ub, fb, gated_tc_mode(runner.plan)),
+            "path_roofline": path_report(w, g, per_step, peaks, ub, fb, gated_tc_mode(runner.plan), without_tables(stages)),
             "tables": {"profile_states_P": g.P, "cached_subset_states_B": g.B, "nnzC": g.nnzC, "q": g.q},
             "fadd_rates_adds_per_s": peaks.get("fadd_rates"),
         }
@@ -574,9 +583,9 @@ def run_native(args):
             gg = r.plan.geometry()
             each_ = r.time_each(r.step, 15, 5)
             s = float(np.median(each_))
-            rep = path_report(ws_, gg, s, peaks, r.plan.type_table_element_bytes(), r.plan.profile_table_element_bytes(),
-                              gated_tc_mode(r.plan))
             st_ = r.stage_profile(3)
+            rep = path_report(ws_, gg, s, peaks, r.plan.type_table_element_bytes(), r.plan.profile_table_element_bytes(),
+                              gated_tc_mode(r.plan), without_tables(st_))
             dom = dominant_kernel_report(ws_, gg, st_, peaks, *table_bytes(r.plan), on_alus(r.plan))
             sweep.append({"workload": name, "dominant": {k: dom[k] for k in ("kernel", "bound", "achieved", "peak", "unit",
                                                                               "frac", "ms", "share")}, "value": ws_.tokens / s, "unit": "tokens/s", "ms_per_step": 1e3 * s,
