@@ -370,9 +370,9 @@ __global__ void __launch_bounds__(32 * (tile_epi_warps(GATED) + 1), 2) tile_prod
         for (int c = 0; c < 2 / PARTS; ++c) {
           const int col = (part + c * PARTS) * 32;
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            if (!prm.addend16) y[c][i] = reinterpret_cast<const uint4*>(prm.addend + at + col)[i];
-            else if (i < 4) y[c][i] = reinterpret_cast<const uint4*>(prm.addend16 + at + col)[i];
+          for (int i = 0; i < 8; i += 2) {
+            if (!prm.addend16) ld_global_v8(prm.addend + at + col + 4 * i, y[c][i], y[c][i + 1]);
+            else if (i < 4) ld_global_v8(prm.addend16 + at + col + 8 * i, y[c][i], y[c][i + 1]);
           }
         }
       }
@@ -693,9 +693,9 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) bwd_tile_fused_tc_kernel(con
       };
       // long-range rows of this thread's columns, fetched while the MMAs run
       auto fetch = [&](const __nv_bfloat16* lr, uint4 (&y)[4]) {
-        const uint4* y4 = reinterpret_cast<const uint4*>(lr + row * TILE + col0);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) y[i] = y4[i];
+        const __nv_bfloat16* from = lr + row * TILE + col0;
+        ld_global_v8(from, y[0], y[1]);
+        ld_global_v8(from + 16, y[2], y[3]);
       };
       // accumulator part (in v) plus long-range part, rounded and stored; GATED: its product with the same part of this
       // row of the operand tile `with` (null: none)
@@ -989,9 +989,11 @@ struct SegOutParams {
 // the output rows leave during the next tile's first two products.  (With P and the state sharing one tile, so that
 // every product waited for the previous one's operand, a tile took about 6000 cycles: 0.240 ms at d = 1, 16 heads of
 // 64 K tokens, where this order takes 0.205; its 1.07 GB need 0.161 at the HBM rate.)
+// The long-range rows are asked for after the state is published: asked for before P is stored, or before the scores are waited
+// for, the loads stand in front of those stores (44 us became 47, 32 heads of 4096 tokens, d = 3).
 // SPLIT: for blocks that are not whole tiles, whose plans keep fp32 tables: the state and the score tile enter their
 // products as a leading bf16 part plus a bf16 remainder (16 bits of the fp32 value), the long-range rows arrive in
-// fp32, and the rows past a block's end load as zeros and are not stored.  (32 heads of 5056 tokens, d = 3: 0.071 ms, and
+// fp32, and the rows past a block's end load as zeros and are not stored.  (32 heads of 5056 tokens, d = 3: 0.062 ms, and
 // 0.028 for the segment totals and their scan, where chunk states, scan, scores, state read and output on the fp32 ALUs
 // took 1.23 ms.)
 constexpr int SEG_EPI_WARPS = 16;
@@ -1228,11 +1230,13 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS + 32 * DIVIDE) segment_output_
 #pragma unroll
         for (int e = 0; e < 32; ++e) v[e] = 0u;
       } else {
-        const uint4* src = reinterpret_cast<const uint4*>(prm.seg_in + (((int64_t)bh * prm.nseg + from) * TILE + m) * TILE + col0);
+        const float* src = prm.seg_in + (((int64_t)bh * prm.nseg + from) * TILE + m) * TILE + col0;
 #pragma unroll
-        for (int q4 = 0; q4 < 8; ++q4) {
-          const uint4 a = *(src + q4);
-          v[4 * q4] = a.x; v[4 * q4 + 1] = a.y; v[4 * q4 + 2] = a.z; v[4 * q4 + 3] = a.w;
+        for (int q8 = 0; q8 < 4; ++q8) {
+          uint4 a, b;
+          ld_global_v8(src + 8 * q8, a, b);
+          v[8 * q8] = a.x; v[8 * q8 + 1] = a.y; v[8 * q8 + 2] = a.z; v[8 * q8 + 3] = a.w;
+          v[8 * q8 + 4] = b.x; v[8 * q8 + 5] = b.y; v[8 * q8 + 6] = b.z; v[8 * q8 + 7] = b.w;
         }
       }
       tmem_st32(tmem_s + lane_base + col0, v);
@@ -1280,10 +1284,12 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS + 32 * DIVIDE) segment_output_
       const bool add_lr = live && t >= prm.n_lr;
       uint4 y[Y32 ? 8 : 4];                        // 32 bf16 or fp32 values
       if (add_lr) {
-        const uint4* y4 = Y32 ? reinterpret_cast<const uint4*>(prm.ylr32 + ((int64_t)bh * prm.T + t) * TILE + col0)
-                              : reinterpret_cast<const uint4*>(prm.ylr + ((int64_t)bh * prm.T + t) * TILE + col0);
+        const int64_t at = ((int64_t)bh * prm.T + t) * TILE + col0;
 #pragma unroll
-        for (int i = 0; i < (Y32 ? 8 : 4); ++i) y[i] = *(y4 + i);
+        for (int i = 0; i < (Y32 ? 8 : 4); i += 2) {
+          if (Y32) ld_global_v8(prm.ylr32 + at + 4 * i, y[i], y[i + 1]);
+          else ld_global_v8(prm.ylr + at + 8 * i, y[i], y[i + 1]);
+        }
       }
       if (!mbar_wait_warp(bar_o, it & 1, wc)) break;
       fence_after_sync();

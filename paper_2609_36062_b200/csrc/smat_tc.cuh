@@ -288,7 +288,18 @@ __device__ __forceinline__ void st_global_v8(void* dst, uint32_t w0, uint32_t w1
                : "memory");
 }
 
-// The same 32 bytes of a caller's array, which is promised to lie on a 16-byte boundary only: `wide` (uniform, from
+// 32-byte load: a whole sector per thread (src 32-byte aligned, as the rows of the workspace are).  Where every lane reads a row of
+// its own, 16-byte loads are twice the requests, each for half a sector, and the stores to shared memory behind them wait: the
+// output kernels took 43 us where they now take 39 (16 K, d = 4, 8 heads), 133 / 121 (d = 2, 16 heads of 23,296, fp32 rows), 75 / 65
+// (d = 3, 32 heads of 5056, normalised), the tile adjoints 70.6 / 68.6 (16 heads of 8192).
+__device__ __forceinline__ void ld_global_v8(const void* src, uint4& a, uint4& b) {
+  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+               : "l"(src)
+               : "memory");
+}
+
+// The store to a caller's array, which is promised to lie on a 16-byte boundary only: `wide` (uniform, from
 // rows_are_wide) says that the array's 256-byte rows start on 32-byte boundaries.
 __device__ __forceinline__ bool rows_are_wide(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31) == 0; }
 __device__ __forceinline__ void st_global_32(void* dst, bool wide, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3,
