@@ -1245,6 +1245,7 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS + 32 * DIVIDE) segment_output_
     }
     const int64_t row_first = seg_tile_row(prm.cut, tile0), row_end = blk ? prm.cut.rows : prm.cut.rows0;
     const bool wide = rows_are_wide(prm.O);
+    const int odd = lane & 1;
     for (int it = 0; it < Lc; ++it) {
       uint8_t* stage = smem + (it & 1) * Lay::STAGE;
       // --- scores of this tile -> masked bf16 P (registers), stored once Q and K have been consumed ---
@@ -1280,20 +1281,27 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS + 32 * DIVIDE) segment_output_
       }
       // --- long-range rows of this tile, fetched while the MMAs run ---
       const int64_t t = row_first + (int64_t)it * TILE + m;
-      const bool live = !SPLIT || t < row_end;
-      const bool add_lr = live && t >= prm.n_lr;
+      // (two lanes to 64 bytes of a row: of the pair's first row, then of its second)
+      const bool add_lr = row_first >= prm.n_lr;   // (a block has such rows or none)
+      const int64_t t0 = t - odd;
       uint4 y[Y32 ? 8 : 4];                        // 32 bf16 or fp32 values
       if (add_lr) {
-        const int64_t at = ((int64_t)bh * prm.T + t) * TILE + col0;
+        const int64_t at = ((int64_t)bh * prm.T + t0) * TILE + col0;
 #pragma unroll
         for (int i = 0; i < (Y32 ? 8 : 4); i += 2) {
-          if (Y32) ld_global_v8(prm.ylr32 + at + 4 * i, y[i], y[i + 1]);
-          else ld_global_v8(prm.ylr + at + 8 * i, y[i], y[i + 1]);
+          const int row = (i >> 1) & 1, part = 2 * (i >> 2) + odd;   // its 32-byte part of the row
+          if (SPLIT && t0 + row >= row_end) {
+            y[i] = y[i + 1] = make_uint4(0u, 0u, 0u, 0u);
+          } else if (Y32) {
+            ld_global_v8(prm.ylr32 + at + row * TILE + 8 * part, y[i], y[i + 1]);
+          } else {
+            ld_global_v8(prm.ylr + at + row * TILE + 16 * part, y[i], y[i + 1]);
+          }
         }
       }
       if (!mbar_wait_warp(bar_o, it & 1, wc)) break;
       fence_after_sync();
-      __nv_bfloat16* dst = prm.O + ((int64_t)bh * prm.T + t) * TILE + col0;
+      __nv_bfloat16* dst = prm.O + ((int64_t)bh * prm.T + t0) * TILE + col0 + 16 * odd;
       const uint32_t tmem_o = tmem_o0 + (it & 1) * TILE;
       uint32_t v[32];
       tmem_ld32(tmem_o + lane_base + col0, v);
@@ -1302,6 +1310,8 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS + 32 * DIVIDE) segment_output_
 #pragma unroll
       for (int e = 0; e < 32; ++e) f[e] = __uint_as_float(v[e]);
       if (add_lr) {
+#pragma unroll
+        for (int i = 0; i < (Y32 ? 8 : 4); i += 4) swap_rows(odd, y[i], y[i + 1], y[i + 2], y[i + 3]);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           float* fi = f + 8 * i;
@@ -1334,14 +1344,17 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS + 32 * DIVIDE) segment_output_
         for (int e = 0; e < 32; ++e) f[e] *= inv;
         if (cq == 3) f[31] = den;
       }
-      uint32_t w[16];
+      uint4 w[4];
 #pragma unroll
-      for (int e = 0; e < 16; ++e) w[e] = pack_bf16(f[2 * e], f[2 * e + 1]);
-      if (live) {
+      for (int c = 0; c < 4; ++c)
+        w[c] = make_uint4(pack_bf16(f[8 * c], f[8 * c + 1]), pack_bf16(f[8 * c + 2], f[8 * c + 3]),
+                          pack_bf16(f[8 * c + 4], f[8 * c + 5]), pack_bf16(f[8 * c + 6], f[8 * c + 7]));
+      swap_rows(odd, w[0], w[1], w[2], w[3]);
 #pragma unroll
-        for (int h8 = 0; h8 < 2; ++h8)   // whole 32-byte sectors
-          st_global_32(dst + 16 * h8, wide, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
-                       w[8 * h8 + 5], w[8 * h8 + 6], w[8 * h8 + 7]);
+      for (int row = 0; row < 2; ++row) {
+        if (!SPLIT || t0 + row < row_end)
+          st_global_32(dst + row * TILE, wide, w[2 * row].x, w[2 * row].y, w[2 * row].z, w[2 * row].w, w[2 * row + 1].x,
+                       w[2 * row + 1].y, w[2 * row + 1].z, w[2 * row + 1].w);
       }
     }
   }
