@@ -362,8 +362,9 @@ __global__ void __launch_bounds__(32 * (tile_epi_warps(GATED) + 1), 2) tile_prod
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_p);   // one arrival per warp
       // the rows to be added travel while the products are formed: 32 columns are eight (fp32) or four (bf16) pieces
-      const int64_t t = (int64_t)b * TILE + m, at = ((int64_t)bh * prm.T + t) * TILE + half * HALF;
-      const bool add_lr = t >= prm.add_lo && t < prm.add_hi;
+      const int odd = lane & 1;
+      const int64_t t = (int64_t)b * TILE + m, at = ((int64_t)bh * prm.T + t - odd) * TILE + half * HALF;
+      const bool add_lr = t >= prm.add_lo && t < prm.add_hi;   // (a tile's rows are all added to, or none)
       uint4 y[2 / PARTS][8];
       if (add_lr) {
 #pragma unroll
@@ -371,8 +372,9 @@ __global__ void __launch_bounds__(32 * (tile_epi_warps(GATED) + 1), 2) tile_prod
           const int col = (part + c * PARTS) * 32;
 #pragma unroll
           for (int i = 0; i < 8; i += 2) {
-            if (!prm.addend16) ld_global_v8(prm.addend + at + col + 4 * i, y[c][i], y[c][i + 1]);
-            else if (i < 4) ld_global_v8(prm.addend16 + at + col + 8 * i, y[c][i], y[c][i + 1]);
+            const int row = (i >> 1) & 1, piece = 2 * (i >> 2) + odd;   // two lanes to a row, 32 bytes each
+            if (!prm.addend16) ld_global_v8(prm.addend + at + row * TILE + col + 8 * piece, y[c][i], y[c][i + 1]);
+            else if (i < 4) ld_global_v8(prm.addend16 + at + row * TILE + col + 16 * piece, y[c][i], y[c][i + 1]);
           }
         }
       }
@@ -394,7 +396,11 @@ __global__ void __launch_bounds__(32 * (tile_epi_warps(GATED) + 1), 2) tile_prod
 #pragma unroll
             for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(fmaf(row_scale, __uint_as_float(vs[e]), __uint_as_float(v[e])));
           }
-          uint32_t w[16];
+          uint4 w[4];
+          if (add_lr) {
+            swap_rows(odd, y[c][0], y[c][1], y[c][2], y[c][3]);
+            if (!prm.addend16) swap_rows(odd, y[c][4], y[c][5], y[c][6], y[c][7]);
+          }
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             float f[8];
@@ -412,14 +418,14 @@ __global__ void __launch_bounds__(32 * (tile_epi_warps(GATED) + 1), 2) tile_prod
               f[0] += __uint_as_float(a.x); f[1] += __uint_as_float(a.y); f[2] += __uint_as_float(a.z); f[3] += __uint_as_float(a.w);
               f[4] += __uint_as_float(d.x); f[5] += __uint_as_float(d.y); f[6] += __uint_as_float(d.z); f[7] += __uint_as_float(d.w);
             }
-            w[4 * i] = pack_bf16(f[0], f[1]); w[4 * i + 1] = pack_bf16(f[2], f[3]);
-            w[4 * i + 2] = pack_bf16(f[4], f[5]); w[4 * i + 3] = pack_bf16(f[6], f[7]);
+            w[i] = make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
           }
-          __nv_bfloat16* dst = prm.Out + at + col;
+          swap_rows(odd, w[0], w[1], w[2], w[3]);
+          __nv_bfloat16* dst = prm.Out + at + col + 16 * odd;
 #pragma unroll
-          for (int h8 = 0; h8 < 2; ++h8)   // whole 32-byte sectors
-            st_global_32(dst + 16 * h8, wide, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
-                         w[8 * h8 + 5], w[8 * h8 + 6], w[8 * h8 + 7]);
+          for (int h = 0; h < 2; ++h)
+            st_global_32(dst + h * TILE, wide, w[2 * h].x, w[2 * h].y, w[2 * h].z, w[2 * h].w, w[2 * h + 1].x, w[2 * h + 1].y,
+                         w[2 * h + 1].z, w[2 * h + 1].w);
         }
       }
     }
@@ -691,17 +697,19 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) bwd_tile_fused_tc_kernel(con
         for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * f);
         tmem_st32(tm_acc + lane_base + col0, v);
       };
+      const int odd = lane & 1;
       // long-range rows of this thread's columns, fetched while the MMAs run
       auto fetch = [&](const __nv_bfloat16* lr, uint4 (&y)[4]) {
-        const __nv_bfloat16* from = lr + row * TILE + col0;
+        const __nv_bfloat16* from = lr + (row - odd) * TILE + col0 + 16 * odd;   // two lanes to a row
         ld_global_v8(from, y[0], y[1]);
-        ld_global_v8(from + 16, y[2], y[3]);
+        ld_global_v8(from + TILE, y[2], y[3]);
       };
       // accumulator part (in v) plus long-range part, rounded and stored; GATED: its product with the same part of this
       // row of the operand tile `with` (null: none)
-      auto finish = [&](const uint32_t (&v)[32], const uint4 (&y)[4], bool add, __nv_bfloat16* out, const uint8_t* with) {
+      auto finish = [&](const uint32_t (&v)[32], uint4 (&y)[4], bool add, __nv_bfloat16* out, const uint8_t* with) {
         float dot = 0.f;
-        uint32_t w[16];
+        uint4 w[4];
+        if (add) swap_rows(odd, y[0], y[1], y[2], y[3]);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           float f[8];
@@ -724,14 +732,14 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) bwd_tile_fused_tc_kernel(con
               dot = fmaf(f[2 * e + 1], __uint_as_float(xx[e] & 0xffff0000u), dot);
             }
           }
-          w[4 * i] = pack_bf16(f[0], f[1]); w[4 * i + 1] = pack_bf16(f[2], f[3]);
-          w[4 * i + 2] = pack_bf16(f[4], f[5]); w[4 * i + 3] = pack_bf16(f[6], f[7]);
+          w[i] = make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
         }
-        __nv_bfloat16* dst = out + row * TILE + col0;
+        swap_rows(odd, w[0], w[1], w[2], w[3]);
+        __nv_bfloat16* dst = out + (row - odd) * TILE + col0 + 16 * odd;
 #pragma unroll
-        for (int h8 = 0; h8 < 2; ++h8)   // whole 32-byte sectors
-          st_global_32(dst + 16 * h8, wide, w[8 * h8], w[8 * h8 + 1], w[8 * h8 + 2], w[8 * h8 + 3], w[8 * h8 + 4],
-                       w[8 * h8 + 5], w[8 * h8 + 6], w[8 * h8 + 7]);
+        for (int h = 0; h < 2; ++h)
+          st_global_32(dst + h * TILE, wide, w[2 * h].x, w[2 * h].y, w[2 * h].z, w[2 * h].w, w[2 * h + 1].x, w[2 * h + 1].y,
+                       w[2 * h + 1].z, w[2 * h + 1].w);
         return dot;
       };
       // a tile lies on one side of the block boundary
@@ -1173,6 +1181,7 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS + 32 * DIVIDE) segment_output_
     const int m = (warp & 3) * 32 + lane;            // TMEM lane: state row i / query row of the tile
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t col0 = cq * 32;
+    const int odd = lane & 1;
     // this thread's 64 bytes (four 16-byte chunks) of its row in the 64-column block that holds its columns
     const uint32_t my_off = (cq >> 1) * BOX_BYTES + m * 128;
     const int ch0 = (cq & 1) * 4;
@@ -1218,9 +1227,10 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS + 32 * DIVIDE) segment_output_
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_s);   // one arrival per warp: 512 arrivals on one barrier serialise
       if (!SPLIT && prm.sin_tiles) {
-        __nv_bfloat16* dst = prm.sin_tiles + (((int64_t)bh * (prm.T / TILE) + tile) * TILE + m) * TILE + col0;
+        __nv_bfloat16* dst = prm.sin_tiles + (((int64_t)bh * (prm.T / TILE) + tile) * TILE + m - odd) * TILE + col0 + 16 * odd;
+        swap_rows(odd, pk[0], pk[1], pk[2], pk[3]);
         st_global_v8(dst, pk[0].x, pk[0].y, pk[0].z, pk[0].w, pk[1].x, pk[1].y, pk[1].z, pk[1].w);
-        st_global_v8(dst + 16, pk[2].x, pk[2].y, pk[2].z, pk[2].w, pk[3].x, pk[3].y, pk[3].z, pk[3].w);
+        st_global_v8(dst + TILE, pk[2].x, pk[2].y, pk[2].z, pk[2].w, pk[3].x, pk[3].y, pk[3].z, pk[3].w);
       }
     };
     {  // state entering the segment: global fp32 -> TMEM (accumulator) and the shared tile
@@ -1245,7 +1255,6 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS + 32 * DIVIDE) segment_output_
     }
     const int64_t row_first = seg_tile_row(prm.cut, tile0), row_end = blk ? prm.cut.rows : prm.cut.rows0;
     const bool wide = rows_are_wide(prm.O);
-    const int odd = lane & 1;
     for (int it = 0; it < Lc; ++it) {
       uint8_t* stage = smem + (it & 1) * Lay::STAGE;
       // --- scores of this tile -> masked bf16 P (registers), stored once Q and K have been consumed ---

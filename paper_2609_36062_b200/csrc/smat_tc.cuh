@@ -304,7 +304,7 @@ __device__ __forceinline__ void ld_global_v8(const void* src, uint4& a, uint4& b
 // 1 (a, b: the first row's; c, d: the second's); afterwards the even lane has the first row, the odd one the second, parts 0 and 1 in
 // order.  Its own inverse.  Output kernel, a row to a lane / two lanes to a row: 38.9 us / 34.9 (16 K, d = 4, 8 heads), 121 / 108.6 (d = 2,
 // 16 heads of 23,296, fp32 rows), 65 / 60 (d = 3, 32 heads of 5056, normalised), 59.4 / 56.3 (d = 1, 16 heads of 16 K); most of it from
-// the stores.
+// the stores.  Tile adjoints and their entering states, a step of 16 heads of 8192 360 / 353.5, gated, 32 of 4096, 456.5 / 454.7.
 __device__ __forceinline__ void swap_rows(int odd, uint4& a, uint4& b, uint4& c, uint4& d) {
   auto swap = [&](uint32_t& u, uint32_t& v) {
     const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? u : v, 1);
