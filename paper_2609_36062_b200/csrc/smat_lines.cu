@@ -502,12 +502,15 @@ LineShape line_shape(const SmatGeo& g, int bh, int rows_are_types, bool dual = f
 }  // namespace
 
 bool smat_lines_supported(const SmatGeo& geo, int bh) {
-  if (geo.dense_G || geo.T >= ((int64_t)1 << 30)) return false;
-  for (int types = 0; types < 2; ++types) {
-    const LineShape s = line_shape(geo, bh, types);
+  if (geo.dense_G || geo.T >= ((int64_t)1 << 30) || geo.n < geo.P || geo.m < geo.B || (uint64_t)geo.B * geo.q >= (1ull << 31))
+    return false;
+  // Quotients by umulhi: items by items of a head, slots by lines.  The two-product launch has the most row blocks (d = 2 with a
+  // prime given by the caller, one head of 1.1 M tokens, q = 32771: 65,542 items a head where the single products have 32,771).
+  for (int launch = 0; launch < 3; ++launch) {
+    const int types = launch == 0;
+    const LineShape s = line_shape(geo, bh, types, launch == 2);
     const int64_t layers = (types ? geo.n / geo.P : geo.m / geo.B) + 1;
-    if (s.items * s.groups * s.blocks >= (1ull << 32) || geo.n < geo.P || geo.m < geo.B || (uint64_t)s.lines * layers * s.lines >= (1ull << 31) || (uint64_t)geo.B * geo.q >= (1ull << 31))
-      return false;
+    if (s.items * s.groups * s.blocks >= (1ull << 32) || (uint64_t)s.lines * layers * s.lines >= (1ull << 31)) return false;
   }
   return true;
 }

@@ -238,3 +238,31 @@ def test_output_buffers_may_be_larger_but_not_smaller_or_strided():
                 backward(bad)
         with pytest.raises(ValueError):
             decode(small[..., :63])
+
+
+class _SmatGeo(ctypes.Structure):   # csrc/smat_geometry.h
+    _fields_ = [(f, ctypes.c_int64) for f in ("T", "c", "n", "m")] + [(f, ctypes.c_int32) for f in ("d", "q", "D")] + \
+               [(f, ctypes.c_int64) for f in ("P", "A", "B", "nnzC")] + [("dense_G", ctypes.c_int32)] + \
+               [("qpow", ctypes.c_int64 * 8), ("dir_group_start", ctypes.c_int64 * 8)]
+
+
+@pytest.mark.parametrize("q,bh,fits", [(32749, 1, True), (32771, 1, False), (1009, 1054, True), (1009, 1055, False)])
+def test_rows_without_tables_keep_every_launch_inside_its_quotients(q, bh, fits):
+    """d = 2, 17 or 18 tokens to a cell and to a type: one row block to a group in the single products, two in the launch that
+    forms dK and dV.  The kernel divides an item's number by the items of a head with one multiplication, which is exact
+    while items x (items of a head) stays below 2^32; beyond it an item would address another head."""
+    n = -(-17 * q // 128) * 128
+    plan = binding.SmatPlan(1, bh, 2 * n, 128, 128, 2, 128, "bf16", q_override=q)   # (sizes that a plan accepts)
+    g = plan.geometry()
+    geo = _SmatGeo(T=g.T, c=g.c, n=g.n, m=g.m, d=2, q=q, D=1, P=g.P, A=g.A, B=g.B, nnzC=g.nnzC)
+    geo.qpow[:2] = (1, q)
+    assert -(-g.n // g.P) in (17, 18)
+    supported = binding.load_library()["_Z20smat_lines_supportedRK7SmatGeoi"]
+    supported.restype, supported.argtypes = ctypes.c_bool, [ctypes.c_void_p, ctypes.c_int]
+    assert supported(ctypes.byref(geo), bh) == fits
+    per = 2 * q
+    items = bh * per
+    inverse = (2 ** 32 + per - 1) // per
+    last_of_a_head = np.arange(per - 1, items, per, dtype=np.uint64)
+    exact = bool(np.all(last_of_a_head * np.uint64(inverse) >> np.uint64(32) == last_of_a_head // np.uint64(per)))
+    assert exact or not fits
