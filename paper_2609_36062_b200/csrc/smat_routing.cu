@@ -12,7 +12,9 @@ namespace {
 
 // What a CTA takes is a chain of passes over its tokens in shared memory, so as many warps as there are counters for, at most 32
 // (16 heads of 35,968 tokens, d = 4: 91 us with 8, 66 with 22; 32 heads of 16 K: 48, 35), several keys of a lane in flight, and
-// no match.any, which takes a step for every different key of a warp: 35 us and 21.
+// no match.any, which takes a step for every different key of a warp: 35 us and 21.  Equal keys are ranked a key at a time; a
+// token at a time, all tokens in one group took 74 us at 35,968 tokens where 60 were taken with match.any and 27 are now, eight groups 73, 66
+// and 39, runs of four tokens 81, 74 and 45.
 constexpr int ROUTE_THREADS = 1024;
 constexpr int ROUTE_AHEAD = 4;   // keys of a lane in flight
 
@@ -24,8 +26,9 @@ constexpr int ROUTE_AHEAD = 4;   // keys of a lane in flight
 //      some CTA reads on its own), exclusive scan -> offs[0 .. G]; row w then becomes the first slot of group g for warp w's
 //      tokens: offs[g] + the counts of the warps before it
 //   3. stable placement: every warp walks ITS range in order, 32 tokens at a time; every lane advances the warp's cursor of
-//      its token's group, those that find it advanced further compare their keys for their rank (match.any takes a step for
-//      every different key, and nearly all 32 are), and writes its token's position.  Ranges are in token order and each warp's slots follow those of the warps before it, so the list of
+//      its token's group, those that find it advanced further rank themselves among the lanes of the same key (one ballot for
+//      each such key, at most 16; match.any takes a step for every different key, and nearly all 32 are), and writes its
+//      token's position.  Ranges are in token order and each warp's slots follow those of the warps before it, so the list of
 //      a group is ascending.
 struct RouteParams {
   const int32_t* key[2];   // [bh][count]
@@ -124,9 +127,11 @@ __global__ void __launch_bounds__(ROUTE_THREADS) routing_lists_kernel(const __gr
         // keys that met others of their kind: few, but where a group is heavy
         const unsigned same = __ballot_sync(0xffffffffu, valid && cursor[valid ? k : 0] - slot > 1);
         int rank = 0;
-        for (unsigned m = same; m; m &= m - 1) {
-          const int from = __ffs(m) - 1;
-          if (__shfl_sync(0xffffffffu, k, from) == k && from < lane) ++rank;
+        for (unsigned m = same; m;) {   // a step for every different one of these keys, 16 at most
+          const int32_t other = __shfl_sync(0xffffffffu, k, __ffs(m) - 1);
+          const unsigned peers = __ballot_sync(0xffffffffu, k == other);
+          if (k == other) rank = __popc(peers & ((1u << lane) - 1));
+          m &= ~peers;
         }
         if (valid) list[slot + rank] = (int32_t)(first + t);
         __syncwarp();

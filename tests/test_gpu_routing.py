@@ -179,3 +179,52 @@ def test_a_heavy_type_is_read_by_many_ctas():
         took.append(sorted(times)[4])
     plan.profile_enable(False)
     assert took[1] <= 2 * took[0], took
+
+
+def test_the_list_builder_takes_no_longer_where_tokens_share_a_cell():
+    """The warps rank equal keys a key at a time, not a token at a time (all tokens in one group then take twice as long as a
+    uniform hash; half as much again is the slack)."""
+    w = synth.Workload("lists", 3, 1, 16, 16384, 128, 128, 128, "bf16", "normalised", 18)
+    _, dev = device_inputs(w)
+    plan = binding.SmatPlan(w.batch, w.heads, w.T, w.d_k, w.d_v, w.d, w.chunk, w.dtype)
+    geo = plan.geometry()
+    prof = torch.randint(geo.P, (w.bh, geo.n), device="cuda", dtype=torch.int32)
+    typ = torch.randint(geo.B, (w.bh, geo.m), device="cuda", dtype=torch.int32)
+    plan.profile_enable(True)
+    took = []
+    for p, t in ((prof, typ), (torch.full_like(prof, 3), torch.full_like(typ, 5)), (prof % 8, typ % 8)):
+        times = []
+        for _ in range(9):
+            plan.forward(dev["q"], dev["k"], dev["v"], prof=p, type=t)
+            torch.cuda.synchronize()
+            times.append(dict(plan.profile_read())["routing_lists"])
+        took.append(sorted(times)[4])
+    plan.profile_enable(False)
+    assert max(took) <= 1.5 * took[0], took
+
+
+# Keys that the 32 lanes of a warp meet: one, two in turn, sixteen twice, four neighbours each, and keys out of range among them
+@pytest.mark.parametrize("pattern", ["one", "two", "sixteen", "fours", "dropped"])
+def test_lists_of_tokens_whose_neighbours_share_cells(pattern):
+    w = synth.Workload("shared", 3, 1, 2, 2048, 128, 128, 128, "bf16", "normalised", 92)
+    host, dev = device_inputs(w, ("q", "k", "v", "do"))
+    geo = so.geometry(w.T, w.chunk, w.d)
+
+    def keys(count, groups, h):
+        t = np.arange(count)
+        k = {"one": 0 * t + 7 + h, "two": 3 + t % 2, "sixteen": t % 16 + 5 * (t // 32), "fours": 11 * (t // 4) + h,
+             "dropped": np.where(t % 3 == h, groups + t % 2, t % 5)}[pattern]
+        return (k if pattern == "dropped" else k % groups).astype(np.int32)
+
+    cells = np.stack([keys(geo.n, geo.P, h) for h in range(2)])
+    types = np.stack([keys(geo.m, geo.B, 1 - h) for h in range(2)])
+    prof, typ = torch.from_numpy(cells).cuda(), torch.from_numpy(types).cuda()
+    plan = binding.SmatPlan(w.batch, w.heads, w.T, w.d_k, w.d_v, w.d, w.chunk, w.dtype)
+    O = plan.forward(dev["q"], dev["k"], dev["v"], prof=prof, type=typ)
+    grads = plan.backward(dev["q"], dev["k"], dev["v"], dev["do"], prof=prof, type=typ)
+    plan.check_status()
+    for h in range(2):
+        Q64, K64, V64, G64 = (synth.as_float64(w, host[x][h]) for x in ("q", "k", "v", "do"))
+        M = so.routed_dense_mask(geo, cells[h], types[h])
+        for got, ref in zip((O, *grads), (so.forward_dense(Q64, K64, V64, M), *so.backward_dense(Q64, K64, V64, G64, M))):
+            assert rel_err(to_numpy64(got[0, h]), ref) <= TOL["bf16"]
