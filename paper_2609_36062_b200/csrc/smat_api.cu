@@ -426,11 +426,15 @@ size_t line_copy_offset(const smat_plan* pl, int where) {
   return pl->off_acc + (where == LINE_COPY_BEHIND ? (size_t)pl->bh * pl->T * 256 : 0);
 }
 
+// bf16 parts of a score in the products that stand for a read of U: three where the plan's tables are fp32 (a score keeps all of its
+// bits, as U did), two for d = 2 with bf16 tables (one rounding there: U is F), else one.
+int table_parts(const smat_plan* pl) { return pl->u_bf16 ? (pl->geo.D == 1 ? 2 : 1) : 3; }
+
 // Long-range rows of the recent tokens (types = 1) or of the distant ones, without tables; see SmatLineArgs.
-SmatLineArgs line_job(int types, const void* x, const void* y, const void* z, void* out, int out_f32, int split,
+SmatLineArgs line_job(int types, const void* x, const void* y, const void* z, void* out, int out_f32, int parts,
                       const float* lam = nullptr) {
   SmatLineArgs a{};
-  a.split = split;
+  a.parts = parts;
   a.rows_are_types = types; a.x1 = x; a.y = y; a.z = z; a.out1 = out; a.out_f32 = out_f32; a.lam = lam;
   return a;
 }
@@ -725,7 +729,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     const int64_t tiles0 = lr ? pl->geo.n / 128 : pl->T / 128, tiles1 = lr ? pl->geo.m / 128 : 0;
     const bool per_tile = (pl->flags & SMAT_FLAG_PER_TILE_STATES) != 0, f32 = forward_rows_f32(pl);
     if (lines) {                                                                             // steps 2-4 in one
-      SmatLineArgs a = line_job(1, Q, K, V, ylr, f32, pl->geo.D == 1);
+      SmatLineArgs a = line_job(1, Q, K, V, ylr, f32, table_parts(pl));
       a.ones = divide;
       pl->forward_left = f32 ? LINE_COPY_BESIDE : LINE_COPY_BEHIND;
       line_copy(cx, &a, pl->forward_left, false);
@@ -770,7 +774,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     const bool lr = !pl->geo.dense_G;
     const int64_t rows0 = lr ? pl->geo.n : pl->T, rows1 = lr ? pl->geo.m : 0;
     if (pl->lines && !cx.routed) {
-      SmatLineArgs a = line_job(1, Q, K, V, ylr, 1, 1);
+      SmatLineArgs a = line_job(1, Q, K, V, ylr, 1, table_parts(pl));
       a.ones = divide;
       line_copy(cx, &a, LINE_COPY_BESIDE, false);
       line_mark(cx, &a, LINE_COPY_BESIDE);
@@ -855,7 +859,7 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
       else
         tabulate(cx, "bwd_tabulate_t", cx.f(pl->off_ubar), cx.f(pl->off_fbar), 1, pl->geo.D == 2 && pl->fbar_bf16);
       // dQ's long-range rows without tables; K and V of the distant tokens are behind them already where the forward left them
-      SmatLineArgs dq_lines = line_job(1, dO, V, K, lrbuf, 0, pl->geo.D == 1);
+      SmatLineArgs dq_lines = line_job(1, dO, V, K, lrbuf, 0, table_parts(pl));
       if (!(after_forward && pl->forward_left == LINE_COPY_BEHIND)) line_copy(cx, &dq_lines, LINE_COPY_BEHIND, true);
       line_mark(cx, &dq_lines, LINE_COPY_BEHIND);
       // per-tile states
@@ -870,7 +874,7 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
         char* lr_v = cx.ws + pl->off_lr3;
         if (lines) {
           line_rows(cx, "bwd_dq_lines", dq_lines);
-          SmatLineArgs a = line_job(0, K, Q, dO, lr_v, 0, 0);
+          SmatLineArgs a = line_job(0, K, Q, dO, lr_v, 0, 1);
           a.x2 = V; a.out2 = lr_k;
           line_rows(cx, "bwd_dkdv_lines", a);
           SMAT_TRY(cx, "bwd_tiles_fused_tc", smat_launch_bwd_tiles_fused_tc(Q, K, V, dO, sin_tiles, cx.ws + pl->off_dbar, lr_q,
@@ -909,7 +913,7 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
       // dK: distant rows add F̄_prof v
       if (!lines) zero_unrouted(cx, SMAT_GM_PROFILE, lrbuf, fbar_is_bf16 ? 256 : 512);
       if (lines)
-        line_rows(cx, "bwd_dk_lines", line_job(0, V, dO, Q, lrbuf, 0, 0));
+        line_rows(cx, "bwd_dk_lines", line_job(0, V, dO, Q, lrbuf, 0, 1));
       else if (fbar_is_bf16)
         SMAT_TRY(cx, "bwd_dk_profile_tc", smat_launch_state_read_tc(V, cx.ws + pl->off_fbar, lrbuf, lrbuf, 1, profs, pl->geo.P,
                                                                     pl->T, pl->bh, status, cx.st));
@@ -921,7 +925,7 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
       // dV: distant rows add F̄_profᵀ k
       if (!lines) zero_unrouted(cx, SMAT_GM_PROFILE, lrbuf, fbar_is_bf16 ? 256 : 512);
       if (lines)
-        line_rows(cx, "bwd_dv_lines", line_job(0, K, Q, dO, lrbuf, 0, 0));
+        line_rows(cx, "bwd_dv_lines", line_job(0, K, Q, dO, lrbuf, 0, 1));
       else if (fbar_is_bf16)
         SMAT_TRY(cx, "bwd_dv_profile_tc", smat_launch_state_read_tc(K, cx.ws + pl->off_fbar, lrbuf, lrbuf, 0, profs, pl->geo.P,
                                                                     pl->T, pl->bh, status, cx.st));
@@ -1037,7 +1041,7 @@ smat_status forward_gated_tc(Ctx& cx, const Gated& gt, const void* Q, const void
   ci.err = cx.err;
   float* ylr = ci.f(in->off_acc);
   if (in->lines) {   // the factors at the boundary enter the scores and the rows
-    line_rows(ci, "read_lines", line_job(1, Q, K, V, ylr, 1, 0, gt.lam));
+    line_rows(ci, "read_lines", line_job(1, Q, K, V, ylr, 1, 1, gt.lam));
   } else if (lr) {
     build_type_table(ci, gt.lr, V);                                                          // steps 2-3 on the rescaled keys
     if (in->u_bf16)
@@ -1094,8 +1098,8 @@ smat_status backward_gated_tc(Ctx& cx, const Gated& gt, const void* Q, const voi
   if (in->lines) {
     lr_q = lr_k = ci.ws + in->off_acc;
     lr_v = ci.ws + in->off_lr3;
-    line_rows(ci, "bwd_dq_lines", line_job(1, dO, V, K, lr_q, 0, 0, gt.lam));
-    SmatLineArgs a = line_job(0, K, Q, dO, lr_v, 0, 0, gt.lam);
+    line_rows(ci, "bwd_dq_lines", line_job(1, dO, V, K, lr_q, 0, 1, gt.lam));
+    SmatLineArgs a = line_job(0, K, Q, dO, lr_v, 0, 1, gt.lam);
     a.x2 = V; a.out2 = lr_k;
     line_rows(ci, "bwd_dkdv_lines", a);
   } else if (lr) {

@@ -295,7 +295,8 @@ struct SmatLineArgs {
   void *out1, *out2;
   int out_f32, rows_are_types;
   int ones;              // Z's last column counts as one (one product, ungated)
-  int split;             // scores enter their products as a bf16 part plus a bf16 remainder (one product, ungated)
+  int parts;             // bf16 parts in which a score enters its product: 1, 2 (16 bits) or 3 (all of fp32); more than one only
+                         // for one product, ungated
   const float* lam;      // gated: prefix sums of the log-gates; terms are multiplied by exp(λ_recent - λ_distant)
   void* copy;            // null, or where K and V of every distant token are left side by side: token t of head b at
   int64_t copy_head;     // row b * copy_head + t of 512 bytes

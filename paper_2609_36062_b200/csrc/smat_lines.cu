@@ -6,8 +6,11 @@
 // tokens against the tokens of all types through the cell, both products from one gather (DUAL).  The rows come from the L2
 // cache, which holds a head's K and V many times over, and nothing but the outputs goes back to memory.
 //
-// Scores are rounded to bf16 once, as the causal tiles' are; tables are rounded once for F and once or three times for U.  Where
-// the plan's tables are fp32, and for d = 2 (one rounding there too), they enter as a leading part and a remainder, 16 bits.
+// Scores are rounded to bf16 once, as the causal tiles' are; tables are rounded once for F and once or three times for U.  In the
+// ungated forward and dQ of d = 2 (one table, rounded once) they enter as a leading part and a remainder, 16 bits, and where
+// the plan's tables would be fp32 (partial tiles, forward only) in three parts, which hold all 24 bits.  The rows' error against fp64 there, in the
+// 2-norm: 1.1e-7 from fp32 tables, 3e-7 to 1.2e-6 with three parts (the matrix instructions' sums), 2.5e-6 with two; of the
+// outputs, rounded to bf16, 1.660e-3 each way.
 //
 // The matrix instructions are those of a warp (m16n8k16): a type has 6 to 20 rows, which fill a tile of 16 and would leave most
 // of a 128-row one of tcgen05 empty, and at 545 TFLOP/s measured they are not what the kernel waits for.
@@ -186,7 +189,7 @@ struct LineSmem {
 // 529 / 255; d = 4, 32 heads of 4096 552 / 190; fp32 tables: d = 3, 32 heads of 5056 503 / 95; d = 2, 32 of 4160 238 / 33.
 // The first form, four warps to an item with the scores exchanged through shared memory, took 156 where this takes 57; with a
 // test for every kind of stage in front of each and all of Z in registers (spills) it was 77.
-template <int RT, bool DUAL, bool GATED, bool SPLIT>
+template <int RT, bool DUAL, bool GATED, int PARTS>
 __global__ void __launch_bounds__(32, LineSmem<RT, DUAL>::warps_per_sm)
 line_products_kernel(const __grid_constant__ LineParams p) {
   using L = LineSmem<RT, DUAL>;
@@ -336,7 +339,7 @@ line_products_kernel(const __grid_constant__ LineParams p) {
       if (!(s & 1)) { tok = ntok; fac = nfac; }
       cp_async_wait<LN_STAGES - 1>();
       __syncwarp();
-      uint32_t ph[NX][RT][4], pl[NX][RT][4];
+      uint32_t pp[PARTS][NX][RT][4];   // the scores, in bf16 parts
 #pragma unroll
       for (int o = 0; o < NX; ++o) {
         float sc[RT][2][4], sd[RT][2][4];   // two sums each: a chain of products is as long as their latencies
@@ -388,11 +391,15 @@ line_products_kernel(const __grid_constant__ LineParams p) {
             for (int hf = 0; hf < 2; ++hf) {
               float v0 = sc[rt][nt][2 * hf] + sd[rt][nt][2 * hf], v1 = sc[rt][nt][2 * hf + 1] + sd[rt][nt][2 * hf + 1];
               if (GATED) { v0 *= f0; v1 *= f1; }
-              const __nv_bfloat162 h2 = __floats2bfloat162_rn(v0, v1);
-              ph[o][rt][2 * nt + hf] = *reinterpret_cast<const uint32_t*>(&h2);
-              if (SPLIT) {
-                const float2 h = __bfloat1622float2(h2);
-                pl[o][rt][2 * nt + hf] = pack_bf16(v0 - h.x, v1 - h.y);
+#pragma unroll
+              for (int part = 0; part < PARTS; ++part) {   // (a remainder is exact)
+                const __nv_bfloat162 h2 = __floats2bfloat162_rn(v0, v1);
+                pp[part][o][rt][2 * nt + hf] = *reinterpret_cast<const uint32_t*>(&h2);
+                if (part + 1 < PARTS) {
+                  const float2 h = __bfloat1622float2(h2);
+                  v0 -= h.x;
+                  v1 -= h.y;
+                }
               }
             }
         }
@@ -426,18 +433,13 @@ line_products_kernel(const __grid_constant__ LineParams p) {
             slot ^= 1;
           }
 #pragma unroll
-          for (int rt = 0; rt < RT; ++rt)
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-              mma16816(acc[o][rt][2 * j + c], ph[o][rt][0], ph[o][rt][1], ph[o][rt][2], ph[o][rt][3], b[c / 2][2 * (c & 1)],
-                       b[c / 2][2 * (c & 1) + 1]);
-          if (SPLIT)
+          for (int part = 0; part < PARTS; ++part)
 #pragma unroll
             for (int rt = 0; rt < RT; ++rt)
 #pragma unroll
               for (int c = 0; c < 8; ++c)
-                mma16816(acc[o][rt][2 * j + c], pl[o][rt][0], pl[o][rt][1], pl[o][rt][2], pl[o][rt][3], b[c / 2][2 * (c & 1)],
-                         b[c / 2][2 * (c & 1) + 1]);
+                mma16816(acc[o][rt][2 * j + c], pp[part][o][rt][0], pp[part][o][rt][1], pp[part][o][rt][2], pp[part][o][rt][3],
+                         b[c / 2][2 * (c & 1)], b[c / 2][2 * (c & 1) + 1]);
         }
       }
     }
@@ -471,11 +473,11 @@ line_products_kernel(const __grid_constant__ LineParams p) {
   }
 }
 
-template <int RT, bool DUAL, bool GATED, bool SPLIT>
+template <int RT, bool DUAL, bool GATED, int PARTS>
 cudaError_t launch_lines(const LineParams& p, cudaStream_t st) {
   using L = LineSmem<RT, DUAL>;
   static_assert(L::warps_per_sm * (L::bytes + 1024) <= 228 * 1024, "the rings of an SM");
-  auto* kernel = line_products_kernel<RT, DUAL, GATED, SPLIT>;
+  auto* kernel = line_products_kernel<RT, DUAL, GATED, PARTS>;
   const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::bytes);
   if (err != cudaSuccess) return err;
   const uint32_t most = (uint32_t)smat_sm_count() * L::warps_per_sm;
@@ -517,7 +519,9 @@ bool smat_lines_supported(const SmatGeo& geo, int bh) {
 
 // The line lies where the gathered bytes (from the L2 cache) pass the tables' (to and from memory) by a limit; the pass in us, with
 // tables / without.  Forward 2.3: d = 3, q = 29, 16 heads, ratio 1.7 (24 K tokens) 648 / 387, 2.1 (28 K) 673 / 607, 2.3 (32 K) 696 / 677, 2.9
-// (40 K) 765 / 850; d = 4, q = 11, 16 heads, 2.0 (10,240) 608 / 536, 2.5 (12,288) 615 / 643.  Plans made for training steps 1.75, since dK
+// (40 K) 765 / 850; d = 4, q = 11, 16 heads, 2.0 (10,240) 608 / 536, 2.5 (12,288) 615 / 643; with fp32 tables d = 2, 16 heads, 2.0
+// (34,880) 1097 / 392; d = 3, 8 heads, 1.4 (41,024) 1159 / 637.  From d = 4 with fp32 tables (three products a stage) 1.85: d = 4, 8
+// heads, 1.7 (16,448) 717 / 671, 2.0 (19,520) 733 / 769, 2.2 (22,592) 748 / 867.  Plans made for training steps 1.75, since dK
 // and dV take two products of a gather: d = 4, 8 heads, 1.5 (7168) 845 / 751, 2.0 (8192) 851 / 876, gated 974 / 1019.  d = 2 with a bf16
 // table 0.75: there is one, and its pooling and read are near the memory rate; 32 heads, 0.7 (4096) 85 / 83 and the training step
 // 250 / 237, 16 heads, 0.8 (6144), the training step 210.7 / 214.5.  Types of less than two tokens leave the row tile empty: 16
@@ -530,7 +534,7 @@ bool smat_lines_pay(const SmatGeo& geo, int bh, int table_bytes, bool trains) {
   const LineShape s = line_shape(geo, bh, 1);
   const double gathered = (double)s.groups * s.blocks * s.slots * 512;
   const double tables = 2.0 * (double)(geo.P + (geo.D == 1 ? 0 : geo.B)) * 16384 * table_bytes;
-  const double limit = geo.D == 1 && table_bytes == 2 ? 0.75 : trains ? 1.75 : 2.3;
+  const double limit = geo.D == 1 && table_bytes == 2 ? 0.75 : trains ? 1.75 : geo.D >= 3 && table_bytes == 4 ? 1.85 : 2.3;
   return s.items >= (table_bytes == 2 ? 6 * SMS : SMS) && gathered <= limit * tables;
 }
 
@@ -608,13 +612,15 @@ cudaError_t smat_launch_line_products(const SmatLineArgs& a, const SmatGeo& geo,
   p.out1 = a.out1; p.out2 = a.out2; p.out_f32 = a.out_f32; p.ones = a.ones;
   p.copy = static_cast<__nv_bfloat16*>(a.copy); p.copy_head = a.copy_head; p.copy_swap = a.copy_swap; p.mark = a.mark; p.mark_value = a.mark_value;
   p.lam = a.lam;
-  if (a.out2) {
-    return a.lam ? launch_lines<1, true, true, false>(p, st) : launch_lines<1, true, false, false>(p, st);
-  }
+  if (a.out2) return a.lam ? launch_lines<1, true, true, 1>(p, st) : launch_lines<1, true, false, 1>(p, st);
   if (line_shape(geo, bh, a.rows_are_types).rt == 1) {
-    if (a.lam) return launch_lines<1, false, true, false>(p, st);
-    return a.split ? launch_lines<1, false, false, true>(p, st) : launch_lines<1, false, false, false>(p, st);
+    if (a.lam) return launch_lines<1, false, true, 1>(p, st);
+    return a.parts == 3   ? launch_lines<1, false, false, 3>(p, st)
+           : a.parts == 2 ? launch_lines<1, false, false, 2>(p, st)
+                          : launch_lines<1, false, false, 1>(p, st);
   }
-  if (a.lam) return launch_lines<2, false, true, false>(p, st);
-  return a.split ? launch_lines<2, false, false, true>(p, st) : launch_lines<2, false, false, false>(p, st);
+  if (a.lam) return launch_lines<2, false, true, 1>(p, st);
+  return a.parts == 3   ? launch_lines<2, false, false, 3>(p, st)
+         : a.parts == 2 ? launch_lines<2, false, false, 2>(p, st)
+                        : launch_lines<2, false, false, 1>(p, st);
 }

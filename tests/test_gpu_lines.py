@@ -123,3 +123,27 @@ def test_non_finite_tokens_reach_no_row_that_does_not_see_them():
     assert not torch.isfinite(dirty[0, 3, geo.n:][~unseen].float()).any(dim=-1).any()
     others = [h for h in range(8) if h != 3]
     assert torch.equal(dirty[0, others], clean[0, others])
+
+
+# (d = 3: 2 heads, 31 rows; d = 2: two tiles of 16 rows; d = 4)
+@pytest.mark.parametrize("d,heads,T", [(3, 2, 2240), (2, 32, 2112), (4, 4, 2240)])
+def test_scores_keep_all_bits_where_tables_would_be_fp32(d, heads, T):
+    """Two tokens of a cell whose scores are 1 + 2^-10 + 2^-20 and 1 + 2^-10 and whose values are opposite: what a row gets is
+    2^-20, exactly, as from an fp32 table (every sum on the way has at most 21 bits).  16 bits of a score would leave nothing."""
+    plan = binding.SmatPlan(1, heads, T, 128, 128, d, 64, "bf16")
+    assert plan.profile_table_element_bytes() == 4
+    geo = so.geometry(T, 64, d)
+    q, k, v = (torch.zeros(1, heads, T, 128, device="cuda", dtype=torch.bfloat16) for _ in range(3))
+    signs = torch.randint(0, 2, (heads, 128), generator=torch.Generator().manual_seed(T)).mul_(2).sub_(1).cuda().bfloat16()
+    first, second = 3, 3 + geo.P
+    assert second < geo.n
+    q[..., :3] = 1
+    k[0, :, (first, second), :2] = torch.tensor([1.0, 2.0 ** -10], device="cuda", dtype=torch.bfloat16)
+    k[0, :, first, 2] = 2.0 ** -20
+    v[0, :, first], v[0, :, second] = signs, -signs
+    O, names = _stages(plan, lambda: plan.forward(q, k, v))
+    assert "read_lines" in names
+    seen = torch.from_numpy(so.mask_col(first, geo)[geo.n:] != 0).cuda()
+    assert seen.any() and not seen.all()
+    assert torch.equal(O[0, :, geo.n:][:, seen], (signs * 2.0 ** -20)[:, None].expand(-1, int(seen.sum()), -1))
+    assert not O[0, :, geo.n:][:, ~seen].any()
