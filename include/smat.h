@@ -250,10 +250,15 @@ smat_status smat_debug_mask(const smat_plan* plan, uint8_t* mask, void* cuda_str
  *                                      fp32-ALU plans, one per 128-token tile (w = 128) on tensor-core plans
  * For d = 1 there is no separate F/U: the single state U_0 = F_0 is carried by the scan, and
  * F and U receive that state (the incoming state of the first recent chunk or tile).
- * Tensor-core plans have per-tile states only after a forward of a plan created with SMAT_FLAG_PER_TILE_STATES, or
- * after smat_backward (plans whose blocks are not whole 128-token tiles: after smat_backward, fp32 per chunk); the
- * two-level form keeps one state per segment of tiles, which is no per-chunk table: there
- * Sin (and, for d = 1, F and U) must be NULL, otherwise SMAT_ERR_UNSUPPORTED is returned.
+ * Tensor-core plans have per-tile states after a forward of a plan created with SMAT_FLAG_PER_TILE_STATES and after
+ * smat_backward (plans whose blocks are not whole 128-token tiles: after smat_backward, fp32 per chunk).  The two-level
+ * form of the other forward passes keeps one state per segment of tiles, which is no per-chunk table: there
+ * Sin (and, for d = 1, F and U) must be NULL, otherwise SMAT_ERR_UNSUPPORTED is returned.  Where a block is no even number
+ * of tiles, or the type table is fp32, that form leaves the per-tile states too if the plan has
+ * SMAT_FLAG_KEEP_FORWARD_TABLES, an fp32 type table, or at most 32768 tokens in all heads; for d = 1 F and U at any size.
+ * Where a forward has formed no tables (see smat_forward), F and U are computed by this call, with the roundings of the
+ * plan's tables, from the K and V that the forward (or backward) left: they verify the routing and the values, but the
+ * pass itself has used no such table.
  * Asynchronous on `cuda_stream`.
  */
 smat_status smat_debug_tables(const smat_plan* plan, const void* workspace, float* F, float* U, float* Sin,

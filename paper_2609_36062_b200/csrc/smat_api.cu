@@ -26,7 +26,8 @@ struct smat_plan {
   size_t off_plist, off_poffs, off_tlist, off_toffs;   // token lists of user-supplied routing (int32)
   size_t off_pheavy, off_theavy;                       // ... and parts of their heavy groups
   size_t off_lr3;         // tensor-core backward: third buffer of bf16 long-range rows (the first two share off_acc)
-  size_t off_sin_tiles;   // KEEP_FORWARD_TABLES on tensor-core plans: the bf16 state entering every tile, left by the forward
+  size_t off_sin_tiles;   // bf16 states entering tiles left_lo .. left_hi - 1, left by a forward in the two-level form (see left_states)
+  int64_t left_lo, left_hi;
   size_t off_lam, off_dlam, off_gq, off_gk, off_glr, off_gdo, off_gv, off_gvlr;   // gated variant (SMAT_FLAG_GATED)
   size_t off_nv, off_ny, off_ndy;   // normalised output (SMAT_FLAG_NORMALIZED): V̄, ȳ and the upstream of the linear pass
   // Gated plans on tensor-core shapes run their FORWARD through a plan of its own (ungated flags, one state per tile)
@@ -47,8 +48,7 @@ struct smat_plan {
   bool fbar_bf16;      // the per-profile adjoint states (transposed tabulation) are kept in bf16
   bool lines;          // positional passes on the tensor cores form the long-range rows without tables (smat_lines.cu)
   mutable int launches;
-  mutable bool tile_states;       // the last call left its incoming states at off_sin (bf16 per 128-token tile; on plans
-                                  // with ragged_tc fp32 per chunk)
+  mutable int states_at;          // TileStates: where the last call left its incoming states
   mutable bool kept_tile_states;  // the last forward left them at off_sin_tiles for the backward (KEEP_FORWARD_TABLES)
   mutable bool kept_gated_forward;  // the last call was the tensor-core gated forward: λ, the rescaled K copies, U and the
                                     // per-tile states are still in the workspace (used under KEEP_FORWARD_TABLES)
@@ -419,6 +419,27 @@ bool forward_rows_f32(const smat_plan* pl) {
          smat_segment_tiles(lr ? pl->geo.n / 128 : pl->T / 128, lr ? pl->geo.m / 128 : 0, pl->bh) < 2;
 }
 
+// Where a call left the states entering its tiles (or chunks): nowhere, at off_sin, or at off_sin_tiles those of tiles left_lo ..
+// left_hi - 1.
+enum TileStates { STATES_NOWHERE = 0, STATES_AT_SIN = 1, STATES_LEFT = 2 };
+// The tiles whose entering states a forward in the two-level form leaves: all where a backward will want them, where the type table
+// is fp32, and where blocks are odd numbers of tiles and the batch is small; a large batch of these at d = 1 the one that is U_0.
+// Stored by every pass, the states of 16 heads of 65,664 tokens (d = 1) took 48 us of 346, of 23,296 (d = 2) 16 of 231, of 22,912
+// (d = 4, 8 heads) 21 of 383; up to 32 K tokens, 8 MB, 0.1 to 0.8 us of 22 to
+// 119.
+void left_states(const smat_plan* pl, int64_t* lo, int64_t* hi) {
+  const int64_t tiles = pl->T / 128;
+  *lo = *hi = 0;
+  if (!pl->tc || (pl->flags & SMAT_FLAG_PER_TILE_STATES)) return;
+  if ((pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES) || (!pl->geo.dense_G && !pl->u_bf16) ||
+      (forward_rows_f32(pl) && (int64_t)pl->bh * pl->T <= 32768)) {
+    *hi = tiles;
+  } else if (forward_rows_f32(pl) && pl->geo.dense_G) {
+    *lo = pl->geo.n / 128;
+    *hi = *lo + 1;
+  }
+}
+
 // Passes that form no tables leave K and V of the distant tokens in their place, for smat_debug_tables: in the long-range
 // buffer, beside the fp32 rows of the recent tokens (mark 1) or behind the bf16 rows of all (mark 2).
 enum LineCopy { LINE_COPY_NONE = 0, LINE_COPY_BESIDE = 1, LINE_COPY_BEHIND = 2 };
@@ -514,7 +535,7 @@ smat_status smat_plan_create(smat_plan** out, int batch, int heads, int64_t T, i
   pl->batch = batch; pl->heads = heads; pl->bh = batch * heads;
   pl->r = d_k; pl->p = d_v; pl->T = T; pl->c = chunk; pl->NC = T / chunk;
   pl->dtype = dtype; pl->flags = flags; pl->rp = (int64_t)d_k * d_v; pl->launches = 0;
-  pl->profiling = false; pl->stages = 0; pl->tile_states = false; pl->kept_tile_states = false;
+  pl->profiling = false; pl->stages = 0; pl->states_at = STATES_NOWHERE; pl->kept_tile_states = false;
   pl->kept_gated_forward = false; pl->forward_left = 0;
   smat_status s = build_geometry(&pl->geo, T, chunk, d, q_override);
   if (s != SMAT_OK) { delete pl; return s; }
@@ -564,8 +585,9 @@ smat_status smat_plan_create(smat_plan** out, int batch, int heads, int64_t T, i
   pl->off_U = off;      off = align_up(off + (g.dense_G ? 0 : (size_t)pl->bh * g.B * entries * (pl->u_bf16 ? 2 : 4)));
   pl->off_acc = off;    off = align_up(off + (size_t)pl->bh * T * wide * sizeof(float));
   pl->off_W = off;      off = align_up(off + (pl->tab_tc ? (size_t)smat_tabulate_tc_scratch_elems(g, pl->rp, pl->bh) * 2 : 0));
+  left_states(pl, &pl->left_lo, &pl->left_hi);
   pl->off_sin_tiles = off;
-  off = align_up(off + (pl->tc && (flags & SMAT_FLAG_KEEP_FORWARD_TABLES) ? (size_t)pl->bh * (T / 128) * entries * 2 : 0));
+  off = align_up(off + (size_t)pl->bh * (pl->left_hi - pl->left_lo) * entries * 2);
   const bool lists = !g.dense_G;
   pl->off_plist = off;  off = align_up(off + (lists ? (size_t)pl->bh * g.n * 4 : 0));
   pl->off_poffs = off;  off = align_up(off + (lists ? (size_t)pl->bh * (g.P + 1) * 4 : 0));
@@ -744,7 +766,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
       else
         state_read(cx, "read_type", {read_job(cx, SMAT_GM_TYPE, Q, cx.f(pl->off_U), 0, ylr)});
     }
-    pl->tile_states = per_tile;
+    pl->states_at = per_tile ? STATES_AT_SIN : forward_rows_f32(pl) && pl->left_hi ? STATES_LEFT : STATES_NOWHERE;
     pl->kept_tile_states = false;
     if (!per_tile) {  // steps 5-7, two-level: segment totals, scan of the totals, fused per-segment output
       const int64_t rows0 = tiles0 * 128, rows1 = tiles1 * 128;
@@ -753,7 +775,8 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
       const bool keep = (pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES) != 0;   // a backward will want the per-tile states
       SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, cx.f(pl->off_sin), ylr, f32, 0, lr ? pl->geo.n : pl->T, O,
                                                                        rows0, rows1, sg.nseg0, sg.nseg1, pl->bh, status, cx.st,
-                                                                       keep ? cx.ws + pl->off_sin_tiles : nullptr, divide));
+                                                                       pl->left_hi ? cx.ws + pl->off_sin_tiles : nullptr, pl->left_lo,
+                                                                       pl->left_hi, divide));
       pl->kept_tile_states = keep;
     } else {
       SMAT_TRY(cx, "chunk_scan_tc", smat_launch_chunk_scan_tc(K, V, cx.ws + pl->off_sin, pl->T, pl->bh, pl->geo.n,
@@ -766,7 +789,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;
   }
   if (pl->ragged_tc) {
-    pl->tile_states = false;
+    pl->states_at = STATES_NOWHERE;
     // Blocks that are not whole tiles: tables as on the fp32-ALU path (steps 2-4), the causal branch in its two-level
     // form over tiles of which the last of a block is partial.
     int* status = reinterpret_cast<int*>(cx.ws + pl->off_status);
@@ -787,7 +810,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     const Segments sg = segment_totals(cx, K, V, rows0, rows1, 2, divide);
     SMAT_TRY(cx, "segment_output_tc", smat_launch_segment_output_tc(Q, K, V, cx.f(pl->off_sin), ylr, 1, 1, lr ? pl->geo.n : pl->T, O, rows0,
                                                                      rows1, sg.nseg0, sg.nseg1, pl->bh, status, cx.st, nullptr,
-                                                                     divide));
+                                                                     0, 0, divide));
     pl->launches = cx.launches;
     return cx.err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;
   }
@@ -836,7 +859,7 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
     // With KEEP_FORWARD_TABLES the preceding forward has left the state entering every tile: no second scan of K, V
     const bool kept = (pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES) && pl->kept_tile_states;
     void* sin_tiles = cx.ws + (kept ? pl->off_sin_tiles : pl->off_sin);
-    pl->tile_states = !kept;
+    pl->states_at = kept ? STATES_LEFT : STATES_AT_SIN;
     const SmatGroupSpec types = group(cx, SMAT_GM_TYPE), profs = group(cx, SMAT_GM_PROFILE);
     const int64_t n = pl->geo.n;
     if (lr) {
@@ -955,7 +978,7 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
   }
   // fp32-ALU path: every state of both directions from one pooling launch; S̄_in_b = Q_bᵀ dO_b and D̄ = its exclusive
   // suffix scan (scan adjoint); Ū_h = Σ q dOᵀ over the type, F̄ = Cᵀ Ū (Eq. "lr-adjoint").
-  pl->tile_states = true;
+  pl->states_at = STATES_AT_SIN;
   float *sin = cx.f(pl->off_sin), *dbar = cx.f(pl->off_dbar);
   float *acc = cx.f(pl->off_acc), *acc_v = cx.f(pl->off_acc2);
   const SmatPoolJob cf = pool_job(cx, SMAT_GM_CHUNK, K, V, sin), cb = pool_job(cx, SMAT_GM_CHUNK, Q, dO, dbar);
@@ -1219,7 +1242,7 @@ smat_status smat_forward_gated(const smat_plan* pl, const void* Q, const void* K
   if (!device_ok()) return SMAT_ERR_ARCH;
   Ctx cx{pl, static_cast<cudaStream_t>(cuda_stream), static_cast<char*>(workspace), cudaSuccess, 0};
   pl->stages = 0;
-  pl->tile_states = false;
+  pl->states_at = STATES_NOWHERE;
   cx.err = clear_status(cx);
   const Gated gt = gated_buffers(cx);
   if (pl->inner) return forward_gated_tc(cx, gt, Q, K, V, log_a, O);
@@ -1252,7 +1275,7 @@ smat_status smat_backward_gated(const smat_plan* pl, const void* Q, const void* 
   if (!device_ok()) return SMAT_ERR_ARCH;
   Ctx cx{pl, static_cast<cudaStream_t>(cuda_stream), static_cast<char*>(workspace), cudaSuccess, 0};
   pl->stages = 0;
-  pl->tile_states = false;
+  pl->states_at = STATES_NOWHERE;
   const bool after_gated_forward = pl->kept_gated_forward;   // read before the pass resets it
   cx.err = clear_status(cx);
   const bool lr = !pl->geo.dense_G;
@@ -1356,19 +1379,23 @@ smat_status smat_debug_tables(const smat_plan* pl, const void* workspace, float*
   const size_t state = (size_t)pl->rp * sizeof(float);
   cudaError_t err = cudaSuccess;
   // blocks that are not whole tiles: per-chunk states exist only after the (fp32-ALU) backward
-  if (pl->ragged_tc && (Sin || (pl->geo.dense_G && (F || U))) && !pl->tile_states) return SMAT_ERR_UNSUPPORTED;
+  if (pl->ragged_tc && (Sin || (pl->geo.dense_G && (F || U))) && pl->states_at == STATES_NOWHERE)
+    return SMAT_ERR_UNSUPPORTED;
   if (pl->tc) {
-    // Tensor-core plans: incoming states exist per 128-token tile (bf16) after a per-tile forward or a backward; the
-    // two-level form keeps only one state per segment of tiles, which is no per-chunk table.
+    // Tensor-core plans: incoming states exist per 128-token tile (bf16) after a per-tile forward or a backward, and where a
+    // forward in the two-level form has left them; the other ones keep only one state per segment of tiles, which is no
+    // per-chunk table.
+    const int64_t tiles = pl->T / 128, lo = pl->states_at == STATES_LEFT ? pl->left_lo : 0,
+                  count = (pl->states_at == STATES_LEFT ? pl->left_hi : tiles) - lo;
     const bool want_states = Sin || (pl->geo.dense_G && (F || U));
-    if (want_states && !pl->tile_states) return SMAT_ERR_UNSUPPORTED;
-    const int64_t tiles = pl->T / 128;
-    if (Sin) err = smat_launch_widen_bf16(ws + pl->off_sin, Sin, (int64_t)pl->bh * tiles * pl->rp, st);
+    if (want_states && (pl->states_at == STATES_NOWHERE || (Sin && count != tiles))) return SMAT_ERR_UNSUPPORTED;
+    const char* states = ws + (pl->states_at == STATES_LEFT ? pl->off_sin_tiles : pl->off_sin);
+    if (Sin) err = smat_launch_widen_bf16(states, Sin, (int64_t)pl->bh * tiles * pl->rp, st);
     if (pl->geo.dense_G) {  // d = 1: the state entering the first recent tile is U_0 = F_0
       for (int t = 0; t < 2; ++t) {
         float* dst = t ? U : F;
         for (int h = 0; dst && h < pl->bh && err == cudaSuccess; ++h)
-          err = smat_launch_widen_bf16(ws + pl->off_sin + ((size_t)h * tiles + pl->geo.n / 128) * pl->rp * 2,
+          err = smat_launch_widen_bf16(states + ((size_t)h * count + pl->geo.n / 128 - lo) * pl->rp * 2,
                                        dst + (size_t)h * pl->rp, pl->rp, st);
       }
       return err == cudaSuccess ? SMAT_OK : SMAT_ERR_LAUNCH;

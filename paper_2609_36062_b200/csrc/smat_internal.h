@@ -286,7 +286,7 @@ cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* to
 cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const void* V, const float* seg_in,
                                           const void* ylr, int ylr_f32, int split, int64_t n_lr, void* O, int64_t rows0, int64_t rows1,
                                           int nseg0, int nseg1, int bh, int* status, cudaStream_t st,
-                                          void* sin_tiles = nullptr, int divide = 0);
+                                          void* sin_tiles = nullptr, int64_t sin_lo = 0, int64_t sin_hi = 0, int divide = 0);
 // Long-range rows without tables (see smat_lines.cu), positional routing, bf16 rows of 128: for every token t of a type (or,
 // rows_are_types = 0, of a cell) out1_t = Σ_s (x1_t · y_s) z_s over the tokens s of the cells of its hyperplane (of the types
 // through the cell), and with out2 also out2_t = Σ_s (x2_t · z_s) y_s.

@@ -983,7 +983,8 @@ struct SegOutParams {
   const __nv_bfloat16* ylr;   // [bh][T][128] long-range rows, bf16 (rows t >= n_lr are added)
   const float* ylr32;         // Y32: the same rows in fp32
   __nv_bfloat16* O;
-  __nv_bfloat16* sin_tiles;   // plain, optional [bh][T/128][128][128]: the bf16 state entering every tile, for a later backward
+  __nv_bfloat16* sin_tiles;   // plain, optional [bh][sin_hi - sin_lo][128][128]: the bf16 states entering these tiles, for a later backward
+  int64_t sin_lo, sin_hi;
   int* status;
 };
 
@@ -1226,8 +1227,9 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS + 32 * DIVIDE) segment_output_
       fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_s);   // one arrival per warp: 512 arrivals on one barrier serialise
-      if (!SPLIT && prm.sin_tiles) {
-        __nv_bfloat16* dst = prm.sin_tiles + (((int64_t)bh * (prm.T / TILE) + tile) * TILE + m - odd) * TILE + col0 + 16 * odd;
+      if (!SPLIT && tile >= prm.sin_lo && tile < prm.sin_hi) {
+        __nv_bfloat16* dst = prm.sin_tiles + (((int64_t)bh * (prm.sin_hi - prm.sin_lo) + tile - prm.sin_lo) * TILE + m - odd) * TILE +
+                             col0 + 16 * odd;
         swap_rows(odd, pk[0], pk[1], pk[2], pk[3]);
         st_global_v8(dst, pk[0].x, pk[0].y, pk[0].z, pk[0].w, pk[1].x, pk[1].y, pk[1].z, pk[1].w);
         st_global_v8(dst + TILE, pk[2].x, pk[2].y, pk[2].z, pk[2].w, pk[3].x, pk[3].y, pk[3].z, pk[3].w);
@@ -2141,7 +2143,8 @@ cudaError_t smat_launch_segment_state_tc(const void* K, const void* V, float* to
 
 cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const void* V, const float* seg_in,
                                           const void* ylr, int ylr_f32, int split, int64_t n_lr, void* O, int64_t rows0, int64_t rows1,
-                                          int nseg0, int nseg1, int bh, int* status, cudaStream_t st, void* sin_tiles, int divide) {
+                                          int nseg0, int nseg1, int bh, int* status, cudaStream_t st, void* sin_tiles, int64_t sin_lo,
+                                          int64_t sin_hi, int divide) {
   const int64_t T = rows0 + rows1;
   SegOutMaps maps;
   const void* src[3] = {Q, K, V};
@@ -2159,6 +2162,7 @@ cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const vo
   prm.cut = segment_cut(rows0, rows1, nseg0, nseg1);
   prm.O = static_cast<__nv_bfloat16*>(O);
   prm.sin_tiles = static_cast<__nv_bfloat16*>(sin_tiles);
+  prm.sin_lo = sin_lo; prm.sin_hi = sin_tiles ? sin_hi : 0;
   prm.status = status;
   if (split && !ylr_f32) return cudaErrorInvalidValue;
   auto kernel = split     ? (divide ? segment_output_tc_kernel<true, true, true> : segment_output_tc_kernel<true, true, false>)
