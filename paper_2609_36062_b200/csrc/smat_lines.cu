@@ -409,14 +409,16 @@ line_products_kernel(const __grid_constant__ LineParams p) {
         for (int i = 0; i < LN_STEP / 2; ++i) {
           const uint32_t r = crow + 2 * i;
           const uint32_t t = __shfl_sync(0xffffffffu, tok.t, half + r);
-          if (!__shfl_sync(0xffffffffu, (int)tok.there, half + r)) continue;
-          uint32_t w[4];
-          uint4* dst = reinterpret_cast<uint4*>(p.copy + ((int64_t)cur.bh * p.copy_head + t) * 256) + cpiece;
-          lds16(ring + tile + piece(r, cpiece), w);
-          dst[p.copy_swap ? 16 : 0] = make_uint4(w[0], w[1], w[2], w[3]);
-          lds16(ring + tile + 4096 + piece(r, cpiece), w);
-          if (p.ones && cpiece == 15) w[3] = __byte_perm(w[3], 0x3f800000u, 0x7610);
-          dst[p.copy_swap ? 0 : 16] = make_uint4(w[0], w[1], w[2], w[3]);
+          if (__shfl_sync(0xffffffffu, (int)tok.there, half + r)) {   // (the halves of the warp copy different rows)
+            uint32_t w[4];
+            uint4* dst = reinterpret_cast<uint4*>(p.copy + ((int64_t)cur.bh * p.copy_head + t) * 256) + cpiece;
+            lds16(ring + tile + piece(r, cpiece), w);
+            dst[p.copy_swap ? 16 : 0] = make_uint4(w[0], w[1], w[2], w[3]);
+            lds16(ring + tile + 4096 + piece(r, cpiece), w);
+            if (p.ones && cpiece == 15) w[3] = __byte_perm(w[3], 0x3f800000u, 0x7610);
+            dst[p.copy_swap ? 0 : 16] = make_uint4(w[0], w[1], w[2], w[3]);
+          }
+          __syncwarp();   // the products behind are instructions of the whole warp
         }
       }
 #pragma unroll
