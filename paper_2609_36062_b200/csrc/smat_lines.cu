@@ -608,6 +608,8 @@ cudaError_t smat_launch_line_tables(const SmatGeo& geo, int bh, const int* mark,
 }
 
 cudaError_t smat_launch_line_products(const SmatLineArgs& a, const SmatGeo& geo, int bh, cudaStream_t st) {
+  // (score parts and the ones column: of one ungated product)
+  if (a.parts < 1 || a.parts > 3 || ((a.parts > 1 || a.ones) && (a.out2 || a.lam))) return cudaErrorInvalidValue;
   LineParams p = line_geometry(geo, line_shape(geo, bh, a.rows_are_types, a.out2 != nullptr), a.rows_are_types);
   using B16 = const __nv_bfloat16;
   p.x1 = static_cast<B16*>(a.x1); p.x2 = static_cast<B16*>(a.x2); p.y = static_cast<B16*>(a.y); p.z = static_cast<B16*>(a.z);

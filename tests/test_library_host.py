@@ -266,3 +266,26 @@ def test_rows_without_tables_keep_every_launch_inside_its_quotients(q, bh, fits)
     last_of_a_head = np.arange(per - 1, items, per, dtype=np.uint64)
     exact = bool(np.all(last_of_a_head * np.uint64(inverse) >> np.uint64(32) == last_of_a_head // np.uint64(per)))
     assert exact or not fits
+
+
+class _LineArgs(ctypes.Structure):   # SmatLineArgs of csrc/smat_internal.h
+    _fields_ = [(f, ctypes.c_void_p) for f in ("x1", "x2", "y", "z", "out1", "out2")] + \
+               [(f, ctypes.c_int) for f in ("out_f32", "rows_are_types", "ones", "parts")] + \
+               [("lam", ctypes.c_void_p), ("copy", ctypes.c_void_p), ("copy_head", ctypes.c_int64), ("copy_swap", ctypes.c_int),
+                ("mark", ctypes.c_void_p), ("mark_value", ctypes.c_int)]
+
+
+@pytest.mark.parametrize("args", [dict(parts=0), dict(parts=4), dict(parts=2, out2=256), dict(parts=3, lam=256),
+                                  dict(parts=1, ones=1, out2=256), dict(parts=1, ones=1, lam=256)])
+def test_rows_without_tables_refuse_what_their_kernels_would_ignore(args):
+    """Several score parts and the ones column exist in the single ungated product only; the launcher says so before it
+    reaches a device (cudaErrorInvalidValue is 1)."""
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("a device is present: a launcher without the check would launch")
+    g = binding.SmatPlan(1, 2, 2048, 128, 128, 3, 128, "bf16").geometry()
+    geo = _SmatGeo(T=g.T, c=g.c, n=g.n, m=g.m, d=3, q=g.q, D=2, P=g.P, A=g.A, B=g.B, nnzC=g.nnzC)
+    geo.qpow[:3], geo.dir_group_start[:2] = (1, g.q, g.q ** 2), (0, g.q)
+    launch = binding.load_library()["_Z25smat_launch_line_productsRK12SmatLineArgsRK7SmatGeoiP11CUstream_st"]
+    launch.restype, launch.argtypes = ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p]
+    assert launch(ctypes.byref(_LineArgs(rows_are_types=1, **args)), ctypes.byref(geo), 2, None) == 1
