@@ -52,7 +52,8 @@ struct smat_plan {
   mutable bool kept_tile_states;  // the last forward left them at off_sin_tiles for the backward (KEEP_FORWARD_TABLES)
   mutable bool kept_gated_forward;  // the last call was the tensor-core gated forward: λ, the rescaled K copies, U and the
                                     // per-tile states are still in the workspace (used under KEEP_FORWARD_TABLES)
-  mutable int forward_left;         // LineCopy: what the last forward left in the tables' place (0: it formed the tables)
+  mutable unsigned forwards_left;   // a bit 1 << LineCopy for each kind of thing that this plan's forwards have left in the tables'
+                                    // place: which of them a workspace holds is known where it is the only one
   // optional per-launch timing (smat_profile_enable): event k is recorded before launch k
   mutable bool profiling;
   mutable cudaEvent_t events[SMAT_MAX_STAGES + 1];
@@ -536,7 +537,7 @@ smat_status smat_plan_create(smat_plan** out, int batch, int heads, int64_t T, i
   pl->r = d_k; pl->p = d_v; pl->T = T; pl->c = chunk; pl->NC = T / chunk;
   pl->dtype = dtype; pl->flags = flags; pl->rp = (int64_t)d_k * d_v; pl->launches = 0;
   pl->profiling = false; pl->stages = 0; pl->states_at = STATES_NOWHERE; pl->kept_tile_states = false;
-  pl->kept_gated_forward = false; pl->forward_left = 0;
+  pl->kept_gated_forward = false; pl->forwards_left = 0;
   smat_status s = build_geometry(&pl->geo, T, chunk, d, q_override);
   if (s != SMAT_OK) { delete pl; return s; }
   const SmatGeo& g = pl->geo;
@@ -742,7 +743,8 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     float* ylr = cx.f(pl->off_acc);
     const bool lr = !pl->geo.dense_G;
     const bool lines = pl->lines && !cx.routed;
-    pl->forward_left = LINE_COPY_NONE;
+    const LineCopy left = !lines ? LINE_COPY_NONE : forward_rows_f32(pl) ? LINE_COPY_BESIDE : LINE_COPY_BEHIND;
+    pl->forwards_left |= 1u << left;
     if (lr && !lines) build_type_table(cx, K, V);                                            // steps 2-3
     // The causal branch is the two-level one wherever the plan does not ask for per-tile states: blocks of any number of tiles
     // are cut into segments that differ by a tile at most (odd numbers took the per-tile form: d = 2, 16 heads of 13,056 tokens
@@ -753,9 +755,8 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
     if (lines) {                                                                             // steps 2-4 in one
       SmatLineArgs a = line_job(1, Q, K, V, ylr, f32, table_parts(pl));
       a.ones = divide;
-      pl->forward_left = f32 ? LINE_COPY_BESIDE : LINE_COPY_BEHIND;
-      line_copy(cx, &a, pl->forward_left, false);
-      line_mark(cx, &a, pl->forward_left);
+      line_copy(cx, &a, left, false);
+      line_mark(cx, &a, left);
       line_rows(cx, "read_lines", a);
     } else if (lr) {                                                                         // step 4
       zero_unrouted(cx, SMAT_GM_TYPE, ylr, f32 ? 512 : 256);
@@ -864,8 +865,8 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
     const int64_t n = pl->geo.n;
     if (lr) {
       const bool lines = pl->lines && !cx.routed;
-      const bool after_forward = (pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES) != 0;
-      if (!lines && !(after_forward && pl->forward_left == LINE_COPY_NONE)) build_type_table(cx, K, V);
+      auto forward_left = [&](LineCopy what) { return (pl->flags & SMAT_FLAG_KEEP_FORWARD_TABLES) && pl->forwards_left == 1u << what; };
+      if (!lines && !forward_left(LINE_COPY_NONE)) build_type_table(cx, K, V);
       // Ū_h = Σ q dOᵀ over the type (Eq. "lr-adjoint"), then F̄ = Cᵀ Ū
       const bool ubar_tc = pl->ubar_tc, ubar_bf16 = pl->ubar_bf16;
       if (lines) {
@@ -883,7 +884,7 @@ smat_status backward_impl(const smat_plan* pl, const void* Q, const void* K, con
         tabulate(cx, "bwd_tabulate_t", cx.f(pl->off_ubar), cx.f(pl->off_fbar), 1, pl->geo.D == 2 && pl->fbar_bf16);
       // dQ's long-range rows without tables; K and V of the distant tokens are behind them already where the forward left them
       SmatLineArgs dq_lines = line_job(1, dO, V, K, lrbuf, 0, table_parts(pl));
-      if (!(after_forward && pl->forward_left == LINE_COPY_BEHIND)) line_copy(cx, &dq_lines, LINE_COPY_BEHIND, true);
+      if (!forward_left(LINE_COPY_BEHIND)) line_copy(cx, &dq_lines, LINE_COPY_BEHIND, true);
       line_mark(cx, &dq_lines, LINE_COPY_BEHIND);
       // per-tile states
       if (!kept)

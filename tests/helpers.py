@@ -29,6 +29,24 @@ def device_inputs(w: synth.Workload, tensors=("q", "k", "v")):
     return host, dev
 
 
+def positional_arrays(plan):
+    """The positional assignment as the explicit arrays of a routed call (packed cells, types): a call with them forms tables
+    on every plan with d > 1, also where the positional call does without."""
+    geo, bh = plan.geometry(), plan.shape[0] * plan.shape[1]
+    prof = (torch.arange(geo.n, device="cuda") % geo.P).int()
+    typ = ((torch.arange(geo.m, device="cuda") + 1) % geo.B).int()
+    return {"prof": prof.repeat(bh, 1), "type": typ.repeat(bh, 1)}
+
+
+def stages(plan, call):
+    """What call() returns, and the names of the kernels that the plan's last pass in it launched."""
+    plan.profile_enable(True)
+    out = call()
+    names = [name for name, _ in plan.profile_read()]
+    plan.profile_enable(False)
+    return out, names
+
+
 def rel_err(got: np.ndarray, ref: np.ndarray) -> float:
     denom = float(np.max(np.abs(ref)))
     return float(np.max(np.abs(got - ref))) / (denom if denom > 0 else 1.0)

@@ -8,7 +8,7 @@ import torch
 from oracle import chunkwise_ref as cw
 from oracle import smat_oracle as so
 from paper_2609_36062_b200 import binding, synth
-from tests.helpers import TOL, device_inputs, rel_err, sample_tokens, to_numpy64
+from tests.helpers import TOL, device_inputs, positional_arrays, rel_err, sample_tokens, to_numpy64
 
 pytestmark = pytest.mark.gpu
 
@@ -147,3 +147,53 @@ def test_scores_keep_all_bits_where_tables_would_be_fp32(d, heads, T):
     assert seen.any() and not seen.all()
     assert torch.equal(O[0, :, geo.n:][:, seen], (signs * 2.0 ** -20)[:, None].expand(-1, int(seen.sum()), -1))
     assert not O[0, :, geo.n:][:, ~seen].any()
+
+
+# even and odd numbers of tiles, row tiles of 16 and 32, several row blocks, partial tiles (forward alone)
+@pytest.mark.parametrize("d,heads,T,c,q", [(3, 8, 2048, 128, 0), (3, 16, 2176, 128, 0), (2, 40, 3456, 128, 0), (3, 20, 2048, 128, 7),
+                                           (4, 8, 4096, 64, 0), (3, 8, 2240, 64, 0)])
+def test_rows_without_tables_agree_with_rows_from_tables(d, heads, T, c, q):
+    """The positional call against the routed one with the same assignment.  Stored values are rounded on both sides (2^-9 of the
+    largest each), tables twice (F, U), scores once, all to eight bits: five times 2^-9 in all."""
+    w = synth.Workload("both", d, 1, heads, T, 128, 128, c, "bf16", "normalised", 500 + T)
+    _, dev = device_inputs(w, ("q", "k", "v", "do"))
+    plan = _plan(w, q=q)
+    arrays = positional_arrays(plan)
+    args = [dev[x] for x in ("q", "k", "v")]
+    a, ran = _stages(plan, lambda: plan.forward(*args))
+    b, ran_tables = _stages(plan, lambda: plan.forward(*args, **arrays))
+    assert "read_lines" in ran and "read_lines" not in ran_tables
+    assert torch.equal(a, plan.forward(*args)) and torch.equal(b, plan.forward(*args, **arrays))   # (each repeats itself)
+    got = [(a, b)]
+    if plan.geometry().n % 128 == 0:
+        got += zip(plan.backward(*args, dev["do"]), plan.backward(*args, dev["do"], **arrays))
+    plan.check_status()
+    for x, y in got:
+        assert rel_err(to_numpy64(x), to_numpy64(y)) <= 5 * 2.0 ** -9
+
+
+@pytest.mark.parametrize("forward,backward", [("positions", "positions"), ("positions", "arrays"), ("arrays", "positions"), ("arrays", "arrays")])
+@pytest.mark.parametrize("between", [None, "positions", "arrays"])
+def test_kept_passes_in_any_order_of_routed_and_positional(forward, backward, between):
+    """KEEP_FORWARD_TABLES on a plan whose positional passes form no tables: a backward builds what the forward of its workspace
+    has not left, whichever forward the plan has run last (`between`: one of other inputs on a workspace of its own)."""
+    w = synth.Workload("orders", 3, 1, 8, 2048, 128, 128, 128, "bf16", "normalised", 97)
+    host, dev = device_inputs(w, ("q", "k", "v", "do"))
+    plan = _plan(w, binding.FLAG_KEEP_FORWARD_TABLES)
+    arrays = positional_arrays(plan)
+    pick = {"positions": {}, "arrays": arrays}
+    args = [dev[x] for x in ("q", "k", "v")]
+    ws = plan.workspace(for_backward=True).fill_(255)             # (nothing of another run's tables)
+    plan.forward(*args, workspace=ws, **pick[forward])
+    if between:
+        plan.forward(dev["k"], dev["q"], dev["do"], workspace=torch.empty_like(ws), **pick[between])
+    grads = plan.backward(*args, dev["do"], workspace=ws, **pick[backward])
+    plan.check_status(ws)
+    F, U, _ = plan.debug_tables(workspace=ws)
+    M = so.dense_mask(w.T, w.chunk, w.d)
+    for h in (0, 7):
+        Q64, K64, V64, G64 = (synth.as_float64(w, host[x][h]) for x in ("q", "k", "v", "do"))
+        for got, ref in zip(grads, so.backward_dense(Q64, K64, V64, G64, M)):
+            assert rel_err(to_numpy64(got[0, h]), ref) <= TOL["bf16"]
+        _, tab = cw.forward(Q64, K64, V64, so.geometry(w.T, w.chunk, w.d), return_tables=True)
+        assert rel_err(to_numpy64(F[h]), tab["F"]) <= 8e-3 and rel_err(to_numpy64(U[h]), tab["U"]) <= 1.2e-2   # (bf16 tables)
