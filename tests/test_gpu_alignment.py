@@ -26,6 +26,9 @@ CASES = [   # name, d, T, chunk, d_k, d_v, dtype, flags
     ("per_tile", 3, 2048, 128, 128, 128, "bf16", binding.FLAG_PER_TILE_STATES),
     ("separate_adjoints", 3, 2048, 128, 128, 128, "bf16", binding.FLAG_SEPARATE_TILE_ADJOINTS),
     ("partial_tiles", 3, 1600, 64, 128, 128, "bf16", 0),
+    ("partial_tiles_tables", 2, 1600, 64, 128, 128, "bf16", 0),
+    ("no_tables", 4, 5120, 128, 128, 128, "bf16", 0),
+    ("no_tables_gated", 4, 5120, 128, 128, 128, "bf16", binding.FLAG_GATED),
     ("partial_tiles_causal", 1, 1088, 64, 128, 128, "bf16", 0),
     ("alu_bf16", 2, 512, 32, 64, 128, "bf16", 0),
     ("alu_f32", 3, 512, 64, 128, 64, "f32", 0),

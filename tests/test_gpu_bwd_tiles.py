@@ -5,7 +5,7 @@ import pytest
 import torch
 
 from paper_2609_36062_b200 import binding, synth
-from tests.helpers import device_inputs, rel_err, to_numpy64
+from tests.helpers import device_inputs, positional_arrays, rel_err, stages, to_numpy64
 
 pytestmark = pytest.mark.gpu
 
@@ -32,3 +32,18 @@ def test_gradients_match_the_alu_path(d, T, heads, gated):
         # the stated bounds of bf16 plans: 2e-2 of the largest gradient, 5e-2 for the gate gradient (a suffix sum of
         # differences of two rounded products)
         assert rel_err(x.double().cpu().numpy(), y.double().cpu().numpy()) <= (5e-2 if i == 3 else 2e-2), i
+
+
+@pytest.mark.parametrize("d,T,heads", [(3, 512, 37), (2, 2560, 23)])
+def test_gradients_through_tables_match_the_alu_path(d, T, heads):
+    """The same with long-range rows from the adjoint tables, where the positional call forms none."""
+    w = synth.Workload("tiles", d, 1, heads, T, 128, 128, 128, "bf16", "normalised", 700 + T)
+    _, dev = device_inputs(w, ("q", "k", "v", "do"))
+    plan = binding.SmatPlan(1, heads, T, 128, 128, d, 128, "bf16")
+    alu = binding.SmatPlan(1, heads, T, 128, 128, d, 128, "bf16", flags=binding.FLAG_SIMT_ONLY)
+    args = [dev[x] for x in ("q", "k", "v", "do")]
+    got, ran = stages(plan, lambda: plan.backward(*args, **positional_arrays(plan)))
+    plan.check_status()
+    assert {"pool_tc", "bwd_pool_type_tc", "bwd_dkdv_profile_tc", "bwd_tiles_fused_tc"} <= set(ran)
+    for x, y in zip(got, alu.backward(*args)):
+        assert rel_err(to_numpy64(x), to_numpy64(y)) <= 2e-2     # the stated bound of bf16 plans

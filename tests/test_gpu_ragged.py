@@ -4,9 +4,10 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import chunkwise_ref as cw
 from oracle import smat_oracle as so
 from paper_2609_36062_b200 import binding, synth
-from tests.helpers import device_inputs, rel_err, to_numpy64
+from tests.helpers import device_inputs, positional_arrays, rel_err, stages, to_numpy64
 
 pytestmark = pytest.mark.gpu
 
@@ -42,17 +43,38 @@ def test_partial_tiles_match_the_dense_oracle(d, T, c):
         assert np.linalg.norm(to_numpy64(O[0, h]) - ref) <= 1.02 * np.linalg.norm(to_numpy64(A[0, h]) - ref)
 
 
-def test_rows_past_a_block_do_not_reach_it():
+# ... and through fp32 tables, where the positional call forms none: the cases of several tiles to a block
+@pytest.mark.parametrize("d,T,c", [(3, 320, 32), (4, 1120, 16), (3, 1472, 64), (2, 2368, 64), (3, 4288, 64)])
+def test_partial_tiles_through_tables_match_the_dense_oracle(d, T, c):
+    w, host, dev = _case(d, T, c)
+    plan = binding.SmatPlan(1, 3, T, 128, 128, d, c, "bf16")
+    O, ran = stages(plan, lambda: plan.forward(dev["q"], dev["k"], dev["v"], **positional_arrays(plan)))
+    plan.check_status()
+    assert {"pool", "read_type", "segment_output_tc"} <= set(ran)
+    F, U, _ = plan.debug_tables()
+    geo = so.geometry(T, c, d)
+    M = so.dense_mask(T, c, d)
+    for h in range(w.bh):
+        Q64, K64, V64 = (synth.as_float64(w, host[x][h]) for x in ("q", "k", "v"))
+        assert rel_err(to_numpy64(O[0, h]), so.forward_dense(Q64, K64, V64, M)) <= 2.0 ** -8   # (as above)
+        _, tab = cw.forward(Q64, K64, V64, geo, return_tables=True)
+        assert rel_err(to_numpy64(F[h]), tab["F"]) <= 1e-5 and rel_err(to_numpy64(U[h]), tab["U"]) <= 1e-5   # fp32 sums
+
+
+@pytest.mark.parametrize("tables", [False, True])
+def test_rows_past_a_block_do_not_reach_it(tables):
     """Non-finite keys and values behind a block's end (of the recent block, of the next head) stay out of its rows."""
     w, _, dev = _case(3, 1472, 64)
     plan = binding.SmatPlan(1, 3, w.T, 128, 128, 3, 64, "bf16")
     n = plan.geometry().n
-    clean = plan.forward(dev["q"], dev["k"], dev["v"])
+    arrays = positional_arrays(plan) if tables else {}
+    clean = plan.forward(dev["q"], dev["k"], dev["v"], **arrays)
     k, v = dev["k"].clone(), dev["v"].clone()
     k[0, 0, n:], v[0, 0, n:] = float("inf"), float("nan")
     k[0, 2], v[0, 2] = float("nan"), float("inf")
-    dirty = plan.forward(dev["q"], k, v)
+    dirty, ran = stages(plan, lambda: plan.forward(dev["q"], k, v, **arrays))
     plan.check_status()
+    assert ("pool" in ran) == tables
     assert torch.equal(dirty[0, 0, :n], clean[0, 0, :n]) and torch.equal(dirty[0, 1], clean[0, 1])
 
 

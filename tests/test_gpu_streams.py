@@ -5,6 +5,7 @@ import pytest
 import torch
 
 from paper_2609_36062_b200 import binding
+from tests.helpers import stages
 
 pytestmark = pytest.mark.gpu
 
@@ -17,6 +18,11 @@ PASSES = [
     ("prefill_short", 3, 4, 32, 1024, 128, 128, "bf16", "prefill", 0),
     ("partial_tiles", 3, 1, 8, 3008, 64, 128, "bf16", "prefill", 0),
     ("gated", 3, 1, 8, 4096, 64, 128, "bf16", "gated", KEEP | binding.FLAG_GATED),
+    # the same through tables, which batches of so few heads form
+    ("train_d3_tables", 3, 1, 4, 4096, 64, 128, "bf16", "train", KEEP),
+    ("prefill_d4_tables", 4, 1, 2, 4096, 128, 128, "bf16", "prefill", 0),
+    ("partial_tiles_tables", 3, 1, 1, 1984, 64, 128, "bf16", "prefill", 0),
+    ("gated_tables", 3, 1, 4, 4096, 64, 128, "bf16", "gated", KEEP | binding.FLAG_GATED),
     ("f32", 2, 1, 4, 1024, 64, 64, "f32", "train", 0),
     ("decode", 3, 4, 16, 2048, 64, 128, "bf16", "decode", 0),
     ("decode_gated", 2, 4, 16, 1024, 64, 64, "f32", "decode", binding.FLAG_GATED),
@@ -85,8 +91,19 @@ class Pass:
             assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("name", [n for n in BY_NAME if n.startswith(("train_d3", "prefill_d4", "partial_tiles", "gated"))])
+def test_the_passes_form_tables_or_not_as_their_names_say(name):
+    p = Pass(name, 5)
+    _, ran = stages(p.plan, p.call)
+    tables = {"pool", "pool_tc", "bwd_pool_type_tc"} & set(ran)
+    lines = {"read_lines", "bwd_dkdv_lines"} & set(ran)
+    assert (bool(tables), bool(lines)) == ((True, False) if name.endswith("_tables") else (False, True))
+
+
 @pytest.mark.parametrize("one,other", [("train_d3", "prefill_d4"), ("prefill_d4", "decode"), ("prefill_short", "prefill_d3_q37"),
-                                       ("gated", "partial_tiles"), ("f32", "decode_gated"), ("train_d3", "train_d3")])
+                                       ("gated", "partial_tiles"), ("f32", "decode_gated"), ("train_d3", "train_d3"),
+                                       ("train_d3_tables", "prefill_d4_tables"), ("gated_tables", "partial_tiles_tables"),
+                                       ("train_d3_tables", "train_d3_tables"), ("train_d3_tables", "train_d3")])
 def test_two_plans_on_two_streams(one, other):
     passes = [Pass(one, 1), Pass(other, 2)]
     want = [p.expect() for p in passes]

@@ -7,7 +7,7 @@ import torch
 
 from oracle import smat_oracle as so
 from paper_2609_36062_b200 import binding, synth
-from tests.helpers import device_inputs, rel_err, to_numpy64
+from tests.helpers import device_inputs, positional_arrays, rel_err, stages, to_numpy64
 
 pytestmark = pytest.mark.gpu
 
@@ -18,8 +18,9 @@ def test_type_table_is_the_incidence_sum_of_the_stored_profile_table(d, T, q, he
     w = synth.Workload("wide", d, 1, heads, T, 128, 128, 128, "bf16", "normalised", 300 + q)
     _, dev = device_inputs(w)
     plan = binding.SmatPlan(1, heads, T, 128, 128, d, 128, "bf16", q_override=q)
-    plan.forward(dev["q"], dev["k"], dev["v"])
+    _, ran = stages(plan, lambda: plan.forward(dev["q"], dev["k"], dev["v"], **positional_arrays(plan)))   # (forms tables)
     plan.check_status()
+    assert ("tabulate_wide" if d == 3 and q > 17 else "tabulate_tc") in ran
     F, U, _ = plan.debug_tables()
     geo = so.geometry(T, 128, d, q)
     types = np.unique(np.concatenate([[0, q - 1, q, geo.B - q - 1, geo.B - q, geo.B - 1],
@@ -43,7 +44,8 @@ def test_transposed_stages_match_the_alu_path(d, T, q):
     _, dev = device_inputs(w, ("q", "k", "v", "do"))
     plan = binding.SmatPlan(1, 3, T, 128, 128, d, 128, "bf16", q_override=q)
     alu = binding.SmatPlan(1, 3, T, 128, 128, d, 128, "bf16", q_override=q, flags=binding.FLAG_SIMT_ONLY)
-    got = plan.backward(dev["q"], dev["k"], dev["v"], dev["do"])
+    got, ran = stages(plan, lambda: plan.backward(dev["q"], dev["k"], dev["v"], dev["do"], **positional_arrays(plan)))
     plan.check_status()
+    assert "bwd_tabulate_t_tc" in ran
     for g, r in zip(got, alu.backward(dev["q"], dev["k"], dev["v"], dev["do"])):
         assert rel_err(to_numpy64(g), to_numpy64(r)) <= 2e-2     # the stated bound of bf16 plans
