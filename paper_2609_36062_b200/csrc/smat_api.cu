@@ -143,7 +143,7 @@ struct Ctx {
   cudaError_t err;
   int launches;
   const smat_plan* rec = nullptr;   // plan whose stage timer records the launches (default: pl)
-  int* clear = nullptr;   // status word that the first pooling launch of the pass sets to zero (see begin_pass)
+  int* clear = nullptr;   // status word that the first launch of the pass sets to zero (see begin_pass)
   bool routed = false;   // profile / type groups come from the token lists in the workspace, not from positions
   const int32_t* prof = nullptr;   // the caller's arrays of a routed call
   const int32_t* type = nullptr;
@@ -191,7 +191,7 @@ cudaError_t clear_status(const Ctx& cx) {
   return err;
 }
 
-// The same, left to the pooling launch where the pass begins with it and has an SM for each of its `pooled` states per head:
+// The same, left to the first launch (pooling, or the rows without tables) where that has an SM for each of the `pooled` states per head:
 // a memset among a few short launches costs as much as one of them.  (More CTAs than SMs are better placed after it: those
 // that start while the pass before drains crowd the SMs that are free first.  d = 1, 8 heads of 2048 tokens, 64 wide, chunk
 // 32, forward and backward: 119 us with the memset, 133 without.)
@@ -470,7 +470,10 @@ void line_mark(const Ctx& cx, SmatLineArgs* a, int where) {
   a->mark = reinterpret_cast<int*>(cx.ws + cx.pl->off_status + LINE_MARK);
   a->mark_value = where;
 }
-void line_rows(Ctx& cx, const char* name, const SmatLineArgs& a) {
+// (the launch that a pass may begin with: it clears the status word where begin_pass has left that to it)
+void line_rows(Ctx& cx, const char* name, SmatLineArgs a) {
+  a.clear = cx.clear;
+  cx.clear = nullptr;
   SMAT_TRY(cx, name, smat_launch_line_products(a, cx.pl->geo, cx.pl->bh, cx.st));
 }
 

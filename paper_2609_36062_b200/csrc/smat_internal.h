@@ -303,6 +303,7 @@ struct SmatLineArgs {
   int copy_swap;         // y is V and z is K
   int* mark;             // null, or a word that is set to mark_value
   int mark_value;
+  int* clear;            // null, or a status word that is set to zero
 };
 // Whether the kernel takes the shape, and whether it is the faster way (table_bytes: of an entry of the tables otherwise; trains: a
 // backward follows every forward).

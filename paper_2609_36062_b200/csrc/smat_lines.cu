@@ -36,6 +36,7 @@ struct LineParams {
   int copy_swap;                          // Y holds V and Z holds K
   int* mark;                              // word that says what the workspace holds (null: not wanted)
   int mark_value;
+  int* clear;                             // status word of a pass that begins with this launch, which waits for nothing that could fail
   const float* lam;                       // gated: prefix sums of the log-gates [bh][T]
   int64_t T;
   uint32_t n, m, P, B, q, D;
@@ -201,7 +202,10 @@ line_products_kernel(const __grid_constant__ LineParams p) {
 
   pdl_trigger();
   pdl_wait();
-  if (p.mark && blockIdx.x == 0 && threadIdx.x == 0) *p.mark = p.mark_value;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (p.mark) *p.mark = p.mark_value;
+    if (p.clear) *p.clear = 0;
+  }
   uint32_t it = blockIdx.x;
 
   struct Item {
@@ -615,6 +619,7 @@ cudaError_t smat_launch_line_products(const SmatLineArgs& a, const SmatGeo& geo,
   p.x1 = static_cast<B16*>(a.x1); p.x2 = static_cast<B16*>(a.x2); p.y = static_cast<B16*>(a.y); p.z = static_cast<B16*>(a.z);
   p.out1 = a.out1; p.out2 = a.out2; p.out_f32 = a.out_f32; p.ones = a.ones;
   p.copy = static_cast<__nv_bfloat16*>(a.copy); p.copy_head = a.copy_head; p.copy_swap = a.copy_swap; p.mark = a.mark; p.mark_value = a.mark_value;
+  p.clear = a.clear;
   p.lam = a.lam;
   if (a.out2) return a.lam ? launch_lines<1, true, true, 1>(p, st) : launch_lines<1, true, false, 1>(p, st);
   if (line_shape(geo, bh, a.rows_are_types).rt == 1) {

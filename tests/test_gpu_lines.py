@@ -197,3 +197,19 @@ def test_kept_passes_in_any_order_of_routed_and_positional(forward, backward, be
             assert rel_err(to_numpy64(got[0, h]), ref) <= TOL["bf16"]
         _, tab = cw.forward(Q64, K64, V64, so.geometry(w.T, w.chunk, w.d), return_tables=True)
         assert rel_err(to_numpy64(F[h]), tab["F"]) <= 8e-3 and rel_err(to_numpy64(U[h]), tab["U"]) <= 1.2e-2   # (bf16 tables)
+
+
+@pytest.mark.parametrize("d,heads,T", [(4, 1, 704), (3, 5, 192), (3, 8, 2240)])   # few states (no memset in front), and many
+def test_a_pass_without_tables_begins_with_a_clean_status_word(d, heads, T):
+    w = synth.Workload("clean", d, 1, heads, T, 128, 128, 64, "bf16", "normalised", 98)
+    host, dev = device_inputs(w)
+    plan = _plan(w)
+    plan.workspace().fill_(255)                                   # as a pass whose waits ran out would leave it
+    O, names = _stages(plan, lambda: plan.forward(dev["q"], dev["k"], dev["v"]))   # (checks the status)
+    assert names[0] == "read_lines"
+    M = so.dense_mask(T, 64, d)
+    Q64, K64, V64 = (synth.as_float64(w, host[x][0]) for x in ("q", "k", "v"))
+    assert rel_err(to_numpy64(O[0, 0]), so.forward_dense(Q64, K64, V64, M)) <= 2.0 ** -8   # (rounding of the stored rows)
+    F, U, _ = plan.debug_tables()
+    _, tab = cw.forward(Q64, K64, V64, so.geometry(T, 64, d), return_tables=True)
+    assert rel_err(to_numpy64(F[0]), tab["F"]) <= 1e-5 and rel_err(to_numpy64(U[0]), tab["U"]) <= 1e-5

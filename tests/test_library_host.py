@@ -272,7 +272,7 @@ class _LineArgs(ctypes.Structure):   # SmatLineArgs of csrc/smat_internal.h
     _fields_ = [(f, ctypes.c_void_p) for f in ("x1", "x2", "y", "z", "out1", "out2")] + \
                [(f, ctypes.c_int) for f in ("out_f32", "rows_are_types", "ones", "parts")] + \
                [("lam", ctypes.c_void_p), ("copy", ctypes.c_void_p), ("copy_head", ctypes.c_int64), ("copy_swap", ctypes.c_int),
-                ("mark", ctypes.c_void_p), ("mark_value", ctypes.c_int)]
+                ("mark", ctypes.c_void_p), ("mark_value", ctypes.c_int), ("clear", ctypes.c_void_p)]
 
 
 @pytest.mark.parametrize("args", [dict(parts=0), dict(parts=4), dict(parts=2, out2=256), dict(parts=3, lam=256),
