@@ -984,8 +984,8 @@ struct SegOutParams {
   const float* ylr32;         // Y32: the same rows in fp32
   __nv_bfloat16* O;
   __nv_bfloat16* sin_tiles;   // plain, optional [bh][sin_hi - sin_lo][128][128]: the bf16 states entering these tiles, for a later backward
-  int64_t sin_lo, sin_hi;
   int* status;
+  int sin_lo, sin_hi;
 };
 
 // One CTA per (segment, head), all 128 output columns.
@@ -1228,8 +1228,8 @@ __global__ void __launch_bounds__(SEG_OUT_THREADS + 32 * DIVIDE) segment_output_
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_s);   // one arrival per warp: 512 arrivals on one barrier serialise
       if (!SPLIT && tile >= prm.sin_lo && tile < prm.sin_hi) {
-        __nv_bfloat16* dst = prm.sin_tiles + (((int64_t)bh * (prm.sin_hi - prm.sin_lo) + tile - prm.sin_lo) * TILE + m - odd) * TILE +
-                             col0 + 16 * odd;
+        const int64_t at = (int64_t)bh * (prm.sin_hi - prm.sin_lo) + tile - prm.sin_lo;
+        __nv_bfloat16* dst = prm.sin_tiles + (at * TILE + m - odd) * TILE + col0 + 16 * odd;
         swap_rows(odd, pk[0], pk[1], pk[2], pk[3]);
         st_global_v8(dst, pk[0].x, pk[0].y, pk[0].z, pk[0].w, pk[1].x, pk[1].y, pk[1].z, pk[1].w);
         st_global_v8(dst + TILE, pk[2].x, pk[2].y, pk[2].z, pk[2].w, pk[3].x, pk[3].y, pk[3].z, pk[3].w);
@@ -2162,7 +2162,7 @@ cudaError_t smat_launch_segment_output_tc(const void* Q, const void* K, const vo
   prm.cut = segment_cut(rows0, rows1, nseg0, nseg1);
   prm.O = static_cast<__nv_bfloat16*>(O);
   prm.sin_tiles = static_cast<__nv_bfloat16*>(sin_tiles);
-  prm.sin_lo = sin_lo; prm.sin_hi = sin_tiles ? sin_hi : 0;
+  prm.sin_lo = (int)sin_lo; prm.sin_hi = sin_tiles ? (int)sin_hi : 0;
   prm.status = status;
   if (split && !ylr_f32) return cudaErrorInvalidValue;
   auto kernel = split     ? (divide ? segment_output_tc_kernel<true, true, true> : segment_output_tc_kernel<true, true, false>)
