@@ -113,8 +113,8 @@ smat_status smat_get_geometry(const smat_plan* plan, smat_geometry* out);
 
 /* 1 when this plan's forward runs its causal branch on the tcgen05 tensor-core kernels (bf16, d_k = d_v = 128,
  * SMAT_FLAG_SIMT_ONLY and SMAT_FLAG_GATED not set), 0 when it runs on the fp32 ALUs.  Plans whose block boundary or
- * recent length is not a multiple of 128 keep fp32 tables and split every fp32 operand of a tensor-core product into
- * two bf16 parts, and their backward runs on the fp32 ALUs (with SMAT_FLAG_PER_TILE_STATES the forward too, and this
+ * recent length is not a multiple of 128 keep fp32 tables, or form none, and split every fp32 operand of a tensor-core
+ * product into two bf16 parts (scores that stand for an fp32 table: three), and their backward runs on the fp32 ALUs (with SMAT_FLAG_PER_TILE_STATES the forward too, and this
  * returns 0).  A property of the shape, not of the device. */
 int smat_uses_tensor_cores(const smat_plan* plan);
 
@@ -146,7 +146,9 @@ size_t smat_workspace_bytes(const smat_plan* plan, int for_backward);
  * Forward pass, Algorithm 1 steps 2-7 (step 1 is implicit: φ = q_i, ψ = k_j, Z_j = k_j v_jᵀ).
  * Reads Q, K, V; writes O (plan dtype).  Where a type's tokens and the keys that it sees are few (short contexts, bf16,
  * d_k = d_v = 128, positional routing), the long-range rows are formed from Q, K and V alone, and K and V of the distant
- * tokens are left in the workspace, from which smat_debug_tables forms the tables.  Else the profile table F and the
+ * tokens are left in the workspace, from which smat_debug_tables forms the tables.  Which way a plan takes depends on its
+ * shape, batch * heads among it, so a head's rows may differ in their rounding between plans of different batch sizes, and
+ * from those of smat_forward_routed with the same assignment, which always forms tables.  Else the profile table F and the
  * type table U ("cached subset states") are left there in the element type the plan keeps them in (fp32, or bf16: see
  * smat_profile_table_element_bytes / smat_type_table_element_bytes).  The incoming states S_in are left as fp32 per
  * chunk (fp32-ALU plans) or as bf16 per 128-token tile (tensor-core plans with SMAT_FLAG_PER_TILE_STATES);

@@ -35,8 +35,8 @@ struct smat_plan {
   smat_plan* inner;
   size_t off_inner;
   bool tc;             // tensor-core kernels for the causal branch
-  bool ragged_tc;      // ... of the forward only, for blocks that are not whole 128-token tiles: fp32 tables, and the
-                       // state and the scores split into two bf16 parts (backward: fp32-ALU kernels)
+  bool ragged_tc;      // ... of the forward only, for blocks that are not whole 128-token tiles: fp32 tables or (lines) none,
+                       // and the state and the scores split into two bf16 parts (backward: fp32-ALU kernels)
   bool u_bf16;         // forward keeps the type table U in bf16 and reads it with the tensor-core typed read
   bool pool_tc;        // forward pools the profile table on the tensor cores (enough tokens per profile)
   bool f_bf16;         // the profile table is kept in bf16 (d = 2: it is the type table; tab_tc: it is an MMA operand)
@@ -794,7 +794,7 @@ smat_status forward_impl(const smat_plan* pl, const void* Q, const void* K, cons
   }
   if (pl->ragged_tc) {
     pl->states_at = STATES_NOWHERE;
-    // Blocks that are not whole tiles: tables as on the fp32-ALU path (steps 2-4), the causal branch in its two-level
+    // Blocks that are not whole tiles: tables as on the fp32-ALU path (steps 2-4) or none, the causal branch in its two-level
     // form over tiles of which the last of a block is partial.
     int* status = reinterpret_cast<int*>(cx.ws + pl->off_status);
     float* ylr = cx.f(pl->off_acc);
@@ -1049,7 +1049,8 @@ void gated_inputs(Ctx& cx, const Gated& gt, const void* Q, const void* K, const 
 }
 
 // Gated forward on the tensor cores (bf16, d_k = d_v = 128, blocks of whole 128-token tiles).  The long-range part is
-// the ungated pipeline on the boundary-rescaled keys and queries; the causal part carries one state per tile: the scan
+// formed without tables, the factors at the boundary in its scores and rows, or it is the ungated pipeline on the
+// boundary-rescaled keys and queries; the causal part carries one state per tile: the scan
 // adds the sums of keys rescaled to the end of their tile and decays the running state by the tile's total gate; the
 // tile kernel multiplies the masked scores by exp(λ_i - λ_j) and the state product of row i by exp(λ_i - λ_{tile start - 1}).
 // Every exponent is a non-positive difference.
@@ -1094,8 +1095,8 @@ bool gated_backward_on_tc(const smat_plan* pl) {
   return in && (pl->geo.dense_G || (in->u_bf16 && in->fbar_bf16));
 }
 
-// Gated backward on the tensor cores: the ungated adjoint pipeline on rescaled copies (Ū from the boundary-scaled
-// queries, the reads of U and F̄ on the boundary-scaled dO, V and K), the decayed scans for S_in (keys rescaled to the
+// Gated backward on the tensor cores: long-range rows without tables, or the ungated adjoint pipeline on rescaled copies (Ū
+// from the boundary-scaled queries, the reads of U and F̄ on the boundary-scaled dO, V and K), the decayed scans for S_in (keys rescaled to the
 // end of their tile) and D̄ (queries rescaled to the start of theirs, reverse order), and the fused tile kernel with
 // the decays on both score tiles and the row factors on the three state products; it also forms dλ_t = q_t·dQ_t - k_t·dK_t.
 smat_status backward_gated_tc(Ctx& cx, const Gated& gt, const void* Q, const void* K, const void* V, const float* log_a,

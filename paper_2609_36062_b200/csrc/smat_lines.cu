@@ -12,8 +12,10 @@
 // 2-norm: 1.1e-7 from fp32 tables, 3e-7 to 1.2e-6 with three parts (the matrix instructions' sums), 2.5e-6 with two; of the
 // outputs, rounded to bf16, 1.660e-3 each way.
 //
-// The matrix instructions are those of a warp (m16n8k16): a type has 6 to 20 rows, which fill a tile of 16 and would leave most
-// of a 128-row one of tcgen05 empty, and at 545 TFLOP/s measured they are not what the kernel waits for.
+// The matrix instructions are those of a warp (m16n8k16): from d = 3 on a type has 3 to 31 rows, which fill a tile or two of 16
+// and would leave most of a 128-row one of tcgen05 empty, and at 545 TFLOP/s measured they are not what the kernel waits for.  (At d = 2
+// a type has 17 to 128 rows and would fill such a tile; there the same kernel takes them in blocks of 32, each of which gathers
+// the keys again, and the rule below counts that.)
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -167,7 +169,7 @@ __device__ __forceinline__ void mma16816_first(float (&c)[4], uint32_t a0, uint3
 }
 
 // 16-byte piece c of row r in a tile of 256-byte rows: pieces 2 q of rows 2 k and 2 k + 1 lie in different bank groups, and so do
-// piece c of rows 0 to 7.  (Rows 272 bytes apart need no exclusive or, but a sector then lands across two: 109 us for 120.)
+// piece c of rows 0 to 7.  (Rows 272 bytes apart need no exclusive or, but a sector then lands across two: 70 us where this takes 60.)
 __device__ __forceinline__ uint32_t piece(uint32_t r, uint32_t c) { return r * 256 + ((c ^ (r & 7)) << 4); }
 
 template <int RT, bool DUAL>
@@ -187,7 +189,8 @@ struct LineSmem {
 // Bound by the instructions that a warp issues for a stage, about 290 one after the other at 12 warps to an SM (8 where a thread's
 // accumulators are 128), not by the gather: 7 to 12 TB/s, where row loads alone reach 16.  Three tables' kernels / this one, us:
 // d = 3, 32 heads of 2048 tokens 137 / 33, of 4096 163 / 57, 128 heads of 8192 917 / 410, 16 heads of 16 K 312 / 147, of 24 K
-// 529 / 255; d = 4, 32 heads of 4096 552 / 190; fp32 tables: d = 3, 32 heads of 5056 503 / 95; d = 2, 32 of 4160 238 / 33.
+// 529 / 255; d = 4, 32 heads of 4096 552 / 190; fp32 tables (scores in three parts: about 370 instructions, with two 89 and 36 us): d = 3,
+// 32 heads of 5056 503 / 105; d = 2, 32 of 4160 238 / 38.
 // The first form, four warps to an item with the scores exchanged through shared memory, took 156 where this takes 57; with a
 // test for every kind of stage in front of each and all of Z in registers (spills) it was 77.
 template <int RT, bool DUAL, bool GATED, int PARTS>
@@ -532,8 +535,9 @@ bool smat_lines_supported(const SmatGeo& geo, int bh) {
 // table 0.75: there is one, and its pooling and read are near the memory rate; 32 heads, 0.7 (4096) 85 / 83 and the training step
 // 250 / 237, 16 heads, 0.8 (6144), the training step 210.7 / 214.5.  Types of less than two tokens leave the row tile empty: 16
 // heads of 5376, d = 4 (1.8) 587 / 580.
-// Items, a warp each: one to an SM, but with bf16 tables half of the warps that the chip runs, for routed calls form tables, and in
-// batches of a few heads positional arrays give the same bits as positions (2 heads of 4096 tokens, d = 3, 45 / 39).
+// Items, a warp each: one to an SM (plans are made without a device: the chip's count), but with bf16 tables half of the warps that
+// the chip runs.  That line is not where the speed turns (2 heads of 4096 tokens, d = 3, 45 with tables, 39 without): below it
+// positional arrays give the same bits as positions, for routed calls form tables on every plan.
 bool smat_lines_pay(const SmatGeo& geo, int bh, int table_bytes, bool trains) {
   constexpr uint64_t SMS = 148;
   if (!smat_lines_supported(geo, bh) || 2 * geo.B > geo.m) return false;

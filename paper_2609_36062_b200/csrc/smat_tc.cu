@@ -1002,8 +1002,8 @@ struct SegOutParams {
 // for, the loads stand in front of those stores (44 us became 47, 32 heads of 4096 tokens, d = 3).
 // SPLIT: for blocks that are not whole tiles, whose plans keep fp32 tables: the state and the score tile enter their
 // products as a leading bf16 part plus a bf16 remainder (16 bits of the fp32 value), the long-range rows arrive in
-// fp32, and the rows past a block's end load as zeros and are not stored.  (32 heads of 5056 tokens, d = 3: 0.062 ms, and
-// 0.028 for the segment totals and their scan, where chunk states, scan, scores, state read and output on the fp32 ALUs
+// fp32, and the rows past a block's end load as zeros and are not stored.  (32 heads of 5056 tokens, d = 3: 0.056 ms, and
+// 0.018 for the segment totals, where chunk states, scan, scores, state read and output on the fp32 ALUs
 // took 1.23 ms.)
 constexpr int SEG_EPI_WARPS = 16;
 constexpr int SEG_OUT_THREADS = 32 * (SEG_EPI_WARPS + 2);
