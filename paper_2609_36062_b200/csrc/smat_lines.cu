@@ -529,8 +529,9 @@ bool smat_lines_supported(const SmatGeo& geo, int bh) {
 // The line lies where the gathered bytes (from the L2 cache) pass the tables' (to and from memory) by a limit; the pass in us, with
 // tables / without.  Forward 2.3: d = 3, q = 29, 16 heads, ratio 1.7 (24 K tokens) 648 / 387, 2.1 (28 K) 673 / 607, 2.3 (32 K) 696 / 677, 2.9
 // (40 K) 765 / 850; d = 4, q = 11, 16 heads, 2.0 (10,240) 608 / 536, 2.5 (12,288) 615 / 643; with fp32 tables d = 2, 16 heads, 2.0
-// (34,880) 1097 / 392; d = 3, 8 heads, 1.4 (41,024) 1159 / 637.  From d = 4 with fp32 tables (three products a stage) 1.85: d = 4, 8
-// heads, 1.7 (16,448) 717 / 671, 2.0 (19,520) 733 / 769, 2.2 (22,592) 748 / 867.  Plans made for training steps 1.75, since dK
+// (34,880) 1097 / 392; d = 3, 8 heads, 1.4 (41,024) 1159 / 637.  d = 4 with fp32 tables (scores in three parts, staged sums) 1.85: 8
+// heads, 1.7 (16,448) 717 / 671, 2.0 (19,520) 733 / 769, 2.2 (22,592) 748 / 867; not beyond, where tables are summed by Algorithm 2: d = 5,
+// 8 heads of 3136 62 ms / 185 us.  Plans made for training steps 1.75, since dK
 // and dV take two products of a gather: d = 4, 8 heads, 1.5 (7168) 845 / 751, 2.0 (8192) 851 / 876, gated 974 / 1019.  d = 2 with a bf16
 // table 0.75: there is one, and its pooling and read are near the memory rate; 32 heads, 0.7 (4096) 85 / 83 and the training step
 // 250 / 237, 16 heads, 0.8 (6144), the training step 210.7 / 214.5.  Types of less than two tokens leave the row tile empty: 16
@@ -544,7 +545,7 @@ bool smat_lines_pay(const SmatGeo& geo, int bh, int table_bytes, bool trains) {
   const LineShape s = line_shape(geo, bh, 1);
   const double gathered = (double)s.groups * s.blocks * s.slots * 512;
   const double tables = 2.0 * (double)(geo.P + (geo.D == 1 ? 0 : geo.B)) * 16384 * table_bytes;
-  const double limit = geo.D == 1 && table_bytes == 2 ? 0.75 : trains ? 1.75 : geo.D >= 3 && table_bytes == 4 ? 1.85 : 2.3;
+  const double limit = geo.D == 1 && table_bytes == 2 ? 0.75 : trains ? 1.75 : geo.D == 3 && table_bytes == 4 ? 1.85 : 2.3;
   return s.items >= (table_bytes == 2 ? 6 * SMS : SMS) && gathered <= limit * tables;
 }
 

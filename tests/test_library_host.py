@@ -289,3 +289,19 @@ def test_rows_without_tables_refuse_what_their_kernels_would_ignore(args):
     launch = binding.load_library()["_Z25smat_launch_line_productsRK12SmatLineArgsRK7SmatGeoiP11CUstream_st"]
     launch.restype, launch.argtypes = ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p]
     assert launch(ctypes.byref(_LineArgs(rows_are_types=1, **args)), ctypes.byref(geo), 2, None) == 1
+
+
+@pytest.mark.parametrize("d,heads,T,without", [(2, 16, 34880, True), (3, 8, 58240, True), (4, 8, 16448, True), (4, 8, 19520, False),
+                                               (4, 8, 22592, False), (5, 8, 3136, True), (5, 8, 14400, True)])
+def test_which_partial_tile_plans_form_no_tables(d, heads, T, without):
+    """Both sides of the rule's lines for fp32 tables: d = 4 gives up sooner than d = 3 (whose tables take longer) and than
+    d = 5 (whose tables are summed by the literal Algorithm 2)."""
+    plan = binding.SmatPlan(1, heads, T, 128, 128, d, 64, "bf16")
+    assert plan.type_table_element_bytes() == 4
+    g = plan.geometry()
+    geo = _SmatGeo(T=g.T, c=g.c, n=g.n, m=g.m, d=d, q=g.q, D=d - 1, P=g.P, A=g.A, B=g.B, nnzC=g.nnzC)
+    geo.qpow[:d] = [g.q ** k for k in range(d)]
+    geo.dir_group_start[:d - 1] = [sum(g.q ** (d - 2 - i) for i in range(k)) for k in range(d - 1)]
+    pay = binding.load_library()["_Z14smat_lines_payRK7SmatGeoiib"]
+    pay.restype, pay.argtypes = ctypes.c_bool, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_bool]
+    assert pay(ctypes.byref(geo), heads, 4, False) == without
